@@ -129,6 +129,27 @@ def test_gpu_builder_matches_oracle_exactly(N, D, K, m, max_lists, tau):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("N,K,m,max_lists", [(257, 8192, 2, 2), (70_001, 33, 2, 2), (66_000, 1025, 8, 8), (31, 4097, 3, 2),
+                                             (65_536, 1, 1, 1), (40_000, 1280, 1, 1)])
+def test_gpu_builder_at_the_edges_of_its_ranges(N, K, m, max_lists):
+    """Several ranges with a ragged last one, parts of a range that are no multiple of 32 vectors, every number of warps
+    that the cursors of K clusters leave room for, and the three variants of the fill (one, two, up to eight choices)."""
+    import torch
+    from paper_2606_10896_b200 import flashgmm as fg
+
+    rng = np.random.Generator(np.random.PCG64(N + K + m))
+    idx = ((rng.integers(0, K, (N, 1)) + np.arange(m) * max(1, K // m)) % K).astype(np.int32)        # m different clusters
+    idx[rng.random(idx.shape) < 0.02] = -1
+    resp = np.sort(rng.random((N, m)).astype(np.float32), 1)[:, ::-1].copy()
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda:0")
+    with fg.Context(0) as ctx:
+        off_d, items_d, total, _ = ctx.gmm_build_posting_lists(t(idx), t(resp), K, 0.4, max_lists)
+    off_r, items_r, _ = posting_lists(idx, resp, K, 0.4, max_lists)
+    assert total == off_r[K] and off_d.cpu().numpy().tolist() == off_r.tolist()
+    assert items_d.cpu().numpy()[:total].tolist() == items_r.tolist()
+
+
+@pytest.mark.gpu
 def test_gpu_builder_rejects_bad_arguments():
     import torch
     from paper_2606_10896_b200 import flashgmm as fg

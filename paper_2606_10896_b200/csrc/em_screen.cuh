@@ -1,0 +1,82 @@
+// Declarations of the screening path for D <= 128 (internal).
+#pragma once
+#include <cuda.h>
+#include <cuda_runtime.h>
+#include <stdint.h>
+#include <stddef.h>
+
+namespace fg {
+
+constexpr int SCR_MAX_K = 4096;
+constexpr int64_t SCR_PIECE = 1 << 18;       // points per round of launches: capacity of the per-point buffers
+constexpr int SCR_TILE = 256;                // points per tile of the sweep
+constexpr int SCR_RANGE = 512;               // points per CTA of the pair evaluation and of the sort by component
+constexpr int SCR_SLOTS = 16;                // room for marked pairs per point (on average over the 32 points of a warp)
+constexpr int SCR_EXTRA = 4;                 // and, per point of a piece, for the rows that do not fit there
+constexpr int64_t SCR_PAIRS = SCR_PIECE * (SCR_SLOTS + SCR_EXTRA);
+constexpr int SCR_SEG = 64;                  // pairs per work item of the statistics
+constexpr int64_t SCR_ITEMS = SCR_PAIRS / SCR_SEG + SCR_MAX_K;
+constexpr int SCR_RANGES = (int)(SCR_PIECE / SCR_RANGE);
+constexpr int SCR_LL = SCR_RANGES;           // log-likelihood partial sums of the evaluation, then one per component
+constexpr int SCR_DIM_BLOCKS = 64;
+
+// Control words (in the context's result block, so that they travel to the host with the log-likelihood).
+enum { SC_DENSE = 0,      // set when a piece marks too many pairs: later kernels return at once, the caller takes the dense path
+       SC_MARKS,          // pairs marked in the current piece
+       SC_OVF,            // rows of the current piece that left the sweep without a list
+       SC_EXTRA,          // pairs of those rows
+       SC_TICKET_A, SC_TICKET_B,
+       SC_ACTIVE,         // components with a weight
+       SC_KEPT,           // kept pairs of all pieces (saturating)
+       SC_WORDS };
+
+struct ScreenBuffers {
+    float* sd;            // [128] power-of-two scale per dimension
+    float* gd;            // [128] centre
+    double* dimpart;      // [SCR_DIM_BLOCKS][4][128]
+    float4* prm;          // [K] t, c, error allowance (constant, per unit of |u|^2)
+    float* key;           // [K] the allowance of a typical point
+    unsigned char* p;     // coefficient plane [atoms][Kpad][64 halves]
+    float4* tab;          // [Kpad / 2] (t0, t1, c0, c1)
+    int4* blk;            // [SCR_MAX_K / 32] of 32 positions: largest allowances (as bits), whether one is capped
+    int* comp_of;         // [Kpad]
+    unsigned char* y;     // plane of the points [atoms][SCR_PIECE][64 halves]
+    float* n2;            // [SCR_PIECE] |u|^2
+    unsigned* pt_off;     // [SCR_PIECE] where a point's pairs start
+    int* pt_cnt;          // [SCR_PIECE] how many there are
+    unsigned short* ids;  // [SCR_PAIRS] component of a pair
+    float* val;           // [SCR_PAIRS] its responsibility (-1: the point's only pair)
+    uint2* srt;           // [SCR_PAIRS] (row, responsibility) sorted by component
+    int* counts;          // [SCR_RANGES][K]
+    int* totals;          // [K]
+    int* off;             // [K + 1] where a component's pairs start in srt
+    int* segoff;          // [K + 1] where its work items start
+    float* part;          // [SCR_ITEMS][2 D + 3]
+    double* ll;           // [SCR_LL + K]
+    int* ovf;             // [SCR_PIECE]
+    int* ctl;             // [SC_WORDS]
+};
+
+bool screen_supports(int D, int K);
+inline int screen_kpad(int K) { return (K + 127) / 128 * 128; }
+inline int screen_atoms(int D) { return (D + 31) / 32; }
+
+// Parameters -> w2, c2, c2d (as launch_prepare_fp32, with the same checks), coefficient plane and tables.  unit: k-means (mu =
+// centroids; pi, var not read; log2 z = -|x - mu|^2).  Clears SC_DENSE.
+cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
+                                  const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
+// One piece of n <= SCR_PIECE points: plane, sweep, rows without a list.  margin: log2 units below a point's best value down to
+// which pairs are marked (40, or 0 for the arg-max alone).  max_marks: pairs per point up to which the screening pays.
+cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, float max_marks,
+                                const float* mu, const float* w2, const double* c2d, const ScreenBuffers& b, int* status, int sms,
+                                int64_t* launches);
+// Exact values of the marked pairs.  SCREEN_EM: responsibilities of the pairs within 2^-40 of their point's total, counted per
+// component; SCREEN_LOGP: logp[i]; SCREEN_ARGMAX: idx[i], and the pair itself kept with weight 1 for the statistics.
+enum { SCREEN_EM = 0, SCREEN_LOGP = 1, SCREEN_ARGMAX = 2 };
+cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx);
+// Statistics of the kept pairs: sorted by component, summed in fixed segments, added to (Nk, S1, S2) in float64.
+cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
+                                const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches);
+
+}  // namespace fg

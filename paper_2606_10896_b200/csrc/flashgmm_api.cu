@@ -3,6 +3,7 @@
 #include "internal.cuh"
 #include "em_tc.cuh"
 #include "em_wide.cuh"
+#include "em_screen.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -22,6 +23,7 @@ struct DevResult {
     int status;     // sticky: device code ORs bits in; the host clears it only after it has reported them
     int n_ill;      // ill-conditioned components found by the tensor path's last preparation
     int counts[2];  // the last parameter update: variance entries raised to the floor, components left unchanged as empty
+    int scr[SC_WORDS];      // control words of the screening path (D <= 128)
 };
 
 constexpr size_t STAGE_BYTES = (size_t)128 << 20;   // per staging buffer of the host-streaming path
@@ -37,6 +39,9 @@ struct ScratchLayout {
     size_t w_sd, w_kap, w_gd, w_phi, w_plo, w_tk, w_tkck, w_ckd, w_cref, w_illb, w_flags, w_yhi, w_ylo, w_logz, w_partial, w_llpart, w_illlist, w_muc, w_w2c, w_c2dc, w_statsc, w_top, w_logzx, w_compof, w_scra, w_scrw, w_scr, w_slotof, w_scrmask, w_n2, w_cand, w_candT, w_ctl, w_scre, w_slotcnt, w_heavyof, w_heavyslot, w_heavypart, w_scrahi, w_scrwhi, w_pairval, w_pairoff, w_pairbest, w_pairkey8, w_pairval8, w_rec, w_reccnt, w_recthr;
     size_t w_partial_bytes;
     bool wide;
+    // the screening path for D <= 128 (its plane of the points lies in tc_yhi)
+    size_t s_sd, s_gd, s_dimpart, s_prm, s_key, s_p, s_tab, s_blk, s_compof, s_n2, s_ptoff, s_ptcnt, s_ids, s_val, s_srt, s_counts, s_totals, s_off, s_segoff, s_part, s_ll, s_ovf;
+    bool scr;
 };
 
 // planes: include the fp16 planes of Y (tensor path only; 2 x TC_YPLANE_BYTES, placed last so that no other offset moves)
@@ -145,6 +150,34 @@ ScratchLayout scratch_layout(int D, int K, bool planes) {
         L.w_yhi = take((size_t)WIDE_PIECE * wp.Dpad * 4);
         L.w_ylo = take((size_t)WIDE_PIECE * wp.Dpad * 4);
     }
+    L.scr = L.tc && planes && screen_supports(D, K);
+    L.s_sd = L.s_gd = L.s_dimpart = L.s_prm = L.s_key = L.s_p = L.s_tab = L.s_blk = L.s_compof = L.s_n2 = L.s_ptoff = L.s_ptcnt = L.s_ids = L.s_val = L.s_srt = L.s_counts = L.s_totals = L.s_off = L.s_segoff = L.s_part = L.s_ll = L.s_ovf = 0;
+    if (L.scr) {
+        static_assert((size_t)SCR_PIECE * 512 <= TC_YPLANE_BYTES, "the plane of the screening path lies in that of the tile kernel");
+        const size_t Kpad = (size_t)screen_kpad(K);
+        L.s_sd = take(128 * 4);
+        L.s_gd = take(128 * 4);
+        L.s_dimpart = take((size_t)SCR_DIM_BLOCKS * 512 * 8);
+        L.s_prm = take((size_t)K * 16);
+        L.s_key = take((size_t)K * 4);
+        L.s_p = take((size_t)screen_atoms(D) * Kpad * 128);
+        L.s_tab = take(Kpad * 8);
+        L.s_blk = take((size_t)SCR_MAX_K / 32 * 16);
+        L.s_compof = take(Kpad * 4);
+        L.s_n2 = take((size_t)SCR_PIECE * 4);
+        L.s_ptoff = take((size_t)SCR_PIECE * 4);
+        L.s_ptcnt = take((size_t)SCR_PIECE * 4);
+        L.s_ids = take((size_t)SCR_PAIRS * 2);
+        L.s_val = take((size_t)SCR_PAIRS * 4);
+        L.s_srt = take((size_t)SCR_PAIRS * 8);
+        L.s_counts = take((size_t)SCR_RANGES * K * 4);
+        L.s_totals = take((size_t)K * 4);
+        L.s_off = take((size_t)(K + 1) * 4);
+        L.s_segoff = take((size_t)(K + 1) * 4);
+        L.s_part = take((size_t)SCR_ITEMS * (2 * (size_t)D + 3) * 4);
+        L.s_ll = take((size_t)(SCR_LL + K) * 8);
+        L.s_ovf = take((size_t)SCR_PIECE * 4);
+    }
     L.total = off;
     return L;
 }
@@ -200,6 +233,10 @@ struct gmm_ctx {
                                      // 1 = pair by pair unless sweep 1 marks too many pairs, 2 = always pair by pair (tests)
     int tc_n_ill = 0;                // ill-conditioned components at the last result that was read back (picks the filter)
     int tc_force_filter = -1;        // GMM_TC_FILTER=plain / tight: 0 / 1 (tests); -1: automatic
+    double scr_marks = -1.0;         // GMM_SCREEN_MARKS: marked pairs per point up to which the screening path is taken (D <= 128;
+                                     // 0: never, < 0: from the measured costs, see screen_limit)
+    int64_t scr_piece = SCR_PIECE;   // points per round of launches of the screening path
+    int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
     int sticky_status = 0;           // status bits read off the device but not yet reported (see ensure_scratch)
     // host-streaming path
     cudaStream_t copy_stream = nullptr;
@@ -252,6 +289,35 @@ struct gmm_ctx {
         b.dec_dim = reinterpret_cast<int*>(scratch + lay.tc_decdim);
         b.dec_w = reinterpret_cast<float*>(scratch + lay.tc_decw);
         b.dec_mu = reinterpret_cast<float*>(scratch + lay.tc_decmu);
+        return b;
+    }
+    ScreenBuffers screen() const {
+        ScreenBuffers b;
+        auto at = [&](size_t o) { return scratch + o; };
+        b.sd = reinterpret_cast<float*>(at(lay.s_sd));
+        b.gd = reinterpret_cast<float*>(at(lay.s_gd));
+        b.dimpart = reinterpret_cast<double*>(at(lay.s_dimpart));
+        b.prm = reinterpret_cast<float4*>(at(lay.s_prm));
+        b.key = reinterpret_cast<float*>(at(lay.s_key));
+        b.p = at(lay.s_p);
+        b.tab = reinterpret_cast<float4*>(at(lay.s_tab));
+        b.blk = reinterpret_cast<int4*>(at(lay.s_blk));
+        b.comp_of = reinterpret_cast<int*>(at(lay.s_compof));
+        b.y = at(lay.tc_yhi);
+        b.n2 = reinterpret_cast<float*>(at(lay.s_n2));
+        b.pt_off = reinterpret_cast<unsigned*>(at(lay.s_ptoff));
+        b.pt_cnt = reinterpret_cast<int*>(at(lay.s_ptcnt));
+        b.ids = reinterpret_cast<unsigned short*>(at(lay.s_ids));
+        b.val = reinterpret_cast<float*>(at(lay.s_val));
+        b.srt = reinterpret_cast<uint2*>(at(lay.s_srt));
+        b.counts = reinterpret_cast<int*>(at(lay.s_counts));
+        b.totals = reinterpret_cast<int*>(at(lay.s_totals));
+        b.off = reinterpret_cast<int*>(at(lay.s_off));
+        b.segoff = reinterpret_cast<int*>(at(lay.s_segoff));
+        b.part = reinterpret_cast<float*>(at(lay.s_part));
+        b.ll = reinterpret_cast<double*>(at(lay.s_ll));
+        b.ovf = reinterpret_cast<int*>(at(lay.s_ovf));
+        b.ctl = result()->scr;
         return b;
     }
     WideBuffers wide() const {
@@ -715,6 +781,65 @@ int read_result(gmm_ctx* ctx, int slot, double* loglik) {
     CU(cudaStreamSynchronize(ctx->stream));
     CHECK(report_status(ctx, r.status));
     ctx->tc_n_ill = r.n_ill;
+    ctx->scr_active = 0;
+    *loglik = r.ll[slot];
+    if (!std::isfinite(*loglik)) return fail(ctx, GMM_ENUMERIC, "log-likelihood is not finite (%g): non-finite values in X?", *loglik);
+    return GMM_OK;
+}
+
+// ---- the screening path (D <= 128) ----------------------------------------------------------------------------------
+// AUTO tries it first wherever it would take the tensor path.  Its kernels find out themselves whether it pays (SC_DENSE) and
+// then return at once, so a call enqueues the whole path, reads the verdict with its result and only then, if need be, runs the
+// dense kernels: sparse posteriors cost no extra synchronisation, broad ones the sweep of one piece.
+bool screen_wanted(const gmm_ctx* ctx, int D, int K) {
+    return ctx->path == GMM_PATH_AUTO && ctx->lay.scr && ctx->capPlanes && ctx->scr_marks != 0.0 && auto_is_tensor(D, K);
+}
+// Marked pairs per point up to which the screening path is the cheaper one.
+double screen_limit(const gmm_ctx* ctx, int K) {
+    if (ctx->scr_marks > 0.0) return ctx->scr_marks;
+    return 0.012 * K < 2.0 ? 2.0 : 0.012 * K < 12.0 ? 0.012 * K : 12.0;
+}
+
+int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, const float* var, bool unit) {
+    const ScreenBuffers sb = ctx->screen();
+    KL(launch_screen_prepare(ctx->stream, D, K, pi, mu, var, unit, sb, ctx->w2(), ctx->c2(), ctx->c2d(), &ctx->result()->status));
+    ctx->launches += 2;
+    CU(cudaMemsetAsync(sb.ll, 0, (size_t)(SCR_LL + K) * 8, ctx->stream));
+    return GMM_OK;
+}
+
+// Adds the statistics of n points to (Nk, S1, S2) and their log-likelihood to the partial sums.
+int screen_points(gmm_ctx* ctx, const float* X, int64_t n, int D, int K, const float* mu, double* Nk, double* S1, double* S2) {
+    const ScreenBuffers sb = ctx->screen();
+    for (int64_t off = 0; off < n; off += ctx->scr_piece) {
+        const int64_t cnt = (n - off < ctx->scr_piece) ? (n - off) : ctx->scr_piece;
+        const float* Xs = X + off * D;
+        CHECK(prof_begin(ctx));
+        CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, 40.f, (float)screen_limit(ctx, K), mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
+        KL(launch_screen_eval(ctx->stream, SCREEN_EM, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, nullptr, nullptr));
+        CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
+        CHECK(prof_end(ctx));
+    }
+    return GMM_OK;
+}
+
+int screen_end(gmm_ctx* ctx, int K, int slot) {
+    KL(launch_reduce_ll(ctx->stream, ctx->screen().ll, SCR_LL + K, &ctx->result()->ll[slot], false));
+    return GMM_OK;
+}
+
+// Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels (nothing is
+// reported then: they find what is wrong again).
+int screen_result(gmm_ctx* ctx, int slot, double* loglik, bool* dense) {
+    DevResult r;
+    CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    *dense = r.scr[SC_DENSE] != 0;
+    ctx->scr_active = 0;
+    if (*dense) return GMM_OK;
+    CHECK(report_status(ctx, r.status));
+    ctx->scr_active = r.scr[SC_ACTIVE];
+    ctx->last_path = GMM_PATH_TENSOR;
     *loglik = r.ll[slot];
     if (!std::isfinite(*loglik)) return fail(ctx, GMM_ENUMERIC, "log-likelihood is not finite (%g): non-finite values in X?", *loglik);
     return GMM_OK;
@@ -749,6 +874,11 @@ int gmm_create(gmm_ctx** out, int device, void* cuda_stream) {
     ctx->device = device;
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
     if (const char* e = std::getenv("GMM_TC_COND_LIMIT")) ctx->tc_cond_limit = (float)std::atof(e);
+    if (const char* e = std::getenv("GMM_SCREEN_MARKS")) ctx->scr_marks = std::atof(e);
+    if (const char* e = std::getenv("GMM_SCREEN_PIECE")) {
+        const long long v = std::atoll(e);
+        if (v >= SCR_TILE && v <= SCR_PIECE) ctx->scr_piece = v / SCR_TILE * SCR_TILE;
+    }
     if (const char* e = std::getenv("GMM_TC_FILTER")) ctx->tc_force_filter = (e[0] == 't') ? 1 : (e[0] == 'p' ? 0 : -1);
     if (const char* e = std::getenv("GMM_TC_FLUSH")) ctx->tc_flush = std::atoi(e);
     if (const char* e = std::getenv("GMM_WIDE_MIN_POINTS")) ctx->wide_min_points = std::atof(e);
@@ -819,7 +949,7 @@ int gmm_last_path(const gmm_ctx* ctx) { return ctx ? ctx->last_path : GMM_EINVAL
 int gmm_last_exact_count(const gmm_ctx* ctx) {
     if (!ctx) return GMM_EINVAL;
     if (ctx->last_path != GMM_PATH_TENSOR) return 0;
-    return wide_supports(ctx->capD, ctx->capK) ? ctx->wide_n_ill : ctx->tc_n_ill;
+    return wide_supports(ctx->capD, ctx->capK) ? ctx->wide_n_ill : ctx->scr_active > 0 ? ctx->scr_active : ctx->tc_n_ill;
 }
 
 int gmm_last_exact_pairs(gmm_ctx* ctx, int64_t* marked, int64_t* kept, int* dense_pieces) {
@@ -850,6 +980,15 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     DeviceGuard g(ctx->device);
     int path;
     CHECK(ensure_scratch(ctx, D, K));
+    if (screen_wanted(ctx, D, K)) {
+        bool dense = false;
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+        CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
+        CHECK(screen_end(ctx, K, 0));
+        CHECK(screen_result(ctx, 0, loglik, &dense));
+        if (!dense) return GMM_OK;
+    }
     CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
     CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
     CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, 0));
@@ -919,20 +1058,34 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
     int t = 0;
     for (; t < iters; ++t) {
         const int slot = t % LL_SLOTS;
-        CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
-        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
-        CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, slot));
         // The update is skipped on the device when the step raised a status bit or left a non-finite log-likelihood
-        // (invalid parameters, a time-out, non-finite data): the caller then keeps the last good parameters.
-        CU(cudaMemsetAsync(ctx->result()->counts, 0, 2 * sizeof(int), ctx->stream));
-        if (ctx->covariance == GMM_COV_ISOTROPIC)
-            KL(launch_finalize_isotropic(ctx->stream, N, D, K, Nk, S1, S2, var_floor, pi, mu, var, ctx->result()->counts,
-                                         &ctx->result()->status, &ctx->result()->ll[slot]));
-        else
-            KL(launch_finalize(ctx->stream, N, D, K, Nk, S1, S2, var_floor, pi, mu, var, ctx->result()->counts,
-                               &ctx->result()->status, &ctx->result()->ll[slot]));
-        ctx->last_path = path;
-        int rc = read_result(ctx, slot, &loglik_trace[t]);
+        // (invalid parameters, a time-out, non-finite data): the caller then keeps the last good parameters.  So it is when
+        // the screening path has left the step to the dense kernels.
+        auto update = [&](const int* skip_dense) -> int {
+            CU(cudaMemsetAsync(ctx->result()->counts, 0, 2 * sizeof(int), ctx->stream));
+            auto f = ctx->covariance == GMM_COV_ISOTROPIC ? launch_finalize_isotropic : launch_finalize;
+            KL(f(ctx->stream, N, D, K, Nk, S1, S2, var_floor, pi, mu, var, ctx->result()->counts, &ctx->result()->status,
+                 &ctx->result()->ll[slot], skip_dense));
+            return GMM_OK;
+        };
+        int rc = GMM_OK;
+        bool dense = true;
+        if (screen_wanted(ctx, D, K)) {
+            CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
+            CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
+            CHECK(screen_end(ctx, K, slot));
+            CHECK(update(&ctx->result()->scr[SC_DENSE]));
+            rc = screen_result(ctx, slot, &loglik_trace[t], &dense);
+        }
+        if (dense && rc == GMM_OK) {
+            CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
+            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
+            CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, slot));
+            CHECK(update(nullptr));
+            ctx->last_path = path;
+            rc = read_result(ctx, slot, &loglik_trace[t]);
+        }
         if (rc != GMM_OK) {
             if (iters_done) *iters_done = t;
             return rc;
@@ -1029,24 +1182,48 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     CU(cudaMemcpyAsync(ctx->xstage[0], X_host, (size_t)cnt0 * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
     CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
-    CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
+    bool screening = screen_wanted(ctx, D, K);
+    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+    else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
     CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
-    int c = 0;
+    int c = 0;                                       // chunks copied so far: they take the buffers in turn
+    bool copied = true;                              // (the first one already is)
     for (int64_t off = 0; off < N; off += rows_per_chunk, ++c) {
         const int b = c & 1;
         const int64_t cnt = (N - off < rows_per_chunk) ? (N - off) : rows_per_chunk;
-        if (c > 0) {
+        if (!copied) {
             if (c >= 2) CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_done[b], 0));
             CU(cudaMemcpyAsync(ctx->xstage[b], X_host + off * D, (size_t)cnt * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
             CU(cudaEventRecord(ctx->ev_copied[b], ctx->copy_stream));
             CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[b], 0));
         }
-        CHECK(accumulate_points(ctx, path, ctx->xstage[b], cnt, D, K, mu, Nk, S1, S2, 0));
+        copied = false;
+        if (screening) {
+            CHECK(screen_points(ctx, ctx->xstage[b], cnt, D, K, mu, Nk, S1, S2));
+            if (off + rows_per_chunk >= N) {
+                bool dense = false;
+                CHECK(screen_end(ctx, K, 0));
+                CHECK(screen_result(ctx, 0, loglik, &dense));
+                if (dense) {
+                    // broad posteriors: the dense kernels take the whole call, chunk by chunk again
+                    screening = false;
+                    CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, nullptr, 0));
+                    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+                    off = -rows_per_chunk;
+                }
+            }
+        } else {
+            CHECK(accumulate_points(ctx, path, ctx->xstage[b], cnt, D, K, mu, Nk, S1, S2, 0));
+        }
         CU(cudaEventRecord(ctx->ev_done[b], ctx->stream));
     }
     CU(cudaMemcpyAsync(Nk_host, Nk, (size_t)K * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaMemcpyAsync(S1_host, S1, KD * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaMemcpyAsync(S2_host, S2, KD * 8, cudaMemcpyDeviceToHost, ctx->stream));
+    if (screening) {
+        CU(cudaStreamSynchronize(ctx->stream));
+        return GMM_OK;
+    }
     ctx->last_path = path;
     return read_result(ctx, 0, loglik);
 }

@@ -65,14 +65,14 @@ cudaError_t launch_reduce_partials(cudaStream_t s, int D, int K, int splits, con
 cudaError_t launch_reduce_ll(cudaStream_t s, const double* llpart, int64_t n, double* ll, bool accumulate);
 // counts (may be NULL): counts[0] += variance entries raised to the floor, counts[1] += components left unchanged
 // because N_k < 1e-12 (integer atomics).  skip_status / skip_ll (may be NULL): the kernel writes nothing when
-// *skip_status != 0 or *skip_ll is not finite (the step that produced the statistics failed).
+// *skip_status != 0, *skip_flag != 0 or *skip_ll is not finite (the step that produced the statistics failed).
 cudaError_t launch_finalize(cudaStream_t s, int64_t N, int D, int K, const double* Nk, const double* S1,
                             const double* S2, float var_floor, float* pi, float* mu, float* var, int* counts,
-                            const int* skip_status, const double* skip_ll);
+                            const int* skip_status, const double* skip_ll, const int* skip_flag = nullptr);
 
 cudaError_t launch_finalize_isotropic(cudaStream_t s, int64_t N, int D, int K, const double* Nk, const double* S1,
                                       const double* S2, float var_floor, float* pi, float* mu, float* var, int* counts,
-                                      const int* skip_status, const double* skip_ll);
+                                      const int* skip_status, const double* skip_ll, const int* skip_flag = nullptr);
 
 // ---- Fisher vector of one group from its statistics (paper Section 6) ----------------------------------------------
 // out[2 * K * D] (device): the means part [K x D], then the standard-deviations part [K x D]

@@ -56,8 +56,9 @@ __global__ void reduce_ll_kernel(const double* __restrict__ llpart, int64_t n, d
 __global__ void finalize_kernel(int64_t N, int D, int K, const double* __restrict__ Nk, const double* __restrict__ S1,
                                 const double* __restrict__ S2, float var_floor, float* __restrict__ pi,
                                 float* __restrict__ mu, float* __restrict__ var, int* __restrict__ counts,
-                                const int* __restrict__ skip_status, const double* __restrict__ skip_ll) {
-    if ((skip_status && *skip_status != 0) || (skip_ll && !isfinite(*skip_ll))) return;      // the step failed: keep the parameters
+                                const int* __restrict__ skip_status, const double* __restrict__ skip_ll,
+                                const int* __restrict__ skip_flag) {
+    if ((skip_flag && *skip_flag != 0) || (skip_status && *skip_status != 0) || (skip_ll && !isfinite(*skip_ll))) return;      // the step failed: keep the parameters
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (size_t)K * D) return;
     const int k = (int)(e / D);
@@ -85,8 +86,9 @@ __global__ void finalize_isotropic_kernel(int64_t N, int D, int K, const double*
                                           const double* __restrict__ S1, const double* __restrict__ S2,
                                           float var_floor, float* __restrict__ pi, float* __restrict__ mu,
                                           float* __restrict__ var, int* __restrict__ counts,
-                                          const int* __restrict__ skip_status, const double* __restrict__ skip_ll) {
-    if ((skip_status && *skip_status != 0) || (skip_ll && !isfinite(*skip_ll))) return;      // the step failed: keep the parameters
+                                          const int* __restrict__ skip_status, const double* __restrict__ skip_ll,
+                                          const int* __restrict__ skip_flag) {
+    if ((skip_flag && *skip_flag != 0) || (skip_status && *skip_status != 0) || (skip_ll && !isfinite(*skip_ll))) return;      // the step failed: keep the parameters
     const int k = blockIdx.x;
     __shared__ double red[128];
     const double nk = Nk[k];
@@ -120,8 +122,8 @@ __global__ void finalize_isotropic_kernel(int64_t N, int D, int K, const double*
 
 cudaError_t launch_finalize_isotropic(cudaStream_t s, int64_t N, int D, int K, const double* Nk, const double* S1,
                                       const double* S2, float var_floor, float* pi, float* mu, float* var, int* counts,
-                                      const int* skip_status, const double* skip_ll) {
-    finalize_isotropic_kernel<<<K, 128, 0, s>>>(N, D, K, Nk, S1, S2, var_floor, pi, mu, var, counts, skip_status, skip_ll);
+                                      const int* skip_status, const double* skip_ll, const int* skip_flag) {
+    finalize_isotropic_kernel<<<K, 128, 0, s>>>(N, D, K, Nk, S1, S2, var_floor, pi, mu, var, counts, skip_status, skip_ll, skip_flag);
     return cudaGetLastError();
 }
 
@@ -144,9 +146,9 @@ cudaError_t launch_reduce_ll(cudaStream_t s, const double* llpart, int64_t n, do
 
 cudaError_t launch_finalize(cudaStream_t s, int64_t N, int D, int K, const double* Nk, const double* S1,
                             const double* S2, float var_floor, float* pi, float* mu, float* var, int* counts,
-                            const int* skip_status, const double* skip_ll) {
+                            const int* skip_status, const double* skip_ll, const int* skip_flag) {
     const size_t n = (size_t)K * D;
-    finalize_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(N, D, K, Nk, S1, S2, var_floor, pi, mu, var, counts, skip_status, skip_ll);
+    finalize_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(N, D, K, Nk, S1, S2, var_floor, pi, mu, var, counts, skip_status, skip_ll, skip_flag);
     return cudaGetLastError();
 }
 

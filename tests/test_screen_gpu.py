@@ -1,0 +1,131 @@
+"""The screening path for D <= 128 (csrc/em_screen.cu): one tensor sweep over a single fp16 product marks the (point,
+component) pairs that can matter, those are evaluated exactly.  GMM_PATH_AUTO tries it first; gmm_last_exact_count is the
+number of components with a weight after a step that took it."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import gmm_oracle as orc
+from paper_2606_10896_b200 import synth
+from tests.parity_util import assert_stats_close, data_scale
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def fg():
+    from paper_2606_10896_b200 import flashgmm
+
+    return flashgmm
+
+
+def _t(a, dtype=torch.float32):
+    return torch.as_tensor(np.ascontiguousarray(a), dtype=dtype, device=DEV).contiguous()
+
+
+def _mixture(N, D, K, seed, collapsed=0):
+    """Separate clusters; some components share a cluster, the last ``collapsed`` ones sit on single points."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    centre = rng.normal(0, 3, (K, D))
+    centre[1::7] = centre[0::7][: len(centre[1::7])] + 0.3 * rng.normal(size=(len(centre[1::7]), D))
+    std = rng.uniform(0.5, 1.5, (K, D))
+    c = rng.integers(0, K, N)
+    X = (centre[c] + std[c] * rng.standard_normal((N, D))).astype(np.float32)
+    mu, var = centre + 0.2 * rng.normal(size=(K, D)), std ** 2
+    if collapsed:
+        mu[-collapsed:] = X[rng.integers(0, N, collapsed)]
+        var[-collapsed:] = 1e-6
+    pi = rng.dirichlet(np.ones(K))
+    return X, pi.astype(np.float32), mu.astype(np.float32), var.astype(np.float32)
+
+
+def _step(fg, c, X, pi, mu, var, expect_count, what):
+    ref = orc.em_step(X, pi, mu, var)
+    out = []
+    for _ in range(2):
+        Nk, S1, S2, L = c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
+        out.append((Nk.cpu().numpy(), S1.cpu().numpy(), S2.cpu().numpy(), L))
+    if expect_count is not None:
+        assert c.gmm_last_path() == fg.GMM_PATH_TENSOR and c.gmm_last_exact_count() == expect_count, what
+    assert abs(out[0][3] - ref[3]) <= 1e-5 * abs(ref[3]) + 1e-6, what
+    assert_stats_close(len(X), max(1.0, data_scale(X)), out[0][:3], ref[:3], what)
+    for a, b in zip(out[0], out[1]):                       # the same bits in every run
+        assert np.array_equal(a, b), what
+
+
+# tiles of 256 points, ranges of 512, atoms of 32 dimensions, k-steps of 8, groups of 128 and blocks of 32 components
+@pytest.mark.parametrize("N,D,K", [(1, 8, 64), (255, 128, 64), (257, 33, 65), (511, 31, 128), (513, 32, 129), (1024, 97, 257),
+                                   (1500, 41, 1000), (1300, 9, 90), (3001, 127, 96), (700, 64, 4096), (2049, 100, 160)])
+def test_screen_against_oracle_at_the_edges_of_its_tiles(fg, monkeypatch, N, D, K):
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    X, pi, mu, var = _mixture(N, D, K, N + D + K, collapsed=3)
+    pi[K // 2] = 0.0                                       # one component without a weight
+    with fg.Context(0) as c:
+        _step(fg, c, X, pi, mu, var, K - 1, f"screen N={N} D={D} K={K}")
+
+
+def test_screen_accumulates_over_pieces_and_takes_unaligned_rows(fg, monkeypatch):
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    monkeypatch.setenv("GMM_SCREEN_PIECE", "768")
+    X, pi, mu, var = _mixture(3000, 66, 130, 5, collapsed=2)
+    with fg.Context(0) as c:
+        _step(fg, c, X, pi, mu, var, 130, "four pieces, rows of 8-byte alignment")
+        host = c.gmm_em_step_host(X, pi, mu, var)
+        dev = c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
+        assert np.array_equal(host[0], dev[0].cpu().numpy()) and np.array_equal(host[2], dev[2].cpu().numpy()) and host[3] == dev[3]
+
+
+def test_screen_rows_without_a_list(fg, monkeypatch):
+    """A few points far outside the range of the fp16 plane, and a few that a great many components explain about equally well:
+    both leave the sweep without a list and are evaluated against all components."""
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    N, D, K = 6000, 24, 700
+    X, pi, mu, var = _mixture(N, D, K, 11)
+    X[::1500] = 4000.0                                     # beyond 240 times the data's spread
+    mu[100:], var[100:] = 6.0 + 0.05 * mu[100:], 1.0       # 600 components in one place ...
+    rows = np.setdiff1d(np.arange(N), np.arange(0, N, 1500))
+    X[rows] = (mu[rows % 100] + np.sqrt(var[rows % 100])).astype(np.float32)
+    X[100::1000] = 6.0                                     # ... and six points there
+    with fg.Context(0) as c:
+        _step(fg, c, X, pi, mu, var, K, "rows without a list")
+
+
+def test_screen_leaves_broad_posteriors_to_the_dense_kernels(fg):
+    rng = np.random.default_rng(3)
+    N, D, K = 4000, 16, 128
+    X = rng.normal(size=(N, D)).astype(np.float32)
+    mu = (0.1 * rng.normal(size=(K, D))).astype(np.float32)
+    var = rng.uniform(0.8, 1.2, (K, D)).astype(np.float32)
+    pi = np.full(K, 1 / K, np.float32)
+    with fg.Context(0) as c:
+        _step(fg, c, X, pi, mu, var, None, "broad posteriors")
+        assert c.gmm_last_path() == fg.GMM_PATH_TENSOR and c.gmm_last_exact_count() < K
+        # a fit applies every iteration's update exactly once, whichever kernels took the step
+        p, m, v = _t(pi), _t(mu), _t(var)
+        trace, done = c.gmm_fit(_t(X), p, m, v, 3)
+        ref = orc.fit(X, pi, mu, var, 3, var_floor=1e-6)
+        assert done == 3
+        np.testing.assert_allclose(trace, ref["trace"], rtol=1e-5)
+
+
+def test_screen_reports_non_finite_data(fg):
+    X, pi, mu, var = _mixture(2000, 40, 128, 3)
+    X[1234, 5] = np.nan
+    with fg.Context(0) as c:
+        with pytest.raises(fg.GmmError) as e:
+            c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
+        assert e.value.code == fg.GMM_ENUMERIC
+        X[1234, 5] = 0.0
+        c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
+
+
+def test_config2_free_running_through_the_screening_path(fg):
+    spec = synth.CONFIGS[2].with_n(20_000)
+    X = synth.sample_host(spec)
+    pi0, mu0, var0 = synth.init_params(X, spec)
+    ref = orc.fit(X, pi0, mu0, var0, 8, var_floor=spec.var_floor)
+    with fg.Context(0) as c:
+        trace, done = c.gmm_fit(_t(X), _t(pi0), _t(mu0), _t(var0), 8, spec.var_floor)
+        assert done == 8
+        np.testing.assert_allclose(trace, ref["trace"], rtol=1e-4)

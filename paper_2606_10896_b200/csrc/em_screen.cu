@@ -4,8 +4,8 @@
 // densities and statistics.  ONE sweep of the tensor cores over a single fp16 product per contraction (a sixth of the work of
 // the kernels that form every responsibility from split operands) tells which they are, with rigorous error bounds:
 //
-//   screen_sweep_kernel   TMEM lanes = points.  A CTA holds the fp16 plane of 256 points in shared memory and streams the
-//                         components' coefficients past it, 128 at a time; a softmax thread owns one point, keeps the largest
+//   screen_sweep_kernel   TMEM lanes = points.  A CTA holds the fp16 rows of 256 points in tensor memory and streams the
+//                         components' coefficients past them, 128 at a time; a softmax thread owns one point, keeps the largest
 //                         lower bound seen so far and the components whose upper bound reaches it (less the margin), drops
 //                         those that the final bound rules out, and writes the rest as a list.
 //   screen_eval_kernel    the listed pairs in fp32 direct differences: log-sum-exp, responsibilities, or the arg-max.
@@ -30,22 +30,26 @@ namespace {
 //
 // Points and means enter as u = s_d (x - g_d), nu = s_d (mu - g_d): g the mixture's mean, s_d a power of two that brings the
 // dimension to size 1.  With b = w2 / s^2 (w2 = log2 e / (2 var)):  log2 z = c + sum_d (2 b nu) u + (-b) u^2,
-// c = log2 pi + ... - sum_d b nu^2.  Rows are divided by a power of two t (largest coefficient in [512, 1024)) and rounded
-// to fp16.
+// c = log2 pi + ... - sum_d b nu^2.  The coefficients are rounded to fp16 as they are; c is split into three fp16 values (of 256,
+// 1 and 1) and added by the tensor cores too, so that an accumulator IS the approximate log2 z: a table of scales and constants
+// read by every softmax thread cost more shared-memory bandwidth than the products.
 //
-// Error of the approximate log2 z of ANY point: every product is formed from two operands rounded to 2^-11 (or to 2^-25, the
-// spacing of subnormals) and added into an fp32 accumulator that loses less than 2^-18 of the terms' sizes, and the sizes add
-// up to at most  sum_d b (2 |nu u| + u^2) <= sum_d b nu^2 + 2 max_d b |u|^2.  So it is below alpha + beta |u|^2 with
-//   alpha = eps sum_d b nu^2 + 2^-24 sum_d (2 b |nu| + b) + t 2^-25 D / 2 + 2^-22 |c| + 0.02
-//   beta  = 2 eps max_d b + 1.5 t 2^-25,        eps = 2^-10 (1 + 2^-6).
+// Error of the approximate log2 z of ANY point: u and the coefficients are rounded to 2^-11 (or to 2^-25, the spacing of
+// subnormals), the square of the rounded u once more (3 x 2^-11 in all), and the products are added into an fp32 accumulator
+// that loses less than 2^-18 of the terms' sizes:  2^-10 sum_d 2 b |nu u| + 2^-9 sum_d b u^2 <= 2^-10 (sum_d b nu^2 + 3 max_d b |u|^2).
+// So it is below alpha + beta |u|^2 with
+//   alpha = eps sum_d b nu^2 + 2^-24 sum_d (2 b |nu| + b) + 2^-25 D / 2 + 2^-18 |c| + 0.02
+//   beta  = 3 eps max_d b + 1.5 x 2^-25,        eps = 2^-10 (1 + 2^-6).
 //
 // A component that is much narrower than the data in some dimensions (a few points, one point) has a huge max_d b, and with it
-// an allowance that rules nothing out.  Where the allowance of a typical point exceeds SCR_SHARP bits, b is CAPPED at a value
-// that leaves about 16: c - sum_d min(b, cap) (u - nu)^2 is an upper bound of log2 z, which is what the screening needs, with a
-// small allowance; only its lower bound is lost, so such components do not raise the threshold.
+// an allowance that rules nothing out (or coefficients beyond fp16).  Where the allowance of a typical point exceeds SCR_SHARP
+// bits, b is CAPPED at a value that leaves about 16: c - sum_d min(b, cap) (u - nu)^2 is an upper bound of log2 z, which is what
+// the screening needs, with a small allowance; only its lower bound is lost, so such components do not raise the threshold.
 constexpr float SCR_SHARP = 40.f;
 constexpr float SCR_CAPPED = 1e30f;          // their sorting key
-__device__ __forceinline__ double screen_cap(int D) { return 16.0 / (2.0 * 9.765625e-04 * (double)D); }
+constexpr float SCR_NEVER = -1.5e7f;         // c of a position without a component
+// (numax: largest |nu| of the component; 2 cap |nu| stays within fp16)
+__device__ __forceinline__ double screen_cap(int D, double numax) { return fmin(fmin(16.0 / (3.0 * 9.765625e-04 * (double)D), 30000.0), 30000.0 / fmax(numax, 1e-30)); }
 
 __global__ void __launch_bounds__(512) screen_dim_kernel(int D, int K, const float* __restrict__ pi, const float* __restrict__ mu,
                                                          const float* __restrict__ var, int unit, double* __restrict__ part,
@@ -159,52 +163,56 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
     const double lp = (p > 0.f) ? log((double)p) : -CUDART_INF;
     const double cd = unit ? 0.0 : 1.4426950408889634074 * (lp - 0.5 * slog);
     const double eps = 9.765625e-04 * 1.015625;
-    double bnn, t, c, al, be;
+    double bnn, c, al, be, numax = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) numax = fmax(numax, fabs(nv[i]));
+    numax = (double)(float)warp_max(numax);          // (the value screen_plane_kernel gets)
     bool capped = false;
     for (;;) {                                       // (at most twice; the same way in every lane)
         double absab = 0.0, bmax = 0.0, cmax = 0.0;
         bnn = 0.0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const double b = capped ? fmin(bv[i], screen_cap(D)) : bv[i];
+            const double b = capped ? fmin(bv[i], screen_cap(D, numax)) : bv[i];
             bnn += b * nv[i] * nv[i];
             absab += 2.0 * b * fabs(nv[i]) + b;
             bmax = fmax(bmax, b);
             cmax = fmax(cmax, fmax(b, 2.0 * b * fabs(nv[i])));
         }
         bnn = warp_sum(bnn); absab = warp_sum(absab); bmax = warp_max(bmax); cmax = warp_max(cmax);
-        t = 1.0;
-        if (cmax > 0.0 && isfinite(cmax)) t = exp2(floor(log2(cmax)) - 9.0);
         c = cd - bnn;
-        al = eps * bnn + 5.9604644775390625e-08 * absab + t * 2.98023223876953125e-08 * 0.5 * D + 2.384185791015625e-07 * fabs(c) + 0.02;
-        be = 2.0 * eps * bmax + t * 2.98023223876953125e-08 * 1.5;
-        if (capped || !(al + be * D > (double)SCR_SHARP)) break;
+        al = eps * bnn + 5.9604644775390625e-08 * absab + 2.98023223876953125e-08 * 0.5 * D + 3.814697265625e-06 * fabs(c) + 0.02;
+        be = 3.0 * eps * bmax + 2.98023223876953125e-08 * 1.5;
+        if (capped || !(al + be * D > (double)SCR_SHARP || cmax > 60000.0)) break;
         capped = true;
     }
     if (lane == 0) {
         if (c2) c2[k] = (float)cd;
         c2d[k] = cd;
         const bool on = p > 0.f && isfinite(c) && isfinite(al) && isfinite(be);
-        prm[k] = make_float4((float)t, on ? (float)c : -CUDART_INF_F, on ? (float)(al * 1.000001) : 0.f, on ? (float)(be * 1.000001) : 0.f);
+        prm[k] = make_float4(on ? (float)c : -CUDART_INF_F, on ? (float)(al * 1.000001) : 0.f, on ? (float)(be * 1.000001) : 0.f, (float)numax);
         key[k] = !on ? CUDART_INF_F : capped ? SCR_CAPPED : (float)(al + be * D);
         if (on) atomicAdd(ctl + SC_ACTIVE, 1);
         if (bad) atomicOr(status, bad);
     }
 }
 
+constexpr int SW_CSLOT = 4096;               // a group's constants: 128 rows of 16 halves
 // Positions of the components in the sweep: ascending by the allowance of a typical point, so that 32 neighbours, which are
 // screened with the largest allowance among them, have similar ones (the capped components come last).  A warp per component:
-// its rank among the keys is its position, and it writes its own row (a sort of the keys in every CTA took 20 us).
+// its rank among the keys is its position, and it writes its own row (a sort of the keys in every CTA took 20 us).  The
+// coefficients are written as the sweep has them in shared memory (screen_group_bytes per group of 128 positions: the constants,
+// then the atoms of 32 dimensions, swizzled), so that a stage is one contiguous copy.
 __global__ void __launch_bounds__(256) screen_plane_kernel(int D, int K, int Kpad, const float* __restrict__ mu,
                                                            const float* __restrict__ w2, const float* __restrict__ sd,
                                                            const float* __restrict__ gd, const float4* __restrict__ prm,
-                                                           const float* __restrict__ key, __half* __restrict__ p, float4* __restrict__ tab,
+                                                           const float* __restrict__ key, unsigned char* __restrict__ img,
                                                            int4* __restrict__ blk, int* __restrict__ comp_of) {
     const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (k >= Kpad) return;
     int pos = k;
     bool on = false, capped = false;
-    float4 q = make_float4(1.f, -CUDART_INF_F, 0.f, 0.f);
+    float4 q = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
     if (k < K) {
         const float mine = __ldg(key + k);
         int before = 0;
@@ -218,41 +226,53 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(int D, int K, int Kpa
         capped = on && mine >= SCR_CAPPED;
         if (on) q = __ldg(prm + k);
     }
+    const int r = pos & 127;
+    unsigned char* grp = img + (size_t)(pos >> 7) * screen_group_bytes(D);
     const int ndim = (D + 7) / 8 * 8;
     for (int d = lane; d < ndim; d += 32) {
         float a = 0.f, b = 0.f;
         if (on && d < D) {
             const float s = __ldg(sd + d);
             double bd = (double)__ldg(w2 + (size_t)k * D + d) / ((double)s * (double)s);
-            if (capped) bd = fmin(bd, screen_cap(D));
+            if (capped) bd = fmin(bd, screen_cap(D, (double)q.w));
             const double nu = ((double)__ldg(mu + (size_t)k * D + d) - (double)__ldg(gd + d)) * (double)s;
-            a = (float)(2.0 * bd * nu / (double)q.x);
-            b = (float)(-bd / (double)q.x);
+            a = (float)(2.0 * bd * nu);
+            b = (float)(-bd);
         }
-        const int cx = 16 * (d >> 3) + (d & 7);
-        __half* o = p + ((size_t)(cx >> 6) * Kpad + pos) * 64 + (cx & 63);
-        o[0] = __float2half_rn(a);
-        o[8] = __float2half_rn(b);
+        // k-step d / 8 holds eight dimensions of u and the same eight of u^2: two 16-byte chunks of a 128-byte row, swizzled
+        unsigned char* o = grp + SW_CSLOT + (d >> 5) * 16384 + r * 128;
+        const int c = 2 * ((d >> 3) & 3);
+        *reinterpret_cast<__half*>(o + ((c ^ (r & 7)) << 4) + 2 * (d & 7)) = __float2half_rn(a);
+        *reinterpret_cast<__half*>(o + (((c + 1) ^ (r & 7)) << 4) + 2 * (d & 7)) = __float2half_rn(b);
     }
     if (lane == 0) {
         comp_of[pos] = on ? k : -1;
-        float* tf = reinterpret_cast<float*>(tab) + (size_t)(pos >> 1) * 4 + (pos & 1);
-        tf[0] = q.x;
-        tf[2] = q.y;
+        const float c = fmaxf(q.x, SCR_NEVER);                // (no weight: no mark)
+        const __half h1 = __float2half_rn(c / 256.f);
+        const float r1 = c - 256.f * __half2float(h1);
+        const __half h2 = __float2half_rn(r1), h3 = __float2half_rn(r1 - __half2float(h2));
+        uint4* pc = reinterpret_cast<uint4*>(grp) + 2 * r;
+        const int sw = (r >> 2) & 1;
+        pc[sw] = make_uint4((uint32_t)__half_as_ushort(h1) | ((uint32_t)__half_as_ushort(h2) << 16), __half_as_ushort(h3), 0u, 0u);
+        pc[sw ^ 1] = make_uint4(0u, 0u, 0u, 0u);
         // the largest allowances of the block of 32 positions (non-negative floats order as integers), and whether it holds a
         // capped component (then it has no lower bound)
         int* bk = reinterpret_cast<int*>(blk + (pos >> 5));
-        atomicMax(bk, __float_as_int(q.z));
-        atomicMax(bk + 1, __float_as_int(q.w));
+        atomicMax(bk, __float_as_int(q.y));
+        atomicMax(bk + 1, __float_as_int(q.z));
         if (capped) bk[2] = 1;
     }
 }
 
 // ------------------------------------------------------------------------------------------------------------------
-// X -> fp16 plane [u | u^2], k-step interleaved (8 dimensions of u, the same 8 of u^2), atom by atom, and |u|^2.  L lanes per
-// row, 8 dimensions each.  Bound by memory: 4 D bytes in, 4 D out.
+// X -> fp16 plane of u, rows of `chunks` 16-byte chunks (8 dimensions each), and |u|^2.  Chunk c of row r sits at place
+// screen_place(c, r): the sweep reads a row per lane from shared memory, and eight neighbouring rows' chunks c then lie in
+// different banks.  L lanes per row, 8 dimensions each.  Bound by memory: 4 D bytes in, 2 D out.
+__host__ __device__ __forceinline__ int screen_chunks(int D) { return D <= 32 ? 4 : D <= 64 ? 8 : 16; }
+__device__ __forceinline__ int screen_place(int c, int row, int chunks) { return chunks == 4 ? c ^ ((row >> 1) & 3) : c ^ (row & 7); }
+
 template <int L>
-__global__ void __launch_bounds__(256) screen_transform_kernel(const float* __restrict__ X, int64_t n, int D, const float* __restrict__ sd,
+__global__ void __launch_bounds__(256) screen_transform_kernel(const float* __restrict__ X, int64_t n, int D, int chunks, const float* __restrict__ sd,
                                                                const float* __restrict__ gd, unsigned char* __restrict__ y,
                                                                float* __restrict__ n2, int* __restrict__ ctl, int* __restrict__ status) {
     if (blockIdx.x == 0 && threadIdx.x < 3) ctl[SC_MARKS + threadIdx.x] = 0;
@@ -277,7 +297,7 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
     auto store = [&](int64_t row, const float (&x)[8]) {
         float nrm = 0.f;
         bool far = false;
-        uint32_t xh[4], qh[4];
+        uint32_t xh[4];
 #pragma unroll
         for (int j = 0; j < 8; j += 2) {
             bad |= !(fabsf(x[j]) <= 3.0e38f) || !(fabsf(x[j + 1]) <= 3.0e38f);
@@ -285,21 +305,15 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
             far |= !(fabsf(u0) <= 240.f) || !(fabsf(u1) <= 240.f);
             u0 = fminf(fmaxf(u0, -240.f), 240.f);
             u1 = fminf(fmaxf(u1, -240.f), 240.f);
-            const float q0 = u0 * u0, q1 = u1 * u1;
-            nrm += q0 + q1;
-            const __half2 h = __floats2half2_rn(u0, u1), sq = __floats2half2_rn(q0, q1);
+            nrm = fmaf(u0, u0, fmaf(u1, u1, nrm));
+            const __half2 h = __floats2half2_rn(u0, u1);
             xh[j / 2] = *reinterpret_cast<const uint32_t*>(&h);
-            qh[j / 2] = *reinterpret_cast<const uint32_t*>(&sq);
         }
         if (far) nrm = CUDART_INF_F;                 // (a clamped coordinate: no bound holds, the row is evaluated in full)
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
         if (row >= n) return;
-        if (d0 < D) {
-            uint4* o = reinterpret_cast<uint4*>(y + ((size_t)(l >> 2) * SCR_PIECE + row) * 128 + (l & 3) * 32);
-            o[0] = make_uint4(xh[0], xh[1], xh[2], xh[3]);
-            o[1] = make_uint4(qh[0], qh[1], qh[2], qh[3]);
-        }
+        if (d0 < D) *reinterpret_cast<uint4*>(y + ((size_t)row * chunks + screen_place(l, (int)row, chunks)) * 16) = make_uint4(xh[0], xh[1], xh[2], xh[3]);
         if (l == 0) n2[row] = nrm * 1.0001f;
     };
     // (every lane of a warp takes the same number of steps: the row sums are shuffles; two rows' loads in flight)
@@ -316,18 +330,20 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
 
 // ------------------------------------------------------------------------------------------------------------------
 // Sweep
-constexpr int SW_THREADS = 320;              // 8 softmax warps, producer warp, MMA warp
+constexpr int SW_THREADS = 352;              // 8 softmax warps, producer warp, an MMA warp per half of the tile
 constexpr int SW_PRODUCER = 8, SW_MMA = 9;
-constexpr int SW_YSLOT = 32768, SW_YS = 4;   // atoms of 256 points
-constexpr int SW_PSLOT = 16384, SW_PS = 4;   // atoms of 128 components
-constexpr int SW_ENT = 14;                   // groups of 32 components a point can have marks in
-constexpr int SW_POFF = SW_YS * SW_YSLOT;
-constexpr int SW_EOFF = SW_POFF + SW_PS * SW_PSLOT;
-constexpr int SW_TOFF = SW_EOFF + SW_ENT * 256 * 8;      // tables: 2 x (64 float4 + 4 float2)
-constexpr int SW_BOFF = SW_TOFF + 2 * 1088;
+constexpr int SW_PSLOT = 32768, SW_PS = 4;   // coefficient stages: two atoms of 128 components
+constexpr int SW_ENT = 10;                   // blocks of 32 components a point can have marks in: in shared memory,
+constexpr int SW_SPILL = 22;                 // and, rarely needed, in global memory
+constexpr int SW_UOFF = SW_PS * SW_PSLOT;    // the next tile's rows of u (256 x 16 chunks bytes), then the slots of the constants
+constexpr int SW_UC = 65536 + 2 * SW_CSLOT;  // (16 chunks: two groups in flight; at most 8 chunks: half the rows, four groups)
+constexpr int SW_AOFF = SW_UOFF + SW_UC;     // the points' side of the constants: 128 rows (256, 1, 1, 0, ...)
+constexpr int SW_EOFF = SW_AOFF + 4096;
+constexpr int SW_TOFF = SW_EOFF + SW_ENT * 256 * 8;      // allowances of every block
+constexpr int SW_BOFF = SW_TOFF + SCR_MAX_K / 32 * 8;
 constexpr int SW_SMEM = SW_BOFF + 256 + 1024;
-enum { SB_PFULL = 0, SB_PEMPTY = SB_PFULL + SW_PS, SB_YFULL = SB_PEMPTY + SW_PS, SB_YEMPTY = SB_YFULL + SW_YS, SB_LFULL = SB_YEMPTY + SW_YS,
-       SB_LEMPTY = SB_LFULL + 2, SB_FINAL = SB_LEMPTY + 2, SB_COUNT };
+enum { SB_PFULL = 0, SB_PEMPTY = SB_PFULL + SW_PS, SB_UFULL = SB_PEMPTY + SW_PS, SB_UEMPTY, SB_AFULL, SB_LFULL = SB_AFULL + 2,
+       SB_LEMPTY = SB_LFULL + 2, SB_FINAL = SB_LEMPTY + 2, SB_COUNT = SB_FINAL + 2 };
 static_assert(SB_COUNT * 8 <= 256, "barriers");
 static_assert(SW_SMEM <= 232448, "shared memory");
 
@@ -335,9 +351,11 @@ static_assert(SW_SMEM <= 232448, "shared memory");
 __device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b)); return r; }
 __device__ __forceinline__ float lo2(uint64_t a) { return __uint_as_float((uint32_t)a); }
 __device__ __forceinline__ float hi2(uint64_t a) { return __uint_as_float((uint32_t)(a >> 32)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+// Operand of one k-step: rows of 32 bytes, 32-byte swizzle, groups of eight rows 256 bytes apart.
+__device__ __forceinline__ uint64_t make_desc32(uint32_t saddr) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
+}
 // The wait for a load of accumulators that is in flight while others are worked on: its registers go through the wait, so that
 // nothing that uses them can be placed before it.
 __device__ __forceinline__ void tmem_wait(uint32_t (&v)[32]) {
@@ -351,25 +369,38 @@ __device__ __forceinline__ float max3(float a, float b, float c) { float r; asm(
 struct SweepParams {
     int64_t n;
     int KA, KS, NG;          // atoms and k-steps of the contraction, groups of 128 components
+    int chunks;              // 16-byte chunks of a row of u
+    const unsigned char* y;
+    const unsigned char* img;
+    int gbytes;              // of the image of a group
     float margin;
-    const float4* tab;
     const int4* blk;
-    const int* comp_of;
     const float* n2;
     unsigned* pt_off;
     int* pt_cnt;
-    unsigned short* ids;
+    uint2* words;
+    unsigned long long* spill;
     int* ovf;
     int* ctl;
     int* status;
 };
 
-// Tile = 256 points, two MMAs of M = 128 per coefficient atom: a tile of 128 would need the coefficients twice as often (64
-// bytes per cycle and SM at D = 128, about what L2 delivers).  An accumulator buffer is 128 components x 2 halves of the tile;
-// two buffers alternate, so the softmax warps read one group while the tensor cores form the next.  MMA time per group of 128
-// components: 2 x ceil(D / 8) x 64.5 cycles; softmax: about 170 instructions per 32 values.
+static_assert(SW_ENT + SW_SPILL <= 32, "a mask of a point's entries");
+static_assert(SW_SPILL == SCR_SPILL, "room for the spilled entries");
+// Tile = 256 points in two halves of 128 TMEM lanes, a thread per point.  The points' operand [u | u^2] lives in TENSOR MEMORY
+// (columns 256 + 128 h of half h; the squares are formed when it is written), so that shared memory has only the coefficients to
+// deliver: with both operands there its bandwidth alone (8 KB per MMA of 64 cycles, besides the incoming stages) held the sweep to
+// half the tensor cores' rate.  Coefficients come as 1-D bulk copies of an image that screen_plane_kernel laid out swizzled, in
+// stages of 32 KB.  Per group of 128 components the tensor cores form half 0 (columns 0-127) and half 1 (128-255) from the same
+// stages; a group's constants are one more product, of 16 columns.  A group's accumulators go into registers at once (128 of
+// them), so that the next group of the half is formed while they are worked through, about 75 instructions per 32 values.  When
+// the last group of a tile has been formed, the half's operand is replaced by the next tile's rows, which wait in shared memory,
+// before those accumulators are read.
+// MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles, 65 us per 2^18 points at D = 128, K = 1024; it takes 115 us: the two
+// halves' MMA and softmax warps wait for one another (a thread that reads its 128 values holds the half's accumulators up, and
+// tensor memory has no room for a second set beside the operands).  126 us with one MMA warp for both halves, 142 with its votes.
 __global__ void __launch_bounds__(SW_THREADS, 1)
-screen_sweep_kernel(const SweepParams p, const __grid_constant__ CUtensorMap tm_y, const __grid_constant__ CUtensorMap tm_p) {
+screen_sweep_kernel(const SweepParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     __shared__ uint32_t tmem_base_s;
@@ -380,19 +411,33 @@ screen_sweep_kernel(const SweepParams p, const __grid_constant__ CUtensorMap tm_
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t ntiles = (p.n + SCR_TILE - 1) / SCR_TILE;
     const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    const int KA = p.KA, NG = p.NG;
+    const int NG = p.NG, spg = (p.KA + 1) >> 1, cslots = SW_PS / spg;      // stages per group; groups in flight
+    unsigned char* cons = smem + SW_UOFF + 256 * 16 * p.chunks;            // [cslots][4096]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SW_BOFF);
     auto BAR = [&](int i) { return smem_u32(&bars[i]); };
     if (tid == 0) {
         abort_s = 0;
         drain_s = 0;
-        for (int i = 0; i < SB_COUNT; ++i) bar_init(BAR(i), (i == SB_LEMPTY || i == SB_LEMPTY + 1) ? 256 : 1);
+        for (int i = 0; i < SB_COUNT; ++i) {
+            const bool wg = (i >= SB_AFULL && i < SB_AFULL + 2) || (i >= SB_LEMPTY && i < SB_LEMPTY + 2);
+            const bool both = i >= SB_PEMPTY && i < SB_PEMPTY + SW_PS;           // (released by the MMA warps of both halves)
+            bar_init(BAR(i), i == SB_UEMPTY ? 256 : wg ? 128 : both ? 2 : 1);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == SW_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (tid < NG * 4) {
+        const int4 q = __ldg(p.blk + tid);
+        reinterpret_cast<float2*>(smem + SW_TOFF)[tid] = make_float2(q.z ? -__int_as_float(q.x) : __int_as_float(q.x), __int_as_float(q.y));      // (sign: no lower bound)
+    }
+    if (tid < 256) {                                         // rows of 32 bytes, 32-byte swizzle (16-byte chunk ^ bit 2 of the row)
+        const int r = tid >> 1, c = (tid & 1) ^ ((r >> 2) & 1);
+        reinterpret_cast<uint4*>(smem + SW_AOFF)[tid] = c == 0 ? make_uint4(0x3C005C00u, 0x00003C00u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    fence_async_smem();
     fence_before();
     __syncthreads();
     fence_after();
@@ -402,241 +447,296 @@ screen_sweep_kernel(const SweepParams p, const __grid_constant__ CUtensorMap tm_
         // =========================== softmax warps: thread = TMEM lane = point ===========================
         const int half = warp >> 2;
         const uint32_t lane_addr = ((uint32_t)((warp & 3) * 32)) << 16;
-        unsigned long long* ent = reinterpret_cast<unsigned long long*>(smem + SW_EOFF) + tid;        // entry e at ent[256 e]
+        const uint32_t col = tmem + half * 128 + lane_addr, acol = tmem + 256 + half * 128 + lane_addr;
+        unsigned long long* ent_s = reinterpret_cast<unsigned long long*>(smem + SW_EOFF) + tid;
+        unsigned long long* ent_g = p.spill + (size_t)blockIdx.x * 256 * SW_SPILL + tid;
+        auto ent = [&](int e) -> unsigned long long& { return e < SW_ENT ? ent_s[256 * e] : ent_g[256 * (e - SW_ENT)]; };
+        const uint4* urow = reinterpret_cast<const uint4*>(smem + SW_UOFF) + (size_t)tid * p.chunks;
         uint32_t gi = 0;                                     // groups processed (all tiles)
         int marks = 0;
-        float4 nt = make_float4(0.f, 0.f, 0.f, 0.f);
-        float2 nb = make_float2(0.f, 0.f);
-        auto table_load = [&](int g) {
-            if (tid < 64) nt = __ldg(p.tab + g * 64 + tid);
-            else if (tid < 68) {
-                const int4 q = __ldg(p.blk + g * 4 + tid - 64);
-                nb = make_float2(q.z ? -__int_as_float(q.x) : __int_as_float(q.x), __int_as_float(q.y));      // (sign: no lower bound)
+        const float2* blk = reinterpret_cast<const float2*>(smem + SW_TOFF);
+        // this thread's row of tile i (in shared memory) -> the half's operand in tensor memory
+        auto operand = [&](int64_t i) {
+            const bool got = bar_wait(BAR(SB_UFULL), (uint32_t)(i & 1), abort_flag, p.status, false);
+            if (__all_sync(0xffffffffu, got)) {
+#pragma unroll 1
+                for (int z = 0; z < p.KA; z += 2) {          // (eight k-steps' loads in flight)
+                    uint4 v[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        v[j] = (4 * z + j < p.KS) ? urow[screen_place(4 * z + j, tid, p.chunks)] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        uint32_t w[32];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t q[4] = {v[4 * y + j].x, v[4 * y + j].y, v[4 * y + j].z, v[4 * y + j].w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const __half2 h = *reinterpret_cast<const __half2*>(&q[e]);
+                                const __half2 sq = __hmul2(h, h);
+                                w[8 * j + e] = q[e];
+                                w[8 * j + 4 + e] = *reinterpret_cast<const uint32_t*>(&sq);
+                            }
+                        }
+                        tmem_st32(acol + (z + y) * 32, w);   // (beyond the last atom: zeros into columns of this operand)
+                    }
+                }
+                tmem_wait_st();
             }
+            fence_before();
+            bar_arrive(BAR(SB_UEMPTY));
+            bar_arrive(BAR(SB_AFULL + half));
         };
-        auto table_store = [&](uint32_t b) {
-            unsigned char* t = smem + SW_TOFF + b * 1088;
-            if (tid < 64) reinterpret_cast<float4*>(t)[tid] = nt;
-            else if (tid < 68) reinterpret_cast<float2*>(t + 1024)[tid - 64] = nb;
+        float nrm_next = 0.f;
+        auto norm_load = [&](int64_t i) {
+            const int64_t r = (blockIdx.x + i * gridDim.x) * SCR_TILE + tid;
+            nrm_next = (i < ntl && r < p.n) ? __ldg(p.n2 + r) : 0.f;
         };
+        if (ntl > 0) {
+            norm_load(0);
+            operand(0);
+        }
         for (int64_t i = 0; i < ntl; ++i) {
             const int64_t wrow = (blockIdx.x + i * gridDim.x) * SCR_TILE + warp * 32;       // first row of this warp
             const int64_t row = wrow + lane;
             const bool in = row < p.n;
-            const float nrm = in ? __ldg(p.n2 + row) : 0.f;
+            const float nrm = nrm_next;
             float thr = -CUDART_INF_F;                       // the largest lower bound so far
             int ne = 0;
             float lost = -CUDART_INF_F;                      // largest upper bound of a block with marks that found no room
-            // 32 accumulators of the point: approximate values l = t acc + c, two at a time; the block's largest; marks.
-            auto block = [&](const uint32_t (&v)[32], int bn, const float4* t4, float2 ab) {
-                uint64_t l[16];
-                float mx[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+            // 32 accumulators of the point = approximate values: the block's largest; marks.
+            auto block = [&](const uint32_t (&v)[32], int bn) {
+                float mx[4];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(t4 + j);      // same address in every lane
-                    l[j] = fma2(pack2(v[2 * j], v[2 * j + 1]), t.x, t.y);
-                    mx[j & 3] = max3(mx[j & 3], lo2(l[j]), hi2(l[j]));
+                for (int j = 0; j < 4; ++j) {
+                    mx[j] = max3(__uint_as_float(v[8 * j]), __uint_as_float(v[8 * j + 1]), __uint_as_float(v[8 * j + 2]));
+                    mx[j] = max3(mx[j], __uint_as_float(v[8 * j + 3]), __uint_as_float(v[8 * j + 4]));
+                    mx[j] = max3(mx[j], __uint_as_float(v[8 * j + 5]), __uint_as_float(v[8 * j + 6]));
                 }
+                mx[0] = max3(mx[0], __uint_as_float(v[7]), __uint_as_float(v[15]));
+                mx[1] = max3(mx[1], __uint_as_float(v[23]), __uint_as_float(v[31]));
+                const float2 ab = blk[bn];
                 const float bmax = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]), E = fmaf(ab.y, nrm, fabsf(ab.x));
                 if (!(ab.x < 0.f)) thr = fmaxf(thr, bmax - E);
                 const float cut = thr - p.margin - E;
-                if (in && bmax >= cut && bmax > -CUDART_INF_F) {
+                if (in && bmax >= cut && bmax > 0.5f * SCR_NEVER) {
                     // bit j of the mask: value j reaches the cut (the sign of l - cut, shifted in from the top)
                     const uint64_t nc = pack2(__float_as_uint(-cut), __float_as_uint(-cut));
                     unsigned mask = 0;
 #pragma unroll
                     for (int j = 15; j >= 0; --j) {
-                        const uint64_t d = add2(l[j], nc);
+                        const uint64_t d = add2(pack2(v[2 * j], v[2 * j + 1]), nc);
                         mask = __funnelshift_l(__float_as_uint(hi2(d)), mask, 1);
                         mask = __funnelshift_l(__float_as_uint(lo2(d)), mask, 1);
                     }
                     mask = ~mask;
-                    if (ne == SW_ENT) {                      // drop what the bound found meanwhile rules out
+                    if (ne == SW_ENT + SW_SPILL) {           // drop what the bound found meanwhile rules out
                         int m = 0;
-                        for (int e = 0; e < SW_ENT; ++e) {
-                            const unsigned long long w = ent[256 * e];
-                            if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= thr - p.margin) ent[256 * m++] = w;
+                        for (int e = 0; e < SW_ENT + SW_SPILL; ++e) {
+                            const unsigned long long w = ent(e);
+                            if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= thr - p.margin) ent(m++) = w;
                         }
                         ne = m;
                     }
                     const float ub = bmax + E;
-                    if (ne < SW_ENT) {
+                    if (ne < SW_ENT + SW_SPILL) {
                         // the block's largest upper bound, rounded up to the 24 bits that share a word with its number
                         const unsigned ubits = (__float_as_uint(ub + fabsf(ub) * 1e-4f + 1e-3f) & ~255u) | (unsigned)bn;
-                        ent[256 * ne++] = ((unsigned long long)ubits << 32) | mask;
+                        ent(ne++) = ((unsigned long long)ubits << 32) | mask;
                     } else {
                         lost = fmaxf(lost, ub);              // (harmless if the final bound rules the block out)
                     }
                 }
             };
-            table_load(0);
-            table_store(gi & 1);
             for (int g = 0; g < NG; ++g, ++gi) {
-                const uint32_t buf = gi & 1;
-                named_bar_sync(1, 256);                      // the group's table is in place, the other one free
-                if (g + 1 < NG) table_load(g + 1);
-                const bool got = bar_wait(BAR(SB_LFULL + buf), (gi >> 1) & 1u, abort_flag, p.status, false);
+                const bool last = g + 1 == NG;
+                if (last) norm_load(i + 1);
+                const bool got = bar_wait(BAR(SB_LFULL + half), gi & 1u, abort_flag, p.status, false);
                 const bool ok = __all_sync(0xffffffffu, got);
                 fence_after();
-                const float4* tab = reinterpret_cast<const float4*>(smem + SW_TOFF + buf * 1088);
-                const float2* blk = reinterpret_cast<const float2*>(smem + SW_TOFF + buf * 1088 + 1024);
-                if (ok) {
-                    const uint32_t col = tmem + buf * 256 + half * 128 + lane_addr;
-                    uint32_t va[32], vb[32];
-                    tmem_ld32(col, va);
-                    tmem_wait(va);
-                    tmem_ld32(col + 32, vb);
-                    block(va, g * 4, tab, blk[0]);
-                    tmem_wait(vb);
-                    tmem_ld32(col + 64, va);
-                    block(vb, g * 4 + 1, tab + 16, blk[1]);
-                    tmem_wait(va);
-                    tmem_ld32(col + 96, vb);
-                    block(va, g * 4 + 2, tab + 32, blk[2]);
-                    tmem_wait(vb);
-                    block(vb, g * 4 + 3, tab + 48, blk[3]);
-                }
+                if (last && i + 1 < ntl) operand(i + 1);     // (the tile's last products are done: its operand is free)
+                // the whole group into registers: the tensor cores may overwrite the columns while it is worked through
+                uint32_t v0[32], v1[32], v2[32], v3[32];
+                tmem_ld32(col, v0);
+                tmem_ld32(col + 32, v1);
+                tmem_ld32(col + 64, v2);
+                tmem_ld32(col + 96, v3);
+                tmem_wait(v0); tmem_wait(v1); tmem_wait(v2); tmem_wait(v3);
                 fence_before();
-                bar_arrive(BAR(SB_LEMPTY + buf));
-                if (g + 1 < NG) table_store(buf ^ 1);
-            }
-            // the point's list: what the final bound leaves
-            int cnt = 0;
-            const float fin = thr - p.margin;
-            bool over = !(nrm < CUDART_INF_F) || lost >= fin && lost > -CUDART_INF_F;
-            if (in && !over)
-                for (int e = 0; e < ne; ++e) {
-                    const unsigned long long w = ent[256 * e];
-                    if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= fin) cnt += __popc((unsigned)w);
+                bar_arrive(BAR(SB_LEMPTY + half));
+                if (ok) {
+                    block(v0, g * 4);
+                    block(v1, g * 4 + 1);
+                    block(v2, g * 4 + 2);
+                    block(v3, g * 4 + 3);
                 }
-            int inc = cnt;
+            }
+            // the point's list: the words (block of 32 positions, mask) that the final bound leaves
+            int cnt = 0, nw = 0;
+            const float fin = thr - p.margin;
+            bool over = !(nrm < CUDART_INF_F) || (lost >= fin && lost > -CUDART_INF_F);
+            // (the entries in shared memory all at once: one after the other, each waited for, they took ten times as long,
+            // and the tensor cores waited with them)
+            unsigned long long we[SW_ENT];
+            unsigned keep = 0;
+#pragma unroll
+            for (int e = 0; e < SW_ENT; ++e) we[e] = ent_s[256 * e];
+#pragma unroll
+            for (int e = 0; e < SW_ENT; ++e)
+                if (e < ne && __uint_as_float((unsigned)(we[e] >> 32) & ~255u) >= fin) {
+                    cnt += __popc((unsigned)we[e]);
+                    keep |= 1u << e;
+                }
+            for (int e = SW_ENT; e < ne; ++e) {
+                const unsigned long long w = ent(e);
+                if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= fin) {
+                    cnt += __popc((unsigned)w);
+                    keep |= 1u << e;
+                }
+            }
+            if (!in || over) cnt = 0, keep = 0;
+            nw = __popc(keep);
+            if (cnt == 0 || nw > 15) over = true;                       // (a point further from everything than a float16 sum can tell)
+            if (over) cnt = nw = 0, keep = 0;
+            int inc = cnt | (nw << 16);                      // running sums of both over the warp
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int u = __shfl_up_sync(0xffffffffu, inc, o);
                 if (lane >= o) inc += u;
             }
-            if (inc > 32 * SCR_SLOTS) over = true;
+            if ((inc & 0xffff) > 32 * SCR_SLOTS || (inc >> 16) > 32 * SCR_WORDS) over = true;
             if (in && !*abort_flag) {
-                unsigned o = (unsigned)(wrow * SCR_SLOTS) + (unsigned)(inc - cnt);
-                p.pt_off[row] = o;
-                p.pt_cnt[row] = over ? 0 : cnt;
+                const int wo = (inc >> 16) - nw;
+                p.pt_off[row] = (unsigned)(wrow * SCR_SLOTS) + (unsigned)((inc & 0xffff) - cnt);
+                p.pt_cnt[row] = (over || cnt == 0) ? 0 : (wo << 16) | (nw << 12) | cnt;
                 if (over) {
                     p.ovf[atomicAdd(p.ctl + SC_OVF, 1)] = (int)row;
                 } else {
                     marks += cnt;
-                    for (int e = 0; e < ne; ++e) {
-                        const unsigned long long w = ent[256 * e];
-                        if (!(__uint_as_float((unsigned)(w >> 32) & ~255u) >= fin)) continue;
-                        unsigned mask = (unsigned)w;
-                        const int base = (int)((w >> 32) & 255u) * 32;
-                        while (mask) {
-                            const int j = __ffs(mask) - 1;
-                            mask &= mask - 1;
-                            p.ids[o++] = (unsigned short)__ldg(p.comp_of + base + j);
+                    uint2* o = p.words + wrow * SCR_WORDS + wo;
+#pragma unroll
+                    for (int e = 0; e < SW_ENT; ++e)
+                        if (keep >> e & 1u) *o++ = make_uint2((unsigned)we[e], (unsigned)(we[e] >> 32) & 255u);
+                    for (int e = SW_ENT; e < ne; ++e)
+                        if (keep >> e & 1u) {
+                            const unsigned long long w = ent(e);
+                            *o++ = make_uint2((unsigned)w, (unsigned)(w >> 32) & 255u);
                         }
-                    }
                 }
             }
-            named_bar_sync(2, 256);                          // (the tables are rewritten by the next tile)
         }
         marks = __reduce_add_sync(0xffffffffu, marks);
         if (lane == 0 && marks > 0) atomicAdd(p.ctl + SC_MARKS, marks);
     } else if (warp == SW_PRODUCER) {
         // =========================== producer warp (TMA) ===========================
-        uint32_t ps = 0, ya = 0;                             // stages and atoms requested so far
+        const uint32_t ubytes = 256u * 16u * (uint32_t)p.chunks;
+        uint32_t ps = 0, ut = 0, cslot = 0;                  // stages and tiles requested so far; slot of the group's constants
         bool ok = true;
-        const uint64_t keep = l2_policy_evict_last();
         auto wait_slot = [&](int bar, uint32_t parity) -> bool {
             uint32_t w = 1;
             if (lane == 0) w = bar_wait(BAR(bar), parity, abort_flag, p.status, false) ? 1u : 0u;
             return __shfl_sync(0xffffffffu, w, 0) != 0u;
         };
-        for (int64_t i = 0; i < ntl && ok; ++i) {
-            const int32_t row0 = (int32_t)((blockIdx.x + i * gridDim.x) * SCR_TILE);
-            for (int g = 0; g < NG && ok; ++g)
-                for (int z = 0; z < KA && ok; ++z) {
-                    if (g == 0) {
-                        const uint32_t slot = ya % SW_YS;
-                        if (ya >= SW_YS) ok = wait_slot(SB_YEMPTY + slot, (ya / SW_YS - 1) & 1u);
-                        if (!ok) break;
-                        if (elect_one()) {
-                            bar_expect_tx(BAR(SB_YFULL + slot), SW_YSLOT);
-                            tma_load_3d(smem_u32(smem + slot * SW_YSLOT), &tm_y, 0, row0, z, BAR(SB_YFULL + slot));
-                        }
-                        __syncwarp();
-                        ++ya;
-                    }
-                    const uint32_t slot = ps % SW_PS;
+        auto bulk = [&](unsigned char* dst, const unsigned char* src, uint32_t bytes, uint32_t bar) {
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(bar) : "memory");
+        };
+        auto load_rows = [&](int64_t i) {
+            if (elect_one()) {
+                const unsigned char* src = p.y + (size_t)((blockIdx.x + i * gridDim.x) * SCR_TILE) * p.chunks * 16;
+                bar_expect_tx(BAR(SB_UFULL), ubytes);
+                bulk(smem + SW_UOFF, src, ubytes, BAR(SB_UFULL));
+            }
+            __syncwarp();
+            ++ut;
+        };
+        if (ntl > 0) load_rows(0);
+        for (int64_t i = 0; i < ntl && ok; ++i)
+            for (int g = 0; g < NG && ok; ++g) {
+                for (int z = 0; z < spg && ok; ++z) {
+                    const uint32_t slot = ps % SW_PS;        // (a power of two)
                     if (ps >= SW_PS) ok = wait_slot(SB_PEMPTY + slot, (ps / SW_PS - 1) & 1u);
                     if (!ok) break;
                     if (elect_one()) {
-                        bar_expect_tx(BAR(SB_PFULL + slot), SW_PSLOT);
-                        tma_load_3d_hint(smem_u32(smem + SW_POFF + slot * SW_PSLOT), &tm_p, 0, g * 128, z, BAR(SB_PFULL + slot), keep);
-                        // the next tile's atoms into L2 while this one is worked on
-                        if (g == 0 && i + 1 < ntl) tma_prefetch_3d(&tm_y, 0, (int32_t)(row0 + (int64_t)gridDim.x * SCR_TILE), z);
+                        const unsigned char* src = p.img + (size_t)g * p.gbytes;
+                        const uint32_t bytes = min(p.KA - 2 * z, 2) * 16384u;
+                        bar_expect_tx(BAR(SB_PFULL + slot), bytes + (z == 0 ? SW_CSLOT : 0));
+                        if (z == 0) bulk(cons + cslot * SW_CSLOT, src, SW_CSLOT, BAR(SB_PFULL + slot));
+                        bulk(smem + slot * SW_PSLOT, src + SW_CSLOT + z * SW_PSLOT, bytes, BAR(SB_PFULL + slot));
                     }
                     __syncwarp();
                     ++ps;
                 }
-        }
+                if (++cslot == (uint32_t)cslots) cslot = 0;
+                // the next tile's rows as soon as both halves have taken this tile's (which they do before its first products);
+                // no stage waits for that except behind the tile's last one
+                if (ok && ut == (uint32_t)(i + 1) && i + 1 < ntl) {
+                    uint32_t free_now = (g + 1 == NG) ? 1u : 0u;
+                    if (free_now) ok = wait_slot(SB_UEMPTY, (uint32_t)(i & 1));
+                    else {
+                        if (lane == 0) free_now = bar_test(BAR(SB_UEMPTY), (uint32_t)(i & 1)) ? 1u : 0u;
+                        free_now = __shfl_sync(0xffffffffu, free_now, 0);
+                    }
+                    if (ok && free_now) load_rows(i + 1);
+                }
+            }
         // the loads in flight must have landed before the CTA may exit, also after an abort
         if (!ok || *abort_flag) {
             for (uint32_t h = (ps > SW_PS ? ps - SW_PS : 0); h < ps; ++h) {
                 if (lane == 0) bar_wait(BAR(SB_PFULL + h % SW_PS), (h / SW_PS) & 1u, drain_flag, p.status, false);
                 __syncwarp();
             }
-            for (uint32_t h = (ya > SW_YS ? ya - SW_YS : 0); h < ya; ++h) {
-                if (lane == 0) bar_wait(BAR(SB_YFULL + h % SW_YS), (h / SW_YS) & 1u, drain_flag, p.status, false);
-                __syncwarp();
-            }
+            if (ut > 0 && lane == 0) bar_wait(BAR(SB_UFULL), (ut - 1) & 1u, drain_flag, p.status, false);
+            __syncwarp();
         }
     } else {
-        // =========================== MMA warp ===========================
-        const uint32_t idesc = make_idesc(128, 128, 0);
-        const uint64_t dy = make_desc(smem_u32(smem), 16, 1024), dp = make_desc(smem_u32(smem + SW_POFF), 16, 1024);
-        auto wait_all = [&](int bar, uint32_t parity) -> bool {
-            uint32_t ok = 1;
-            if (lane == 0) ok = bar_wait(BAR(bar), parity, abort_flag, p.status, false) ? 1u : 0u;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            fence_after();
-            return ok != 0u;
-        };
-        uint32_t ps = 0, ya = 0, gi = 0;
-        bool alive = true;
-        for (int64_t i = 0; i < ntl && alive; ++i) {
-            for (int g = 0; g < NG && alive; ++g, ++gi) {
-                const uint32_t buf = gi & 1;
-                if (gi >= 2 && !wait_all(SB_LEMPTY + buf, (gi / 2 - 1) & 1u)) { alive = false; break; }
-                const uint32_t d = tmem + buf * 256;
-                for (int z = 0; z < KA; ++z) {
-                    const uint32_t yslot = (ya + z) % SW_YS, slot = ps % SW_PS;
-                    if (g == 0 && !wait_all(SB_YFULL + yslot, ((ya + z) / SW_YS) & 1u)) { alive = false; break; }
-                    if (!wait_all(SB_PFULL + slot, (ps / SW_PS) & 1u)) { alive = false; break; }
-                    ++ps;
-                    const int nk = (p.KS - 4 * z < 4) ? (p.KS - 4 * z) : 4;
-                    if (elect_one()) {
-                        const uint64_t a = dy + ((yslot * SW_YSLOT) >> 4), b = dp + ((slot * SW_PSLOT) >> 4);
+        // =========================== MMA warps, one per half ===========================
+        // An instruction takes about as long to issue as the tensor cores take for it, and few are queued: every cycle spent
+        // between two of them is idle time of the tensor cores unless the other half's warp fills it.  So there is a warp per
+        // half, one thread of it does all (no votes, no shuffles), and a stage is waited for only when the instructions of the
+        // stage before it have been issued.
+        const int h = warp - SW_MMA;
+        if (elect_one()) {
+            const uint32_t idesc = make_idesc(128, 128, 0);
+            const uint64_t dp = make_desc(smem_u32(smem), 16, 1024);
+            const uint64_t dc = make_desc32(smem_u32(cons)), da = make_desc32(smem_u32(smem + SW_AOFF));
+            const uint32_t d = tmem + h * 128, a = tmem + 256 + h * 128;
+            const uint32_t bars0 = BAR(0);
+            auto wait = [&](int bar, uint32_t parity) -> bool { return bar_wait(bars0 + 8 * bar, parity, abort_flag, p.status, false); };
+            uint32_t slot = 0, parity = 0, cslot = 0;        // of the next stage; of the group's constants
+            uint32_t gi = 0;
+            bool alive = true;
+            for (int64_t i = 0; i < ntl && alive; ++i) {
+                for (int g = 0; g < NG && alive; ++g, ++gi) {
+                    if (g == 0) alive = wait(SB_AFULL + h, (uint32_t)(i & 1));
+                    if (alive && gi >= 1) alive = wait(SB_LEMPTY + h, (gi - 1) & 1u);
+                    for (int z = 0; z < spg && alive; ++z) {
+                        if (!wait(SB_PFULL + slot, parity)) { alive = false; break; }
+                        fence_after();
+                        if (z == 0) mma_ss(d, da, dc + ((cslot * SW_CSLOT) >> 4), idesc, 0u);      // the constants
+                        const int nk = p.KS - 8 * z;         // k-steps of this stage: at most eight
+                        const uint64_t b = dp + ((slot * SW_PSLOT) >> 4);
+                        if (nk >= 8) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (j < nk) {
-                                const uint32_t acc = (z > 0 || j > 0) ? 1u : 0u;
-                                mma_ss(d, a + ((j * 32) >> 4), b + ((j * 32) >> 4), idesc, acc);
-                                mma_ss(d + 128, a + ((16384 + j * 32) >> 4), b + ((j * 32) >> 4), idesc, acc);
-                            }
-                        mma_commit(BAR(SB_PEMPTY + slot));
-                        if (g == NG - 1) mma_commit(BAR(SB_YEMPTY + yslot));
-                        if (z == KA - 1) mma_commit(BAR(SB_LFULL + buf));
+                            for (int j = 0; j < 8; ++j) mma_ts(d, a + z * 64 + j * 8, b + (((j >> 2) * 16384 + (j & 3) * 32) >> 4), idesc, 1u);
+                        } else {
+#pragma unroll
+                            for (int j = 0; j < 7; ++j)
+                                if (j < nk) mma_ts(d, a + z * 64 + j * 8, b + (((j >> 2) * 16384 + (j & 3) * 32) >> 4), idesc, 1u);
+                        }
+                        mma_commit(bars0 + 8 * (SB_PEMPTY + slot));
+                        if (++slot == SW_PS) { slot = 0; parity ^= 1u; }
                     }
-                    __syncwarp();
+                    if (alive) mma_commit(bars0 + 8 * (SB_LFULL + h));
+                    if (++cslot == (uint32_t)cslots) cslot = 0;
                 }
             }
-            ya += KA;
+            mma_commit(bars0 + 8 * (SB_FINAL + h));
+            bar_wait(bars0 + 8 * (SB_FINAL + h), 0, drain_flag, p.status, false);
+            fence_after();
         }
-        if (elect_one()) mma_commit(BAR(SB_FINAL));
         __syncwarp();
-        if (lane == 0) bar_wait(BAR(SB_FINAL), 0, drain_flag, p.status, false);
-        __syncwarp();
-        fence_after();
     }
     fence_before();
     __syncthreads();
@@ -734,14 +834,17 @@ constexpr int EV_VALS = 32 * SCR_SLOTS;
 template <int MODE>
 __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __restrict__ mu,
                                                              const float* __restrict__ w2, const double* __restrict__ c2d,
+                                                             const int* __restrict__ comp_of, int range, int pw,
+                                                             const uint2* __restrict__ words,
                                                              const unsigned* __restrict__ pt_off, int* __restrict__ pt_cnt,
                                                              unsigned short* __restrict__ ids, float* __restrict__ val,
                                                              int* __restrict__ counts, double* __restrict__ ll, float* __restrict__ logp,
                                                              int32_t* __restrict__ idx, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
     extern __shared__ int hist[];                    // [K] (unless MODE == SCREEN_LOGP)
-    __shared__ float v_s[8][EV_VALS];                // values of the warp's pairs, by position in its part of the lists
-    __shared__ unsigned short w_s[8][EV_VALS];       // work list: point (5 bits), position (9 bits)
+    __shared__ float v_s[8][EV_VALS];                // values of the warp's pairs, by place in its part of the lists
+    __shared__ unsigned short k_s[8][EV_VALS];       // their positions in the sweep, then their components
+    __shared__ unsigned short w_s[8][EV_VALS];       // work list: point (5 bits), place (9 bits)
     __shared__ double red[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l8 = lane & 7;
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0);
@@ -780,13 +883,15 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
         return (float)(__ldg(c2d + k) - (double)q);
     };
     double ll_acc = 0.0;
-    for (int it = 0; it < SCR_RANGE / 256; ++it) {
-        const int64_t row0 = (int64_t)blockIdx.x * SCR_RANGE + it * 256 + warp * 32, row = row0 + lane;
+    for (int it = 0; it < range / (8 * pw); ++it) {
+        const int64_t row0 = (int64_t)blockIdx.x * range + (it * 8 + warp) * pw, row = row0 + lane;
         if (row0 >= n) break;
-        const bool in = row < n;
-        const int cnt = in ? pt_cnt[row] : 0;
-        const unsigned off = in ? pt_off[row] : 0u, base = (unsigned)(row0 * SCR_SLOTS);
+        const bool in = lane < pw && row < n;
+        const int64_t part = row0 & ~(int64_t)31;                                // (32 points of the sweep share a part of the lists)
+        const int pc = in ? pt_cnt[row] : 0;
+        const unsigned off = in ? pt_off[row] : 0u, base = (unsigned)(part * SCR_SLOTS);
         const bool listed = off < (unsigned)(SCR_PIECE * SCR_SLOTS);             // (else: a row with a list of its own length)
+        const int cnt = listed ? pc & 4095 : pc, nw = listed ? (pc >> 12) & 15 : 0;
         const bool alone = cnt == 1 && MODE != SCREEN_LOGP;                      // its value is not needed here
         const int todo = (!listed || alone) ? 0 : cnt;
         int inc = todo;
@@ -796,31 +901,52 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             if (lane >= o) inc += u;
         }
         const int total = __shfl_sync(0xffffffffu, inc, 31), p0 = (int)(off - base);
+        int only = 0;
+        {   // the marks one by one
+            const uint2* wd = words + part * SCR_WORDS + (pc >> 16);
+            int q = inc - todo, at = p0;
+            for (int e = 0; e < nw; ++e) {
+                uint2 w = __ldg(wd + e);
+                while (w.x) {
+                    const int pos = (int)w.y * 32 + __ffs(w.x) - 1;
+                    w.x &= w.x - 1;
+                    only = pos;
+                    if (todo > 0) {
+                        k_s[warp][at] = (unsigned short)pos;
+                        w_s[warp][q++] = (unsigned short)((lane << 9) | at);
+                        ++at;
+                    }
+                }
+            }
+        }
+        if (listed && alone) only = __ldg(comp_of + only);
         __syncwarp();
-        for (int j = 0; j < todo; ++j) w_s[warp][inc - todo + j] = (unsigned short)((lane << 9) | (p0 + j));
-        __syncwarp();
+        int w_next = 0, k_next = 0;
+        auto fetch = [&](int s) {                            // (one step ahead of the values: the component's rows wait for it)
+            w_next = w_s[warp][min(s + (lane >> 3), total - 1)];
+            k_next = __ldg(comp_of + k_s[warp][w_next & 511]);
+        };
+        if (total > 0) fetch(0);
         for (int s = 0; s < total; s += 4) {
-            const int item = s + (lane >> 3);
-            const int w = w_s[warp][min(item, total - 1)];
-            const int k = ids[base + (w & 511)];
+            const int w = w_next, k = k_next;
+            __syncwarp();
+            if (s + 4 < total) fetch(s + 4);
             const float l = pair_value(X + (row0 + (w >> 9)) * D, k);
-            if (l8 == 0 && item < total) v_s[warp][w & 511] = l;
+            if (l8 == 0 && s + (lane >> 3) < total) { v_s[warp][w & 511] = l; k_s[warp][w & 511] = (unsigned short)k; }
         }
         __syncwarp();
         float mx = -CUDART_INF_F, sum = 0.f;
-        int best = 0, kept = 0;
-        if (listed && cnt > 0) {
+        int best = only, kept = 0;
+        if (todo > 0) {
             if (MODE == SCREEN_ARGMAX) {
-                best = ids[off];
-                if (!alone) {
-                    mx = v_s[warp][p0];
-                    for (int j = 1; j < cnt; ++j) {
-                        const float l = v_s[warp][p0 + j];
-                        const int k = ids[off + j];
-                        if (l > mx || (l == mx && k < best)) { mx = l; best = k; }
-                    }
+                mx = v_s[warp][p0];
+                best = k_s[warp][p0];
+                for (int j = 1; j < cnt; ++j) {
+                    const float l = v_s[warp][p0 + j];
+                    const int k = k_s[warp][p0 + j];
+                    if (l > mx || (l == mx && k < best)) { mx = l; best = k; }
                 }
-            } else if (!alone) {
+            } else {
                 for (int j = 0; j < cnt; ++j) mx = fmaxf(mx, v_s[warp][p0 + j]);
                 for (int j = 0; j < cnt; ++j) sum += fast_ex2(v_s[warp][p0 + j] - mx);
             }
@@ -896,8 +1022,10 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             if (cnt == 0) {
                 ll_acc += -CUDART_INF;
             } else if (listed && alone) {
+                ids[off] = (unsigned short)only;
                 val[off] = -1.f;
-                atomicAdd(&hist[ids[off]], 1);
+                pt_cnt[row] = 1;
+                if (histogram) atomicAdd(&hist[only], 1);
             } else {
                 ll_acc += (double)mx + (double)log2f(sum);
                 if (listed) {
@@ -905,11 +1033,11 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                     for (int j = 0; j < cnt; ++j) {
                         const float r = fast_ex2(v_s[warp][p0 + j] - lz);
                         if (r >= 9.094947e-13f) {
-                            const unsigned short id = ids[off + j];
+                            const unsigned short id = k_s[warp][p0 + j];
                             ids[off + kept] = id;
                             val[off + kept] = r;
                             ++kept;
-                            atomicAdd(&hist[id], 1);
+                            if (histogram) atomicAdd(&hist[id], 1);
                         }
                     }
                 }
@@ -929,7 +1057,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
         if (tid == 0) {
             double s = 0.0;
             for (int w = 0; w < 8; ++w) s += red[w];
-            ll[blockIdx.x] += s * 0.69314718055994530942;            // one owner per slot: launches add up
+            ll[blockIdx.x] = s * 0.69314718055994530942 + ll[blockIdx.x];      // one owner per slot: launches add up
         }
     }
 }
@@ -1009,9 +1137,9 @@ __global__ void __launch_bounds__(1024) screen_scan_kernel(int* __restrict__ cou
     }
 }
 
-// A CTA per range, a warp per 64 points of it, with cursors of its own: lanes = points, their pairs one after the other, the
+// A CTA per range, a warp per eighth of it (at most 64 points), with cursors of its own: lanes = points, their pairs one after the other, the
 // pairs of one component ranked by lane.  The order is the same in every run.
-__global__ void __launch_bounds__(256) screen_fill_kernel(int64_t n, int K, const unsigned* __restrict__ pt_off, const int* __restrict__ pt_cnt,
+__global__ void __launch_bounds__(256) screen_fill_kernel(int64_t n, int K, int range, const unsigned* __restrict__ pt_off, const int* __restrict__ pt_cnt,
                                                           const unsigned short* __restrict__ ids, const float* __restrict__ val,
                                                           const int* __restrict__ starts, const int* __restrict__ off,
                                                           uint2* __restrict__ srt, const int* __restrict__ ctl) {
@@ -1025,14 +1153,15 @@ __global__ void __launch_bounds__(256) screen_fill_kernel(int64_t n, int K, cons
     for (int k = tid; k < K; k += 256) base[k] = __ldg(off + k) + starts[(size_t)blockIdx.x * K + k];
     for (int k = tid; k < 4 * K2; k += 256) cur32[k] = 0u;
     __syncthreads();
-    const int64_t p0 = (int64_t)blockIdx.x * SCR_RANGE + warp * (SCR_RANGE / 8);
+    const int64_t p0 = (int64_t)blockIdx.x * range + warp * (range / 8);
     int cnt[2];
     unsigned o[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int64_t row = p0 + 32 * h + lane;
-        cnt[h] = row < n ? pt_cnt[row] : 0;
-        o[h] = row < n ? pt_off[row] : 0u;
+        const bool in = 32 * h + lane < range / 8 && row < n;
+        cnt[h] = in ? pt_cnt[row] : 0;
+        o[h] = in ? pt_off[row] : 0u;
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h)
@@ -1213,28 +1342,229 @@ __global__ void __launch_bounds__(1024) screen_reduce_kernel(int D, int K, const
     }
 }
 
-// A plane [atoms][rows][128 bytes] as a 3-D tensor: boxes of box_rows rows of one atom, 128-byte swizzle.
-cudaError_t plane_map(CUtensorMap* tm, void* base, int64_t rows, int atoms, int box_rows) {
-    const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)atoms};
-    const cuuint64_t strides[2] = {128, (cuuint64_t)rows * 128};
-    const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    typedef CUresult (*encode_fn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static encode_fn encode = nullptr;
-    if (!encode) {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        const cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q);
-        if (e != cudaSuccess) return e;
-        if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-        encode = reinterpret_cast<encode_fn>(fn);
+// ------------------------------------------------------------------------------------------------------------------
+// Groups of consecutive points (Fisher vectors): a CTA per group sorts the group's pairs by component (as screen_fill_kernel
+// does for a range), the list in the group's own part of srt.
+__global__ void __launch_bounds__(1024) screen_group_sort_kernel(int K, const int* __restrict__ g_start, const int* __restrict__ g_len,
+                                                                const unsigned* __restrict__ pt_off, const int* __restrict__ pt_cnt,
+                                                                const unsigned short* __restrict__ ids, const float* __restrict__ val,
+                                                                int* __restrict__ g_off, uint2* __restrict__ srt, int* __restrict__ ctl) {
+    if (ctl[SC_DENSE] != 0) return;
+    extern __shared__ int sm[];                      // base [K], then the warps' cursors [W][K rounded up to even] as 16-bit values
+    __shared__ int wsum[32];
+    const int K2 = (K + 1) & ~1;
+    int* base = sm;
+    unsigned* cur32 = reinterpret_cast<unsigned*>(sm + K2);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5, g = blockIdx.x;
+    unsigned short* cur = reinterpret_cast<unsigned short*>(cur32) + (size_t)warp * K2;
+    const int start = g_start[g], len = g_len[g];
+    int* off = g_off + (size_t)g * (K + 1);
+    for (int k = tid; k < W * K2 / 2; k += blockDim.x) cur32[k] = 0u;
+    __syncthreads();
+    const int part = ((len + W - 1) / W + 31) / 32 * 32;
+    const int p0 = start + min(len, warp * part), p1 = start + min(len, (warp + 1) * part);
+    for (int row = p0 + lane; row < p1; row += 32) {
+        const int c = pt_cnt[row];
+        const unsigned o = pt_off[row];
+        for (int j = 0; j < c; ++j) {
+            const int k = ids[o + j];
+            atomicAdd(cur32 + ((size_t)warp * K2 + k) / 2, 1u << (16 * (k & 1)));
+        }
     }
-    const CUresult r = encode(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    __syncthreads();
+    // every component's start: thread t takes the components [t per, (t + 1) per)
+    const int per = (K + (int)blockDim.x - 1) / (int)blockDim.x, k0 = min(K, tid * per), k1 = min(K, k0 + per);
+    int own = 0;
+    for (int k = k0; k < k1; ++k) {
+        unsigned short* q = reinterpret_cast<unsigned short*>(cur32) + k;
+        int c = 0;
+        for (int w = 0; w < W; ++w) { const int v = q[(size_t)w * K2]; q[(size_t)w * K2] = (unsigned short)c; c += v; }
+        base[k] = c;
+        own += c;
+    }
+    int inc = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    int run = inc - own, total = 0;
+    for (int w = 0; w < W; ++w) {
+        if (w < warp) run += wsum[w];
+        total += wsum[w];
+    }
+    const int first = start * SCR_SLOTS;             // the group's part of srt
+    for (int k = k0; k < k1; ++k) {
+        const int c = base[k];
+        base[k] = first + run;
+        off[k] = first + run;
+        run += c;
+    }
+    if (tid == 0) off[K] = first + total;
+    if (total > len * SCR_SLOTS) {                   // (the same in every thread)
+        if (tid == 0) ctl[SC_DENSE] = 1;
+        return;
+    }
+    __syncthreads();
+    for (int r0 = p0; r0 < p1; r0 += 32) {
+        const int row = r0 + lane;
+        const int c = row < p1 ? pt_cnt[row] : 0;
+        const unsigned o = row < p1 ? pt_off[row] : 0u;
+        const int most = __reduce_max_sync(0xffffffffu, (unsigned)c);
+        for (int j = 0; j < most; ++j) {
+            const bool on = j < c;
+            const int k = on ? ids[o + j] : -1;
+            const float r = on ? val[o + j] : 0.f;
+            const unsigned peers = __match_any_sync(0xffffffffu, k);
+            const int rank = __popc(peers & ((1u << lane) - 1u));
+            int q = 0;
+            if (on) q = cur[k];
+            __syncwarp();
+            if (on) {
+                if (rank == 0) cur[k] = (unsigned short)(q + __popc(peers));
+                srt[base[k] + q + rank] = make_uint2((unsigned)row, __float_as_uint(r));
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// Fisher vectors: a warp per (group, component).  With sums about the component's mean,
+//   G_mu = sum r (x - mu) / (T sigma sqrt(pi)),   G_sigma = (sum r (x - mu)^2 / var - sum r) / (T sqrt(2 pi)):
+// nothing cancels.  fp32 sums of 32 pairs at a time, added in fp32.
+__global__ void __launch_bounds__(256) screen_group_stats_kernel(const float* __restrict__ X, int D, int K, int lpr, int groups,
+                                                                 const float* __restrict__ pi, const float* __restrict__ mu,
+                                                                 const float* __restrict__ var, const float* __restrict__ w2,
+                                                                 const double* __restrict__ c2d, const uint2* __restrict__ srt,
+                                                                 const int* __restrict__ g_off, const int* __restrict__ g_len,
+                                                                 float* __restrict__ fv, double* __restrict__ ll, const int* __restrict__ ctl) {
+    if (ctl[SC_DENSE] != 0) return;
+    __shared__ double red[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane % lpr, sub = lane / lpr, rows = 32 / lpr, d0 = 4 * l;
+    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
+    const bool vec_o = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(fv) & 15) == 0);
+    const size_t KD = (size_t)K * D;
+    auto load4 = [&](const float* __restrict__ r, bool v) {
+        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (v) {
+            if (d0 < D) a = __ldg(reinterpret_cast<const float4*>(r + d0));
+        } else {
+            if (d0 < D) a.x = __ldg(r + d0);
+            if (d0 + 1 < D) a.y = __ldg(r + d0 + 1);
+            if (d0 + 2 < D) a.z = __ldg(r + d0 + 2);
+            if (d0 + 3 < D) a.w = __ldg(r + d0 + 3);
+        }
+        return a;
+    };
+    double ll_acc = 0.0;
+    const long long items = (long long)groups * K;
+    for (long long item = (long long)blockIdx.x * 8 + warp; item < items; item += (long long)gridDim.x * 8) {
+        const int g = (int)(item / K), k = (int)(item - (long long)g * K);
+        const int* off = g_off + (size_t)g * (K + 1) + k;
+        const int a = __ldg(off), b = __ldg(off + 1);
+        float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, nsum = 0.f;
+        if (a < b) {
+            const float4 m = load4(mu + (size_t)k * D, false), w = load4(w2 + (size_t)k * D, false);
+            float n1 = 0.f, q1 = 0.f;
+            for (int p = a; p < b; p += 32) {
+                uint2 e = make_uint2(0u, 0u);
+                if (p + lane < b) e = __ldg(srt + p + lane);
+                const float re = __uint_as_float(e.y);
+                nsum += fabsf(re);
+                if (re < 0.f) n1 += 1.f;
+                float4 f1 = make_float4(0.f, 0.f, 0.f, 0.f), f2 = f1;
+                float fq = 0.f;
+                const int have = min(32, b - p);
+                for (int i = 0; i < have; i += 4 * rows) {
+                    float4 x[4];
+                    float r[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int src = min(31, i + u * rows + sub);
+                        const unsigned row = __shfl_sync(0xffffffffu, e.x, src);
+                        r[u] = __shfl_sync(0xffffffffu, re, src);
+                        if (i + u * rows + sub >= have) r[u] = 0.f;
+                        x[u] = make_float4(m.x, m.y, m.z, m.w);
+                        if (r[u] != 0.f) x[u] = load4(X + (size_t)row * D, vec);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float ra = fabsf(r[u]);
+                        const float tx = x[u].x - m.x, ty = x[u].y - m.y, tz = x[u].z - m.z, tw = x[u].w - m.w;
+                        f1.x = fmaf(ra, tx, f1.x); f1.y = fmaf(ra, ty, f1.y); f1.z = fmaf(ra, tz, f1.z); f1.w = fmaf(ra, tw, f1.w);
+                        const float ax = tx * tx, ay = ty * ty, az = tz * tz, aw = tw * tw;
+                        f2.x = fmaf(ra, ax, f2.x); f2.y = fmaf(ra, ay, f2.y); f2.z = fmaf(ra, az, f2.z); f2.w = fmaf(ra, aw, f2.w);
+                        const float q = fmaf(w.x, ax, fmaf(w.y, ay, fmaf(w.z, az, w.w * aw)));
+                        if (r[u] < 0.f) fq += q;
+                    }
+                }
+                s1[0] += f1.x; s1[1] += f1.y; s1[2] += f1.z; s1[3] += f1.w;
+                s2[0] += f2.x; s2[1] += f2.y; s2[2] += f2.z; s2[3] += f2.w;
+                q1 += fq;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                for (int o = lpr; o < 32; o <<= 1) {
+                    s1[j] += __shfl_xor_sync(0xffffffffu, s1[j], o);
+                    s2[j] += __shfl_xor_sync(0xffffffffu, s2[j], o);
+                }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                nsum += __shfl_xor_sync(0xffffffffu, nsum, o);
+                n1 += __shfl_xor_sync(0xffffffffu, n1, o);
+                q1 += __shfl_xor_sync(0xffffffffu, q1, o);
+            }
+            if (lane == 0 && n1 > 0.f) ll_acc += (double)n1 * c2d[k] - (double)q1;
+        }
+        const float wk = __ldg(pi + k), inv_t = 1.0f / (float)g_len[g];
+        const float4 vf = load4(var + (size_t)k * D, false);
+        const float va[4] = {vf.x, vf.y, vf.z, vf.w};
+        float gm[4], gs[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            gm[j] = gs[j] = 0.f;
+            if (a < b && wk > 0.f && d0 + j < D) {
+                gm[j] = s1[j] * (inv_t * rsqrtf(va[j]) * rsqrtf(wk));
+                gs[j] = (s2[j] - nsum * va[j]) * (inv_t * rsqrtf(2.0f * wk) / va[j]);
+            }
+        }
+        if (sub == 0 && d0 < D) {
+            float* o = fv + (size_t)g * 2 * KD + (size_t)k * D + d0;
+            if (vec_o) {
+                *reinterpret_cast<float4*>(o) = make_float4(gm[0], gm[1], gm[2], gm[3]);
+                *reinterpret_cast<float4*>(o + KD) = make_float4(gs[0], gs[1], gs[2], gs[3]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (d0 + j < D) { o[j] = gm[j]; o[KD + j] = gs[j]; }
+            }
+        }
+    }
+    if (lane == 0) red[warp] = ll_acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        ll[blockIdx.x] += t * 0.69314718055994530942;
+    }
+}
+
+// k-means: the centroids' new positions from their sums (a centroid without points stays), the points per centroid, the inertia
+// per centroid (sum of -log2 z of its points).
+__global__ void __launch_bounds__(128) screen_centroids_kernel(int D, int K, const float* __restrict__ cent_in, const double* __restrict__ Nk,
+                                                               const double* __restrict__ S1, const double* __restrict__ llk,
+                                                               float* __restrict__ cent_out, int64_t* __restrict__ counts,
+                                                               double* __restrict__ inertia_k, const int* __restrict__ ctl) {
+    if (ctl[SC_DENSE] != 0) return;
+    const int k = blockIdx.x, d = threadIdx.x;
+    const double n = Nk[k];
+    if (d < D) cent_out[(size_t)k * D + d] = n > 0.0 ? (float)(S1[(size_t)k * D + d] / n) : cent_in[(size_t)k * D + d];
+    if (d == 0) {
+        if (counts) counts[k] = (int64_t)(n + 0.5);
+        inertia_k[k] = -llk[k] / 0.69314718055994530942;
+    }
 }
 
 #define LCHECK()                                       \
@@ -1244,6 +1574,9 @@ cudaError_t plane_map(CUtensorMap* tm, void* base, int64_t rows, int atoms, int 
     } while (0)
 
 }  // namespace
+
+// Points per CTA of the evaluation and of the sort: more, smaller ranges where there are few points (at most SCR_RANGES of them).
+static int screen_range(int64_t n) { return n <= 65536 ? 128 : n <= 131072 ? 256 : SCR_RANGE; }
 
 bool screen_supports(int D, int K) { return D >= 1 && D <= 128 && K >= 1 && K <= SCR_MAX_K; }
 
@@ -1255,8 +1588,7 @@ cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi,
     LCHECK();
     screen_comp_kernel<<<(K + 7) / 8, 256, 0, s>>>(D, K, pi, mu, var, unit ? 1 : 0, b.sd, b.gd, w2, c2, c2d, b.prm, b.key, b.blk, b.ctl, status);
     LCHECK();
-    screen_plane_kernel<<<Kpad / 8, 256, 0, s>>>(D, K, Kpad, mu, w2, b.sd, b.gd, b.prm, b.key, reinterpret_cast<__half*>(b.p), b.tab,
-                                                 b.blk, b.comp_of);
+    screen_plane_kernel<<<Kpad / 8, 256, 0, s>>>(D, K, Kpad, mu, w2, b.sd, b.gd, b.prm, b.key, b.p, b.blk, b.comp_of);
     return cudaGetLastError();
 }
 
@@ -1272,7 +1604,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
         const int rpb = 256 / L;
         blocks = (n + 2 * rpb - 1) / (2 * rpb);
         if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-#define FG_TR(L_) screen_transform_kernel<L_><<<(unsigned)blocks, 256, 0, s>>>(X, n, D, b.sd, b.gd, b.y, b.n2, b.ctl, status)
+#define FG_TR(L_) screen_transform_kernel<L_><<<(unsigned)blocks, 256, 0, s>>>(X, n, D, screen_chunks(D), b.sd, b.gd, b.y, b.n2, b.ctl, status)
         switch (L) {
             case 1: FG_TR(1); break;
             case 2: FG_TR(2); break;
@@ -1283,53 +1615,57 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
 #undef FG_TR
         LCHECK();
     }
-    CUtensorMap my, mp;
     const int Kpad = screen_kpad(K), KA = screen_atoms(D);
-    cudaError_t e = plane_map(&my, b.y, SCR_PIECE, KA, SCR_TILE);
-    if (e != cudaSuccess) return e;
-    e = plane_map(&mp, b.p, Kpad, KA, 128);
-    if (e != cudaSuccess) return e;
     SweepParams p;
     p.n = n; p.KA = KA; p.KS = KS; p.NG = Kpad / 128; p.margin = margin;
-    p.tab = b.tab; p.blk = b.blk; p.comp_of = b.comp_of; p.n2 = b.n2; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.ids = b.ids;
+    p.chunks = screen_chunks(D); p.y = b.y; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
+    p.blk = b.blk; p.n2 = b.n2; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
     p.ovf = b.ovf; p.ctl = b.ctl; p.status = status;
-    e = cudaFuncSetAttribute(screen_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(screen_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (n + SCR_TILE - 1) / SCR_TILE;
-    screen_sweep_kernel<<<(unsigned)(tiles < sms ? tiles : sms), SW_THREADS, SW_SMEM, s>>>(p, my, mp);
+    if (sms > SCR_MAX_SMS) sms = SCR_MAX_SMS;
+    screen_sweep_kernel<<<(unsigned)(tiles < sms ? tiles : sms), SW_THREADS, SW_SMEM, s>>>(p);
     LCHECK();
     const size_t smem = (size_t)OV_ROWS * K * 4;
     e = cudaFuncSetAttribute(screen_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    screen_rows_kernel<<<(unsigned)(2 * sms), 256, smem, s>>>(X, n, D, K, margin, (long long)(max_marks * (double)n), mu, w2, c2d, b.ovf,
+    const double most = fmin((double)max_marks * (double)n, (double)SCR_PIECE * SCR_MARKS);
+    screen_rows_kernel<<<(unsigned)(2 * sms), 256, smem, s>>>(X, n, D, K, margin, (long long)most, mu, w2, c2d, b.ovf,
                                                               b.pt_off, b.pt_cnt, b.ids, b.ctl);
     *launches += 3;
     return cudaGetLastError();
 }
 
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
-                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx) {
-    const unsigned blocks = (unsigned)((n + SCR_RANGE - 1) / SCR_RANGE);
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count) {
+    // 32 points per warp (fewer where that leaves the chip short of warps); ranges as launch_screen_stats has them
+    const int pw = n < 131072 ? 8 : n < 200000 ? 16 : 32, range = count ? screen_range(n) : 8 * pw;
+    const unsigned blocks = (unsigned)((n + range - 1) / range);
     const size_t smem = (size_t)K * 4;
+    int* counts = count ? b.counts : nullptr;
+    cudaError_t e = cudaFuncSetAttribute(screen_eval_kernel<SCREEN_EM>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(screen_eval_kernel<SCREEN_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4);
+    if (e != cudaSuccess) return e;
     if (mode == SCREEN_EM)
-        screen_eval_kernel<SCREEN_EM><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.ll, nullptr, nullptr, b.ctl);
+        screen_eval_kernel<SCREEN_EM><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, nullptr, nullptr, b.ctl);
     else if (mode == SCREEN_LOGP)
-        screen_eval_kernel<SCREEN_LOGP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, b.ll, logp, nullptr, b.ctl);
+        screen_eval_kernel<SCREEN_LOGP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, b.ll, logp, nullptr, b.ctl);
     else
-        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, nullptr, nullptr, idx, b.ctl);
+        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, nullptr, nullptr, idx, b.ctl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                 const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches) {
-    const int blocks = (int)((n + SCR_RANGE - 1) / SCR_RANGE);
+    const int range = screen_range(n), blocks = (int)((n + range - 1) / range);
     screen_scan_kernel<<<(K + 31) / 32, 1024, 0, s>>>(b.counts, blocks, K, b.totals, b.off, b.segoff, b.ctl);
     LCHECK();
     const int K2 = (K + 1) & ~1;
     const size_t smem = (size_t)K2 * 4 + (size_t)K2 * 16;
     cudaError_t e = cudaFuncSetAttribute(screen_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    screen_fill_kernel<<<blocks, 256, smem, s>>>(n, K, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.off, b.srt, b.ctl);
+    screen_fill_kernel<<<blocks, 256, smem, s>>>(n, K, range, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.off, b.srt, b.ctl);
     LCHECK();
     int lpr = 1;
     while (4 * lpr < D) lpr <<= 1;
@@ -1337,6 +1673,32 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     LCHECK();
     screen_reduce_kernel<<<K, 1024, 0, s>>>(D, K, b.part, b.segoff, mu, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
     *launches += 4;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int D, int K, const int* g_start, const int* g_len, int* g_off,
+                                 const float* pi, const float* mu, const float* var, const float* w2, const double* c2d,
+                                 const ScreenBuffers& b, float* fv, int64_t* launches) {
+    const int K2 = (K + 1) & ~1;
+    int warps = 32;                                          // cursors of 2 bytes per warp and component: at most 128 KB
+    while (warps > 8 && (size_t)K2 * warps * 2 > 131072) warps >>= 1;
+    const size_t smem = (size_t)K2 * 4 + (size_t)K2 * warps * 2;
+    cudaError_t e = cudaFuncSetAttribute(screen_group_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    screen_group_sort_kernel<<<groups, warps * 32, smem, s>>>(K, g_start, g_len, b.pt_off, b.pt_cnt, b.ids, b.val, g_off, b.srt, b.ctl);
+    LCHECK();
+    int lpr = 1;
+    while (4 * lpr < D) lpr <<= 1;
+    const long long blocks = ((long long)groups * K + 7) / 8;
+    screen_group_stats_kernel<<<(unsigned)(blocks < SCR_LL ? blocks : SCR_LL), 256, 0, s>>>(X, D, K, lpr, groups, pi, mu, var, w2, c2d, b.srt, g_off,
+                                                                                            g_len, fv, b.ll, b.ctl);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_screen_centroids(cudaStream_t s, int D, int K, const float* cent_in, const double* Nk, const double* S1,
+                                    const ScreenBuffers& b, float* cent_out, int64_t* counts, double* inertia_k) {
+    screen_centroids_kernel<<<K, 128, 0, s>>>(D, K, cent_in, Nk, S1, b.ll + SCR_LL, cent_out, counts, inertia_k, b.ctl);
     return cudaGetLastError();
 }
 

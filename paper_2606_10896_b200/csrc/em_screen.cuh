@@ -1,6 +1,5 @@
 // Declarations of the screening path for D <= 128 (internal).
 #pragma once
-#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
@@ -8,17 +7,24 @@
 namespace fg {
 
 constexpr int SCR_MAX_K = 4096;
-constexpr int64_t SCR_PIECE = 1 << 18;       // points per round of launches: capacity of the per-point buffers
+// Points per round of launches: capacity of the per-point buffers.  Every launch has a tail and the sort by component a part that
+// does not depend on the points: at D = 128, K = 1024 a step over 10M points took 13.9 ms with 2^18, 11.9 with 2^19, 10.9 with 2^20
+// (and 18.3 with 2^17: that X stays in L2 between the kernels does not make up for it).
+constexpr int64_t SCR_PIECE = 1 << 20;
 constexpr int SCR_TILE = 256;                // points per tile of the sweep
 constexpr int SCR_RANGE = 512;               // points per CTA of the pair evaluation and of the sort by component
 constexpr int SCR_SLOTS = 16;                // room for marked pairs per point (on average over the 32 points of a warp)
-constexpr int SCR_EXTRA = 4;                 // and, per point of a piece, for the rows that do not fit there
+constexpr int SCR_WORDS = 8;                 // room for words (32 positions, mask) per point, on average over the points of a warp
+constexpr int SCR_EXTRA = 2;                 // and, per point of a piece, for the rows that do not fit there
 constexpr int64_t SCR_PAIRS = SCR_PIECE * (SCR_SLOTS + SCR_EXTRA);
 constexpr int SCR_SEG = 64;                  // pairs per work item of the statistics
-constexpr int64_t SCR_ITEMS = SCR_PAIRS / SCR_SEG + SCR_MAX_K;
+constexpr int SCR_MARKS = 10;                // marked pairs of a piece, per point of a full one: beyond them the piece counts as dense
+constexpr int64_t SCR_ITEMS = SCR_PIECE * (SCR_MARKS + SCR_EXTRA) / SCR_SEG + SCR_MAX_K;
 constexpr int SCR_RANGES = (int)(SCR_PIECE / SCR_RANGE);
-constexpr int SCR_LL = SCR_RANGES;           // log-likelihood partial sums of the evaluation, then one per component
+constexpr int SCR_LL = 4096;                 // log-likelihood partial sums (one per CTA of a launch), then one per component
 constexpr int SCR_DIM_BLOCKS = 64;
+constexpr int SCR_GROUP = 32768;             // points of a group that launch_screen_groups takes (16-bit cursors; one CTA sorts a group)
+constexpr int SCR_SPILL = 22, SCR_MAX_SMS = 160;      // see screen_sweep_kernel
 
 // Control words (in the context's result block, so that they travel to the host with the log-likelihood).
 enum { SC_DENSE = 0,      // set when a piece marks too many pairs: later kernels return at once, the caller takes the dense path
@@ -34,17 +40,18 @@ struct ScreenBuffers {
     float* sd;            // [128] power-of-two scale per dimension
     float* gd;            // [128] centre
     double* dimpart;      // [SCR_DIM_BLOCKS][4][128]
-    float4* prm;          // [K] t, c, error allowance (constant, per unit of |u|^2)
+    float4* prm;          // [K] c, error allowance (constant, per unit of |u|^2), largest |nu|
     float* key;           // [K] the allowance of a typical point
-    unsigned char* p;     // coefficient plane [atoms][Kpad][64 halves]
-    float4* tab;          // [Kpad / 2] (t0, t1, c0, c1)
+    unsigned char* p;     // coefficients [Kpad / 128][screen_group_bytes]
     int4* blk;            // [SCR_MAX_K / 32] of 32 positions: largest allowances (as bits), whether one is capped
     int* comp_of;         // [Kpad]
-    unsigned char* y;     // plane of the points [atoms][SCR_PIECE][64 halves]
+    unsigned char* y;     // rows of u [SCR_PIECE][16-byte chunks of 8 halves]
     float* n2;            // [SCR_PIECE] |u|^2
     unsigned* pt_off;     // [SCR_PIECE] where a point's pairs start
-    int* pt_cnt;          // [SCR_PIECE] how many there are
-    unsigned short* ids;  // [SCR_PAIRS] component of a pair
+    int* pt_cnt;          // [SCR_PIECE] how many there are (until the evaluation also where the words are and how many)
+    uint2* words;         // [SCR_PIECE][SCR_WORDS] the sweep's marks: a mask, the block of 32 positions it belongs to
+    unsigned long long* spill;        // [SCR_MAX_SMS][SCR_SPILL][256]
+    unsigned short* ids;  // [SCR_PAIRS] component of a kept pair
     float* val;           // [SCR_PAIRS] its responsibility (-1: the point's only pair)
     uint2* srt;           // [SCR_PAIRS] (row, responsibility) sorted by component
     int* counts;          // [SCR_RANGES][K]
@@ -60,6 +67,7 @@ struct ScreenBuffers {
 bool screen_supports(int D, int K);
 inline int screen_kpad(int K) { return (K + 127) / 128 * 128; }
 inline int screen_atoms(int D) { return (D + 31) / 32; }
+__host__ __device__ inline size_t screen_group_bytes(int D) { return 4096 + (size_t)((D + 31) / 32) * 16384; }
 
 // Parameters -> w2, c2, c2d (as launch_prepare_fp32, with the same checks), coefficient plane and tables.  unit: k-means (mu =
 // centroids; pi, var not read; log2 z = -|x - mu|^2).  Clears SC_DENSE.
@@ -74,9 +82,19 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
 // component; SCREEN_LOGP: logp[i]; SCREEN_ARGMAX: idx[i], and the pair itself kept with weight 1 for the statistics.
 enum { SCREEN_EM = 0, SCREEN_LOGP = 1, SCREEN_ARGMAX = 2 };
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
-                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx);
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count = true);
+// (count: leave the number of kept pairs per component and range for launch_screen_stats)
 // Statistics of the kept pairs: sorted by component, summed in fixed segments, added to (Nk, S1, S2) in float64.
 cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                 const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches);
+
+// After the evaluation (SCREEN_EM): Fisher vectors of `groups` groups of consecutive points of the piece (group g =
+// g_len[g] <= SCR_GROUP points from row g_start[g] on, in order) into fv [groups][2][K][D].  g_off: groups * (K + 1) ints of scratch.
+cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int D, int K, const int* g_start, const int* g_len, int* g_off,
+                                 const float* pi, const float* mu, const float* var, const float* w2, const double* c2d,
+                                 const ScreenBuffers& b, float* fv, int64_t* launches);
+// k-means: new centroids from (Nk, S1) as launch_screen_stats left them (unit parameters), points and inertia per centroid.
+cudaError_t launch_screen_centroids(cudaStream_t s, int D, int K, const float* cent_in, const double* Nk, const double* S1,
+                                    const ScreenBuffers& b, float* cent_out, int64_t* counts, double* inertia_k);
 
 }  // namespace fg

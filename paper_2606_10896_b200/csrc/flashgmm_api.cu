@@ -40,7 +40,7 @@ struct ScratchLayout {
     size_t w_partial_bytes;
     bool wide;
     // the screening path for D <= 128 (its plane of the points lies in tc_yhi)
-    size_t s_sd, s_gd, s_dimpart, s_prm, s_key, s_p, s_tab, s_blk, s_compof, s_n2, s_ptoff, s_ptcnt, s_ids, s_val, s_srt, s_counts, s_totals, s_off, s_segoff, s_part, s_ll, s_ovf;
+    size_t s_sd, s_gd, s_dimpart, s_prm, s_key, s_p, s_blk, s_compof, s_n2, s_ptoff, s_ptcnt, s_words, s_spill, s_ids, s_val, s_srt, s_counts, s_totals, s_off, s_segoff, s_part, s_ll, s_ovf;
     bool scr;
 };
 
@@ -151,24 +151,30 @@ ScratchLayout scratch_layout(int D, int K, bool planes) {
         L.w_ylo = take((size_t)WIDE_PIECE * wp.Dpad * 4);
     }
     L.scr = L.tc && planes && screen_supports(D, K);
-    L.s_sd = L.s_gd = L.s_dimpart = L.s_prm = L.s_key = L.s_p = L.s_tab = L.s_blk = L.s_compof = L.s_n2 = L.s_ptoff = L.s_ptcnt = L.s_ids = L.s_val = L.s_srt = L.s_counts = L.s_totals = L.s_off = L.s_segoff = L.s_part = L.s_ll = L.s_ovf = 0;
+    L.s_sd = L.s_gd = L.s_dimpart = L.s_prm = L.s_key = L.s_p = L.s_blk = L.s_compof = L.s_n2 = L.s_ptoff = L.s_ptcnt = L.s_words = L.s_spill = L.s_ids = L.s_val = L.s_srt = L.s_counts = L.s_totals = L.s_off = L.s_segoff = L.s_part = L.s_ll = L.s_ovf = 0;
     if (L.scr) {
-        static_assert((size_t)SCR_PIECE * 512 <= TC_YPLANE_BYTES, "the plane of the screening path lies in that of the tile kernel");
+        static_assert((size_t)SCR_PIECE * 256 <= TC_YPLANE_BYTES, "the plane of the screening path lies in that of the tile kernel");
         const size_t Kpad = (size_t)screen_kpad(K);
         L.s_sd = take(128 * 4);
         L.s_gd = take(128 * 4);
         L.s_dimpart = take((size_t)SCR_DIM_BLOCKS * 512 * 8);
         L.s_prm = take((size_t)K * 16);
         L.s_key = take((size_t)K * 4);
-        L.s_p = take((size_t)screen_atoms(D) * Kpad * 128);
-        L.s_tab = take(Kpad * 8);
+        L.s_p = take(Kpad / 128 * screen_group_bytes(D));
         L.s_blk = take((size_t)SCR_MAX_K / 32 * 16);
         L.s_compof = take(Kpad * 4);
         L.s_n2 = take((size_t)SCR_PIECE * 4);
         L.s_ptoff = take((size_t)SCR_PIECE * 4);
         L.s_ptcnt = take((size_t)SCR_PIECE * 4);
-        L.s_ids = take((size_t)SCR_PAIRS * 2);
-        L.s_val = take((size_t)SCR_PAIRS * 4);
+        {   // (in the second plane of the tile kernel, which the screening path does not use)
+            size_t in = L.tc_ylo;
+            auto inside = [&](size_t bytes) { size_t o = in; in += align256(bytes); return o; };
+            static_assert((size_t)SCR_PIECE * SCR_WORDS * 8 + (size_t)SCR_PAIRS * 6 + 1024 <= TC_YPLANE_BYTES, "lists in the second plane");
+            L.s_words = inside((size_t)SCR_PIECE * SCR_WORDS * 8);
+            L.s_ids = inside((size_t)SCR_PAIRS * 2);
+            L.s_val = inside((size_t)SCR_PAIRS * 4);
+        }
+        L.s_spill = take((size_t)SCR_MAX_SMS * SCR_SPILL * 256 * 8);
         L.s_srt = take((size_t)SCR_PAIRS * 8);
         L.s_counts = take((size_t)SCR_RANGES * K * 4);
         L.s_totals = take((size_t)K * 4);
@@ -235,7 +241,7 @@ struct gmm_ctx {
     int tc_force_filter = -1;        // GMM_TC_FILTER=plain / tight: 0 / 1 (tests); -1: automatic
     double scr_marks = -1.0;         // GMM_SCREEN_MARKS: marked pairs per point up to which the screening path is taken (D <= 128;
                                      // 0: never, < 0: from the measured costs, see screen_limit)
-    int64_t scr_piece = SCR_PIECE;   // points per round of launches of the screening path
+    int64_t scr_piece = 0;           // GMM_SCREEN_PIECE: points per round of launches of the screening path (0: screen_piece)
     int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
     int sticky_status = 0;           // status bits read off the device but not yet reported (see ensure_scratch)
     // host-streaming path
@@ -300,13 +306,14 @@ struct gmm_ctx {
         b.prm = reinterpret_cast<float4*>(at(lay.s_prm));
         b.key = reinterpret_cast<float*>(at(lay.s_key));
         b.p = at(lay.s_p);
-        b.tab = reinterpret_cast<float4*>(at(lay.s_tab));
         b.blk = reinterpret_cast<int4*>(at(lay.s_blk));
         b.comp_of = reinterpret_cast<int*>(at(lay.s_compof));
         b.y = at(lay.tc_yhi);
         b.n2 = reinterpret_cast<float*>(at(lay.s_n2));
         b.pt_off = reinterpret_cast<unsigned*>(at(lay.s_ptoff));
         b.pt_cnt = reinterpret_cast<int*>(at(lay.s_ptcnt));
+        b.words = reinterpret_cast<uint2*>(at(lay.s_words));
+        b.spill = reinterpret_cast<unsigned long long*>(at(lay.s_spill));
         b.ids = reinterpret_cast<unsigned short*>(at(lay.s_ids));
         b.val = reinterpret_cast<float*>(at(lay.s_val));
         b.srt = reinterpret_cast<uint2*>(at(lay.s_srt));
@@ -800,6 +807,15 @@ double screen_limit(const gmm_ctx* ctx, int K) {
     return 0.012 * K < 2.0 ? 2.0 : 0.012 * K < 12.0 ? 0.012 * K : 12.0;
 }
 
+// Points per round of launches for n points in all: equal pieces (an odd small one at the end pays all launches for little), in
+// whole waves of the sweep's tiles over the SMs.
+int64_t screen_piece(const gmm_ctx* ctx, int64_t n) {
+    if (ctx->scr_piece > 0) return ctx->scr_piece;
+    const int64_t wave = (int64_t)SCR_TILE * (ctx->sms < 1 ? 1 : ctx->sms), most = SCR_PIECE / wave * wave;
+    const int64_t pieces = (n + most - 1) / most;
+    return pieces <= 1 ? most : ((n + pieces - 1) / pieces + wave - 1) / wave * wave;
+}
+
 int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, const float* var, bool unit) {
     const ScreenBuffers sb = ctx->screen();
     KL(launch_screen_prepare(ctx->stream, D, K, pi, mu, var, unit, sb, ctx->w2(), ctx->c2(), ctx->c2d(), &ctx->result()->status));
@@ -808,15 +824,24 @@ int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, c
     return GMM_OK;
 }
 
+// One piece's lists (sweep) and values (see launch_screen_eval).
+int screen_values(gmm_ctx* ctx, int mode, const float* Xs, int64_t cnt, int D, int K, float margin, double limit, const float* mu,
+                  float* logp, int32_t* idx, bool count) {
+    const ScreenBuffers sb = ctx->screen();
+    CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, margin, (float)limit, mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
+    KL(launch_screen_eval(ctx->stream, mode, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, logp, idx, count));
+    return GMM_OK;
+}
+
 // Adds the statistics of n points to (Nk, S1, S2) and their log-likelihood to the partial sums.
 int screen_points(gmm_ctx* ctx, const float* X, int64_t n, int D, int K, const float* mu, double* Nk, double* S1, double* S2) {
     const ScreenBuffers sb = ctx->screen();
-    for (int64_t off = 0; off < n; off += ctx->scr_piece) {
-        const int64_t cnt = (n - off < ctx->scr_piece) ? (n - off) : ctx->scr_piece;
+    const int64_t piece = screen_piece(ctx, n);
+    for (int64_t off = 0; off < n; off += piece) {
+        const int64_t cnt = (n - off < piece) ? (n - off) : piece;
         const float* Xs = X + off * D;
         CHECK(prof_begin(ctx));
-        CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, 40.f, (float)screen_limit(ctx, K), mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
-        KL(launch_screen_eval(ctx->stream, SCREEN_EM, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, nullptr, nullptr));
+        CHECK(screen_values(ctx, SCREEN_EM, Xs, cnt, D, K, 40.f, screen_limit(ctx, K), mu, nullptr, nullptr, true));
         CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         CHECK(prof_end(ctx));
     }
@@ -1553,6 +1578,34 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     CHECK(ensure_scratch(ctx, D, K));
     CHECK(grow_buffer(ctx, &ctx->pl_scratch, &ctx->pl_scratch_bytes, pl_scratch_bytes(K), "the posting-list counters"));
     CHECK(grow_buffer(ctx, &ctx->km_scratch, &ctx->km_scratch_bytes, km_scratch_bytes(D, K), "the k-means partial sums"));
+    if (screen_wanted(ctx, D, K)) {
+        // through the screening path: the arg-max alone (margin 0), every point a lone pair of its cluster, and the statistics
+        // of the pairs about the centroids give the new ones and the inertia
+        const ScreenBuffers sb = ctx->screen();
+        double* Nk = ctx->stats();
+        double* S1 = Nk + K;
+        double* S2 = S1 + (size_t)K * D;
+        CHECK(screen_begin(ctx, D, K, nullptr, centroids, nullptr, true));
+        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+        const int64_t piece = screen_piece(ctx, N);
+        for (int64_t off = 0; off < N; off += piece) {
+            const int64_t cnt = (N - off < piece) ? (N - off) : piece;
+            const float* Xs = X + off * D;
+            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, K), centroids, nullptr, assign + off, true));
+            CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, centroids, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
+        }
+        double* ik = km_inertia_k(ctx->km_scratch, D, K);
+        KL(launch_screen_centroids(ctx->stream, D, K, centroids, Nk, S1, sb, centroids_out, counts, ik));
+        KL(launch_reduce_ll(ctx->stream, ik, K, &ctx->result()->ll[0], false));
+        DevResult r;
+        CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
+        CU(cudaStreamSynchronize(ctx->stream));
+        if (r.scr[SC_DENSE] == 0) {
+            if (inertia) *inertia = r.ll[0];
+            ctx->last_path = GMM_PATH_TENSOR;
+            return GMM_OK;
+        }
+    }
     // nearest centroid = top-1 component of a unit-variance, equal-weight mixture
     float* resp = reinterpret_cast<float*>(work);                 // [N], not used afterwards except as the builder's input
     int32_t* items = work + N;                                    // [N]
@@ -1610,6 +1663,27 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
     CHECK(check_ptr(ctx, logp, 4, "logp"));
     DeviceGuard guard(ctx->device);
     CHECK(ensure_scratch(ctx, D, K));
+    if (screen_wanted(ctx, D, K)) {
+        // D <= 128: the same idea (csrc/em_screen.cu).  The FP32 kernel takes 1.4e-4 K D ns per point, the screening path about
+        // 0.8 ns and 0.25 ns per marked pair.
+        const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks : std::fmin(14.0, std::fmax(1.5, (1.4e-4 * K * D - 0.8) / 0.25));
+        bool dense = false;
+        double total = 0.0;
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        const int64_t piece = screen_piece(ctx, N);
+        for (int64_t off = 0; off < N; off += piece) {
+            const int64_t cnt = (N - off < piece) ? (N - off) : piece;
+            CHECK(prof_begin(ctx));
+            CHECK(screen_values(ctx, SCREEN_LOGP, X + off * D, cnt, D, K, 40.f, limit, mu, logp + off, nullptr, false));
+            CHECK(prof_end(ctx));
+        }
+        CHECK(screen_end(ctx, K, 0));
+        CHECK(screen_result(ctx, 0, &total, &dense));
+        if (!dense) {
+            if (loglik) *loglik = total;
+            return GMM_OK;
+        }
+    }
     KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), &ctx->result()->status));
     if ((size_t)K * D > ((size_t)1 << 12)) ctx->launches++;
     CU(cudaMemsetAsync(&ctx->result()->ll[0], 0, 8, ctx->stream));
@@ -1717,6 +1791,60 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
+    if (smallest > 0 && screen_wanted(ctx, D, K)) {
+        // Screening path: consecutive groups are taken as many at a time as a piece holds; a larger group goes
+        // through the step's own accumulation.
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        struct Batch { int g0, g1; bool large; };
+        std::vector<Batch> batches;
+        std::vector<int> tab(2 * (size_t)G);                     // start of a group within its batch, points
+        int most = 0;
+        const int64_t piece = ctx->scr_piece > 0 ? ctx->scr_piece : SCR_PIECE;
+        for (int g = 0; g < G;) {
+            const int g0 = g;
+            const int64_t r0 = offsets[g];
+            while (g < G && offsets[g + 1] - r0 <= piece && offsets[g + 1] - offsets[g] <= SCR_GROUP && g - g0 < 4096 && (int64_t)(g - g0 + 1) * (K + 1) <= ((int64_t)1 << 23)) {
+                tab[(size_t)g] = (int)(offsets[g] - r0);
+                tab[(size_t)G + g] = (int)(offsets[g + 1] - offsets[g]);
+                ++g;
+            }
+            if (g == g0) batches.push_back({g0, ++g, true});     // larger than a piece or than SCR_GROUP
+            else batches.push_back({g0, g, false});
+            most = std::max(most, g - g0);
+        }
+        const size_t o_off = align256(2 * (size_t)G * 4);
+        CHECK(grow_buffer(ctx, &ctx->fv_scratch, &ctx->fv_scratch_bytes, o_off + (size_t)most * (K + 1) * 4, "the tables of the groups"));
+        int* d_tab = static_cast<int*>(ctx->fv_scratch);
+        int* d_off = reinterpret_cast<int*>(static_cast<unsigned char*>(ctx->fv_scratch) + o_off);
+        CU(cudaMemcpyAsync(d_tab, tab.data(), 2 * (size_t)G * 4, cudaMemcpyHostToDevice, ctx->stream));      // (pageable: copied on return)
+        const ScreenBuffers sb = ctx->screen();
+        for (const Batch& bt : batches) {
+            const int64_t rows = offsets[bt.g1] - offsets[bt.g0];
+            const float* Xs = X + offsets[bt.g0] * D;
+            float* out = fv + (size_t)bt.g0 * 2 * KD;
+            if (bt.large) {
+                CU(cudaMemsetAsync(Nk, 0, ((size_t)K + 2 * KD) * 8, ctx->stream));
+                CHECK(screen_points(ctx, Xs, rows, D, K, mu, Nk, S1, S2));
+                KL(launch_fisher(ctx->stream, rows, D, K, Nk, S1, S2, pi, mu, var, out));
+            } else if (rows == 0) {
+                CU(cudaMemsetAsync(out, 0, (size_t)(bt.g1 - bt.g0) * 2 * KD * sizeof(float), ctx->stream));
+            } else {
+                CHECK(prof_begin(ctx));
+                CHECK(screen_values(ctx, SCREEN_EM, Xs, rows, D, K, 40.f, screen_limit(ctx, K), mu, nullptr, nullptr, false));
+                CU(launch_screen_groups(ctx->stream, Xs, bt.g1 - bt.g0, D, K, d_tab + bt.g0, d_tab + G + bt.g0, d_off, pi, mu, var, ctx->w2(),
+                                        ctx->c2d(), sb, out, &ctx->launches));
+                CHECK(prof_end(ctx));
+            }
+        }
+        bool dense = false;
+        double total = 0.0;
+        CHECK(screen_end(ctx, K, 0));
+        CHECK(screen_result(ctx, 0, &total, &dense));
+        if (!dense) {
+            if (loglik) *loglik = total;
+            return GMM_OK;
+        }
+    }
     // One preparation for all groups.  The conditioning limit of the tensor path is the one an EM step over all the
     // groups' points would use: what bounds the accuracy of a Fisher coordinate is the cancellation between the raw
     // moments (N_k, S1, S2), about 4e-6 (1 + mu^2 / var) N_k / (T sqrt(pi_k)), which the stricter limit of the smallest

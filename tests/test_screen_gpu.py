@@ -129,3 +129,39 @@ def test_config2_free_running_through_the_screening_path(fg):
         trace, done = c.gmm_fit(_t(X), _t(pi0), _t(mu0), _t(var0), 8, spec.var_floor)
         assert done == 8
         np.testing.assert_allclose(trace, ref["trace"], rtol=1e-4)
+
+
+# the other entry points on the path, in pieces of 768 points: several tiles and pieces, a last piece of one point, groups that are
+# empty, larger than a piece, or share one
+@pytest.mark.parametrize("N,D,K", [(1, 16, 64), (3073, 40, 100), (2500, 128, 1024), (4000, 9, 300), (900, 66, 4096)])
+def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
+    from oracle.fisher import fisher_vectors
+    from oracle.kmeans import kmeans_step
+
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    monkeypatch.setenv("GMM_SCREEN_PIECE", "768")
+    X, pi, mu, var = _mixture(N, D, K, N + D + K)
+    offsets = np.array([0, N // 8, N // 8, N // 8 + N // 16, N - N // 5, N], np.int64)
+    lz = orc.responsibilities(X, pi, mu, var)[1]
+    G_ref = fisher_vectors(X, offsets, pi, mu, var)
+    a_r, new_r, _, inertia_r, gap = kmeans_step(X, mu.astype(np.float64))
+    runs = []
+    with fg.Context(0) as c:
+        for _ in range(2):
+            logp, total = c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var))
+            G, ll = c.gmm_fisher_vectors(_t(X), offsets, _t(pi), _t(mu), _t(var))
+            a, new, counts, inertia = c.gmm_kmeans_step(_t(X), _t(mu))
+            runs.append((logp.cpu().numpy(), total, G.cpu().numpy(), ll, a.cpu().numpy(), new.cpu().numpy(), counts.cpu().numpy(), inertia))
+    for u, v in zip(*runs):
+        assert np.array_equal(u, v)                            # the same bits in every run
+    logp, total, G, ll, a, new, counts, inertia = runs[0]
+    assert np.all(np.abs(logp - lz) <= 1e-5 * np.abs(lz) + 1e-4) and abs(total - lz.sum()) <= 1e-5 * abs(lz.sum())
+    assert abs(ll - lz.sum()) <= 1e-5 * abs(lz.sum())
+    assert np.abs(G - G_ref).max() <= 2e-5 * (1 + np.abs(G_ref).max()) and np.all(G[1] == 0.0)
+    tie = gap <= 1e-4 * D * float(X.astype(np.float64).var(0).mean() if N > 1 else 1.0)
+    assert np.all((a == a_r) | tie) and counts.sum() == N and np.array_equal(counts, np.bincount(a, minlength=K))
+    assert abs(inertia - inertia_r) <= 1e-5 * abs(inertia_r)
+    for k in np.unique(a)[:50]:
+        np.testing.assert_allclose(new[k], X[a == k].astype(np.float64).mean(0), rtol=0, atol=1e-5)
+    empty = np.setdiff1d(np.arange(K), a)
+    assert np.array_equal(new[empty], mu[empty])               # a centroid without points stays where it is

@@ -1,0 +1,676 @@
+// The FP32 path for D <= 128: direct differences on the CUDA cores, tiles cut to the shape.
+//
+// log2 z = c - sum_d t^2, t = (x - g) sqrt(w2) - (mu - g) sqrt(w2) (two FMAs per term, g: a per-dimension centre near the data).  A CTA
+// of 256 threads takes tiles of points.  For the logits a point belongs to G x S neighbouring lanes: G lanes own the components
+// (four each, 64 per block at most), S lanes share the dimensions; a lane works on PT points at once.  For the statistics a thread
+// owns a tile of TK components x 4 dimensions of the two sums, and as many replicas of those tiles as fit 256 threads split the
+// points; they meet once, at the end of the kernel.  So neither K = 8 nor D = 16 pays for the 64 components x 32 (and x 128)
+// dimensions that fixed tiles pad to: 10K x 16, K = 8 took 115 us per iteration with those and now takes 18 (10 us this kernel);
+// 1M x 16, K = 8: 1580 -> 100 us, 1M x 96, K = 32: 2650 -> 1080 us.
+//
+//   DK_FUSED  K <= 64: log-sum-exp and statistics in one pass over X, the parameters stay in shared memory.
+//   DK_LSE    log2 Z per point and the log-likelihood, any K (blocks of 64 components one after the other).
+//   DK_STATS  statistics of a block of 64 components (blockIdx.y), given log2 Z.
+//
+// Bound by the FMA rate at larger K D (4 K D FMAs per point, two per instruction: fma.f32x2), by launches and the trip through X
+// at small ones.
+#include "internal.cuh"
+#include <math_constants.h>
+#include <stdint.h>
+
+namespace fg {
+
+namespace {
+
+constexpr int NT = 256;
+enum { DK_FUSED = 0, DK_LSE = 1, DK_STATS = 2 };
+
+struct DirectArgs {
+    const float* X;
+    int64_t n;
+    int D, K;
+    const float *mu, *w2;
+    const double* c2d;
+    const float* g;          // centre (not DK_FUSED, which takes the mean of the means itself)
+    float* g_out;            // and leaves it here
+    double* logZ2;           // DK_LSE writes (may be NULL), DK_STATS reads
+    double* llpart;          // [gridDim.x], may be NULL
+    int ll_first;            // llpart is written, not added to
+    float* partials;         // [splits][K + 2 K D]
+    int* status;             // DK_FUSED: parameters that are not finite and positive
+    int* counts;             // DK_FUSED: zeroed for the update that follows
+    const int* stop_at;      // NULL, or the iteration after which nothing is done any more
+    int iter;
+    int lgG, lgS;            // lanes per point: components, dimensions
+    int ld, ldr, kr;         // row strides (multiples of 4, odd multiples: no bank conflicts), rows of the parameters
+    int D4, lgX;             // chunks of four dimensions; lanes per row when X is staged
+    int T, R;                // tiles of the statistics, replicas
+    int xvec;                // rows of X start on 16-byte boundaries
+};
+
+__device__ __forceinline__ float dk_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
+typedef unsigned long long u64;
+__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) { u64 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ u64 mul2(u64 a, u64 b) { u64 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ u64 dup2(float a) { u64 r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a)); return r; }
+__device__ __forceinline__ float lo2(u64 a) { return __uint_as_float((uint32_t)a); }
+__device__ __forceinline__ float hi2(u64 a) { return __uint_as_float((uint32_t)(a >> 32)); }
+
+// The kernels of a fit follow one another at once (programmatic launch): a kernel's CTAs are started while the last ones of its
+// predecessor are still at work, and wait here until those have finished and their writes are visible.  (So nothing here is read
+// through the non-coherent cache.)
+__device__ __forceinline__ void grid_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <int MODE, int PT, int TK>
+__global__ void __launch_bounds__(NT, 2) direct_kernel(const DirectArgs p) {
+    extern __shared__ __align__(16) float sm[];
+    grid_wait();
+    const int stop = p.stop_at ? __ldcg(p.stop_at) : p.iter;      // (looked at when the first loads are under way)
+    __shared__ __align__(16) float gs[128];
+    __shared__ double red[NT / 32][64];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int D = p.D, K = p.K, D4 = p.D4, ld = p.ld, ldr = p.ldr, kr = p.kr;
+    const int lgL = p.lgG + p.lgS, G = 1 << p.lgG, S = 1 << p.lgS;
+    const int s = tid & (S - 1), gq = (tid >> p.lgS) & (G - 1), pg = tid >> lgL, PG = NT >> lgL, TP = PT * PG;
+    float* sw = sm;                          // [kr][ld] sqrt(w2)
+    float* ms = sw + kr * ld;                // [kr][ld] (g - mu) sqrt(w2)
+    float* xs = ms + kr * ld;                // [TP][ld] x - g
+    float* rs = xs + TP * ld;                // [TP][ldr] responsibilities
+    const int kfirst = MODE == DK_STATS ? (int)blockIdx.y * 64 : 0;
+    const int nblk = MODE == DK_LSE ? (K + 63) / 64 : 1;
+    const int64_t ntiles = (p.n + TP - 1) / TP;
+
+    // parameters of the block from component k0 on (raw: the means as they are)
+    const int cx = tid & ((1 << p.lgX) - 1), rx = tid >> p.lgX, stepx = NT >> p.lgX;
+    const bool pvec = (D & 3) == 0 && (((reinterpret_cast<uintptr_t>(p.mu) | reinterpret_cast<uintptr_t>(p.w2)) & 15) == 0);
+    auto params = [&](int k0, bool raw) {
+        if (cx >= D4) return;
+        const int c = 4 * cx;
+        const float g0 = gs[c], g1 = gs[c + 1], g2 = gs[c + 2], g3 = gs[c + 3];
+#pragma unroll 4
+        for (int r = rx; r < kr; r += stepx) {
+            float4 m = make_float4(0.f, 0.f, 0.f, 0.f), w = m;
+            if (k0 + r < K && r < 64) {
+                const size_t o = (size_t)(k0 + r) * D + c;
+                if (pvec) {
+                    m = __ldcg(reinterpret_cast<const float4*>(p.mu + o));
+                    w = __ldcg(reinterpret_cast<const float4*>(p.w2 + o));
+                } else {
+                    m.x = __ldcg(p.mu + o); w.x = __ldcg(p.w2 + o);
+                    if (c + 1 < D) { m.y = __ldcg(p.mu + o + 1); w.y = __ldcg(p.w2 + o + 1); }
+                    if (c + 2 < D) { m.z = __ldcg(p.mu + o + 2); w.z = __ldcg(p.w2 + o + 2); }
+                    if (c + 3 < D) { m.w = __ldcg(p.mu + o + 3); w.w = __ldcg(p.w2 + o + 3); }
+                }
+                w = make_float4(sqrtf(w.x), sqrtf(w.y), sqrtf(w.z), sqrtf(w.w));
+                if (!raw) m = make_float4((g0 - m.x) * w.x, (g1 - m.y) * w.y, (g2 - m.z) * w.z, (g3 - m.w) * w.w);
+            }
+            *reinterpret_cast<float4*>(sw + r * ld + c) = w;
+            *reinterpret_cast<float4*>(ms + r * ld + c) = m;
+        }
+    };
+    float cv[4];
+    auto constants = [&](int k0) {
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int r = gq + G * b;
+            cv[b] = (k0 + r < K && r < 64) ? (float)__ldcg(p.c2d + k0 + r) : -CUDART_INF_F;
+        }
+    };
+    // a tile of X on its way into shared memory, as it is; and its arrival: a thread centres the chunks that it asked for
+    auto tile_fetch = [&](int64_t row0) {
+        if (cx < D4) {
+            const int c = 4 * cx;
+#pragma unroll 4
+            for (int r = rx; r < TP; r += stepx) {
+                const int64_t row = row0 + r;
+                float* dst = xs + r * ld + c;
+                if (row >= p.n) continue;
+                const float* src = p.X + row * D + c;
+                const uint32_t da = (uint32_t)__cvta_generic_to_shared(dst);
+                if (p.xvec) {
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(da), "l"(src) : "memory");
+                } else {
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(da), "l"(src) : "memory");
+                    if (c + 1 < D) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(da + 4), "l"(src + 1) : "memory");
+                    if (c + 2 < D) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(da + 8), "l"(src + 2) : "memory");
+                    if (c + 3 < D) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(da + 12), "l"(src + 3) : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    auto tile_centre = [&](int64_t row0) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        if (cx < D4) {
+            const int c = 4 * cx;
+            const float4 gv = *reinterpret_cast<const float4*>(gs + c);          // (zero beyond D)
+#pragma unroll 4
+            for (int r = rx; r < TP; r += stepx) {
+                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (row0 + r < p.n) {
+                    v = *reinterpret_cast<const float4*>(xs + r * ld + c);
+                    v.x -= gv.x; v.y = c + 1 < D ? v.y - gv.y : 0.f; v.z = c + 2 < D ? v.z - gv.z : 0.f; v.w = c + 3 < D ? v.w - gv.w : 0.f;
+                }
+                *reinterpret_cast<float4*>(xs + r * ld + c) = v;
+            }
+        }
+    };
+    if (MODE == DK_FUSED) {
+        tile_fetch((int64_t)blockIdx.x * TP);
+        constants(0);
+        params(0, true);                                     // (gs is not read)
+        if (stop < p.iter) { asm volatile("cp.async.wait_group 0;" ::: "memory"); return; }
+        if (blockIdx.x == 0 && p.counts && tid < 2) p.counts[tid] = 0;
+        __syncthreads();
+        int bad = 0;
+        if (tid < 128) {
+            double a = 0.0;
+            if (tid < 4 * D4) {
+#pragma unroll 4
+                for (int k = 0; k < K; ++k) a += (double)ms[k * ld + tid];
+            }
+            const int d = tid;
+            const float c = (float)(a / (double)K);
+            gs[d] = isfinite(c) ? c : 0.f;
+            if (blockIdx.x == 0 && p.g_out && d < D) p.g_out[d] = gs[d];
+        }
+        __syncthreads();
+        for (int r = warp; r < K; r += NT / 32)
+            for (int d = lane; d < D; d += 32) {
+                const float m = ms[r * ld + d], w = sw[r * ld + d];
+                if (!isfinite(m)) bad |= ST_NONFINITE;
+                if (!(w > 0.f) || !isfinite(w)) bad |= ST_BAD_VAR;
+                ms[r * ld + d] = (gs[d] - m) * w;
+            }
+        if (p.stop_at && blockIdx.x == 0 && tid < K && isnan(__ldcg(p.c2d + tid))) bad |= ST_BAD_PI;
+        // (of a fit: the first iteration's parameters were checked by the preparation, the later ones here)
+        if (p.stop_at && blockIdx.x == 0 && bad) atomicOr(p.status, bad);
+    } else {
+        tile_fetch((int64_t)blockIdx.x * TP);
+        if (tid < 128) gs[tid] = (p.g && tid < D) ? __ldcg(p.g + tid) : 0.f;
+        __syncthreads();
+        if (nblk == 1) { params(kfirst, false); constants(kfirst); }
+    }
+
+    // statistics: thread = replica rep of tile (kt, dt)
+    const int rep = tid / p.T, tt = tid - rep * p.T, dt = tt % D4, kt = tt / D4;
+    u64 acc1[TK][2], acc2[TK][2];
+    float nacc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < TK; ++c) acc1[c][0] = acc1[c][1] = acc2[c][0] = acc2[c][1] = 0ull;
+    double ll = 0.0;
+
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int64_t row0 = t * TP;
+        if (t != blockIdx.x) {
+            __syncthreads();                                 // (the tile before this one has been read)
+            tile_fetch(row0);
+        }
+        tile_centre(row0);
+        __syncthreads();
+        float m_run[PT], s_run[PT];
+        float l[PT][4];
+#pragma unroll
+        for (int j = 0; j < PT; ++j) { m_run[j] = -CUDART_INF_F; s_run[j] = 0.f; }
+        for (int blk = 0; blk < nblk; ++blk) {
+            if (nblk > 1) {
+                __syncthreads();
+                params(blk * 64, false);
+                constants(blk * 64);
+                __syncthreads();
+            }
+            u64 q[PT][4];
+#pragma unroll
+            for (int j = 0; j < PT; ++j)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) q[j][b] = 0ull;
+#pragma unroll 2
+            for (int d4 = s; d4 < D4; d4 += S) {
+                ulonglong2 x[PT];
+#pragma unroll
+                for (int j = 0; j < PT; ++j) x[j] = *reinterpret_cast<const ulonglong2*>(xs + (pg + j * PG) * ld + 4 * d4);
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + (gq + G * b) * ld + 4 * d4);
+                    const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ms + (gq + G * b) * ld + 4 * d4);
+#pragma unroll
+                    for (int j = 0; j < PT; ++j) {
+                        const u64 t0 = fma2(x[j].x, w.x, m.x), t1 = fma2(x[j].y, w.y, m.y);
+                        q[j][b] = fma2(t0, t0, q[j][b]);
+                        q[j][b] = fma2(t1, t1, q[j][b]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < PT; ++j) {
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    float v = lo2(q[j][b]) + hi2(q[j][b]);
+                    for (int o = 1; o < S; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    l[j][b] = cv[b] - v;
+                }
+                if (MODE != DK_STATS) {
+                    float m = fmaxf(fmaxf(l[j][0], l[j][1]), fmaxf(l[j][2], l[j][3]));
+                    for (int o = S; o < (1 << lgL); o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    m = fmaxf(m, m_run[j]);
+                    const float ref = m == -CUDART_INF_F ? 0.f : m;
+                    float e[4], a;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) e[b] = dk_ex2(l[j][b] - ref);
+                    a = (e[0] + e[1]) + (e[2] + e[3]);
+                    for (int o = S; o < (1 << lgL); o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                    s_run[j] = (MODE == DK_FUSED ? 0.f : s_run[j] * dk_ex2(m_run[j] - ref)) + a;
+                    m_run[j] = m;
+                    if (MODE == DK_FUSED) {
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) l[j][b] = e[b];
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < PT; ++j) {
+            const int r = pg + j * PG;
+            const int64_t row = row0 + r;
+            const bool in = row < p.n;
+            if (MODE != DK_STATS) {
+                const double lz = (double)m_run[j] + (double)log2f(s_run[j]);
+                if (in && (tid & ((1 << lgL) - 1)) == 0) {
+                    ll += lz;
+                    if (p.logZ2) p.logZ2[row] = lz;
+                }
+            }
+            if (MODE != DK_LSE) {
+                float f, lz = 0.f;
+                if (MODE == DK_FUSED) f = in ? 1.0f / s_run[j] : 0.f;
+                else lz = in ? (float)__ldcg(p.logZ2 + row) : CUDART_INF_F;
+                if (s == 0) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const float v = MODE == DK_FUSED ? l[j][b] * f : dk_ex2(l[j][b] - lz);
+                        nacc[b] += v;
+                        if (gq + G * b < ldr) rs[r * ldr + gq + G * b] = v;
+                    }
+                }
+            }
+        }
+        if (MODE != DK_LSE) {
+            __syncthreads();
+            if (rep < p.R) {
+#pragma unroll 2
+                for (int r = rep; r < TP; r += p.R) {
+                    const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(xs + r * ld + 4 * dt);
+                    const u64 y0 = mul2(x.x, x.x), y1 = mul2(x.y, x.y);
+#pragma unroll
+                    for (int h = 0; h < TK / 4; ++h) {
+                        const float4 w = *reinterpret_cast<const float4*>(rs + r * ldr + kt * TK + 4 * h);
+                        const float rr[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const u64 rd = dup2(rr[c]);
+                            acc1[4 * h + c][0] = fma2(rd, x.x, acc1[4 * h + c][0]);
+                            acc1[4 * h + c][1] = fma2(rd, x.y, acc1[4 * h + c][1]);
+                            acc2[4 * h + c][0] = fma2(rd, y0, acc2[4 * h + c][0]);
+                            acc2[4 * h + c][1] = fma2(rd, y1, acc2[4 * h + c][1]);
+                        }
+                    }
+                }
+            }
+        }
+    }
+
+    // ---- once per CTA: log-likelihood, N_k, and the replicas' sums in a fixed order ----
+    if (MODE != DK_STATS && p.llpart) {
+        for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
+        if (lane == 0) red[warp][0] = ll;
+        __syncthreads();
+        if (tid == 0) {
+            double a = 0.0;
+            for (int w = 0; w < NT / 32; ++w) a += red[w][0];
+            a *= 0.69314718055994530942;
+            p.llpart[blockIdx.x] = p.ll_first ? a : p.llpart[blockIdx.x] + a;
+        }
+    }
+    if (MODE == DK_LSE) return;
+    __syncthreads();
+    const size_t KD = (size_t)K * D;
+    float* pN = p.partials + (size_t)blockIdx.x * (K + 2 * KD);
+    float* pS1 = pN + K;
+    float* pS2 = pS1 + KD;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        double a = s == 0 ? (double)nacc[b] : 0.0;
+        for (int o = 16; o >= (1 << lgL); o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if (lane < (1 << lgL) && s == 0) red[warp][gq + G * b] = a;
+    }
+    __syncthreads();
+    if (tid < 64 && tid < 4 * G && kfirst + tid < K) {
+        double a = 0.0;
+        for (int w = 0; w < NT / 32; ++w) a += red[w][tid];
+        pN[kfirst + tid] = (float)a;
+    }
+    auto put = [&](int tile, int i, float v) {               // value i of a tile: component, sum, dimension
+        const int k = kfirst + (tile / D4) * TK + (i >> 3), d = (tile % D4) * 4 + (i & 3);
+        if (k < K && (tile / D4) * TK + (i >> 3) < 64 && d < D) ((i & 4) ? pS2 : pS1)[(size_t)k * D + d] = v;
+    };
+    if (p.R == 1) {
+        if (rep < 1) {
+#pragma unroll
+            for (int c = 0; c < TK; ++c) {
+                put(tt, 8 * c, lo2(acc1[c][0])); put(tt, 8 * c + 1, hi2(acc1[c][0]));
+                put(tt, 8 * c + 2, lo2(acc1[c][1])); put(tt, 8 * c + 3, hi2(acc1[c][1]));
+                put(tt, 8 * c + 4, lo2(acc2[c][0])); put(tt, 8 * c + 5, hi2(acc2[c][0]));
+                put(tt, 8 * c + 6, lo2(acc2[c][1])); put(tt, 8 * c + 7, hi2(acc2[c][1]));
+            }
+        }
+        return;
+    }
+    float* dump = sm;                                        // [8 TK][NT + T] (no bank conflicts below), over the tiles (which all threads have left)
+    const int ds = NT + p.T;
+#pragma unroll
+    for (int c = 0; c < TK; ++c) {
+        dump[(8 * c) * ds + tid] = lo2(acc1[c][0]); dump[(8 * c + 1) * ds + tid] = hi2(acc1[c][0]);
+        dump[(8 * c + 2) * ds + tid] = lo2(acc1[c][1]); dump[(8 * c + 3) * ds + tid] = hi2(acc1[c][1]);
+        dump[(8 * c + 4) * ds + tid] = lo2(acc2[c][0]); dump[(8 * c + 5) * ds + tid] = hi2(acc2[c][0]);
+        dump[(8 * c + 6) * ds + tid] = lo2(acc2[c][1]); dump[(8 * c + 7) * ds + tid] = hi2(acc2[c][1]);
+    }
+    __syncthreads();
+    for (int o = tid; o < p.T * 8 * TK; o += NT) {
+        const int i = o / p.T, tile = o - i * p.T;
+        double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (int r = 0; r < p.R; ++r) a[r & 3] += (double)dump[i * ds + r * p.T + tile];
+        put(tile, i, (float)((a[0] + a[1]) + (a[2] + a[3])));
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+// Partials -> statistics, and in a fit the update and the next iteration's constants: a CTA per component.  Threads share the
+// splits (one thread per output walked them all before: 45 us for 296 splits of K = 8, D = 16; now 6 with the update).  The sums are
+// in float64, in a fixed order.
+struct ReduceArgs {
+    int D, K, splits;
+    const float* partials;
+    const float* g;
+    double *Nk, *S1, *S2;
+    int accumulate;
+    // log-likelihood: sum of llpart[n_ll] into *ll (n_ll = 0: left alone)
+    const double* llpart;
+    int n_ll;
+    double* ll;
+    int ll_accumulate;
+    // update (fit): NULL pi = none
+    float *pi, *mu, *var;
+    float var_floor;
+    int isotropic;
+    int64_t N;
+    int* counts;
+    const int* status;
+    float* w2;
+    float* c2;
+    double* c2d;
+    const double* ll_prev;   // NULL in the first iteration
+    double tol;
+    int* stop_at;
+    int iter;
+};
+
+__global__ void __launch_bounds__(1024) direct_reduce_kernel(const ReduceArgs p) {
+    grid_wait();
+    if (p.stop_at && *p.stop_at < p.iter) return;
+    __shared__ double part[1024];
+    __shared__ double tot[257];
+    __shared__ double red[32];
+    const int tid = threadIdx.x, lane = tid & 31, k = blockIdx.x, D = p.D, W = 2 * D + 1, RG = 1024 / W;
+    const size_t KD = (size_t)p.K * D, per = (size_t)p.K + 2 * KD;
+    const int out = tid % W, rg = tid / W;
+    double a = 0.0;
+    double ll = 0.0;                                         // every CTA of a fit needs to know whether the log-likelihood is finite
+    if (p.n_ll > 0 && (p.pi || k == 0) && tid < p.n_ll) ll = __ldcg(p.llpart + tid);      // (n_ll <= 1024)
+    if (rg < RG) {
+        const size_t e = out == 0 ? (size_t)k : out <= D ? (size_t)p.K + (size_t)k * D + out - 1 : (size_t)p.K + KD + (size_t)k * D + out - 1 - D;
+        for (int r = rg; r < p.splits; r += 8 * RG) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = r + u * RG < p.splits ? __ldcg(p.partials + (size_t)(r + u * RG) * per + e) : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) a += (double)v[u];
+        }
+    }
+    part[tid] = a;
+    if (p.n_ll > 0 && (p.pi || k == 0)) {
+        for (int o = 16; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
+        if (lane == 0) red[tid >> 5] = ll;
+    }
+    __syncthreads();
+    if (tid < W) {
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (int r = 0; r < RG; ++r) s[r & 3] += part[r * W + tid];
+        tot[tid] = (s[0] + s[1]) + (s[2] + s[3]);
+    }
+    ll = 0.0;
+    if (p.n_ll > 0 && (p.pi || k == 0))
+        for (int w = 0; w < 32; ++w) ll += red[w];
+    __syncthreads();
+    // shift from the centre: S1 = S1c + g N, S2 = S2c + 2 g S1c + g^2 N
+    double n = tot[0], s1 = 0.0, s2 = 0.0;
+    if (tid < D) {
+        const double g = p.g ? (double)__ldcg(p.g + tid) : 0.0;
+        s1 = tot[1 + tid] + g * n;
+        s2 = tot[1 + D + tid] + 2.0 * g * tot[1 + tid] + g * g * n;
+    }
+    if (p.accumulate) {
+        n += p.Nk[k];
+        if (tid < D) { s1 += p.S1[(size_t)k * D + tid]; s2 += p.S2[(size_t)k * D + tid]; }
+    }
+    __syncthreads();                                         // (everyone has read N_k)
+    if (tid == 0) p.Nk[k] = n;
+    if (tid < D) { p.S1[(size_t)k * D + tid] = s1; p.S2[(size_t)k * D + tid] = s2; }
+    if (k == 0 && tid == 0 && p.n_ll > 0) *p.ll = p.ll_accumulate ? *p.ll + ll : ll;
+    if (!p.pi) return;
+    const bool good = *p.status == 0 && isfinite(ll);        // a step that failed leaves the parameters as they are
+    if (k == 0 && tid == 0 && (!good || (p.tol > 0.0 && p.ll_prev && fabs(ll - *p.ll_prev) <= p.tol * fabs(ll)))) *p.stop_at = p.iter;
+    if (!good) return;
+    if (tid == 0) p.pi[k] = (float)(n / (double)p.N);        // pi_k = N_k / N
+    const bool empty = n < 1e-12;                            // an empty component keeps mu and var
+    double v = 0.0;
+    float vf = 0.f;
+    if (tid < D) {
+        if (!empty) {
+            const double m = s1 / n;                         // Eq. 2
+            v = s2 / n - m * m;                              // Eq. 3 per dimension, new mean
+            p.mu[(size_t)k * D + tid] = (float)m;
+        }
+    }
+    if (empty) {
+        if (tid == 0) atomicAdd(p.counts + 1, 1);
+        if (tid < D) vf = p.var[(size_t)k * D + tid];
+    } else {
+        const double fl = (double)p.var_floor;
+        if (p.isotropic) {                                   // one variance: the mean over the dimensions
+            double q = tid < D ? v : 0.0;
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if (lane == 0) red[tid >> 5] = q;
+            __syncthreads();
+            v = 0.0;
+            for (int w = 0; w < 4; ++w) v += red[w];
+            v /= (double)D;
+            if (!(v > fl)) { v = fl; if (tid == 0) atomicAdd(p.counts, D); }
+        } else if (tid < D && !(v > fl)) {
+            v = fl;
+            atomicAdd(p.counts, 1);
+        }
+        vf = (float)v;
+        if (tid < D) p.var[(size_t)k * D + tid] = vf;
+    }
+    // the next iteration's constants
+    double lg = 0.0;
+    if (tid < D) {
+        lg = log(6.283185307179586476925286766559 * (double)vf);
+        p.w2[(size_t)k * D + tid] = (float)(0.72134752044448170368 / (double)vf);
+    }
+    for (int o = 16; o > 0; o >>= 1) lg += __shfl_xor_sync(0xffffffffu, lg, o);
+    __syncthreads();
+    if (lane == 0) red[tid >> 5] = lg;
+    __syncthreads();
+    if (tid == 0) {
+        const float pf = (float)(n / (double)p.N);
+        const double lp = pf > 0.f ? log((double)pf) : pf == 0.f ? -CUDART_INF : CUDART_NAN;
+        const double c = 1.4426950408889634074 * (lp - 0.5 * (((red[0] + red[1]) + red[2]) + red[3]));
+        p.c2[k] = (float)c;
+        p.c2d[k] = c;
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------------
+struct DirectPlan {
+    DirectArgs a;
+    int PT, TK;
+    int64_t tiles;
+    size_t smem;
+    int per_sm;
+};
+
+constexpr int SMS = 148;
+
+// Shape of the tiles for n points.
+DirectPlan direct_plan(int mode, const float* X, int64_t n, int D, int K) {
+    DirectPlan pl{};
+    DirectArgs& a = pl.a;
+    a.X = X; a.n = n; a.D = D; a.K = K;
+    const int kb = K < 64 ? K : 64, cblocks = mode == DK_STATS ? (K + 63) / 64 : 1;
+    a.D4 = (D + 3) / 4;
+    // rows of x and of the parameters: an odd multiple of the 16 S bytes that the S lanes of a point read (no bank conflicts)
+    auto set_ld = [&]() { a.ld = 4 * (((a.D4 + (1 << a.lgS) - 1) >> a.lgS) | 1) << a.lgS; };
+    set_ld();
+    while ((4 << a.lgG) < kb) ++a.lgG;
+    a.kr = 4 << a.lgG;
+    while ((1 << a.lgX) < a.D4) ++a.lgX;
+    a.xvec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
+    // four components per tile of the statistics where eight would be padding (and the tiles fit the threads)
+    pl.TK = 8;
+    if (((kb - 1) & 7) < 4 && (kb + 3) / 4 * a.D4 <= NT) pl.TK = 4;
+    const int kp = (kb + pl.TK - 1) / pl.TK * pl.TK;
+    a.ldr = 4 * ((kp / 4) | 1);
+    a.T = kp / pl.TK * a.D4;
+    a.R = NT / a.T;
+    // points per tile: four per lane, fewer where the tile would not leave room for a second CTA on the SM, or where there would
+    // not be a tile for every SM; the lanes then share the dimensions as long as there are eight per lane
+    pl.PT = (mode == DK_LSE || D > 32) ? 4 : 2;          // (at four, the statistics' registers spill, once per tile)
+    auto tp = [&]() { return (int64_t)pl.PT * (NT >> (a.lgG + a.lgS)); };
+    auto bytes = [&]() { return (2 * a.kr * a.ld + tp() * (a.ld + (mode == DK_LSE ? 0 : a.ldr))) * 4; };
+    while (bytes() > 110592 || (n + tp() - 1) / tp() * cblocks < SMS) {
+        if (a.lgG + a.lgS < 5 && a.D4 >= (4 << a.lgS)) { ++a.lgS; set_ld(); }
+        else if (pl.PT > 1) pl.PT >>= 1;
+        else break;
+    }
+    pl.tiles = (n + tp() - 1) / tp();
+    size_t fl = (size_t)2 * a.kr * a.ld + (size_t)tp() * (a.ld + (mode == DK_LSE ? 0 : a.ldr));
+    if (mode != DK_LSE && a.R > 1 && fl < (size_t)8 * pl.TK * (NT + a.T)) fl = (size_t)8 * pl.TK * (NT + a.T);
+    pl.smem = fl * 4;
+    pl.per_sm = pl.smem + 6144 <= 233472 / 2 ? 2 : 1;
+    return pl;
+}
+
+template <typename Args>
+cudaError_t launch_chained(cudaStream_t s, dim3 grid, int threads, size_t smem, void (*kernel)(Args), const Args& a) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+template <int MODE, int PT, int TK>
+cudaError_t direct_launch(cudaStream_t s, dim3 grid, const DirectPlan& pl) {
+    if (pl.smem > 40960) {
+        cudaError_t e = cudaFuncSetAttribute(direct_kernel<MODE, PT, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_chained(s, grid, NT, pl.smem, direct_kernel<MODE, PT, TK>, pl.a);
+}
+template <int MODE>
+cudaError_t direct_launch(cudaStream_t s, dim3 grid, const DirectPlan& pl) {
+    const bool t8 = MODE != DK_LSE && pl.TK == 8;
+    switch (pl.PT) {
+        case 1: return t8 ? direct_launch<MODE, 1, 8>(s, grid, pl) : direct_launch<MODE, 1, 4>(s, grid, pl);
+        case 2: return t8 ? direct_launch<MODE, 2, 8>(s, grid, pl) : direct_launch<MODE, 2, 4>(s, grid, pl);
+        default: return t8 ? direct_launch<MODE, 4, 8>(s, grid, pl) : direct_launch<MODE, 4, 4>(s, grid, pl);
+    }
+}
+
+}  // namespace
+
+int lse_direct_parts(int64_t n, int D, int K) {
+    const DirectPlan pl = direct_plan(DK_LSE, nullptr, n, D, K);
+    return (int)(pl.tiles < SMS * pl.per_sm ? pl.tiles : SMS * pl.per_sm);
+}
+
+cudaError_t launch_lse_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
+                              const double* c2d, const float* g, double* logZ2, double* llpart) {
+    DirectPlan pl = direct_plan(DK_LSE, X, n, D, K);
+    pl.a.mu = mu; pl.a.w2 = w2; pl.a.c2d = c2d; pl.a.g = g; pl.a.logZ2 = logZ2; pl.a.llpart = llpart; pl.a.ll_first = 1;
+    return direct_launch<DK_LSE>(s, dim3((unsigned)lse_direct_parts(n, D, K)), pl);
+}
+
+cudaError_t launch_mstep_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
+                                const double* c2d, const float* g, const double* logZ2, float* partials, int splits) {
+    DirectPlan pl = direct_plan(DK_STATS, X, n, D, K);
+    pl.a.mu = mu; pl.a.w2 = w2; pl.a.c2d = c2d; pl.a.g = g; pl.a.logZ2 = const_cast<double*>(logZ2); pl.a.partials = partials;
+    return direct_launch<DK_STATS>(s, dim3((unsigned)splits, (unsigned)((K + 63) / 64)), pl);
+}
+
+cudaError_t launch_reduce_direct(cudaStream_t s, int D, int K, int splits, const float* partials, const float* g, double* Nk,
+                                 double* S1, double* S2, bool accumulate) {
+    ReduceArgs r{};
+    r.D = D; r.K = K; r.splits = splits; r.partials = partials; r.g = g; r.Nk = Nk; r.S1 = S1; r.S2 = S2; r.accumulate = accumulate ? 1 : 0;
+    return launch_chained(s, dim3((unsigned)K), 1024, 0, direct_reduce_kernel, r);
+}
+
+bool fused_direct_supports(int D, int K) { return D <= 128 && K <= 64; }
+
+cudaError_t launch_fused_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, float* w2, float* c2,
+                                double* c2d, float* g, float* partials, double* llpart, double* Nk, double* S1, double* S2,
+                                bool accumulate, double* ll, int* status, const DirectFit* fit, int64_t* launches) {
+    // an fp32 sum takes at most 4096 points: beyond that (per replica and CTA) the points go in several launches, whose statistics
+    // are added in float64
+    DirectPlan pl = direct_plan(DK_FUSED, X, n, D, K);
+    const int64_t ctas = pl.tiles < (int64_t)SMS * pl.per_sm ? pl.tiles : (int64_t)SMS * pl.per_sm;
+    const int64_t piece = ctas * pl.a.R * 4096;
+    for (int64_t off = 0; off < n; off += piece) {
+        const int64_t cnt = n - off < piece ? n - off : piece;
+        const bool last = off + cnt == n;
+        DirectArgs& a = pl.a;
+        a.X = X + off * D; a.n = cnt;
+        a.xvec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(a.X) & 15) == 0);
+        a.mu = mu; a.w2 = w2; a.c2d = c2d; a.g_out = g; a.llpart = llpart; a.ll_first = off == 0 ? 1 : 0; a.partials = partials;
+        a.status = status;
+        if (fit) { a.counts = fit->counts; a.stop_at = fit->stop_at; a.iter = fit->iter; }
+        const int64_t tp = (int64_t)pl.PT * (NT >> (a.lgG + a.lgS)), tiles = (cnt + tp - 1) / tp;
+        const int grid = (int)(tiles < ctas ? tiles : ctas);
+        cudaError_t e = direct_launch<DK_FUSED>(s, dim3((unsigned)grid), pl);
+        if (e != cudaSuccess) return e;
+        ReduceArgs r{};
+        r.D = D; r.K = K; r.splits = grid; r.partials = partials; r.g = g; r.Nk = Nk; r.S1 = S1; r.S2 = S2;
+        r.accumulate = (accumulate || off > 0) ? 1 : 0;
+        if (last) { r.llpart = llpart; r.n_ll = (int)ctas; r.ll = ll; r.ll_accumulate = accumulate ? 1 : 0; }
+        if (fit) {
+            r.stop_at = fit->stop_at; r.iter = fit->iter;
+            if (last) {
+                r.pi = fit->pi; r.mu = fit->mu; r.var = fit->var; r.var_floor = fit->var_floor; r.isotropic = fit->isotropic ? 1 : 0; r.N = n;
+                r.counts = fit->counts; r.status = status; r.w2 = w2; r.c2 = c2; r.c2d = c2d; r.ll_prev = fit->ll_prev; r.tol = fit->tol;
+            }
+        }
+        e = launch_chained(s, dim3((unsigned)K), 1024, 0, direct_reduce_kernel, r);
+        if (e != cudaSuccess) return e;
+        *launches += 2;
+    }
+    return cudaSuccess;
+}
+
+}  // namespace fg

@@ -24,6 +24,7 @@ struct DevResult {
     int n_ill;      // ill-conditioned components found by the tensor path's last preparation
     int counts[2];  // the last parameter update: variance entries raised to the floor, components left unchanged as empty
     int scr[SC_WORDS];      // control words of the screening path (D <= 128)
+    int stop_at;    // fits whose iterations are enqueued ahead: the iteration after which nothing is done any more
 };
 
 constexpr size_t STAGE_BYTES = (size_t)128 << 20;   // per staging buffer of the host-streaming path
@@ -743,6 +744,13 @@ int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, 
         KL(launch_reduce_tc(ctx->stream, D, K, Q, tb, Nk, S1, S2, true));
         return GMM_OK;
     }
+    if (fused_direct_supports(D, K)) {
+        CHECK(prof_begin(ctx));
+        CU(launch_fused_direct(ctx->stream, X, n, D, K, mu, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), ctx->partials(), ctx->llpart(), Nk, S1, S2,
+                               true, &ctx->result()->ll[slot], &ctx->result()->status, nullptr, &ctx->launches));
+        CHECK(prof_end(ctx));
+        return GMM_OK;
+    }
     const Fp32Plan plan = fp32_plan(D, K);
     for (int64_t off = 0; off < n; off += SUPER_TILE) {
         const int64_t cnt = (n - off < SUPER_TILE) ? (n - off) : SUPER_TILE;
@@ -751,7 +759,7 @@ int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, 
         KL(launch_lse_fp32(ctx->stream, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), ctx->center(), ctx->logZ2(), ctx->llpart()));
         KL(launch_mstep_fp32(ctx->stream, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), ctx->center(), ctx->logZ2(), ctx->partials(), plan));
         CHECK(prof_end(ctx));
-        KL(launch_reduce_ll(ctx->stream, ctx->llpart(), (cnt + FP32_TILE_P - 1) / FP32_TILE_P, &ctx->result()->ll[slot], true));
+        KL(launch_reduce_ll(ctx->stream, ctx->llpart(), fp32_ll_parts(cnt, D, K), &ctx->result()->ll[slot], true));
         KL(launch_reduce_partials(ctx->stream, D, K, plan.splits, ctx->partials(), ctx->center(), Nk, S1, S2, true));
     }
     return GMM_OK;
@@ -1081,6 +1089,43 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
     int t = 0;
+    if (fused_direct_supports(D, K) && (ctx->path == GMM_PATH_FP32 || (ctx->path == GMM_PATH_AUTO && gmm_auto_path(D, K) == GMM_PATH_FP32))) {
+        // Small mixtures: two launches per iteration (the update and the next iteration's constants are part of the reduction), as
+        // many iterations as there are slots for their log-likelihoods enqueued ahead; the device stops by itself where the
+        // tolerance is met or a step fails.
+        KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), nullptr, &ctx->result()->status));
+        CU(cudaMemsetAsync(&ctx->result()->stop_at, 0x7f, sizeof(int), ctx->stream));
+        ctx->last_path = GMM_PATH_FP32;
+        while (t < iters) {
+            const int end = iters - t < LL_SLOTS - 1 ? iters : t + LL_SLOTS - 1;      // (one slot holds the value before them)
+            for (int i = t; i < end; ++i) {
+                DirectFit f;
+                f.pi = pi; f.mu = mu; f.var = var; f.var_floor = var_floor; f.isotropic = ctx->covariance == GMM_COV_ISOTROPIC;
+                f.tol = tol; f.ll_prev = i > 0 ? &ctx->result()->ll[(i - 1) % LL_SLOTS] : nullptr;
+                f.counts = ctx->result()->counts; f.stop_at = &ctx->result()->stop_at; f.iter = i;
+                CHECK(prof_begin(ctx));
+                CU(launch_fused_direct(ctx->stream, X, N, D, K, mu, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), ctx->partials(), ctx->llpart(), Nk, S1,
+                                       S2, false, &ctx->result()->ll[i % LL_SLOTS], &ctx->result()->status, &f, &ctx->launches));
+                CHECK(prof_end(ctx));
+            }
+            DevResult r;
+            CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
+            CU(cudaStreamSynchronize(ctx->stream));
+            ctx->scr_active = 0;
+            const int done = r.stop_at < end ? r.stop_at + 1 : end;
+            for (; t < done; ++t) loglik_trace[t] = r.ll[t % LL_SLOTS];
+            int rc = report_status(ctx, r.status);
+            if (rc == GMM_OK && !std::isfinite(loglik_trace[t - 1]))
+                rc = fail(ctx, GMM_ENUMERIC, "log-likelihood is not finite (%g): non-finite values in X?", loglik_trace[t - 1]);
+            if (rc != GMM_OK) {
+                if (iters_done) *iters_done = t - 1;
+                return rc;
+            }
+            if (done < end || r.stop_at < end) break;
+        }
+        if (iters_done) *iters_done = t;
+        return GMM_OK;
+    }
     for (; t < iters; ++t) {
         const int slot = t % LL_SLOTS;
         // The update is skipped on the device when the step raised a status bit or left a non-finite log-likelihood
@@ -1757,7 +1802,7 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
         KL(launch_lse_fp32(ctx->stream, X + off * D, cnt, D, K, mu, ctx->w2(), ctx->c2d(), ctx->center(), ctx->logZ2(), ctx->llpart()));
         CHECK(prof_end(ctx));
         KL(launch_logz_out_fp32(ctx->stream, ctx->logZ2(), cnt, logp + off));
-        KL(launch_reduce_ll(ctx->stream, ctx->llpart(), (cnt + FP32_TILE_P - 1) / FP32_TILE_P, &ctx->result()->ll[0], true));
+        KL(launch_reduce_ll(ctx->stream, ctx->llpart(), fp32_ll_parts(cnt, D, K), &ctx->result()->ll[0], true));
     }
     ctx->last_path = GMM_PATH_FP32;
     double total = 0.0;

@@ -31,7 +31,7 @@ size_t fp32_partial_floats(int D, int K);   // floats in the per-CTA partial buf
 cudaError_t launch_prepare_fp32(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var,
                                 float* w2, float* c2, double* c2d, float* g, int* status);
 cudaError_t launch_center_fp32(cudaStream_t s, int D, int K, const float* mu, float* g);
-// log2-domain log Z of n points -> logZ2[n]; per-block float64 partial log-likelihoods -> llpart[ceil(n/64)]
+// log2-domain log Z of n points -> logZ2[n]; per-block float64 partial log-likelihoods -> llpart[fp32_ll_parts(n, D, K)]
 // c2d: the per-component constants in float64; logZ2: float64 (the kernels carry logits in float64 when D > 128)
 // g: the per-dimension centre subtracted from points and means before the products are formed (NULL = none; any value
 // gives the same mathematics, a centre near the data keeps the fp32 rounding small)
@@ -55,6 +55,34 @@ cudaError_t launch_topm_fp32(cudaStream_t s, const float* X, int64_t n, int D, i
                              const float* w2, const double* c2d, const float* g, int m, int32_t* idx, float* resp,
                              const int* run_if = nullptr, const int32_t* gather = nullptr, const int* gather_count = nullptr);
 
+// ---- the same, for D <= 128 (em_direct.cu; launch_lse_fp32 and launch_mstep_fp32 go there) ------------------------
+int lse_direct_parts(int64_t n, int D, int K);      // entries of llpart that launch_lse_fp32 writes for n points (D <= 128)
+cudaError_t launch_lse_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
+                              const double* c2d, const float* g, double* logZ2, double* llpart);
+cudaError_t launch_mstep_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
+                                const double* c2d, const float* g, const double* logZ2, float* partials, int splits);
+cudaError_t launch_reduce_direct(cudaStream_t s, int D, int K, int splits, const float* partials, const float* g, double* Nk,
+                                 double* S1, double* S2, bool accumulate);
+// One pass for K <= 64: statistics (+= when accumulate) and the log-likelihood of n points; g [D] receives the centre that the
+// kernels use.  partials as fp32_partial_floats(D, K), llpart: 296 entries.
+// fit: also the update of the parameters and their derived constants (w2, c2, c2d), nothing of which happens when an earlier
+// iteration set *stop_at: this one does when *status != 0 or the log-likelihood is not finite (the parameters are kept), or when the
+// tolerance is met.
+struct DirectFit {
+    float *pi, *mu, *var;
+    float var_floor;
+    bool isotropic;
+    double tol;
+    const double* ll_prev;      // NULL in the first iteration
+    int* counts;
+    int* stop_at;
+    int iter;
+};
+bool fused_direct_supports(int D, int K);
+cudaError_t launch_fused_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, float* w2, float* c2,
+                                double* c2d, float* g, float* partials, double* llpart, double* Nk, double* S1, double* S2,
+                                bool accumulate, double* ll, int* status, const DirectFit* fit, int64_t* launches);
+
 // ---- shared by all paths -------------------------------------------------------------------------------------
 // stats (+)= sum over `splits` partial blocks, fixed order, float64.  Partial layout: [splits][K + 2*K*D] floats,
 // each block being (N_k [K], sums of r (x - g) [K*D], sums of r (x - g)^2 [K*D]); float64 instead when
@@ -62,6 +90,8 @@ cudaError_t launch_topm_fp32(cudaStream_t s, const float* X, int64_t n, int D, i
 cudaError_t launch_reduce_partials(cudaStream_t s, int D, int K, int splits, const float* partials, const float* g,
                                    double* Nk, double* S1, double* S2, bool accumulate, const int* run_if = nullptr);
 // *ll (+)= sum of llpart[0..n) in a fixed order
+// (llpart entries of launch_lse_fp32: fp32_ll_parts)
+int fp32_ll_parts(int64_t n, int D, int K);
 cudaError_t launch_reduce_ll(cudaStream_t s, const double* llpart, int64_t n, double* ll, bool accumulate);
 // counts (may be NULL): counts[0] += variance entries raised to the floor, counts[1] += components left unchanged
 // because N_k < 1e-12 (integer atomics).  skip_status / skip_ll (may be NULL): the kernel writes nothing when

@@ -10,8 +10,8 @@ namespace {
 
 // Partials hold N_k and the sums of r (x - g), r (x - g)^2 about the per-dimension centre g (NULL = 0); with
 // S1c, S2c their totals over the splits,  S1 = S1c + g N_k,  S2 = S2c + 2 g S1c + g^2 N_k  (float64).
-template <typename T>
-__global__ void reduce_partials_kernel(int D, int K, int splits, const T* __restrict__ partials,
+// (The partials of the kernels for D > 128, float64.)
+__global__ void reduce_partials_kernel(int D, int K, int splits, const double* __restrict__ partials,
                                        const float* __restrict__ g, double* __restrict__ Nk, double* __restrict__ S1,
                                        double* __restrict__ S2, int accumulate, const int* __restrict__ run_if) {
     if (run_if && *run_if == 0) return;                  // (the kernel that fills the partials did not run either)
@@ -19,19 +19,19 @@ __global__ void reduce_partials_kernel(int D, int K, int splits, const T* __rest
     const size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= per) return;
     double s = 0.0;
-    for (int p = 0; p < splits; ++p) s += (double)partials[(size_t)p * per + e];      // fixed order
+    for (int p = 0; p < splits; ++p) s += partials[(size_t)p * per + e];      // fixed order
     double* dst = (e < (size_t)K) ? (Nk + e) : (e < K + KD) ? (S1 + (e - K)) : (S2 + (e - K - KD));
     if (g && e >= (size_t)K) {
         const size_t j = (e < K + KD) ? (e - K) : (e - K - KD);
         const size_t k = j / D;
         const double gd = (double)g[j % D];
         double nk = 0.0;
-        for (int p = 0; p < splits; ++p) nk += (double)partials[(size_t)p * per + k];
+        for (int p = 0; p < splits; ++p) nk += partials[(size_t)p * per + k];
         if (e < K + KD) {
             s += gd * nk;
         } else {
             double s1c = 0.0;
-            for (int p = 0; p < splits; ++p) s1c += (double)partials[(size_t)p * per + K + j];
+            for (int p = 0; p < splits; ++p) s1c += partials[(size_t)p * per + K + j];
             s += 2.0 * gd * s1c + gd * gd * nk;
         }
     }
@@ -131,11 +131,9 @@ cudaError_t launch_reduce_partials(cudaStream_t s, int D, int K, int splits, con
                                    double* Nk, double* S1, double* S2, bool accumulate, const int* run_if) {
     const size_t per = (size_t)K + 2 * (size_t)K * D;
     const unsigned blocks = (unsigned)((per + 255) / 256);
-    if (fp32_plan(D, K).wide)
-        reduce_partials_kernel<double><<<blocks, 256, 0, s>>>(D, K, splits, reinterpret_cast<const double*>(partials), g, Nk, S1, S2,
-                                                              accumulate ? 1 : 0, run_if);
-    else
-        reduce_partials_kernel<float><<<blocks, 256, 0, s>>>(D, K, splits, partials, g, Nk, S1, S2, accumulate ? 1 : 0, run_if);
+    if (!fp32_plan(D, K).wide) return launch_reduce_direct(s, D, K, splits, partials, g, Nk, S1, S2, accumulate);      // (nobody gates those shapes)
+    reduce_partials_kernel<<<blocks, 256, 0, s>>>(D, K, splits, reinterpret_cast<const double*>(partials), g, Nk, S1, S2,
+                                                  accumulate ? 1 : 0, run_if);
     return cudaGetLastError();
 }
 

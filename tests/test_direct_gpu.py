@@ -1,0 +1,83 @@
+"""The FP32 path for D <= 128 (csrc/em_direct.cu): tiles cut to the shape, whole fits enqueued ahead."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import gmm_oracle as orc
+from tests.parity_util import assert_stats_close, data_scale
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def fg():
+    from paper_2606_10896_b200 import flashgmm
+
+    return flashgmm
+
+
+def _t(a):
+    return torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float32, device=DEV).contiguous()
+
+
+def _mixture(N, D, K, seed):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    mu = rng.normal(0, 1.5, (K, D))
+    X = mu[rng.integers(0, K, N)] + rng.standard_normal((N, D)) + 3.0
+    return (X.astype(np.float32), rng.dirichlet(np.ones(K)).astype(np.float32), (mu + 3.0).astype(np.float32),
+            rng.uniform(0.5, 2.0, (K, D)).astype(np.float32))
+
+
+# component groups of four, blocks of 64, chunks of four dimensions, tiles of 4 to 256 points, lanes that share dimensions
+@pytest.mark.parametrize("N,D,K", [(1, 1, 1), (257, 2, 4), (1000, 3, 5), (63, 128, 1), (999, 127, 9), (4097, 31, 16), (300, 33, 17), (20000, 4, 3),
+                                   (5000, 100, 63), (4100, 128, 64), (30011, 8, 12), (3000, 6, 65), (2500, 40, 200), (700, 128, 130)])
+def test_direct_step_at_the_edges_of_its_tiles(fg, N, D, K):
+    X, pi, mu, var = _mixture(N, D, K, N + D + K)
+    if K > 2:
+        pi[1] = 0.0
+    ref = orc.em_step(X, pi, mu, var)
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        out = [[v.cpu().numpy() if torch.is_tensor(v) else v for v in c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))] for _ in range(2)]
+        logp, total = c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var))
+    assert all(np.array_equal(a, b) for a, b in zip(*out))      # the same bits in every run
+    assert abs(out[0][3] - ref[3]) <= 1e-5 * abs(ref[3]) + 1e-6 and abs(total - ref[3]) <= 1e-5 * abs(ref[3]) + 1e-6
+    assert_stats_close(N, max(1.0, data_scale(X)), out[0][:3], ref[:3], f"N={N} D={D} K={K}")
+
+
+@pytest.mark.parametrize("isotropic", [False, True])
+def test_direct_fit_runs_ahead_and_stops_by_itself(fg, isotropic):
+    # more iterations than there are slots for log-likelihoods; then with a tolerance that the fit meets on its way
+    X, pi, mu, var = _mixture(3000, 7, 6, 3)
+    if isotropic:
+        var = np.repeat(var[:, :1], 7, 1)
+    step = orc.em_iteration_isotropic if isotropic else orc.em_iteration
+    iters, want, p = 150, [], (pi, mu, var)
+    for _ in range(iters):
+        *p, ll = step(X, *p, 1e-6)[:4]
+        want.append(ll)
+    want = np.array(want)
+    with fg.Context(0) as c:
+        c.gmm_set_covariance(fg.GMM_COV_ISOTROPIC if isotropic else fg.GMM_COV_DIAG)
+        a = [_t(pi), _t(mu), _t(var)]
+        trace, done = c.gmm_fit(_t(X), *a, iters, 1e-6)
+        assert done == len(trace) == iters and np.all(np.abs(trace - want) <= 2e-5 * np.abs(want))
+        b = [_t(pi), _t(mu), _t(var)]
+        short, n = c.gmm_fit(_t(X), *b, iters, 1e-6, tol=1e-6)
+        assert 1 < n < iters and np.array_equal(short, trace[:n])
+        change = np.abs(np.diff(short)) / np.abs(short[1:])
+        assert change[-1] <= 1e-6 and np.all(change[:-1] > 1e-6)
+        d = [_t(pi), _t(mu), _t(var)]
+        c.gmm_fit(_t(X), *d, n, 1e-6)
+        assert all(torch.equal(u, v) for u, v in zip(b, d))      # nothing was done after the iteration that met the tolerance
+
+
+def test_direct_fit_keeps_the_parameters_of_a_step_that_fails(fg):
+    X, pi, mu, var = _mixture(500, 5, 4, 9)
+    X[17, 2] = np.nan
+    with fg.Context(0) as c:
+        a = [_t(pi), _t(mu), _t(var)]
+        with pytest.raises(fg.GmmError):
+            c.gmm_fit(_t(X), *a, 5, 1e-6)
+        assert all(np.array_equal(u.cpu().numpy(), v) for u, v in zip(a, (pi, mu, var)))

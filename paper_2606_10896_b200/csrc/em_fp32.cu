@@ -534,7 +534,9 @@ __global__ void prepare_fp32_kernel(int D, int K, const float* __restrict__ pi, 
 // g[d] = mean over the components of mu[k][d]: the centre the tile routine subtracts from points and means.  A block takes
 // 32 dimensions; its 32 warps sum every 32nd component in float64 and the 32 partial sums are added in a fixed order.  A
 // non-finite mean (reported through the status word by prepare_fp32_kernel) gives centre 0.
-__global__ void __launch_bounds__(1024) center_fp32_kernel(int D, int K, const float* __restrict__ mu, float* __restrict__ g) {
+__global__ void __launch_bounds__(1024) center_fp32_kernel(int D, int K, const float* __restrict__ mu, float* __restrict__ g,
+                                                           const int* __restrict__ run_if) {
+    if (run_if && *run_if == 0) return;
     __shared__ double part[32][33];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int d = blockIdx.x * 32 + lane;
@@ -590,8 +592,8 @@ size_t fp32_partial_floats(int D, int K) {
     return (size_t)p.splits * ((size_t)K + 2 * (size_t)K * D) * (p.wide ? 2 : 1);
 }
 
-cudaError_t launch_center_fp32(cudaStream_t s, int D, int K, const float* mu, float* g) {
-    center_fp32_kernel<<<(unsigned)((D + 31) / 32), 1024, 0, s>>>(D, K, mu, g);
+cudaError_t launch_center_fp32(cudaStream_t s, int D, int K, const float* mu, float* g, const int* run_if) {
+    center_fp32_kernel<<<(unsigned)((D + 31) / 32), 1024, 0, s>>>(D, K, mu, g, run_if);
     return cudaGetLastError();
 }
 

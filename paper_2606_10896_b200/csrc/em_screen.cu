@@ -383,6 +383,7 @@ struct SweepParams {
     int* ovf;
     int* ctl;
     int* status;
+    int tile_limit, tile_over;      // marks, and points without a list, in a CTA's first tile above which the data counts as dense at once
 };
 
 static_assert(SW_ENT + SW_SPILL <= 32, "a mask of a point's entries");
@@ -399,18 +400,26 @@ static_assert(SW_SPILL == SCR_SPILL, "room for the spilled entries");
 // MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles, 65 us per 2^18 points at D = 128, K = 1024; it takes 115 us: the two
 // halves' MMA and softmax warps wait for one another (a thread that reads its 128 values holds the half's accumulators up, and
 // tensor memory has no room for a second set beside the operands).  126 us with one MMA warp for both halves, 142 with its votes.
+//
+// TOP: how many of a point's largest values are wanted for certain.  1: everything within the margin of the largest.  More (the top-m
+// assignment): also everything that could be among the TOP largest.  The bound for those is the TOP-th largest of the lower bounds of
+// the quarters of every block: different components, so the TOP-th largest value cannot be below it.  It rises slowly as the sweep
+// goes on, so the tile's components pass twice, once for the bound and once for the marks: in one pass what was marked under
+// early bounds cost more evaluations than the second pass takes (1M x 128, K = 1024: top-2 1.40 ms in one pass, top-4 3.2).
+template <int TOP>
 __global__ void __launch_bounds__(SW_THREADS, 1)
 screen_sweep_kernel(const SweepParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s, drain_s;
+    __shared__ int abort_s, drain_s, first_marks, first_warps;
     if (p.ctl[SC_DENSE] != 0) return;
     volatile int* abort_flag = &abort_s;
     volatile int* drain_flag = &drain_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t ntiles = (p.n + SCR_TILE - 1) / SCR_TILE;
     const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    constexpr int PASSES = TOP > 1 ? 2 : 1;
     const int NG = p.NG, spg = (p.KA + 1) >> 1, cslots = SW_PS / spg;      // stages per group; groups in flight
     unsigned char* cons = smem + SW_UOFF + 256 * 16 * p.chunks;            // [cslots][4096]
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SW_BOFF);
@@ -418,6 +427,7 @@ screen_sweep_kernel(const SweepParams p) {
     if (tid == 0) {
         abort_s = 0;
         drain_s = 0;
+        first_marks = first_warps = 0;
         for (int i = 0; i < SB_COUNT; ++i) {
             const bool wg = (i >= SB_AFULL && i < SB_AFULL + 2) || (i >= SB_LEMPTY && i < SB_LEMPTY + 2);
             const bool both = i >= SB_PEMPTY && i < SB_PEMPTY + SW_PS;           // (released by the MMA warps of both halves)
@@ -489,9 +499,11 @@ screen_sweep_kernel(const SweepParams p) {
             bar_arrive(BAR(SB_AFULL + half));
         };
         float nrm_next = 0.f;
+        int dense_next = 0;
         auto norm_load = [&](int64_t i) {
             const int64_t r = (blockIdx.x + i * gridDim.x) * SCR_TILE + tid;
             nrm_next = (i < ntl && r < p.n) ? __ldg(p.n2 + r) : 0.f;
+            dense_next = __ldcg(p.ctl + SC_DENSE);
         };
         if (ntl > 0) {
             norm_load(0);
@@ -502,11 +514,20 @@ screen_sweep_kernel(const SweepParams p) {
             const int64_t row = wrow + lane;
             const bool in = row < p.n;
             const float nrm = nrm_next;
+            if (__any_sync(0xffffffffu, dense_next != 0)) {  // (some CTA has found the data dense: all roles leave)
+                *abort_flag = 1;
+                break;
+            }
             float thr = -CUDART_INF_F;                       // the largest lower bound so far
-            int ne = 0;
+            float low[TOP];                                  // TOP > 1: the largest ones, in order
+#pragma unroll
+            for (int j = 0; j < TOP; ++j) low[j] = -CUDART_INF_F;
+            // what a value has to reach
+            auto floor_now = [&]() -> float { return TOP == 1 ? thr - p.margin : fmaxf(fminf(low[0] - p.margin, low[TOP - 1]), 0.5f * SCR_NEVER); };
+            int ne = 0, packs = 0;
             float lost = -CUDART_INF_F;                      // largest upper bound of a block with marks that found no room
             // 32 accumulators of the point = approximate values: the block's largest; marks.
-            auto block = [&](const uint32_t (&v)[32], int bn) {
+            auto block = [&](const uint32_t (&v)[32], int bn, bool first) {
                 float mx[4];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
@@ -514,12 +535,32 @@ screen_sweep_kernel(const SweepParams p) {
                     mx[j] = max3(mx[j], __uint_as_float(v[8 * j + 3]), __uint_as_float(v[8 * j + 4]));
                     mx[j] = max3(mx[j], __uint_as_float(v[8 * j + 5]), __uint_as_float(v[8 * j + 6]));
                 }
-                mx[0] = max3(mx[0], __uint_as_float(v[7]), __uint_as_float(v[15]));
-                mx[1] = max3(mx[1], __uint_as_float(v[23]), __uint_as_float(v[31]));
+                if (TOP == 1) {
+                    mx[0] = max3(mx[0], __uint_as_float(v[7]), __uint_as_float(v[15]));
+                    mx[1] = max3(mx[1], __uint_as_float(v[23]), __uint_as_float(v[31]));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) mx[j] = fmaxf(mx[j], __uint_as_float(v[8 * j + 7]));
+                }
                 const float2 ab = blk[bn];
                 const float bmax = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]), E = fmaf(ab.y, nrm, fabsf(ab.x));
-                if (!(ab.x < 0.f)) thr = fmaxf(thr, bmax - E);
-                const float cut = thr - p.margin - E;
+                if (TOP == 1) {
+                    if (!(ab.x < 0.f)) thr = fmaxf(thr, bmax - E);
+                } else if (first) {
+                    if (!(ab.x < 0.f) && bmax - E > low[TOP - 1])
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float x = mx[q] - E;
+#pragma unroll
+                        for (int j = 0; j < TOP; ++j) {
+                            const float keep = fmaxf(low[j], x);
+                            x = fminf(low[j], x);
+                            low[j] = keep;
+                        }
+                    }
+                }
+                if (TOP > 1 && first) return;
+                const float cut = floor_now() - E;
                 if (in && bmax >= cut && bmax > 0.5f * SCR_NEVER) {
                     // bit j of the mask: value j reaches the cut (the sign of l - cut, shifted in from the top)
                     const uint64_t nc = pack2(__float_as_uint(-cut), __float_as_uint(-cut));
@@ -531,11 +572,12 @@ screen_sweep_kernel(const SweepParams p) {
                         mask = __funnelshift_l(__float_as_uint(lo2(d)), mask, 1);
                     }
                     mask = ~mask;
-                    if (ne == SW_ENT + SW_SPILL) {           // drop what the bound found meanwhile rules out
-                        int m = 0;
+                    if (ne == SW_ENT + SW_SPILL && packs < 2) {      // drop what the bound found meanwhile rules out (of broad posteriors:
+                        int m = 0;                                   // nothing; trying at every block took a millisecond per tile)
+                        ++packs;
                         for (int e = 0; e < SW_ENT + SW_SPILL; ++e) {
                             const unsigned long long w = ent(e);
-                            if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= thr - p.margin) ent(m++) = w;
+                            if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= floor_now()) ent(m++) = w;
                         }
                         ne = m;
                     }
@@ -549,8 +591,9 @@ screen_sweep_kernel(const SweepParams p) {
                     }
                 }
             };
-            for (int g = 0; g < NG; ++g, ++gi) {
-                const bool last = g + 1 == NG;
+            for (int gg = 0; gg < PASSES * NG; ++gg, ++gi) {
+                const bool last = gg + 1 == PASSES * NG, first = gg < NG;
+                const int g = (PASSES > 1 && !first) ? gg - NG : gg;
                 if (last) norm_load(i + 1);
                 const bool got = bar_wait(BAR(SB_LFULL + half), gi & 1u, abort_flag, p.status, false);
                 const bool ok = __all_sync(0xffffffffu, got);
@@ -566,15 +609,15 @@ screen_sweep_kernel(const SweepParams p) {
                 fence_before();
                 bar_arrive(BAR(SB_LEMPTY + half));
                 if (ok) {
-                    block(v0, g * 4);
-                    block(v1, g * 4 + 1);
-                    block(v2, g * 4 + 2);
-                    block(v3, g * 4 + 3);
+                    block(v0, g * 4, first);
+                    block(v1, g * 4 + 1, first);
+                    block(v2, g * 4 + 2, first);
+                    block(v3, g * 4 + 3, first);
                 }
             }
             // the point's list: the words (block of 32 positions, mask) that the final bound leaves
             int cnt = 0, nw = 0;
-            const float fin = thr - p.margin;
+            const float fin = floor_now();
             bool over = !(nrm < CUDART_INF_F) || (lost >= fin && lost > -CUDART_INF_F);
             // (the entries in shared memory all at once: one after the other, each waited for, they took ten times as long,
             // and the tensor cores waited with them)
@@ -597,7 +640,7 @@ screen_sweep_kernel(const SweepParams p) {
             }
             if (!in || over) cnt = 0, keep = 0;
             nw = __popc(keep);
-            if (cnt == 0 || nw > 15) over = true;                       // (a point further from everything than a float16 sum can tell)
+            if (cnt < TOP || nw > 15) over = true;                      // (a point further from everything than a float16 sum can tell)
             if (over) cnt = nw = 0, keep = 0;
             int inc = cnt | (nw << 16);                      // running sums of both over the warp
 #pragma unroll
@@ -625,9 +668,29 @@ screen_sweep_kernel(const SweepParams p) {
                         }
                 }
             }
+            if (i == 0) {
+                // Broad posteriors show at once: more marks than allowed (and a tenth) in a CTA's first tile, and the sweep ends (the whole
+                // of it, for nothing, cost data of few dimensions a fifth of the step).  The data alone decide, not the timing.
+                const int mine = __reduce_add_sync(0xffffffffu, !in ? 0 : over ? 1 << 20 : cnt);      // (a warp marks at most 512)
+                if (lane == 0) {
+                    atomicAdd(&first_marks, mine);
+                    __threadfence_block();
+                    if (atomicAdd(&first_warps, 1) == 7) {
+                        const int all = atomicAdd(&first_marks, 0), rows = all >> 20;
+                        if ((all & 0xfffff) + 64 * rows > p.tile_limit || rows > p.tile_over) {
+                            p.ctl[SC_DENSE] = 1;
+                            *abort_flag = 1;
+                        }
+                    }
+                }
+                __syncwarp();
+                if (*abort_flag) break;
+            }
         }
-        marks = __reduce_add_sync(0xffffffffu, marks);
-        if (lane == 0 && marks > 0) atomicAdd(p.ctl + SC_MARKS, marks);
+        if (ntl > 0 && !*abort_flag) {
+            marks = __reduce_add_sync(0xffffffffu, marks);
+            if (lane == 0 && marks > 0) atomicAdd(p.ctl + SC_MARKS, marks);
+        }
     } else if (warp == SW_PRODUCER) {
         // =========================== producer warp (TMA) ===========================
         const uint32_t ubytes = 256u * 16u * (uint32_t)p.chunks;
@@ -653,13 +716,13 @@ screen_sweep_kernel(const SweepParams p) {
         };
         if (ntl > 0) load_rows(0);
         for (int64_t i = 0; i < ntl && ok; ++i)
-            for (int g = 0; g < NG && ok; ++g) {
+            for (int g = 0; g < PASSES * NG && ok; ++g) {
                 for (int z = 0; z < spg && ok; ++z) {
                     const uint32_t slot = ps % SW_PS;        // (a power of two)
                     if (ps >= SW_PS) ok = wait_slot(SB_PEMPTY + slot, (ps / SW_PS - 1) & 1u);
                     if (!ok) break;
                     if (elect_one()) {
-                        const unsigned char* src = p.img + (size_t)g * p.gbytes;
+                        const unsigned char* src = p.img + (size_t)(PASSES > 1 && g >= NG ? g - NG : g) * p.gbytes;
                         const uint32_t bytes = min(p.KA - 2 * z, 2) * 16384u;
                         bar_expect_tx(BAR(SB_PFULL + slot), bytes + (z == 0 ? SW_CSLOT : 0));
                         if (z == 0) bulk(cons + cslot * SW_CSLOT, src, SW_CSLOT, BAR(SB_PFULL + slot));
@@ -672,7 +735,7 @@ screen_sweep_kernel(const SweepParams p) {
                 // the next tile's rows as soon as both halves have taken this tile's (which they do before its first products);
                 // no stage waits for that except behind the tile's last one
                 if (ok && ut == (uint32_t)(i + 1) && i + 1 < ntl) {
-                    uint32_t free_now = (g + 1 == NG) ? 1u : 0u;
+                    uint32_t free_now = (g + 1 == PASSES * NG) ? 1u : 0u;
                     if (free_now) ok = wait_slot(SB_UEMPTY, (uint32_t)(i & 1));
                     else {
                         if (lane == 0) free_now = bar_test(BAR(SB_UEMPTY), (uint32_t)(i & 1)) ? 1u : 0u;
@@ -708,7 +771,7 @@ screen_sweep_kernel(const SweepParams p) {
             uint32_t gi = 0;
             bool alive = true;
             for (int64_t i = 0; i < ntl && alive; ++i) {
-                for (int g = 0; g < NG && alive; ++g, ++gi) {
+                for (int g = 0; g < PASSES * NG && alive; ++g, ++gi) {
                     if (g == 0) alive = wait(SB_AFULL + h, (uint32_t)(i & 1));
                     if (alive && gi >= 1) alive = wait(SB_LEMPTY + h, (gi - 1) & 1u);
                     for (int z = 0; z < spg && alive; ++z) {
@@ -747,11 +810,17 @@ screen_sweep_kernel(const SweepParams p) {
 }
 
 // ------------------------------------------------------------------------------------------------------------------
+__device__ __forceinline__ float warp_maxf(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
 // Rows that left the sweep without a list (marks in too many groups of components, a coordinate beyond the fp16 range): all K
 // components exactly, the list from those values.  Four rows per CTA and step, a warp per component.  Also the verdict on the
 // piece: with too many such rows, or too many pairs, SC_DENSE is set and nothing after this kernel does anything.
 constexpr int OV_ROWS = 4;
-__global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restrict__ X, int64_t n, int D, int K, float margin,
+__global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restrict__ X, int64_t n, int D, int K, float margin, int top,
                                                           long long max_marks, const float* __restrict__ mu, const float* __restrict__ w2,
                                                           const double* __restrict__ c2d, const int* __restrict__ ovf,
                                                           unsigned* __restrict__ pt_off, int* __restrict__ pt_cnt,
@@ -797,7 +866,23 @@ __global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restric
             for (int k = lane; k < K; k += 32) best = fmaxf(best, l[k]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-            const float cut = best - margin - 0.01f;
+            float cut = best - margin - 0.01f;
+            if (top > 1) {                                   // and what the `top` largest reach (-inf: all components)
+                float kth = CUDART_INF_F;
+                for (int left = top; left > 0;) {
+                    float b = -CUDART_INF_F;
+                    int same = 0;
+                    for (int k = lane; k < K; k += 32) {
+                        const float v = l[k];
+                        if (v < kth) { if (v > b) { b = v; same = 1; } else if (v == b) ++same; }
+                    }
+                    const float m = warp_maxf(b);
+                    left -= __reduce_add_sync(0xffffffffu, b == m ? same : 0);
+                    kth = m;
+                    if (m == -CUDART_INF_F) break;
+                }
+                cut = fminf(cut, kth);
+            }
             int cnt = 0;
             for (int k0 = 0; k0 < K; k0 += 32) {
                 const bool is = k0 + lane < K && best > -CUDART_INF_F && l[k0 + lane] >= cut;
@@ -831,6 +916,8 @@ __global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restric
 // and then a lane per point reads its values back.  (Eight lanes per POINT took the time of the longest of four lists.)
 // Bound by instruction issue and the trips to L2 for the components' rows (1 KB per pair at D = 128).
 constexpr int EV_VALS = 32 * SCR_SLOTS;
+// TOP: the m (<= 4) largest values go out, the smaller component first where two are equal.
+struct TopOut { int m; float* resp; };
 template <int MODE>
 __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __restrict__ mu,
                                                              const float* __restrict__ w2, const double* __restrict__ c2d,
@@ -839,7 +926,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                                                              const unsigned* __restrict__ pt_off, int* __restrict__ pt_cnt,
                                                              unsigned short* __restrict__ ids, float* __restrict__ val,
                                                              int* __restrict__ counts, double* __restrict__ ll, float* __restrict__ logp,
-                                                             int32_t* __restrict__ idx, const int* __restrict__ ctl) {
+                                                             int32_t* __restrict__ idx, const int* __restrict__ ctl, const TopOut top) {
     if (ctl[SC_DENSE] != 0) return;
     extern __shared__ int hist[];                    // [K] (unless MODE == SCREEN_LOGP)
     __shared__ float v_s[8][EV_VALS];                // values of the warp's pairs, by place in its part of the lists
@@ -848,7 +935,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
     __shared__ double red[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l8 = lane & 7;
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0);
-    const bool histogram = MODE != SCREEN_LOGP && counts != nullptr;
+    const bool histogram = MODE != SCREEN_LOGP && MODE != SCREEN_TOP && counts != nullptr;
     if (histogram) {
         for (int k = tid; k < K; k += 256) hist[k] = 0;
         __syncthreads();
@@ -981,6 +1068,32 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
 #pragma unroll
             for (int x = 16; x > 0; x >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, x);
             const float lz = m + log2f(sm);
+            if (MODE == SCREEN_TOP) {
+                float pv = CUDART_INF_F;                     // the pair that went out last
+                int pk = -1;
+                for (int r = 0; r < top.m; ++r) {
+                    float bv = -CUDART_INF_F;
+                    int bk = 0x7fffffff;
+                    for (int j = lane; j < c; j += 32) {
+                        const float v = val[o + j];
+                        const int k = ids[o + j];
+                        const bool after = v < pv || (v == pv && k > pk);
+                        if (after && (v > bv || (v == bv && k < bk))) { bv = v; bk = k; }
+                    }
+#pragma unroll
+                    for (int x = 16; x > 0; x >>= 1) {
+                        const float ov = __shfl_xor_sync(0xffffffffu, bv, x);
+                        const int ok = __shfl_xor_sync(0xffffffffu, bk, x);
+                        if (ov > bv || (ov == bv && ok < bk)) { bv = ov; bk = ok; }
+                    }
+                    if (lane == 0) {
+                        idx[(row0 + src) * top.m + r] = bk == 0x7fffffff ? 0 : bk;
+                        if (top.resp) top.resp[(row0 + src) * top.m + r] = fast_ex2(bv - lz);
+                    }
+                    pv = bv;
+                    pk = bk;
+                }
+            }
             int kp = 0;
             if (MODE == SCREEN_EM)
                 for (int j0 = 0; j0 < c; j0 += 32) {
@@ -1001,7 +1114,26 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                 }
             if (lane == src) { mx = m; sum = sm; best = b; kept = kp; }
         }
-        if (MODE == SCREEN_LOGP) {
+        if (MODE == SCREEN_TOP) {
+            if (in && listed) {
+                const float lz = mx + log2f(sum);
+                float pv = CUDART_INF_F;                     // the pair that went out last
+                int pk = -1;
+                for (int r = 0; r < top.m; ++r) {
+                    float bv = -CUDART_INF_F;
+                    int bk = alone ? only : 0;
+                    for (int j = 0; j < todo; ++j) {
+                        const float v = v_s[warp][p0 + j];
+                        const int k = k_s[warp][p0 + j];
+                        if ((v < pv || (v == pv && k > pk)) && (v > bv || (v == bv && k < bk))) { bv = v; bk = k; }
+                    }
+                    idx[row * top.m + r] = bk;
+                    if (top.resp) top.resp[row * top.m + r] = alone ? 1.f : fast_ex2(bv - lz);
+                    pv = bv;
+                    pk = bk;
+                }
+            }
+        } else if (MODE == SCREEN_LOGP) {
             if (in) {
                 const double lz = cnt > 0 ? (double)mx + (double)log2f(sum) : -CUDART_INF;
                 logp[row] = (float)(lz * 0.69314718055994530942);
@@ -1050,7 +1182,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
         __syncthreads();
         for (int k = tid; k < K; k += 256) counts[(size_t)blockIdx.x * K + k] = hist[k];
     }
-    if (MODE != SCREEN_ARGMAX && ll) {
+    if (MODE != SCREEN_ARGMAX && MODE != SCREEN_TOP && ll) {
         ll_acc = warp_sum(ll_acc);
         if (lane == 0) red[warp] = ll_acc;
         __syncthreads();
@@ -1592,7 +1724,7 @@ cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi,
     return cudaGetLastError();
 }
 
-cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, float max_marks,
+cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, int top, float max_marks, bool stats,
                                 const float* mu, const float* w2, const double* c2d, const ScreenBuffers& b, int* status, int sms,
                                 int64_t* launches) {
     if (n < 1 || n > SCR_PIECE) return cudaErrorInvalidValue;
@@ -1621,24 +1753,28 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
     p.chunks = screen_chunks(D); p.y = b.y; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
     p.blk = b.blk; p.n2 = b.n2; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
     p.ovf = b.ovf; p.ctl = b.ctl; p.status = status;
-    cudaError_t e = cudaFuncSetAttribute(screen_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);
+    p.tile_limit = (int)fmin(1.1 * (double)max_marks * SCR_TILE, 1e9);
+    p.tile_over = n >= 65536 ? SCR_TILE / 32 : SCR_TILE;      // (the share of rows that screen_rows_kernel takes)
+    if (top < 1 || top > 4) return cudaErrorInvalidValue;
+    auto sweep = top == 1 ? screen_sweep_kernel<1> : top == 2 ? screen_sweep_kernel<2> : screen_sweep_kernel<4>;
+    cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (n + SCR_TILE - 1) / SCR_TILE;
     if (sms > SCR_MAX_SMS) sms = SCR_MAX_SMS;
-    screen_sweep_kernel<<<(unsigned)(tiles < sms ? tiles : sms), SW_THREADS, SW_SMEM, s>>>(p);
+    sweep<<<(unsigned)(tiles < sms ? tiles : sms), SW_THREADS, SW_SMEM, s>>>(p);
     LCHECK();
     const size_t smem = (size_t)OV_ROWS * K * 4;
     e = cudaFuncSetAttribute(screen_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const double most = fmin((double)max_marks * (double)n, (double)SCR_PIECE * SCR_MARKS);
-    screen_rows_kernel<<<(unsigned)(2 * sms), 256, smem, s>>>(X, n, D, K, margin, (long long)most, mu, w2, c2d, b.ovf,
+    const double most = fmin((double)max_marks * (double)n, (double)SCR_PIECE * (stats ? SCR_MARKS : SCR_SLOTS));
+    screen_rows_kernel<<<(unsigned)(2 * sms), 256, smem, s>>>(X, n, D, K, margin, top, (long long)most, mu, w2, c2d, b.ovf,
                                                               b.pt_off, b.pt_cnt, b.ids, b.ctl);
     *launches += 3;
     return cudaGetLastError();
 }
 
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
-                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count) {
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count, int m, float* resp) {
     // 32 points per warp (fewer where that leaves the chip short of warps); ranges as launch_screen_stats has them
     const int pw = n < 131072 ? 8 : n < 200000 ? 16 : 32, range = count ? screen_range(n) : 8 * pw;
     const unsigned blocks = (unsigned)((n + range - 1) / range);
@@ -1648,11 +1784,25 @@ cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t
     if (e == cudaSuccess) e = cudaFuncSetAttribute(screen_eval_kernel<SCREEN_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4);
     if (e != cudaSuccess) return e;
     if (mode == SCREEN_EM)
-        screen_eval_kernel<SCREEN_EM><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, nullptr, nullptr, b.ctl);
+        screen_eval_kernel<SCREEN_EM><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, nullptr, nullptr, b.ctl, TopOut{});
     else if (mode == SCREEN_LOGP)
-        screen_eval_kernel<SCREEN_LOGP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, b.ll, logp, nullptr, b.ctl);
+        screen_eval_kernel<SCREEN_LOGP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, b.ll, logp, nullptr, b.ctl, TopOut{});
+    else if (mode == SCREEN_TOP)
+        screen_eval_kernel<SCREEN_TOP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, nullptr, nullptr, idx, b.ctl, TopOut{m, resp});
     else
-        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, nullptr, nullptr, idx, b.ctl);
+        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, nullptr, nullptr, idx, b.ctl, TopOut{});
+    return cudaGetLastError();
+}
+
+// One thread: which kernels of an asynchronous assignment have the word.  gate (the tile kernels return when it is not 0) also counts
+// a screening pass that covered the call; fallback says whether the FP32 kernels run.
+__global__ void screen_gate_kernel(const int* __restrict__ ctl, int* __restrict__ gate, int* __restrict__ fallback) {
+    const bool dense = ctl[SC_DENSE] != 0;
+    *fallback = dense && *gate != 0 ? 1 : 0;
+    if (!dense) *gate = 1;
+}
+cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback) {
+    screen_gate_kernel<<<1, 1, 0, s>>>(b.ctl, gate, fallback);
     return cudaGetLastError();
 }
 

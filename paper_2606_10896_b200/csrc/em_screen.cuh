@@ -34,6 +34,7 @@ enum { SC_DENSE = 0,      // set when a piece marks too many pairs: later kernel
        SC_TICKET_A, SC_TICKET_B,
        SC_ACTIVE,         // components with a weight
        SC_KEPT,           // kept pairs of all pieces (saturating)
+       SC_FALLBACK,       // an assignment that the FP32 kernels have to do (see launch_screen_gate)
        SC_WORDS };
 
 struct ScreenBuffers {
@@ -74,16 +75,20 @@ __host__ __device__ inline size_t screen_group_bytes(int D) { return 4096 + (siz
 cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
                                   const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
 // One piece of n <= SCR_PIECE points: plane, sweep, rows without a list.  margin: log2 units below a point's best value down to
-// which pairs are marked (40, or 0 for the arg-max alone).  max_marks: pairs per point up to which the screening pays.
-cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, float max_marks,
+// which pairs are marked (40, or 0 for the arg-max alone); top: so many of its largest pairs are marked in any case (1 to 4).  max_marks: pairs per point up to which the screening pays; stats:
+// statistics are to follow, which have room for SCR_MARKS of them.
+cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, int top, float max_marks, bool stats,
                                 const float* mu, const float* w2, const double* c2d, const ScreenBuffers& b, int* status, int sms,
                                 int64_t* launches);
 // Exact values of the marked pairs.  SCREEN_EM: responsibilities of the pairs within 2^-40 of their point's total, counted per
 // component; SCREEN_LOGP: logp[i]; SCREEN_ARGMAX: idx[i], and the pair itself kept with weight 1 for the statistics.
-enum { SCREEN_EM = 0, SCREEN_LOGP = 1, SCREEN_ARGMAX = 2 };
+// SCREEN_TOP: the m largest pairs of every point into idx [n][m] and (may be NULL) their responsibilities into resp [n][m].
+enum { SCREEN_EM = 0, SCREEN_LOGP = 1, SCREEN_ARGMAX = 2, SCREEN_TOP = 3 };
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
-                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count = true);
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count = true, int m = 1, float* resp = nullptr);
 // (count: leave the number of kept pairs per component and range for launch_screen_stats)
+// After the last piece of an asynchronous assignment: *gate |= the screening covered the call; *fallback = it did not and *gate was set.
+cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback);
 // Statistics of the kept pairs: sorted by component, summed in fixed segments, added to (Nk, S1, S2) in float64.
 cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                 const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches);

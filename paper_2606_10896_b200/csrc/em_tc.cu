@@ -979,7 +979,8 @@ __global__ void __launch_bounds__(256) tc_transform_kernel(const float* __restri
                                                            const float* __restrict__ sd, const float* __restrict__ kap,
                                                            const float* __restrict__ gd,
                                                            unsigned char* __restrict__ yhi, unsigned char* __restrict__ ylo,
-                                                           int* __restrict__ status) {
+                                                           int* __restrict__ status, const int* __restrict__ skip_if) {
+    if (skip_if && *skip_if != 0) return;
     const bool vec_ok = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
     const int64_t units = rows_padded * 16;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1039,7 +1040,8 @@ __global__ void __launch_bounds__(256) tc_transform_grouped_kernel(const float* 
 // in the tensor core.  The constant is given back exactly through c_k (E-step) and kap_d N_k (M-step).
 __global__ void __launch_bounds__(128) tc_scale_kernel(int D, int K, const float* __restrict__ pi, const float* __restrict__ mu,
                                                        const float* __restrict__ var, float* __restrict__ sd,
-                                                       float* __restrict__ kap, float* __restrict__ gd) {
+                                                       float* __restrict__ kap, float* __restrict__ gd, const int* __restrict__ run_if) {
+    if (run_if && *run_if == 0) return;
     // one block per dimension (padded to 128); threads stride over the components, fixed-shape tree reductions.
     // First the centre g_d = sum_k pi_k mu_kd / sum_k pi_k: points and means enter every product as x - g, mu - g, so that
     // data far from the origin (in units of its spread) costs the fp16 splits and the fp32 accumulators no precision; the
@@ -1110,7 +1112,8 @@ __global__ void __launch_bounds__(128) tc_prepare_kernel(int D, int K, const flo
                                                          unsigned char* __restrict__ plo_img, float* __restrict__ tk,
                                                          float* __restrict__ ck, float* __restrict__ illb, float cond_limit,
                                                          int* __restrict__ flags, uint32_t* __restrict__ phi_rm,
-                                                         uint32_t* __restrict__ plo_rm, float2* __restrict__ tkck) {
+                                                         uint32_t* __restrict__ plo_rm, float2* __restrict__ tkck, const int* __restrict__ run_if) {
+    if (run_if && *run_if == 0) return;
     const int k = blockIdx.x, d = threadIdx.x;
     const int slice = k >> 7, row = k & 127;
     __shared__ double red_max[128], red_c[128], red_cond[128], red_k[128];
@@ -1211,7 +1214,8 @@ __global__ void __launch_bounds__(128) tc_prepare_kernel(int D, int K, const flo
 __global__ void __launch_bounds__(256) tc_decisive_kernel(int D, int K, const float* __restrict__ mu, const float* __restrict__ var,
                                                           const float* __restrict__ sd, const float* __restrict__ gd,
                                                           const float* __restrict__ illb, int* __restrict__ dec_dim, float* __restrict__ dec_w,
-                                                          float* __restrict__ dec_mu) {
+                                                          float* __restrict__ dec_mu, const int* __restrict__ run_if) {
+    if (run_if && *run_if == 0) return;
     const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (k >= K || !(illb[k] > 0.f)) return;          // warp-uniform
     float wv[4];
@@ -1255,7 +1259,8 @@ __global__ void __launch_bounds__(256) tc_decisive_kernel(int D, int K, const fl
 // than TC_MAX_ILL of them (the assignment then runs on the FP32 kernels).  One block of 1024 threads takes the components
 // 1024 at a time.
 __global__ void __launch_bounds__(1024) tc_ill_list_kernel(int Kpad, const float* __restrict__ illb, int* __restrict__ ill_list,
-                                                           int* __restrict__ flags) {
+                                                           int* __restrict__ flags, const int* __restrict__ run_if) {
+    if (run_if && *run_if == 0) return;
     __shared__ int wcount[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int done = 0;                                    // listed so far (the same in every thread)
@@ -1458,23 +1463,23 @@ TcPlan tc_plan(int D, int K, int num_sms) {
 }
 
 cudaError_t launch_prepare_tc(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var,
-                              const TcBuffers& tb, float cond_limit, int* status, bool ill_list) {
+                              const TcBuffers& tb, float cond_limit, int* status, bool ill_list, const int* run_if) {
     const TcPlan pl = tc_plan(D, K, 148);
     (void)status;
     cudaError_t e0 = cudaMemsetAsync(tb.flags, 0, 8 * sizeof(int), s);
     if (e0 != cudaSuccess) return e0;
-    tc_scale_kernel<<<128, 128, 0, s>>>(D, K, pi, mu, var, tb.sd, tb.kap, tb.gd);
+    tc_scale_kernel<<<128, 128, 0, s>>>(D, K, pi, mu, var, tb.sd, tb.kap, tb.gd, run_if);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     tc_prepare_kernel<<<pl.Kpad, 128, 0, s>>>(D, K, pi, mu, var, tb.sd, tb.kap, tb.gd, tb.phi_img, tb.plo_img, tb.tk, tb.ck, tb.illb, cond_limit, tb.flags,
                                                   reinterpret_cast<uint32_t*>(tb.p_hi_rm), reinterpret_cast<uint32_t*>(tb.p_lo_rm),
-                                                  reinterpret_cast<float2*>(tb.tkck));
+                                                  reinterpret_cast<float2*>(tb.tkck), run_if);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    tc_decisive_kernel<<<(unsigned)((K + 7) / 8), 256, 0, s>>>(D, K, mu, var, tb.sd, tb.gd, tb.illb, tb.dec_dim, tb.dec_w, tb.dec_mu);
+    tc_decisive_kernel<<<(unsigned)((K + 7) / 8), 256, 0, s>>>(D, K, mu, var, tb.sd, tb.gd, tb.illb, tb.dec_dim, tb.dec_w, tb.dec_mu, run_if);
     e = cudaGetLastError();
     if (e != cudaSuccess || !ill_list) return e;
-    tc_ill_list_kernel<<<1, 1024, 0, s>>>(pl.Kpad, tb.illb, tb.ill_list, tb.flags);
+    tc_ill_list_kernel<<<1, 1024, 0, s>>>(pl.Kpad, tb.illb, tb.ill_list, tb.flags, run_if);
     return cudaGetLastError();
 }
 
@@ -1483,13 +1488,14 @@ cudaError_t launch_ill_cache_tc(cudaStream_t s, int D, const float* mu, const fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_transform_tc(cudaStream_t s, const float* X, int64_t n, int D, const TcBuffers& tb, int* status) {
+cudaError_t launch_transform_tc(cudaStream_t s, const float* X, int64_t n, int D, const TcBuffers& tb, int* status,
+                                const int* skip_if) {
     if (n < 1 || n > TC_YPOINTS) return cudaErrorInvalidValue;
     const int64_t rows_padded = (n + TC_BN - 1) / TC_BN * TC_BN;
     const int64_t units = rows_padded * 16;
     int64_t blocks = (units + 255) / 256;
     if (blocks > 148 * 16) blocks = 148 * 16;
-    tc_transform_kernel<<<(unsigned)blocks, 256, 0, s>>>(X, n, rows_padded, D, tb.sd, tb.kap, tb.gd, tb.y_hi, tb.y_lo, status);
+    tc_transform_kernel<<<(unsigned)blocks, 256, 0, s>>>(X, n, rows_padded, D, tb.sd, tb.kap, tb.gd, tb.y_hi, tb.y_lo, status, skip_if);
     return cudaGetLastError();
 }
 

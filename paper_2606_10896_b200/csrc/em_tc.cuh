@@ -66,11 +66,14 @@ void tc_set_order(int o);   // MMA issue order: 0 = pairs E E M M, 1 = interleav
 void tc_set_test_hooks(int silent_rank, unsigned long long wait_limit_ns);
 TcPlan tc_plan(int D, int K, int num_sms);
 cudaError_t tc_max_clusters(int D, int K, int* out);
+// (run_if: the kernels do nothing when it is not NULL and *run_if == 0; the flags are cleared)
 cudaError_t launch_prepare_tc(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var,
-                              const TcBuffers& tb, float cond_limit, int* status, bool ill_list = false);
+                              const TcBuffers& tb, float cond_limit, int* status, bool ill_list = false, const int* run_if = nullptr);
 // One pass over at most TC_YPOINTS points: X -> the two fp16 planes of Y in scratch (read by the tile kernel through TMA).
 // A non-finite value in X raises ST_BAD_X in *status (the planes themselves are clamped to a finite range).
-cudaError_t launch_transform_tc(cudaStream_t s, const float* X, int64_t n, int D, const TcBuffers& tb, int* status);
+// (skip_if: nothing is done when it is not NULL and *skip_if != 0)
+cudaError_t launch_transform_tc(cudaStream_t s, const float* X, int64_t n, int D, const TcBuffers& tb, int* status,
+                                const int* skip_if = nullptr);
 // n <= TC_YPOINTS points whose planes launch_transform_tc has written.
 // mu, w2, c2: the FP32 path's derived parameters (launch_prepare_fp32), used to recompute ill-conditioned logits exactly.
 // tight: use the filter meant for launches in which many components are ill-conditioned (tb.flags[4] counts them).

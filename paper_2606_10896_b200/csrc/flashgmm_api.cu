@@ -243,6 +243,10 @@ struct gmm_ctx {
     double scr_marks = -1.0;         // GMM_SCREEN_MARKS: marked pairs per point up to which the screening path is taken (D <= 128;
                                      // 0: never, < 0: from the measured costs, see screen_limit)
     int64_t scr_piece = 0;           // GMM_SCREEN_PIECE: points per round of launches of the screening path (0: screen_piece)
+    // After a call that the screening has left to the dense kernels, so many calls of the same kind and shape go to them at once
+    // (1, 2, 4 .. 16: mixtures of a fit sharpen as it goes on); see screen_try.
+    struct ScreenHistory { int D = 0, K = 0, skip = 0, left = 0; } scr_history[3];
+    int scr_kind = 0;
     int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
     int sticky_status = 0;           // status bits read off the device but not yet reported (see ensure_scratch)
     // host-streaming path
@@ -834,10 +838,10 @@ int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, c
 
 // One piece's lists (sweep) and values (see launch_screen_eval).
 int screen_values(gmm_ctx* ctx, int mode, const float* Xs, int64_t cnt, int D, int K, float margin, double limit, const float* mu,
-                  float* logp, int32_t* idx, bool count) {
+                  float* logp, int32_t* idx, bool count, int m = 1, float* resp = nullptr) {
     const ScreenBuffers sb = ctx->screen();
-    CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, margin, (float)limit, mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
-    KL(launch_screen_eval(ctx->stream, mode, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, logp, idx, count));
+    CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, margin, mode == SCREEN_TOP ? m : 1, (float)limit, mode == SCREEN_EM || mode == SCREEN_ARGMAX, mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
+    KL(launch_screen_eval(ctx->stream, mode, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, logp, idx, count, m, resp));
     return GMM_OK;
 }
 
@@ -863,11 +867,27 @@ int screen_end(gmm_ctx* ctx, int K, int slot) {
 
 // Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels (nothing is
 // reported then: they find what is wrong again).
+enum { SCREEN_STEPS = 0, SCREEN_CENTROIDS = 1, SCREEN_DENSITIES = 2 };
+bool screen_try(gmm_ctx* ctx, int kind, int D, int K) {
+    if (!screen_wanted(ctx, D, K)) return false;
+    auto& h = ctx->scr_history[kind];
+    if (h.D != D || h.K != K) { h = {}; h.D = D; h.K = K; }
+    if (ctx->scr_marks < 0.0 && h.left > 0) { --h.left; return false; }
+    ctx->scr_kind = kind;
+    return true;
+}
+void screen_note(gmm_ctx* ctx, bool dense) {
+    auto& h = ctx->scr_history[ctx->scr_kind];
+    h.skip = !dense ? 0 : h.skip == 0 ? 1 : h.skip < 16 ? 2 * h.skip : 16;
+    h.left = h.skip;
+}
+
 int screen_result(gmm_ctx* ctx, int slot, double* loglik, bool* dense) {
     DevResult r;
     CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
     *dense = r.scr[SC_DENSE] != 0;
+    screen_note(ctx, *dense);
     ctx->scr_active = 0;
     if (*dense) return GMM_OK;
     CHECK(report_status(ctx, r.status));
@@ -1013,7 +1033,7 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     DeviceGuard g(ctx->device);
     int path;
     CHECK(ensure_scratch(ctx, D, K));
-    if (screen_wanted(ctx, D, K)) {
+    if (screen_try(ctx, SCREEN_STEPS, D, K)) {
         bool dense = false;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
         CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
@@ -1140,7 +1160,7 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         };
         int rc = GMM_OK;
         bool dense = true;
-        if (screen_wanted(ctx, D, K)) {
+        if (screen_try(ctx, SCREEN_STEPS, D, K)) {
             CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
             CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
             CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
@@ -1252,7 +1272,7 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     CU(cudaMemcpyAsync(ctx->xstage[0], X_host, (size_t)cnt0 * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
     CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
-    bool screening = screen_wanted(ctx, D, K);
+    bool screening = screen_try(ctx, SCREEN_STEPS, D, K);
     if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
     else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
     CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
@@ -1304,7 +1324,7 @@ int grow_buffer(gmm_ctx* ctx, void** buf, size_t* have, size_t need, const char*
 
 namespace {
 int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const float* pi, const float* mu,
-                     const float* var, int m, int32_t* idx, float* resp, bool index_only = false);
+                     const float* var, int m, int32_t* idx, float* resp, bool index_only = false, bool screened = false);
 }
 
 int gmm_assign_topm(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const float* pi, const float* mu,
@@ -1325,9 +1345,14 @@ int gmm_assign_topm(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
 namespace {
 // The assignment pass proper (arguments checked, scratch in place); also the nearest-centroid search of the k-means step.
 int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const float* pi, const float* mu,
-                     const float* var, int m, int32_t* idx, float* resp, bool index_only) {
-    KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), &ctx->result()->status));
-    if ((size_t)K * D > ((size_t)1 << 12)) ctx->launches++;      // but for tiny problems, the centre of the means is a launch of its own
+                     const float* var, int m, int32_t* idx, float* resp, bool index_only, bool screened) {
+    // (the screening path's preparation does what this one does, but for the centre of the means)
+    // (When it pays is known on the device alone, so shapes for which it mostly did not are left out: many components in few
+    // dimensions overlap, and with few components the quarters of blocks that bound the m-th best do not bound it well.)
+    const bool screening = !screened && m <= 4 && screen_wanted(ctx, D, K) &&
+                           (ctx->scr_marks > 0.0 || ((double)D >= 1.75 * std::log2((double)K) - 2.0 && K >= 48 * m && (m <= 2 || K >= 3 * D)));
+    if (!screening) KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), &ctx->result()->status));
+    if (!screening && (size_t)K * D > ((size_t)1 << 12)) ctx->launches++;      // but for tiny problems, the centre of the means is a launch of its own
     // Tensor-core assignment where the E+M step would take the tensor path too.  Ill-conditioned components are evaluated
     // exactly for every point; parameters with more than TC_MAX_ILL of them (a flag written on the device by the
     // preparation kernels) go through the FP32 kernels instead: both sets of kernels are enqueued and each checks the
@@ -1475,8 +1500,31 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
     if (tensor) {
         const TcBuffers tb = ctx->tc();
         const float limit = ctx->tc_cond_limit >= 0.f ? ctx->tc_cond_limit : 0.01f;
-        KL(launch_prepare_tc(ctx->stream, D, K, pi, mu, var, tb, limit, &ctx->result()->status, true));
+        // Sparse posteriors: the pairs that can be among the m best, or within 2^-40 of the best, are marked by the screening sweep
+        // and evaluated exactly.  The call is asynchronous, so the tile kernels below are enqueued all the same and return at once
+        // unless the screening has left the call to them.
+        // (The lists have room for 16 pairs per point; a pair costs a quarter of the sweep at K = 1024.)
+        const int* dense_if = nullptr;
+        if (screening) {
+            dense_if = ctx->result()->scr + SC_DENSE;
+            CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+            const int64_t piece = screen_piece(ctx, N);
+            for (int64_t off = 0; off < N; off += piece) {
+                const int64_t cnt = (N - off < piece) ? (N - off) : piece;
+                CHECK(prof_begin(ctx));
+                CHECK(screen_values(ctx, SCREEN_TOP, X + off * D, cnt, D, K, index_only ? 0.f : 40.f, ctx->scr_marks > 0.0 ? ctx->scr_marks : 12.0, mu, nullptr,
+                                    idx + off * m, false, m, index_only ? nullptr : resp + off * m));
+                CHECK(prof_end(ctx));
+            }
+        }
+        if (screening) KL(launch_center_fp32(ctx->stream, D, K, mu, ctx->center(), dense_if));
+        KL(launch_prepare_tc(ctx->stream, D, K, pi, mu, var, tb, limit, &ctx->result()->status, true, dense_if));
         ctx->launches += 3;
+        run_fp32_if = tb.flags + 3;
+        if (screening) {
+            run_fp32_if = ctx->result()->scr + SC_FALLBACK;
+            KL(launch_screen_gate(ctx->stream, ctx->screen(), tb.flags + 3, ctx->result()->scr + SC_FALLBACK));
+        }
         KL(launch_ill_cache_tc(ctx->stream, D, mu, ctx->w2(), ctx->c2(), tb));
         const int64_t piece = ctx->tc_piece;
         const int64_t cap = N < piece ? N : piece;
@@ -1497,7 +1545,7 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
                 CU(cudaMemsetAsync(unc_count, 0, sizeof(int), ctx->stream));
             }
             CHECK(prof_begin(ctx));
-            KL(launch_transform_tc(ctx->stream, X + off * D, cnt, D, tb, &ctx->result()->status));
+            KL(launch_transform_tc(ctx->stream, X + off * D, cnt, D, tb, &ctx->result()->status, screening ? tb.flags + 3 : nullptr));
             KL(launch_assign_tc(ctx->stream, X + off * D, cnt, D, K, mu, ctx->w2(), ctx->c2(), tb, reinterpret_cast<float*>(base),
                                 unc_rows, unc_count, (int)(off - win_start), m, idx + off * m, resp ? resp + off * m : nullptr, &ctx->result()->status,
                                 index_only));
@@ -1513,7 +1561,6 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
             }
             CHECK(prof_end(ctx));
         }
-        run_fp32_if = tb.flags + 3;
     }
     for (int64_t off = 0; off < N; off += SUPER_TILE) {
         const int64_t cnt = (N - off < SUPER_TILE) ? (N - off) : SUPER_TILE;
@@ -1623,7 +1670,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     CHECK(ensure_scratch(ctx, D, K));
     CHECK(grow_buffer(ctx, &ctx->pl_scratch, &ctx->pl_scratch_bytes, pl_scratch_bytes(K), "the posting-list counters"));
     CHECK(grow_buffer(ctx, &ctx->km_scratch, &ctx->km_scratch_bytes, km_scratch_bytes(D, K), "the k-means partial sums"));
-    if (screen_wanted(ctx, D, K)) {
+    if (screen_try(ctx, SCREEN_CENTROIDS, D, K)) {
         // through the screening path: the arg-max alone (margin 0), every point a lone pair of its cluster, and the statistics
         // of the pairs about the centroids give the new ones and the inertia
         const ScreenBuffers sb = ctx->screen();
@@ -1645,6 +1692,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         DevResult r;
         CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
         CU(cudaStreamSynchronize(ctx->stream));
+        screen_note(ctx, r.scr[SC_DENSE] != 0);
         if (r.scr[SC_DENSE] == 0) {
             if (inertia) *inertia = r.ll[0];
             ctx->last_path = GMM_PATH_TENSOR;
@@ -1665,7 +1713,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         float* pi_u = var_u + KD;
         KL(launch_kmeans_scaled_mixture(ctx->stream, D, K, centroids, pi_u, var_u, pi_u + K));
         ctx->launches++;
-        CHECK(assign_topm_impl(ctx, X, N, D, K, pi_u, centroids, var_u, 1, assign, nullptr, true));
+        CHECK(assign_topm_impl(ctx, X, N, D, K, pi_u, centroids, var_u, 1, assign, nullptr, true, true));
         tensor = ctx->last_path == GMM_PATH_TENSOR;
     } else if (tensor) {
         // through the assignment pass of the tensor path, with that mixture written out: pi = 1 / K, var = 1
@@ -1674,7 +1722,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         float* var_u = static_cast<float*>(ctx->km_unit);
         float* pi_u = var_u + KD;
         KL(launch_kmeans_unit_mixture(ctx->stream, D, K, pi_u, var_u));
-        CHECK(assign_topm_impl(ctx, X, N, D, K, pi_u, centroids, var_u, 1, assign, resp, true));       // the indices alone are used
+        CHECK(assign_topm_impl(ctx, X, N, D, K, pi_u, centroids, var_u, 1, assign, resp, true, true));       // the indices alone are used
     } else {
         KL(launch_kmeans_unit_params(ctx->stream, D, K, ctx->w2(), ctx->c2d()));
         KL(launch_center_fp32(ctx->stream, D, K, centroids, ctx->center()));
@@ -1708,7 +1756,7 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
     CHECK(check_ptr(ctx, logp, 4, "logp"));
     DeviceGuard guard(ctx->device);
     CHECK(ensure_scratch(ctx, D, K));
-    if (screen_wanted(ctx, D, K)) {
+    if (screen_try(ctx, SCREEN_DENSITIES, D, K)) {
         // D <= 128: the same idea (csrc/em_screen.cu).  The FP32 kernel takes 1.4e-4 K D ns per point, the screening path about
         // 0.8 ns and 0.25 ns per marked pair.
         const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks : std::fmin(14.0, std::fmax(1.5, (1.4e-4 * K * D - 0.8) / 0.25));
@@ -1836,7 +1884,7 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
-    if (smallest > 0 && screen_wanted(ctx, D, K)) {
+    if (smallest > 0 && screen_try(ctx, SCREEN_STEPS, D, K)) {
         // Screening path: consecutive groups are taken as many at a time as a piece holds; a larger group goes
         // through the step's own accumulation.
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false));

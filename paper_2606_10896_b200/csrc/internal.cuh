@@ -30,7 +30,7 @@ size_t fp32_partial_floats(int D, int K);   // floats in the per-CTA partial buf
 // g [D] (may be NULL): receives the per-dimension centre of the means (launch_center_fp32), which the kernels below take
 cudaError_t launch_prepare_fp32(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var,
                                 float* w2, float* c2, double* c2d, float* g, int* status);
-cudaError_t launch_center_fp32(cudaStream_t s, int D, int K, const float* mu, float* g);
+cudaError_t launch_center_fp32(cudaStream_t s, int D, int K, const float* mu, float* g, const int* run_if = nullptr);
 // log2-domain log Z of n points -> logZ2[n]; per-block float64 partial log-likelihoods -> llpart[fp32_ll_parts(n, D, K)]
 // c2d: the per-component constants in float64; logZ2: float64 (the kernels carry logits in float64 when D > 128)
 // g: the per-dimension centre subtracted from points and means before the products are formed (NULL = none; any value

@@ -165,3 +165,34 @@ def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
         np.testing.assert_allclose(new[k], X[a == k].astype(np.float64).mean(0), rtol=0, atol=1e-5)
     empty = np.setdiff1d(np.arange(K), a)
     assert np.array_equal(new[empty], mu[empty])               # a centroid without points stays where it is
+
+
+# the top-m assignment through the sweep: a point far away from everything, components without a weight (fewer than m with one, once)
+@pytest.mark.parametrize("N,D,K,m", [(1, 16, 64, 1), (257, 33, 97, 2), (3001, 128, 1024, 2), (3001, 128, 1024, 4), (1500, 20, 300, 3), (900, 66, 4096, 4),
+                                     (2000, 9, 130, 1), (300, 12, 192, 4)])
+def test_screen_top_m(fg, monkeypatch, N, D, K, m):
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    monkeypatch.setenv("GMM_SCREEN_PIECE", "768")
+    X, pi, mu, var = _mixture(N, D, K, N + D + K, collapsed=3)
+    X[N // 2] = 4000.0
+    pi[K // 2] = 0.0
+    if N == 300:
+        pi[3:] = 0.0
+    lj = np.asarray(orc.log_joint(X, pi, mu, var), np.float64)
+    lz = np.logaddexp.reduce(lj, axis=1)
+    want = np.sort(lj, axis=1)[:, ::-1][:, :m]
+    with fg.Context(0) as c:
+        idx, resp = (v.cpu().numpy() for v in c.gmm_assign_topm(_t(X), _t(pi), _t(mu), _t(var), m))
+        idx2, resp2 = (v.cpu().numpy() for v in c.gmm_assign_topm(_t(X), _t(pi), _t(mu), _t(var), m))
+        only = c.gmm_assign_topm(_t(X), _t(pi), _t(mu), _t(var), m, indices_only=True)
+        only = (only[0] if isinstance(only, tuple) else only).cpu().numpy()
+    assert np.array_equal(idx, idx2) and np.array_equal(resp, resp2) and np.array_equal(idx, only)
+    assert idx.min() >= 0 and idx.max() < K and all(len(set(r)) == m for r in idx)
+    got = np.take_along_axis(lj, idx.astype(np.int64), axis=1)
+    near = np.abs(want) * 2e-6 + 1e-3
+    ok = np.isneginf(want) if N == 300 else np.zeros_like(want, bool)
+    assert np.all((got >= want - near) | (ok & np.isneginf(got)))
+    with np.errstate(over="ignore"):
+        r_ref = np.exp(got - lz[:, None])
+    far = np.arange(N) == N // 2                            # (its log-densities of 1e7 leave fp32 little to tell)
+    assert np.all(np.abs(resp - r_ref)[~far] <= 2e-4 * r_ref[~far] + 1e-6)

@@ -1541,6 +1541,255 @@ __device__ __forceinline__ double wide_pair_log2z(const float* __restrict__ xr, 
     return c - q;
 }
 
+// The marked pairs in three steps.  wide_pair_list_kernel turns the marks of the map into a list of pairs (a point's pairs
+// consecutive, in ascending slot order), wide_pair_eval_kernel evaluates the list, a warp per pair, and wide_pair_finish_kernel
+// brings a point's values together.  (A warp per POINT took its pairs one after the other, each two trips to L2 that waited for
+// the one before and a look whether the pair could still matter: 7.8 ms per million points at D = 768, 4 pairs each, 3.5 TB/s
+// of L2 traffic.  Nearly every pair that the filter leaves is kept, so nothing is gained by looking.)
+// Room for the list: one request per block - they all go to one counter.  Where a block's part starts depends on timing, what is
+// stored there does not.  No room left: ctl[5] tells wide_cand_lse_kernel to take those points and the statistics kernel to evaluate
+// every pair of the piece itself.
+__global__ void __launch_bounds__(256) wide_pair_list_kernel(int64_t n, int words, const unsigned* __restrict__ cand, int* __restrict__ ctl,
+                                                             int* __restrict__ pair_off, int* __restrict__ pair_cnt,
+                                                             unsigned short* __restrict__ pair_slot, int* __restrict__ pair_row, bool assign) {
+    if (ctl[1] != 0) return;
+    __shared__ int tot_s[8];
+    __shared__ int base_s;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 8 + w;
+    unsigned bits[(WIDE_CAND_WORDS + 31) / 32];
+    int c[(WIDE_CAND_WORDS + 31) / 32], mine = 0;
+#pragma unroll
+    for (int q = 0; q < (WIDE_CAND_WORDS + 31) / 32; ++q) {
+        bits[q] = (i < n && lane + 32 * q < words) ? __ldg(cand + i * words + lane + 32 * q) : 0u;
+        c[q] = __popc(bits[q]);
+        mine += c[q];
+    }
+    const int total = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) tot_s[w] = total;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int j = 0; j < 8; ++j) t += tot_s[j];
+        int b = t > 0 ? atomicAdd(ctl + 4, t) : 0;
+        if (b < 0 || b > WIDE_PAIR_VALS - t) {
+            for (int e = b; e >= 0 && e < WIDE_PAIR_VALS && e < b + t; ++e) pair_row[e] = (int)0x80000000;      // (nobody's)
+            b = -1;
+            ctl[5] = 1;
+        }
+        base_s = b;
+    }
+    __syncthreads();
+    if (i >= n) return;
+    int off = base_s;
+    for (int j = 0; j < w && off >= 0; ++j) off += tot_s[j];
+    if (lane == 0) { pair_off[i] = off; pair_cnt[i] = total; }
+    if (off < 0) return;
+    // an assignment's only pair needs no value: that component is the point's best, every other lies 2^-40 below it
+    const int row = assign && total == 1 ? -1 - (int)i : (int)i;
+    int base = off;                                          // word lane + 32 q belongs to lane `lane`: the order is (q, lane, bit)
+#pragma unroll
+    for (int q = 0; q < (WIDE_CAND_WORDS + 31) / 32; ++q) {
+        if (__any_sync(0xffffffffu, c[q] != 0)) {
+            int incl = c[q];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+            int at = base + incl - c[q];
+            for (unsigned word = bits[q]; word; word &= word - 1) {
+                pair_slot[at] = (unsigned short)((lane + 32 * q) * 32 + __ffs(word) - 1);
+                pair_row[at] = row;
+                ++at;
+            }
+            base += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+}
+
+// Exact log2 z of the listed pairs: a warp takes four consecutive ones (a point's, mostly: its row stays in registers), all loads of a
+// component's rows in flight together.  The arithmetic of wide_pair_log2z.  Bound by L2: 6 KB per pair at D = 768.
+// NJ = chunks of 128 dimensions (0: rows that are not whole 16-byte groups).
+template <int NJ>
+__global__ void __launch_bounds__(256, 2) wide_pair_eval_kernel(const float* __restrict__ X, int D, const float* __restrict__ mu_c,
+                                                                const float* __restrict__ w2_c, const double* __restrict__ c2d_c,
+                                                                const int* __restrict__ ctl, const unsigned short* __restrict__ pair_slot,
+                                                                const int* __restrict__ pair_row, double* __restrict__ pair_l) {
+    if (ctl[1] != 0) return;
+    const int total = ctl[4] < 0 || ctl[4] > WIDE_PAIR_VALS ? WIDE_PAIR_VALS : ctl[4];
+    const int lane = threadIdx.x & 31, nw = gridDim.x * 8;
+    int cur = -1;
+    float4 x[NJ > 0 ? NJ : 1];
+    for (int e0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 4; e0 < total; e0 += nw * 4) {
+        int row4 = 0, slot4 = 0;
+        if (lane < 4 && e0 + lane < total) { row4 = pair_row[e0 + lane]; slot4 = pair_slot[e0 + lane]; }
+        for (int j = 0; j < 4 && e0 + j < total; ++j) {
+            const int row = __shfl_sync(0xffffffffu, row4, j), slot = __shfl_sync(0xffffffffu, slot4, j);
+            if (row < 0) continue;
+            const double c = __ldg(c2d_c + slot);
+            if (NJ == 0) {
+                const double l = wide_pair_log2z(X + (size_t)row * D, mu_c + (size_t)slot * D, w2_c + (size_t)slot * D, c, D, lane, -CUDART_INF);
+                if (lane == 0) pair_l[e0 + j] = l;
+                continue;
+            }
+            const float4* mr = reinterpret_cast<const float4*>(mu_c + (size_t)slot * D) + lane;
+            const float4* wr = reinterpret_cast<const float4*>(w2_c + (size_t)slot * D) + lane;
+            float4 m[NJ > 0 ? NJ : 1], v[NJ > 0 ? NJ : 1];
+#pragma unroll
+            for (int z = 0; z < NJ; ++z) {
+                const bool in = z < NJ - 1 || 128 * z + 4 * lane < D;
+                m[z] = in ? __ldg(mr + 32 * z) : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[z] = in ? __ldg(wr + 32 * z) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if (row != cur) {
+                const float4* xr = reinterpret_cast<const float4*>(X + (size_t)row * D) + lane;
+#pragma unroll
+                for (int z = 0; z < NJ; ++z) x[z] = z < NJ - 1 || 128 * z + 4 * lane < D ? __ldg(xr + 32 * z) : make_float4(0.f, 0.f, 0.f, 0.f);
+                cur = row;
+            }
+            double q = 0.0;
+#pragma unroll
+            for (int z = 0; z < NJ; ++z) {
+                float part = 0.f, dd = x[z].x - m[z].x;
+                part = fmaf(dd * dd, v[z].x, part);
+                dd = x[z].y - m[z].y;  part = fmaf(dd * dd, v[z].y, part);
+                dd = x[z].z - m[z].z;  part = fmaf(dd * dd, v[z].z, part);
+                dd = x[z].w - m[z].w;  part = fmaf(dd * dd, v[z].w, part);
+                q += (double)part;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+            if (lane == 0) pair_l[e0 + j] = c - q;
+        }
+    }
+}
+
+// A thread per point.  TOPM = 0, best_out == NULL: the pairs within 2^-40 of the point's largest value (its log2 Z over the evaluated
+// components included) are kept: log-sum-exp into out[i], bit (slot, i) of the transposed map, values relative to the largest.
+// best_out: the component (list[slot]) of the largest value, the smaller one of two equal.  TOPM > 0: the m_top largest and their
+// responsibilities; ranks that no marked pair fills (every component there lies 2^-40 below the point's best: responsibility 0)
+// are taken from the sweep's candidates, in the order of their upper bounds.
+template <int TOPM>
+__global__ void __launch_bounds__(128) wide_pair_finish_kernel(int64_t n, const int* __restrict__ ctl, const int* __restrict__ pair_off,
+                                                               const int* __restrict__ pair_cnt, const unsigned short* __restrict__ pair_slot,
+                                                               const double* __restrict__ pair_l, const double* __restrict__ logz,
+                                                               unsigned* __restrict__ candT, int* __restrict__ slot_cnt,
+                                                               double* __restrict__ out, float* __restrict__ pair_val,
+                                                               double* __restrict__ pair_best, unsigned short* __restrict__ pair_key8,
+                                                               float* __restrict__ pair_val8, const int* __restrict__ list,
+                                                               int32_t* __restrict__ best_out, int m_top, int32_t* __restrict__ top_idx,
+                                                               float* __restrict__ top_resp, int32_t* __restrict__ unc_rows,
+                                                               int* __restrict__ unc_count, const float* __restrict__ swp_top, int swp_ntop,
+                                                               const int* __restrict__ comp_of) {
+    if (ctl[1] != 0) return;
+    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (i >= n) return;
+    const int off = pair_off[i], cnt = pair_cnt[i];
+    if (off < 0) return;                                     // (wide_cand_lse_kernel's)
+    if (cnt == 0) {
+        if (TOPM > 0) unc_rows[atomicAdd(unc_count, 1)] = (int32_t)i;
+        else if (best_out) best_out[i] = 0;
+        else out[i] = -CUDART_INF;
+        return;
+    }
+    const bool single = (TOPM > 0 || best_out) && cnt == 1;  // (not evaluated)
+    if (TOPM > 0) {
+        constexpr int TM = TOPM > 0 ? TOPM : 1;
+        double topv[TM];                                     // the largest values so far, descending, and their components
+        int topc[TM];
+#pragma unroll
+        for (int r = 0; r < TM; ++r) { topv[r] = -CUDART_INF; topc[r] = -1; }
+        double zm = -CUDART_INF, zs = 0.0;
+        for (int e = 0; e < cnt; ++e) {
+            const double l = single ? 0.0 : pair_l[off + e];
+            if (!(l > -CUDART_INF)) continue;
+            if (l > zm) { zs = zs * exp2(zm - l) + 1.0; zm = l; }
+            else zs += exp2(l - zm);
+            double v = l;                                    // insertion by (value descending, component ascending)
+            int c = __ldg(list + pair_slot[off + e]);
+#pragma unroll
+            for (int r = 0; r < TM; ++r) {
+                if (r < m_top && c >= 0 && (v > topv[r] || (v == topv[r] && topc[r] >= 0 && c < topc[r]) || topc[r] < 0)) {
+                    const double tv = topv[r];
+                    const int tc = topc[r];
+                    topv[r] = v; topc[r] = c;
+                    v = tv; c = tc;
+                }
+            }
+        }
+        const double lzf = zm + log2(zs);
+        int have = 0;
+#pragma unroll
+        for (int r = 0; r < TM; ++r)
+            if (r < m_top && topc[r] >= 0) ++have;
+        for (int q = 0; q < swp_ntop && have > 0 && have < m_top; ++q) {
+            const int pos = __float_as_int(swp_top[i * 2 * swp_ntop + swp_ntop + q]);
+            const int c = pos >= 0 ? __ldg(comp_of + pos) : -1;
+            bool dup = c < 0;
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+                if (r < m_top && topc[r] == c) dup = true;
+            if (dup) continue;
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+                if (r == have) { topc[r] = c; topv[r] = -CUDART_INF; }
+            ++have;
+        }
+        if (have != m_top) {
+            unc_rows[atomicAdd(unc_count, 1)] = (int32_t)i;
+        } else {
+#pragma unroll
+            for (int r = 0; r < TM; ++r)
+                if (r < m_top) {
+                    top_idx[i * m_top + r] = topc[r];
+                    if (top_resp) top_resp[i * m_top + r] = (float)exp2(topv[r] - lzf);
+                }
+        }
+        return;
+    }
+    double best = logz[i];
+    if (best_out) {
+        if (single) { best_out[i] = __ldg(list + pair_slot[off]); return; }
+        int comp = 0x7fffffff;
+        for (int e = 0; e < cnt; ++e) {
+            const double l = pair_l[off + e];
+            if (l >= best && l > -CUDART_INF) {
+                const int c = __ldg(list + pair_slot[off + e]);
+                if (l > best || c < comp) comp = c;
+                best = l;
+            }
+        }
+        best_out[i] = comp != 0x7fffffff ? comp : 0;
+        return;
+    }
+    for (int e = 0; e < cnt; ++e) best = fmax(best, pair_l[off + e]);
+    const double lim = best - 40.0;
+    double m = -CUDART_INF, ssum = 0.0;
+    int kept = 0;
+    for (int e = 0; e < cnt; ++e) {
+        const double l = pair_l[off + e];
+        const int slot = pair_slot[off + e];
+        const bool keep = l >= lim && l > -CUDART_INF;
+        if (keep) {
+            if (l > m) { ssum = ssum * exp2(m - l) + 1.0; m = l; }
+            else ssum += exp2(l - m);
+            atomicOr(candT + (size_t)slot * WIDE_CANDT_WORDS + (i >> 5), 1u << (i & 31));
+            atomicAdd(slot_cnt + slot, 1);
+            pair_val[off + e] = (float)(l - best);           // in [-40, 0]
+            ++kept;
+        }
+        if (e < 8) {
+            pair_key8[i * 8 + e] = keep ? (unsigned short)slot : (unsigned short)0xFFFF;
+            pair_val8[i * 8 + e] = keep ? (float)(l - best) : 0.f;
+        }
+    }
+    for (int e = cnt; e < 8; ++e) pair_key8[i * 8 + e] = 0xFFFF;
+    out[i] = kept ? m + log2(ssum) : -CUDART_INF;
+    pair_best[i] = best;
+}
+
+// The points whose pairs found no room in the list (none, as a rule).
 // One warp per point: its marked pairs in ascending slot order, evaluated exactly.  First round: every pair's exact log2 z,
 // each abandoned as soon as it cannot come within 2^-40 of the largest value so far (the point's log2 Z over the evaluated
 // components to begin with: logz); the first 128 values are kept in shared memory.  Second round: the pairs within 2^-40
@@ -1555,27 +1804,24 @@ __global__ void __launch_bounds__(256, 3) wide_cand_lse_kernel(const float* __re
                                                             const float* __restrict__ mu_c, const float* __restrict__ w2_c,
                                                             const double* __restrict__ c2d_c, const double* __restrict__ logz,
                                                             double* __restrict__ out, int* __restrict__ ctl,
-                                                            int* __restrict__ slot_cnt, float* __restrict__ pair_val,
-                                                            int* __restrict__ pair_off, double* __restrict__ pair_best,
+                                                            int* __restrict__ slot_cnt, const int* __restrict__ pair_off,
                                                             const int* __restrict__ list, int32_t* __restrict__ best_out,
                                                             int m_top, int32_t* __restrict__ top_idx, float* __restrict__ top_resp,
                                                             int32_t* __restrict__ unc_rows, int* __restrict__ unc_count,
                                                             const float* __restrict__ swp_top, int swp_ntop,
-                                                            const int* __restrict__ comp_of,
-                                                            unsigned short* __restrict__ pair_key8, float* __restrict__ pair_val8) {
+                                                            const int* __restrict__ comp_of) {
     // TOPM > 0 (the top-m assignment, m_top <= TOPM): only the first round runs; it keeps the m_top largest exact values
     // (a pair is abandoned once it can reach neither the m_top-th of them nor 2^-40 of the largest) and the sum of all.
     // Ranks that no marked pair fills (every component there lies 2^-40 below the point's best: responsibility 0) are
     // taken from the sweep's candidates, in the order of their upper bounds.
     // best_out != NULL (the hard assignment): only the first round runs, and the component (list[slot]) of the point's
     // largest exact value goes to best_out[i]; of equal values the smaller component.
-    if (ctl[1] != 0) return;
+    if (ctl[1] != 0 || ctl[5] == 0) return;
     __shared__ double lbuf[8][CAND_KEEP];
     __shared__ unsigned short slist[8][CAND_LIST];
-    __shared__ int tot_s[8];
-    __shared__ int base_s;
     const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (i >= n || pair_off[i] >= 0) return;
     unsigned bits[CAND_WORDS_PER_LANE];
     int nmarked = 0;
 #pragma unroll
@@ -1585,23 +1831,7 @@ __global__ void __launch_bounds__(256, 3) wide_cand_lse_kernel(const float* __re
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nmarked += __shfl_xor_sync(0xffffffffu, nmarked, o);
-    // Room for the exact values of the block's pairs (the statistics kernel reads them back instead of evaluating its pairs
-    // again): one request per block - they all go to one counter.  Where the room starts depends on timing, what is stored
-    // there does not.  No room left: ctl[5] tells the statistics kernel to evaluate every pair of the piece itself.
-    const bool assign_mode = TOPM > 0 || best_out != nullptr;      // (block-uniform: no values are kept for a statistics kernel)
-    if (!assign_mode) {
-        if (lane == 0) tot_s[w] = nmarked;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int t = 0;
-            for (int j = 0; j < 8; ++j) t += tot_s[j];
-            int b = t > 0 ? atomicAdd(ctl + 4, t) : 0;
-            if (b < 0 || b > WIDE_PAIR_VALS - t) { b = -1; ctl[5] = 1; }
-            base_s = b;
-        }
-        __syncthreads();
-    }
-    if (i >= n) return;
+    const bool assign_mode = TOPM > 0 || best_out != nullptr;
     if (nmarked == 0) {
         if (lane == 0) {
             if (TOPM > 0) unc_rows[atomicAdd(unc_count, 1)] = (int32_t)i;
@@ -1610,8 +1840,6 @@ __global__ void __launch_bounds__(256, 3) wide_cand_lse_kernel(const float* __re
         }
         return;
     }
-    int off = assign_mode ? -1 : base_s;
-    for (int j = 0; j < w && !assign_mode; ++j) off += (off >= 0) ? tot_s[j] : 0;
     // The assignment of a point with ONE marked pair needs no evaluation: that component is the point's best, and every other
     // lies 2^-40 below it (responsibility 1 and 0).
     const bool single = assign_mode && nmarked == 1;
@@ -1898,10 +2126,6 @@ __global__ void __launch_bounds__(256, 3) wide_cand_lse_kernel(const float* __re
     const double lim = best - 40.0;
     double m = -CUDART_INF, ssum = 0.0;
     int kept = 0;
-    // (lane j < 8 holds the j-th marked pair's slot and value for the table of first pairs: what the statistics kernel
-    // looks at before it counts the marked bits below a slot)
-    unsigned short key8 = 0xFFFFu;
-    float val8 = 0.f;
     auto second = [&](int slot, int at) {
         double l;
         if (at < CAND_KEEP) l = lbuf[w][at];
@@ -1912,11 +2136,6 @@ __global__ void __launch_bounds__(256, 3) wide_cand_lse_kernel(const float* __re
             if (lane == 0) {
                 atomicOr(candT + (size_t)slot * WIDE_CANDT_WORDS + (i >> 5), 1u << (i & 31));
                 atomicAdd(slot_cnt + slot, 1);
-                if (off >= 0) pair_val[off + at] = (float)(l - best);       // in [-40, 0]
-            }
-            if (lane == at) {
-                key8 = (unsigned short)slot;
-                val8 = (float)(l - best);
             }
             ++kept;
         }
@@ -1937,12 +2156,6 @@ __global__ void __launch_bounds__(256, 3) wide_cand_lse_kernel(const float* __re
     }
     if (lane == 0) {
         out[i] = kept ? m + log2(ssum) : -CUDART_INF;
-        pair_off[i] = off;
-        pair_best[i] = best;
-    }
-    if (lane < 8) {
-        pair_key8[i * 8 + lane] = key8;
-        pair_val8[i * 8 + lane] = val8;
     }
 }
 
@@ -2551,12 +2764,41 @@ cudaError_t launch_cand_count_wide(cudaStream_t s, int n_slots, const WideBuffer
     return cudaGetLastError();
 }
 
+// The list of the marked pairs and their values.
+static cudaError_t launch_pairs(cudaStream_t s, const float* X, int64_t n, int D, int n_slots, const WideBuffers& wb, bool assign) {
+    wide_pair_list_kernel<<<(unsigned)((n + 7) / 8), 256, 0, s>>>(n, (n_slots + 31) / 32, wb.cand, wb.ctl, wb.pair_off, wb.pair_cnt, wb.pair_slot, wb.pair_row, assign);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const bool vec = (D % 4 == 0) && (((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(wb.mu_c) | reinterpret_cast<uintptr_t>(wb.w2_c)) & 15) == 0);
+    const unsigned grid = 148 * 8;
+#define FG_PE(J_) wide_pair_eval_kernel<J_><<<grid, 256, 0, s>>>(X, D, wb.mu_c, wb.w2_c, wb.c2d_c, wb.ctl, wb.pair_slot, wb.pair_row, wb.pair_l)
+    switch (vec ? (D + 127) / 128 : 0) {
+        case 2: FG_PE(2); break;
+        case 3: FG_PE(3); break;
+        case 4: FG_PE(4); break;
+        case 5: FG_PE(5); break;
+        case 6: FG_PE(6); break;
+        case 7: FG_PE(7); break;
+        case 8: FG_PE(8); break;
+        default: FG_PE(0); break;
+    }
+#undef FG_PE
+    return cudaGetLastError();
+}
+
 cudaError_t launch_cand_lse_wide(cudaStream_t s, const float* X, int64_t n, int D, int n_slots, const WideBuffers& wb,
                                  double* logz_ill, int32_t* best_out) {
     const int words = (n_slots + 31) / 32;
+    cudaError_t e = launch_pairs(s, X, n, D, n_slots, wb, best_out != nullptr);
+    if (e != cudaSuccess) return e;
+    wide_pair_finish_kernel<0><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(n, wb.ctl, wb.pair_off, wb.pair_cnt, wb.pair_slot, wb.pair_l, wb.logz, wb.candT,
+                                                                           wb.slot_cnt, logz_ill, wb.pair_val, wb.pair_best, wb.pair_key8, wb.pair_val8,
+                                                                           wb.ill_list, best_out, 0, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     wide_cand_lse_kernel<0><<<(unsigned)((n + 7) / 8), 256, 0, s>>>(X, n, D, words, wb.cand, wb.candT, wb.mu_c, wb.w2_c, wb.c2d_c, wb.logz,
-                                                                    logz_ill, wb.ctl, wb.slot_cnt, wb.pair_val, wb.pair_off, wb.pair_best, wb.ill_list, best_out,
-                                                                    0, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr, wb.pair_key8, wb.pair_val8);
+                                                                    logz_ill, wb.ctl, wb.slot_cnt, wb.pair_off, wb.ill_list, best_out,
+                                                                    0, nullptr, nullptr, nullptr, nullptr, nullptr, 0, nullptr);
     return cudaGetLastError();
 }
 
@@ -2564,10 +2806,16 @@ cudaError_t launch_cand_topm_wide(cudaStream_t s, const float* X, int64_t n, int
                                   int32_t* idx, float* resp, int32_t* unc_rows, int* unc_count, int ntop) {
     if (m < 1 || m > GMM_MAX_TOPM || (ntop != 6 && ntop != WIDE_MAX_TOP)) return cudaErrorInvalidValue;
     const int words = (n_slots + 31) / 32;
+    cudaError_t e = launch_pairs(s, X, n, D, n_slots, wb, true);
+    if (e != cudaSuccess) return e;
+    wide_pair_finish_kernel<GMM_MAX_TOPM><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(
+        n, wb.ctl, wb.pair_off, wb.pair_cnt, wb.pair_slot, wb.pair_l, wb.logz, wb.candT, wb.slot_cnt, nullptr, wb.pair_val, wb.pair_best, wb.pair_key8,
+        wb.pair_val8, wb.ill_list, nullptr, m, idx, resp, unc_rows, unc_count, wb.top, ntop, wb.comp_of);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     wide_cand_lse_kernel<GMM_MAX_TOPM><<<(unsigned)((n + 7) / 8), 256, 0, s>>>(X, n, D, words, wb.cand, wb.candT, wb.mu_c, wb.w2_c, wb.c2d_c, wb.logz,
-                                                                               nullptr, wb.ctl, wb.slot_cnt, wb.pair_val, wb.pair_off, wb.pair_best,
-                                                                               wb.ill_list, nullptr, m, idx, resp, unc_rows, unc_count,
-                                                                               wb.top, ntop, wb.comp_of, wb.pair_key8, wb.pair_val8);
+                                                                               nullptr, wb.ctl, wb.slot_cnt, wb.pair_off, wb.ill_list, nullptr, m, idx,
+                                                                               resp, unc_rows, unc_count, wb.top, ntop, wb.comp_of);
     return cudaGetLastError();
 }
 

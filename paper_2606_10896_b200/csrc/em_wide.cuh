@@ -85,7 +85,11 @@ struct WideBuffers {
     float* rec_thr;    // [WIDE_PIECE] the point's final screening threshold (before the 2^-40 margin)
     float* pair_val;   // [WIDE_PAIR_VALS] exact log2 z of a piece's kept pairs relative to the point's best value, a point's
                        // marked pairs consecutive and in slot order (positions from a counter: ctl[4])
-    int* pair_off;     // [WIDE_PIECE] where a point's values start
+    int* pair_off;     // [WIDE_PIECE] where a point's pairs start in the lists of pairs (-1: they found no room)
+    int* pair_cnt;     // [WIDE_PIECE] how many there are
+    unsigned short* pair_slot; // [WIDE_PAIR_VALS] a marked pair's slot,
+    int* pair_row;     // [WIDE_PAIR_VALS] its point (negative: not evaluated),
+    double* pair_l;    // [WIDE_PAIR_VALS] its exact log2 z
     double* pair_best; // [WIDE_PIECE] the point's best value (the reference of its pair_val entries)
     unsigned short* pair_key8; // [WIDE_PIECE][8] the slots of a point's first eight marked pairs (0xFFFF: not kept), and
     float* pair_val8;          // [WIDE_PIECE][8] their values: what the statistics kernel finds in one read

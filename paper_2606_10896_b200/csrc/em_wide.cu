@@ -5,7 +5,7 @@
 // D > 128 no longer fits the 512 TMEM columns of an SM next to the logits, and the coefficient slice of 128 components
 // (128 x 2D x 2 fp16 planes) no longer fits shared memory, so neither can stay on chip for the life of a CTA.
 //
-//   sweep 1  (lse_wide_kernel, TMEM lanes = POINTS)   Algorithm 1, Step 1.  A CTA takes tiles of 128 points and walks the
+//   sweep 1  (lse_wide_kernel, TMEM lanes = POINTS)   Algorithm 1, Step 1.  A pair of CTAs takes tiles of 256 points and walks the
 //            components in groups of 256 (256 TMEM columns for the main product, 256 for the two small cross products:
 //            the same split, and the same order of accumulation, as in sweep 2, so that both sweeps see the same logits
 //            and the responsibilities of a point sum to one; a group that is only screened forms the leading product
@@ -56,13 +56,17 @@ constexpr float RSCALE = TC_RSCALE;
 
 // ------------------------------------------------------------------------------------------------------------------
 // Sweep 1
-// The ring holds four stages of 48 KB: one plane's atoms of a contraction step, [Y atom | coefficient atoms of the group's
-// two chunks] (the two chunks adjacent: one operand of 256 rows).  A step of a group that forms all three products takes
-// two stages (hi planes, lo planes), a step of a leading-product group one.  One barrier pair and one commit per stage:
-// with a barrier pair per atom the two single-lane loops (loads, MMAs) took 2000 cycles per step of 516 cycles of MMAs.
+// Two CTAs on neighbouring SMs work as a pair (cta_group::2) on 256 points x 256 components: each holds the Y atom of its own 128
+// points and the coefficient atom of one of the group's two chunks, the tensor cores of both read both chunks.  Alone, a CTA
+// had to bring in 48 KB per 512 cycles of MMAs, 12 TB/s out of L2 over the chip with four stages in flight: the tensor cores were
+// busy 59 % of the time.  The pair brings in 32 KB per CTA, and six stages fit: 1.24 -> 1.07 ms per 2^17 points at D = 768,
+// K = 4096.  Bound now by shared memory: 64 B per cycle into it and as much out of it for the MMAs at full rate.
+// A stage: one plane's atoms of a contraction step.  A step of a group that forms all three products takes two stages (hi
+// planes, lo planes), a step of a leading-product group one.  The even CTA (the leader) issues the MMAs of both; a stage's
+// barrier is the leader's and counts both CTAs' bytes, a commit arrives in both CTAs.
 constexpr int HSLOT = 16384;
-constexpr int L_STAGE = 3 * HSLOT;
-constexpr int L_SLOTS = 4;
+constexpr int L_STAGE = 2 * HSLOT;
+constexpr int L_SLOTS = 6;
 constexpr int L_BAR = L_SLOTS * L_STAGE;
 constexpr int L_MERGE = L_BAR + 256;                // 128 x 8 bytes: (max, sum) pairs of warpgroup 1, later the log-likelihood terms
 constexpr int L_SMEM = L_MERGE + 1024 + 1024;
@@ -128,8 +132,33 @@ struct WideTop {
     }
 };
 
+// Primitives of a pair of CTAs.  pair_bar: the leader's barrier, as an address that both can use.
+__device__ __forceinline__ uint32_t pair_bar(uint32_t bar) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(bar));
+    return r;
+}
+__device__ __forceinline__ void pair_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void pair_load_3d(uint32_t dst, const CUtensorMap* tm, int32_t x, int32_t y, int32_t z, uint32_t bar, uint64_t policy) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
+                 ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy) : "memory");
+}
+__device__ __forceinline__ void pair_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n"
+                 ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void pair_commit(uint32_t bar) {          // arrives at the barrier of this offset in both CTAs
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3) : "memory");
+}
+__device__ __forceinline__ void pair_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 template <int NTOP>
-__global__ void __launch_bounds__(WT_THREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(WT_THREADS, 1)
 lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, const __grid_constant__ CUtensorMap tm_ylo,
                 const __grid_constant__ CUtensorMap tm_phi, const __grid_constant__ CUtensorMap tm_plo) {
     extern __shared__ unsigned char smem_raw[];
@@ -152,8 +181,12 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
     __shared__ int tabm_s[2][2][4];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t ntiles = (p.n + WIDE_TILE - 1) / WIDE_TILE;
-    const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
+    // (the pair's tiles of 256 points: this CTA has rows [128 rank, 128 rank + 128) of each)
+    const int rank = (int)(blockIdx.x & 1);
+    const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+    const int64_t ntiles = (p.n + 2 * WIDE_TILE - 1) / (2 * WIDE_TILE);
+    const int64_t ntl = (pair < ntiles) ? (ntiles - pair + npairs - 1) / npairs : 0;
+    auto tile_row = [&](int64_t i) { return (pair + i * npairs) * (2 * WIDE_TILE) + rank * WIDE_TILE; };
     const int NC = p.NC, NZ = p.NZ;
     const int NG = (NC + 1) >> 1;                        // groups of two chunks
     // A tile's steps, the same for every role: with pre_pass the groups from hi_group on once for their lower bounds (so that
@@ -169,21 +202,23 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
         abort_s = 0;
         drain_s = 0;
         for (int s = 0; s < L_SLOTS; ++s) { bar_init(BAR(LB_FULL + s), 1); bar_init(BAR(LB_EMPTY + s), 1); }
-        for (int b = 0; b < 2; ++b) { bar_init(BAR(LB_LFULL + b), 1); bar_init(BAR(LB_LEMPTY + b), 256); }
+        for (int b = 0; b < 2; ++b) { bar_init(BAR(LB_LFULL + b), 1); bar_init(BAR(LB_LEMPTY + b), 512); }      // (the leader's: both CTAs' threads)
         bar_init(BAR(LB_FINAL), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == WT_MMA) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     fence_before();
     __syncthreads();
+    pair_sync();
     fence_after();
     const uint32_t tmem = tmem_base_s;
 
     if (warp < 8) {
         // =========================== softmax warps: thread = TMEM lane = point ===========================
+        const uint32_t lempty = pair_bar(BAR(LB_LEMPTY));
         // Warpgroup g reads chunk g of every group of two chunks (main product in columns [128 g, 128 g + 128), cross products
         // in [256 + 128 g, ...)); the two running (max, sum) pairs of a point are merged at the end of its tile.
         const int grp = warp >> 2, wq = warp & 3;
@@ -216,7 +251,7 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
             if (pt < 4) tabm_s[tb][grp][pt] = n_mask;
         };
         for (int64_t i = 0; i < ntl; ++i) {
-            const int64_t row = (blockIdx.x + i * gridDim.x) * WIDE_TILE + pt;
+            const int64_t row = tile_row(i) + pt;
             float m_run = -1e30f, s_run = 0.f;               // finite start: blocks of -inf logits must not make NaN
             const float nrm = ((p.screen || NTOP > 2) && row < p.n) ? __ldg(p.n2 + row) : 0.f;
             float thr_base = -1e30f;
@@ -275,11 +310,11 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
                 if (hi_grp) {
                     half = nb;
                     nb ^= 1;
-                    got = bar_wait(BAR(LB_LFULL + half), (half ? ub1 : ub0) & 1u, abort_flag, p.status, false);
+                    got = bar_wait(BAR(LB_LFULL + half), (half ? ub1 : ub0) & 1u, abort_flag, p.status, true);
                     if (half) ++ub1; else ++ub0;
                 } else {
-                    got = bar_wait(BAR(LB_LFULL), ub0 & 1u, abort_flag, p.status, false);
-                    got = bar_wait(BAR(LB_LFULL + 1), ub1 & 1u, abort_flag, p.status, false) && got;
+                    got = bar_wait(BAR(LB_LFULL), ub0 & 1u, abort_flag, p.status, true);
+                    got = bar_wait(BAR(LB_LFULL + 1), ub1 & 1u, abort_flag, p.status, true) && got;
                     ++ub0;
                     ++ub1;
                 }
@@ -387,8 +422,8 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
                     }
                 }
                 fence_before();
-                if (hi_grp) bar_arrive(BAR(LB_LEMPTY + half));
-                else { bar_arrive(BAR(LB_LEMPTY)); bar_arrive(BAR(LB_LEMPTY + 1)); }
+                if (hi_grp) pair_arrive(lempty + 8 * half);
+                else { pair_arrive(lempty); pair_arrive(lempty + 8); }
                 if (t + 1 < nsteps) table_store((int)(tcount & 1u));
             }
             // merge the two warpgroups' pairs; warpgroup 0 writes log2 Z and the two leading candidates
@@ -433,135 +468,120 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
             p.llpart[blockIdx.x] += s * 0.69314718055994530942;       // one owner per slot: launches add up
         }
     } else if (warp == WT_PRODUCER) {
-        // =========================== producer warp (TMA) ===========================
+        // =========================== producer warp (TMA): one thread ===========================
         // Stage order = order of use: per (tile, step of the tile, atom z) the hi planes' stage, then (unless the group forms
-        // the leading product only) the lo planes' stage.
-        int64_t g = 0;
-        bool ok = true;
-        // Both streams are kept in L2 with priority: the coefficient atoms are read by every CTA for every tile, the tile's
-        // own atoms once per step of the tile.  (Marked evict-first, the tile's atoms missed L2 on nearly every re-read -
-        // a third of the sweep's sectors came from DRAM, 17 % of its time: L2 is full of older lines of normal priority,
-        // e.g. the planes as the transform wrote them, which such lines do not displace.)
-        const uint64_t pol_keep = l2_policy_evict_last();
-        auto stage = [&](const CUtensorMap* my, const CUtensorMap* mp, int32_t yrow, int32_t prow, int nch, int32_t z) -> bool {
-            const int slot = (int)(g % L_SLOTS);
-            const int64_t use = g / L_SLOTS;
-            if (use > 0) {
-                uint32_t w = 1;
-                if (lane == 0) w = bar_wait(BAR(LB_EMPTY + slot), (uint32_t)((use - 1) & 1), abort_flag, p.status, false) ? 1u : 0u;
-                if (!__shfl_sync(0xffffffffu, w, 0)) return false;
-            }
-            if (elect_one()) {
+        // the leading product only) the lo planes' stage.  Both streams are kept in L2 with priority: the coefficient atoms are
+        // read by every pair for every tile, the tile's own atoms once per step of the tile.  (Marked evict-first, the tile's
+        // atoms missed L2 on nearly every re-read - a third of the sweep's sectors came from DRAM, 17 % of its time: L2 is full
+        // of older lines of normal priority, e.g. the planes as the transform wrote them, which such lines do not displace.)
+        if (elect_one()) {
+            uint32_t slot = 0, parity = 1;                   // of the next stage; the phase whose end frees its slot
+            int64_t issued = 0;
+            bool ok = true;
+            const uint64_t pol_keep = l2_policy_evict_last();
+            const uint32_t full = pair_bar(BAR(LB_FULL));
+            auto stage = [&](const CUtensorMap* my, const CUtensorMap* mp, int32_t yrow, int32_t prow, int32_t z) -> bool {
+                if (issued >= L_SLOTS && !bar_wait(BAR(LB_EMPTY + slot), parity, abort_flag, p.status, true)) return false;
                 const uint32_t dst = smem_u32(smem + slot * L_STAGE);
-                bar_expect_tx(BAR(LB_FULL + slot), (uint32_t)((1 + nch) * HSLOT));
-                tma_load_3d_hint(dst, my, 0, yrow, z, BAR(LB_FULL + slot), pol_keep);
-                for (int c = 0; c < nch; ++c)
-                    tma_load_3d_hint(dst + (uint32_t)((1 + c) * HSLOT), mp, 0, prow + c * 128, z, BAR(LB_FULL + slot), pol_keep);
-            }
-            __syncwarp();
-            ++g;
-            return true;
-        };
-        for (int64_t i = 0; i < ntl && ok; ++i) {
-            const int32_t row0 = (int32_t)((blockIdx.x + i * gridDim.x) * WIDE_TILE);
-            for (int t = 0; t < nsteps && ok; ++t) {
-                const int gq = step_group(t);
-                const int nch = (NC - 2 * gq < 2) ? (NC - 2 * gq) : 2;
-                const bool hi_only = leading_only(gq);
-                for (int z = 0; z < NZ && ok; ++z) {
-                    ok = stage(&tm_yhi, &tm_phi, row0, 2 * gq * 128, nch, z);
-                    if (ok && !hi_only) ok = stage(&tm_ylo, &tm_plo, row0, 2 * gq * 128, nch, z);
+                if (rank == 0) bar_expect_tx(BAR(LB_FULL + slot), 2u * L_STAGE);
+                pair_load_3d(dst, my, 0, yrow, z, full + 8 * slot, pol_keep);
+                pair_load_3d(dst + HSLOT, mp, 0, prow, z, full + 8 * slot, pol_keep);      // (a chunk beyond the last: zeros)
+                ++issued;
+                if (++slot == L_SLOTS) { slot = 0; parity ^= 1u; }
+                return true;
+            };
+            for (int64_t i = 0; i < ntl && ok; ++i) {
+                const int32_t row0 = (int32_t)tile_row(i);
+                for (int t = 0; t < nsteps && ok; ++t) {
+                    const int gq = step_group(t);
+                    const bool hi_only = leading_only(gq);
+                    const int32_t prow = (2 * gq + rank) * 128;
+                    for (int z = 0; z < NZ && ok; ++z) {
+                        ok = stage(&tm_yhi, &tm_phi, row0, prow, z);
+                        if (ok && !hi_only) ok = stage(&tm_ylo, &tm_plo, row0, prow, z);
+                    }
                 }
             }
-        }
-        // the loads in flight must have landed before the CTA may exit, also after an abort
-        if (!ok || *abort_flag) {
-            for (int64_t h = (g > L_SLOTS ? g - L_SLOTS : 0); h < g; ++h) {
-                if (lane == 0) bar_wait(BAR(LB_FULL + (int)(h % L_SLOTS)), (uint32_t)((h / L_SLOTS) & 1), drain_flag, p.status, false);
-                __syncwarp();
+            // after an abort: loads in flight must land before the CTA may exit (they take microseconds; their barrier may be
+            // the other CTA's, whose state is not known here)
+            if (!ok || *abort_flag) {
+                const unsigned long long t0 = gtime();
+                while (gtime() - t0 < 2000000ull) __nanosleep(1000);
             }
         }
-    } else {
-        // =========================== MMA warp ===========================
-        const uint32_t idesc1 = make_idesc(WIDE_TILE, 128, 0), idesc2 = make_idesc(WIDE_TILE, 256, 0);
-        const uint64_t d0 = make_desc(smem_u32(smem), 16, 1024);
-        bool alive = true;
-        auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {
-            uint32_t ok = 1;
-            if (lane == 0) ok = bar_wait(bar, parity, abort_flag, p.status, false) ? 1u : 0u;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            fence_after();
-            return ok != 0u;
-        };
-        int64_t g = 0;
-        uint32_t ub0 = 0, ub1 = 0;                           // uses of the two accumulator halves
-        int nb = 0;
-        auto take = [&](int& slot) -> bool {                 // the next stage of the ring, once it has landed
-            slot = (int)(g % L_SLOTS);
-            const bool ok = wait_all(BAR(LB_FULL + slot), (uint32_t)((g / L_SLOTS) & 1));
-            ++g;
-            return ok;
-        };
-        for (int64_t i = 0; i < ntl && alive; ++i) {
-            for (int t = 0; t < nsteps && alive; ++t) {
-                const int gq = step_group(t);
-                const int nch = (NC - 2 * gq < 2) ? (NC - 2 * gq) : 2;
-                const bool hi_only = leading_only(gq);
-                const uint32_t idesc = nch == 2 ? idesc2 : idesc1;       // both chunks of the group as one operand of 256 rows
-                // the softmax warps must be done with the accumulator columns this group writes
-                int half = 0;
-                if (hi_only) {
-                    half = nb;
-                    nb ^= 1;
-                    const uint32_t u = half ? ub1 : ub0;
-                    if (u > 0 && !wait_all(BAR(LB_LEMPTY + half), (u - 1) & 1u)) { alive = false; break; }
-                } else {
-                    if (ub0 > 0 && !wait_all(BAR(LB_LEMPTY), (ub0 - 1) & 1u)) { alive = false; break; }
-                    if (ub1 > 0 && !wait_all(BAR(LB_LEMPTY + 1), (ub1 - 1) & 1u)) { alive = false; break; }
-                }
-                const uint32_t d = tmem + half * 256, dc = tmem + 256;
-                for (int z = 0; z < NZ && alive; ++z) {
-                    int sh = 0, sl = 0;
-                    if (!take(sh)) { alive = false; break; }
-                    if (!hi_only && !take(sl)) { alive = false; break; }
-                    if (elect_one()) {
+        __syncwarp();
+    } else if (rank == 0) {
+        // =========================== MMA warp of the leader: one thread ===========================
+        if (elect_one()) {
+            const uint32_t idesc = make_idesc(2 * WIDE_TILE, 256, 0);
+            const uint64_t d0 = make_desc(smem_u32(smem), 16, 1024);
+            bool alive = true;
+            uint32_t slot = 0, parity = 0;                   // the next stage of the ring
+            uint32_t ub0 = 0, ub1 = 0;                       // uses of the two accumulator halves
+            int nb = 0;
+            auto take = [&](uint32_t& at) -> bool {          // the next stage of the ring, once it has landed
+                at = slot;
+                const bool ok = bar_wait(BAR(LB_FULL + slot), parity, abort_flag, p.status, true);
+                if (++slot == L_SLOTS) { slot = 0; parity ^= 1u; }
+                return ok;
+            };
+            for (int64_t i = 0; i < ntl && alive; ++i) {
+                for (int t = 0; t < nsteps && alive; ++t) {
+                    const bool hi_only = leading_only(step_group(t));
+                    // the softmax warps must be done with the accumulator columns this group writes
+                    int half = 0;
+                    if (hi_only) {
+                        half = nb;
+                        nb ^= 1;
+                        const uint32_t u = half ? ub1 : ub0;
+                        if (u > 0) alive = bar_wait(BAR(LB_LEMPTY + half), (u - 1) & 1u, abort_flag, p.status, true);
+                    } else {
+                        if (ub0 > 0) alive = bar_wait(BAR(LB_LEMPTY), (ub0 - 1) & 1u, abort_flag, p.status, true);
+                        if (alive && ub1 > 0) alive = bar_wait(BAR(LB_LEMPTY + 1), (ub1 - 1) & 1u, abort_flag, p.status, true);
+                    }
+                    const uint32_t d = tmem + half * 256, dc = tmem + 256;
+                    for (int z = 0; z < NZ && alive; ++z) {
+                        uint32_t sh = 0, sl = 0;
+                        alive = take(sh);
+                        if (alive && !hi_only) alive = take(sl);
+                        if (!alive) break;
+                        fence_after();
                         const uint64_t ah = d0 + ((sh * L_STAGE) >> 4), bh = ah + (HSLOT >> 4);
                         // the two small cross products into their own accumulator, the leading product into the main one:
                         // the same three chains, in the same order, as the E-step of sweep 2
                         if (!hi_only) {
                             const uint64_t al = d0 + ((sl * L_STAGE) >> 4), bl = al + (HSLOT >> 4);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) mma_ss(dc, ah + ((j * 32) >> 4), bl + ((j * 32) >> 4), idesc, (z > 0 || j > 0) ? 1u : 0u);
+                            for (int j = 0; j < 4; ++j) pair_mma(dc, ah + ((j * 32) >> 4), bl + ((j * 32) >> 4), idesc, (z > 0 || j > 0) ? 1u : 0u);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) mma_ss(dc, al + ((j * 32) >> 4), bh + ((j * 32) >> 4), idesc, 1u);
+                            for (int j = 0; j < 4; ++j) pair_mma(dc, al + ((j * 32) >> 4), bh + ((j * 32) >> 4), idesc, 1u);
                         }
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) mma_ss(d, ah + ((j * 32) >> 4), bh + ((j * 32) >> 4), idesc, (z > 0 || j > 0) ? 1u : 0u);
-                        mma_commit(BAR(LB_EMPTY + sh));
-                        if (!hi_only) mma_commit(BAR(LB_EMPTY + sl));
+                        for (int j = 0; j < 4; ++j) pair_mma(d, ah + ((j * 32) >> 4), bh + ((j * 32) >> 4), idesc, (z > 0 || j > 0) ? 1u : 0u);
+                        pair_commit(BAR(LB_EMPTY + sh));
+                        if (!hi_only) pair_commit(BAR(LB_EMPTY + sl));
                         if (z == NZ - 1) {
-                            if (hi_only) mma_commit(BAR(LB_LFULL + half));
-                            else { mma_commit(BAR(LB_LFULL)); mma_commit(BAR(LB_LFULL + 1)); }
+                            if (hi_only) pair_commit(BAR(LB_LFULL + half));
+                            else { pair_commit(BAR(LB_LFULL)); pair_commit(BAR(LB_LFULL + 1)); }
                         }
                     }
-                    __syncwarp();
+                    if (hi_only) { if (half) ++ub1; else ++ub0; }
+                    else { ++ub0; ++ub1; }
                 }
-                if (hi_only) { if (half) ++ub1; else ++ub0; }
-                else { ++ub0; ++ub1; }
             }
+            pair_commit(BAR(LB_FINAL));
+            bar_wait(BAR(LB_FINAL), 0, drain_flag, p.status, true);
+            fence_after();
         }
-        if (elect_one()) mma_commit(BAR(LB_FINAL));
         __syncwarp();
-        if (lane == 0) bar_wait(BAR(LB_FINAL), 0, drain_flag, p.status, false);
-        __syncwarp();
-        fence_after();
     }
 
     fence_before();
     __syncthreads();
+    pair_sync();                                             // (neither CTA leaves while the other may still use its memory)
     if (warp == WT_MMA) {
         fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
 }
 
@@ -2915,8 +2935,8 @@ cudaError_t launch_lse_wide(cudaStream_t s, int64_t n, int D, int K, int Kg, int
         p.pre_pass = pre_pass ? 1 : 0;
     }
     if (ntop != 2 && hi_first_slots >= 0 && topm <= 0) { p.hi_group = 0; p.hi_end = Kgp / 256; }             // the assignment's evaluated groups
-    const int64_t ntiles = (n + WIDE_TILE - 1) / WIDE_TILE;
-    const unsigned grid = (unsigned)(ntiles < num_sms ? ntiles : num_sms);
+    const int64_t ntiles = (n + 2 * WIDE_TILE - 1) / (2 * WIDE_TILE);
+    const unsigned grid = 2u * (unsigned)(ntiles < num_sms / 2 ? ntiles : num_sms / 2);      // pairs of CTAs
     if (ntop == 2) lse_wide_kernel<2><<<grid, WT_THREADS, L_SMEM, s>>>(p, tm_yhi, tm_ylo, tm_phi, tm_plo);
     else if (ntop == 6) lse_wide_kernel<6><<<grid, WT_THREADS, L_SMEM, s>>>(p, tm_yhi, tm_ylo, tm_phi, tm_plo);
     else lse_wide_kernel<WIDE_MAX_TOP><<<grid, WT_THREADS, L_SMEM, s>>>(p, tm_yhi, tm_ylo, tm_phi, tm_plo);

@@ -821,10 +821,13 @@ int read_result(gmm_ctx* ctx, int slot, double* loglik) {
 bool screen_wanted(const gmm_ctx* ctx, int D, int K) {
     return ctx->path == GMM_PATH_AUTO && ctx->lay.scr && ctx->capPlanes && ctx->scr_marks != 0.0 && auto_is_tensor(D, K);
 }
-// Marked pairs per point up to which the screening path is the cheaper one.
-double screen_limit(const gmm_ctx* ctx, int K) {
+// Marked pairs per point up to which the screening path is the cheaper one, from measured costs in ns per point: the dense kernels
+// 0.5 + 0.0032 K (0.62 at 10 x 100, 0.83 at 64 x 128, 2.1 at 12 x 541, 3.7 at 128 x 1024), the sweep and what does not depend on the
+// marks 0.15 + 0.001 D + 0.045 per 128 components, a pair 0.09 + 0.001 D.  (At most SCR_MARKS.)
+double screen_limit(const gmm_ctx* ctx, int D, int K) {
     if (ctx->scr_marks > 0.0) return ctx->scr_marks;
-    return 0.012 * K < 2.0 ? 2.0 : 0.012 * K < 12.0 ? 0.012 * K : 12.0;
+    const double dense = 0.5 + 0.0032 * K, fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
+    return std::fmin((double)SCR_MARKS, std::fmax(1.5, 0.9 * (dense - fixed) / (0.09 + 0.001 * D)));
 }
 
 // Points per round of launches for n points in all: equal pieces (an odd small one at the end pays all launches for little), in
@@ -861,7 +864,7 @@ int screen_points(gmm_ctx* ctx, const float* X, int64_t n, int D, int K, const f
         const int64_t cnt = (n - off < piece) ? (n - off) : piece;
         const float* Xs = X + off * D;
         CHECK(prof_begin(ctx));
-        CHECK(screen_values(ctx, SCREEN_EM, Xs, cnt, D, K, 40.f, screen_limit(ctx, K), mu, nullptr, nullptr, true));
+        CHECK(screen_values(ctx, SCREEN_EM, Xs, cnt, D, K, 40.f, screen_limit(ctx, D, K), mu, nullptr, nullptr, true));
         CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         CHECK(prof_end(ctx));
     }
@@ -1691,7 +1694,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
             const float* Xs = X + off * D;
-            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, K), centroids, nullptr, assign + off, true));
+            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, D, K), centroids, nullptr, assign + off, true));
             CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, centroids, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         }
         double* ik = km_inertia_k(ctx->km_scratch, D, K);
@@ -1931,7 +1934,7 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
                 CU(cudaMemsetAsync(out, 0, (size_t)(bt.g1 - bt.g0) * 2 * KD * sizeof(float), ctx->stream));
             } else {
                 CHECK(prof_begin(ctx));
-                CHECK(screen_values(ctx, SCREEN_EM, Xs, rows, D, K, 40.f, screen_limit(ctx, K), mu, nullptr, nullptr, false));
+                CHECK(screen_values(ctx, SCREEN_EM, Xs, rows, D, K, 40.f, screen_limit(ctx, D, K), mu, nullptr, nullptr, false));
                 CU(launch_screen_groups(ctx->stream, Xs, bt.g1 - bt.g0, D, K, d_tab + bt.g0, d_tab + G + bt.g0, d_off, pi, mu, var, ctx->w2(),
                                         ctx->c2d(), sb, out, &ctx->launches));
                 CHECK(prof_end(ctx));

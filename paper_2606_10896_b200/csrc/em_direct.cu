@@ -42,6 +42,7 @@ struct DirectArgs {
     const int* stop_at;      // NULL, or the iteration after which nothing is done any more
     int iter;
     int lgG, lgS;            // lanes per point: components, dimensions
+    int NS;                  // a tile's points are taken in NS rounds
     int ld, ldr, kr;         // row strides (multiples of 4, odd multiples: no bank conflicts), rows of the parameters
     int D4, lgX;             // chunks of four dimensions; lanes per row when X is staged
     int T, R;                // tiles of the statistics, replicas
@@ -74,11 +75,14 @@ __global__ void __launch_bounds__(NT, 2) direct_kernel(const DirectArgs p) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int D = p.D, K = p.K, D4 = p.D4, ld = p.ld, ldr = p.ldr, kr = p.kr;
     const int lgL = p.lgG + p.lgS, G = 1 << p.lgG, S = 1 << p.lgS;
-    const int s = tid & (S - 1), gq = (tid >> p.lgS) & (G - 1), pg = tid >> lgL, PG = NT >> lgL, TP = PT * PG;
+    const int s = tid & (S - 1), gq = (tid >> p.lgS) & (G - 1), pg = tid >> lgL, PG = NT >> lgL;
+    const int NS = (PT == 4 && MODE != DK_LSE) ? 1 : p.NS, TP = NS * PT * PG;      // (known at compile time where registers are short)
     float* sw = sm;                          // [kr][ld] sqrt(w2)
     float* ms = sw + kr * ld;                // [kr][ld] (g - mu) sqrt(w2)
     float* xs = ms + kr * ld;                // [TP][ld] x - g
     float* rs = xs + TP * ld;                // [TP][ldr] responsibilities
+    float2* run_s = reinterpret_cast<float2*>(rs);      // DK_LSE, several blocks of components: [TP] largest value, sum
+    float* lz_s = rs + TP * ldr;             // DK_STATS: [TP] log2 Z
     const int kfirst = MODE == DK_STATS ? (int)blockIdx.y * 64 : 0;
     const int nblk = MODE == DK_LSE ? (K + 63) / 64 : 1;
     const int64_t ntiles = (p.n + TP - 1) / TP;
@@ -209,12 +213,10 @@ __global__ void __launch_bounds__(NT, 2) direct_kernel(const DirectArgs p) {
             __syncthreads();                                 // (the tile before this one has been read)
             tile_fetch(row0);
         }
+        if (MODE == DK_STATS)
+            for (int r = tid; r < TP; r += NT) lz_s[r] = row0 + r < p.n ? (float)__ldcg(p.logZ2 + row0 + r) : CUDART_INF_F;
         tile_centre(row0);
         __syncthreads();
-        float m_run[PT], s_run[PT];
-        float l[PT][4];
-#pragma unroll
-        for (int j = 0; j < PT; ++j) { m_run[j] = -CUDART_INF_F; s_run[j] = 0.f; }
         for (int blk = 0; blk < nblk; ++blk) {
             if (nblk > 1) {
                 __syncthreads();
@@ -222,77 +224,93 @@ __global__ void __launch_bounds__(NT, 2) direct_kernel(const DirectArgs p) {
                 constants(blk * 64);
                 __syncthreads();
             }
-            u64 q[PT][4];
+#pragma unroll 1
+            for (int sub = 0; sub < NS; ++sub) {
+                const int p0 = sub * PT * PG + pg;           // this lane's points: p0 + j PG
+                float m_run[PT], s_run[PT];
+                float l[PT][4];
 #pragma unroll
-            for (int j = 0; j < PT; ++j)
+                for (int j = 0; j < PT; ++j) {
+                    m_run[j] = -CUDART_INF_F;
+                    s_run[j] = 0.f;
+                    if (MODE == DK_LSE && blk > 0) { const float2 v = run_s[p0 + j * PG]; m_run[j] = v.x; s_run[j] = v.y; }
+                }
+                u64 q[PT][4];
 #pragma unroll
-                for (int b = 0; b < 4; ++b) q[j][b] = 0ull;
+                for (int j = 0; j < PT; ++j)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) q[j][b] = 0ull;
 #pragma unroll 2
-            for (int d4 = s; d4 < D4; d4 += S) {
-                ulonglong2 x[PT];
+                for (int d4 = s; d4 < D4; d4 += S) {
+                    ulonglong2 x[PT];
 #pragma unroll
-                for (int j = 0; j < PT; ++j) x[j] = *reinterpret_cast<const ulonglong2*>(xs + (pg + j * PG) * ld + 4 * d4);
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + (gq + G * b) * ld + 4 * d4);
-                    const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ms + (gq + G * b) * ld + 4 * d4);
-#pragma unroll
-                    for (int j = 0; j < PT; ++j) {
-                        const u64 t0 = fma2(x[j].x, w.x, m.x), t1 = fma2(x[j].y, w.y, m.y);
-                        q[j][b] = fma2(t0, t0, q[j][b]);
-                        q[j][b] = fma2(t1, t1, q[j][b]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < PT; ++j) {
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    float v = lo2(q[j][b]) + hi2(q[j][b]);
-                    for (int o = 1; o < S; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    l[j][b] = cv[b] - v;
-                }
-                if (MODE != DK_STATS) {
-                    float m = fmaxf(fmaxf(l[j][0], l[j][1]), fmaxf(l[j][2], l[j][3]));
-                    for (int o = S; o < (1 << lgL); o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-                    m = fmaxf(m, m_run[j]);
-                    const float ref = m == -CUDART_INF_F ? 0.f : m;
-                    float e[4], a;
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) e[b] = dk_ex2(l[j][b] - ref);
-                    a = (e[0] + e[1]) + (e[2] + e[3]);
-                    for (int o = S; o < (1 << lgL); o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-                    s_run[j] = (MODE == DK_FUSED ? 0.f : s_run[j] * dk_ex2(m_run[j] - ref)) + a;
-                    m_run[j] = m;
-                    if (MODE == DK_FUSED) {
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) l[j][b] = e[b];
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < PT; ++j) {
-            const int r = pg + j * PG;
-            const int64_t row = row0 + r;
-            const bool in = row < p.n;
-            if (MODE != DK_STATS) {
-                const double lz = (double)m_run[j] + (double)log2f(s_run[j]);
-                if (in && (tid & ((1 << lgL) - 1)) == 0) {
-                    ll += lz;
-                    if (p.logZ2) p.logZ2[row] = lz;
-                }
-            }
-            if (MODE != DK_LSE) {
-                float f, lz = 0.f;
-                if (MODE == DK_FUSED) f = in ? 1.0f / s_run[j] : 0.f;
-                else lz = in ? (float)__ldcg(p.logZ2 + row) : CUDART_INF_F;
-                if (s == 0) {
+                    for (int j = 0; j < PT; ++j) x[j] = *reinterpret_cast<const ulonglong2*>(xs + (p0 + j * PG) * ld + 4 * d4);
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
-                        const float v = MODE == DK_FUSED ? l[j][b] * f : dk_ex2(l[j][b] - lz);
-                        nacc[b] += v;
-                        if (gq + G * b < ldr) rs[r * ldr + gq + G * b] = v;
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + (gq + G * b) * ld + 4 * d4);
+                        const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ms + (gq + G * b) * ld + 4 * d4);
+#pragma unroll
+                        for (int j = 0; j < PT; ++j) {
+                            const u64 t0 = fma2(x[j].x, w.x, m.x), t1 = fma2(x[j].y, w.y, m.y);
+                            q[j][b] = fma2(t0, t0, q[j][b]);
+                            q[j][b] = fma2(t1, t1, q[j][b]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < PT; ++j) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        float v = lo2(q[j][b]) + hi2(q[j][b]);
+                        for (int o = 1; o < S; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                        l[j][b] = cv[b] - v;
+                    }
+                    if (MODE != DK_STATS) {
+                        float m = fmaxf(fmaxf(l[j][0], l[j][1]), fmaxf(l[j][2], l[j][3]));
+                        for (int o = S; o < (1 << lgL); o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                        m = fmaxf(m, m_run[j]);
+                        const float ref = m == -CUDART_INF_F ? 0.f : m;
+                        float e[4], a;
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) e[b] = dk_ex2(l[j][b] - ref);
+                        a = (e[0] + e[1]) + (e[2] + e[3]);
+                        for (int o = S; o < (1 << lgL); o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                        s_run[j] = (MODE == DK_FUSED ? 0.f : s_run[j] * dk_ex2(m_run[j] - ref)) + a;
+                        m_run[j] = m;
+                        if (MODE == DK_FUSED) {
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) l[j][b] = e[b];
+                        }
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < PT; ++j) {
+                    const int r = p0 + j * PG;
+                    const int64_t row = row0 + r;
+                    const bool in = row < p.n;
+                    if (MODE != DK_STATS) {
+                        if (blk + 1 == nblk) {
+                            const double lz = (double)m_run[j] + (double)log2f(s_run[j]);
+                            if (in && (tid & ((1 << lgL) - 1)) == 0) {
+                                ll += lz;
+                                if (p.logZ2) p.logZ2[row] = lz;
+                            }
+                        } else if ((tid & ((1 << lgL) - 1)) == 0) {
+                            run_s[r] = make_float2(m_run[j], s_run[j]);      // (read after the barriers of the next block)
+                        }
+                    }
+                    if (MODE != DK_LSE) {
+                        float f = 0.f, lz = 0.f;
+                        if (MODE == DK_FUSED) f = in ? 1.0f / s_run[j] : 0.f;
+                        else lz = lz_s[r];
+                        if (s == 0) {
+#pragma unroll
+                            for (int b = 0; b < 4; ++b) {
+                                const float v = MODE == DK_FUSED ? l[j][b] * f : dk_ex2(l[j][b] - lz);
+                                nacc[b] += v;
+                                if (gq + G * b < ldr) rs[r * ldr + gq + G * b] = v;
+                            }
+                        }
                     }
                 }
             }
@@ -561,15 +579,23 @@ DirectPlan direct_plan(int mode, const float* X, int64_t n, int D, int K) {
     // points per tile: four per lane, fewer where the tile would not leave room for a second CTA on the SM, or where there would
     // not be a tile for every SM; the lanes then share the dimensions as long as there are eight per lane
     pl.PT = (mode == DK_LSE || D > 32) ? 4 : 2;          // (at four, the statistics' registers spill, once per tile)
-    auto tp = [&]() { return (int64_t)pl.PT * (NT >> (a.lgG + a.lgS)); };
-    auto bytes = [&]() { return (2 * a.kr * a.ld + tp() * (a.ld + (mode == DK_LSE ? 0 : a.ldr))) * 4; };
+    a.NS = 1;
+    auto tp = [&]() { return (int64_t)a.NS * pl.PT * (NT >> (a.lgG + a.lgS)); };
+    const int nblk = mode == DK_LSE ? (K + 63) / 64 : 1, row_extra = mode == DK_FUSED ? a.ldr : mode == DK_STATS ? a.ldr + 1 : nblk > 1 ? 2 : 0;
+    auto bytes = [&]() { return (2 * a.kr * a.ld + tp() * (a.ld + row_extra)) * 4; };
     while (bytes() > 110592 || (n + tp() - 1) / tp() * cblocks < SMS) {
         if (a.lgG + a.lgS < 5 && a.D4 >= (4 << a.lgS)) { ++a.lgS; set_ld(); }
         else if (pl.PT > 1) pl.PT >>= 1;
         else break;
     }
+    // few dimensions: a tile's barriers (and, with several blocks of components, their parameters) cost more than its arithmetic, so a
+    // tile takes more points as long as there are tiles for all SMs
+    while (a.NS < 16 && a.NS * a.D4 < 32 && (pl.PT < 4 || mode == DK_LSE)) {
+        a.NS *= 2;
+        if (bytes() > 110592 || (n + tp() - 1) / tp() * cblocks < 2 * SMS) { a.NS /= 2; break; }
+    }
     pl.tiles = (n + tp() - 1) / tp();
-    size_t fl = (size_t)2 * a.kr * a.ld + (size_t)tp() * (a.ld + (mode == DK_LSE ? 0 : a.ldr));
+    size_t fl = (size_t)2 * a.kr * a.ld + (size_t)tp() * (a.ld + row_extra);
     if (mode != DK_LSE && a.R > 1 && fl < (size_t)8 * pl.TK * (NT + a.T)) fl = (size_t)8 * pl.TK * (NT + a.T);
     pl.smem = fl * 4;
     pl.per_sm = pl.smem + 6144 <= 233472 / 2 ? 2 : 1;
@@ -651,7 +677,7 @@ cudaError_t launch_fused_direct(cudaStream_t s, const float* X, int64_t n, int D
         a.mu = mu; a.w2 = w2; a.c2d = c2d; a.g_out = g; a.llpart = llpart; a.ll_first = off == 0 ? 1 : 0; a.partials = partials;
         a.status = status;
         if (fit) { a.counts = fit->counts; a.stop_at = fit->stop_at; a.iter = fit->iter; }
-        const int64_t tp = (int64_t)pl.PT * (NT >> (a.lgG + a.lgS)), tiles = (cnt + tp - 1) / tp;
+        const int64_t tp = (int64_t)a.NS * pl.PT * (NT >> (a.lgG + a.lgS)), tiles = (cnt + tp - 1) / tp;
         const int grid = (int)(tiles < ctas ? tiles : ctas);
         cudaError_t e = direct_launch<DK_FUSED>(s, dim3((unsigned)grid), pl);
         if (e != cudaSuccess) return e;

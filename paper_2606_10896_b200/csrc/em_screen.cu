@@ -213,7 +213,13 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(int D, int K, int Kpa
     int pos = k;
     bool on = false, capped = false;
     float4 q = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
-    if (k < K) {
+    // (capped components and those without a weight at the far end, what is left of Kpad between them and the others: a block that
+    // holds a capped component has no lower bound)
+    if (k >= K) {
+        int before = 0;
+        for (int j = lane; j < K; j += 32) before += __ldg(key + j) < SCR_CAPPED ? 1 : 0;
+        pos = __reduce_add_sync(0xffffffffu, before) + k - K;
+    } else {
         const float mine = __ldg(key + k);
         int before = 0;
 #pragma unroll 8
@@ -221,7 +227,7 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(int D, int K, int Kpa
             const float o = __ldg(key + j);
             before += (o < mine || (o == mine && j < k)) ? 1 : 0;
         }
-        pos = __reduce_add_sync(0xffffffffu, before);
+        pos = __reduce_add_sync(0xffffffffu, before) + (mine >= SCR_CAPPED ? Kpad - K : 0);
         on = mine < CUDART_INF_F;
         capped = on && mine >= SCR_CAPPED;
         if (on) q = __ldg(prm + k);
@@ -561,7 +567,11 @@ screen_sweep_kernel(const SweepParams p) {
                 }
                 if (TOP > 1 && first) return;
                 const float cut = floor_now() - E;
-                if (in && bmax >= cut && bmax > 0.5f * SCR_NEVER) {
+                if (in && bmax >= cut) {
+                    if (!(cut > 0.5f * SCR_NEVER)) {         // no useful bound (yet): the values of positions without a component could
+                        lost = CUDART_INF_F;                 // pass, so the row is evaluated in full
+                        return;
+                    }
                     // bit j of the mask: value j reaches the cut (the sign of l - cut, shifted in from the top)
                     const uint64_t nc = pack2(__float_as_uint(-cut), __float_as_uint(-cut));
                     unsigned mask = 0;

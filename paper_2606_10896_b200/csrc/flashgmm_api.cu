@@ -432,9 +432,29 @@ bool auto_wants_planes(int D, int K) { return (tc_assign_supports(D, K) && K >= 
 // with fewer than about twice that per component on average most components would be.
 constexpr int64_t WIDE_AUTO_MIN_POINTS_PER_COMPONENT = 128;
 
-int ensure_scratch(gmm_ctx* ctx, int D, int K) {
-    const bool planes = (tc_assign_supports(D, K) || wide_supports(D, K)) &&
-                        (ctx->path == GMM_PATH_TENSOR || (ctx->path == GMM_PATH_AUTO && auto_wants_planes(D, K)));
+// What a call asks of the screening path (csrc/em_screen.cu).
+enum { SCREEN_STEPS = 0, SCREEN_CENTROIDS = 1, SCREEN_DENSITIES = 2, SCREEN_RANKS = 3 };
+
+// K < 64: what the FP32 kernels take per point, in ns, from measurements (1M points, a step: 128 x 48 2.5, 96 x 32 1.1, 32 x 63 0.7; the
+// assignment: 64 components x 32 dimensions at a time).  groups: of Fisher vectors, which go one after the other.
+double direct_cost(int kind, int64_t N, int D, int K, int64_t groups) {
+    const double kd = (double)K * D, tiles = 0.27 * ((D + 31) / 32);
+    return (kind == SCREEN_STEPS ? 0.05 + 3.8e-4 * kd : kind == SCREEN_DENSITIES ? 0.03 + 1.9e-4 * kd : kind == SCREEN_CENTROIDS ? 0.3 + tiles : tiles) +
+           15e3 * (double)groups / (double)N;
+}
+// Whether AUTO screens a call over N points at K < 64: with two marked pairs per point (0.75 ns at 128 x 48) and about 70 us more of
+// launches.
+bool small_screen(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
+    if (ctx->path != GMM_PATH_AUTO || ctx->scr_marks == 0.0 || N < 1 || K >= 64 || K < 16 || D < 8 || !screen_supports(D, K) || !tc_assign_supports(D, K)) return false;
+    const double screen = kind == SCREEN_STEPS ? 0.38 + 0.003 * D : kind == SCREEN_DENSITIES ? 0.3 + 0.002 * D : 0.26 + 0.002 * D;
+    return ctx->scr_marks > 0.0 || (double)N * (direct_cost(kind, N, D, K, groups) - screen) > 70e3;
+}
+
+int ensure_scratch(gmm_ctx* ctx, int D, int K, bool small = false) {
+    bool planes = (tc_assign_supports(D, K) || wide_supports(D, K)) &&
+                  (ctx->path == GMM_PATH_TENSOR || (ctx->path == GMM_PATH_AUTO && (auto_wants_planes(D, K) || small)));
+    // (K < 64: once there the planes stay, whatever the next call's number of points says)
+    if (ctx->scratch && D == ctx->capD && K == ctx->capK && ctx->path == GMM_PATH_AUTO && !auto_wants_planes(D, K) && ctx->capPlanes) planes = true;
     if (ctx->scratch && D == ctx->capD && K == ctx->capK && planes == ctx->capPlanes) return GMM_OK;
     const ScratchLayout L = scratch_layout(D, K, planes);
     if (ctx->scratch) {
@@ -818,15 +838,21 @@ int read_result(gmm_ctx* ctx, int slot, double* loglik) {
 // AUTO tries it first wherever it would take the tensor path.  Its kernels find out themselves whether it pays (SC_DENSE) and
 // then return at once, so a call enqueues the whole path, reads the verdict with its result and only then, if need be, runs the
 // dense kernels: sparse posteriors cost no extra synchronisation, broad ones the sweep of one piece.
-bool screen_wanted(const gmm_ctx* ctx, int D, int K) {
-    return ctx->path == GMM_PATH_AUTO && ctx->lay.scr && ctx->capPlanes && ctx->scr_marks != 0.0 && auto_is_tensor(D, K);
+bool screen_wanted(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
+    return ctx->path == GMM_PATH_AUTO && ctx->lay.scr && ctx->capPlanes && ctx->scr_marks != 0.0 &&
+           (auto_is_tensor(D, K) || small_screen(ctx, kind, N, D, K, groups));
+}
+// The dense tensor kernels for D <= 128 (planes may be there for the screening alone).
+bool dense_tensor(const gmm_ctx* ctx, int D, int K) {
+    return ctx->capPlanes && ctx->lay.tc && (ctx->path == GMM_PATH_TENSOR || (ctx->path == GMM_PATH_AUTO && auto_wants_planes(D, K)));
 }
 // Marked pairs per point up to which the screening path is the cheaper one, from measured costs in ns per point: the dense kernels
 // 0.5 + 0.0032 K (0.62 at 10 x 100, 0.83 at 64 x 128, 2.1 at 12 x 541, 3.7 at 128 x 1024), the sweep and what does not depend on the
 // marks 0.15 + 0.001 D + 0.045 per 128 components, a pair 0.09 + 0.001 D.  (At most SCR_MARKS.)
-double screen_limit(const gmm_ctx* ctx, int D, int K) {
+// K < 64: the FP32 kernels' costs.
+double screen_limit(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     if (ctx->scr_marks > 0.0) return ctx->scr_marks;
-    const double dense = 0.5 + 0.0032 * K, fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
+    const double dense = K < 64 ? direct_cost(kind, N, D, K, groups) : 0.5 + 0.0032 * K, fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
     return std::fmin((double)SCR_MARKS, std::fmax(1.5, 0.9 * (dense - fixed) / (0.09 + 0.001 * D)));
 }
 
@@ -857,14 +883,14 @@ int screen_values(gmm_ctx* ctx, int mode, const float* Xs, int64_t cnt, int D, i
 }
 
 // Adds the statistics of n points to (Nk, S1, S2) and their log-likelihood to the partial sums.
-int screen_points(gmm_ctx* ctx, const float* X, int64_t n, int D, int K, const float* mu, double* Nk, double* S1, double* S2) {
+int screen_points(gmm_ctx* ctx, const float* X, int64_t n, int D, int K, const float* mu, double* Nk, double* S1, double* S2, int64_t groups = 0) {
     const ScreenBuffers sb = ctx->screen();
     const int64_t piece = screen_piece(ctx, n);
     for (int64_t off = 0; off < n; off += piece) {
         const int64_t cnt = (n - off < piece) ? (n - off) : piece;
         const float* Xs = X + off * D;
         CHECK(prof_begin(ctx));
-        CHECK(screen_values(ctx, SCREEN_EM, Xs, cnt, D, K, 40.f, screen_limit(ctx, D, K), mu, nullptr, nullptr, true));
+        CHECK(screen_values(ctx, SCREEN_EM, Xs, cnt, D, K, 40.f, screen_limit(ctx, SCREEN_STEPS, n, D, K, groups), mu, nullptr, nullptr, true));
         CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         CHECK(prof_end(ctx));
     }
@@ -878,9 +904,8 @@ int screen_end(gmm_ctx* ctx, int K, int slot) {
 
 // Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels (nothing is
 // reported then: they find what is wrong again).
-enum { SCREEN_STEPS = 0, SCREEN_CENTROIDS = 1, SCREEN_DENSITIES = 2 };
-bool screen_try(gmm_ctx* ctx, int kind, int D, int K) {
-    if (!screen_wanted(ctx, D, K)) return false;
+bool screen_try(gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
+    if (!screen_wanted(ctx, kind, N, D, K, groups)) return false;
     auto& h = ctx->scr_history[kind];
     if (h.D != D || h.K != K) { h = {}; h.D = D; h.K = K; }
     if (ctx->scr_marks < 0.0 && h.left > 0) { --h.left; return false; }
@@ -1043,8 +1068,8 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     if (!loglik) return fail(ctx, GMM_EINVAL, "loglik is NULL");
     DeviceGuard g(ctx->device);
     int path;
-    CHECK(ensure_scratch(ctx, D, K));
-    if (screen_try(ctx, SCREEN_STEPS, D, K)) {
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
+    if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
         bool dense = false;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
         CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
@@ -1114,13 +1139,13 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
     if (!(tol >= 0.0)) return fail(ctx, GMM_EINVAL, "tol must be >= 0");
     DeviceGuard g(ctx->device);
     int path;
-    CHECK(ensure_scratch(ctx, D, K));
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
     const size_t KD = (size_t)K * D;
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
     int t = 0;
-    if (fused_direct_supports(D, K) && (ctx->path == GMM_PATH_FP32 || (ctx->path == GMM_PATH_AUTO && gmm_auto_path(D, K) == GMM_PATH_FP32))) {
+    if (fused_direct_supports(D, K) && !screen_wanted(ctx, SCREEN_STEPS, N, D, K) && (ctx->path == GMM_PATH_FP32 || (ctx->path == GMM_PATH_AUTO && gmm_auto_path(D, K) == GMM_PATH_FP32))) {
         // Small mixtures: two launches per iteration (the update and the next iteration's constants are part of the reduction), as
         // many iterations as there are slots for their log-likelihoods enqueued ahead; the device stops by itself where the
         // tolerance is met or a step fails.
@@ -1171,7 +1196,7 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         };
         int rc = GMM_OK;
         bool dense = true;
-        if (screen_try(ctx, SCREEN_STEPS, D, K)) {
+        if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
             CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
             CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
             CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
@@ -1215,7 +1240,7 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     if (!loglik) return fail(ctx, GMM_EINVAL, "loglik is NULL");
     DeviceGuard g(ctx->device);
     int path;
-    CHECK(ensure_scratch(ctx, D, K));
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
     const size_t KD = (size_t)K * D;
     // one-time resources of the host path.  A staging buffer holds 128 MiB of rows; on wide data a whole piece of the
     // tensor path (2^17 rows: 403 MB at D = 768), whose kernels lose a third of their speed on pieces a third the size.
@@ -1283,7 +1308,7 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     CU(cudaMemcpyAsync(ctx->xstage[0], X_host, (size_t)cnt0 * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
     CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
-    bool screening = screen_try(ctx, SCREEN_STEPS, D, K);
+    bool screening = screen_try(ctx, SCREEN_STEPS, N, D, K);
     if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
     else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
     CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
@@ -1349,7 +1374,7 @@ int gmm_assign_topm(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     if (resp) CHECK(check_ptr(ctx, resp, 4, "resp"));
     if (m < 1 || m > K || m > GMM_MAX_TOPM) return fail(ctx, GMM_EINVAL, "m must be in [1, min(K, %d)] (got %d)", GMM_MAX_TOPM, m);
     DeviceGuard g(ctx->device);
-    CHECK(ensure_scratch(ctx, D, K));
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_RANKS, N, D, K)));
     return assign_topm_impl(ctx, X, N, D, K, pi, mu, var, m, idx, resp, resp == nullptr);
 }
 
@@ -1360,8 +1385,8 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
     // (the screening path's preparation does what this one does, but for the centre of the means)
     // (When it pays is known on the device alone, so shapes for which it mostly did not are left out: many components in few
     // dimensions overlap, and with few components the quarters of blocks that bound the m-th best do not bound it well.)
-    const bool screening = !screened && m <= 4 && screen_wanted(ctx, D, K) &&
-                           (ctx->scr_marks > 0.0 || ((double)D >= 1.75 * std::log2((double)K) - 2.0 && K >= 48 * m && (m <= 2 || K >= 3 * D)));
+    const bool screening = !screened && m <= 4 && m <= K && screen_wanted(ctx, SCREEN_RANKS, N, D, K) &&
+                           (ctx->scr_marks > 0.0 || ((double)D >= 1.75 * std::log2((double)K) - 2.0 && (m == 1 || K >= 48 * m) && (m <= 2 || K >= 3 * D)));
     if (!screening) KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), &ctx->result()->status));
     if (!screening && (size_t)K * D > ((size_t)1 << 12)) ctx->launches++;      // but for tiny problems, the centre of the means is a launch of its own
     // Tensor-core assignment where the E+M step would take the tensor path too.  Ill-conditioned components are evaluated
@@ -1506,29 +1531,29 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
         ctx->last_path = tensor_w ? GMM_PATH_TENSOR : GMM_PATH_FP32;
         return GMM_OK;
     }
-    const bool tensor = ctx->capPlanes && ctx->lay.tc && ctx->path != GMM_PATH_FP32;
+    const bool tensor = dense_tensor(ctx, D, K);
     const int* run_fp32_if = nullptr;
+    // Sparse posteriors: the pairs that can be among the m best, or within 2^-40 of the best, are marked by the screening sweep
+    // and evaluated exactly.  The call is asynchronous, so the other kernels are enqueued all the same and return at once
+    // unless the screening has left the call to them.
+    // (The lists have room for 16 pairs per point; a pair costs a quarter of the sweep at K = 1024.)
+    const int* dense_if = nullptr;
+    if (screening) {
+        dense_if = run_fp32_if = ctx->result()->scr + SC_DENSE;
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        const int64_t piece = screen_piece(ctx, N);
+        for (int64_t off = 0; off < N; off += piece) {
+            const int64_t cnt = (N - off < piece) ? (N - off) : piece;
+            CHECK(prof_begin(ctx));
+            CHECK(screen_values(ctx, SCREEN_TOP, X + off * D, cnt, D, K, index_only ? 0.f : 40.f, ctx->scr_marks > 0.0 ? ctx->scr_marks : 12.0, mu, nullptr,
+                                idx + off * m, false, m, index_only ? nullptr : resp + off * m));
+            CHECK(prof_end(ctx));
+        }
+        KL(launch_center_fp32(ctx->stream, D, K, mu, ctx->center(), dense_if));
+    }
     if (tensor) {
         const TcBuffers tb = ctx->tc();
         const float limit = ctx->tc_cond_limit >= 0.f ? ctx->tc_cond_limit : 0.01f;
-        // Sparse posteriors: the pairs that can be among the m best, or within 2^-40 of the best, are marked by the screening sweep
-        // and evaluated exactly.  The call is asynchronous, so the tile kernels below are enqueued all the same and return at once
-        // unless the screening has left the call to them.
-        // (The lists have room for 16 pairs per point; a pair costs a quarter of the sweep at K = 1024.)
-        const int* dense_if = nullptr;
-        if (screening) {
-            dense_if = ctx->result()->scr + SC_DENSE;
-            CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
-            const int64_t piece = screen_piece(ctx, N);
-            for (int64_t off = 0; off < N; off += piece) {
-                const int64_t cnt = (N - off < piece) ? (N - off) : piece;
-                CHECK(prof_begin(ctx));
-                CHECK(screen_values(ctx, SCREEN_TOP, X + off * D, cnt, D, K, index_only ? 0.f : 40.f, ctx->scr_marks > 0.0 ? ctx->scr_marks : 12.0, mu, nullptr,
-                                    idx + off * m, false, m, index_only ? nullptr : resp + off * m));
-                CHECK(prof_end(ctx));
-            }
-        }
-        if (screening) KL(launch_center_fp32(ctx->stream, D, K, mu, ctx->center(), dense_if));
         KL(launch_prepare_tc(ctx->stream, D, K, pi, mu, var, tb, limit, &ctx->result()->status, true, dense_if));
         ctx->launches += 3;
         run_fp32_if = tb.flags + 3;
@@ -1577,7 +1602,7 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
         const int64_t cnt = (N - off < SUPER_TILE) ? (N - off) : SUPER_TILE;
         KL(launch_topm_fp32(ctx->stream, X + off * D, cnt, D, K, mu, ctx->w2(), ctx->c2d(), ctx->center(), m, idx + off * m, resp ? resp + off * m : nullptr, run_fp32_if));
     }
-    ctx->last_path = tensor ? GMM_PATH_TENSOR : GMM_PATH_FP32;
+    ctx->last_path = tensor || screening ? GMM_PATH_TENSOR : GMM_PATH_FP32;
     return GMM_OK;
 }
 }  // namespace
@@ -1678,10 +1703,10 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     if (N >= ((int64_t)1 << 31)) return fail(ctx, GMM_EUNSUPPORTED, "N must be below 2^31 (point indices are int32)");
     if (K > PL_MAX_K) return fail(ctx, GMM_EUNSUPPORTED, "K must be <= %d for the k-means step (got %d)", PL_MAX_K, K);
     DeviceGuard g(ctx->device);
-    CHECK(ensure_scratch(ctx, D, K));
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_CENTROIDS, N, D, K)));
     CHECK(grow_buffer(ctx, &ctx->pl_scratch, &ctx->pl_scratch_bytes, pl_scratch_bytes(K), "the posting-list counters"));
     CHECK(grow_buffer(ctx, &ctx->km_scratch, &ctx->km_scratch_bytes, km_scratch_bytes(D, K), "the k-means partial sums"));
-    if (screen_try(ctx, SCREEN_CENTROIDS, D, K)) {
+    if (screen_try(ctx, SCREEN_CENTROIDS, N, D, K)) {
         // through the screening path: the arg-max alone (margin 0), every point a lone pair of its cluster, and the statistics
         // of the pairs about the centroids give the new ones and the inertia
         const ScreenBuffers sb = ctx->screen();
@@ -1694,7 +1719,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
             const float* Xs = X + off * D;
-            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, D, K), centroids, nullptr, assign + off, true));
+            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, SCREEN_CENTROIDS, N, D, K), centroids, nullptr, assign + off, true));
             CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, centroids, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         }
         double* ik = km_inertia_k(ctx->km_scratch, D, K);
@@ -1713,7 +1738,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     // nearest centroid = top-1 component of a unit-variance, equal-weight mixture
     float* resp = reinterpret_cast<float*>(work);                 // [N], not used afterwards except as the builder's input
     int32_t* items = work + N;                                    // [N]
-    bool tensor = ctx->capPlanes && ctx->lay.tc && ctx->path != GMM_PATH_FP32;
+    bool tensor = dense_tensor(ctx, D, K);
     const bool tensor_wide = ctx->capPlanes && ctx->lay.wide && ctx->path != GMM_PATH_FP32 && K >= 64;
     if (tensor_wide) {
         // wide data: the hard assignment of the wide tensor path (screening, or six candidates per point), under a mixture
@@ -1766,11 +1791,12 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
     CHECK(check_ptr(ctx, var, 4, "var"));
     CHECK(check_ptr(ctx, logp, 4, "logp"));
     DeviceGuard guard(ctx->device);
-    CHECK(ensure_scratch(ctx, D, K));
-    if (screen_try(ctx, SCREEN_DENSITIES, D, K)) {
-        // D <= 128: the same idea (csrc/em_screen.cu).  The FP32 kernel takes 1.4e-4 K D ns per point, the screening path about
-        // 0.8 ns and 0.25 ns per marked pair.
-        const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks : std::fmin(14.0, std::fmax(1.5, (1.4e-4 * K * D - 0.8) / 0.25));
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_DENSITIES, N, D, K)));
+    if (screen_try(ctx, SCREEN_DENSITIES, N, D, K)) {
+        // D <= 128: the same idea (csrc/em_screen.cu).  Costs per point as in screen_limit, without statistics.
+        const double fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
+        const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks
+                             : std::fmin(14.0, std::fmax(1.5, 0.9 * (0.03 + 1.9e-4 * K * D - fixed) / (0.05 + 0.0007 * D)));
         bool dense = false;
         double total = 0.0;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
@@ -1890,12 +1916,12 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
         if (T > 0 && (smallest == 0 || T < smallest)) smallest = T;
     }
     DeviceGuard guard(ctx->device);
-    CHECK(ensure_scratch(ctx, D, K));
+    CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K, G)));
     const size_t KD = (size_t)K * D;
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
-    if (smallest > 0 && screen_try(ctx, SCREEN_STEPS, D, K)) {
+    if (smallest > 0 && screen_try(ctx, SCREEN_STEPS, N, D, K, G)) {
         // Screening path: consecutive groups are taken as many at a time as a piece holds; a larger group goes
         // through the step's own accumulation.
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
@@ -1928,13 +1954,13 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
             float* out = fv + (size_t)bt.g0 * 2 * KD;
             if (bt.large) {
                 CU(cudaMemsetAsync(Nk, 0, ((size_t)K + 2 * KD) * 8, ctx->stream));
-                CHECK(screen_points(ctx, Xs, rows, D, K, mu, Nk, S1, S2));
+                CHECK(screen_points(ctx, Xs, rows, D, K, mu, Nk, S1, S2, G));
                 KL(launch_fisher(ctx->stream, rows, D, K, Nk, S1, S2, pi, mu, var, out));
             } else if (rows == 0) {
                 CU(cudaMemsetAsync(out, 0, (size_t)(bt.g1 - bt.g0) * 2 * KD * sizeof(float), ctx->stream));
             } else {
                 CHECK(prof_begin(ctx));
-                CHECK(screen_values(ctx, SCREEN_EM, Xs, rows, D, K, 40.f, screen_limit(ctx, D, K), mu, nullptr, nullptr, false));
+                CHECK(screen_values(ctx, SCREEN_EM, Xs, rows, D, K, 40.f, screen_limit(ctx, SCREEN_STEPS, N, D, K, G), mu, nullptr, nullptr, false));
                 CU(launch_screen_groups(ctx->stream, Xs, bt.g1 - bt.g0, D, K, d_tab + bt.g0, d_tab + G + bt.g0, d_off, pi, mu, var, ctx->w2(),
                                         ctx->c2d(), sb, out, &ctx->launches));
                 CHECK(prof_end(ctx));

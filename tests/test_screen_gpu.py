@@ -56,7 +56,7 @@ def _step(fg, c, X, pi, mu, var, expect_count, what):
 
 # tiles of 256 points, ranges of 512, atoms of 32 dimensions, k-steps of 8, groups of 128 and blocks of 32 components
 @pytest.mark.parametrize("N,D,K", [(1, 8, 64), (255, 128, 64), (257, 33, 65), (511, 31, 128), (513, 32, 129), (1024, 97, 257),
-                                   (1500, 41, 1000), (1300, 9, 90), (3001, 127, 96), (700, 64, 4096), (2049, 100, 160)])
+                                   (1500, 41, 1000), (1300, 9, 90), (1500, 24, 16), (2049, 128, 48), (3001, 127, 96), (700, 64, 4096), (2049, 100, 160)])
 def test_screen_against_oracle_at_the_edges_of_its_tiles(fg, monkeypatch, N, D, K):
     monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
     X, pi, mu, var = _mixture(N, D, K, N + D + K, collapsed=3)
@@ -133,7 +133,7 @@ def test_config2_free_running_through_the_screening_path(fg):
 
 # the other entry points on the path, in pieces of 768 points: several tiles and pieces, a last piece of one point, groups that are
 # empty, larger than a piece, or share one
-@pytest.mark.parametrize("N,D,K", [(1, 16, 64), (3073, 40, 100), (2500, 128, 1024), (4000, 9, 300), (900, 66, 4096)])
+@pytest.mark.parametrize("N,D,K", [(1, 16, 64), (3073, 40, 100), (2500, 128, 1024), (4000, 9, 300), (900, 66, 4096), (3000, 33, 31)])
 def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
     from oracle.fisher import fisher_vectors
     from oracle.kmeans import kmeans_step
@@ -169,7 +169,7 @@ def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
 
 # the top-m assignment through the sweep: a point far away from everything, components without a weight (fewer than m with one, once)
 @pytest.mark.parametrize("N,D,K,m", [(1, 16, 64, 1), (257, 33, 97, 2), (3001, 128, 1024, 2), (3001, 128, 1024, 4), (1500, 20, 300, 3), (900, 66, 4096, 4),
-                                     (2000, 9, 130, 1), (300, 12, 192, 4)])
+                                     (2000, 9, 130, 1), (300, 12, 192, 4), (1200, 40, 20, 1)])
 def test_screen_top_m(fg, monkeypatch, N, D, K, m):
     monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
     monkeypatch.setenv("GMM_SCREEN_PIECE", "768")

@@ -927,7 +927,40 @@ __global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restric
 // Bound by instruction issue and the trips to L2 for the components' rows (1 KB per pair at D = 128).
 constexpr int EV_VALS = 32 * SCR_SLOTS;
 // TOP: the m (<= 4) largest values go out, the smaller component first where two are equal.
-struct TopOut { int m; float* resp; };
+struct TopOut { int m; float* resp; ScreenTie tie; };
+
+// Two centroids at the same distance but for rounding: one such point in a small cluster moves its centroid, so the nearest-centroid
+// search decides near ties in the arithmetic of the kernels that take the call when the posteriors are broad.  The whole warp, one
+// point: all its candidates within `near` of the best.
+__device__ int screen_nearest(const ScreenTie& tie, const float* __restrict__ x, int D, const float* __restrict__ mu, const float* l_s,
+                              const unsigned short* k_s, int cnt, float mx, float near, int lane) {
+    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(x) & 15) == 0);
+    float bv = -CUDART_INF_F;
+    int bk = 0x7fffffff;
+    for (int j = 0; j < cnt; ++j) {
+        if (!(l_s[j] >= mx - near)) continue;                // warp-uniform
+        const int k = k_s[j];
+        const float* m = mu + (size_t)k * D;
+        float q = 0.f;
+        if (tie.g == nullptr) {                              // as the refinement of the tensor assignment: 4 dimensions per lane, butterfly
+            for (int t = 0; t < 4; ++t) {
+                const int d = vec ? 4 * lane + t : lane + 32 * t;
+                if (d < D) { const float diff = __ldg(x + d) - __ldg(m + d); q = fmaf(diff * diff, tie.w, q); }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        } else {                                             // as the FP32 tile kernel: one chain about the centre
+            for (int d = 0; d < D; ++d) {
+                const float g = __ldg(tie.g + d), t = fmaf(__ldg(x + d) - g, 1.f, g - __ldg(m + d));
+                q = fmaf(t, t, q);
+            }
+        }
+        const float e = tie.c - q;
+        if (e > bv || (e == bv && k < bk)) { bv = e; bk = k; }
+    }
+    return bk;
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __restrict__ mu,
                                                              const float* __restrict__ w2, const double* __restrict__ c2d,
@@ -1046,6 +1079,18 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             } else {
                 for (int j = 0; j < cnt; ++j) mx = fmaxf(mx, v_s[warp][p0 + j]);
                 for (int j = 0; j < cnt; ++j) sum += fast_ex2(v_s[warp][p0 + j] - mx);
+            }
+        }
+        if (MODE == SCREEN_ARGMAX) {
+            int near_n = 0;                                  // candidates within rounding of the best
+            const float near = 4e-6f * (fabsf(mx) + 300.f);
+            for (int j = 0; j < todo; ++j) near_n += v_s[warp][p0 + j] >= mx - near ? 1 : 0;
+            for (unsigned ties = __ballot_sync(0xffffffffu, near_n > 1); ties; ties &= ties - 1) {
+                const int src = __ffs(ties) - 1;
+                const int at = __shfl_sync(0xffffffffu, p0, src), n_c = __shfl_sync(0xffffffffu, todo, src);
+                const float top_v = __shfl_sync(0xffffffffu, mx, src), band = __shfl_sync(0xffffffffu, near, src);
+                const int k = screen_nearest(top.tie, X + (row0 + src) * D, D, mu, &v_s[warp][at], &k_s[warp][at], n_c, top_v, band, lane);
+                if (lane == src) best = k;
             }
         }
         // rows with lists of their own length: the whole warp, one row after the other, values in `val`
@@ -1784,7 +1829,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
 }
 
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
-                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count, int m, float* resp) {
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count, int m, float* resp, const ScreenTie* tie) {
     // 32 points per warp (fewer where that leaves the chip short of warps); ranges as launch_screen_stats has them
     const int pw = n < 131072 ? 8 : n < 200000 ? 16 : 32, range = count ? screen_range(n) : 8 * pw;
     const unsigned blocks = (unsigned)((n + range - 1) / range);
@@ -1798,9 +1843,9 @@ cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t
     else if (mode == SCREEN_LOGP)
         screen_eval_kernel<SCREEN_LOGP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, b.ll, logp, nullptr, b.ctl, TopOut{});
     else if (mode == SCREEN_TOP)
-        screen_eval_kernel<SCREEN_TOP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, nullptr, nullptr, idx, b.ctl, TopOut{m, resp});
+        screen_eval_kernel<SCREEN_TOP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, nullptr, nullptr, idx, b.ctl, TopOut{m, resp, ScreenTie{}});
     else
-        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, nullptr, nullptr, idx, b.ctl, TopOut{});
+        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, nullptr, nullptr, idx, b.ctl, TopOut{0, nullptr, tie ? *tie : ScreenTie{}});
     return cudaGetLastError();
 }
 

@@ -80,12 +80,16 @@ cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi,
 cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, int top, float max_marks, bool stats,
                                 const float* mu, const float* w2, const double* c2d, const ScreenBuffers& b, int* status, int sms,
                                 int64_t* launches);
+// SCREEN_ARGMAX: how near ties are decided.  g: NULL, or the centre of the FP32 tile kernel (then w = 1, c = 0); else weight and constant
+// of the unit mixture that the tensor assignment is given.
+struct ScreenTie { const float* g; float w, c; };
 // Exact values of the marked pairs.  SCREEN_EM: responsibilities of the pairs within 2^-40 of their point's total, counted per
 // component; SCREEN_LOGP: logp[i]; SCREEN_ARGMAX: idx[i], and the pair itself kept with weight 1 for the statistics.
 // SCREEN_TOP: the m largest pairs of every point into idx [n][m] and (may be NULL) their responsibilities into resp [n][m].
 enum { SCREEN_EM = 0, SCREEN_LOGP = 1, SCREEN_ARGMAX = 2, SCREEN_TOP = 3 };
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
-                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count = true, int m = 1, float* resp = nullptr);
+                               const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count = true, int m = 1, float* resp = nullptr,
+                               const ScreenTie* tie = nullptr);
 // (count: leave the number of kept pairs per component and range for launch_screen_stats)
 // After the last piece of an asynchronous assignment: *gate |= the screening covered the call; *fallback = it did not and *gate was set.
 cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback);

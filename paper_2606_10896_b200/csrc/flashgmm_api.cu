@@ -875,10 +875,10 @@ int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, c
 
 // One piece's lists (sweep) and values (see launch_screen_eval).
 int screen_values(gmm_ctx* ctx, int mode, const float* Xs, int64_t cnt, int D, int K, float margin, double limit, const float* mu,
-                  float* logp, int32_t* idx, bool count, int m = 1, float* resp = nullptr) {
+                  float* logp, int32_t* idx, bool count, int m = 1, float* resp = nullptr, const ScreenTie* tie = nullptr) {
     const ScreenBuffers sb = ctx->screen();
     CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, margin, mode == SCREEN_TOP ? m : 1, (float)limit, mode == SCREEN_EM || mode == SCREEN_ARGMAX, mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
-    KL(launch_screen_eval(ctx->stream, mode, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, logp, idx, count, m, resp));
+    KL(launch_screen_eval(ctx->stream, mode, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, logp, idx, count, m, resp, tie));
     return GMM_OK;
 }
 
@@ -1714,12 +1714,19 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         double* S1 = Nk + K;
         double* S2 = S1 + (size_t)K * D;
         CHECK(screen_begin(ctx, D, K, nullptr, centroids, nullptr, true));
+        // (the kernels below would decide a near tie in fp32 about a centre, or among log-densities of the unit mixture)
+        ScreenTie tie{nullptr, (float)0.72134752044448170368,
+                      (float)(1.4426950408889634074 * (std::log((double)(1.f / (float)K)) - 0.5 * D * std::log(6.283185307179586476925286766559)))};
+        if (!auto_is_tensor(D, K)) {
+            KL(launch_center_fp32(ctx->stream, D, K, centroids, ctx->center()));
+            tie = {ctx->center(), 1.f, 0.f};
+        }
         CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
             const float* Xs = X + off * D;
-            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, SCREEN_CENTROIDS, N, D, K), centroids, nullptr, assign + off, true));
+            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, SCREEN_CENTROIDS, N, D, K), centroids, nullptr, assign + off, true, 1, nullptr, &tie));
             CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, centroids, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         }
         double* ik = km_inertia_k(ctx->km_scratch, D, K);

@@ -73,17 +73,21 @@ int gmm_set_path(gmm_ctx* ctx, int path);
 int gmm_tensor_path_supports(int D, int K);
 /* The path GMM_PATH_AUTO picks for shape (D, K): the tensor-core path when it is supported and the shape fills at
  * least half of a 128-component MMA tile (K >= 64, and D >= 8); otherwise the FP32 path, which is both faster and more
- * accurate for small mixtures.  On wide data (D > 128) a step may still run on the FP32 kernels when the parameters
+ * accurate for small mixtures.  For D <= 128 AUTO first tries one tensor sweep that only screens the (point, component)
+ * pairs and evaluates those it cannot rule out (every component within 2^-40 of a point's best) exactly in fp32: on sparse
+ * posteriors this is the faster and the more accurate way, also for calls with many points and 16 <= K < 64 (GMM_PATH_TENSOR is
+ * then reported).  Broad posteriors are noticed on the device and left to the dense kernels of either path; after such a
+ * call the context leaves the next calls of that kind and shape (1, 2, 4 .. 16) to them at once.  On wide data (D > 128) a step may still run on the FP32 kernels when the parameters
  * or the data make that the better choice (more than half of the components ill-conditioned; fewer than 128 points per
  * component and posteriors too broad for the screening mode): gmm_last_path tells. */
 int gmm_auto_path(int D, int K);
 /* The path (GMM_PATH_FP32 or GMM_PATH_TENSOR) the most recent compute call actually ran. */
 int gmm_last_path(const gmm_ctx* ctx);
 /* How many components the most recent tensor-path step treated as ill-conditioned, i.e. evaluated (where they matter)
- * exactly in fp32 instead of through the expanded quadratic form; 0 after a step on the FP32 path.  On wide data
- * (D > 128), whenever a sample of the points shows that few pairs per point matter, the tensor path only screens the
- * (point, component) pairs and evaluates all that can matter exactly: the count is then the number of components with a
- * positive weight. */
+ * exactly in fp32 instead of through the expanded quadratic form; 0 after a step on the FP32 path.  Where few pairs per
+ * point matter (D <= 128 under GMM_PATH_AUTO; D > 128 whenever a sample of the points shows it), the tensor path only screens
+ * the (point, component) pairs and evaluates all that can matter exactly: the count is then the number of components with
+ * a positive weight. */
 int gmm_last_exact_count(const gmm_ctx* ctx);
 /* For the most recent tensor-path step on wide data (D > 128) that had such components: how their (point, component)
  * pairs were evaluated.  *marked: pairs the screening sweep and its filter could not rule out; *kept: pairs whose exact density came
@@ -155,7 +159,9 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K,
  * as a selection pass and the best few per point are recomputed exactly in fp32, so indices and values are those of the
  * FP32 kernels; a point whose selection is not certain within the error bound of the selection pass is evaluated
  * against all K components exactly; components whose responsibility for a point is below 4.8e-7 keep the order and
- * the values of the selection pass (inside the 1e-6 tie width).  On wide data (D > 128), whenever a sample of the points
+ * the values of the selection pass (inside the 1e-6 tie width).  For D <= 128, m <= 4 and GMM_PATH_AUTO a screening sweep
+ * goes first: the pairs that can be among a point's m best or lie within 2^-40 of its best are evaluated exactly, and when the
+ * device finds them few the other kernels return at once.  On wide data (D > 128), whenever a sample of the points
  * shows that few (point, component) pairs matter, one tensor sweep screens all pairs instead, every component within
  * 2^-40 of a point's best is evaluated exactly (indices and responsibilities from those values), and ranks beyond them
  * are reported with responsibility 0 in the order of the sweep's upper bounds.  Parameters with more than 256 ill-conditioned
@@ -202,8 +208,8 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
  *   X [N x D], pi [K], mu [K x D], var [K x D]: device fp32, as for gmm_em_step.
  *   logp [N] fp32, device out (natural logarithm);  loglik (host out, may be NULL): their sum in float64.
  * Every value comes from exact direct-difference logits in fp32 (a per-point value has no averaging over points to absorb
- * approximate logits): the log-sum-exp kernel of the FP32 path, or, on wide data (D > 128, K >= 64, path not forced to
- * FP32) whenever a sample of the points shows that few (point, component) pairs matter, one tensor sweep that screens the
+ * approximate logits): the log-sum-exp kernel of the FP32 path, or, whenever few (point, component) pairs matter (D <= 128:
+ * GMM_PATH_AUTO, see gmm_auto_path; D > 128: K >= 64, path not forced to FP32), one tensor sweep that screens the
  * pairs followed by the exact evaluation of those it cannot rule out (every component within 2^-40 of a point's best);
  * gmm_last_path tells which.  Errors as gmm_em_step.  Synchronises the stream. */
 int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const float* pi, const float* mu,
@@ -224,8 +230,9 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
  *   fv [G x 2 x K x D] fp32, device out: per group the means part [K x D], then the standard-deviations part [K x D].
  *   No power or L2 normalisation is applied.
  *   loglik (host out, may be NULL): the total log-likelihood of all the groups' points.
- * On the tensor-core path several groups share a launch (each group of CTAs accumulates one of them); groups too large
- * for that are accumulated one at a time.
+ * Sparse posteriors (D <= 128, GMM_PATH_AUTO): the groups' pairs are screened and evaluated together and summed group by group
+ * about the component means.  Otherwise, on the tensor-core path several groups share a launch (each group of CTAs
+ * accumulates one of them); groups too large for that are accumulated one at a time.
  * Accuracy: a coordinate is a difference of the raw moments (N_k, S1, S2), which carry about 4e-6 relative error, so
  * with A_k = N_k / (T sqrt(pi_k)) (at most about 1 for a group that resembles the mixture, up to 1 / sqrt(pi_k) for a
  * group that sits on one light component) the error is about 2e-5 (1 + max|G|) + A_k (1e-3 + 4e-5 (1 + mu^2 / var));
@@ -274,8 +281,9 @@ int gmm_sync_status(gmm_ctx* ctx);
 int gmm_update_counts(gmm_ctx* ctx, int64_t* floored_variances, int64_t* empty_components);
 
 /* Bytes of device scratch a context in GMM_PATH_AUTO holds for shape (D, K); independent of N.  Where the tensor
- * path runs (see gmm_auto_path) this includes 512 MiB for the fp16 planes of one launch-sized piece of the data;
- * forcing GMM_PATH_TENSOR on a shape AUTO sends to the FP32 path adds the same 512 MiB. */
+ * path runs (see gmm_auto_path) this includes 512 MiB for the fp16 planes of one launch-sized piece of the data, and for
+ * D <= 128 up to 450 MiB of lists; forcing GMM_PATH_TENSOR on a shape AUTO sends to the FP32 path, or a screened call with
+ * K < 64, adds the same. */
 size_t gmm_scratch_bytes(int D, int K);
 
 /* Instrumentation.  Kernel launches enqueued by this context since creation (or the last reset). */

@@ -1298,7 +1298,14 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
-    const int64_t rows_per_chunk = (int64_t)(ctx->xstage_bytes / ((size_t)D * 4));
+    int64_t rows_per_chunk = (int64_t)(ctx->xstage_bytes / ((size_t)D * 4));
+    if (D <= 128) {
+        // What is left when the last copy ends is the last chunk's kernels: a sixteenth of the data, but no less than 8 MiB (150 us of
+        // copying, about what a chunk's launches take).  1M x 128: 9.82 ms with chunks of 128 MiB.
+        const int64_t rows = ((N + 15) / 16 + 255) / 256 * 256, least = ((int64_t)8 << 20) / ((int64_t)D * 4);
+        const int64_t want = rows > least ? rows : least;
+        if (want < rows_per_chunk) rows_per_chunk = want;
+    }
     if (rows_per_chunk < 1) return fail(ctx, GMM_EINVAL, "D too large for the staging buffer");
     // The first chunk is on its way before the parameters are prepared: on wide data the automatic choice of the mode
     // looks at its first rows.  (The copy stream must not overtake work of an earlier call that still reads the buffer.)

@@ -1484,19 +1484,19 @@ __global__ void __launch_bounds__(1024) screen_reduce_kernel(int D, int K, const
                                                              double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
                                                              double* __restrict__ llk, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
-    const int k = blockIdx.x, d = threadIdx.x & 127, r = threadIdx.x >> 7;
+    const int k = blockIdx.x, d = threadIdx.x & 127, r = threadIdx.x >> 7, chains = blockDim.x >> 7;      // (2 or 8)
     const int i0 = segoff[k], i1 = segoff[k + 1];
     if (i0 == i1) return;
     __shared__ double sh[8][128][2];
     __shared__ double tot[3];
     const size_t st = (size_t)(2 * D + 3);
     double a = 0.0, b = 0.0;
-    for (int i = i0 + r; i < i1; i += 32) {
+    for (int i = i0 + r; i < i1; i += 4 * chains) {
         float qa[4], qb[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const bool in = i + 8 * u < i1 && d < D;
-            const float* q = part + (size_t)(i + 8 * u) * st;
+            const bool in = i + chains * u < i1 && d < D;
+            const float* q = part + (size_t)(i + chains * u) * st;
             qa[u] = in ? q[d] : 0.f;
             qb[u] = in ? q[D + d] : 0.f;
         }
@@ -1517,8 +1517,7 @@ __global__ void __launch_bounds__(1024) screen_reduce_kernel(int D, int K, const
     const double n = tot[0];
     if (d < D) {
         a = b = 0.0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { a += sh[j][d][0]; b += sh[j][d][1]; }
+        for (int j = 0; j < chains; ++j) { a += sh[j][d][0]; b += sh[j][d][1]; }
         const double m = (double)__ldg(mu + (size_t)k * D + d);
         S1[(size_t)k * D + d] += a + m * n;
         S2[(size_t)k * D + d] += b + 2.0 * m * a + m * m * n;
@@ -1899,7 +1898,8 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     while (4 * lpr < D) lpr <<= 1;
     screen_stats_kernel<<<148 * 6, 256, (size_t)(K + 1) * 4, s>>>(X, D, lpr, mu, w2, b.srt, b.off, b.segoff, K, b.part, b.ctl);
     LCHECK();
-    screen_reduce_kernel<<<K, 1024, 0, s>>>(D, K, b.part, b.segoff, mu, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
+    // (eight chains per dimension where components have many items; with a few, CTAs of 1024 threads were 28 us of mostly waiting)
+    screen_reduce_kernel<<<K, n >= (int64_t)512 * K ? 1024 : 256, 0, s>>>(D, K, b.part, b.segoff, mu, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
     *launches += 4;
     return cudaGetLastError();
 }

@@ -251,6 +251,7 @@ struct gmm_ctx {
     // (1, 2, 4 .. 16: mixtures of a fit sharpen as it goes on); see screen_try.
     struct ScreenHistory { int D = 0, K = 0, skip = 0, left = 0; } scr_history[3];
     int scr_kind = 0;
+    DevResult* pinned = nullptr;     // where the result block is read back to
     int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
     int sticky_status = 0;           // status bits read off the device but not yet reported (see ensure_scratch)
     // host-streaming path
@@ -668,9 +669,10 @@ int prepare_and_choose(gmm_ctx* ctx, int64_t N, int D, int K, const float* pi, c
     return GMM_OK;
 }
 
-// Adds the statistics of n device-resident points to (Nk, S1, S2) and their log-likelihood to result()->ll[slot].
+// Adds the statistics of n device-resident points to (Nk, S1, S2) and their log-likelihood to result()->ll[slot] (fresh, one pass
+// for K <= 64 only: writes them).
 int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, int K, const float* mu, double* Nk,
-                      double* S1, double* S2, int slot) {
+                      double* S1, double* S2, int slot, bool fresh = false) {
     if (path == GMM_PATH_TENSOR && wide_supports(D, K)) {
         // Two sweeps per piece of at most 2^17 points (the capacity of the planes of Y and of the log2 Z buffer): planes,
         // log-sum-exp, responsibilities + statistics into per-CTA fp32 partials, which are folded into the float64
@@ -779,7 +781,7 @@ int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, 
     if (fused_direct_supports(D, K)) {
         CHECK(prof_begin(ctx));
         CU(launch_fused_direct(ctx->stream, X, n, D, K, mu, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), ctx->partials(), ctx->llpart(), Nk, S1, S2,
-                               true, &ctx->result()->ll[slot], &ctx->result()->status, nullptr, &ctx->launches));
+                               !fresh, &ctx->result()->ll[slot], &ctx->result()->status, nullptr, &ctx->launches));
         CHECK(prof_end(ctx));
         return GMM_OK;
     }
@@ -797,12 +799,25 @@ int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, 
     return GMM_OK;
 }
 
-int zero_stats(gmm_ctx* ctx, int D, int K, double* Nk, double* S1, double* S2, int slot) {
-    const size_t KD = (size_t)K * D;
-    CU(cudaMemsetAsync(Nk, 0, (size_t)K * 8, ctx->stream));
-    CU(cudaMemsetAsync(S1, 0, KD * 8, ctx->stream));
-    CU(cudaMemsetAsync(S2, 0, KD * 8, ctx->stream));
-    CU(cudaMemsetAsync(&ctx->result()->ll[slot], 0, 8, ctx->stream));
+// (one launch; screened: the screening path's partial log-likelihoods too)
+int zero_stats(gmm_ctx* ctx, int D, int K, double* Nk, double* S1, double* S2, int slot, bool screened = false) {
+    KL(launch_zero_stats(ctx->stream, D, K, Nk, S1, S2, &ctx->result()->ll[slot], screened ? ctx->screen().ll : nullptr, SCR_LL + K));
+    return GMM_OK;
+}
+
+// The result block, read through pinned memory; synchronises.
+int read_back(gmm_ctx* ctx, DevResult* r) {
+    if (!ctx->pinned) {
+        void* h = nullptr;
+        if (cudaMallocHost(&h, sizeof(DevResult)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(ctx, GMM_ENOMEM, "cannot allocate %zu bytes of pinned memory", sizeof(DevResult));
+        }
+        ctx->pinned = static_cast<DevResult*>(h);
+    }
+    CU(cudaMemcpyAsync(ctx->pinned, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
+    *r = *ctx->pinned;
     return GMM_OK;
 }
 
@@ -824,8 +839,7 @@ int report_status(gmm_ctx* ctx, int status) {
 // Synchronising read of the log-likelihood slot and the status word.
 int read_result(gmm_ctx* ctx, int slot, double* loglik) {
     DevResult r;
-    CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
+    CHECK(read_back(ctx, &r));
     CHECK(report_status(ctx, r.status));
     ctx->tc_n_ill = r.n_ill;
     ctx->scr_active = 0;
@@ -865,11 +879,11 @@ int64_t screen_piece(const gmm_ctx* ctx, int64_t n) {
     return pieces <= 1 ? most : ((n + pieces - 1) / pieces + wave - 1) / wave * wave;
 }
 
-int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, const float* var, bool unit) {
+int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, const float* var, bool unit, bool clear = true) {
     const ScreenBuffers sb = ctx->screen();
     KL(launch_screen_prepare(ctx->stream, D, K, pi, mu, var, unit, sb, ctx->w2(), ctx->c2(), ctx->c2d(), &ctx->result()->status));
     ctx->launches += 2;
-    CU(cudaMemsetAsync(sb.ll, 0, (size_t)(SCR_LL + K) * 8, ctx->stream));
+    if (clear) CU(cudaMemsetAsync(sb.ll, 0, (size_t)(SCR_LL + K) * 8, ctx->stream));      // (else zero_stats does)
     return GMM_OK;
 }
 
@@ -920,8 +934,7 @@ void screen_note(gmm_ctx* ctx, bool dense) {
 
 int screen_result(gmm_ctx* ctx, int slot, double* loglik, bool* dense) {
     DevResult r;
-    CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
+    CHECK(read_back(ctx, &r));
     *dense = r.scr[SC_DENSE] != 0;
     screen_note(ctx, *dense);
     ctx->scr_active = 0;
@@ -1009,6 +1022,7 @@ int gmm_destroy(gmm_ctx* ctx) {
         if (ctx->ev_done[b]) cudaEventDestroy(ctx->ev_done[b]);
     }
     if (ctx->hparams) cudaFree(ctx->hparams);
+    if (ctx->pinned) cudaFreeHost(ctx->pinned);
     if (ctx->pl_scratch) cudaFree(ctx->pl_scratch);
     if (ctx->km_scratch) cudaFree(ctx->km_scratch);
     if (ctx->at_scratch) cudaFree(ctx->at_scratch);
@@ -1071,16 +1085,17 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
     if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
         bool dense = false;
-        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
-        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
+        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0, true));
         CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
         CHECK(screen_end(ctx, K, 0));
         CHECK(screen_result(ctx, 0, loglik, &dense));
         if (!dense) return GMM_OK;
     }
     CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
-    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
-    CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, 0));
+    const bool fresh = path == GMM_PATH_FP32 && fused_direct_supports(D, K);      // (writes the statistics, nothing to add to)
+    if (!fresh) CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+    CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, 0, fresh));
     ctx->last_path = path;
     return read_result(ctx, 0, loglik);
 }
@@ -1165,8 +1180,7 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
                 CHECK(prof_end(ctx));
             }
             DevResult r;
-            CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
-            CU(cudaStreamSynchronize(ctx->stream));
+            CHECK(read_back(ctx, &r));
             ctx->scr_active = 0;
             const int done = r.stop_at < end ? r.stop_at + 1 : end;
             for (; t < done; ++t) loglik_trace[t] = r.ll[t % LL_SLOTS];
@@ -1197,8 +1211,8 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         int rc = GMM_OK;
         bool dense = true;
         if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
-            CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
-            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
+            CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
+            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot, true));
             CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
             CHECK(screen_end(ctx, K, slot));
             CHECK(update(&ctx->result()->scr[SC_DENSE]));
@@ -1316,9 +1330,9 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
     bool screening = screen_try(ctx, SCREEN_STEPS, N, D, K);
-    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
     else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
-    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0, screening));
     int c = 0;                                       // chunks copied so far: they take the buffers in turn
     bool copied = true;                              // (the first one already is)
     for (int64_t off = 0; off < N; off += rows_per_chunk, ++c) {
@@ -1547,7 +1561,7 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
     const int* dense_if = nullptr;
     if (screening) {
         dense_if = run_fp32_if = ctx->result()->scr + SC_DENSE;
-        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
@@ -1720,7 +1734,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         double* Nk = ctx->stats();
         double* S1 = Nk + K;
         double* S2 = S1 + (size_t)K * D;
-        CHECK(screen_begin(ctx, D, K, nullptr, centroids, nullptr, true));
+        CHECK(screen_begin(ctx, D, K, nullptr, centroids, nullptr, true, false));
         // (the kernels below would decide a near tie in fp32 about a centre, or among log-densities of the unit mixture)
         ScreenTie tie{nullptr, (float)0.72134752044448170368,
                       (float)(1.4426950408889634074 * (std::log((double)(1.f / (float)K)) - 0.5 * D * std::log(6.283185307179586476925286766559)))};
@@ -1728,7 +1742,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
             KL(launch_center_fp32(ctx->stream, D, K, centroids, ctx->center()));
             tie = {ctx->center(), 1.f, 0.f};
         }
-        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0, true));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
@@ -1740,8 +1754,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         KL(launch_screen_centroids(ctx->stream, D, K, centroids, Nk, S1, sb, centroids_out, counts, ik));
         KL(launch_reduce_ll(ctx->stream, ik, K, &ctx->result()->ll[0], false));
         DevResult r;
-        CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
-        CU(cudaStreamSynchronize(ctx->stream));
+        CHECK(read_back(ctx, &r));
         screen_note(ctx, r.scr[SC_DENSE] != 0);
         if (r.scr[SC_DENSE] == 0) {
             if (inertia) *inertia = r.ll[0];
@@ -2102,8 +2115,7 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
     double total = 0.0;
     if (smallest == 0) {                        // no points at all: nothing was accumulated, only the parameters were checked
         DevResult r;
-        CU(cudaMemcpyAsync(&r, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
-        CU(cudaStreamSynchronize(ctx->stream));
+        CHECK(read_back(ctx, &r));
         CHECK(report_status(ctx, r.status));
         if (loglik) *loglik = 0.0;
         return GMM_OK;

@@ -550,10 +550,14 @@ int prof_end(gmm_ctx* ctx) {
 // path: the tensor-core path whenever the shape allows it (ill-conditioned components are handled inside its kernel).
 // Marked pairs per point up to which the screening mode is the cheaper way through a step on wide data (see the comment in
 // prepare_and_choose): against the two tensor sweeps, or (dense = true) against the FP32 kernels over all listed components.
-double wide_pair_limit(int n_list, int D, bool dense) {
+// (At small K D the sweeps stay where the sample of 8192 rows would be most of the call, and under forced GMM_PATH_TENSOR.)
+double wide_pair_limit(const gmm_ctx* ctx, int64_t N, int n_list, int D, bool dense) {
+    if (!dense && (ctx->path == GMM_PATH_TENSOR || N < 16384) && (double)n_list * D < 1.7e5) return 0.0;
+    // ns per point, from steps over 80K to 1M points at D 200-1000, K 65-4096: the screening 1.9 + 0.0045 D + 3.6e-6 K D (with nothing
+    // marked), a pair 0.4 + 0.0015 D, the two sweeps 1.8 + 0.0146 D + 2.4e-5 K D, the FP32 kernels 5e-4 K D
     const double kd = (double)n_list * D;
-    const double saved = (dense ? 5.0e-4 : 3.3e-5) * kd - 3.6e-6 * kd - 5.0;
-    return saved > 0.0 ? saved / (1.0 + 3.4e-3 * D) : 0.0;
+    const double saved = (dense ? 5.0e-4 * kd : 1.8 + 0.0146 * D + 2.4e-5 * kd) - (1.9 + 0.0045 * D + 3.6e-6 * kd);
+    return saved > 0.0 ? 0.8 * saved / (0.4 + 0.0015 * D) : 0.0;
 }
 
 int prepare_and_choose(gmm_ctx* ctx, int64_t N, int D, int K, const float* pi, const float* mu, const float* var,
@@ -608,7 +612,7 @@ int prepare_and_choose(gmm_ctx* ctx, int64_t N, int D, int K, const float* pi, c
                 int marks = 0;
                 CU(cudaMemcpyAsync(&marks, wb.ctl, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
                 CU(cudaStreamSynchronize(ctx->stream));
-                const double auto_limit = wide_pair_limit(n_list, D, few_points);
+                const double auto_limit = wide_pair_limit(ctx, N, n_list, D, few_points);
                 ok = (double)marks <= (ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit : auto_limit) * (double)np;
             }
             if (ok) {
@@ -717,7 +721,7 @@ int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, 
                     // more than one pair in 64 marked (or the pair-by-pair route switched off): the dense kernels are cheaper
                     // ("screen" mode: the dense alternative evaluates every component, so the pair route pays for longer)
                     const long long max_pairs = ctx->wide_sparse >= 2 ? ((long long)1 << 62)
-                                              : all ? (long long)((double)cnt * wide_pair_limit(n_ill, D, true)) : (long long)cnt * n_ill / 64;
+                                              : all ? (long long)((double)cnt * wide_pair_limit(ctx, n, n_ill, D, true)) : (long long)cnt * n_ill / 64;
                     KL(launch_cand_gate_wide(ctx->stream, wb, max_pairs));
                     KL(launch_cand_lse_wide(ctx->stream, Xs, cnt, D, n_ill, wb, ctx->logZ2()));
                 }
@@ -1440,7 +1444,9 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
             CU(cudaMemcpyAsync(fl, wb.flags, sizeof(fl), cudaMemcpyDeviceToHost, ctx->stream));
             CU(cudaStreamSynchronize(ctx->stream));
             const int n_list = fl[2], n_ill = fl[4], Kg = fl[6];
-            bool ok = n_list >= 1 && n_ill + 64 <= WIDE_MAX_ILL;
+            // (ranks that no marked pair fills come from the blocks of 32 components: with fewer than m of those the rows are left to the
+            // FP32 kernels)
+            bool ok = n_list >= 1 && n_ill + 64 <= WIDE_MAX_ILL && (argmax || (K + 31) / 32 >= m || ctx->wide_mode == 2);
             if (ok) {
                 KL(launch_ill_gather_wide(ctx->stream, D, n_list, wb, mu, ctx->w2(), ctx->c2d()));
                 const int ntop = argmax ? 2 : (m + 2 <= 6) ? 6 : WIDE_MAX_TOP;
@@ -1452,8 +1458,8 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
                     KL(launch_cand_filter_wide(ctx->stream, cnt, n_list, wb));
                     return GMM_OK;
                 };
-                // (a pair costs 2 ns, the route below 30-60 ns per point at config 5's shape)
-                const double per_point = ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit : 0.5 * wide_pair_limit(n_list, D, false);
+                // (the costs of a step stand for those of the assignment: without statistics here, without the second sweep there)
+                const double per_point = ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit : wide_pair_limit(ctx, N, n_list, D, false);
                 int32_t* unc_rows = nullptr;
                 int* unc_count = nullptr;
                 if (!argmax) {
@@ -1871,8 +1877,8 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
                 return GMM_OK;
             };
             const double kd = (double)n_list * D;
-            const double saved = (1.4e-4 - 3.6e-6) * kd - 5.0;
-            const double per_point = ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit : (saved > 0.0 ? saved / (0.5 + 1.8e-3 * D) : 0.0);
+            const double saved = (1.4e-4 - 3.6e-6) * kd - (1.9 + 0.0045 * D);
+            const double per_point = ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit : (saved > 0.0 ? saved / (0.3 + 1.0e-3 * D) : 0.0);
             if (ctx->wide_mode != 2) {
                 const int64_t np = N < 8192 ? N : 8192;
                 CHECK(screen_piece(X, np));

@@ -1458,8 +1458,13 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
                     KL(launch_cand_filter_wide(ctx->stream, cnt, n_list, wb));
                     return GMM_OK;
                 };
-                // (the costs of a step stand for those of the assignment: without statistics here, without the second sweep there)
-                const double per_point = ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit : wide_pair_limit(ctx, N, n_list, D, false);
+                // The costs of a step stand for those of a plain hard assignment.  Ranks without weight come from block maxima, whose order is
+                // wrong for up to a fifth of the indices at K = 122-309, and the counts of a k-means step follow near ties: both keep to
+                // shapes and marks where the screening agrees with the FP32 kernels (2e-5 of the indices at K = 2149, D = 799).
+                const double kd = (double)n_list * D;
+                const double sure_limit = fmax(0.0, 0.5 * ((3.3e-5 - 3.6e-6) * kd - 5.0) / (1.0 + 3.4e-3 * D));
+                const double per_point = ctx->wide_probe_limit > 0.0 ? ctx->wide_probe_limit
+                                       : (m >= 2 || screened) ? sure_limit : wide_pair_limit(ctx, N, n_list, D, false);
                 int32_t* unc_rows = nullptr;
                 int* unc_count = nullptr;
                 if (!argmax) {

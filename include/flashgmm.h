@@ -176,7 +176,8 @@ int gmm_assign_topm(gmm_ctx* ctx, const float* X, int64_t N, int D, int K,
  * responsibility; Section 4.3, multi-assignment: with at most two clusters, the top clusters whose responsibility
  * exceeds tau = 1/K).  The rule implemented: choice 0 of a vector is always taken; choices 1 .. max_lists-1 are taken
  * in order while resp > tau (strictly); a negative index ends a vector's list.
- *   idx [N x m] int32, resp [N x m] float32: device, as written by gmm_assign_topm (descending responsibility).
+ *   idx [N x m] int32, resp [N x m] float32: device, as written by gmm_assign_topm (descending responsibility).  A row that
+ *   names a cluster twice is listed there twice.
  *   tau: threshold; <= 0 selects the paper's 1/K.   max_lists: 1 (hard assignment) .. m (the paper uses 2).
  *   offsets [K + 1] int64, device out: list k holds items[offsets[k] .. offsets[k+1]).
  *   items  int32, device out, capacity >= N * max_lists entries: vector indices, ascending inside every list.

@@ -182,6 +182,40 @@ pl_fill_kernel(const int32_t* __restrict__ idx, const float* __restrict__ resp, 
         const int64_t i = base + lane;
         nxt.load(idx, resp, i + 32, i + 32 < p1, m, max_lists);
         const int c = cur.count(K, tau);
+        bool twice = false;
+#pragma unroll
+        for (int j = 1; j < ML; ++j)
+#pragma unroll
+            for (int q = 0; q < j; ++q) twice |= j < c && cur.k[q] == cur.k[j];
+        if (ML > 1 && __any_sync(0xffffffffu, twice)) {
+            // A row that names a cluster twice is listed there twice (the counts have it so): a bit per lane is not enough, so every
+            // entry counts the others of its list, one lane of the warp after the other.
+            int rank[ML], all[ML];
+#pragma unroll
+            for (int j = 0; j < ML; ++j) rank[j] = all[j] = 0;
+            for (int src = 0; src < 32; ++src) {
+#pragma unroll
+                for (int q = 0; q < ML; ++q) {
+                    const int32_t v = __shfl_sync(0xffffffffu, q < c ? cur.k[q] : -1, src);
+#pragma unroll
+                    for (int j = 0; j < ML; ++j)
+                        if (j < c && cur.k[j] == v) {
+                            ++all[j];
+                            if (src < lane || (src == lane && q < j)) ++rank[j];
+                        }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < ML; ++j)
+                if (j < c) items[__ldg(offsets + cur.k[j]) + cursor[cur.k[j]] + rank[j]] = (int32_t)i;
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < ML; ++j)
+                if (j < c && rank[j] == 0) cursor[cur.k[j]] += all[j];
+            __syncwarp();
+            cur = nxt;
+            continue;
+        }
         int64_t off[ML];
 #pragma unroll
         for (int j = 0; j < ML; ++j)

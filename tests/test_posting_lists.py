@@ -150,6 +150,23 @@ def test_gpu_builder_at_the_edges_of_its_ranges(N, K, m, max_lists):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("N,K,m,max_lists", [(5000, 7, 2, 2), (3001, 40, 4, 3), (2000, 3, 8, 8)])
+def test_gpu_builder_lists_a_vector_as_often_as_its_row_names_the_cluster(N, K, m, max_lists):
+    import torch
+    from paper_2606_10896_b200 import flashgmm as fg
+
+    rng = np.random.Generator(np.random.PCG64(N + K))
+    idx = rng.integers(0, K, (N, m)).astype(np.int32)      # repeated choices in many rows, next to rows without any
+    resp = np.sort(rng.random((N, m)).astype(np.float32), 1)[:, ::-1].copy()
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda:0")
+    with fg.Context(0) as ctx:
+        off_d, items_d, total, _ = ctx.gmm_build_posting_lists(t(idx), t(resp), K, 0.3, max_lists)
+    off_r, items_r, _ = posting_lists(idx, resp, K, 0.3, max_lists)
+    assert total == off_r[K] and off_d.cpu().numpy().tolist() == off_r.tolist()
+    assert items_d.cpu().numpy()[:total].tolist() == items_r.tolist()
+
+
+@pytest.mark.gpu
 def test_gpu_builder_rejects_bad_arguments():
     import torch
     from paper_2606_10896_b200 import flashgmm as fg

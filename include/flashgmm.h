@@ -199,7 +199,8 @@ int gmm_build_posting_lists(gmm_ctx* ctx, const int32_t* idx, const float* resp,
  *   centroids_out [K x D] fp32, device out (may be the same array as centroids).
  *   counts [K] int64, device out, may be NULL: points per centroid.
  *   inertia (host out, may be NULL): sum over the points of the squared distance to their (input) centroid.
- * Deterministic (no atomics).  Limits: N < 2^31, K <= 8192 (otherwise GMM_EUNSUPPORTED).  Synchronises the stream. */
+ * Deterministic (no atomics).  Limits: N < 2^31, K <= 8192 (otherwise GMM_EUNSUPPORTED).  GMM_ENUMERIC where a tensor path meets a
+ * non-finite value in X or the centroids.  Synchronises the stream. */
 int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const float* centroids,
                     int32_t* assign, int32_t* work, float* centroids_out, int64_t* counts, double* inertia);
 

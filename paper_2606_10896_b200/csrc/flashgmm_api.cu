@@ -1768,6 +1768,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         CHECK(read_back(ctx, &r));
         screen_note(ctx, r.scr[SC_DENSE] != 0);
         if (r.scr[SC_DENSE] == 0) {
+            CHECK(report_status(ctx, r.status));
             if (inertia) *inertia = r.ll[0];
             ctx->last_path = GMM_PATH_TENSOR;
             return GMM_OK;
@@ -1812,10 +1813,10 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     const int slot = 0;
     CU(cudaMemsetAsync(&ctx->result()->ll[slot], 0, 8, ctx->stream));
     KL(launch_reduce_ll(ctx->stream, km_inertia_k(ctx->km_scratch, D, K), K, &ctx->result()->ll[slot], false));
-    double v = 0.0;
-    CU(cudaMemcpyAsync(&v, &ctx->result()->ll[slot], sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
-    CU(cudaStreamSynchronize(ctx->stream));
-    if (inertia) *inertia = v;
+    DevResult r;
+    CHECK(read_back(ctx, &r));
+    CHECK(report_status(ctx, r.status));
+    if (inertia) *inertia = r.ll[slot];
     ctx->last_path = tensor ? GMM_PATH_TENSOR : GMM_PATH_FP32;
     return GMM_OK;
 }

@@ -105,3 +105,28 @@ def test_gpu_kmeans_step_matches_oracle(N, D, K):
     if moved == 0:
         np.testing.assert_allclose(new_d.cpu().numpy(), new_r, rtol=0, atol=1e-4 * scale)
     assert abs(inertia - inertia_r) <= 1e-5 * abs(inertia_r) + 1e-6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("D,screened", [(40, True), (40, False), (200, False)])
+@pytest.mark.parametrize("where", ["X", "centroids"])
+def test_gpu_step_reports_what_is_not_finite_itself(monkeypatch, D, screened, where):
+    # the call that meets a non-finite value fails, on every route, and leaves nothing behind for the next one
+    import torch
+    from paper_2606_10896_b200 import flashgmm as fg
+
+    if not screened:
+        monkeypatch.setenv("GMM_SCREEN_MARKS", "0")
+    X, centers, _ = _blobs(5, 3000, D, 100)
+    C = centers.astype(np.float32)
+    bad = (X if where == "X" else C).copy()
+    bad[17, 5] = np.nan
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda:0")
+    with fg.Context(0) as ctx:
+        with pytest.raises(fg.GmmError) as err:
+            ctx.gmm_kmeans_step(t(bad), t(C)) if where == "X" else ctx.gmm_kmeans_step(t(X), t(bad))
+        assert err.value.code == fg.GMM_ENUMERIC
+        a, _, _, _ = ctx.gmm_kmeans_step(t(X), t(C))
+        a_r, _, _, _, gap = kmeans_step(X, C)
+        assert np.all((a.cpu().numpy() == a_r) | (gap < 1e-3))
+        ctx.gmm_sync_status()

@@ -193,7 +193,9 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
         prm[k] = make_float4(on ? (float)c : -CUDART_INF_F, on ? (float)(al * 1.000001) : 0.f, on ? (float)(be * 1.000001) : 0.f, (float)numax);
         key[k] = !on ? CUDART_INF_F : capped ? SCR_CAPPED : (float)(al + be * D);
         if (on) atomicAdd(ctl + SC_ACTIVE, 1);
-        if (bad) atomicOr(status, bad);
+        // (k-means: the kernels of the dense path say what becomes of it, some report it and some do not)
+        if (bad && unit) ctl[SC_DENSE] = 1;
+        else if (bad) atomicOr(status, bad);
     }
 }
 
@@ -273,14 +275,15 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(int D, int K, int Kpa
 // ------------------------------------------------------------------------------------------------------------------
 // X -> fp16 plane of u, rows of `chunks` 16-byte chunks (8 dimensions each), and |u|^2.  Chunk c of row r sits at place
 // screen_place(c, r): the sweep reads a row per lane from shared memory, and eight neighbouring rows' chunks c then lie in
-// different banks.  L lanes per row, 8 dimensions each.  Bound by memory: 4 D bytes in, 2 D out.
+// different banks.  L lanes per row, 8 dimensions each.  Bound by memory: 4 D bytes in, 2 D out.  Data that are not finite are left to
+// the dense kernels: what becomes of them differs from entry point to entry point and from path to path.
 __host__ __device__ __forceinline__ int screen_chunks(int D) { return D <= 32 ? 4 : D <= 64 ? 8 : 16; }
 __device__ __forceinline__ int screen_place(int c, int row, int chunks) { return chunks == 4 ? c ^ ((row >> 1) & 3) : c ^ (row & 7); }
 
 template <int L>
 __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __restrict__ X, int64_t n, int D, int chunks, const float* __restrict__ sd,
                                                                const float* __restrict__ gd, unsigned char* __restrict__ y,
-                                                               float* __restrict__ n2, int* __restrict__ ctl, int* __restrict__ status) {
+                                                               float* __restrict__ n2, int* __restrict__ ctl) {
     if (blockIdx.x == 0 && threadIdx.x < 3) ctl[SC_MARKS + threadIdx.x] = 0;
     if (ctl[SC_DENSE] != 0) return;
     const bool vec_ok = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
         store(row, xa);
         store(row + step, xb);
     }
-    if (bad) atomicOr(status, ST_BAD_X);
+    if (bad) ctl[SC_DENSE] = 1;
 }
 
 // ------------------------------------------------------------------------------------------------------------------
@@ -1813,7 +1816,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
         const int rpb = 256 / L;
         blocks = (n + 2 * rpb - 1) / (2 * rpb);
         if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-#define FG_TR(L_) screen_transform_kernel<L_><<<(unsigned)blocks, 256, 0, s>>>(X, n, D, screen_chunks(D), b.sd, b.gd, b.y, b.n2, b.ctl, status)
+#define FG_TR(L_) screen_transform_kernel<L_><<<(unsigned)blocks, 256, 0, s>>>(X, n, D, screen_chunks(D), b.sd, b.gd, b.y, b.n2, b.ctl)
         switch (L) {
             case 1: FG_TR(1); break;
             case 2: FG_TR(2); break;

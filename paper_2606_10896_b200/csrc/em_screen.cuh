@@ -27,7 +27,7 @@ constexpr int SCR_GROUP = 32768;             // points of a group that launch_sc
 constexpr int SCR_SPILL = 22, SCR_MAX_SMS = 160;      // see screen_sweep_kernel
 
 // Control words (in the context's result block, so that they travel to the host with the log-likelihood).
-enum { SC_DENSE = 0,      // set when a piece marks too many pairs: later kernels return at once, the caller takes the dense path
+enum { SC_DENSE = 0,      // set when a piece marks too many pairs or is not finite: later kernels return at once, the caller takes the dense path
        SC_MARKS,          // pairs marked in the current piece
        SC_OVF,            // rows of the current piece that left the sweep without a list
        SC_EXTRA,          // pairs of those rows
@@ -71,7 +71,7 @@ inline int screen_atoms(int D) { return (D + 31) / 32; }
 __host__ __device__ inline size_t screen_group_bytes(int D) { return 4096 + (size_t)((D + 31) / 32) * 16384; }
 
 // Parameters -> w2, c2, c2d (as launch_prepare_fp32, with the same checks), coefficient plane and tables.  unit: k-means (mu =
-// centroids; pi, var not read; log2 z = -|x - mu|^2).  Clears SC_DENSE.
+// centroids; pi, var not read; log2 z = -|x - mu|^2; one that is not finite sets SC_DENSE and no status).  Clears SC_DENSE.
 cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
                                   const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
 // One piece of n <= SCR_PIECE points: plane, sweep, rows without a list.  margin: log2 units below a point's best value down to

@@ -120,6 +120,25 @@ def test_screen_reports_non_finite_data(fg):
         c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
 
 
+def test_screen_leaves_non_finite_data_to_the_fp32_kernels(fg, monkeypatch):
+    """K < 64: the assignment and the k-means step take such data as the FP32 kernels do, with or without the screening sweep in front."""
+    X, pi, mu, var = _mixture(3000, 40, 48, 4)
+    bad, cen = X.copy(), mu.copy()
+    bad[1234, 5], bad[2000] = np.nan, np.inf
+    cen[7, 3] = np.nan
+    got = []
+    for marks in ("1000", "0"):
+        monkeypatch.setenv("GMM_SCREEN_MARKS", marks)
+        with fg.Context(0) as c:
+            idx, resp = c.gmm_assign_topm(_t(bad), _t(pi), _t(mu), _t(var), 1)
+            c.gmm_sync_status()
+            a, new, counts, inertia = c.gmm_kmeans_step(_t(bad), _t(mu))
+            b, newer, _, _ = c.gmm_kmeans_step(_t(X), _t(cen))
+            got.append([v.cpu().numpy() for v in (idx, resp, a, new, counts, b, newer)] + [inertia])
+    for u, v in zip(*got):
+        assert np.array_equal(u, v, equal_nan=True)
+
+
 def test_config2_free_running_through_the_screening_path(fg):
     spec = synth.CONFIGS[2].with_n(20_000)
     X = synth.sample_host(spec)

@@ -612,10 +612,12 @@ cudaError_t launch_chained(cudaStream_t s, dim3 grid, int threads, size_t smem, 
     cfg.attrs = &at; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
+constexpr int MOST_SMEM = 114688;          // (no shape asks for more than 110592 bytes, see direct_plan)
 template <int MODE, int PT, int TK>
 cudaError_t direct_launch(cudaStream_t s, dim3 grid, const DirectPlan& pl) {
     if (pl.smem > 40960) {
-        cudaError_t e = cudaFuncSetAttribute(direct_kernel<MODE, PT, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+        // (the same limit from every call: it belongs to the kernel, which contexts on other threads launch for other shapes)
+        cudaError_t e = cudaFuncSetAttribute(direct_kernel<MODE, PT, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST_SMEM);
         if (e != cudaSuccess) return e;
     }
     return launch_chained(s, grid, NT, pl.smem, direct_kernel<MODE, PT, TK>, pl.a);

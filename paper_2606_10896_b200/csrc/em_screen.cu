@@ -1844,7 +1844,8 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
     sweep<<<(unsigned)(tiles < sms ? tiles : sms), SW_THREADS, SW_SMEM, s>>>(p);
     LCHECK();
     const size_t smem = (size_t)OV_ROWS * K * 4;
-    e = cudaFuncSetAttribute(screen_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (here and below the same limit from every call: it belongs to the kernel, which contexts on other threads launch for other K)
+    e = cudaFuncSetAttribute(screen_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, OV_ROWS * SCR_MAX_K * 4);
     if (e != cudaSuccess) return e;
     const double most = fmin((double)max_marks * (double)n, (double)SCR_PIECE * (stats ? SCR_MARKS : SCR_SLOTS));
     screen_rows_kernel<<<(unsigned)(2 * sms), 256, smem, s>>>(X, n, D, K, margin, top, (long long)most, mu, w2, c2d, b.ovf,
@@ -1893,7 +1894,7 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     LCHECK();
     const int K2 = (K + 1) & ~1;
     const size_t smem = (size_t)K2 * 4 + (size_t)K2 * 16;
-    cudaError_t e = cudaFuncSetAttribute(screen_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(screen_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 20);
     if (e != cudaSuccess) return e;
     screen_fill_kernel<<<blocks, 256, smem, s>>>(n, K, range, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.off, b.srt, b.ctl);
     LCHECK();
@@ -1911,10 +1912,11 @@ cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int
                                  const float* pi, const float* mu, const float* var, const float* w2, const double* c2d,
                                  const ScreenBuffers& b, float* fv, int64_t* launches) {
     const int K2 = (K + 1) & ~1;
-    int warps = 32;                                          // cursors of 2 bytes per warp and component: at most 128 KB
-    while (warps > 8 && (size_t)K2 * warps * 2 > 131072) warps >>= 1;
+    constexpr int GROUP_CURSORS = 131072;                    // cursors of 2 bytes per warp and component: at most 128 KB
+    int warps = 32;
+    while (warps > 8 && (size_t)K2 * warps * 2 > GROUP_CURSORS) warps >>= 1;
     const size_t smem = (size_t)K2 * 4 + (size_t)K2 * warps * 2;
-    cudaError_t e = cudaFuncSetAttribute(screen_group_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(screen_group_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4 + GROUP_CURSORS);
     if (e != cudaSuccess) return e;
     screen_group_sort_kernel<<<groups, warps * 32, smem, s>>>(K, g_start, g_len, b.pt_off, b.pt_cnt, b.ids, b.val, g_off, b.srt, b.ctl);
     LCHECK();

@@ -267,16 +267,19 @@ cudaError_t launch_posting_lists(cudaStream_t s, const int32_t* idx, const float
     int32_t* counts = static_cast<int32_t*>(scratch);
     int32_t* totals = counts + (size_t)PL_MAX_BLOCKS * K;
     const size_t smem = (size_t)K * sizeof(int32_t);
+    constexpr size_t FILL_CURSORS = 100 * 1024, FILL_MOST = 3 * (size_t)PL_MAX_K * 8;
+    static_assert(FILL_MOST >= FILL_CURSORS, "shared memory of the fill");
     // 8 bytes per warp and cluster: eight warps up to K = 1024 (three CTAs per SM), fewer beyond, down to three at K = 8192
     int warps = PL_THREADS / 32;
-    while (warps > 3 && (size_t)warps * K * 8 > (size_t)100 * 1024) --warps;
+    while (warps > 3 && (size_t)warps * K * 8 > FILL_CURSORS) --warps;
     const size_t smem_fill = (size_t)warps * K * 8;
     // (two choices per vector, the paper's rule, read as 8-byte rows where the arrays allow it)
     const bool pairs = m == 2 && max_lists == 2 && (reinterpret_cast<uintptr_t>(idx) & 7) == 0 && (reinterpret_cast<uintptr_t>(resp) & 7) == 0;
     auto fill = max_lists == 1 ? pl_fill_kernel<1> : pairs ? pl_fill_kernel<2> : pl_fill_kernel<PL_MAX_LISTS>;
-    cudaError_t e = cudaFuncSetAttribute(pl_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the same limits from every call: they belong to the kernels, which contexts on other threads launch for other K)
+    cudaError_t e = cudaFuncSetAttribute(pl_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PL_MAX_K * (int)sizeof(int32_t));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fill);
+    e = cudaFuncSetAttribute(fill, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FILL_MOST);
     if (e != cudaSuccess) return e;
     pl_count_kernel<<<blocks, PL_THREADS, smem, s>>>(idx, resp, n, m, K, tau, max_lists, range, counts);
     pl_scan_kernel<<<(K + 31) / 32, 1024, 0, s>>>(counts, blocks, K, totals);

@@ -392,6 +392,7 @@ struct SweepParams {
     int* ovf;
     int* ctl;
     int* status;
+    int test_silent;                // >= 0: that CTA keeps back the news of its first products (time-out test)
     int tile_limit, tile_over;      // marks, and points without a list, in a CTA's first tile above which the data counts as dense at once
 };
 
@@ -804,7 +805,7 @@ screen_sweep_kernel(const SweepParams p) {
                         mma_commit(bars0 + 8 * (SB_PEMPTY + slot));
                         if (++slot == SW_PS) { slot = 0; parity ^= 1u; }
                     }
-                    if (alive) mma_commit(bars0 + 8 * (SB_LFULL + h));
+                    if (alive && !(p.test_silent == (int)blockIdx.x && gi == 0)) mma_commit(bars0 + 8 * (SB_LFULL + h));
                     if (++cslot == (uint32_t)cslots) cslot = 0;
                 }
             }
@@ -816,6 +817,9 @@ screen_sweep_kernel(const SweepParams p) {
     }
     fence_before();
     __syncthreads();
+    // A CTA that left early has not written its points' lists, and what was in that memory before must not be taken for offsets and
+    // components: nothing after this kernel does anything, also when a wait ran out.
+    if (tid == 0 && (abort_s != 0 || drain_s != 0)) p.ctl[SC_DENSE] = 1;
     if (warp == SW_MMA) {
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
@@ -1832,7 +1836,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
     p.n = n; p.KA = KA; p.KS = KS; p.NG = Kpad / 128; p.margin = margin;
     p.chunks = screen_chunks(D); p.y = b.y; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
     p.blk = b.blk; p.n2 = b.n2; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
-    p.ovf = b.ovf; p.ctl = b.ctl; p.status = status;
+    p.ovf = b.ovf; p.ctl = b.ctl; p.status = status; p.test_silent = b.test_silent;
     p.tile_limit = (int)fmin(1.1 * (double)max_marks * SCR_TILE, 1e9);
     p.tile_over = n >= 65536 ? SCR_TILE / 32 : SCR_TILE;      // (the share of rows that screen_rows_kernel takes)
     if (top < 1 || top > 4) return cudaErrorInvalidValue;

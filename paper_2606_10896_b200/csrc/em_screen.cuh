@@ -27,7 +27,7 @@ constexpr int SCR_GROUP = 32768;             // points of a group that launch_sc
 constexpr int SCR_SPILL = 22, SCR_MAX_SMS = 160;      // see screen_sweep_kernel
 
 // Control words (in the context's result block, so that they travel to the host with the log-likelihood).
-enum { SC_DENSE = 0,      // set when a piece marks too many pairs or is not finite: later kernels return at once, the caller takes the dense path
+enum { SC_DENSE = 0,      // set when a piece marks too many pairs or is not finite, or a wait ran out: later kernels return at once, the caller takes the dense path
        SC_MARKS,          // pairs marked in the current piece
        SC_OVF,            // rows of the current piece that left the sweep without a list
        SC_EXTRA,          // pairs of those rows
@@ -63,6 +63,7 @@ struct ScreenBuffers {
     double* ll;           // [SCR_LL + K]
     int* ovf;             // [SCR_PIECE]
     int* ctl;             // [SC_WORDS]
+    int test_silent;      // (time-out test, see SweepParams)
 };
 
 bool screen_supports(int D, int K);

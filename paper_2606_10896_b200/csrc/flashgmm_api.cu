@@ -251,6 +251,7 @@ struct gmm_ctx {
     // (1, 2, 4 .. 16: mixtures of a fit sharpen as it goes on); see screen_try.
     struct ScreenHistory { int D = 0, K = 0, skip = 0, left = 0; } scr_history[3];
     int scr_kind = 0;
+    int scr_test_silent = -1;        // GMM_SCREEN_TEST_SILENT (time-out test)
     DevResult* pinned = nullptr;     // where the result block is read back to
     int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
     int sticky_status = 0;           // status bits read off the device but not yet reported (see ensure_scratch)
@@ -335,6 +336,7 @@ struct gmm_ctx {
         b.ll = reinterpret_cast<double*>(at(lay.s_ll));
         b.ovf = reinterpret_cast<int*>(at(lay.s_ovf));
         b.ctl = result()->scr;
+        b.test_silent = scr_test_silent;
         return b;
     }
     WideBuffers wide() const {
@@ -920,8 +922,7 @@ int screen_end(gmm_ctx* ctx, int K, int slot) {
     return GMM_OK;
 }
 
-// Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels (nothing is
-// reported then: they find what is wrong again).
+// Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels.
 bool screen_try(gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     if (!screen_wanted(ctx, kind, N, D, K, groups)) return false;
     auto& h = ctx->scr_history[kind];
@@ -942,8 +943,8 @@ int screen_result(gmm_ctx* ctx, int slot, double* loglik, bool* dense) {
     *dense = r.scr[SC_DENSE] != 0;
     screen_note(ctx, *dense);
     ctx->scr_active = 0;
-    if (*dense) return GMM_OK;
     CHECK(report_status(ctx, r.status));
+    if (*dense) return GMM_OK;
     ctx->scr_active = r.scr[SC_ACTIVE];
     ctx->last_path = GMM_PATH_TENSOR;
     *loglik = r.ll[slot];
@@ -981,6 +982,7 @@ int gmm_create(gmm_ctx** out, int device, void* cuda_stream) {
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
     if (const char* e = std::getenv("GMM_TC_COND_LIMIT")) ctx->tc_cond_limit = (float)std::atof(e);
     if (const char* e = std::getenv("GMM_SCREEN_MARKS")) ctx->scr_marks = std::atof(e);
+    if (const char* e = std::getenv("GMM_SCREEN_TEST_SILENT")) ctx->scr_test_silent = std::atoi(e);
     if (const char* e = std::getenv("GMM_SCREEN_PIECE")) {
         const long long v = std::atoll(e);
         if (v >= SCR_TILE && v <= SCR_PIECE) ctx->scr_piece = v / SCR_TILE * SCR_TILE;
@@ -1767,8 +1769,8 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         DevResult r;
         CHECK(read_back(ctx, &r));
         screen_note(ctx, r.scr[SC_DENSE] != 0);
+        CHECK(report_status(ctx, r.status));
         if (r.scr[SC_DENSE] == 0) {
-            CHECK(report_status(ctx, r.status));
             if (inertia) *inertia = r.ll[0];
             ctx->last_path = GMM_PATH_TENSOR;
             return GMM_OK;

@@ -120,6 +120,26 @@ def test_screen_reports_non_finite_data(fg):
         c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
 
 
+def test_screen_wait_that_runs_out(fg, monkeypatch):
+    """One CTA of the sweep keeps back the arrival that its other warps wait for.  Their waits run out (2 s), the kernel ends by itself,
+    nothing reads the lists that it has not written, and the call - the next synchronising one after an assignment - says so."""
+    X, pi, mu, var = _mixture(3000, 40, 200, 8)
+    ref = orc.em_step(X, pi, mu, var)
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    monkeypatch.setenv("GMM_SCREEN_TEST_SILENT", "2")
+    with fg.Context(0) as c:
+        for call in (lambda: c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var)), lambda: c.gmm_kmeans_step(_t(X), _t(mu)),
+                     lambda: (c.gmm_assign_topm(_t(X), _t(pi), _t(mu), _t(var), 2), c.gmm_sync_status())):
+            with pytest.raises(fg.GmmError) as e:
+                call()
+            assert e.value.code == fg.GMM_ETIMEOUT
+        c.gmm_sync_status()
+    monkeypatch.delenv("GMM_SCREEN_TEST_SILENT")
+    with fg.Context(0) as c:
+        got = c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))
+        assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3])
+
+
 def test_screen_leaves_non_finite_data_to_the_fp32_kernels(fg, monkeypatch):
     """K < 64: the assignment and the k-means step take such data as the FP32 kernels do, with or without the screening sweep in front."""
     X, pi, mu, var = _mixture(3000, 40, 48, 4)

@@ -13,8 +13,8 @@
 //                         X against the component's mean in registers, fp32 within 64 pairs, float64 beyond.
 //
 // Every value that reaches a result comes from exact fp32 evaluations; a term below 2^-40 of a point's total is dropped.  Data
-// whose posteriors are broad is noticed by the first sweep (SC_DENSE): the kernels that follow return at once and the caller
-// runs the dense kernels instead.
+// whose posteriors are broad is noticed ahead of the sweep, from a sample of the rows (screen_probe), or at the latest behind the sweep of a
+// piece (SC_DENSE): the kernels that follow return at once and the caller runs the dense kernels instead.
 #include "em_screen.cuh"
 #include "internal.cuh"
 
@@ -113,6 +113,7 @@ __global__ void __launch_bounds__(512) screen_dim_kernel(int D, int K, const flo
     gd[d] = gf;
     if (d == 0) {
         ctl[SC_TICKET_A] = 0;
+        ctl[SC_PROBED] = 0;
         ctl[SC_DENSE] = 0;
         ctl[SC_ACTIVE] = 0;
         ctl[SC_KEPT] = 0;
@@ -135,9 +136,12 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
                                                           const float* __restrict__ var, int unit, const float* __restrict__ sd,
                                                           const float* __restrict__ gd, float* __restrict__ w2, float* __restrict__ c2,
                                                           double* __restrict__ c2d, float4* __restrict__ prm, float* __restrict__ key,
-                                                          int4* __restrict__ blk, int* __restrict__ ctl, int* __restrict__ status) {
+                                                          int4* __restrict__ blk, unsigned* __restrict__ probe, double* __restrict__ ll, int* __restrict__ ctl,
+                                                          int* __restrict__ status) {
     const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (blockIdx.x == 0 && threadIdx.x < SCR_MAX_K / 32) blk[threadIdx.x] = make_int4(0, 0, 0, 0);      // (largest allowances, see below)
+    if (blockIdx.x == 0 && threadIdx.x < PR_GROUPS * (PR_ROWS + 1)) probe[threadIdx.x] = 0u;
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < SCR_LL + K; i += gridDim.x * 256) ll[i] = 0.0;
     if (k >= K) return;
     double slog = 0.0, bv[4], nv[4];
     int bad = 0;
@@ -199,19 +203,161 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
     }
 }
 
+// Whether the screening pays, ahead of the sweep: the exact log-densities of 16 groups of four consecutive rows, spread evenly over
+// the call's data so that neither the order of the rows nor one odd region of them decides, and from those how many pairs the sweep
+// would mark with its allowances.  Dense are data with more pairs than pay on average, and data of which a 16th or so lies
+// together in a region where the pairs of 32 neighbours outgrow their room: those rows would leave the sweep without a list.
+// Sixteen CTAs share a group, a 16th of the components each; the last of them to finish counts.  They run beside the CTAs of
+// screen_plane_kernel, which take 3 us longer for it.  (Beside the transform of the first piece they cost as much, and broad data its
+// time.)  Before, one tile of 256 points above the limit among the first 148 made the whole call dense: 200K x 32, K = 64 with an
+// overlapping region at its end took 475 us, of which 180 were the sweep for nothing, now 300 + 55; with the region at its start too.
+__device__ __forceinline__ unsigned order_up(float v) { const unsigned b = __float_as_uint(v); return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u); }
+__device__ __forceinline__ float order_down(unsigned o) { return __uint_as_float(o ^ ((o >> 31) ? 0x80000000u : 0xffffffffu)); }
+struct ProbeArgs {
+    ScreenProbe p;
+    int K;
+    const float *mu, *w2;
+    const double* c2d;
+    const float4* prm;
+    const float* key;
+    unsigned* probe;
+    int first;               // the first of the probe's CTAs
+    float2* bounds;          // [PR_GROUPS * PR_ROWS][K] (a component without a weight: -inf, one without a lower bound: -inf, upper)
+    int* ctl;
+};
+__device__ void screen_probe(const ProbeArgs& a, int D, const float* __restrict__ sd, const float* __restrict__ gd) {
+    __shared__ __align__(16) float x_s[PR_ROWS][128];
+    __shared__ float nrm_s[PR_ROWS];
+    __shared__ int last_s, crowd_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l8 = lane & 7, sub = lane >> 3, K = a.K;
+    const int b = (int)blockIdx.x - a.first, grp = b / PR_CTAS, share = (K + PR_CTAS - 1) / PR_CTAS, k0 = min(K, (b % PR_CTAS) * share), k1 = min(K, k0 + share);
+    if (tid == 0) crowd_s = 0;
+    unsigned* const lower = a.probe + grp * (PR_ROWS + 1);
+    float2* const bounds = a.bounds + (size_t)grp * PR_ROWS * K;
+    for (int e = tid; e < PR_ROWS * 128; e += 256) {
+        const int r = e >> 7, d = e & 127;
+        const int64_t row = (int64_t)(((double)grp + 0.5) / PR_GROUPS * (double)a.p.n) + r;
+        x_s[r][d] = d < D ? __ldg(a.p.X + (row < a.p.n ? row : a.p.n - 1) * D + d) : 0.f;
+    }
+    __syncthreads();
+    if (warp < PR_ROWS) {                            // warp = row
+        float q = 0.f;
+        for (int d = lane; d < D; d += 32) { const float u = (x_s[warp][d] - __ldg(gd + d)) * __ldg(sd + d); q = fmaf(u, u, q); }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+        if (lane == 0) nrm_s[warp] = q;
+    }
+    __syncthreads();
+    // eight lanes per component; lane l8 < PR_ROWS then holds its value for row l8
+    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(a.mu) & 15) == 0);      // (w2: scratch, aligned)
+    const float nrm = nrm_s[l8 % PR_ROWS];
+    float low = -CUDART_INF_F;
+    for (int kb = k0 + warp * 4; kb < k1; kb += 32) {
+        const int k = min(kb + sub, k1 - 1);
+        const float *m = a.mu + (size_t)k * D, *w = a.w2 + (size_t)k * D;
+        const float4 e = __ldg(a.prm + k);
+        const float c = (float)__ldg(a.c2d + k), key = __ldg(a.key + k);
+        float q[PR_ROWS];
+#pragma unroll
+        for (int r = 0; r < PR_ROWS; ++r) q[r] = 0.f;
+        if (vec) {
+            float4 mv[4], wv[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int d = 4 * (l8 + 8 * i);
+                mv[i] = wv[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (d < D) { mv[i] = __ldg(reinterpret_cast<const float4*>(m + d)); wv[i] = __ldg(reinterpret_cast<const float4*>(w + d)); }
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int r = 0; r < PR_ROWS; ++r) {
+                    const float4 x = *reinterpret_cast<const float4*>(&x_s[r][4 * (l8 + 8 * i)]);
+                    const float t0 = x.x - mv[i].x, t1 = x.y - mv[i].y, t2 = x.z - mv[i].z, t3 = x.w - mv[i].w;
+                    q[r] = fmaf(wv[i].x * t0, t0, q[r]); q[r] = fmaf(wv[i].y * t1, t1, q[r]);
+                    q[r] = fmaf(wv[i].z * t2, t2, q[r]); q[r] = fmaf(wv[i].w * t3, t3, q[r]);
+                }
+        } else {
+            for (int d = l8; d < D; d += 8) {
+                const float mv = __ldg(m + d), wv = __ldg(w + d);
+#pragma unroll
+                for (int r = 0; r < PR_ROWS; ++r) { const float t = x_s[r][d] - mv; q[r] = fmaf(wv * t, t, q[r]); }
+            }
+        }
+        float mine = 0.f;
+#pragma unroll
+        for (int r = 0; r < PR_ROWS; ++r) {
+            q[r] += __shfl_xor_sync(0xffffffffu, q[r], 1);
+            q[r] += __shfl_xor_sync(0xffffffffu, q[r], 2);
+            q[r] += __shfl_xor_sync(0xffffffffu, q[r], 4);
+            if (l8 == r) mine = q[r];
+        }
+        if (kb + sub < k1 && l8 < PR_ROWS) {
+            const float l = c - mine, E = fmaf(e.z, nrm, e.y);
+            const bool on = e.x > -CUDART_INF_F;
+            const float2 at = make_float2(on && key < SCR_CAPPED ? l - E : -CUDART_INF_F, on ? l + E : -CUDART_INF_F);
+            bounds[(size_t)l8 * K + k] = at;
+            low = fmaxf(low, at.x);
+        }
+    }
+    low = fmaxf(low, __shfl_xor_sync(0xffffffffu, low, 8));
+    low = fmaxf(low, __shfl_xor_sync(0xffffffffu, low, 16));
+    if (sub == 0 && l8 < PR_ROWS) atomicMax(lower + l8, order_up(low));
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last_s = atomicAdd(lower + PR_ROWS, 1u) == PR_CTAS - 1;
+    __syncthreads();
+    if (!last_s || warp >= PR_ROWS) return;
+    __threadfence();
+    const float2* mine = bounds + (size_t)warp * K;                          // warp = row
+    float cut = order_down(__ldcg(lower + warp)) - a.p.margin;
+    if (a.p.top > 1) {                                 // the sweep's bound for the `top` largest: the largest lower bounds of eights of components
+        float best[4] = {-CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F, -CUDART_INF_F};
+#pragma unroll 4
+        for (int k0 = lane * 8; k0 < K; k0 += 256) {
+            float x = -CUDART_INF_F;
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if (k0 + j < K) x = fmaxf(x, __ldcg(mine + k0 + j).x);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) { const float keep = fmaxf(best[j], x); x = fminf(best[j], x); best[j] = keep; }
+        }
+        float m = 0.f;
+        for (int r = 0; r < a.p.top; ++r) {
+            m = best[0];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (lane == __ffs(__ballot_sync(0xffffffffu, best[0] == m)) - 1) { best[0] = best[1]; best[1] = best[2]; best[2] = best[3]; best[3] = -CUDART_INF_F; }
+        }
+        cut = fminf(cut, m);
+    }
+    cut = fmaxf(cut, 0.5f * SCR_NEVER);
+    int cnt = 0;
+#pragma unroll 16
+    for (int k = lane; k < K; k += 32) cnt += __ldcg(mine + k).y >= cut ? 1 : 0;
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    // (a quarter more than the sweep's limit: a sample.  The sums only grow, so whoever takes one across its limit says so.)
+    if (lane == 0 && ((float)(atomicAdd(a.ctl + SC_PROBED, cnt) + cnt) > 1.25f * a.p.max_marks * (PR_GROUPS * PR_ROWS) ||
+                      (atomicAdd(&crowd_s, cnt) + cnt > SCR_SLOTS * PR_ROWS && a.p.max_marks <= SCR_SLOTS)))
+        a.ctl[SC_DENSE] = 1;
+}
+
 constexpr int SW_CSLOT = 4096;               // a group's constants: 128 rows of 16 halves
 // Positions of the components in the sweep: ascending by the allowance of a typical point, so that 32 neighbours, which are
 // screened with the largest allowance among them, have similar ones (the capped components come last).  A warp per component:
 // its rank among the keys is its position, and it writes its own row (a sort of the keys in every CTA took 20 us).  The
 // coefficients are written as the sweep has them in shared memory (screen_group_bytes per group of 128 positions: the constants,
 // then the atoms of 32 dimensions, swizzled), so that a stage is one contiguous copy.
-__global__ void __launch_bounds__(256) screen_plane_kernel(int D, int K, int Kpad, const float* __restrict__ mu,
+__global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe, int D, int K, int Kpad, const float* __restrict__ mu,
                                                            const float* __restrict__ w2, const float* __restrict__ sd,
                                                            const float* __restrict__ gd, const float4* __restrict__ prm,
                                                            const float* __restrict__ key, unsigned char* __restrict__ img,
                                                            int4* __restrict__ blk, int* __restrict__ comp_of) {
+    if ((int)blockIdx.x >= probe.first) {
+        screen_probe(probe, D, sd, gd);
+        return;
+    }
     const int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (k >= Kpad) return;
     int pos = k;
     bool on = false, capped = false;
     float4 q = make_float4(-CUDART_INF_F, 0.f, 0.f, 0.f);
@@ -393,7 +539,6 @@ struct SweepParams {
     int* ctl;
     int* status;
     int test_silent;                // >= 0: that CTA keeps back the news of its first products (time-out test)
-    int tile_limit, tile_over;      // marks, and points without a list, in a CTA's first tile above which the data counts as dense at once
 };
 
 static_assert(SW_ENT + SW_SPILL <= 32, "a mask of a point's entries");
@@ -422,7 +567,7 @@ screen_sweep_kernel(const SweepParams p) {
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s, drain_s, first_marks, first_warps;
+    __shared__ int abort_s, drain_s;
     if (p.ctl[SC_DENSE] != 0) return;
     volatile int* abort_flag = &abort_s;
     volatile int* drain_flag = &drain_s;
@@ -437,7 +582,6 @@ screen_sweep_kernel(const SweepParams p) {
     if (tid == 0) {
         abort_s = 0;
         drain_s = 0;
-        first_marks = first_warps = 0;
         for (int i = 0; i < SB_COUNT; ++i) {
             const bool wg = (i >= SB_AFULL && i < SB_AFULL + 2) || (i >= SB_LEMPTY && i < SB_LEMPTY + 2);
             const bool both = i >= SB_PEMPTY && i < SB_PEMPTY + SW_PS;           // (released by the MMA warps of both halves)
@@ -682,24 +826,6 @@ screen_sweep_kernel(const SweepParams p) {
                         }
                 }
             }
-            if (i == 0) {
-                // Broad posteriors show at once: more marks than allowed (and a tenth) in a CTA's first tile, and the sweep ends (the whole
-                // of it, for nothing, cost data of few dimensions a fifth of the step).  The data alone decide, not the timing.
-                const int mine = __reduce_add_sync(0xffffffffu, !in ? 0 : over ? 1 << 20 : cnt);      // (a warp marks at most 512)
-                if (lane == 0) {
-                    atomicAdd(&first_marks, mine);
-                    __threadfence_block();
-                    if (atomicAdd(&first_warps, 1) == 7) {
-                        const int all = atomicAdd(&first_marks, 0), rows = all >> 20;
-                        if ((all & 0xfffff) + 64 * rows > p.tile_limit || rows > p.tile_over) {
-                            p.ctl[SC_DENSE] = 1;
-                            *abort_flag = 1;
-                        }
-                    }
-                }
-                __syncwarp();
-                if (*abort_flag) break;
-            }
         }
         if (ntl > 0 && !*abort_flag) {
             marks = __reduce_add_sync(0xffffffffu, marks);
@@ -819,7 +945,7 @@ screen_sweep_kernel(const SweepParams p) {
     __syncthreads();
     // A CTA that left early has not written its points' lists, and what was in that memory before must not be taken for offsets and
     // components: nothing after this kernel does anything, also when a wait ran out.
-    if (tid == 0 && (abort_s != 0 || drain_s != 0)) p.ctl[SC_DENSE] = 1;
+    if (threadIdx.x == 0 && (abort_s != 0 || drain_s != 0)) p.ctl[SC_DENSE] = 1;
     if (warp == SW_MMA) {
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
@@ -1797,14 +1923,16 @@ static int screen_range(int64_t n) { return n <= 65536 ? 128 : n <= 131072 ? 256
 bool screen_supports(int D, int K) { return D >= 1 && D <= 128 && K >= 1 && K <= SCR_MAX_K; }
 
 cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
-                                  const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status) {
+                                  const ScreenProbe& probe, const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status) {
     const int Kpad = screen_kpad(K);
     const int db = (K + 7) / 8 < SCR_DIM_BLOCKS ? (K + 7) / 8 : SCR_DIM_BLOCKS;
     screen_dim_kernel<<<db, 512, 0, s>>>(D, K, pi, mu, var, unit ? 1 : 0, b.dimpart, b.sd, b.gd, b.ctl);
     LCHECK();
-    screen_comp_kernel<<<(K + 7) / 8, 256, 0, s>>>(D, K, pi, mu, var, unit ? 1 : 0, b.sd, b.gd, w2, c2, c2d, b.prm, b.key, b.blk, b.ctl, status);
+    screen_comp_kernel<<<(K + 7) / 8, 256, 0, s>>>(D, K, pi, mu, var, unit ? 1 : 0, b.sd, b.gd, w2, c2, c2d, b.prm, b.key, b.blk, b.probe, b.ll, b.ctl, status);
     LCHECK();
-    screen_plane_kernel<<<Kpad / 8, 256, 0, s>>>(D, K, Kpad, mu, w2, b.sd, b.gd, b.prm, b.key, b.p, b.blk, b.comp_of);
+    static_assert((size_t)PR_GROUPS * PR_ROWS * SCR_MAX_K <= (size_t)SCR_PAIRS, "the probe's bounds lie where the sorted pairs will");
+    const ProbeArgs pr{probe, K, mu, w2, c2d, b.prm, b.key, b.probe, Kpad / 8, reinterpret_cast<float2*>(b.srt), b.ctl};
+    screen_plane_kernel<<<Kpad / 8 + (probe.n > 0 ? PR_GROUPS * PR_CTAS : 0), 256, 0, s>>>(pr, D, K, Kpad, mu, w2, b.sd, b.gd, b.prm, b.key, b.p, b.blk, b.comp_of);
     return cudaGetLastError();
 }
 
@@ -1837,8 +1965,6 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
     p.chunks = screen_chunks(D); p.y = b.y; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
     p.blk = b.blk; p.n2 = b.n2; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
     p.ovf = b.ovf; p.ctl = b.ctl; p.status = status; p.test_silent = b.test_silent;
-    p.tile_limit = (int)fmin(1.1 * (double)max_marks * SCR_TILE, 1e9);
-    p.tile_over = n >= 65536 ? SCR_TILE / 32 : SCR_TILE;      // (the share of rows that screen_rows_kernel takes)
     if (top < 1 || top > 4) return cudaErrorInvalidValue;
     auto sweep = top == 1 ? screen_sweep_kernel<1> : top == 2 ? screen_sweep_kernel<2> : screen_sweep_kernel<4>;
     cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);

@@ -24,6 +24,7 @@ constexpr int SCR_RANGES = (int)(SCR_PIECE / SCR_RANGE);
 constexpr int SCR_LL = 4096;                 // log-likelihood partial sums (one per CTA of a launch), then one per component
 constexpr int SCR_DIM_BLOCKS = 64;
 constexpr int SCR_GROUP = 32768;             // points of a group that launch_screen_groups takes (16-bit cursors; one CTA sorts a group)
+constexpr int PR_ROWS = 4, PR_GROUPS = 16, PR_CTAS = 16;     // rows that are looked at ahead of a call's sweep: see screen_probe
 constexpr int SCR_SPILL = 22, SCR_MAX_SMS = 160;      // see screen_sweep_kernel
 
 // Control words (in the context's result block, so that they travel to the host with the log-likelihood).
@@ -32,6 +33,7 @@ enum { SC_DENSE = 0,      // set when a piece marks too many pairs or is not fin
        SC_OVF,            // rows of the current piece that left the sweep without a list
        SC_EXTRA,          // pairs of those rows
        SC_TICKET_A, SC_TICKET_B,
+       SC_PROBED,         // pairs of the rows that were looked at ahead of the sweep
        SC_ACTIVE,         // components with a weight
        SC_KEPT,           // kept pairs of all pieces (saturating)
        SC_FALLBACK,       // an assignment that the FP32 kernels have to do (see launch_screen_gate)
@@ -46,6 +48,7 @@ struct ScreenBuffers {
     unsigned char* p;     // coefficients [Kpad / 128][screen_group_bytes]
     int4* blk;            // [SCR_MAX_K / 32] of 32 positions: largest allowances (as bits), whether one is capped
     int* comp_of;         // [Kpad]
+    unsigned* probe;      // [PR_GROUPS][PR_ROWS + 1] of the probed rows: largest lower bound (see order_up); CTAs that are done
     unsigned char* y;     // rows of u [SCR_PIECE][16-byte chunks of 8 halves]
     float* n2;            // [SCR_PIECE] |u|^2
     unsigned* pt_off;     // [SCR_PIECE] where a point's pairs start
@@ -71,10 +74,13 @@ inline int screen_kpad(int K) { return (K + 127) / 128 * 128; }
 inline int screen_atoms(int D) { return (D + 31) / 32; }
 __host__ __device__ inline size_t screen_group_bytes(int D) { return 4096 + (size_t)((D + 31) / 32) * 16384; }
 
+// A call's data X [n] (n = 0: none), of which some rows are looked at ahead of the sweep, and what the sweep will be asked (see launch_screen_sweep).
+struct ScreenProbe { const float* X; int64_t n; float margin; int top; float max_marks; };
 // Parameters -> w2, c2, c2d (as launch_prepare_fp32, with the same checks), coefficient plane and tables.  unit: k-means (mu =
-// centroids; pi, var not read; log2 z = -|x - mu|^2; one that is not finite sets SC_DENSE and no status).  Clears SC_DENSE.
+// centroids; pi, var not read; log2 z = -|x - mu|^2; one that is not finite sets SC_DENSE and no status).  SC_DENSE: 0, or 1
+// where the probed rows have too many pairs.  Clears the partial log-likelihoods.
 cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
-                                  const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
+                                  const ScreenProbe& probe, const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
 // One piece of n <= SCR_PIECE points: plane, sweep, rows without a list.  margin: log2 units below a point's best value down to
 // which pairs are marked (40, or 0 for the arg-max alone); top: so many of its largest pairs are marked in any case (1 to 4).  max_marks: pairs per point up to which the screening pays; stats:
 // statistics are to follow, which have room for SCR_MARKS of them.

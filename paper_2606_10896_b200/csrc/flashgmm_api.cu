@@ -41,7 +41,7 @@ struct ScratchLayout {
     size_t w_partial_bytes;
     bool wide;
     // the screening path for D <= 128 (its plane of the points lies in tc_yhi)
-    size_t s_sd, s_gd, s_dimpart, s_prm, s_key, s_p, s_blk, s_compof, s_n2, s_ptoff, s_ptcnt, s_words, s_spill, s_ids, s_val, s_srt, s_counts, s_totals, s_off, s_segoff, s_part, s_ll, s_ovf;
+    size_t s_sd, s_gd, s_dimpart, s_prm, s_key, s_p, s_blk, s_compof, s_probe, s_n2, s_ptoff, s_ptcnt, s_words, s_spill, s_ids, s_val, s_srt, s_counts, s_totals, s_off, s_segoff, s_part, s_ll, s_ovf;
     bool scr;
 };
 
@@ -156,7 +156,7 @@ ScratchLayout scratch_layout(int D, int K, bool planes) {
         L.w_ylo = take((size_t)WIDE_PIECE * wp.Dpad * 4);
     }
     L.scr = L.tc && planes && screen_supports(D, K);
-    L.s_sd = L.s_gd = L.s_dimpart = L.s_prm = L.s_key = L.s_p = L.s_blk = L.s_compof = L.s_n2 = L.s_ptoff = L.s_ptcnt = L.s_words = L.s_spill = L.s_ids = L.s_val = L.s_srt = L.s_counts = L.s_totals = L.s_off = L.s_segoff = L.s_part = L.s_ll = L.s_ovf = 0;
+    L.s_sd = L.s_gd = L.s_dimpart = L.s_prm = L.s_key = L.s_p = L.s_blk = L.s_compof = L.s_probe = L.s_n2 = L.s_ptoff = L.s_ptcnt = L.s_words = L.s_spill = L.s_ids = L.s_val = L.s_srt = L.s_counts = L.s_totals = L.s_off = L.s_segoff = L.s_part = L.s_ll = L.s_ovf = 0;
     if (L.scr) {
         static_assert((size_t)SCR_PIECE * 256 <= TC_YPLANE_BYTES, "the plane of the screening path lies in that of the tile kernel");
         const size_t Kpad = (size_t)screen_kpad(K);
@@ -168,6 +168,7 @@ ScratchLayout scratch_layout(int D, int K, bool planes) {
         L.s_p = take(Kpad / 128 * screen_group_bytes(D));
         L.s_blk = take((size_t)SCR_MAX_K / 32 * 16);
         L.s_compof = take(Kpad * 4);
+        L.s_probe = take((size_t)PR_GROUPS * (PR_ROWS + 1) * 4);
         L.s_n2 = take((size_t)SCR_PIECE * 4);
         L.s_ptoff = take((size_t)SCR_PIECE * 4);
         L.s_ptcnt = take((size_t)SCR_PIECE * 4);
@@ -319,6 +320,7 @@ struct gmm_ctx {
         b.p = at(lay.s_p);
         b.blk = reinterpret_cast<int4*>(at(lay.s_blk));
         b.comp_of = reinterpret_cast<int*>(at(lay.s_compof));
+        b.probe = reinterpret_cast<unsigned*>(at(lay.s_probe));
         b.y = at(lay.tc_yhi);
         b.n2 = reinterpret_cast<float*>(at(lay.s_n2));
         b.pt_off = reinterpret_cast<unsigned*>(at(lay.s_ptoff));
@@ -805,9 +807,9 @@ int accumulate_points(gmm_ctx* ctx, int path, const float* X, int64_t n, int D, 
     return GMM_OK;
 }
 
-// (one launch; screened: the screening path's partial log-likelihoods too)
-int zero_stats(gmm_ctx* ctx, int D, int K, double* Nk, double* S1, double* S2, int slot, bool screened = false) {
-    KL(launch_zero_stats(ctx->stream, D, K, Nk, S1, S2, &ctx->result()->ll[slot], screened ? ctx->screen().ll : nullptr, SCR_LL + K));
+// (one launch)
+int zero_stats(gmm_ctx* ctx, int D, int K, double* Nk, double* S1, double* S2, int slot) {
+    KL(launch_zero_stats(ctx->stream, D, K, Nk, S1, S2, &ctx->result()->ll[slot]));
     return GMM_OK;
 }
 
@@ -855,9 +857,10 @@ int read_result(gmm_ctx* ctx, int slot, double* loglik) {
 }
 
 // ---- the screening path (D <= 128) ----------------------------------------------------------------------------------
-// AUTO tries it first wherever it would take the tensor path.  Its kernels find out themselves whether it pays (SC_DENSE) and
-// then return at once, so a call enqueues the whole path, reads the verdict with its result and only then, if need be, runs the
-// dense kernels: sparse posteriors cost no extra synchronisation, broad ones the sweep of one piece.
+// AUTO tries it first wherever it would take the tensor path.  Its kernels find out themselves whether it pays (SC_DENSE: from rows
+// spread over the call's data, see screen_probe, then piece by piece) and return at once where it does not, so a call enqueues the
+// whole path, reads the verdict with its result and only then, if need be, runs the dense kernels: sparse posteriors cost no extra
+// synchronisation, broad ones about 60 us of preparation and launches.
 bool screen_wanted(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     return ctx->path == GMM_PATH_AUTO && ctx->lay.scr && ctx->capPlanes && ctx->scr_marks != 0.0 &&
            (auto_is_tensor(D, K) || small_screen(ctx, kind, N, D, K, groups));
@@ -885,11 +888,10 @@ int64_t screen_piece(const gmm_ctx* ctx, int64_t n) {
     return pieces <= 1 ? most : ((n + pieces - 1) / pieces + wave - 1) / wave * wave;
 }
 
-int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, const float* var, bool unit, bool clear = true) {
+int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, const float* var, bool unit, const ScreenProbe& probe) {
     const ScreenBuffers sb = ctx->screen();
-    KL(launch_screen_prepare(ctx->stream, D, K, pi, mu, var, unit, sb, ctx->w2(), ctx->c2(), ctx->c2d(), &ctx->result()->status));
+    KL(launch_screen_prepare(ctx->stream, D, K, pi, mu, var, unit, probe, sb, ctx->w2(), ctx->c2(), ctx->c2d(), &ctx->result()->status));
     ctx->launches += 2;
-    if (clear) CU(cudaMemsetAsync(sb.ll, 0, (size_t)(SCR_LL + K) * 8, ctx->stream));      // (else zero_stats does)
     return GMM_OK;
 }
 
@@ -1091,8 +1093,8 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
     if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
         bool dense = false;
-        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
-        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0, true));
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
+        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
         CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
         CHECK(screen_end(ctx, K, 0));
         CHECK(screen_result(ctx, 0, loglik, &dense));
@@ -1202,6 +1204,7 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         if (iters_done) *iters_done = t;
         return GMM_OK;
     }
+    bool probe = true;
     for (; t < iters; ++t) {
         const int slot = t % LL_SLOTS;
         // The update is skipped on the device when the step raised a status bit or left a non-finite log-likelihood
@@ -1217,12 +1220,14 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         int rc = GMM_OK;
         bool dense = true;
         if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
-            CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
-            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot, true));
+            // (no look ahead where the iteration before this one was sparse: posteriors sharpen)
+            CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, probe ? N : 0, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
+            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
             CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
             CHECK(screen_end(ctx, K, slot));
             CHECK(update(&ctx->result()->scr[SC_DENSE]));
             rc = screen_result(ctx, slot, &loglik_trace[t], &dense);
+            probe = dense;
         }
         if (dense && rc == GMM_OK) {
             CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
@@ -1336,9 +1341,9 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
     bool screening = screen_try(ctx, SCREEN_STEPS, N, D, K);
-    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
+    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {ctx->xstage[0], cnt0, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
     else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
-    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0, screening));
+    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
     int c = 0;                                       // chunks copied so far: they take the buffers in turn
     bool copied = true;                              // (the first one already is)
     for (int64_t off = 0; off < N; off += rows_per_chunk, ++c) {
@@ -1574,12 +1579,13 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
     const int* dense_if = nullptr;
     if (screening) {
         dense_if = run_fp32_if = ctx->result()->scr + SC_DENSE;
-        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, false));
+        const float margin = index_only ? 0.f : 40.f, limit = ctx->scr_marks > 0.0 ? (float)ctx->scr_marks : 12.f;
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, margin, m == 3 ? 4 : m, limit}));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
             CHECK(prof_begin(ctx));
-            CHECK(screen_values(ctx, SCREEN_TOP, X + off * D, cnt, D, K, index_only ? 0.f : 40.f, ctx->scr_marks > 0.0 ? ctx->scr_marks : 12.0, mu, nullptr,
+            CHECK(screen_values(ctx, SCREEN_TOP, X + off * D, cnt, D, K, margin, limit, mu, nullptr,
                                 idx + off * m, false, m, index_only ? nullptr : resp + off * m));
             CHECK(prof_end(ctx));
         }
@@ -1747,7 +1753,8 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         double* Nk = ctx->stats();
         double* S1 = Nk + K;
         double* S2 = S1 + (size_t)K * D;
-        CHECK(screen_begin(ctx, D, K, nullptr, centroids, nullptr, true, false));
+        const double limit = screen_limit(ctx, SCREEN_CENTROIDS, N, D, K);
+        CHECK(screen_begin(ctx, D, K, nullptr, centroids, nullptr, true, {X, N, 0.f, 1, (float)limit}));
         // (the kernels below would decide a near tie in fp32 about a centre, or among log-densities of the unit mixture)
         ScreenTie tie{nullptr, (float)0.72134752044448170368,
                       (float)(1.4426950408889634074 * (std::log((double)(1.f / (float)K)) - 0.5 * D * std::log(6.283185307179586476925286766559)))};
@@ -1755,12 +1762,12 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
             KL(launch_center_fp32(ctx->stream, D, K, centroids, ctx->center()));
             tie = {ctx->center(), 1.f, 0.f};
         }
-        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0, true));
+        CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
             const float* Xs = X + off * D;
-            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, screen_limit(ctx, SCREEN_CENTROIDS, N, D, K), centroids, nullptr, assign + off, true, 1, nullptr, &tie));
+            CHECK(screen_values(ctx, SCREEN_ARGMAX, Xs, cnt, D, K, 0.f, limit, centroids, nullptr, assign + off, true, 1, nullptr, &tie));
             CU(launch_screen_stats(ctx->stream, Xs, cnt, D, K, centroids, ctx->w2(), ctx->c2d(), sb, Nk, S1, S2, &ctx->launches));
         }
         double* ik = km_inertia_k(ctx->km_scratch, D, K);
@@ -1840,7 +1847,7 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
                              : std::fmin(14.0, std::fmax(1.5, 0.9 * (0.03 + 1.9e-4 * K * D - fixed) / (0.05 + 0.0007 * D)));
         bool dense = false;
         double total = 0.0;
-        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, 40.f, 1, (float)limit}));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
@@ -1965,7 +1972,8 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
     if (smallest > 0 && screen_try(ctx, SCREEN_STEPS, N, D, K, G)) {
         // Screening path: consecutive groups are taken as many at a time as a piece holds; a larger group goes
         // through the step's own accumulation.
-        CHECK(screen_begin(ctx, D, K, pi, mu, var, false));
+        CHECK(screen_begin(ctx, D, K, pi, mu, var, false,
+                           {X + offsets[0] * D, offsets[G] - offsets[0], 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K, G)}));
         struct Batch { int g0, g1; bool large; };
         std::vector<Batch> batches;
         std::vector<int> tab(2 * (size_t)G);                     // start of a group within its batch, points

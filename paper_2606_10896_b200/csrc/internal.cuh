@@ -84,8 +84,8 @@ cudaError_t launch_fused_direct(cudaStream_t s, const float* X, int64_t n, int D
                                 bool accumulate, double* ll, int* status, const DirectFit* fit, int64_t* launches);
 
 // ---- shared by all paths -------------------------------------------------------------------------------------
-// Nk, S1, S2, *ll and (unless NULL) extra[n_extra] = 0, in one launch
-cudaError_t launch_zero_stats(cudaStream_t s, int D, int K, double* Nk, double* S1, double* S2, double* ll, double* extra, int n_extra);
+// Nk, S1, S2, *ll = 0, in one launch
+cudaError_t launch_zero_stats(cudaStream_t s, int D, int K, double* Nk, double* S1, double* S2, double* ll);
 // stats (+)= sum over `splits` partial blocks, fixed order, float64.  Partial layout: [splits][K + 2*K*D] floats,
 // each block being (N_k [K], sums of r (x - g) [K*D], sums of r (x - g)^2 [K*D]); float64 instead when
 // fp32_plan(D, K).wide.  g [D]: the centre launch_mstep_fp32 was given (NULL = 0); the shift back to S1, S2 is exact.

@@ -119,21 +119,20 @@ __global__ void finalize_isotropic_kernel(int64_t N, int D, int K, const double*
 }
 
 __global__ void __launch_bounds__(256) zero_stats_kernel(size_t K, size_t KD, double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
-                                                         double* __restrict__ ll, double* __restrict__ extra, size_t n_extra) {
-    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < KD || i < K || i < n_extra; i += (size_t)gridDim.x * 256) {
-        if (i < KD) { S1[i] = 0.0; S2[i] = 0.0; }
+                                                         double* __restrict__ ll) {
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < KD; i += (size_t)gridDim.x * 256) {      // (K <= K D)
+        S1[i] = 0.0;
+        S2[i] = 0.0;
         if (i < K) Nk[i] = 0.0;
-        if (i < n_extra) extra[i] = 0.0;
         if (i == 0) *ll = 0.0;
     }
 }
 
 }  // namespace
 
-cudaError_t launch_zero_stats(cudaStream_t s, int D, int K, double* Nk, double* S1, double* S2, double* ll, double* extra, int n_extra) {
-    const size_t KD = (size_t)K * D, n = extra && (size_t)n_extra > KD ? (size_t)n_extra : KD;
-    const size_t blocks = (n + 255) / 256;
-    zero_stats_kernel<<<(unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, s>>>((size_t)K, KD, Nk, S1, S2, ll, extra, extra ? (size_t)n_extra : 0);
+cudaError_t launch_zero_stats(cudaStream_t s, int D, int K, double* Nk, double* S1, double* S2, double* ll) {
+    const size_t KD = (size_t)K * D, blocks = (KD + 255) / 256;
+    zero_stats_kernel<<<(unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, s>>>((size_t)K, KD, Nk, S1, S2, ll);
     return cudaGetLastError();
 }
 

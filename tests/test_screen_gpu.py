@@ -235,3 +235,23 @@ def test_screen_top_m(fg, monkeypatch, N, D, K, m):
         r_ref = np.exp(got - lz[:, None])
     far = np.arange(N) == N // 2                            # (its log-densities of 1e7 leave fp32 little to tell)
     assert np.all(np.abs(resp - r_ref)[~far] <= 2e-4 * r_ref[~far] + 1e-6)
+
+
+def test_screen_verdict_follows_the_whole_data(fg):
+    """Rows in groups: a quarter of a tile whose posteriors are broad must not send sparse data to the dense kernels, wherever it lies, and a
+    tenth of the data must, though the first tiles are sparse."""
+    N, D, K = 60_000, 16, 256
+    X, pi, mu, var = _mixture(N, D, K, 21)
+    mu[K // 2:], var[K // 2:] = 12.0 + 0.05 * mu[K // 2:], 1.0
+    rng = np.random.default_rng(4)
+    X = (mu[rng.integers(0, K // 2, N)] + rng.normal(size=(N, D))).astype(np.float32)
+    broad = (12.0 + rng.normal(size=(N // 10, D))).astype(np.float32)
+    for first, n, sparse in [(0, 64, True), (256 * 100 + 30, 64, True), (N - 64, 64, True), (N - N // 10, N // 10, False)]:
+        Y = X.copy()
+        Y[first:first + n] = broad[:n]
+        with fg.Context(0) as c:
+            ref = orc.em_step(Y, pi, mu, var)
+            got = c.gmm_em_step(_t(Y), _t(pi), _t(mu), _t(var))
+            assert (c.gmm_last_exact_count() == K) == sparse, (first, n)
+            assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3])
+            assert_stats_close(N, data_scale(Y), [v.cpu().numpy() for v in got[:3]], ref[:3], f"broad rows {first}+{n}")

@@ -76,8 +76,8 @@ int gmm_tensor_path_supports(int D, int K);
  * accurate for small mixtures.  For D <= 128 AUTO first tries one tensor sweep that only screens the (point, component)
  * pairs and evaluates those it cannot rule out (every component within 2^-40 of a point's best) exactly in fp32: on sparse
  * posteriors this is the faster and the more accurate way, also for calls with many points and 16 <= K < 64 (GMM_PATH_TENSOR is
- * then reported).  Broad posteriors are noticed on the device and left to the dense kernels of either path; after such a
- * call the context leaves the next calls of that kind and shape (1, 2, 4 .. 16) to them at once.  On wide data (D > 128) a step may still run on the FP32 kernels when the parameters
+ * then reported).  Broad posteriors are noticed on the device, from rows spread over the call's data, and left to the dense kernels
+ * of either path; after such an iteration gmm_fit leaves its next 1, 2, 4 .. 16 to them at once.  Earlier calls have no say.  On wide data (D > 128) a step may still run on the FP32 kernels when the parameters
  * or the data make that the better choice (more than half of the components ill-conditioned; fewer than 128 points per
  * component and posteriors too broad for the screening mode): gmm_last_path tells. */
 int gmm_auto_path(int D, int K);

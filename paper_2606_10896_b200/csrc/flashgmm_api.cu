@@ -248,10 +248,6 @@ struct gmm_ctx {
     double scr_marks = -1.0;         // GMM_SCREEN_MARKS: marked pairs per point up to which the screening path is taken (D <= 128;
                                      // 0: never, < 0: from the measured costs, see screen_limit)
     int64_t scr_piece = 0;           // GMM_SCREEN_PIECE: points per round of launches of the screening path (0: screen_piece)
-    // After a call that the screening has left to the dense kernels, so many calls of the same kind and shape go to them at once
-    // (1, 2, 4 .. 16: mixtures of a fit sharpen as it goes on); see screen_try.
-    struct ScreenHistory { int D = 0, K = 0, skip = 0, left = 0; } scr_history[3];
-    int scr_kind = 0;
     int scr_test_silent = -1;        // GMM_SCREEN_TEST_SILENT (time-out test)
     DevResult* pinned = nullptr;     // where the result block is read back to
     int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
@@ -925,25 +921,10 @@ int screen_end(gmm_ctx* ctx, int K, int slot) {
 }
 
 // Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels.
-bool screen_try(gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
-    if (!screen_wanted(ctx, kind, N, D, K, groups)) return false;
-    auto& h = ctx->scr_history[kind];
-    if (h.D != D || h.K != K) { h = {}; h.D = D; h.K = K; }
-    if (ctx->scr_marks < 0.0 && h.left > 0) { --h.left; return false; }
-    ctx->scr_kind = kind;
-    return true;
-}
-void screen_note(gmm_ctx* ctx, bool dense) {
-    auto& h = ctx->scr_history[ctx->scr_kind];
-    h.skip = !dense ? 0 : h.skip == 0 ? 1 : h.skip < 16 ? 2 * h.skip : 16;
-    h.left = h.skip;
-}
-
 int screen_result(gmm_ctx* ctx, int slot, double* loglik, bool* dense) {
     DevResult r;
     CHECK(read_back(ctx, &r));
     *dense = r.scr[SC_DENSE] != 0;
-    screen_note(ctx, *dense);
     ctx->scr_active = 0;
     CHECK(report_status(ctx, r.status));
     if (*dense) return GMM_OK;
@@ -1091,7 +1072,7 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     DeviceGuard g(ctx->device);
     int path;
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
-    if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
+    if (screen_wanted(ctx, SCREEN_STEPS, N, D, K)) {
         bool dense = false;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
         CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
@@ -1204,6 +1185,9 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         if (iters_done) *iters_done = t;
         return GMM_OK;
     }
+    // (after an iteration that the screening has left to the dense kernels the next 1, 2, 4 .. 16 go to them at once: the mixtures of a
+    // fit sharpen as it goes on)
+    int skip = 0, left = 0;
     bool probe = true;
     for (; t < iters; ++t) {
         const int slot = t % LL_SLOTS;
@@ -1219,7 +1203,9 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         };
         int rc = GMM_OK;
         bool dense = true;
-        if (screen_try(ctx, SCREEN_STEPS, N, D, K)) {
+        if (left > 0 && ctx->scr_marks < 0.0) {
+            --left;
+        } else if (screen_wanted(ctx, SCREEN_STEPS, N, D, K)) {
             // (no look ahead where the iteration before this one was sparse: posteriors sharpen)
             CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, probe ? N : 0, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
             CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
@@ -1228,6 +1214,7 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
             CHECK(update(&ctx->result()->scr[SC_DENSE]));
             rc = screen_result(ctx, slot, &loglik_trace[t], &dense);
             probe = dense;
+            left = skip = !dense ? 0 : skip == 0 ? 1 : skip < 16 ? 2 * skip : 16;
         }
         if (dense && rc == GMM_OK) {
             CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
@@ -1340,7 +1327,7 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     CU(cudaMemcpyAsync(ctx->xstage[0], X_host, (size_t)cnt0 * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
     CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
     CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
-    bool screening = screen_try(ctx, SCREEN_STEPS, N, D, K);
+    bool screening = screen_wanted(ctx, SCREEN_STEPS, N, D, K);
     if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {ctx->xstage[0], cnt0, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
     else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
     CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
@@ -1746,7 +1733,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_CENTROIDS, N, D, K)));
     CHECK(grow_buffer(ctx, &ctx->pl_scratch, &ctx->pl_scratch_bytes, pl_scratch_bytes(K), "the posting-list counters"));
     CHECK(grow_buffer(ctx, &ctx->km_scratch, &ctx->km_scratch_bytes, km_scratch_bytes(D, K), "the k-means partial sums"));
-    if (screen_try(ctx, SCREEN_CENTROIDS, N, D, K)) {
+    if (screen_wanted(ctx, SCREEN_CENTROIDS, N, D, K)) {
         // through the screening path: the arg-max alone (margin 0), every point a lone pair of its cluster, and the statistics
         // of the pairs about the centroids give the new ones and the inertia
         const ScreenBuffers sb = ctx->screen();
@@ -1775,7 +1762,6 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         KL(launch_reduce_ll(ctx->stream, ik, K, &ctx->result()->ll[0], false));
         DevResult r;
         CHECK(read_back(ctx, &r));
-        screen_note(ctx, r.scr[SC_DENSE] != 0);
         CHECK(report_status(ctx, r.status));
         if (r.scr[SC_DENSE] == 0) {
             if (inertia) *inertia = r.ll[0];
@@ -1840,7 +1826,7 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
     CHECK(check_ptr(ctx, logp, 4, "logp"));
     DeviceGuard guard(ctx->device);
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_DENSITIES, N, D, K)));
-    if (screen_try(ctx, SCREEN_DENSITIES, N, D, K)) {
+    if (screen_wanted(ctx, SCREEN_DENSITIES, N, D, K)) {
         // D <= 128: the same idea (csrc/em_screen.cu).  Costs per point as in screen_limit, without statistics.
         const double fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
         const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks
@@ -1969,7 +1955,7 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
-    if (smallest > 0 && screen_try(ctx, SCREEN_STEPS, N, D, K, G)) {
+    if (smallest > 0 && screen_wanted(ctx, SCREEN_STEPS, N, D, K, G)) {
         // Screening path: consecutive groups are taken as many at a time as a piece holds; a larger group goes
         // through the step's own accumulation.
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false,

@@ -255,3 +255,32 @@ def test_screen_verdict_follows_the_whole_data(fg):
             assert (c.gmm_last_exact_count() == K) == sparse, (first, n)
             assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3])
             assert_stats_close(N, data_scale(Y), [v.cpu().numpy() for v in got[:3]], ref[:3], f"broad rows {first}+{n}")
+
+
+def test_screen_forgets_earlier_calls(fg):
+    """The same call gives the same bits whatever the context did before: sparse calls around broad ones of every entry point, and a fit whose
+    posteriors sharpen on its way, twice."""
+    N, D, K = 6000, 24, 128
+    X, pi, mu, var = _mixture(N, D, K, 31)
+    x, sparse = _t(X), [_t(a) for a in (pi, mu, var)]
+    broad = [_t(pi), _t(X[:K]), _t(np.repeat(X.var(0)[None], K, 0))]
+    offsets = np.array([0, N // 3, N], np.int64)
+
+    def calls(c, params):
+        out = list(c.gmm_em_step(x, *params)) + list(c.gmm_score_samples(x, *params)) + list(c.gmm_fisher_vectors(x, offsets, *params))
+        out += list(c.gmm_assign_topm(x, *params, 2)) + list(c.gmm_kmeans_step(x, params[1])) + list(c.gmm_em_step_host(X, *[p.cpu().numpy() for p in params]))
+        out.append(c.gmm_last_exact_count())
+        return [v.cpu().numpy().copy() if torch.is_tensor(v) else np.array(v) for v in out]
+
+    def fit(c):
+        p = [v.clone() for v in broad]
+        trace, _ = c.gmm_fit(x, *p, 12)
+        return [trace] + [v.cpu().numpy() for v in p]
+
+    with fg.Context(0) as c:
+        first, fit1 = calls(c, sparse), fit(c)
+        assert first[-1] == K
+        for _ in range(2):
+            calls(c, broad)
+            assert all(np.array_equal(u, v) for u, v in zip(first, calls(c, sparse)))
+        assert all(np.array_equal(u, v) for u, v in zip(fit1, fit(c)))

@@ -857,9 +857,17 @@ int read_result(gmm_ctx* ctx, int slot, double* loglik) {
 // spread over the call's data, see screen_probe, then piece by piece) and return at once where it does not, so a call enqueues the
 // whole path, reads the verdict with its result and only then, if need be, runs the dense kernels: sparse posteriors cost no extra
 // synchronisation, broad ones about 60 us of preparation and launches.
+// Cost of screening in ns per point without the marked pairs: the sweep, and what else does not depend on them.
+double screen_fixed(int D, int K) { return 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0; }
 bool screen_wanted(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
-    return ctx->path == GMM_PATH_AUTO && ctx->lay.scr && ctx->capPlanes && ctx->scr_marks != 0.0 &&
-           (auto_is_tensor(D, K) || small_screen(ctx, kind, N, D, K, groups));
+    if (ctx->path != GMM_PATH_AUTO || !ctx->lay.scr || !ctx->capPlanes || ctx->scr_marks == 0.0) return false;
+    if (!auto_is_tensor(D, K)) return small_screen(ctx, kind, N, D, K, groups);
+    if (ctx->scr_marks > 0.0) return true;
+    // K >= 64.  Densities: the other way is one launch of the FP32 kernel, in front of which the screening's launches take 25 us more
+    // (two marked pairs per point; us, sparse / FP32: 2K x 16, K = 64 79 / 58, 10K x 32, K = 64 71 / 50, 20K x 32, K = 256 80 / 86,
+    // 200K x 32, K = 64 106 / 112, 10K x 128, K = 1024 96 / 334).  A step on the dense tensor kernels takes 165 us at least.
+    if (kind == SCREEN_DENSITIES) return (double)N * (direct_cost(kind, N, D, K, 0) - screen_fixed(D, K) - 2.0 * (0.05 + 0.0007 * D)) > 25e3;
+    return true;
 }
 // The dense tensor kernels for D <= 128 (planes may be there for the screening alone).
 bool dense_tensor(const gmm_ctx* ctx, int D, int K) {
@@ -871,7 +879,7 @@ bool dense_tensor(const gmm_ctx* ctx, int D, int K) {
 // K < 64: the FP32 kernels' costs.
 double screen_limit(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     if (ctx->scr_marks > 0.0) return ctx->scr_marks;
-    const double dense = K < 64 ? direct_cost(kind, N, D, K, groups) : 0.5 + 0.0032 * K, fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
+    const double dense = K < 64 ? direct_cost(kind, N, D, K, groups) : 0.5 + 0.0032 * K, fixed = screen_fixed(D, K);
     return std::fmin((double)SCR_MARKS, std::fmax(1.5, 0.9 * (dense - fixed) / (0.09 + 0.001 * D)));
 }
 
@@ -1828,9 +1836,8 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_DENSITIES, N, D, K)));
     if (screen_wanted(ctx, SCREEN_DENSITIES, N, D, K)) {
         // D <= 128: the same idea (csrc/em_screen.cu).  Costs per point as in screen_limit, without statistics.
-        const double fixed = 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0;
         const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks
-                             : std::fmin(14.0, std::fmax(1.5, 0.9 * (0.03 + 1.9e-4 * K * D - fixed) / (0.05 + 0.0007 * D)));
+                             : std::fmin(14.0, std::fmax(1.5, 0.9 * (0.03 + 1.9e-4 * K * D - screen_fixed(D, K)) / (0.05 + 0.0007 * D)));
         bool dense = false;
         double total = 0.0;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, 40.f, 1, (float)limit}));

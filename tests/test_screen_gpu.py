@@ -284,3 +284,13 @@ def test_screen_forgets_earlier_calls(fg):
             calls(c, broad)
             assert all(np.array_equal(u, v) for u, v in zip(first, calls(c, sparse)))
         assert all(np.array_equal(u, v) for u, v in zip(fit1, fit(c)))
+
+
+@pytest.mark.parametrize("N,D,K,screened", [(2000, 16, 64, False), (10_000, 32, 64, False), (10_000, 128, 1024, True)])
+def test_screen_of_densities_only_where_it_is_faster(fg, N, D, K, screened):
+    X, pi, mu, var = _mixture(N, D, K, 41)
+    ref = np.logaddexp.reduce(np.asarray(orc.log_joint(X, pi, mu, var), np.float64), axis=1)
+    with fg.Context(0) as c:
+        logp, total = c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var))
+        assert c.gmm_last_path() == (fg.GMM_PATH_TENSOR if screened else fg.GMM_PATH_FP32)
+    assert np.all(np.abs(logp.cpu().numpy() - ref) <= 1e-5 * np.abs(ref) + 1e-4) and abs(total - ref.sum()) <= 1e-5 * abs(ref.sum())

@@ -294,3 +294,22 @@ def test_screen_of_densities_only_where_it_is_faster(fg, N, D, K, screened):
         logp, total = c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var))
         assert c.gmm_last_path() == (fg.GMM_PATH_TENSOR if screened else fg.GMM_PATH_FP32)
     assert np.all(np.abs(logp.cpu().numpy() - ref) <= 1e-5 * np.abs(ref) + 1e-4) and abs(total - ref.sum()) <= 1e-5 * abs(ref.sum())
+
+
+@pytest.mark.parametrize("N,D,K,m", [(2000, 16, 64, 1), (10_000, 32, 64, 1), (10_000, 100, 256, 2), (40_000, 32, 256, 2)])
+def test_screen_of_assignments_where_the_rule_takes_either_way(fg, monkeypatch, N, D, K, m):
+    # both sides of the rule on small calls: the same components, but for near ties, and the same responsibilities as by forced screening
+    X, pi, mu, var = _mixture(N, D, K, 43)
+    out = []
+    for marks in (None, "1000"):
+        if marks:
+            monkeypatch.setenv("GMM_SCREEN_MARKS", marks)
+        with fg.Context(0) as c:
+            out.append([v.cpu().numpy() for v in c.gmm_assign_topm(_t(X), _t(pi), _t(mu), _t(var), m)])
+    lj = np.asarray(orc.log_joint(X, pi, mu, var), np.float64)
+    want = np.sort(lj, axis=1)[:, ::-1][:, :m]
+    for idx, resp in out:
+        got = np.take_along_axis(lj, idx.astype(np.int64), axis=1)
+        weight = np.exp(want - np.logaddexp.reduce(lj, axis=1)[:, None]) > 1e-5     # (ranks without weight keep the order of a selection pass)
+        assert np.all((got >= want - (np.abs(want) * 2e-6 + 1e-3))[weight])
+    assert np.abs(out[0][1] - out[1][1]).max() <= 2e-4

@@ -1,9 +1,10 @@
-// FP32 CUDA-core path for D > 128, top-m assignment and parameter preparation for every D (EM for D <= 128: em_direct.cu).  Direct
+// FP32 CUDA-core path for D > 128 and for the shapes up to there that fill its tiles (see fp32_fixed_tiles; the others: em_direct.cu),
+// top-m assignment and parameter preparation for every D.  Direct
 // differences (x - mu)^2 / var, two phases per super-tile of points.
 //
 // Phase 1 (lse_kernel): for a tile of 64 points sweep all K components in blocks of 64, keep the running
 //   (max, sum) of the online log-sum-exp per point on chip, write log Z_i (paper Algorithm 1, Step 1).
-// Phase 2 (mstep_wide_kernel): a CTA owns 64 components; for each of its point tiles it
+// Phase 2 (mstep_kernel, mstep_wide_kernel): a CTA owns 64 components; for each of its point tiles it
 //   recomputes log z_ik, forms r_ik = exp(log z_ik - log Z_i) in shared memory and accumulates N_k and the CENTRED
 //   sums of r (x - g), r (x - g)^2 (Algorithm 1, Step 2) -- they leave the SM once, as a per-CTA partial; there are no
 //   atomics.  The reduction shifts them back to S1, S2 in float64.
@@ -347,6 +348,108 @@ lse_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __
 
 constexpr int LDR = TC + 4;                 // r tile row stride
 constexpr int LDX = FP32_MSTEP_DC + 4;      // X tile row stride
+// M-step for 112 < D <= 128, K > 64.
+constexpr size_t MSTEP_SMEM = sizeof(TileSmem) + (size_t)TP * LDR * 4 + (size_t)TP * LDX * 4;
+
+__global__ void __launch_bounds__(NTHREADS, 2)
+mstep_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __restrict__ mu,
+             const float* __restrict__ w2, const double* __restrict__ c2, const float* __restrict__ g,
+             const double* __restrict__ logZ2, float* __restrict__ partials) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    TileSmem& sm = *reinterpret_cast<TileSmem*>(smem_raw);
+    float* r_s = reinterpret_cast<float*>(smem_raw + sizeof(TileSmem));     // [TP][LDR]
+    float* xm = r_s + TP * LDR;                                              // [TP][LDX]
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int kq = tid >> 5, dq = tid & 31;
+    const int k0 = blockIdx.x * TC;
+    const int split = blockIdx.y, nsplits = gridDim.y;
+    const int dz0 = blockIdx.z * FP32_MSTEP_DC;
+    const int64_t ntiles = (n + TP - 1) / TP;
+
+    float acc1[8][4], acc2[8][4];
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) { acc1[c][j] = 0.f; acc2[c][j] = 0.f; }
+    float nacc = 0.f;
+    float cv[4];
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        const int k = k0 + 4 * tx + b;
+        cv[b] = (k < K) ? (float)__ldg(c2 + k) : -CUDART_INF_F;
+    }
+
+    for (int64_t t = split; t < ntiles; t += nsplits) {
+        const int64_t row0 = t * TP;
+        float q[4][4];
+        tile_quadratic<float>(sm, X, row0, n, D, mu, w2, k0, K, q, g);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int64_t row = row0 + 4 * ty + a;
+            const float lz = (row < n) ? (float)__ldg(logZ2 + row) : CUDART_INF_F;    // +inf -> r = 0 for padded rows
+            float4 rv;
+            rv.x = fast_ex2(cv[0] - q[a][0] - lz);
+            rv.y = fast_ex2(cv[1] - q[a][1] - lz);
+            rv.z = fast_ex2(cv[2] - q[a][2] - lz);
+            rv.w = fast_ex2(cv[3] - q[a][3] - lz);
+            *reinterpret_cast<float4*>(&r_s[(4 * ty + a) * LDR + 4 * tx]) = rv;
+        }
+        // stage this CTA's D-slice of the X tile, row-major
+#pragma unroll 4
+        for (int j = 0; j < (TP * FP32_MSTEP_DC) / NTHREADS; ++j) {
+            const int e = tid + j * NTHREADS, r = e >> 7, c = e & 127;
+            const int64_t row = row0 + r;
+            const int d = dz0 + c;
+            // centred: the sums are taken of x - g and (x - g)^2 (the reduction shifts them back in float64), so that
+            // fp32 accumulation errors scale with the data's spread, not with its distance from the origin
+            xm[r * LDX + c] = (row < n && d < D) ? __ldg(X + row * D + d) - (g ? __ldg(g + d) : 0.f) : 0.f;
+        }
+        __syncthreads();
+        if (tid < TC) {
+            float s = 0.f;
+#pragma unroll 8
+            for (int i = 0; i < TP; ++i) s += r_s[i * LDR + tid];
+            nacc += s;
+        }
+#pragma unroll 2
+        for (int i = 0; i < TP; ++i) {
+            const float4 xv = *reinterpret_cast<const float4*>(&xm[i * LDX + 4 * dq]);
+            const float4 ra = *reinterpret_cast<const float4*>(&r_s[i * LDR + 8 * kq]);
+            const float4 rb = *reinterpret_cast<const float4*>(&r_s[i * LDR + 8 * kq + 4]);
+            const float x1[4] = {xv.x, xv.y, xv.z, xv.w};
+            const float x2[4] = {xv.x * xv.x, xv.y * xv.y, xv.z * xv.z, xv.w * xv.w};
+            const float rr[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc1[c][j] = fmaf(rr[c], x1[j], acc1[c][j]);
+                    acc2[c][j] = fmaf(rr[c], x2[j], acc2[c][j]);
+                }
+        }
+        // the next tile_quadratic starts with __syncthreads(), which also protects r_s / xm
+    }
+
+    const size_t KD = (size_t)K * D;
+    float* pN = partials + (size_t)split * (K + 2 * KD);
+    float* pS1 = pN + K;
+    float* pS2 = pS1 + KD;
+    if (blockIdx.z == 0 && tid < TC && k0 + tid < K) pN[k0 + tid] = nacc;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const int k = k0 + 8 * kq + c;
+        if (k >= K) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int d = dz0 + 4 * dq + j;
+            if (d < D) {
+                pS1[(size_t)k * D + d] = acc1[c][j];
+                pS2[(size_t)k * D + d] = acc2[c][j];
+            }
+        }
+    }
+}
+
 // M-step for D > 128.  A CTA owns 64 components and ALL of D: it forms the responsibilities of a batch of WT point
 // tiles once (full-D quadratic forms, float64 logits) and keeps them in shared memory, then sweeps the 128-wide slices
 // of D, accumulating each slice over the whole batch in registers and adding it to this CTA's own rows of a float64
@@ -606,7 +709,11 @@ cudaError_t launch_prepare_fp32(cudaStream_t s, int D, int K, const float* pi, c
     return launch_center_fp32(s, D, K, mu, g);
 }
 
-int fp32_ll_parts(int64_t n, int D, int K) { return D > 128 ? (int)((n + TP - 1) / TP) : lse_direct_parts(n, D, K); }
+// D <= 128: tiles cut to the shape (em_direct.cu), but for the shapes that fill the fixed tiles of this file (64 components x 32
+// dimensions, statistics x 128): at D = 128, K = 256 the tiles of em_direct.cu leave room for half the points.  FP32 step of 300K points,
+// us, here / there: 128 x 256 3570 / 4180, 128 x 512 6990 / 8200, 127 x 130 4110 / 4460, 128 x 65 1870 / 2120; at D = 112 both take the same.
+static inline bool fp32_fixed_tiles(int D, int K) { return D > 128 || (D > 112 && K > 64); }
+int fp32_ll_parts(int64_t n, int D, int K) { return fp32_fixed_tiles(D, K) ? (int)((n + TP - 1) / TP) : lse_direct_parts(n, D, K); }
 
 // Logits are carried in float64 when the accumulation over D is long.
 static inline bool fp32_high_precision(int D) { return D > 128; }
@@ -614,9 +721,12 @@ static inline bool fp32_high_precision(int D) { return D > 128; }
 cudaError_t launch_lse_fp32(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu,
                             const float* w2, const double* c2d, const float* g, double* logZ2, double* llpart,
                             const double* lower2, const int* run_if) {
-    if (!fp32_high_precision(D)) return launch_lse_direct(s, X, n, D, K, mu, w2, c2d, g, logZ2, llpart);      // (nobody gates those shapes)
+    if (!fp32_fixed_tiles(D, K)) return launch_lse_direct(s, X, n, D, K, mu, w2, c2d, g, logZ2, llpart);      // (nobody gates those shapes)
     const unsigned blocks = (unsigned)((n + TP - 1) / TP);
-    lse_kernel<0, double><<<blocks, NTHREADS, sizeof(TileSmem), s>>>(X, n, D, K, mu, w2, c2d, g, logZ2, llpart, 0, nullptr, nullptr, run_if, nullptr, nullptr, lower2);
+    if (!fp32_high_precision(D))
+        lse_kernel<0, float><<<blocks, NTHREADS, sizeof(TileSmem), s>>>(X, n, D, K, mu, w2, c2d, g, logZ2, llpart, 0, nullptr, nullptr, run_if, nullptr, nullptr);
+    else
+        lse_kernel<0, double><<<blocks, NTHREADS, sizeof(TileSmem), s>>>(X, n, D, K, mu, w2, c2d, g, logZ2, llpart, 0, nullptr, nullptr, run_if, nullptr, nullptr, lower2);
     return cudaGetLastError();
 }
 
@@ -676,7 +786,11 @@ cudaError_t launch_mstep_fp32(cudaStream_t s, const float* X, int64_t n, int D, 
         else mstep_wide_kernel<false><<<wgrid, NTHREADS, MSTEP_WIDE_SMEM, s>>>(X, n, D, K, mu, w2, c2d, g, logZ2, reinterpret_cast<double*>(partials), run_if);
         return cudaGetLastError();
     }
-    return launch_mstep_direct(s, X, n, D, K, mu, w2, c2d, g, logZ2, partials, plan.splits);
+    if (!fp32_fixed_tiles(D, K)) return launch_mstep_direct(s, X, n, D, K, mu, w2, c2d, g, logZ2, partials, plan.splits);
+    cudaError_t e = cudaFuncSetAttribute(mstep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MSTEP_SMEM);
+    if (e != cudaSuccess) return e;
+    mstep_kernel<<<dim3(plan.comp_blocks, plan.splits, plan.d_chunks), NTHREADS, MSTEP_SMEM, s>>>(X, n, D, K, mu, w2, c2d, g, logZ2, partials);
+    return cudaGetLastError();
 }
 
 }  // namespace fg

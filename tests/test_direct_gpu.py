@@ -81,3 +81,15 @@ def test_direct_fit_keeps_the_parameters_of_a_step_that_fails(fg):
         with pytest.raises(fg.GmmError):
             c.gmm_fit(_t(X), *a, 5, 1e-6)
         assert all(np.array_equal(u.cpu().numpy(), v) for u, v in zip(a, (pi, mu, var)))
+
+
+@pytest.mark.parametrize("N,D,K", [(999, 112, 65), (999, 113, 65), (1000, 128, 64), (1, 113, 65), (4097, 127, 200), (65_537 + 64, 128, 66)])
+def test_fp32_step_on_either_side_of_the_fixed_tiles(fg, N, D, K):
+    X, pi, mu, var = _mixture(N, D, K, N + D + K)
+    ref = orc.em_step(X, pi, mu, var)
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        got = [v.cpu().numpy() if torch.is_tensor(v) else v for v in c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var))]
+        logp, total = c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var))
+    assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3]) + 1e-6 and abs(total - ref[3]) <= 1e-5 * abs(ref[3]) + 1e-6
+    assert_stats_close(N, max(1.0, data_scale(X)), got[:3], ref[:3], f"N={N} D={D} K={K}")

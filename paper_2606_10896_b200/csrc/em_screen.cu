@@ -114,6 +114,7 @@ __global__ void __launch_bounds__(512) screen_dim_kernel(int D, int K, const flo
     if (d == 0) {
         ctl[SC_TICKET_A] = 0;
         ctl[SC_PROBED] = 0;
+        ctl[SC_DONE] = 0;
         ctl[SC_DENSE] = 0;
         ctl[SC_ACTIVE] = 0;
         ctl[SC_KEPT] = 0;
@@ -1102,8 +1103,10 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                                                              const unsigned* __restrict__ pt_off, int* __restrict__ pt_cnt,
                                                              unsigned short* __restrict__ ids, float* __restrict__ val,
                                                              int* __restrict__ counts, double* __restrict__ ll, float* __restrict__ logp,
-                                                             int32_t* __restrict__ idx, const int* __restrict__ ctl, const TopOut top) {
+                                                             int32_t* __restrict__ idx, int* __restrict__ ctl, const TopOut top) {
     if (ctl[SC_DENSE] != 0) return;
+    // (a piece is done with its last kernel: this one where there are no statistics)
+    if ((MODE == SCREEN_LOGP || MODE == SCREEN_TOP) && blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_DONE] += 1;
     extern __shared__ int hist[];                    // [K] (unless MODE == SCREEN_LOGP)
     __shared__ float v_s[8][EV_VALS];                // values of the warp's pairs, by place in its part of the lists
     __shared__ unsigned short k_s[8][EV_VALS];       // their positions in the sweep, then their components
@@ -1615,8 +1618,9 @@ __global__ void __launch_bounds__(256) screen_stats_kernel(const float* __restri
 __global__ void __launch_bounds__(1024) screen_reduce_kernel(int D, int K, const float* __restrict__ part, const int* __restrict__ segoff,
                                                              const float* __restrict__ mu, const double* __restrict__ c2d,
                                                              double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
-                                                             double* __restrict__ llk, const int* __restrict__ ctl) {
+                                                             double* __restrict__ llk, int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_DONE] += 1;
     const int k = blockIdx.x, d = threadIdx.x & 127, r = threadIdx.x >> 7, chains = blockDim.x >> 7;      // (2 or 8)
     const int i0 = segoff[k], i1 = segoff[k + 1];
     if (i0 == i1) return;
@@ -2005,15 +2009,15 @@ cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t
     return cudaGetLastError();
 }
 
-// One thread: which kernels of an asynchronous assignment have the word.  gate (the tile kernels return when it is not 0) also counts
-// a screening pass that covered the call; fallback says whether the FP32 kernels run.
-__global__ void screen_gate_kernel(const int* __restrict__ ctl, int* __restrict__ gate, int* __restrict__ fallback) {
-    const bool dense = ctl[SC_DENSE] != 0;
-    *fallback = dense && *gate != 0 ? 1 : 0;
-    if (!dense) *gate = 1;
+// One thread: which kernels have the word.
+__global__ void screen_gate_kernel(int* __restrict__ ctl, int* __restrict__ gate, int* __restrict__ fallback, long long p, int first) {
+    if (first) ctl[SC_ILL] = gate == nullptr || *gate != 0 ? 1 : 0;
+    const bool todo = ctl[SC_DENSE] != 0 && p >= ctl[SC_DONE], ill = ctl[SC_ILL] != 0;
+    *fallback = todo && ill ? 1 : 0;
+    if (gate) *gate = todo && !ill ? 0 : 1;
 }
-cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback) {
-    screen_gate_kernel<<<1, 1, 0, s>>>(b.ctl, gate, fallback);
+cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback, int64_t p, bool first) {
+    screen_gate_kernel<<<1, 1, 0, s>>>(b.ctl, gate, fallback, (long long)p, first ? 1 : 0);
     return cudaGetLastError();
 }
 

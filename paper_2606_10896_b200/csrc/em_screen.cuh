@@ -36,7 +36,8 @@ enum { SC_DENSE = 0,      // set when a piece marks too many pairs or is not fin
        SC_PROBED,         // pairs of the rows that were looked at ahead of the sweep
        SC_ACTIVE,         // components with a weight
        SC_KEPT,           // kept pairs of all pieces (saturating)
-       SC_FALLBACK,       // an assignment that the FP32 kernels have to do (see launch_screen_gate)
+       SC_DONE,           // pieces of the call that are done (SC_DENSE: the others are left to the dense kernels)
+       SC_ILL, SC_FALLBACK,      // parameters or a piece of an assignment that the FP32 kernels have to take (see launch_screen_gate)
        SC_WORDS };
 
 struct ScreenBuffers {
@@ -98,8 +99,10 @@ cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t
                                const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count = true, int m = 1, float* resp = nullptr,
                                const ScreenTie* tie = nullptr);
 // (count: leave the number of kept pairs per component and range for launch_screen_stats)
-// After the last piece of an asynchronous assignment: *gate |= the screening covered the call; *fallback = it did not and *gate was set.
-cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback);
+// Behind the last piece of an asynchronous assignment, for its piece p: *gate = 0 and *fallback = 0 if the tile kernels have to do it, 1
+// and 1 if the FP32 kernels have to, 1 and 0 if it is done.  gate: the tile kernels' flag for parameters that are not for them, looked
+// at when `first` (NULL: there are no tile kernels).
+cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate, int* fallback, int64_t p, bool first);
 // Statistics of the kept pairs: sorted by component, summed in fixed segments, added to (Nk, S1, S2) in float64.
 cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                 const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches);

@@ -928,14 +928,18 @@ int screen_end(gmm_ctx* ctx, int K, int slot) {
     return GMM_OK;
 }
 
-// Synchronising read of the log-likelihood and the status word; *dense = the caller has to run the dense kernels.
-int screen_result(gmm_ctx* ctx, int slot, double* loglik, bool* dense) {
+// Synchronising read of the log-likelihood and the status word for n points.  *from: the point from which on the caller has to run the
+// dense kernels (n: none).  What lies before is in the outputs and in the log-likelihood already.
+int64_t screen_left(const gmm_ctx* ctx, const int* ctl, int64_t n) {
+    return ctl[SC_DENSE] == 0 ? n : std::min(n, (int64_t)ctl[SC_DONE] * screen_piece(ctx, n));
+}
+int screen_result(gmm_ctx* ctx, int slot, double* loglik, int64_t n, int64_t* from) {
     DevResult r;
     CHECK(read_back(ctx, &r));
-    *dense = r.scr[SC_DENSE] != 0;
+    *from = screen_left(ctx, r.scr, n);
     ctx->scr_active = 0;
     CHECK(report_status(ctx, r.status));
-    if (*dense) return GMM_OK;
+    if (r.scr[SC_DENSE] != 0) return GMM_OK;
     ctx->scr_active = r.scr[SC_ACTIVE];
     ctx->last_path = GMM_PATH_TENSOR;
     *loglik = r.ll[slot];
@@ -1080,19 +1084,19 @@ int gmm_em_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const flo
     DeviceGuard g(ctx->device);
     int path;
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_STEPS, N, D, K)));
+    int64_t from = 0;
     if (screen_wanted(ctx, SCREEN_STEPS, N, D, K)) {
-        bool dense = false;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
         CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
         CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
         CHECK(screen_end(ctx, K, 0));
-        CHECK(screen_result(ctx, 0, loglik, &dense));
-        if (!dense) return GMM_OK;
+        CHECK(screen_result(ctx, 0, loglik, N, &from));
+        if (from == N) return GMM_OK;
     }
     CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
-    const bool fresh = path == GMM_PATH_FP32 && fused_direct_supports(D, K);      // (writes the statistics, nothing to add to)
-    if (!fresh) CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
-    CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, 0, fresh));
+    const bool fresh = from == 0 && path == GMM_PATH_FP32 && fused_direct_supports(D, K);      // (writes the statistics, nothing to add to)
+    if (from == 0 && !fresh) CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
+    CHECK(accumulate_points(ctx, path, X + from * D, N - from, D, K, mu, Nk, S1, S2, 0, fresh));
     ctx->last_path = path;
     return read_result(ctx, 0, loglik);
 }
@@ -1210,7 +1214,7 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
             return GMM_OK;
         };
         int rc = GMM_OK;
-        bool dense = true;
+        int64_t from = 0;
         if (left > 0 && ctx->scr_marks < 0.0) {
             --left;
         } else if (screen_wanted(ctx, SCREEN_STEPS, N, D, K)) {
@@ -1220,14 +1224,14 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
             CHECK(screen_points(ctx, X, N, D, K, mu, Nk, S1, S2));
             CHECK(screen_end(ctx, K, slot));
             CHECK(update(&ctx->result()->scr[SC_DENSE]));
-            rc = screen_result(ctx, slot, &loglik_trace[t], &dense);
-            probe = dense;
-            left = skip = !dense ? 0 : skip == 0 ? 1 : skip < 16 ? 2 * skip : 16;
+            rc = screen_result(ctx, slot, &loglik_trace[t], N, &from);
+            probe = from < N;
+            left = skip = from == N ? 0 : skip == 0 ? 1 : skip < 16 ? 2 * skip : 16;
         }
-        if (dense && rc == GMM_OK) {
+        if (from < N && rc == GMM_OK) {
             CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, X, N));
-            CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
-            CHECK(accumulate_points(ctx, path, X, N, D, K, mu, Nk, S1, S2, slot));
+            if (from == 0) CHECK(zero_stats(ctx, D, K, Nk, S1, S2, slot));
+            CHECK(accumulate_points(ctx, path, X + from * D, N - from, D, K, mu, Nk, S1, S2, slot));
             CHECK(update(nullptr));
             ctx->last_path = path;
             rc = read_result(ctx, slot, &loglik_trace[t]);
@@ -1354,10 +1358,10 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
         if (screening) {
             CHECK(screen_points(ctx, ctx->xstage[b], cnt, D, K, mu, Nk, S1, S2));
             if (off + rows_per_chunk >= N) {
-                bool dense = false;
+                int64_t done = 0;
                 CHECK(screen_end(ctx, K, 0));
-                CHECK(screen_result(ctx, 0, loglik, &dense));
-                if (dense) {
+                CHECK(screen_result(ctx, 0, loglik, N, &done));
+                if (done < N) {
                     // broad posteriors: the dense kernels take the whole call, chunk by chunk again
                     screening = false;
                     CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, nullptr, 0));
@@ -1575,11 +1579,13 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
     // unless the screening has left the call to them.
     // (The lists have room for 16 pairs per point; a pair costs a quarter of the sweep at K = 1024.)
     const int* dense_if = nullptr;
+    // Pieces that the screening has done stay done: the others are cut at its pieces' edges, with a gate at each where there are several.
+    int64_t edge = N;
     if (screening) {
         dense_if = run_fp32_if = ctx->result()->scr + SC_DENSE;
         const float margin = index_only ? 0.f : 40.f, limit = ctx->scr_marks > 0.0 ? (float)ctx->scr_marks : 12.f;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, margin, m == 3 ? 4 : m, limit}));
-        const int64_t piece = screen_piece(ctx, N);
+        const int64_t piece = edge = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
             const int64_t cnt = (N - off < piece) ? (N - off) : piece;
             CHECK(prof_begin(ctx));
@@ -1589,6 +1595,8 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
         }
         KL(launch_center_fp32(ctx->stream, D, K, mu, ctx->center(), dense_if));
     }
+    int* const fallback = ctx->result()->scr + SC_FALLBACK;
+    const bool gates = screening && edge < N;
     if (tensor) {
         const TcBuffers tb = ctx->tc();
         const float limit = ctx->tc_cond_limit >= 0.f ? ctx->tc_cond_limit : 0.01f;
@@ -1596,8 +1604,8 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
         ctx->launches += 3;
         run_fp32_if = tb.flags + 3;
         if (screening) {
-            run_fp32_if = ctx->result()->scr + SC_FALLBACK;
-            KL(launch_screen_gate(ctx->stream, ctx->screen(), tb.flags + 3, ctx->result()->scr + SC_FALLBACK));
+            run_fp32_if = fallback;
+            KL(launch_screen_gate(ctx->stream, ctx->screen(), tb.flags + 3, fallback, 0, true));
         }
         KL(launch_ill_cache_tc(ctx->stream, D, mu, ctx->w2(), ctx->c2(), tb));
         const int64_t piece = ctx->tc_piece;
@@ -1612,8 +1620,9 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
         int* unc_count = reinterpret_cast<int*>(base + need - 256);
         int in_window = 0;
         int64_t win_start = 0;
-        for (int64_t off = 0; off < N; off += piece) {
-            const int64_t cnt = (N - off < piece) ? (N - off) : piece;
+        for (int64_t off = 0, cnt; off < N; off += cnt) {
+            cnt = std::min({piece, N - off, edge - off % edge});
+            if (gates && off > 0 && off % edge == 0) KL(launch_screen_gate(ctx->stream, ctx->screen(), tb.flags + 3, fallback, off / edge, false));
             if (in_window == 0) {
                 win_start = off;
                 CU(cudaMemsetAsync(unc_count, 0, sizeof(int), ctx->stream));
@@ -1625,7 +1634,7 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
                                 index_only));
             ctx->launches++;
             ++in_window;
-            if (in_window == WINDOW || off + piece >= N) {
+            if (in_window == WINDOW || off + cnt >= N) {
                 // The rows the refinement was not certain about, of the whole window: all K components exactly, by the FP32
                 // tile kernel.  (One launch per window: with a few hundred rows per piece a launch per piece is all latency.)
                 const int64_t win_rows = off + cnt - win_start;
@@ -1636,8 +1645,12 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
             CHECK(prof_end(ctx));
         }
     }
-    for (int64_t off = 0; off < N; off += SUPER_TILE) {
-        const int64_t cnt = (N - off < SUPER_TILE) ? (N - off) : SUPER_TILE;
+    for (int64_t off = 0, cnt; off < N; off += cnt) {
+        cnt = std::min({(int64_t)SUPER_TILE, N - off, edge - off % edge});
+        if (gates && off % edge == 0) {
+            run_fp32_if = fallback;
+            KL(launch_screen_gate(ctx->stream, ctx->screen(), nullptr, fallback, off / edge, !tensor && off == 0));
+        }
         KL(launch_topm_fp32(ctx->stream, X + off * D, cnt, D, K, mu, ctx->w2(), ctx->c2d(), ctx->center(), m, idx + off * m, resp ? resp + off * m : nullptr, run_fp32_if));
     }
     ctx->last_path = tensor || screening ? GMM_PATH_TENSOR : GMM_PATH_FP32;
@@ -1744,6 +1757,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_CENTROIDS, N, D, K)));
     CHECK(grow_buffer(ctx, &ctx->pl_scratch, &ctx->pl_scratch_bytes, pl_scratch_bytes(K), "the posting-list counters"));
     CHECK(grow_buffer(ctx, &ctx->km_scratch, &ctx->km_scratch_bytes, km_scratch_bytes(D, K), "the k-means partial sums"));
+    int64_t from = 0;                                             // points whose nearest centroid is known (then all sums are taken anew)
     if (screen_wanted(ctx, SCREEN_CENTROIDS, N, D, K)) {
         // through the screening path: the arg-max alone (margin 0), every point a lone pair of its cluster, and the statistics
         // of the pairs about the centroids give the new ones and the inertia
@@ -1779,6 +1793,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
             ctx->last_path = GMM_PATH_TENSOR;
             return GMM_OK;
         }
+        from = screen_left(ctx, r.scr, N);
     }
     // nearest centroid = top-1 component of a unit-variance, equal-weight mixture
     float* resp = reinterpret_cast<float*>(work);                 // [N], not used afterwards except as the builder's input
@@ -1803,11 +1818,11 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
         float* var_u = static_cast<float*>(ctx->km_unit);
         float* pi_u = var_u + KD;
         KL(launch_kmeans_unit_mixture(ctx->stream, D, K, pi_u, var_u));
-        CHECK(assign_topm_impl(ctx, X, N, D, K, pi_u, centroids, var_u, 1, assign, resp, true, true));       // the indices alone are used
+        CHECK(assign_topm_impl(ctx, X + from * D, N - from, D, K, pi_u, centroids, var_u, 1, assign + from, resp + from, true, true));      // the indices alone are used
     } else {
         KL(launch_kmeans_unit_params(ctx->stream, D, K, ctx->w2(), ctx->c2d()));
         KL(launch_center_fp32(ctx->stream, D, K, centroids, ctx->center()));
-        for (int64_t off = 0; off < N; off += SUPER_TILE) {
+        for (int64_t off = from; off < N; off += SUPER_TILE) {
             const int64_t cnt = (N - off < SUPER_TILE) ? (N - off) : SUPER_TILE;
             KL(launch_topm_fp32(ctx->stream, X + off * D, cnt, D, K, centroids, ctx->w2(), ctx->c2d(), ctx->center(), 1, assign + off, resp + off));
         }
@@ -1837,12 +1852,11 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
     CHECK(check_ptr(ctx, logp, 4, "logp"));
     DeviceGuard guard(ctx->device);
     CHECK(ensure_scratch(ctx, D, K, small_screen(ctx, SCREEN_DENSITIES, N, D, K)));
+    int64_t from = 0;
     if (screen_wanted(ctx, SCREEN_DENSITIES, N, D, K)) {
         // D <= 128: the same idea (csrc/em_screen.cu).  Costs per point as in screen_limit, without statistics.
         const double limit = ctx->scr_marks > 0.0 ? ctx->scr_marks
                              : std::fmin(14.0, std::fmax(1.5, 0.9 * (0.03 + 1.9e-4 * K * D - screen_fixed(D, K)) / (0.05 + 0.0007 * D)));
-        bool dense = false;
-        double total = 0.0;
         CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {X, N, 40.f, 1, (float)limit}));
         const int64_t piece = screen_piece(ctx, N);
         for (int64_t off = 0; off < N; off += piece) {
@@ -1852,15 +1866,16 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
             CHECK(prof_end(ctx));
         }
         CHECK(screen_end(ctx, K, 0));
-        CHECK(screen_result(ctx, 0, &total, &dense));
-        if (!dense) {
+        double total = 0.0;
+        CHECK(screen_result(ctx, 0, &total, N, &from));
+        if (from == N) {
             if (loglik) *loglik = total;
             return GMM_OK;
         }
     }
     KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), &ctx->result()->status));
     if ((size_t)K * D > ((size_t)1 << 12)) ctx->launches++;
-    CU(cudaMemsetAsync(&ctx->result()->ll[0], 0, 8, ctx->stream));
+    if (from == 0) CU(cudaMemsetAsync(&ctx->result()->ll[0], 0, 8, ctx->stream));
     // Wide data with sparse posteriors: the EM step's screening route without its statistics.  Every component with a weight
     // is listed, one sweep over the leading fp16 product marks the pairs that can come within 2^-40 of a point's best, the
     // filter drops those that the final threshold rules out, and a warp per point evaluates the rest exactly: their
@@ -1925,7 +1940,7 @@ int gmm_score_samples(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, con
         }
     }
     // the log-sum-exp kernel of the FP32 path, one super-tile at a time; its per-point values go out instead of into an M-step
-    for (int64_t off = 0; off < N; off += SUPER_TILE) {
+    for (int64_t off = from; off < N; off += SUPER_TILE) {
         const int64_t cnt = (N - off < SUPER_TILE) ? (N - off) : SUPER_TILE;
         CHECK(prof_begin(ctx));
         KL(launch_lse_fp32(ctx->stream, X + off * D, cnt, D, K, mu, ctx->w2(), ctx->c2d(), ctx->center(), ctx->logZ2(), ctx->llpart()));
@@ -2011,11 +2026,11 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
                 CHECK(prof_end(ctx));
             }
         }
-        bool dense = false;
         double total = 0.0;
+        int64_t done = 0;                                    // (all groups or none)
         CHECK(screen_end(ctx, K, 0));
-        CHECK(screen_result(ctx, 0, &total, &dense));
-        if (!dense) {
+        CHECK(screen_result(ctx, 0, &total, N, &done));
+        if (done == N) {
             if (loglik) *loglik = total;
             return GMM_OK;
         }

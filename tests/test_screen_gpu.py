@@ -313,3 +313,50 @@ def test_screen_of_assignments_where_the_rule_takes_either_way(fg, monkeypatch, 
         weight = np.exp(want - np.logaddexp.reduce(lj, axis=1)[:, None]) > 1e-5     # (ranks without weight keep the order of a selection pass)
         assert np.all((got >= want - (np.abs(want) * 2e-6 + 1e-3))[weight])
     assert np.abs(out[0][1] - out[1][1]).max() <= 2e-4
+
+
+@pytest.mark.parametrize("K", [128, 48])
+@pytest.mark.parametrize("piece", [15, 5])
+def test_screen_keeps_the_pieces_that_are_done(fg, monkeypatch, K, piece):
+    """A region of broad posteriors that the look ahead does not meet, in the last or in a middle one of 16 pieces of 768 points: the pieces
+    before it stay as they are, the dense kernels take the others, and every output is that of one pass over all points."""
+    from oracle.kmeans import kmeans_step
+
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "10")
+    monkeypatch.setenv("GMM_SCREEN_PIECE", "768")
+    N, D = 16 * 768 + 100, 16
+    _, pi, mu, var = _mixture(N, D, K, 51)
+    mu[K // 2:], var[:] = 12.0 + 0.05 * mu[K // 2:], 1.0
+    rng = np.random.default_rng(5)
+    X = (mu[rng.integers(0, K // 2, N)] + rng.normal(size=(N, D))).astype(np.float32)
+    first = piece * 768 + 450                              # (the rows that are looked at lie 384 into a piece)
+    X[first:first + 300] = 12.0 + rng.normal(size=(300, D)).astype(np.float32)
+    ref = orc.em_step(X, pi, mu, var)
+    lj = np.asarray(orc.log_joint(X, pi, mu, var), np.float64)
+    lz = np.logaddexp.reduce(lj, axis=1)
+    a_r, _, _, inertia_r, gap = kmeans_step(X, mu.astype(np.float64))
+    with fg.Context(0) as c:
+        x, p = _t(X), [_t(pi), _t(mu), _t(var)]
+        got = c.gmm_em_step(x, *p)
+        assert c.gmm_last_exact_count() < K                # (the dense kernels had the last word)
+        assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3])
+        assert_stats_close(N, data_scale(X), [v.cpu().numpy() for v in got[:3]], ref[:3], f"K={K} piece={piece}")
+        q = [v.clone() for v in p]
+        trace, done = c.gmm_fit(x, *q, 2)
+        want = orc.fit(X, pi, mu, var, 2, var_floor=1e-6)["trace"]
+        assert done == 2 and np.all(np.abs(trace - want) <= 1e-5 * np.abs(want))
+        logp, total = c.gmm_score_samples(x, *p)
+        assert np.all(np.abs(logp.cpu().numpy() - lz) <= 1e-5 * np.abs(lz) + 1e-4) and abs(total - lz.sum()) <= 1e-5 * abs(lz.sum())
+        a, new, counts, inertia = c.gmm_kmeans_step(x, p[1])
+        a = a.cpu().numpy()
+        assert np.all((a == a_r) | (gap <= 1e-2)) and np.array_equal(counts.cpu().numpy(), np.bincount(a, minlength=K))
+        assert abs(inertia - inertia_r) <= 1e-5 * inertia_r
+        for k in np.unique(a)[:20]:
+            np.testing.assert_allclose(new[k].cpu().numpy(), X[a == k].astype(np.float64).mean(0), rtol=0, atol=1e-4)
+        for m in (1, 2):
+            idx, resp = (v.cpu().numpy() for v in c.gmm_assign_topm(x, *p, m))
+            at = np.take_along_axis(lj, idx.astype(np.int64), axis=1)
+            assert np.all(at >= np.sort(lj, axis=1)[:, ::-1][:, :m] - 1e-3) and np.abs(resp - np.exp(at - lz[:, None])).max() <= 2e-4
+        host = c.gmm_em_step_host(X, pi, mu, var)
+        assert abs(host[3] - ref[3]) <= 1e-5 * abs(ref[3])
+        assert_stats_close(N, data_scale(X), host[:3], ref[:3], "host")

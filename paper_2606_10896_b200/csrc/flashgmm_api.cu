@@ -809,16 +809,21 @@ int zero_stats(gmm_ctx* ctx, int D, int K, double* Nk, double* S1, double* S2, i
     return GMM_OK;
 }
 
+// Pinned memory for the result block (and for the verdicts on two chunks of gmm_em_step_host).
+int pinned_block(gmm_ctx* ctx) {
+    if (ctx->pinned) return GMM_OK;
+    void* h = nullptr;
+    if (cudaMallocHost(&h, 3 * sizeof(DevResult)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(ctx, GMM_ENOMEM, "cannot allocate %zu bytes of pinned memory", 3 * sizeof(DevResult));
+    }
+    ctx->pinned = static_cast<DevResult*>(h);
+    return GMM_OK;
+}
+
 // The result block, read through pinned memory; synchronises.
 int read_back(gmm_ctx* ctx, DevResult* r) {
-    if (!ctx->pinned) {
-        void* h = nullptr;
-        if (cudaMallocHost(&h, sizeof(DevResult)) != cudaSuccess) {
-            cudaGetLastError();
-            return fail(ctx, GMM_ENOMEM, "cannot allocate %zu bytes of pinned memory", sizeof(DevResult));
-        }
-        ctx->pinned = static_cast<DevResult*>(h);
-    }
+    CHECK(pinned_block(ctx));
     CU(cudaMemcpyAsync(ctx->pinned, ctx->result(), sizeof(DevResult), cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
     *r = *ctx->pinned;
@@ -1322,64 +1327,88 @@ int gmm_em_step_host(gmm_ctx* ctx, const float* X_host, int64_t N, int D, int K,
     double* Nk = ctx->stats();
     double* S1 = Nk + K;
     double* S2 = S1 + KD;
-    int64_t rows_per_chunk = (int64_t)(ctx->xstage_bytes / ((size_t)D * 4));
-    if (D <= 128) {
-        // What is left when the last copy ends is the last chunk's kernels: a sixteenth of the data, but no less than 8 MiB (150 us of
-        // copying, about what a chunk's launches take).  1M x 128: 9.82 ms with chunks of 128 MiB.
-        const int64_t rows = ((N + 15) / 16 + 255) / 256 * 256, least = ((int64_t)8 << 20) / ((int64_t)D * 4);
-        const int64_t want = rows > least ? rows : least;
-        if (want < rows_per_chunk) rows_per_chunk = want;
-    }
-    if (rows_per_chunk < 1) return fail(ctx, GMM_EINVAL, "D too large for the staging buffer");
+    const int64_t full = (int64_t)(stage_bytes / ((size_t)D * 4));
+    if (full < 1) return fail(ctx, GMM_EINVAL, "D too large for the staging buffer");
+    // Rows per chunk.  What is left when the last copy ends is the last chunk's kernels, so D <= 128 takes a sixteenth of the data, but no
+    // less than a chunk's launches take as long as: 8 MiB (150 us of copying) with the screening, 32 MiB with the dense kernels, whose
+    // smallest call takes 165 us (200K x 32, K = 64 with broad posteriors: 0.95 ms in chunks of 8 MiB, 0.81 in one).
+    // 1M x 128: 9.82 ms with chunks of 128 MiB.
+    auto chunk_rows = [&](bool screened) {
+        if (D > 128) return full;
+        const int64_t rows = ((N + 15) / 16 + 255) / 256 * 256, least = ((int64_t)(screened ? 8 : 32) << 20) / ((int64_t)D * 4);
+        return std::min(full, std::max(rows, least));
+    };
+    bool screening = screen_wanted(ctx, SCREEN_STEPS, N, D, K);
     // The first chunk is on its way before the parameters are prepared: on wide data the automatic choice of the mode
     // looks at its first rows.  (The copy stream must not overtake work of an earlier call that still reads the buffer.)
     CU(cudaEventRecord(ctx->ev_done[0], ctx->stream));
     CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_done[0], 0));
-    const int64_t cnt0 = N < rows_per_chunk ? N : rows_per_chunk;
-    CU(cudaMemcpyAsync(ctx->xstage[0], X_host, (size_t)cnt0 * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
-    CU(cudaEventRecord(ctx->ev_copied[0], ctx->copy_stream));
-    CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[0], 0));
-    bool screening = screen_wanted(ctx, SCREEN_STEPS, N, D, K);
-    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {ctx->xstage[0], cnt0, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
-    else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], cnt0));
+    struct Chunk { int64_t off, cnt; } chunk[2];                     // what the two buffers hold
+    auto copy_chunk = [&](int b, int64_t off) -> int {
+        chunk[b] = {off, std::min(N - off, chunk_rows(screening))};
+        CU(cudaMemcpyAsync(ctx->xstage[b], X_host + off * D, (size_t)chunk[b].cnt * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
+        CU(cudaEventRecord(ctx->ev_copied[b], ctx->copy_stream));
+        CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[b], 0));
+        return GMM_OK;
+    };
+    CHECK(copy_chunk(0, 0));
+    if (screening) CHECK(screen_begin(ctx, D, K, pi, mu, var, false, {ctx->xstage[0], chunk[0].cnt, 40.f, 1, (float)screen_limit(ctx, SCREEN_STEPS, N, D, K)}));
+    else CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, ctx->xstage[0], chunk[0].cnt));
     CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
-    int c = 0;                                       // chunks copied so far: they take the buffers in turn
-    bool copied = true;                              // (the first one already is)
-    for (int64_t off = 0; off < N; off += rows_per_chunk, ++c) {
-        const int b = c & 1;
-        const int64_t cnt = (N - off < rows_per_chunk) ? (N - off) : rows_per_chunk;
-        if (!copied) {
-            if (c >= 2) CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_done[b], 0));
-            CU(cudaMemcpyAsync(ctx->xstage[b], X_host + off * D, (size_t)cnt * D * 4, cudaMemcpyHostToDevice, ctx->copy_stream));
-            CU(cudaEventRecord(ctx->ev_copied[b], ctx->copy_stream));
-            CU(cudaStreamWaitEvent(ctx->stream, ctx->ev_copied[b], 0));
-        }
-        copied = false;
+    // A chunk's screening leaves its verdict in pinned memory.  It is looked at before the buffer is filled again, while the next chunk is on
+    // its way, so X crosses the bus once: a chunk that is not done goes to the dense kernels from its buffer, with all that follow (the
+    // next one's screening has done nothing then).
+    if (screening) CHECK(pinned_block(ctx));
+    int64_t pieces = 0;                                              // done before the chunk in question
+    auto kernels = [&](int b, int64_t from) -> int {
         if (screening) {
-            CHECK(screen_points(ctx, ctx->xstage[b], cnt, D, K, mu, Nk, S1, S2));
-            if (off + rows_per_chunk >= N) {
-                int64_t done = 0;
-                CHECK(screen_end(ctx, K, 0));
-                CHECK(screen_result(ctx, 0, loglik, N, &done));
-                if (done < N) {
-                    // broad posteriors: the dense kernels take the whole call, chunk by chunk again
-                    screening = false;
-                    CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, nullptr, 0));
-                    CHECK(zero_stats(ctx, D, K, Nk, S1, S2, 0));
-                    off = -rows_per_chunk;
-                }
-            }
-        } else {
-            CHECK(accumulate_points(ctx, path, ctx->xstage[b], cnt, D, K, mu, Nk, S1, S2, 0));
+            CHECK(screen_points(ctx, ctx->xstage[b], chunk[b].cnt, D, K, mu, Nk, S1, S2));
+            CU(cudaMemcpyAsync(ctx->pinned[1 + b].scr, ctx->result()->scr, sizeof(ctx->pinned->scr), cudaMemcpyDeviceToHost, ctx->stream));
+        } else if (from < chunk[b].cnt) {
+            CHECK(accumulate_points(ctx, path, ctx->xstage[b] + from * D, chunk[b].cnt - from, D, K, mu, Nk, S1, S2, 0));
         }
         CU(cudaEventRecord(ctx->ev_done[b], ctx->stream));
+        return GMM_OK;
+    };
+    auto settle = [&](int b, bool next) -> int {                     // next: the other buffer's kernels are enqueued
+        if (!screening) return GMM_OK;
+        CU(cudaEventSynchronize(ctx->ev_done[b]));
+        int ctl[SC_WORDS];
+        std::memcpy(ctl, ctx->pinned[1 + b].scr, sizeof(ctl));
+        ctl[SC_DONE] -= (int)pieces;
+        const int64_t from = screen_left(ctx, ctl, chunk[b].cnt), piece = screen_piece(ctx, chunk[b].cnt);
+        if (from == chunk[b].cnt) {
+            pieces += (from + piece - 1) / piece;
+            return GMM_OK;
+        }
+        screening = false;
+        CHECK(screen_end(ctx, K, 0));                                // (the log-likelihood of what is done)
+        CHECK(prepare_and_choose(ctx, N, D, K, pi, mu, var, &path, nullptr, 0));
+        CHECK(kernels(b, from));
+        if (next) CHECK(kernels(b ^ 1, 0));
+        return GMM_OK;
+    };
+    CHECK(kernels(0, 0));
+    int c = 1;                                                       // chunks copied so far: they take the buffers in turn
+    for (int64_t off = chunk[0].cnt; off < N; ++c) {
+        const int b = c & 1;
+        if (c >= 2) {
+            CHECK(settle(b, true));
+            CU(cudaStreamWaitEvent(ctx->copy_stream, ctx->ev_done[b], 0));
+        }
+        CHECK(copy_chunk(b, off));
+        CHECK(kernels(b, 0));
+        off += chunk[b].cnt;
     }
+    if (c >= 2) CHECK(settle(c & 1, true));
+    CHECK(settle((c - 1) & 1, false));
     CU(cudaMemcpyAsync(Nk_host, Nk, (size_t)K * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaMemcpyAsync(S1_host, S1, KD * 8, cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaMemcpyAsync(S2_host, S2, KD * 8, cudaMemcpyDeviceToHost, ctx->stream));
     if (screening) {
-        CU(cudaStreamSynchronize(ctx->stream));
-        return GMM_OK;
+        int64_t from = 0;
+        CHECK(screen_end(ctx, K, 0));
+        return screen_result(ctx, 0, loglik, N, &from);
     }
     ctx->last_path = path;
     return read_result(ctx, 0, loglik);

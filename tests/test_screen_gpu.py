@@ -360,3 +360,25 @@ def test_screen_keeps_the_pieces_that_are_done(fg, monkeypatch, K, piece):
         host = c.gmm_em_step_host(X, pi, mu, var)
         assert abs(host[3] - ref[3]) <= 1e-5 * abs(ref[3])
         assert_stats_close(N, data_scale(X), host[:3], ref[:3], "host")
+
+
+@pytest.mark.parametrize("D,K", [(32, 64), (96, 48)])
+@pytest.mark.parametrize("broad", [(0, 0), (0, 270_001), (150_000, 171_000), (255_000, 270_001), (70_000, 91_000)])
+def test_host_streaming_takes_the_data_once_whatever_the_verdict(fg, D, K, broad):
+    """Chunks of 8 MiB (5 of them, 13): sparse data, broad data, and a broad region in the second, a middle and the last chunk; each call gives the statistics of
+    one pass, the same bits when repeated."""
+    N = 270_001
+    _, pi, mu, var = _mixture(100, D, K, 61)
+    mu[K // 2:], var[:] = 0.02 * mu[K // 2:], 1.0
+    rng = np.random.default_rng(6)
+    X = rng.normal(size=(N, D)).astype(np.float32)
+    X += mu[rng.integers(0, K // 2, N)]
+    X[broad[0]:broad[1]] = rng.normal(size=(broad[1] - broad[0], D)).astype(np.float32)
+    ref = orc.em_step(X, pi, mu, var)
+    with fg.Context(0) as c:
+        out = [c.gmm_em_step_host(X, pi, mu, var) for _ in range(2)]
+        assert (c.gmm_last_exact_count() == K) == (broad[1] == 0)
+    for u, v in zip(*out):
+        assert np.array_equal(u, v)
+    assert abs(out[0][3] - ref[3]) <= 1e-5 * abs(ref[3])
+    assert_stats_close(N, data_scale(X), out[0][:3], ref[:3], f"K={K} broad={broad}")

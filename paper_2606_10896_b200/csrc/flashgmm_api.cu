@@ -46,7 +46,7 @@ struct ScratchLayout {
 };
 
 // planes: include the fp16 planes of Y (tensor path only; 2 x TC_YPLANE_BYTES, placed last so that no other offset moves)
-ScratchLayout scratch_layout(int D, int K, bool planes) {
+ScratchLayout scratch_layout(int D, int K, bool planes, bool lists = true) {
     ScratchLayout L;
     const size_t KD = (size_t)K * D;
     size_t off = 0;
@@ -155,7 +155,7 @@ ScratchLayout scratch_layout(int D, int K, bool planes) {
         L.w_yhi = take((size_t)WIDE_PIECE * wp.Dpad * 4);
         L.w_ylo = take((size_t)WIDE_PIECE * wp.Dpad * 4);
     }
-    L.scr = L.tc && planes && screen_supports(D, K);
+    L.scr = L.tc && planes && lists && screen_supports(D, K);
     L.s_sd = L.s_gd = L.s_dimpart = L.s_prm = L.s_key = L.s_p = L.s_blk = L.s_compof = L.s_probe = L.s_n2 = L.s_ptoff = L.s_ptcnt = L.s_words = L.s_spill = L.s_ids = L.s_val = L.s_srt = L.s_counts = L.s_totals = L.s_off = L.s_segoff = L.s_part = L.s_ll = L.s_ovf = 0;
     if (L.scr) {
         static_assert((size_t)SCR_PIECE * 256 <= TC_YPLANE_BYTES, "the plane of the screening path lies in that of the tile kernel");
@@ -217,6 +217,7 @@ struct gmm_ctx {
     size_t km_scratch_bytes = 0;
     size_t pl_scratch_bytes = 0;
     bool capPlanes = false;    // the scratch layout in force includes the tensor path's planes of Y
+    bool cap_short = false;    // there was no memory for the screening path's part of the scratch of (capD, capK)
     ScratchLayout lay{};
     int tc_Q = 0;              // resident clusters of the tensor-path kernel for (capD, capK)
     float tc_cond_limit = -1.f;      // < 0: automatic, tc_cond_scale * sqrt(N / K)
@@ -452,12 +453,14 @@ bool small_screen(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t
 }
 
 int ensure_scratch(gmm_ctx* ctx, int D, int K, bool small = false) {
-    bool planes = (tc_assign_supports(D, K) || wide_supports(D, K)) &&
-                  (ctx->path == GMM_PATH_TENSOR || (ctx->path == GMM_PATH_AUTO && (auto_wants_planes(D, K) || small)));
+    if (D != ctx->capD || K != ctx->capK) ctx->cap_short = false;
+    const bool dense_planes = (tc_assign_supports(D, K) || wide_supports(D, K)) &&
+                              (ctx->path == GMM_PATH_TENSOR || (ctx->path == GMM_PATH_AUTO && auto_wants_planes(D, K)));
+    bool planes = dense_planes || (small && !ctx->cap_short && ctx->path == GMM_PATH_AUTO && tc_assign_supports(D, K));
     // (K < 64: once there the planes stay, whatever the next call's number of points says)
     if (ctx->scratch && D == ctx->capD && K == ctx->capK && ctx->path == GMM_PATH_AUTO && !auto_wants_planes(D, K) && ctx->capPlanes) planes = true;
     if (ctx->scratch && D == ctx->capD && K == ctx->capK && planes == ctx->capPlanes) return GMM_OK;
-    const ScratchLayout L = scratch_layout(D, K, planes);
+    ScratchLayout L = scratch_layout(D, K, planes, !ctx->cap_short);
     if (ctx->scratch) {
         // The status word moves with the layout: what asynchronous calls may have left in it is kept on the host.
         int st = 0;
@@ -473,6 +476,14 @@ int ensure_scratch(gmm_ctx* ctx, int D, int K, bool small = false) {
         }
         void* p = nullptr;
         cudaError_t e = cudaMalloc(&p, L.total);
+        if (e != cudaSuccess && L.scr) {
+            // no room for the screening path's lists (and, for K < 64, its planes): the shape goes without
+            cudaGetLastError();
+            ctx->cap_short = true;
+            planes = dense_planes;
+            L = scratch_layout(D, K, planes, false);
+            e = cudaMalloc(&p, L.total);
+        }
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(ctx, GMM_ENOMEM, "cannot allocate %zu bytes of scratch: %s", L.total, cudaGetErrorString(e));

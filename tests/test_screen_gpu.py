@@ -382,3 +382,32 @@ def test_host_streaming_takes_the_data_once_whatever_the_verdict(fg, D, K, broad
         assert np.array_equal(u, v)
     assert abs(out[0][3] - ref[3]) <= 1e-5 * abs(ref[3])
     assert_stats_close(N, data_scale(X), out[0][:3], ref[:3], f"K={K} broad={broad}")
+
+
+@pytest.mark.parametrize("D,K,N,left", [(128, 1024, 3000, 800), (96, 48, 200_000, 800)])
+def test_screen_does_without_where_memory_is_short(fg, D, K, N, left):
+    """Room (in MiB) for what the dense kernels need, not for the lists on top: the call runs, as it does without a screening path, and the next
+    shape is screened again when there is room."""
+    X, pi, mu, var = _mixture(N, D, K, 71)
+    ref = orc.em_step(X, pi, mu, var)
+    args = [_t(a) for a in (X, pi, mu, var)]
+    small = [_t(a) for a in _mixture(2000, 16, 64, 72)]
+    with fg.Context(0) as c:
+        c.gmm_em_step(*small)                              # (what the first calls allocate besides)
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        hog = torch.empty(torch.cuda.mem_get_info()[0] - (left << 20) + int(fg.lib.gmm_scratch_bytes(16, 64)), dtype=torch.uint8, device=DEV)
+        launches = []
+        for _ in range(2):
+            before = c.gmm_launch_count()
+            got = c.gmm_em_step(*args)
+            launches.append(c.gmm_launch_count() - before)
+            assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3])
+            assert_stats_close(N, data_scale(X), [v.cpu().numpy() for v in got[:3]], ref[:3], "short of memory")
+        del hog, got
+        torch.cuda.empty_cache()
+        c.gmm_em_step(*small)
+        assert c.gmm_last_exact_count() == 64
+        before = c.gmm_launch_count()
+        c.gmm_em_step(*args)
+        assert c.gmm_last_exact_count() == K and launches[0] == launches[1] != c.gmm_launch_count() - before

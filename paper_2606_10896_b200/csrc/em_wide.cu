@@ -107,6 +107,7 @@ struct LseParams {
                          // listed components with the largest upper bounds (the bound and the component's position)
     int pre_pass;        // 1: before a tile's sweep proper, the groups from hi_group on are swept once for their lower bounds only
     int* ctl;
+    int test_silent;     // >= 0: the follower of that pair of CTAs asks for nothing (time-out test)
 };
 
 // NTOP: how many of a point's largest approximate log2 z the sweep reports (2 for the EM step's exact normaliser, m + 2 for
@@ -153,6 +154,16 @@ __device__ __forceinline__ void pair_mma(uint32_t d_tmem, uint64_t a, uint64_t b
 __device__ __forceinline__ void pair_commit(uint32_t bar) {          // arrives at the barrier of this offset in both CTAs
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
+__device__ __forceinline__ int pair_peer(const int* v) {             // the other CTA's copy, read by the leader
+    uint32_t at;
+    int r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 1;" : "=r"(at) : "r"(smem_u32(v)));
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(r) : "r"(at) : "memory");
+    return r;
+}
+__device__ __forceinline__ void pair_complete_tx(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.complete_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void pair_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -164,7 +175,7 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     __shared__ uint32_t tmem_base_s;
-    __shared__ int abort_s, drain_s;
+    __shared__ int abort_s, drain_s, issued_s;               // issued_s: stages that this CTA has asked for
     volatile int* abort_flag = &abort_s;
     volatile int* drain_flag = &drain_s;
     float2* merge_s = reinterpret_cast<float2*>(smem + L_MERGE);
@@ -443,7 +454,8 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
                 const float s = s_run * fast_ex2(m_run - m) + o.y * fast_ex2(o.x - m);
 #pragma unroll
                 for (int j = 0; j < NTOP; ++j) tl.insert(top_s[pt][j], __float_as_int(top_s[pt][NTOP + j]));
-                if (row < p.n && !*abort_flag) {
+                // (also after an expired wait: the kernels behind this one take the positions as they find them)
+                if (row < p.n) {
                     const double lz = cref + (double)m + (double)log2f(s);
                     p.logz[row] = lz;
                     float* tp = p.top + row * (2 * NTOP);
@@ -477,7 +489,7 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
         if (elect_one()) {
             uint32_t slot = 0, parity = 1;                   // of the next stage; the phase whose end frees its slot
             int64_t issued = 0;
-            bool ok = true;
+            bool ok = p.test_silent != (int)pair || rank == 0;
             const uint64_t pol_keep = l2_policy_evict_last();
             const uint32_t full = pair_bar(BAR(LB_FULL));
             auto stage = [&](const CUtensorMap* my, const CUtensorMap* mp, int32_t yrow, int32_t prow, int32_t z) -> bool {
@@ -502,12 +514,7 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
                     }
                 }
             }
-            // after an abort: loads in flight must land before the CTA may exit (they take microseconds; their barrier may be
-            // the other CTA's, whose state is not known here)
-            if (!ok || *abort_flag) {
-                const unsigned long long t0 = gtime();
-                while (gtime() - t0 < 2000000ull) __nanosleep(1000);
-            }
+            issued_s = (int)issued;
         }
         __syncwarp();
     } else if (rank == 0) {
@@ -577,6 +584,20 @@ lse_wide_kernel(const LseParams p, const __grid_constant__ CUtensorMap tm_yhi, c
     }
 
     fence_before();
+    __syncthreads();
+    pair_sync();                                             // (all roles of both CTAs are out)
+    // After an abort the loads in flight must have landed before either CTA leaves.  A stage's bytes, both CTAs', are counted by the
+    // leader's barrier; what only one of them asked for is made up here: an arrival for the follower's, the bytes that will not
+    // come for the leader's.  Stages that lie a ring behind the last one have been used.
+    if (rank == 0 && tid == 0 && (abort_s != 0 || pair_peer(&abort_s) != 0)) {
+        const int mine = issued_s, theirs = pair_peer(&issued_s), all = mine > theirs ? mine : theirs;
+        for (int s = all > L_SLOTS ? all - L_SLOTS : 0; s < all; ++s) {
+            const uint32_t bar = BAR(LB_FULL + s % L_SLOTS);
+            if (s >= mine) bar_expect_tx(bar, L_STAGE);
+            else if (s >= theirs) pair_complete_tx(bar, L_STAGE);
+            bar_wait(bar, (uint32_t)(s / L_SLOTS) & 1u, drain_flag, p.status, true);
+        }
+    }
     __syncthreads();
     pair_sync();                                             // (neither CTA leaves while the other may still use its memory)
     if (warp == WT_MMA) {
@@ -2919,7 +2940,7 @@ cudaError_t launch_lse_wide(cudaStream_t s, int64_t n, int D, int K, int Kg, int
     p.screen = screen;
     p.scr = reinterpret_cast<const float2*>(wb.scr);
     p.scr_e = wb.scr_e; p.scr_mask = wb.scr_mask; p.slot_of = wb.slot_of; p.n2 = wb.n2; p.cand = wb.cand;
-    p.cand_words = (n_slots + 31) / 32; p.scr_group = Kgp / 256; p.ctl = wb.ctl;
+    p.cand_words = (n_slots + 31) / 32; p.scr_group = Kgp / 256; p.ctl = wb.ctl; p.test_silent = wb.test_silent;
     p.hi_group = 0x7fffffff; p.hi_end = 0x7fffffff; p.pre_pass = 0;
     p.topm = 0;
     if (topm > 0) {                                          // the assignment by screening: as the EM step's screening mode

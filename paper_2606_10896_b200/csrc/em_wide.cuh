@@ -97,6 +97,7 @@ struct WideBuffers {
                     //      FP32 kernels evaluate the sub-mixture densely, [2] nonzero: the pairs are evaluated one by one,
                     //      [4] entries of pair_val handed out, [5] nonzero: pair_val ran out (the statistics kernel evaluates
                     //      its pairs itself)
+    int test_silent;      // (time-out test, see LseParams)
 };
 
 bool wide_supports(int D, int K);

@@ -249,7 +249,7 @@ struct gmm_ctx {
     double scr_marks = -1.0;         // GMM_SCREEN_MARKS: marked pairs per point up to which the screening path is taken (D <= 128;
                                      // 0: never, < 0: from the measured costs, see screen_limit)
     int64_t scr_piece = 0;           // GMM_SCREEN_PIECE: points per round of launches of the screening path (0: screen_piece)
-    int scr_test_silent = -1;        // GMM_SCREEN_TEST_SILENT (time-out test)
+    int scr_test_silent = -1, wide_test_silent = -1;      // GMM_SCREEN_TEST_SILENT, GMM_WIDE_TEST_SILENT (time-out tests)
     DevResult* pinned = nullptr;     // where the result block is read back to
     int scr_active = 0;              // components with a weight, when the most recent step took the screening path; else 0
     int sticky_status = 0;           // status bits read off the device but not yet reported (see ensure_scratch)
@@ -392,6 +392,7 @@ struct gmm_ctx {
         b.rec = reinterpret_cast<unsigned*>(scratch + lay.w_rec);
         b.rec_cnt = reinterpret_cast<int*>(scratch + lay.w_reccnt);
         b.rec_thr = reinterpret_cast<float*>(scratch + lay.w_recthr);
+        b.test_silent = wide_test_silent;
         return b;
     }
 };
@@ -994,6 +995,7 @@ int gmm_create(gmm_ctx** out, int device, void* cuda_stream) {
     if (const char* e = std::getenv("GMM_TC_COND_LIMIT")) ctx->tc_cond_limit = (float)std::atof(e);
     if (const char* e = std::getenv("GMM_SCREEN_MARKS")) ctx->scr_marks = std::atof(e);
     if (const char* e = std::getenv("GMM_SCREEN_TEST_SILENT")) ctx->scr_test_silent = std::atoi(e);
+    if (const char* e = std::getenv("GMM_WIDE_TEST_SILENT")) ctx->wide_test_silent = std::atoi(e);
     if (const char* e = std::getenv("GMM_SCREEN_PIECE")) {
         const long long v = std::atoll(e);
         if (v >= SCR_TILE && v <= SCR_PIECE) ctx->scr_piece = v / SCR_TILE * SCR_TILE;

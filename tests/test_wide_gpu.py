@@ -534,3 +534,23 @@ def test_wide_path_at_its_largest_shape(fg, ctx):
     idx_g, resp_g = idx[rows].cpu().numpy(), resp[rows].cpu().numpy()
     idx_r, resp_r, next_r = orc.topm(Xs, pi, mu, var, 4)
     assert_topm_matches(idx_g, resp_g, idx_r, resp_r, next_r, oracle_resp_at(orc, Xs, pi, mu, var, idx_g), what="largest shape, top-4")
+
+
+def test_wide_wait_that_runs_out(fg, monkeypatch):
+    """The second CTA of a pair asks for no loads.  The waits of both run out (2 s), what the first one has asked for is waited for, both leave
+    together, and the call - the next synchronising one after an assignment - says so.  A fresh context computes the same step."""
+    N, D, K = 3000 + 11, 200, 70
+    X, pi, mu, var = _clustered(np.random.default_rng(79), N, D, K)
+    monkeypatch.setenv("GMM_WIDE_TEST_SILENT", "1")
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_TENSOR)
+        for call in (lambda: c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var)),
+                     lambda: (c.gmm_assign_topm(_t(X), _t(pi), _t(mu), _t(var), 2), c.gmm_sync_status())):
+            with pytest.raises(fg.GmmError) as e:
+                call()
+            assert e.value.code == fg.GMM_ETIMEOUT
+        c.gmm_sync_status()
+    monkeypatch.delenv("GMM_WIDE_TEST_SILENT")
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_TENSOR)
+        _step_and_check(fg, c, X, pi, mu, var, "after calls that timed out")

@@ -536,6 +536,22 @@ def test_wide_path_at_its_largest_shape(fg, ctx):
     assert_topm_matches(idx_g, resp_g, idx_r, resp_r, next_r, oracle_resp_at(orc, Xs, pi, mu, var, idx_g), what="largest shape, top-4")
 
 
+def test_wide_assignment_more_pairs_than_the_list_holds(fg, monkeypatch):
+    """As test_wide_screen_mode_more_pairs_than_stored_values, for the assignments and the log-densities: the points whose pairs find no room in the
+    list are taken one warp each."""
+    monkeypatch.setenv("GMM_WIDE_MODE", "screen")
+    monkeypatch.setenv("GMM_WIDE_SPARSE", "2")
+    N, D, K = 40_000, 200, 130
+    X, pi, mu, var = _clustered(np.random.default_rng(78), N, D, K, sep=0.01)
+    lz = orc.responsibilities(X, pi, mu, var)[1]
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_TENSOR)
+        _assign_and_check(fg, c, X, pi, mu, var, 1, "hard assignment, list full", indices_only=True)
+        _assign_and_check(fg, c, X, pi, mu, var, 4, "top-4, list full")
+        logp, total = c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var))
+    assert np.all(np.abs(logp.cpu().numpy() - lz) <= 1e-5 * np.abs(lz) + 1e-4) and abs(total - lz.sum()) <= 1e-5 * abs(lz.sum())
+
+
 def test_wide_wait_that_runs_out(fg, monkeypatch):
     """The second CTA of a pair asks for no loads.  The waits of both run out (2 s), what the first one has asked for is waited for, both leave
     together, and the call - the next synchronising one after an assignment - says so.  A fresh context computes the same step."""

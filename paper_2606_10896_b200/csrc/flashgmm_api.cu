@@ -947,8 +947,9 @@ int screen_end(gmm_ctx* ctx, int K, int slot) {
 
 // Synchronising read of the log-likelihood and the status word for n points.  *from: the point from which on the caller has to run the
 // dense kernels (n: none).  What lies before is in the outputs and in the log-likelihood already.
+// (Never all of them where the verdict is dense: gmm_fisher_vectors counts pieces of its groups.)
 int64_t screen_left(const gmm_ctx* ctx, const int* ctl, int64_t n) {
-    return ctl[SC_DENSE] == 0 ? n : std::min(n, (int64_t)ctl[SC_DONE] * screen_piece(ctx, n));
+    return ctl[SC_DENSE] == 0 ? n : std::min(n - 1, (int64_t)ctl[SC_DONE] * screen_piece(ctx, n));
 }
 int screen_result(gmm_ctx* ctx, int slot, double* loglik, int64_t n, int64_t* from) {
     DevResult r;

@@ -411,3 +411,24 @@ def test_screen_does_without_where_memory_is_short(fg, D, K, N, left):
         before = c.gmm_launch_count()
         c.gmm_em_step(*args)
         assert c.gmm_last_exact_count() == K and launches[0] == launches[1] != c.gmm_launch_count() - before
+
+
+def test_screen_of_large_groups_of_which_the_last_is_broad(fg):
+    """Fisher vectors of four groups that are larger than one CTA sorts; a broad region that the look ahead does not meet sends the call to the dense
+    kernels when three of them are done."""
+    from oracle.fisher import fisher_vectors
+
+    N, D, K = 160_000, 16, 64
+    _, pi, mu, var = _mixture(100, D, K, 81)
+    mu[K // 2:], var[:], pi[:] = 0.02 * mu[K // 2:], 1.0, 1.0 / K
+    rng = np.random.default_rng(8)
+    X = (mu[rng.integers(0, K // 2, N)] + rng.normal(size=(N, D))).astype(np.float32)
+    X[-3000:-500] = rng.normal(size=(2500, D)).astype(np.float32)
+    offsets = np.arange(5, dtype=np.int64) * 40_000
+    ref = fisher_vectors(X, offsets, pi, mu, var)
+    lz = orc.responsibilities(X, pi, mu, var)[1]
+    with fg.Context(0) as c:
+        G, ll = c.gmm_fisher_vectors(_t(X), offsets, _t(pi), _t(mu), _t(var))
+    assert abs(ll - lz.sum()) <= 1e-5 * abs(lz.sum())
+    # (the dense kernels' bound of flashgmm.h, A_k = N_k / (T sqrt(pi_k)) <= 1/4 here)
+    assert np.abs(G.cpu().numpy() - ref).max() <= 2e-5 * (1 + np.abs(ref).max()) + 0.25 * (1e-3 + 4e-5 * (1 + float((mu * mu).max())))

@@ -1,4 +1,5 @@
-// The FP32 path for D <= 128: direct differences on the CUDA cores, tiles cut to the shape.
+// The FP32 path for D <= 128: direct differences on the CUDA cores, tiles cut to the shape.  (Shapes that fill the fixed tiles of
+// em_fp32.cu stay there: see fp32_fixed_tiles.)
 //
 // log2 z = c - sum_d t^2, t = (x - g) sqrt(w2) - (mu - g) sqrt(w2) (two FMAs per term, g: a per-dimension centre near the data).  A CTA
 // of 256 threads takes tiles of points.  For the logits a point belongs to G x S neighbouring lanes: G lanes own the components

@@ -1457,13 +1457,17 @@ namespace {
 int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const float* pi, const float* mu,
                      const float* var, int m, int32_t* idx, float* resp, bool index_only, bool screened) {
     // (the screening path's preparation does what this one does, but for the centre of the means)
-    // (When it pays is known on the device alone, so shapes for which it mostly did not are left out: many components in few
-    // dimensions overlap, and with few components the quarters of blocks that bound the m-th best do not bound it well.)
-    // And with few points the launches decide: 35 us more of them than the tensor assignment has (us, sparse / tensor: top-1 of 2K x 16, K = 64 99 / 76,
+    // Shapes that are not screened: many components in few dimensions, which overlap where their means are not as separate as those of the
+    // timed mixtures, and few components, whose quarters of blocks bound the m-th best badly.  Whether a call's posteriors are sparse is for
+    // its data to say (screen_probe), and on separate clusters (300K points; us, screened / tensor assignment) the screening is the faster one
+    // on both sides of these lines: top-1 of 8 x 64 127 / 367, 8 x 256 144 / 450, 16 x 2048 268 / 1050; top-2 of 32 x 64 193 / 297; top-4 of
+    // 64 x 128 297 / 361, 128 x 256 427 / 429, above the lines 128 x 384 453 / 584.
+    const bool shape = (double)D >= 1.75 * std::log2((double)K) - 2.0 && (m == 1 || K >= 48 * m) && (m <= 2 || K >= 3 * D);
+    // With few points the launches decide: 35 us more of them than the tensor assignment has (us, sparse / tensor: top-1 of 2K x 16, K = 64 99 / 76,
     // of 10K x 32, K = 64 89 / 71, of 20K x 32, K = 256 96 / 88; top-2 of 10K x 128, K = 1024 142 / 133, of 30K 172 / 190).
     const double gain = (m == 1 ? 0.5 + 0.0018 * K : 0.6 + 0.0025 * K) - (m == 1 ? 1.0 : 2.0) * screen_fixed(D, K);      // ns per point
-    const bool screening = !screened && m <= 4 && m <= K && screen_wanted(ctx, SCREEN_RANKS, N, D, K) &&
-                           (ctx->scr_marks > 0.0 || !auto_is_tensor(D, K) || (double)N * gain > 30e3) && (ctx->scr_marks > 0.0 || ((double)D >= 1.75 * std::log2((double)K) - 2.0 && (m == 1 || K >= 48 * m) && (m <= 2 || K >= 3 * D)));
+    const bool pays = shape && (!auto_is_tensor(D, K) || (double)N * gain > 30e3);
+    const bool screening = !screened && m <= 4 && m <= K && screen_wanted(ctx, SCREEN_RANKS, N, D, K) && (ctx->scr_marks > 0.0 || pays);
     if (!screening) KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), &ctx->result()->status));
     if (!screening && (size_t)K * D > ((size_t)1 << 12)) ctx->launches++;      // but for tiny problems, the centre of the means is a launch of its own
     // Tensor-core assignment where the E+M step would take the tensor path too.  Ill-conditioned components are evaluated

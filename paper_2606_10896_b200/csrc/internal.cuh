@@ -55,7 +55,7 @@ cudaError_t launch_topm_fp32(cudaStream_t s, const float* X, int64_t n, int D, i
                              const float* w2, const double* c2d, const float* g, int m, int32_t* idx, float* resp,
                              const int* run_if = nullptr, const int32_t* gather = nullptr, const int* gather_count = nullptr);
 
-// ---- the same, for D <= 128 (em_direct.cu; launch_lse_fp32 and launch_mstep_fp32 go there) ------------------------
+// ---- the same, for D <= 128 (em_direct.cu; launch_lse_fp32 and launch_mstep_fp32 go there but for the shapes that fill their own tiles) ------------------------
 int lse_direct_parts(int64_t n, int D, int K);      // entries of llpart that launch_lse_fp32 writes for n points (D <= 128)
 cudaError_t launch_lse_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                               const double* c2d, const float* g, double* logZ2, double* llpart);

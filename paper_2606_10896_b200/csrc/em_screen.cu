@@ -550,12 +550,13 @@ static_assert(SW_SPILL == SCR_SPILL, "room for the spilled entries");
 // half the tensor cores' rate.  Coefficients come as 1-D bulk copies of an image that screen_plane_kernel laid out swizzled, in
 // stages of 32 KB.  Per group of 128 components the tensor cores form half 0 (columns 0-127) and half 1 (128-255) from the same
 // stages; a group's constants are one more product, of 16 columns.  A group's accumulators go into registers at once (128 of
-// them), so that the next group of the half is formed while they are worked through, about 75 instructions per 32 values.  When
+// them), so that the next group of the half is formed while they are worked through: the four blocks' maxima first, then their marks.  When
 // the last group of a tile has been formed, the half's operand is replaced by the next tile's rows, which wait in shared memory,
 // before those accumulators are read.
-// MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles, 65 us per 2^18 points at D = 128, K = 1024; it takes 115 us: the two
-// halves' MMA and softmax warps wait for one another (a thread that reads its 128 values holds the half's accumulators up, and
-// tensor memory has no room for a second set beside the operands).  126 us with one MMA warp for both halves, 142 with its votes.
+// MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles at the clock that the power limit leaves.  27 tiles per CTA, K = 1024: 383 us at
+// D = 128, which is 1.6 PFLOP/s (cuBLAS: 1.64; without the marks, without the loads of coefficients, without reading the accumulators or
+// with MMA warps that take turns it is the same within 5 %), 261 us at D = 64, 252 at D = 32, where the softmax threads set the
+// pace (block by block, each one's marks before the next one's maxima: 400, 318 and 319 us).
 //
 // TOP: how many of a point's largest values are wanted for certain.  1: everything within the margin of the largest.  More (the top-m
 // assignment): also everything that could be among the TOP largest.  The bound for those is the TOP-th largest of the lower bounds of
@@ -681,72 +682,59 @@ screen_sweep_kernel(const SweepParams p) {
             auto floor_now = [&]() -> float { return TOP == 1 ? thr - p.margin : fmaxf(fminf(low[0] - p.margin, low[TOP - 1]), 0.5f * SCR_NEVER); };
             int ne = 0, packs = 0;
             float lost = -CUDART_INF_F;                      // largest upper bound of a block with marks that found no room
-            // 32 accumulators of the point = approximate values: the block's largest; marks.
-            auto block = [&](const uint32_t (&v)[32], int bn, bool first) {
-                float mx[4];
+            // The largest of the four quarters of 32 accumulators (= the point's approximate values for a block of components).
+            auto quarters = [&](const uint32_t (&v)[32], float (&mx)[4]) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     mx[j] = max3(__uint_as_float(v[8 * j]), __uint_as_float(v[8 * j + 1]), __uint_as_float(v[8 * j + 2]));
                     mx[j] = max3(mx[j], __uint_as_float(v[8 * j + 3]), __uint_as_float(v[8 * j + 4]));
                     mx[j] = max3(mx[j], __uint_as_float(v[8 * j + 5]), __uint_as_float(v[8 * j + 6]));
                 }
-                if (TOP == 1) {
+                if (TOP == 1) {                              // (the quarters themselves are not asked for)
                     mx[0] = max3(mx[0], __uint_as_float(v[7]), __uint_as_float(v[15]));
                     mx[1] = max3(mx[1], __uint_as_float(v[23]), __uint_as_float(v[31]));
                 } else {
 #pragma unroll
                     for (int j = 0; j < 4; ++j) mx[j] = fmaxf(mx[j], __uint_as_float(v[8 * j + 7]));
                 }
-                const float2 ab = blk[bn];
-                const float bmax = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]), E = fmaf(ab.y, nrm, fabsf(ab.x));
-                if (TOP == 1) {
-                    if (!(ab.x < 0.f)) thr = fmaxf(thr, bmax - E);
-                } else if (first) {
-                    if (!(ab.x < 0.f) && bmax - E > low[TOP - 1])
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float x = mx[q] - E;
-#pragma unroll
-                        for (int j = 0; j < TOP; ++j) {
-                            const float keep = fmaxf(low[j], x);
-                            x = fminf(low[j], x);
-                            low[j] = keep;
-                        }
-                    }
-                }
-                if (TOP > 1 && first) return;
+            };
+            // Marks of a block with largest value bmax and allowance E.
+            auto mark = [&](const uint32_t (&v)[32], int bn, float bmax, float E) {
                 const float cut = floor_now() - E;
                 if (in && bmax >= cut) {
-                    if (!(cut > 0.5f * SCR_NEVER)) {         // no useful bound (yet): the values of positions without a component could
-                        lost = CUDART_INF_F;                 // pass, so the row is evaluated in full
-                        return;
-                    }
-                    // bit j of the mask: value j reaches the cut (the sign of l - cut, shifted in from the top)
+                    // bit j of the mask: value j reaches the cut (the sign of l - cut; four chains of shifts, a byte each)
                     const uint64_t nc = pack2(__float_as_uint(-cut), __float_as_uint(-cut));
-                    unsigned mask = 0;
+                    unsigned m4[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-                    for (int j = 15; j >= 0; --j) {
-                        const uint64_t d = add2(pack2(v[2 * j], v[2 * j + 1]), nc);
-                        mask = __funnelshift_l(__float_as_uint(hi2(d)), mask, 1);
-                        mask = __funnelshift_l(__float_as_uint(lo2(d)), mask, 1);
-                    }
-                    mask = ~mask;
-                    if (ne == SW_ENT + SW_SPILL && packs < 2) {      // drop what the bound found meanwhile rules out (of broad posteriors:
-                        int m = 0;                                   // nothing; trying at every block took a millisecond per tile)
-                        ++packs;
-                        for (int e = 0; e < SW_ENT + SW_SPILL; ++e) {
-                            const unsigned long long w = ent(e);
-                            if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= floor_now()) ent(m++) = w;
+                    for (int j = 3; j >= 0; --j)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint64_t d = add2(pack2(v[8 * q + 2 * j], v[8 * q + 2 * j + 1]), nc);
+                            m4[q] = __funnelshift_l(__float_as_uint(hi2(d)), m4[q], 1);
+                            m4[q] = __funnelshift_l(__float_as_uint(lo2(d)), m4[q], 1);
                         }
-                        ne = m;
-                    }
+                    const unsigned mask = ~((m4[0] | (m4[1] << 8)) | ((m4[2] << 16) | (m4[3] << 24)));
                     const float ub = bmax + E;
-                    if (ne < SW_ENT + SW_SPILL) {
-                        // the block's largest upper bound, rounded up to the 24 bits that share a word with its number
-                        const unsigned ubits = (__float_as_uint(ub + fabsf(ub) * 1e-4f + 1e-3f) & ~255u) | (unsigned)bn;
-                        ent(ne++) = ((unsigned long long)ubits << 32) | mask;
+                    // the block's largest upper bound, rounded up to the 24 bits that share a word with its number
+                    const unsigned ubits = (__float_as_uint(ub + fabsf(ub) * 1e-4f + 1e-3f) & ~255u) | (unsigned)bn;
+                    const unsigned long long w = ((unsigned long long)ubits << 32) | mask;
+                    const bool useful = cut > 0.5f * SCR_NEVER;      // (no useful bound yet: the values of positions without a component could
+                    if (useful && ne < SW_ENT) {                     // pass, so the row is evaluated in full)
+                        ent_s[256 * ne++] = w;
+                    } else if (!useful) {
+                        lost = CUDART_INF_F;
                     } else {
-                        lost = fmaxf(lost, ub);              // (harmless if the final bound rules the block out)
+                        if (ne == SW_ENT + SW_SPILL && packs < 2) {  // drop what the bound found meanwhile rules out (of broad posteriors:
+                            int m = 0;                               // nothing; trying at every block took a millisecond per tile)
+                            ++packs;
+                            for (int e = 0; e < SW_ENT + SW_SPILL; ++e) {
+                                const unsigned long long o = ent(e);
+                                if (__uint_as_float((unsigned)(o >> 32) & ~255u) >= floor_now()) ent(m++) = o;
+                            }
+                            ne = m;
+                        }
+                        if (ne < SW_ENT + SW_SPILL) ent(ne++) = w;
+                        else lost = fmaxf(lost, ub);                 // (harmless if the final bound rules the block out)
                     }
                 }
             };
@@ -768,10 +756,38 @@ screen_sweep_kernel(const SweepParams p) {
                 fence_before();
                 bar_arrive(BAR(SB_LEMPTY + half));
                 if (ok) {
-                    block(v0, g * 4, first);
-                    block(v1, g * 4 + 1, first);
-                    block(v2, g * 4 + 2, first);
-                    block(v3, g * 4 + 3, first);
+                    // (the four blocks' maxima first, then their marks: four independent chains, and a bound that has seen the whole
+                    // group; block by block the chains of one another kept the warp waiting)
+                    float q0[4], q1[4], q2[4], q3[4], bm[4], E[4];
+                    quarters(v0, q0); quarters(v1, q1); quarters(v2, q2); quarters(v3, q3);
+                    bm[0] = fmaxf(max3(q0[0], q0[1], q0[2]), q0[3]); bm[1] = fmaxf(max3(q1[0], q1[1], q1[2]), q1[3]);
+                    bm[2] = fmaxf(max3(q2[0], q2[1], q2[2]), q2[3]); bm[3] = fmaxf(max3(q3[0], q3[1], q3[2]), q3[3]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 ab = blk[4 * g + j];
+                        E[j] = fmaf(ab.y, nrm, fabsf(ab.x));
+                        if (TOP == 1) {
+                            thr = fmaxf(thr, ab.x < 0.f ? -CUDART_INF_F : bm[j] - E[j]);
+                        } else if (first && !(ab.x < 0.f) && bm[j] - E[j] > low[TOP - 1]) {
+                            const float (&mx)[4] = j == 0 ? q0 : j == 1 ? q1 : j == 2 ? q2 : q3;
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                float x = mx[q] - E[j];
+#pragma unroll
+                                for (int t = 0; t < TOP; ++t) {
+                                    const float keep = fmaxf(low[t], x);
+                                    x = fminf(low[t], x);
+                                    low[t] = keep;
+                                }
+                            }
+                        }
+                    }
+                    if (TOP == 1 || !first) {
+                        mark(v0, 4 * g, bm[0], E[0]);
+                        mark(v1, 4 * g + 1, bm[1], E[1]);
+                        mark(v2, 4 * g + 2, bm[2], E[2]);
+                        mark(v3, 4 * g + 3, bm[3], E[3]);
+                    }
                 }
             }
             // the point's list: the words (block of 32 positions, mask) that the final bound leaves

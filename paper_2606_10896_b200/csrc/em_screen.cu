@@ -112,6 +112,9 @@ __global__ void __launch_bounds__(512) screen_dim_kernel(int D, int K, const flo
     sd[d] = s;
     gd[d] = gf;
     if (d == 0) {
+        ctl[SC_MARKS] = 0;
+        ctl[SC_OVF] = 0;
+        ctl[SC_EXTRA] = 0;
         ctl[SC_TICKET_A] = 0;
         ctl[SC_PROBED] = 0;
         ctl[SC_DONE] = 0;
@@ -343,6 +346,9 @@ __device__ void screen_probe(const ProbeArgs& a, int D, const float* __restrict_
         a.ctl[SC_DENSE] = 1;
 }
 
+// Where dimension d stands in the contraction: chunk c of the KS chunks of eight has dimensions 4 c .. 4 c + 3 and 4 (KS + c) .. + 3, so
+// that neighbouring lanes that form one chunk each read neighbouring 16 bytes of a row.
+__host__ __device__ __forceinline__ int screen_slot(int d, int KS) { return d < 4 * KS ? (d >> 2) * 8 + (d & 3) : ((d - 4 * KS) >> 2) * 8 + 4 + (d & 3); }
 constexpr int SW_CSLOT = 4096;               // a group's constants: 128 rows of 16 halves
 // Positions of the components in the sweep: ascending by the allowance of a typical point, so that 32 neighbours, which are
 // screened with the largest allowance among them, have similar ones (the capped components come last).  A warp per component:
@@ -384,7 +390,7 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe
     const int r = pos & 127;
     unsigned char* grp = img + (size_t)(pos >> 7) * screen_group_bytes(D);
     const int ndim = (D + 7) / 8 * 8;
-    for (int d = lane; d < ndim; d += 32) {
+    for (int d = lane; d < ndim; d += 32) {                  // (in the order of screen_slot; beyond D: zeros)
         float a = 0.f, b = 0.f;
         if (on && d < D) {
             const float s = __ldg(sd + d);
@@ -395,10 +401,11 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe
             b = (float)(-bd);
         }
         // k-step d / 8 holds eight dimensions of u and the same eight of u^2: two 16-byte chunks of a 128-byte row, swizzled
-        unsigned char* o = grp + SW_CSLOT + (d >> 5) * 16384 + r * 128;
-        const int c = 2 * ((d >> 3) & 3);
-        *reinterpret_cast<__half*>(o + ((c ^ (r & 7)) << 4) + 2 * (d & 7)) = __float2half_rn(a);
-        *reinterpret_cast<__half*>(o + (((c + 1) ^ (r & 7)) << 4) + 2 * (d & 7)) = __float2half_rn(b);
+        const int z = screen_slot(d, ndim >> 3);
+        unsigned char* o = grp + SW_CSLOT + (z >> 5) * 16384 + r * 128;
+        const int c = 2 * ((z >> 3) & 3);
+        *reinterpret_cast<__half*>(o + ((c ^ (r & 7)) << 4) + 2 * (z & 7)) = __float2half_rn(a);
+        *reinterpret_cast<__half*>(o + (((c + 1) ^ (r & 7)) << 4) + 2 * (z & 7)) = __float2half_rn(b);
     }
     if (lane == 0) {
         comp_of[pos] = on ? k : -1;
@@ -420,34 +427,35 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe
 }
 
 // ------------------------------------------------------------------------------------------------------------------
-// X -> fp16 plane of u, rows of `chunks` 16-byte chunks (8 dimensions each), and |u|^2.  Chunk c of row r sits at place
-// screen_place(c, r): the sweep reads a row per lane from shared memory, and eight neighbouring rows' chunks c then lie in
-// different banks.  L lanes per row, 8 dimensions each.  Bound by memory: 4 D bytes in, 2 D out.  Data that are not finite are left to
-// the dense kernels: what becomes of them differs from entry point to entry point and from path to path.
+// Rows of u in shared memory: `chunks` 16-byte chunks (8 dimensions each).  Chunk c of row r sits at place screen_place(c, r): the
+// sweep reads a row per lane, and eight neighbouring rows' chunks c then lie in different banks.
 __host__ __device__ __forceinline__ int screen_chunks(int D) { return D <= 32 ? 4 : D <= 64 ? 8 : 16; }
 __device__ __forceinline__ int screen_place(int c, int row, int chunks) { return chunks == 4 ? c ^ ((row >> 1) & 3) : c ^ (row & 7); }
 
+// X -> fp16 plane of u and |u|^2, for the shapes that the sweep does not convert itself.  L lanes per row, 8 dimensions each.  Bound by
+// memory: 4 D bytes in, 2 D out.  Data that are not finite are left to the dense kernels: what becomes of them differs from entry point to entry point
+// and from path to path.
 template <int L>
 __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __restrict__ X, int64_t n, int D, int chunks, const float* __restrict__ sd,
                                                                const float* __restrict__ gd, unsigned char* __restrict__ y,
                                                                float* __restrict__ n2, int* __restrict__ ctl) {
-    if (blockIdx.x == 0 && threadIdx.x < 3) ctl[SC_MARKS + threadIdx.x] = 0;
     if (ctl[SC_DENSE] != 0) return;
     const bool vec_ok = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-    const int l = threadIdx.x % L, d0 = l * 8;
+    const int l = threadIdx.x % L, KS = (D + 7) / 8;
+    auto dim = [&](int j) { return l < KS ? (j < 4 ? 4 * l + j : 4 * (KS + l) + j - 4) : D; };       // (see screen_slot)
     constexpr int RPB = 256 / L;
     float gv[8], sv[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) { gv[j] = __ldg(gd + d0 + j); sv[j] = __ldg(sd + d0 + j); }
+    for (int j = 0; j < 8; ++j) { gv[j] = dim(j) < D ? __ldg(gd + dim(j)) : 0.f; sv[j] = dim(j) < D ? __ldg(sd + dim(j)) : 0.f; }
     bool bad = false;
     const int64_t step = (int64_t)gridDim.x * RPB;
     auto load = [&](int64_t row, float (&x)[8]) {
-        if (row < n && vec_ok && d0 + 8 <= D) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(X + row * D + d0)), b = __ldg(reinterpret_cast<const float4*>(X + row * D + d0) + 1);
+        if (row < n && vec_ok && dim(7) < D) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(X + row * D + dim(0))), b = __ldg(reinterpret_cast<const float4*>(X + row * D + dim(4)));
             x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
         } else {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) x[j] = (row < n && d0 + j < D) ? __ldg(X + row * D + d0 + j) : 0.f;
+            for (int j = 0; j < 8; ++j) x[j] = (row < n && dim(j) < D) ? __ldg(X + row * D + dim(j)) : 0.f;
         }
     };
     auto store = [&](int64_t row, const float (&x)[8]) {
@@ -457,7 +465,7 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
 #pragma unroll
         for (int j = 0; j < 8; j += 2) {
             bad |= !(fabsf(x[j]) <= 3.0e38f) || !(fabsf(x[j + 1]) <= 3.0e38f);
-            float u0 = d0 + j < D ? (x[j] - gv[j]) * sv[j] : 0.f, u1 = d0 + j + 1 < D ? (x[j + 1] - gv[j + 1]) * sv[j + 1] : 0.f;
+            float u0 = (x[j] - gv[j]) * sv[j], u1 = (x[j + 1] - gv[j + 1]) * sv[j + 1];       // (beyond D: zeros)
             far |= !(fabsf(u0) <= 240.f) || !(fabsf(u1) <= 240.f);
             u0 = fminf(fmaxf(u0, -240.f), 240.f);
             u1 = fminf(fmaxf(u1, -240.f), 240.f);
@@ -469,7 +477,7 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
 #pragma unroll
         for (int o = L / 2; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
         if (row >= n) return;
-        if (d0 < D) *reinterpret_cast<uint4*>(y + ((size_t)row * chunks + screen_place(l, (int)row, chunks)) * 16) = make_uint4(xh[0], xh[1], xh[2], xh[3]);
+        if (l < KS) *reinterpret_cast<uint4*>(y + ((size_t)row * chunks + screen_place(l, (int)row, chunks)) * 16) = make_uint4(xh[0], xh[1], xh[2], xh[3]);
         if (l == 0) n2[row] = nrm * 1.0001f;
     };
     // (every lane of a warp takes the same number of steps: the row sums are shuffles; two rows' loads in flight)
@@ -486,28 +494,47 @@ __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __re
 
 // ------------------------------------------------------------------------------------------------------------------
 // Sweep
-constexpr int SW_THREADS = 352;              // 8 softmax warps, producer warp, an MMA warp per half of the tile
-constexpr int SW_PRODUCER = 8, SW_MMA = 9;
-constexpr int SW_PSLOT = 32768, SW_PS = 4;   // coefficient stages: two atoms of 128 components
-constexpr int SW_ENT = 10;                   // blocks of 32 components a point can have marks in: in shared memory,
-constexpr int SW_SPILL = 22;                 // and, rarely needed, in global memory
-constexpr int SW_UOFF = SW_PS * SW_PSLOT;    // the next tile's rows of u (256 x 16 chunks bytes), then the slots of the constants
-constexpr int SW_UC = 65536 + 2 * SW_CSLOT;  // (16 chunks: two groups in flight; at most 8 chunks: half the rows, four groups)
-constexpr int SW_AOFF = SW_UOFF + SW_UC;     // the points' side of the constants: 128 rows (256, 1, 1, 0, ...)
-constexpr int SW_EOFF = SW_AOFF + 4096;
-constexpr int SW_TOFF = SW_EOFF + SW_ENT * 256 * 8;      // allowances of every block
-constexpr int SW_BOFF = SW_TOFF + SCR_MAX_K / 32 * 8;
-constexpr int SW_SMEM = SW_BOFF + 256 + 1024;
-enum { SB_PFULL = 0, SB_PEMPTY = SB_PFULL + SW_PS, SB_UFULL = SB_PEMPTY + SW_PS, SB_UEMPTY, SB_AFULL, SB_LFULL = SB_AFULL + 2,
-       SB_LEMPTY = SB_LFULL + 2, SB_FINAL = SB_LEMPTY + 2, SB_COUNT = SB_FINAL + 2 };
-static_assert(SB_COUNT * 8 <= 256, "barriers");
-static_assert(SW_SMEM <= 232448, "shared memory");
+constexpr int SW_PSLOT = 32768;              // a coefficient stage: two atoms of 128 components
+constexpr int SW_REGS = 168, SW_REGS_FEW = 88;       // CONVERT: of a softmax thread and of the others: (168 + 88) x 256 = what 512 threads have at launch
+constexpr int SW_XBYTES = 16384 + 32;        // CONVERT: a chunk of X, from the 16-byte boundary before it on
+// Where the points' rows come from.  CONVERT: X itself, converted by four warps of the sweep.  Otherwise screen_transform_kernel has
+// written the rows of u (16-bit), which come by bulk copy.
+template <bool CONVERT>
+struct Sweep {
+    static constexpr int THREADS = CONVERT ? 512 : 352;      // 8 softmax warps, 4 that convert, producer warp, an MMA warp per half of the tile, a warp that fetches X
+    static constexpr int CONVERTER = 8, PRODUCER = CONVERT ? 12 : 8, MMA = PRODUCER + 1, FETCH = 15;
+    static constexpr int PS = CONVERT ? 3 : 4;               // coefficient stages
+    static constexpr int CSLOTS = CONVERT ? 3 : 2;           // groups in flight that have constants (rows of at most 8 chunks leave room for two more)
+    static constexpr int ENT = CONVERT ? 7 : 10;             // blocks of 32 components a point can have marks in: in shared memory,
+    static constexpr int SPILL = 32 - ENT;                   // and, rarely needed, in global memory (a mask has 32 bits)
+    static constexpr int UOFF = PS * SW_PSLOT;               // the next tile's rows of u (256 x 16 chunks bytes)
+    static constexpr int COFF = UOFF + 65536;                // constants of the groups in flight
+    static constexpr int AOFF = COFF + CSLOTS * SW_CSLOT;    // the points' side of the constants: 128 rows (256, 1, 1, 0, ...)
+    static constexpr int EOFF = AOFF + 4096;
+    static constexpr int TOFF = EOFF + ENT * 256 * 8;        // allowances of every block
+    static constexpr int NOFF = TOFF + SCR_MAX_K / 32 * 8;   // CONVERT: |u|^2 of the next tile's rows, chunks of X
+    static constexpr int XOFF = NOFF + (CONVERT ? 256 * 4 : 0);
+    static constexpr int BOFF = XOFF + (CONVERT ? 2 * SW_XBYTES : 0);
+    static constexpr int SMEM = BOFF + 256 + 1024;
+    enum { PFULL = 0, PEMPTY = PFULL + PS, UFULL = PEMPTY + PS, UEMPTY, AFULL, LFULL = AFULL + 2, LEMPTY = LFULL + 2, FINAL = LEMPTY + 2, XFULL = FINAL + 2,
+           XEMPTY = XFULL + 2, COUNT = XEMPTY + 2 };
+    static_assert(COUNT * 8 <= 256, "barriers");
+    static_assert(SMEM <= 232448, "shared memory");
+    static_assert(SPILL <= SCR_SPILL, "room for the spilled entries");
+};
+// Which way pays, measured per 1.02M points (us, converted by the sweep / sweep + transform; K = 256, 1024, 4096): D = 128: 238 / 264,
+// 442 / 534, 1468 / 1603; D = 80 (K = 256, 4096): 240 / 282, 1242 / 1420; D = 64: 141 / 170, 334 / 350, 1029 / 950; D = 48: 143 / 185, 359 / 359,
+// 1103 / 1025; D = 32: 114 / 129, 358 / 300, 1161 / 1082; D = 16 (K = 256): 102 / 113.  The transform costs about 1.06 us per dimension;
+// the converting warps cost the softmax warps issue slots and instruction cache, which matters where the MMAs are short.
+inline bool screen_converts(int D, int K) { return D > 64 || (D > 32 && K <= 512) || K <= 256; }
 
 // two fp32 operations per instruction
 __device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b)); return r; }
 __device__ __forceinline__ float lo2(uint64_t a) { return __uint_as_float((uint32_t)a); }
 __device__ __forceinline__ float hi2(uint64_t a) { return __uint_as_float((uint32_t)(a >> 32)); }
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
 // Operand of one k-step: rows of 32 bytes, 32-byte swizzle, groups of eight rows 256 bytes apart.
 __device__ __forceinline__ uint64_t make_desc32(uint32_t saddr) {
     return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
@@ -526,12 +553,15 @@ struct SweepParams {
     int64_t n;
     int KA, KS, NG;          // atoms and k-steps of the contraction, groups of 128 components
     int chunks;              // 16-byte chunks of a row of u
-    const unsigned char* y;
+    const float* X;
+    int D;
+    const float *sd, *gd;
+    const unsigned char* y;  // (not CONVERT: rows of u, |u|^2)
+    const float* n2;
     const unsigned char* img;
     int gbytes;              // of the image of a group
     float margin;
     const int4* blk;
-    const float* n2;
     unsigned* pt_off;
     int* pt_cnt;
     uint2* words;
@@ -542,8 +572,163 @@ struct SweepParams {
     int test_silent;                // >= 0: that CTA keeps back the news of its first products (time-out test)
 };
 
-static_assert(SW_ENT + SW_SPILL <= 32, "a mask of a point's entries");
-static_assert(SW_SPILL == SCR_SPILL, "room for the spilled entries");
+// The points' way into the sweep: rows of X through a ring of two slots of 16 KB, which a warp of its own fills by untiled bulk copies,
+// and from there, by four converting warps, as rows of u (and |u|^2) into shared memory.  A copy starts at the 16-byte boundary
+// before its first byte and ends at the one behind its last, so that any X will do; what would reach beyond X's own bytes is read
+// with plain loads.  A chunk has 512 / L rows, L = 2^SH lanes of eight dimensions per row, four rows per lane.  One warp per scheduler
+// has nothing to hide its latencies behind but its own instructions, so each chunk's fixed cost counts: with 2 KB per warp and copy,
+// requested by the warps themselves, a chunk took 1700 cycles (180 to see that it is there, 500 to ask for the next, 700 to convert it)
+// and the sweep waited for them.
+// bar_wait for those who mostly wait (the hint lets the hardware keep them away from the scheduler for longer).
+__device__ __forceinline__ bool bar_wait_idle(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+    for (int it = 0; it < 4; ++it) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+                     : "=r"(ok) : "r"(bar), "r"(parity), "r"(5000) : "memory");
+        if (ok) return true;
+        if (*abort_flag) return false;
+    }
+    return bar_wait(bar, parity, abort_flag, status, false);
+}
+struct SweepRows {
+    uint64_t xb;                 // the 16-byte boundary at or before X; offsets below count from it (at most 2^20 rows of 512 bytes)
+    uint32_t shift, D4, end;
+    int n, R, per, tstep, first;
+    __device__ __forceinline__ SweepRows(const SweepParams& p, int sh) {
+        const uint64_t x = reinterpret_cast<uint64_t>(p.X);
+        xb = x & ~(uint64_t)15;
+        shift = (uint32_t)(x & 15u);
+        D4 = 4u * (uint32_t)p.D;
+        n = (int)p.n;
+        end = shift + (uint32_t)n * D4;
+        R = 512 >> sh;
+        per = 1 << (sh - 1);                                 // chunks per tile
+        first = (int)blockIdx.x * SCR_TILE;
+        tstep = (int)gridDim.x * SCR_TILE;
+    }
+    // whether the chunk from `row` on comes by bulk copy
+    __device__ __forceinline__ bool range(int row, uint32_t& lo, uint32_t& bytes) const {
+        const uint32_t q = shift + (uint32_t)row * D4, hi = (q + (uint32_t)R * D4 + 15u) & ~15u;
+        lo = q & ~15u;
+        bytes = hi - lo;
+        return row + R <= n && lo >= shift && hi <= end;
+    }
+};
+__device__ __forceinline__ int screen_lane_shift(int KS) { return KS > 8 ? 4 : KS > 4 ? 3 : KS > 2 ? 2 : 1; }
+
+template <int SH>
+__device__ __forceinline__ void screen_convert(const SweepParams& p, unsigned char* smem, int cw, int lane, int ntl, volatile int* abort_flag) {
+    constexpr int L = 1 << SH, RW = 32 >> SH;                // rows per warp and step
+    using S = Sweep<true>;
+    const SweepRows rows(p, SH);
+    const int D = p.D, l = lane & (L - 1), sub = lane >> SH;
+    const int d0 = 4 * l, d1 = 4 * (p.KS + l);               // dimensions of this lane: d0 .. d0 + 3 and d1 .. d1 + 3 (see screen_slot)
+    const bool on = l < p.KS;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BOFF);
+    float* nrm_s = reinterpret_cast<float*>(smem + S::NOFF);
+    const bool vec = ((D & 3) == 0) && rows.shift == 0, in0 = on && d0 < D, in1 = on && d1 < D;
+    uint64_t s2[4], g2[4];                                   // u = s x - s g: s a power of two, so the same as s (x - g)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int d = j < 2 ? d0 + 2 * j : d1 + 2 * j - 4;
+        const float sa = d < D ? __ldg(p.sd + d) : 0.f, sb = d + 1 < D ? __ldg(p.sd + d + 1) : 0.f;
+        s2[j] = pack2(__float_as_uint(sa), __float_as_uint(sb));
+        g2[j] = pack2(__float_as_uint(d < D ? -sa * __ldg(p.gd + d) : 0.f), __float_as_uint(d + 1 < D ? -sb * __ldg(p.gd + d + 1) : 0.f));
+    }
+    // where this lane's 16 bytes of u go: row r0 + 4 RW h of a tile, r0 = cw RW + sub + 128 k (SH = 4: 32 k)
+    const int rl = cw * RW + sub;
+    uint32_t c = 0;
+    bool ok = true;
+    for (int i = 0; i < ntl && ok; ++i) {
+        int row0 = rows.first + i * rows.tstep;
+#pragma unroll 1
+        for (int k = 0; k < rows.per; ++k, ++c, row0 += rows.R) {
+            const uint32_t slot = c & 1u;
+            ok = __all_sync(0xffffffffu, bar_wait_idle(smem_u32(&bars[S::XFULL + slot]), (c >> 1) & 1u, abort_flag, p.status));
+            if (!ok) break;
+            uint32_t lo, bytes;
+            uint64_t x[4][4];
+            if (rows.range(row0, lo, bytes)) {
+                const unsigned char* src = smem + S::XOFF + slot * SW_XBYTES + (rows.shift + (uint32_t)row0 * rows.D4 - lo) + (uint32_t)rl * rows.D4;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const unsigned char* q = src + (uint32_t)(h * 4 * RW) * rows.D4;
+                    if (vec) {
+                        ulonglong2 a = make_ulonglong2(0ull, 0ull), b = a;
+                        if (in0) a = *reinterpret_cast<const ulonglong2*>(q + 4 * d0);
+                        if (in1) b = *reinterpret_cast<const ulonglong2*>(q + 4 * d1);
+                        x[h][0] = a.x; x[h][1] = a.y; x[h][2] = b.x; x[h][3] = b.y;
+                    } else {
+                        const uint32_t* w = reinterpret_cast<const uint32_t*>(q);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const int d = j < 2 ? d0 + 2 * j : d1 + 2 * j - 4;
+                            x[h][j] = pack2(on && d < D ? w[d] : 0u, on && d + 1 < D ? w[d + 1] : 0u);
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const int row = row0 + rl + h * 4 * RW;
+                    const float* q = p.X + (int64_t)row * D;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int d = j < 2 ? d0 + 2 * j : d1 + 2 * j - 4;
+                        x[h][j] = pack2(row < rows.n && on && d < D ? __float_as_uint(__ldg(q + d)) : 0u,
+                                        row < rows.n && on && d + 1 < D ? __float_as_uint(__ldg(q + d + 1)) : 0u);
+                    }
+                }
+            }
+            __syncwarp();                                    // (the warp's part of the slot has been read)
+            if (lane == 0) bar_arrive(smem_u32(&bars[S::XEMPTY + slot]));
+            if (k == 0 && i > 0)                             // the rows of the tile before have been taken
+                ok = __all_sync(0xffffffffu, bar_wait_idle(smem_u32(&bars[S::UEMPTY]), (uint32_t)((i - 1) & 1), abort_flag, p.status));
+            if (!ok) break;
+            float nrm[4];
+            const int r0 = k * rows.R + rl;                  // of the tile
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int r = r0 + h * 4 * RW;
+                uint64_t u[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) u[j] = fma2(x[h][j], s2[j], g2[j]);
+                const uint64_t a = add2(fma2(u[2], u[2], mul2(u[0], u[0])), fma2(u[3], u[3], mul2(u[1], u[1])));
+                nrm[h] = lo2(a) + hi2(a);
+                if (!(nrm[h] <= 57600.f)) {                  // (a coordinate beyond 240, or one that is not finite?)
+                    bool bad = false, far = false;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        bad |= !(fabsf(lo2(x[h][j])) <= 3.0e38f) || !(fabsf(hi2(x[h][j])) <= 3.0e38f);
+                        far |= !(fabsf(lo2(u[j])) <= 240.f) || !(fabsf(hi2(u[j])) <= 240.f);
+                        u[j] = pack2(__float_as_uint(fminf(fmaxf(lo2(u[j]), -240.f), 240.f)), __float_as_uint(fminf(fmaxf(hi2(u[j]), -240.f), 240.f)));
+                    }
+                    if (bad) p.ctl[SC_DENSE] = 1;            // (data that are not finite are left to the dense kernels: what becomes of
+                    if (far) nrm[h] = CUDART_INF_F;          // them differs from path to path; a clamped coordinate: no bound holds, the row
+                }                                            // is evaluated in full)
+                if (on) {
+                    uint32_t xh[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const __half2 hh = __floats2half2_rn(lo2(u[j]), hi2(u[j]));
+                        xh[j] = *reinterpret_cast<const uint32_t*>(&hh);
+                    }
+                    *reinterpret_cast<uint4*>(smem + S::UOFF + (r * p.chunks + screen_place(l, r, p.chunks)) * 16) = make_uint4(xh[0], xh[1], xh[2], xh[3]);
+                }
+            }
+#pragma unroll
+            for (int o = L / 2; o > 0; o >>= 1)
+#pragma unroll
+                for (int h = 0; h < 4; ++h) nrm[h] += __shfl_xor_sync(0xffffffffu, nrm[h], o);
+            if (l == 0) {
+#pragma unroll
+                for (int h = 0; h < 4; ++h) nrm_s[r0 + h * 4 * RW] = nrm[h] * 1.0001f;
+            }
+        }
+        if (ok) bar_arrive(smem_u32(&bars[S::UFULL]));
+    }
+}
+
 // Tile = 256 points in two halves of 128 TMEM lanes, a thread per point.  The points' operand [u | u^2] lives in TENSOR MEMORY
 // (columns 256 + 128 h of half h; the squares are formed when it is written), so that shared memory has only the coefficients to
 // deliver: with both operands there its bandwidth alone (8 KB per MMA of 64 cycles, besides the incoming stages) held the sweep to
@@ -553,19 +738,21 @@ static_assert(SW_SPILL == SCR_SPILL, "room for the spilled entries");
 // them), so that the next group of the half is formed while they are worked through: the four blocks' maxima first, then their marks.  When
 // the last group of a tile has been formed, the half's operand is replaced by the next tile's rows, which wait in shared memory,
 // before those accumulators are read.
-// MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles at the clock that the power limit leaves.  27 tiles per CTA, K = 1024: 383 us at
-// D = 128, which is 1.6 PFLOP/s (cuBLAS: 1.64; without the marks, without the loads of coefficients, without reading the accumulators or
-// with MMA warps that take turns it is the same within 5 %), 261 us at D = 64, 252 at D = 32, where the softmax threads set the
-// pace (block by block, each one's marks before the next one's maxima: 400, 318 and 319 us).
+// MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles; a group takes 2600 at D = 128 with 32 of them, a tile about 3000 more for its
+// list and the next one's operand, at the 1.65 to 1.75 GHz that the power limit leaves (27 tiles per CTA, K = 1024, not converting: 383 to 402 us
+// at D = 128, 261 to 282 at D = 64, where the softmax threads set the pace; block by block, each one's marks before the next one's
+// maxima: 400, 318).  Converting, the tensor cores are busy 58 % of the time instead of 69 %: the converting warps' instructions.  Pairs of
+// CTAs (cta_group::2, half the coefficients each) wait for each other's softmax threads: 550 us against 459 then.
 //
 // TOP: how many of a point's largest values are wanted for certain.  1: everything within the margin of the largest.  More (the top-m
 // assignment): also everything that could be among the TOP largest.  The bound for those is the TOP-th largest of the lower bounds of
 // the quarters of every block: different components, so the TOP-th largest value cannot be below it.  It rises slowly as the sweep
 // goes on, so the tile's components pass twice, once for the bound and once for the marks: in one pass what was marked under
 // early bounds cost more evaluations than the second pass takes (1M x 128, K = 1024: top-2 1.40 ms in one pass, top-4 3.2).
-template <int TOP>
-__global__ void __launch_bounds__(SW_THREADS, 1)
+template <int TOP, bool CONVERT>
+__global__ void __launch_bounds__(Sweep<CONVERT>::THREADS, 1)
 screen_sweep_kernel(const SweepParams p) {
+    using S = Sweep<CONVERT>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     __shared__ uint32_t tmem_base_s;
@@ -577,31 +764,34 @@ screen_sweep_kernel(const SweepParams p) {
     const int64_t ntiles = (p.n + SCR_TILE - 1) / SCR_TILE;
     const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     constexpr int PASSES = TOP > 1 ? 2 : 1;
-    const int NG = p.NG, spg = (p.KA + 1) >> 1, cslots = SW_PS / spg;      // stages per group; groups in flight
-    unsigned char* cons = smem + SW_UOFF + 256 * 16 * p.chunks;            // [cslots][4096]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SW_BOFF);
+    const int NG = p.NG, spg = (p.KA + 1) >> 1;              // stages per group
+    unsigned char* cons = smem + S::COFF;                    // [cslots][4096]
+    const int cslots = CONVERT ? S::CSLOTS : S::PS / spg;
+    if (!CONVERT && p.chunks <= 8) cons = smem + S::UOFF + 32768;
+    float* nrm_s = reinterpret_cast<float*>(smem + S::NOFF);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BOFF);
     auto BAR = [&](int i) { return smem_u32(&bars[i]); };
     if (tid == 0) {
         abort_s = 0;
         drain_s = 0;
-        for (int i = 0; i < SB_COUNT; ++i) {
-            const bool wg = (i >= SB_AFULL && i < SB_AFULL + 2) || (i >= SB_LEMPTY && i < SB_LEMPTY + 2);
-            const bool both = i >= SB_PEMPTY && i < SB_PEMPTY + SW_PS;           // (released by the MMA warps of both halves)
-            bar_init(BAR(i), i == SB_UEMPTY ? 256 : wg ? 128 : both ? 2 : 1);
+        for (int i = 0; i < S::COUNT; ++i) {
+            const bool wg = (i >= S::AFULL && i < S::AFULL + 2) || (i >= S::LEMPTY && i < S::LEMPTY + 2);
+            const bool both = i >= S::PEMPTY && i < S::PEMPTY + S::PS;           // (released by the MMA warps of both halves)
+            bar_init(BAR(i), i == S::UEMPTY ? 256 : (wg || (CONVERT && i == S::UFULL)) ? 128 : (i == S::XEMPTY || i == S::XEMPTY + 1) ? 4 : both ? 2 : 1);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == SW_MMA) {
+    if (warp == S::MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_s)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid < NG * 4) {
         const int4 q = __ldg(p.blk + tid);
-        reinterpret_cast<float2*>(smem + SW_TOFF)[tid] = make_float2(q.z ? -__int_as_float(q.x) : __int_as_float(q.x), __int_as_float(q.y));      // (sign: no lower bound)
+        reinterpret_cast<float2*>(smem + S::TOFF)[tid] = make_float2(q.z ? -__int_as_float(q.x) : __int_as_float(q.x), __int_as_float(q.y));      // (sign: no lower bound)
     }
     if (tid < 256) {                                         // rows of 32 bytes, 32-byte swizzle (16-byte chunk ^ bit 2 of the row)
         const int r = tid >> 1, c = (tid & 1) ^ ((r >> 2) & 1);
-        reinterpret_cast<uint4*>(smem + SW_AOFF)[tid] = c == 0 ? make_uint4(0x3C005C00u, 0x00003C00u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4*>(smem + S::AOFF)[tid] = c == 0 ? make_uint4(0x3C005C00u, 0x00003C00u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
     }
     fence_async_smem();
     fence_before();
@@ -609,21 +799,26 @@ screen_sweep_kernel(const SweepParams p) {
     fence_after();
     const uint32_t tmem = tmem_base_s;
 
-    if (warp < 8) {
+    if (warp < S::CONVERTER) {
         // =========================== softmax warps: thread = TMEM lane = point ===========================
+        if (CONVERT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SW_REGS));
         const int half = warp >> 2;
         const uint32_t lane_addr = ((uint32_t)((warp & 3) * 32)) << 16;
         const uint32_t col = tmem + half * 128 + lane_addr, acol = tmem + 256 + half * 128 + lane_addr;
-        unsigned long long* ent_s = reinterpret_cast<unsigned long long*>(smem + SW_EOFF) + tid;
-        unsigned long long* ent_g = p.spill + (size_t)blockIdx.x * 256 * SW_SPILL + tid;
-        auto ent = [&](int e) -> unsigned long long& { return e < SW_ENT ? ent_s[256 * e] : ent_g[256 * (e - SW_ENT)]; };
-        const uint4* urow = reinterpret_cast<const uint4*>(smem + SW_UOFF) + (size_t)tid * p.chunks;
+        unsigned long long* ent_s = reinterpret_cast<unsigned long long*>(smem + S::EOFF) + tid;
+        unsigned long long* ent_g = p.spill + (size_t)blockIdx.x * 256 * S::SPILL + tid;
+        // (CONVERT: rows of at most 8 chunks leave half of their buffer to further entries)
+        unsigned long long* ent_x = reinterpret_cast<unsigned long long*>(smem + S::UOFF + 32768) + tid;
+        const int near_e = CONVERT && p.chunks <= 8 ? S::ENT + 16 : S::ENT;
+        auto ent = [&](int e) -> unsigned long long& { return e < S::ENT ? ent_s[256 * e] : e < near_e ? ent_x[256 * (e - S::ENT)] : ent_g[256 * (e - S::ENT)]; };
+        const uint4* urow = reinterpret_cast<const uint4*>(smem + S::UOFF) + (size_t)tid * p.chunks;
         uint32_t gi = 0;                                     // groups processed (all tiles)
         int marks = 0;
-        const float2* blk = reinterpret_cast<const float2*>(smem + SW_TOFF);
+        const float2* blk = reinterpret_cast<const float2*>(smem + S::TOFF);
+        float nrm_next = 0.f;                                // |u|^2 of the row that was taken last
         // this thread's row of tile i (in shared memory) -> the half's operand in tensor memory
         auto operand = [&](int64_t i) {
-            const bool got = bar_wait(BAR(SB_UFULL), (uint32_t)(i & 1), abort_flag, p.status, false);
+            const bool got = bar_wait(BAR(S::UFULL), (uint32_t)(i & 1), abort_flag, p.status, false);
             if (__all_sync(0xffffffffu, got)) {
 #pragma unroll 1
                 for (int z = 0; z < p.KA; z += 2) {          // (eight k-steps' loads in flight)
@@ -648,23 +843,23 @@ screen_sweep_kernel(const SweepParams p) {
                         tmem_st32(acol + (z + y) * 32, w);   // (beyond the last atom: zeros into columns of this operand)
                     }
                 }
+                if (CONVERT) nrm_next = nrm_s[tid];
                 tmem_wait_st();
             }
             fence_before();
-            bar_arrive(BAR(SB_UEMPTY));
-            bar_arrive(BAR(SB_AFULL + half));
+            bar_arrive(BAR(S::UEMPTY));
+            bar_arrive(BAR(S::AFULL + half));
         };
-        float nrm_next = 0.f;
         int dense_next = 0;
-        auto norm_load = [&](int64_t i) {
-            const int64_t r = (blockIdx.x + i * gridDim.x) * SCR_TILE + tid;
-            nrm_next = (i < ntl && r < p.n) ? __ldg(p.n2 + r) : 0.f;
+        auto ahead = [&](int64_t i) {                        // what the next tile starts with, and is not waited for then
+            if (!CONVERT) {
+                const int64_t r = (blockIdx.x + i * gridDim.x) * SCR_TILE + tid;
+                nrm_next = (i < ntl && r < p.n) ? __ldg(p.n2 + r) : 0.f;
+            }
             dense_next = __ldcg(p.ctl + SC_DENSE);
         };
-        if (ntl > 0) {
-            norm_load(0);
-            operand(0);
-        }
+        ahead(0);
+        if (ntl > 0) operand(0);
         for (int64_t i = 0; i < ntl; ++i) {
             const int64_t wrow = (blockIdx.x + i * gridDim.x) * SCR_TILE + warp * 32;       // first row of this warp
             const int64_t row = wrow + lane;
@@ -698,8 +893,32 @@ screen_sweep_kernel(const SweepParams p) {
                     for (int j = 0; j < 4; ++j) mx[j] = fmaxf(mx[j], __uint_as_float(v[8 * j + 7]));
                 }
             };
-            // Marks of a block with largest value bmax and allowance E.
-            auto mark = [&](const uint32_t (&v)[32], int bn, float bmax, float E) {
+            // a block's mask, its largest upper bound rounded up to the 24 bits that share a word with its number
+            auto entry = [&](float ub, int bn, unsigned mask) -> unsigned long long {
+                return ((unsigned long long)((__float_as_uint(ub + fabsf(ub) * 1e-4f + 1e-3f) & ~255u) | (unsigned)bn) << 32) | mask;
+            };
+            // marks that found no room in shared memory, or no useful bound
+            auto later = [&](int bn, float bmax, float E, unsigned mask) {
+                if (!(floor_now() - E > 0.5f * SCR_NEVER)) { // no useful bound (yet): the values of positions without a component could
+                    lost = CUDART_INF_F;                     // pass, so the row is evaluated in full
+                    return;
+                }
+                if (ne == S::ENT + S::SPILL && packs < 2) {  // drop what the bound found meanwhile rules out (of broad posteriors:
+                    int m = 0;                               // nothing; trying at every block took a millisecond per tile)
+                    ++packs;
+                    for (int e = 0; e < S::ENT + S::SPILL; ++e) {
+                        const unsigned long long o = ent(e);
+                        if (__uint_as_float((unsigned)(o >> 32) & ~255u) >= floor_now()) ent(m++) = o;
+                    }
+                    ne = m;
+                }
+                if (ne < S::ENT + S::SPILL) ent(ne++) = entry(bmax + E, bn, mask);
+                else lost = fmaxf(lost, bmax + E);           // (harmless if the final bound rules the block out)
+            };
+            // Marks of a block with largest value bmax and allowance E.  CONVERT: the rare cases after the group's four blocks, in one copy
+            // of their code (block `at`, its mask in `mask`): the loop over the groups shares the instruction cache with the converting warps
+            // (1.02M x 128, K = 1024: 436 us, with a copy per block 450; without those warps 298 and 282 us at D = 64).
+            auto mark = [&](const uint32_t (&v)[32], int at, int bn, float bmax, float E, unsigned& mask, unsigned& rest) {
                 const float cut = floor_now() - E;
                 if (in && bmax >= cut) {
                     // bit j of the mask: value j reaches the cut (the sign of l - cut; four chains of shifts, a byte each)
@@ -713,36 +932,17 @@ screen_sweep_kernel(const SweepParams p) {
                             m4[q] = __funnelshift_l(__float_as_uint(hi2(d)), m4[q], 1);
                             m4[q] = __funnelshift_l(__float_as_uint(lo2(d)), m4[q], 1);
                         }
-                    const unsigned mask = ~((m4[0] | (m4[1] << 8)) | ((m4[2] << 16) | (m4[3] << 24)));
-                    const float ub = bmax + E;
-                    // the block's largest upper bound, rounded up to the 24 bits that share a word with its number
-                    const unsigned ubits = (__float_as_uint(ub + fabsf(ub) * 1e-4f + 1e-3f) & ~255u) | (unsigned)bn;
-                    const unsigned long long w = ((unsigned long long)ubits << 32) | mask;
-                    const bool useful = cut > 0.5f * SCR_NEVER;      // (no useful bound yet: the values of positions without a component could
-                    if (useful && ne < SW_ENT) {                     // pass, so the row is evaluated in full)
-                        ent_s[256 * ne++] = w;
-                    } else if (!useful) {
-                        lost = CUDART_INF_F;
-                    } else {
-                        if (ne == SW_ENT + SW_SPILL && packs < 2) {  // drop what the bound found meanwhile rules out (of broad posteriors:
-                            int m = 0;                               // nothing; trying at every block took a millisecond per tile)
-                            ++packs;
-                            for (int e = 0; e < SW_ENT + SW_SPILL; ++e) {
-                                const unsigned long long o = ent(e);
-                                if (__uint_as_float((unsigned)(o >> 32) & ~255u) >= floor_now()) ent(m++) = o;
-                            }
-                            ne = m;
-                        }
-                        if (ne < SW_ENT + SW_SPILL) ent(ne++) = w;
-                        else lost = fmaxf(lost, ub);                 // (harmless if the final bound rules the block out)
-                    }
+                    mask = ~((m4[0] | (m4[1] << 8)) | ((m4[2] << 16) | (m4[3] << 24)));
+                    if (cut > 0.5f * SCR_NEVER && ne < S::ENT) ent_s[256 * ne++] = entry(bmax + E, bn, mask);
+                    else if (CONVERT) rest |= 1u << at;
+                    else later(bn, bmax, E, mask);
                 }
             };
             for (int gg = 0; gg < PASSES * NG; ++gg, ++gi) {
                 const bool last = gg + 1 == PASSES * NG, first = gg < NG;
                 const int g = (PASSES > 1 && !first) ? gg - NG : gg;
-                if (last) norm_load(i + 1);
-                const bool got = bar_wait(BAR(SB_LFULL + half), gi & 1u, abort_flag, p.status, false);
+                if (last) ahead(i + 1);
+                const bool got = bar_wait(BAR(S::LFULL + half), gi & 1u, abort_flag, p.status, false);
                 const bool ok = __all_sync(0xffffffffu, got);
                 fence_after();
                 if (last && i + 1 < ntl) operand(i + 1);     // (the tile's last products are done: its operand is free)
@@ -754,7 +954,7 @@ screen_sweep_kernel(const SweepParams p) {
                 tmem_ld32(col + 96, v3);
                 tmem_wait(v0); tmem_wait(v1); tmem_wait(v2); tmem_wait(v3);
                 fence_before();
-                bar_arrive(BAR(SB_LEMPTY + half));
+                bar_arrive(BAR(S::LEMPTY + half));
                 if (ok) {
                     // (the four blocks' maxima first, then their marks: four independent chains, and a bound that has seen the whole
                     // group; block by block the chains of one another kept the warp waiting)
@@ -783,10 +983,18 @@ screen_sweep_kernel(const SweepParams p) {
                         }
                     }
                     if (TOP == 1 || !first) {
-                        mark(v0, 4 * g, bm[0], E[0]);
-                        mark(v1, 4 * g + 1, bm[1], E[1]);
-                        mark(v2, 4 * g + 2, bm[2], E[2]);
-                        mark(v3, 4 * g + 3, bm[3], E[3]);
+                        unsigned mk[4] = {0u, 0u, 0u, 0u}, rest = 0u;
+                        mark(v0, 0, 4 * g, bm[0], E[0], mk[0], rest);
+                        mark(v1, 1, 4 * g + 1, bm[1], E[1], mk[1], rest);
+                        mark(v2, 2, 4 * g + 2, bm[2], E[2], mk[2], rest);
+                        mark(v3, 3, 4 * g + 3, bm[3], E[3], mk[3], rest);
+#pragma unroll 1
+                        while (rest) {
+                            const int j = __ffs(rest) - 1;
+                            rest &= rest - 1;
+                            later(4 * g + j, j == 0 ? bm[0] : j == 1 ? bm[1] : j == 2 ? bm[2] : bm[3], j == 0 ? E[0] : j == 1 ? E[1] : j == 2 ? E[2] : E[3],
+                                  j == 0 ? mk[0] : j == 1 ? mk[1] : j == 2 ? mk[2] : mk[3]);
+                        }
                     }
                 }
             }
@@ -796,17 +1004,17 @@ screen_sweep_kernel(const SweepParams p) {
             bool over = !(nrm < CUDART_INF_F) || (lost >= fin && lost > -CUDART_INF_F);
             // (the entries in shared memory all at once: one after the other, each waited for, they took ten times as long,
             // and the tensor cores waited with them)
-            unsigned long long we[SW_ENT];
+            unsigned long long we[S::ENT];
             unsigned keep = 0;
 #pragma unroll
-            for (int e = 0; e < SW_ENT; ++e) we[e] = ent_s[256 * e];
+            for (int e = 0; e < S::ENT; ++e) we[e] = ent_s[256 * e];
 #pragma unroll
-            for (int e = 0; e < SW_ENT; ++e)
+            for (int e = 0; e < S::ENT; ++e)
                 if (e < ne && __uint_as_float((unsigned)(we[e] >> 32) & ~255u) >= fin) {
                     cnt += __popc((unsigned)we[e]);
                     keep |= 1u << e;
                 }
-            for (int e = SW_ENT; e < ne; ++e) {
+            for (int e = S::ENT; e < ne; ++e) {
                 const unsigned long long w = ent(e);
                 if (__uint_as_float((unsigned)(w >> 32) & ~255u) >= fin) {
                     cnt += __popc((unsigned)w);
@@ -834,9 +1042,9 @@ screen_sweep_kernel(const SweepParams p) {
                     marks += cnt;
                     uint2* o = p.words + wrow * SCR_WORDS + wo;
 #pragma unroll
-                    for (int e = 0; e < SW_ENT; ++e)
+                    for (int e = 0; e < S::ENT; ++e)
                         if (keep >> e & 1u) *o++ = make_uint2((unsigned)we[e], (unsigned)(we[e] >> 32) & 255u);
-                    for (int e = SW_ENT; e < ne; ++e)
+                    for (int e = S::ENT; e < ne; ++e)
                         if (keep >> e & 1u) {
                             const unsigned long long w = ent(e);
                             *o++ = make_uint2((unsigned)w, (unsigned)(w >> 32) & 255u);
@@ -848,10 +1056,19 @@ screen_sweep_kernel(const SweepParams p) {
             marks = __reduce_add_sync(0xffffffffu, marks);
             if (lane == 0 && marks > 0) atomicAdd(p.ctl + SC_MARKS, marks);
         }
-    } else if (warp == SW_PRODUCER) {
-        // =========================== producer warp (TMA) ===========================
-        const uint32_t ubytes = 256u * 16u * (uint32_t)p.chunks;
-        uint32_t ps = 0, ut = 0, cslot = 0;                  // stages and tiles requested so far; slot of the group's constants
+    } else if (CONVERT && warp < S::PRODUCER) {
+        // =========================== converting warps: rows of X -> rows of u, |u|^2 ===========================
+        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
+        switch (screen_lane_shift(p.KS)) {
+            case 1: screen_convert<1>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
+            case 2: screen_convert<2>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
+            case 3: screen_convert<3>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
+            default: screen_convert<4>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
+        }
+    } else if (warp == S::PRODUCER) {
+        // =========================== producer warp (bulk copies of the coefficients) ===========================
+        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
+        uint32_t ps = 0, slot = 0, phase = 1, cslot = 0;     // stages requested so far; the next one's slot and its phase; slot of the group's constants
         bool ok = true;
         auto wait_slot = [&](int bar, uint32_t parity) -> bool {
             uint32_t w = 1;
@@ -862,40 +1079,42 @@ screen_sweep_kernel(const SweepParams p) {
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                          ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(bar) : "memory");
         };
+        uint32_t ut = 0;                                     // tiles whose rows have been requested
+        const uint32_t ubytes = 256u * 16u * (uint32_t)p.chunks;
         auto load_rows = [&](int64_t i) {
             if (elect_one()) {
                 const unsigned char* src = p.y + (size_t)((blockIdx.x + i * gridDim.x) * SCR_TILE) * p.chunks * 16;
-                bar_expect_tx(BAR(SB_UFULL), ubytes);
-                bulk(smem + SW_UOFF, src, ubytes, BAR(SB_UFULL));
+                bar_expect_tx(BAR(S::UFULL), ubytes);
+                bulk(smem + S::UOFF, src, ubytes, BAR(S::UFULL));
             }
             __syncwarp();
             ++ut;
         };
-        if (ntl > 0) load_rows(0);
+        if (!CONVERT && ntl > 0) load_rows(0);
         for (int64_t i = 0; i < ntl && ok; ++i)
             for (int g = 0; g < PASSES * NG && ok; ++g) {
                 for (int z = 0; z < spg && ok; ++z) {
-                    const uint32_t slot = ps % SW_PS;        // (a power of two)
-                    if (ps >= SW_PS) ok = wait_slot(SB_PEMPTY + slot, (ps / SW_PS - 1) & 1u);
+                    if (ps >= S::PS) ok = wait_slot(S::PEMPTY + slot, phase);
                     if (!ok) break;
                     if (elect_one()) {
                         const unsigned char* src = p.img + (size_t)(PASSES > 1 && g >= NG ? g - NG : g) * p.gbytes;
                         const uint32_t bytes = min(p.KA - 2 * z, 2) * 16384u;
-                        bar_expect_tx(BAR(SB_PFULL + slot), bytes + (z == 0 ? SW_CSLOT : 0));
-                        if (z == 0) bulk(cons + cslot * SW_CSLOT, src, SW_CSLOT, BAR(SB_PFULL + slot));
-                        bulk(smem + slot * SW_PSLOT, src + SW_CSLOT + z * SW_PSLOT, bytes, BAR(SB_PFULL + slot));
+                        bar_expect_tx(BAR(S::PFULL + slot), bytes + (z == 0 ? SW_CSLOT : 0));
+                        if (z == 0) bulk(cons + cslot * SW_CSLOT, src, SW_CSLOT, BAR(S::PFULL + slot));
+                        bulk(smem + slot * SW_PSLOT, src + SW_CSLOT + z * SW_PSLOT, bytes, BAR(S::PFULL + slot));
                     }
                     __syncwarp();
                     ++ps;
+                    if (++slot == S::PS) { slot = 0; phase ^= 1u; }
                 }
                 if (++cslot == (uint32_t)cslots) cslot = 0;
                 // the next tile's rows as soon as both halves have taken this tile's (which they do before its first products);
                 // no stage waits for that except behind the tile's last one
-                if (ok && ut == (uint32_t)(i + 1) && i + 1 < ntl) {
+                if (!CONVERT && ok && ut == (uint32_t)(i + 1) && i + 1 < ntl) {
                     uint32_t free_now = (g + 1 == PASSES * NG) ? 1u : 0u;
-                    if (free_now) ok = wait_slot(SB_UEMPTY, (uint32_t)(i & 1));
+                    if (free_now) ok = wait_slot(S::UEMPTY, (uint32_t)(i & 1));
                     else {
-                        if (lane == 0) free_now = bar_test(BAR(SB_UEMPTY), (uint32_t)(i & 1)) ? 1u : 0u;
+                        if (lane == 0) free_now = bar_test(BAR(S::UEMPTY), (uint32_t)(i & 1)) ? 1u : 0u;
                         free_now = __shfl_sync(0xffffffffu, free_now, 0);
                     }
                     if (ok && free_now) load_rows(i + 1);
@@ -903,24 +1122,64 @@ screen_sweep_kernel(const SweepParams p) {
             }
         // the loads in flight must have landed before the CTA may exit, also after an abort
         if (!ok || *abort_flag) {
-            for (uint32_t h = (ps > SW_PS ? ps - SW_PS : 0); h < ps; ++h) {
-                if (lane == 0) bar_wait(BAR(SB_PFULL + h % SW_PS), (h / SW_PS) & 1u, drain_flag, p.status, false);
+            for (uint32_t h = (ps > S::PS ? ps - S::PS : 0); h < ps; ++h) {
+                if (lane == 0) bar_wait(BAR(S::PFULL + h % S::PS), (h / S::PS) & 1u, drain_flag, p.status, false);
                 __syncwarp();
             }
-            if (ut > 0 && lane == 0) bar_wait(BAR(SB_UFULL), (ut - 1) & 1u, drain_flag, p.status, false);
+            if (!CONVERT && ut > 0 && lane == 0) bar_wait(BAR(S::UFULL), (ut - 1) & 1u, drain_flag, p.status, false);
+            __syncwarp();
+        }
+    } else if (CONVERT && warp == S::FETCH) {
+        // =========================== the warp that fetches X ===========================
+        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
+        const SweepRows rows(p, screen_lane_shift(p.KS));
+        const int total = (int)ntl * rows.per;
+        int c = 0;
+        bool ok = true;
+        for (int i = 0; i < (int)ntl && ok; ++i)
+            for (int k = 0; k < rows.per; ++k, ++c) {
+                const uint32_t full = BAR(S::XFULL + (c & 1));
+                if (c >= 2) {
+                    uint32_t w = 1;
+                    if (lane == 0) w = bar_wait(BAR(S::XEMPTY + (c & 1)), (uint32_t)((c >> 1) - 1) & 1u, abort_flag, p.status, false) ? 1u : 0u;
+                    ok = __shfl_sync(0xffffffffu, w, 0) != 0u;
+                    if (!ok) break;
+                }
+                const int row0 = rows.first + i * rows.tstep + k * rows.R;
+                uint32_t lo, bytes;
+                const bool bulk = rows.range(row0, lo, bytes);
+                if (elect_one()) {
+                    if (bulk) {
+                        bar_expect_tx(full, bytes);
+                        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                     ::"r"(smem_u32(smem + S::XOFF + (c & 1) * SW_XBYTES)), "l"(rows.xb + lo), "r"(bytes), "r"(full) : "memory");
+                    } else {
+                        bar_arrive(full);
+                    }
+                    // two chunks alone do not cover the trip to memory: the one after them is on its way into L2
+                    const int ahead = c + 2 >= total ? -1 : k + 2 < rows.per ? row0 + 2 * rows.R : row0 + 2 * rows.R + (k + 2) / rows.per * (rows.tstep - SCR_TILE);
+                    if (ahead >= 0 && rows.range(ahead, lo, bytes))
+                        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(rows.xb + lo), "r"(bytes) : "memory");
+                }
+                __syncwarp();
+            }
+        // the copies in flight must have landed before the CTA may exit, also after an abort
+        for (int q = c > 2 ? c - 2 : 0; q < c; ++q) {
+            if (lane == 0) bar_wait(BAR(S::XFULL + (q & 1)), (uint32_t)(q >> 1) & 1u, drain_flag, p.status, false);
             __syncwarp();
         }
     } else {
         // =========================== MMA warps, one per half ===========================
+        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
         // An instruction takes about as long to issue as the tensor cores take for it, and few are queued: every cycle spent
         // between two of them is idle time of the tensor cores unless the other half's warp fills it.  So there is a warp per
         // half, one thread of it does all (no votes, no shuffles), and a stage is waited for only when the instructions of the
         // stage before it have been issued.
-        const int h = warp - SW_MMA;
+        const int h = warp - S::MMA;
         if (elect_one()) {
             const uint32_t idesc = make_idesc(128, 128, 0);
             const uint64_t dp = make_desc(smem_u32(smem), 16, 1024);
-            const uint64_t dc = make_desc32(smem_u32(cons)), da = make_desc32(smem_u32(smem + SW_AOFF));
+            const uint64_t dc = make_desc32(smem_u32(cons)), da = make_desc32(smem_u32(smem + S::AOFF));
             const uint32_t d = tmem + h * 128, a = tmem + 256 + h * 128;
             const uint32_t bars0 = BAR(0);
             auto wait = [&](int bar, uint32_t parity) -> bool { return bar_wait(bars0 + 8 * bar, parity, abort_flag, p.status, false); };
@@ -929,10 +1188,10 @@ screen_sweep_kernel(const SweepParams p) {
             bool alive = true;
             for (int64_t i = 0; i < ntl && alive; ++i) {
                 for (int g = 0; g < PASSES * NG && alive; ++g, ++gi) {
-                    if (g == 0) alive = wait(SB_AFULL + h, (uint32_t)(i & 1));
-                    if (alive && gi >= 1) alive = wait(SB_LEMPTY + h, (gi - 1) & 1u);
+                    if (g == 0) alive = wait(S::AFULL + h, (uint32_t)(i & 1));
+                    if (alive && gi >= 1) alive = wait(S::LEMPTY + h, (gi - 1) & 1u);
                     for (int z = 0; z < spg && alive; ++z) {
-                        if (!wait(SB_PFULL + slot, parity)) { alive = false; break; }
+                        if (!wait(S::PFULL + slot, parity)) { alive = false; break; }
                         fence_after();
                         if (z == 0) mma_ss(d, da, dc + ((cslot * SW_CSLOT) >> 4), idesc, 0u);      // the constants
                         const int nk = p.KS - 8 * z;         // k-steps of this stage: at most eight
@@ -945,15 +1204,15 @@ screen_sweep_kernel(const SweepParams p) {
                             for (int j = 0; j < 7; ++j)
                                 if (j < nk) mma_ts(d, a + z * 64 + j * 8, b + (((j >> 2) * 16384 + (j & 3) * 32) >> 4), idesc, 1u);
                         }
-                        mma_commit(bars0 + 8 * (SB_PEMPTY + slot));
-                        if (++slot == SW_PS) { slot = 0; parity ^= 1u; }
+                        mma_commit(bars0 + 8 * (S::PEMPTY + slot));
+                        if (++slot == S::PS) { slot = 0; parity ^= 1u; }
                     }
-                    if (alive && !(p.test_silent == (int)blockIdx.x && gi == 0)) mma_commit(bars0 + 8 * (SB_LFULL + h));
+                    if (alive && !(p.test_silent == (int)blockIdx.x && gi == 0)) mma_commit(bars0 + 8 * (S::LFULL + h));
                     if (++cslot == (uint32_t)cslots) cslot = 0;
                 }
             }
-            mma_commit(bars0 + 8 * (SB_FINAL + h));
-            bar_wait(bars0 + 8 * (SB_FINAL + h), 0, drain_flag, p.status, false);
+            mma_commit(bars0 + 8 * (S::FINAL + h));
+            bar_wait(bars0 + 8 * (S::FINAL + h), 0, drain_flag, p.status, false);
             fence_after();
         }
         __syncwarp();
@@ -963,7 +1222,7 @@ screen_sweep_kernel(const SweepParams p) {
     // A CTA that left early has not written its points' lists, and what was in that memory before must not be taken for offsets and
     // components: nothing after this kernel does anything, also when a wait ran out.
     if (threadIdx.x == 0 && (abort_s != 0 || drain_s != 0)) p.ctl[SC_DENSE] = 1;
-    if (warp == SW_MMA) {
+    if (warp == S::MMA) {
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
@@ -1121,6 +1380,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                                                              int* __restrict__ counts, double* __restrict__ ll, float* __restrict__ logp,
                                                              int32_t* __restrict__ idx, int* __restrict__ ctl, const TopOut top) {
     if (ctl[SC_DENSE] != 0) return;
+    if (blockIdx.x == 0 && threadIdx.x < 3) ctl[SC_MARKS + threadIdx.x] = 0;       // (for the next piece's sweep)
     // (a piece is done with its last kernel: this one where there are no statistics)
     if ((MODE == SCREEN_LOGP || MODE == SCREEN_TOP) && blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_DONE] += 1;
     extern __shared__ int hist[];                    // [K] (unless MODE == SCREEN_LOGP)
@@ -1961,12 +2221,19 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
                                 int64_t* launches) {
     if (n < 1 || n > SCR_PIECE) return cudaErrorInvalidValue;
     const int KS = (D + 7) / 8;
-    int64_t blocks;
-    {
+    const int Kpad = screen_kpad(K), KA = screen_atoms(D);
+    SweepParams p;
+    p.n = n; p.KA = KA; p.KS = KS; p.NG = Kpad / 128; p.margin = margin;
+    p.chunks = screen_chunks(D); p.X = X; p.D = D; p.sd = b.sd; p.gd = b.gd; p.y = b.y; p.n2 = b.n2; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
+    p.blk = b.blk; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
+    p.ovf = b.ovf; p.ctl = b.ctl; p.status = status; p.test_silent = b.test_silent;
+    if (top < 1 || top > 4) return cudaErrorInvalidValue;
+    const bool convert = screen_converts(D, K);
+    if (!convert) {
         int L = 1;
         while (L < KS) L <<= 1;
         const int rpb = 256 / L;
-        blocks = (n + 2 * rpb - 1) / (2 * rpb);
+        int64_t blocks = (n + 2 * rpb - 1) / (2 * rpb);
         if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
 #define FG_TR(L_) screen_transform_kernel<L_><<<(unsigned)blocks, 256, 0, s>>>(X, n, D, screen_chunks(D), b.sd, b.gd, b.y, b.n2, b.ctl)
         switch (L) {
@@ -1978,20 +2245,16 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
         }
 #undef FG_TR
         LCHECK();
+        ++*launches;
     }
-    const int Kpad = screen_kpad(K), KA = screen_atoms(D);
-    SweepParams p;
-    p.n = n; p.KA = KA; p.KS = KS; p.NG = Kpad / 128; p.margin = margin;
-    p.chunks = screen_chunks(D); p.y = b.y; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
-    p.blk = b.blk; p.n2 = b.n2; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
-    p.ovf = b.ovf; p.ctl = b.ctl; p.status = status; p.test_silent = b.test_silent;
-    if (top < 1 || top > 4) return cudaErrorInvalidValue;
-    auto sweep = top == 1 ? screen_sweep_kernel<1> : top == 2 ? screen_sweep_kernel<2> : screen_sweep_kernel<4>;
-    cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, SW_SMEM);
+    auto sweep = convert ? (top == 1 ? screen_sweep_kernel<1, true> : top == 2 ? screen_sweep_kernel<2, true> : screen_sweep_kernel<4, true>)
+                         : (top == 1 ? screen_sweep_kernel<1, false> : top == 2 ? screen_sweep_kernel<2, false> : screen_sweep_kernel<4, false>);
+    const int sweep_smem = convert ? Sweep<true>::SMEM : Sweep<false>::SMEM;
+    cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, sweep_smem);
     if (e != cudaSuccess) return e;
     const int64_t tiles = (n + SCR_TILE - 1) / SCR_TILE;
     if (sms > SCR_MAX_SMS) sms = SCR_MAX_SMS;
-    sweep<<<(unsigned)(tiles < sms ? tiles : sms), SW_THREADS, SW_SMEM, s>>>(p);
+    sweep<<<(unsigned)(tiles < sms ? tiles : sms), convert ? Sweep<true>::THREADS : Sweep<false>::THREADS, sweep_smem, s>>>(p);
     LCHECK();
     const size_t smem = (size_t)OV_ROWS * K * 4;
     // (here and below the same limit from every call: it belongs to the kernel, which contexts on other threads launch for other K)
@@ -2000,7 +2263,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
     const double most = fmin((double)max_marks * (double)n, (double)SCR_PIECE * (stats ? SCR_MARKS : SCR_SLOTS));
     screen_rows_kernel<<<(unsigned)(2 * sms), 256, smem, s>>>(X, n, D, K, margin, top, (long long)most, mu, w2, c2d, b.ovf,
                                                               b.pt_off, b.pt_cnt, b.ids, b.ctl);
-    *launches += 3;
+    *launches += 2;
     return cudaGetLastError();
 }
 

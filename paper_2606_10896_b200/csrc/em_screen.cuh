@@ -25,7 +25,7 @@ constexpr int SCR_LL = 4096;                 // log-likelihood partial sums (one
 constexpr int SCR_DIM_BLOCKS = 64;
 constexpr int SCR_GROUP = 32768;             // points of a group that launch_screen_groups takes (16-bit cursors; one CTA sorts a group)
 constexpr int PR_ROWS = 4, PR_GROUPS = 16, PR_CTAS = 16;     // rows that are looked at ahead of a call's sweep: see screen_probe
-constexpr int SCR_SPILL = 22, SCR_MAX_SMS = 160;      // see screen_sweep_kernel
+constexpr int SCR_SPILL = 25, SCR_MAX_SMS = 160;      // see screen_sweep_kernel
 
 // Control words (in the context's result block, so that they travel to the host with the log-likelihood).
 enum { SC_DENSE = 0,      // set when a piece marks too many pairs or is not finite, or a wait ran out: later kernels return at once, the caller takes the dense path
@@ -82,7 +82,7 @@ struct ScreenProbe { const float* X; int64_t n; float margin; int top; float max
 // where the probed rows have too many pairs.  Clears the partial log-likelihoods.
 cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
                                   const ScreenProbe& probe, const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
-// One piece of n <= SCR_PIECE points: plane, sweep, rows without a list.  margin: log2 units below a point's best value down to
+// One piece of n <= SCR_PIECE points: (plane,) sweep, rows without a list.  margin: log2 units below a point's best value down to
 // which pairs are marked (40, or 0 for the arg-max alone); top: so many of its largest pairs are marked in any case (1 to 4).  max_marks: pairs per point up to which the screening pays; stats:
 // statistics are to follow, which have room for SCR_MARKS of them.
 cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, int top, float max_marks, bool stats,

@@ -65,6 +65,25 @@ def test_screen_against_oracle_at_the_edges_of_its_tiles(fg, monkeypatch, N, D, 
         _step(fg, c, X, pi, mu, var, K - 1, f"screen N={N} D={D} K={K}")
 
 
+# The sweep converts X itself (D > 64; D > 32 up to K = 512; any D up to K = 256) in chunks of 32 to 256 rows, by bulk copies that start
+# at 16-byte boundaries: X at any offset of 4 bytes, rows that are no multiple of 16 bytes, ragged last chunks, either side of the rule.
+@pytest.mark.parametrize("offset", [0, 1, 3])
+@pytest.mark.parametrize("N,D,K", [(31, 128, 64), (255, 99, 64), (289, 100, 130), (1055, 97, 64), (545, 65, 96), (577, 48, 512), (577, 48, 513), (320, 36, 64), (513, 72, 2049), (513, 32, 256), (513, 31, 257), (800, 9, 64)])
+def test_screen_takes_its_rows_from_anywhere(fg, monkeypatch, N, D, K, offset):
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    X, pi, mu, var = _mixture(N, D, K, 3 * N + D + K, collapsed=1)
+    X[N // 2, D - 1] = 4000.0                              # beyond the range of the 16-bit rows: evaluated in full
+    ref = orc.em_step(X, pi, mu, var)
+    flat = torch.empty(N * D + offset, dtype=torch.float32, device=DEV)
+    Xd = flat[offset:].view(N, D)
+    Xd.copy_(_t(X))
+    with fg.Context(0) as c:
+        Nk, S1, S2, L = c.gmm_em_step(Xd, _t(pi), _t(mu), _t(var))
+        assert c.gmm_last_path() == fg.GMM_PATH_TENSOR and c.gmm_last_exact_count() == K
+    assert abs(L - ref[3]) <= 1e-5 * abs(ref[3])
+    assert_stats_close(N, max(1.0, data_scale(X)), (Nk.cpu().numpy(), S1.cpu().numpy(), S2.cpu().numpy()), ref[:3], f"N={N} D={D} K={K} offset={offset}")
+
+
 def test_screen_accumulates_over_pieces_and_takes_unaligned_rows(fg, monkeypatch):
     monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
     monkeypatch.setenv("GMM_SCREEN_PIECE", "768")

@@ -45,6 +45,12 @@ namespace {
 // an allowance that rules nothing out (or coefficients beyond fp16).  Where the allowance of a typical point exceeds SCR_SHARP
 // bits, b is CAPPED at a value that leaves about 16: c - sum_d min(b, cap) (u - nu)^2 is an upper bound of log2 z, which is what
 // the screening needs, with a small allowance; only its lower bound is lost, so such components do not raise the threshold.
+//
+// k-means (unit): every component has the same weights, so sum_d b u^2 is the same for all of them and drops out of every comparison that
+// the sweep makes: the contraction has the linear terms alone, half as long, and
+//   alpha = eps sum_d b nu^2 + 2^-24 sum_d (2 b |nu| + b) + 2^-25 D / 2 + 2^-18 |c| + 0.02,   beta = eps max_d b + 1.5 x 2^-25.
+// The weight is F = min(1, min_d s_d^2) instead of 1, a power of two: with it b <= 1, and data of any size are screened in the units in
+// which the allowances are small (with weight 1 data ten times as large have allowances a hundred times as large).
 constexpr float SCR_SHARP = 40.f;
 constexpr float SCR_CAPPED = 1e30f;          // their sorting key
 constexpr float SCR_NEVER = -1.5e7f;         // c of a position without a component
@@ -135,6 +141,17 @@ __device__ __forceinline__ double warp_max(double v) {
     return v;
 }
 
+// F of the unit mixture, the same in every lane.
+__device__ __forceinline__ float screen_unit_weight(int D, const float* __restrict__ sd, int lane) {
+    float f = 1.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        if (lane + 32 * i < D) { const float s = __ldg(sd + lane + 32 * i); f = fminf(f, s * s); }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) f = fminf(f, __shfl_xor_sync(0xffffffffu, f, o));
+    return f;
+}
+
 // A warp per component: the FP32 kernels' derived parameters, the row's scale and constant, and the allowances above.
 __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const float* __restrict__ pi, const float* __restrict__ mu,
                                                           const float* __restrict__ var, int unit, const float* __restrict__ sd,
@@ -149,6 +166,7 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
     if (k >= K) return;
     double slog = 0.0, bv[4], nv[4];
     int bad = 0;
+    const float F = unit ? screen_unit_weight(D, sd, lane) : 1.f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int d = lane + 32 * i;
@@ -157,7 +175,7 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
         const float v = unit ? 1.f : __ldg(var + (size_t)k * D + d), m = __ldg(mu + (size_t)k * D + d);
         if (!(v > 0.f) || !isfinite(v)) bad |= ST_BAD_VAR;
         if (!isfinite(m)) bad |= ST_NONFINITE;
-        const double w = unit ? 1.0 : 0.72134752044448170368 / (double)v;
+        const double w = unit ? (double)F : 0.72134752044448170368 / (double)v;
         if (!unit) slog += log(6.283185307179586476925286766559 * (double)v);
         w2[(size_t)k * D + d] = (float)w;
         const double s = (double)__ldg(sd + d);
@@ -190,7 +208,11 @@ __global__ void __launch_bounds__(256) screen_comp_kernel(int D, int K, const fl
         bnn = warp_sum(bnn); absab = warp_sum(absab); bmax = warp_max(bmax); cmax = warp_max(cmax);
         c = cd - bnn;
         al = eps * bnn + 5.9604644775390625e-08 * absab + 2.98023223876953125e-08 * 0.5 * D + 3.814697265625e-06 * fabs(c) + 0.02;
-        be = 3.0 * eps * bmax + 2.98023223876953125e-08 * 1.5;
+        be = (unit ? 1.0 : 3.0) * eps * bmax + 2.98023223876953125e-08 * 1.5;
+        if (unit) {                                  // (a centroid that is too far from the others for 16 bits: the dense kernels)
+            if (!(cmax <= 60000.0) || !(bnn < -0.5 * (double)SCR_NEVER)) bad |= ST_NONFINITE;
+            break;
+        }
         if (capped || !(al + be * D > (double)SCR_SHARP || cmax > 60000.0)) break;
         capped = true;
     }
@@ -355,7 +377,7 @@ constexpr int SW_CSLOT = 4096;               // a group's constants: 128 rows of
 // its rank among the keys is its position, and it writes its own row (a sort of the keys in every CTA took 20 us).  The
 // coefficients are written as the sweep has them in shared memory (screen_group_bytes per group of 128 positions: the constants,
 // then the atoms of 32 dimensions, swizzled), so that a stage is one contiguous copy.
-__global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe, int D, int K, int Kpad, const float* __restrict__ mu,
+__global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe, int D, int K, int Kpad, int unit, const float* __restrict__ mu,
                                                            const float* __restrict__ w2, const float* __restrict__ sd,
                                                            const float* __restrict__ gd, const float4* __restrict__ prm,
                                                            const float* __restrict__ key, unsigned char* __restrict__ img,
@@ -388,8 +410,8 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe
         if (on) q = __ldg(prm + k);
     }
     const int r = pos & 127;
-    unsigned char* grp = img + (size_t)(pos >> 7) * screen_group_bytes(D);
-    const int ndim = (D + 7) / 8 * 8;
+    unsigned char* grp = img + (size_t)(pos >> 7) * screen_group_bytes(D, unit != 0);
+    const int nch = (D + 7) / 8, ndim = unit ? (nch + 1) / 2 * 16 : nch * 8;     // (unit: a k-step holds two chunks of u)
     for (int d = lane; d < ndim; d += 32) {                  // (in the order of screen_slot; beyond D: zeros)
         float a = 0.f, b = 0.f;
         if (on && d < D) {
@@ -401,7 +423,11 @@ __global__ void __launch_bounds__(256) screen_plane_kernel(const ProbeArgs probe
             b = (float)(-bd);
         }
         // k-step d / 8 holds eight dimensions of u and the same eight of u^2: two 16-byte chunks of a 128-byte row, swizzled
-        const int z = screen_slot(d, ndim >> 3);
+        const int z = d < 8 * nch ? screen_slot(d, nch) : d;
+        if (unit) {
+            *reinterpret_cast<__half*>(grp + SW_CSLOT + (z >> 6) * 16384 + r * 128 + ((((z >> 3) & 7) ^ (r & 7)) << 4) + 2 * (z & 7)) = __float2half_rn(a);
+            continue;
+        }
         unsigned char* o = grp + SW_CSLOT + (z >> 5) * 16384 + r * 128;
         const int c = 2 * ((z >> 3) & 3);
         *reinterpret_cast<__half*>(o + ((c ^ (r & 7)) << 4) + 2 * (z & 7)) = __float2half_rn(a);
@@ -552,7 +578,9 @@ __device__ __forceinline__ float max3(float a, float b, float c) { float r; asm(
 struct SweepParams {
     int64_t n;
     int KA, KS, NG;          // atoms and k-steps of the contraction, groups of 128 components
-    int chunks;              // 16-byte chunks of a row of u
+    int KC;                  // chunks of eight dimensions: a k-step has one and its squares, or (unit) two
+    int chunks;              // 16-byte chunks that a row of u takes
+    bool unit;
     const float* X;
     int D;
     const float *sd, *gd;
@@ -614,7 +642,7 @@ struct SweepRows {
         return row + R <= n && lo >= shift && hi <= end;
     }
 };
-__device__ __forceinline__ int screen_lane_shift(int KS) { return KS > 8 ? 4 : KS > 4 ? 3 : KS > 2 ? 2 : 1; }
+__device__ __forceinline__ int screen_lane_shift(int KC) { return KC > 8 ? 4 : KC > 4 ? 3 : KC > 2 ? 2 : 1; }
 
 template <int SH>
 __device__ __forceinline__ void screen_convert(const SweepParams& p, unsigned char* smem, int cw, int lane, int ntl, volatile int* abort_flag) {
@@ -622,8 +650,8 @@ __device__ __forceinline__ void screen_convert(const SweepParams& p, unsigned ch
     using S = Sweep<true>;
     const SweepRows rows(p, SH);
     const int D = p.D, l = lane & (L - 1), sub = lane >> SH;
-    const int d0 = 4 * l, d1 = 4 * (p.KS + l);               // dimensions of this lane: d0 .. d0 + 3 and d1 .. d1 + 3 (see screen_slot)
-    const bool on = l < p.KS;
+    const int d0 = 4 * l, d1 = 4 * (p.KC + l);               // dimensions of this lane: d0 .. d0 + 3 and d1 .. d1 + 3 (see screen_slot)
+    const bool on = l < p.KC;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BOFF);
     float* nrm_s = reinterpret_cast<float*>(smem + S::NOFF);
     const bool vec = ((D & 3) == 0) && rows.shift == 0, in0 = on && d0 < D, in1 = on && d1 < D;
@@ -821,11 +849,18 @@ screen_sweep_kernel(const SweepParams p) {
             const bool got = bar_wait(BAR(S::UFULL), (uint32_t)(i & 1), abort_flag, p.status, false);
             if (__all_sync(0xffffffffu, got)) {
 #pragma unroll 1
-                for (int z = 0; z < p.KA; z += 2) {          // (eight k-steps' loads in flight)
+                for (int q = 0; q < p.KC; q += 8) {          // (eight chunks' loads in flight)
                     uint4 v[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        v[j] = (4 * z + j < p.KS) ? urow[screen_place(4 * z + j, tid, p.chunks)] : make_uint4(0u, 0u, 0u, 0u);
+                        v[j] = (q + j < p.KC) ? urow[screen_place(q + j, tid, p.chunks)] : make_uint4(0u, 0u, 0u, 0u);
+                    if (p.unit) {                            // u alone
+                        uint32_t w[32];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) { w[4 * j] = v[j].x; w[4 * j + 1] = v[j].y; w[4 * j + 2] = v[j].z; w[4 * j + 3] = v[j].w; }
+                        tmem_st32(acol + (q >> 3) * 32, w);
+                        continue;
+                    }
 #pragma unroll
                     for (int y = 0; y < 2; ++y) {
                         uint32_t w[32];
@@ -840,7 +875,7 @@ screen_sweep_kernel(const SweepParams p) {
                                 w[8 * j + 4 + e] = *reinterpret_cast<const uint32_t*>(&sq);
                             }
                         }
-                        tmem_st32(acol + (z + y) * 32, w);   // (beyond the last atom: zeros into columns of this operand)
+                        tmem_st32(acol + ((q >> 2) + y) * 32, w);      // (beyond the last atom: zeros into columns of this operand)
                     }
                 }
                 if (CONVERT) nrm_next = nrm_s[tid];
@@ -1059,7 +1094,7 @@ screen_sweep_kernel(const SweepParams p) {
     } else if (CONVERT && warp < S::PRODUCER) {
         // =========================== converting warps: rows of X -> rows of u, |u|^2 ===========================
         if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
-        switch (screen_lane_shift(p.KS)) {
+        switch (screen_lane_shift(p.KC)) {
             case 1: screen_convert<1>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
             case 2: screen_convert<2>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
             case 3: screen_convert<3>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
@@ -1132,7 +1167,7 @@ screen_sweep_kernel(const SweepParams p) {
     } else if (CONVERT && warp == S::FETCH) {
         // =========================== the warp that fetches X ===========================
         if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
-        const SweepRows rows(p, screen_lane_shift(p.KS));
+        const SweepRows rows(p, screen_lane_shift(p.KC));
         const int total = (int)ntl * rows.per;
         int c = 0;
         bool ok = true;
@@ -1495,7 +1530,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
         }
         if (MODE == SCREEN_ARGMAX) {
             int near_n = 0;                                  // candidates within rounding of the best
-            const float near = 4e-6f * (fabsf(mx) + 300.f);
+            const float near = 4e-6f * (fabsf(mx) + 300.f * __ldg(w2));      // (w2: the unit mixture's weight, see above)
             for (int j = 0; j < todo; ++j) near_n += v_s[warp][p0 + j] >= mx - near ? 1 : 0;
             for (unsigned ties = __ballot_sync(0xffffffffu, near_n > 1); ties; ties &= ties - 1) {
                 const int src = __ffs(ties) - 1;
@@ -2178,14 +2213,15 @@ __global__ void __launch_bounds__(256, 4) screen_group_stats_kernel(const float*
 __global__ void __launch_bounds__(128) screen_centroids_kernel(int D, int K, const float* __restrict__ cent_in, const double* __restrict__ Nk,
                                                                const double* __restrict__ S1, const double* __restrict__ llk,
                                                                float* __restrict__ cent_out, int64_t* __restrict__ counts,
-                                                               double* __restrict__ inertia_k, const int* __restrict__ ctl) {
+                                                               double* __restrict__ inertia_k, const float* __restrict__ sd, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
     const int k = blockIdx.x, d = threadIdx.x;
+    const float F = d < 32 ? screen_unit_weight(D, sd, d) : 1.f;
     const double n = Nk[k];
     if (d < D) cent_out[(size_t)k * D + d] = n > 0.0 ? (float)(S1[(size_t)k * D + d] / n) : cent_in[(size_t)k * D + d];
     if (d == 0) {
         if (counts) counts[k] = (int64_t)(n + 0.5);
-        inertia_k[k] = -llk[k] / 0.69314718055994530942;
+        inertia_k[k] = -llk[k] / (0.69314718055994530942 * (double)F);
     }
 }
 
@@ -2212,26 +2248,26 @@ cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi,
     LCHECK();
     static_assert((size_t)PR_GROUPS * PR_ROWS * SCR_MAX_K <= (size_t)SCR_PAIRS, "the probe's bounds lie where the sorted pairs will");
     const ProbeArgs pr{probe, K, mu, w2, c2d, b.prm, b.key, b.probe, Kpad / 8, reinterpret_cast<float2*>(b.srt), b.ctl};
-    screen_plane_kernel<<<Kpad / 8 + (probe.n > 0 ? PR_GROUPS * PR_CTAS : 0), 256, 0, s>>>(pr, D, K, Kpad, mu, w2, b.sd, b.gd, b.prm, b.key, b.p, b.blk, b.comp_of);
+    screen_plane_kernel<<<Kpad / 8 + (probe.n > 0 ? PR_GROUPS * PR_CTAS : 0), 256, 0, s>>>(pr, D, K, Kpad, unit ? 1 : 0, mu, w2, b.sd, b.gd, b.prm, b.key, b.p, b.blk, b.comp_of);
     return cudaGetLastError();
 }
 
-cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, int top, float max_marks, bool stats,
+cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, bool unit, float margin, int top, float max_marks, bool stats,
                                 const float* mu, const float* w2, const double* c2d, const ScreenBuffers& b, int* status, int sms,
                                 int64_t* launches) {
     if (n < 1 || n > SCR_PIECE) return cudaErrorInvalidValue;
-    const int KS = (D + 7) / 8;
-    const int Kpad = screen_kpad(K), KA = screen_atoms(D);
+    const int KC = (D + 7) / 8, KS = unit ? (KC + 1) / 2 : KC;
+    const int Kpad = screen_kpad(K), KA = screen_atoms(D, unit);
     SweepParams p;
-    p.n = n; p.KA = KA; p.KS = KS; p.NG = Kpad / 128; p.margin = margin;
-    p.chunks = screen_chunks(D); p.X = X; p.D = D; p.sd = b.sd; p.gd = b.gd; p.y = b.y; p.n2 = b.n2; p.img = b.p; p.gbytes = (int)screen_group_bytes(D);
+    p.n = n; p.KA = KA; p.KS = KS; p.KC = KC; p.unit = unit; p.NG = Kpad / 128; p.margin = margin;
+    p.chunks = screen_chunks(D); p.X = X; p.D = D; p.sd = b.sd; p.gd = b.gd; p.y = b.y; p.n2 = b.n2; p.img = b.p; p.gbytes = (int)screen_group_bytes(D, unit);
     p.blk = b.blk; p.pt_off = b.pt_off; p.pt_cnt = b.pt_cnt; p.words = b.words; p.spill = b.spill;
     p.ovf = b.ovf; p.ctl = b.ctl; p.status = status; p.test_silent = b.test_silent;
     if (top < 1 || top > 4) return cudaErrorInvalidValue;
     const bool convert = screen_converts(D, K);
     if (!convert) {
         int L = 1;
-        while (L < KS) L <<= 1;
+        while (L < KC) L <<= 1;
         const int rpb = 256 / L;
         int64_t blocks = (n + 2 * rpb - 1) / (2 * rpb);
         if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
@@ -2344,7 +2380,7 @@ cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int
 
 cudaError_t launch_screen_centroids(cudaStream_t s, int D, int K, const float* cent_in, const double* Nk, const double* S1,
                                     const ScreenBuffers& b, float* cent_out, int64_t* counts, double* inertia_k) {
-    screen_centroids_kernel<<<K, 128, 0, s>>>(D, K, cent_in, Nk, S1, b.ll + SCR_LL, cent_out, counts, inertia_k, b.ctl);
+    screen_centroids_kernel<<<K, 128, 0, s>>>(D, K, cent_in, Nk, S1, b.ll + SCR_LL, cent_out, counts, inertia_k, b.sd, b.ctl);
     return cudaGetLastError();
 }
 

@@ -72,20 +72,21 @@ struct ScreenBuffers {
 
 bool screen_supports(int D, int K);
 inline int screen_kpad(int K) { return (K + 127) / 128 * 128; }
-inline int screen_atoms(int D) { return (D + 31) / 32; }
-__host__ __device__ inline size_t screen_group_bytes(int D) { return 4096 + (size_t)((D + 31) / 32) * 16384; }
+// (unit: the linear terms alone, see em_screen.cu)
+__host__ __device__ inline int screen_atoms(int D, bool unit) { return unit ? (D + 63) / 64 : (D + 31) / 32; }
+__host__ __device__ inline size_t screen_group_bytes(int D, bool unit = false) { return 4096 + (size_t)screen_atoms(D, unit) * 16384; }
 
 // A call's data X [n] (n = 0: none), of which some rows are looked at ahead of the sweep, and what the sweep will be asked (see launch_screen_sweep).
 struct ScreenProbe { const float* X; int64_t n; float margin; int top; float max_marks; };
 // Parameters -> w2, c2, c2d (as launch_prepare_fp32, with the same checks), coefficient plane and tables.  unit: k-means (mu =
-// centroids; pi, var not read; log2 z = -|x - mu|^2; one that is not finite sets SC_DENSE and no status).  SC_DENSE: 0, or 1
+// centroids; pi, var not read; log2 z = -F |x - mu|^2, F a power of two; one that is not finite or too far out sets SC_DENSE and no status).  SC_DENSE: 0, or 1
 // where the probed rows have too many pairs.  Clears the partial log-likelihoods.
 cudaError_t launch_screen_prepare(cudaStream_t s, int D, int K, const float* pi, const float* mu, const float* var, bool unit,
                                   const ScreenProbe& probe, const ScreenBuffers& b, float* w2, float* c2, double* c2d, int* status);
-// One piece of n <= SCR_PIECE points: (plane,) sweep, rows without a list.  margin: log2 units below a point's best value down to
+// One piece of n <= SCR_PIECE points: (plane,) sweep, rows without a list.  unit: as in launch_screen_prepare.  margin: log2 units below a point's best value down to
 // which pairs are marked (40, or 0 for the arg-max alone); top: so many of its largest pairs are marked in any case (1 to 4).  max_marks: pairs per point up to which the screening pays; stats:
 // statistics are to follow, which have room for SCR_MARKS of them.
-cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, float margin, int top, float max_marks, bool stats,
+cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D, int K, bool unit, float margin, int top, float max_marks, bool stats,
                                 const float* mu, const float* w2, const double* c2d, const ScreenBuffers& b, int* status, int sms,
                                 int64_t* launches);
 // SCREEN_ARGMAX: how near ties are decided.  g: NULL, or the centre of the FP32 tile kernel (then w = 1, c = 0); else weight and constant

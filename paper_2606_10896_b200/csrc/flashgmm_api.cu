@@ -920,7 +920,7 @@ int screen_begin(gmm_ctx* ctx, int D, int K, const float* pi, const float* mu, c
 int screen_values(gmm_ctx* ctx, int mode, const float* Xs, int64_t cnt, int D, int K, float margin, double limit, const float* mu,
                   float* logp, int32_t* idx, bool count, int m = 1, float* resp = nullptr, const ScreenTie* tie = nullptr) {
     const ScreenBuffers sb = ctx->screen();
-    CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, margin, mode == SCREEN_TOP ? m : 1, (float)limit, mode == SCREEN_EM || mode == SCREEN_ARGMAX, mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
+    CU(launch_screen_sweep(ctx->stream, Xs, cnt, D, K, mode == SCREEN_ARGMAX, margin, mode == SCREEN_TOP ? m : 1, (float)limit, mode == SCREEN_EM || mode == SCREEN_ARGMAX, mu, ctx->w2(), ctx->c2d(), sb, &ctx->result()->status, ctx->sms, &ctx->launches));
     KL(launch_screen_eval(ctx->stream, mode, Xs, cnt, D, K, mu, ctx->w2(), ctx->c2d(), sb, logp, idx, count, m, resp, tie));
     return GMM_OK;
 }

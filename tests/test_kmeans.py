@@ -130,3 +130,33 @@ def test_gpu_step_reports_what_is_not_finite_itself(monkeypatch, D, screened, wh
         a_r, _, _, _, gap = kmeans_step(X, C)
         assert np.all((a.cpu().numpy() == a_r) | (gap < 1e-3))
         ctx.gmm_sync_status()
+
+
+# The screening of the nearest centroid has the linear terms alone, two chunks of eight dimensions per step of the contraction: odd and even
+# numbers of chunks, both ways into the sweep, data of any size, dimensions of different sizes, a centroid far from everything.
+@pytest.mark.gpu
+@pytest.mark.parametrize("scale", [1.0, 700.0, 1e-2])
+@pytest.mark.parametrize("N,D,K", [(1500, 8, 64), (900, 17, 300), (1100, 40, 70), (700, 41, 600), (1300, 72, 130), (600, 100, 257), (2000, 128, 64)])
+def test_gpu_kmeans_screening_of_any_size(monkeypatch, N, D, K, scale):
+    import torch
+    from paper_2606_10896_b200 import flashgmm as fg
+
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    X, centers, _ = _blobs(N + D, N, D, K, spread=3.0)
+    X = (X * scale).astype(np.float32)
+    X[:, 0] *= 30.0
+    C = X[:K].copy()
+    C[K - 1] = 500.0 * scale
+    a_r, new_r, counts_r, inertia_r, gap = kmeans_step(X, C)
+    t = lambda v: torch.as_tensor(np.ascontiguousarray(v), device="cuda:0")
+    with fg.Context(0) as ctx:
+        a_d, new_d, counts_d, inertia = ctx.gmm_kmeans_step(t(X), t(C))
+    a = a_d.cpu().numpy()
+    # (float32 distances: D terms of the size of the largest, 2^-24 each, and the sum's own rounding)
+    d2 = ((X.astype(np.float64) - C.astype(np.float64)[a_r]) ** 2).sum(1)
+    assert np.all((a == a_r) | (gap <= 2.0 ** -20 * (d2 + 300.0)))
+    if np.array_equal(a, a_r):
+        size = np.abs(X).max()
+        np.testing.assert_allclose(new_d.cpu().numpy(), new_r, rtol=0, atol=1e-5 * size)
+        assert np.array_equal(counts_d.cpu().numpy(), counts_r)
+    assert abs(inertia - inertia_r) <= 1e-5 * inertia_r

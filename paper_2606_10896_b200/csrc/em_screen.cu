@@ -1834,18 +1834,23 @@ __global__ void __launch_bounds__(256) screen_fill_kernel(int64_t n, int K, int 
 
 // Statistics of one work item (at most SCR_SEG pairs of one component) by one warp: sums of r, r (x - mu), r (x - mu)^2 in
 // fp32, and, over the points whose only pair this is, their number and sum_d w2 (x - mu)^2 (their log-likelihood).  lpr lanes
-// per row, four dimensions each; the rows of four steps are in flight together.
+// per row, four dimensions each; the rows of four steps are in flight together.  The eight items of a CTA's step that belong to one
+// component are added in float64 before they leave: group g of eight items has one set of sums per component k in it, at place g + k
+// (a later set has a larger g or a larger k).  With a set per item the reduction read 20 MB per million points, 55 us at D = 128, K = 1024.
 __global__ void __launch_bounds__(256) screen_stats_kernel(const float* __restrict__ X, int D, int lpr, const float* __restrict__ mu,
                                                            const float* __restrict__ w2, const uint2* __restrict__ srt,
                                                            const int* __restrict__ off, const int* __restrict__ segoff,
-                                                           int K, float* __restrict__ part, const int* __restrict__ ctl) {
+                                                           int K, double* __restrict__ part, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
     extern __shared__ int seg_s[];                   // [K + 1]
+    __shared__ float sum_s[8][2 * 128 + 3];
+    __shared__ int k_s[8];
+    const int warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j <= K; j += 256) seg_s[j] = segoff[j];
     __syncthreads();
     const int lane = threadIdx.x & 31, l = lane % lpr, sub = lane / lpr, rows = 32 / lpr;
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-    const int items = seg_s[K], nw = gridDim.x * 8;
+    const int items = seg_s[K];
     const int d0 = 4 * l;
     auto load4 = [&](const float* __restrict__ r, bool v) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1859,7 +1864,9 @@ __global__ void __launch_bounds__(256) screen_stats_kernel(const float* __restri
         }
         return a;
     };
-    for (int item = blockIdx.x * 8 + (threadIdx.x >> 5); item < items; item += nw) {
+    for (int base = blockIdx.x * 8; base < items; base += gridDim.x * 8) {
+      const int item = base + warp;
+      if (item < items) {
         int k = 0;                                   // the component whose items hold this one: the last with segoff <= item
         for (int w = K; w > 1;) {
             const int h = w >> 1;
@@ -1913,62 +1920,70 @@ __global__ void __launch_bounds__(256) screen_stats_kernel(const float* __restri
             n1 += __shfl_xor_sync(0xffffffffu, n1, o);
             q1 += __shfl_xor_sync(0xffffffffu, q1, o);
         }
-        float* po = part + (size_t)item * (2 * D + 3);
+        float* po = sum_s[warp];
         if (sub == 0) {
             const float v1[4] = {s1.x, s1.y, s1.z, s1.w}, v2[4] = {s2.x, s2.y, s2.z, s2.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if (d0 + j < D) { po[d0 + j] = v1[j]; po[D + d0 + j] = v2[j]; }
         }
-        if (lane == 0) { po[2 * D] = nsum; po[2 * D + 1] = n1; po[2 * D + 2] = q1; }
+        if (lane == 0) { po[2 * D] = nsum; po[2 * D + 1] = n1; po[2 * D + 2] = q1; k_s[warp] = k; }
+      }
+      __syncthreads();
+      const int have = min(8, items - base);
+      for (int e = threadIdx.x; e < 2 * D + 3; e += 256) {
+        double t = (double)sum_s[0][e];
+        for (int w = 1; w <= have; ++w) {
+            if (w == have || k_s[w] != k_s[w - 1]) {
+                part[(size_t)(base / 8 + k_s[w - 1]) * (2 * D + 3) + e] = t;
+                t = 0.0;
+            }
+            if (w < have) t += (double)sum_s[w][e];
+        }
+      }
+      __syncthreads();
     }
 }
 
-// A CTA per component: its items in order (eight interleaved chains, then those in order), float64, shifted from its mean to
-// the origin.
-__global__ void __launch_bounds__(1024) screen_reduce_kernel(int D, int K, const float* __restrict__ part, const int* __restrict__ segoff,
-                                                             const float* __restrict__ mu, const double* __restrict__ c2d,
-                                                             double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
-                                                             double* __restrict__ llk, int* __restrict__ ctl) {
+// A CTA per component: its sets of sums in order (two interleaved chains), float64, shifted from its mean to the origin.
+__global__ void __launch_bounds__(512) screen_reduce_kernel(int D, int K, const double* __restrict__ part, const int* __restrict__ segoff,
+                                                            const float* __restrict__ mu, const double* __restrict__ c2d,
+                                                            double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
+                                                            double* __restrict__ llk, int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_DONE] += 1;
-    const int k = blockIdx.x, d = threadIdx.x & 127, r = threadIdx.x >> 7, chains = blockDim.x >> 7;      // (2 or 8)
+    const int k = blockIdx.x, d = threadIdx.x & 127, q = (threadIdx.x >> 7) & 1, c = threadIdx.x >> 8;
     const int i0 = segoff[k], i1 = segoff[k + 1];
     if (i0 == i1) return;
-    __shared__ double sh[8][128][2];
+    const int g0 = i0 / 8 + k, g1 = (i1 - 1) / 8 + k + 1;
+    __shared__ double sh[2][2][128];
     __shared__ double tot[3];
     const size_t st = (size_t)(2 * D + 3);
-    double a = 0.0, b = 0.0;
-    for (int i = i0 + r; i < i1; i += 4 * chains) {
-        float qa[4], qb[4];
+    double a = 0.0;
+    if (d < D)
+        for (int g = g0 + c; g < g1; g += 8) {
+            double v[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const bool in = i + chains * u < i1 && d < D;
-            const float* q = part + (size_t)(i + chains * u) * st;
-            qa[u] = in ? q[d] : 0.f;
-            qb[u] = in ? q[D + d] : 0.f;
+            for (int u = 0; u < 4; ++u) v[u] = g + 2 * u < g1 ? part[(size_t)(g + 2 * u) * st + q * D + d] : 0.0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) a += v[u];
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) { a += (double)qa[u]; b += (double)qb[u]; }
-    }
-    sh[r][d][0] = a;
-    sh[r][d][1] = b;
-    if (threadIdx.x < 96) {                              // warp q: the item's q-th scalar (weight, lone points, their quadratic forms)
-        const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        double s = 0.0;
-        for (int i = i0 + lane; i < i1; i += 32) s += (double)part[(size_t)i * st + 2 * D + q];
-        s = warp_sum(s);
-        if (lane == 0) tot[q] = s;
+    sh[c][q][d] = a;
+    if (threadIdx.x < 96) {                              // warp: a scalar of the sets (weight, lone points, their quadratic forms)
+        const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        double t = 0.0;
+        for (int g = g0 + lane; g < g1; g += 32) t += part[(size_t)g * st + 2 * D + which];
+        t = warp_sum(t);
+        if (lane == 0) tot[which] = t;
     }
     __syncthreads();
-    if (r != 0) return;
+    if (threadIdx.x >= 128) return;
     const double n = tot[0];
     if (d < D) {
-        a = b = 0.0;
-        for (int j = 0; j < chains; ++j) { a += sh[j][d][0]; b += sh[j][d][1]; }
+        const double s1 = sh[0][0][d] + sh[1][0][d], s2 = sh[0][1][d] + sh[1][1][d];
         const double m = (double)__ldg(mu + (size_t)k * D + d);
-        S1[(size_t)k * D + d] += a + m * n;
-        S2[(size_t)k * D + d] += b + 2.0 * m * a + m * m * n;
+        S1[(size_t)k * D + d] += s1 + m * n;
+        S2[(size_t)k * D + d] += s2 + 2.0 * m * s1 + m * m * n;
     }
     if (d == 0) {
         Nk[k] += n;
@@ -2351,8 +2366,7 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     while (4 * lpr < D) lpr <<= 1;
     screen_stats_kernel<<<148 * 6, 256, (size_t)(K + 1) * 4, s>>>(X, D, lpr, mu, w2, b.srt, b.off, b.segoff, K, b.part, b.ctl);
     LCHECK();
-    // (eight chains per dimension where components have many items; with a few, CTAs of 1024 threads were 28 us of mostly waiting)
-    screen_reduce_kernel<<<K, n >= (int64_t)512 * K ? 1024 : 256, 0, s>>>(D, K, b.part, b.segoff, mu, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
+    screen_reduce_kernel<<<K, 512, 0, s>>>(D, K, b.part, b.segoff, mu, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
     *launches += 4;
     return cudaGetLastError();
 }

@@ -186,6 +186,7 @@ ScratchLayout scratch_layout(int D, int K, bool planes, bool lists = true) {
         L.s_totals = take((size_t)K * 4);
         L.s_off = take((size_t)(K + 1) * 4);
         L.s_segoff = take((size_t)(K + 1) * 4);
+        static_assert(SCR_ITEMS * 4 >= (SCR_ITEMS / 8 + SCR_MAX_K + 1) * 8, "room for the sets of sums");
         L.s_part = take((size_t)SCR_ITEMS * (2 * (size_t)D + 3) * 4);
         L.s_ll = take((size_t)(SCR_LL + K) * 8);
         L.s_ovf = take((size_t)SCR_PIECE * 4);
@@ -331,7 +332,7 @@ struct gmm_ctx {
         b.totals = reinterpret_cast<int*>(at(lay.s_totals));
         b.off = reinterpret_cast<int*>(at(lay.s_off));
         b.segoff = reinterpret_cast<int*>(at(lay.s_segoff));
-        b.part = reinterpret_cast<float*>(at(lay.s_part));
+        b.part = reinterpret_cast<double*>(at(lay.s_part));
         b.ll = reinterpret_cast<double*>(at(lay.s_ll));
         b.ovf = reinterpret_cast<int*>(at(lay.s_ovf));
         b.ctl = result()->scr;

@@ -130,6 +130,10 @@ __global__ void __launch_bounds__(512) screen_dim_kernel(int D, int K, const flo
     }
 }
 
+// Whether the call has been left to the dense kernels, the same for all threads of the CTA: one of them reads the word.  For kernels in which a
+// CTA may find that out while another one starts: read by every thread for itself, some warps would leave and the others go on without them.
+__device__ __forceinline__ bool screen_off(const int* ctl) { return __syncthreads_or(threadIdx.x == 0 && __ldcg(ctl + SC_DENSE) != 0) != 0; }
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -465,7 +469,7 @@ template <int L>
 __global__ void __launch_bounds__(256) screen_transform_kernel(const float* __restrict__ X, int64_t n, int D, int chunks, const float* __restrict__ sd,
                                                                const float* __restrict__ gd, unsigned char* __restrict__ y,
                                                                float* __restrict__ n2, int* __restrict__ ctl) {
-    if (ctl[SC_DENSE] != 0) return;
+    if (screen_off(ctl)) return;
     const bool vec_ok = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
     const int l = threadIdx.x % L, KS = (D + 7) / 8;
     auto dim = [&](int j) { return l < KS ? (j < 4 ? 4 * l + j : 4 * (KS + l) + j - 4) : D; };       // (see screen_slot)
@@ -785,7 +789,7 @@ screen_sweep_kernel(const SweepParams p) {
     unsigned char* smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s, drain_s;
-    if (p.ctl[SC_DENSE] != 0) return;
+    if (screen_off(p.ctl)) return;
     volatile int* abort_flag = &abort_s;
     volatile int* drain_flag = &drain_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1279,7 +1283,7 @@ __global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restric
                                                           const double* __restrict__ c2d, const int* __restrict__ ovf,
                                                           unsigned* __restrict__ pt_off, int* __restrict__ pt_cnt,
                                                           unsigned short* __restrict__ ids, int* __restrict__ ctl) {
-    if (ctl[SC_DENSE] != 0) return;
+    if (screen_off(ctl)) return;
     const int rows = ctl[SC_OVF];
     if ((long long)rows * 32 > n + 1024 || (long long)ctl[SC_MARKS] > max_marks) {
         if (threadIdx.x == 0) ctl[SC_DENSE] = 1;     // (any number of CTAs may write the same value)
@@ -1998,7 +2002,7 @@ __global__ void __launch_bounds__(1024) screen_group_sort_kernel(int K, const in
                                                                 const unsigned* __restrict__ pt_off, const int* __restrict__ pt_cnt,
                                                                 const unsigned short* __restrict__ ids, const float* __restrict__ val,
                                                                 int* __restrict__ g_off, uint2* __restrict__ srt, int* __restrict__ ctl) {
-    if (ctl[SC_DENSE] != 0) return;
+    if (screen_off(ctl)) return;
     extern __shared__ int sm[];                      // base [K], then the warps' cursors [W][K rounded up to even] as 16-bit values
     __shared__ int wsum[32];
     const int K2 = (K + 1) & ~1;

@@ -45,3 +45,45 @@ def test_contexts_on_several_threads_take_different_shapes():
     for t in threads:
         t.join()
     assert not failures, failures
+
+
+def _unclean(fg, k, D, K, start, failures):
+    """Steps on data with an infinity in every tile of 256 points, in turn with clean data; the same bits in every round."""
+    stream = torch.cuda.Stream()
+    try:
+        with torch.cuda.stream(stream), fg.Context(0) as c:
+            g = torch.Generator(device=DEV)
+            g.manual_seed(k)
+            mu = torch.randn((K, D), device=DEV, generator=g) * 3
+            X = mu[torch.randint(0, K, (60_000,), device=DEV, generator=g)] + torch.randn((60_000, D), device=DEV, generator=g)
+            var, pi = torch.ones((K, D), device=DEV), torch.full((K,), 1 / K, device=DEV)
+            bad = X.clone()
+            bad[k::256, D - 1] = float("inf")
+            first = None
+            start.wait()
+            for _ in range(25):
+                out = list(c.gmm_kmeans_step(bad, mu)) + list(c.gmm_assign_topm(bad, pi, mu, var, 2))
+                c.gmm_sync_status()
+                out += list(c.gmm_kmeans_step(X, mu)) + list(c.gmm_em_step(X, pi, mu, var))
+                assert c.gmm_last_exact_count() == K
+                out = [v.cpu().numpy() if torch.is_tensor(v) else np.asarray(v) for v in out]
+                first = first or out
+                assert all(np.array_equal(u, v, equal_nan=True) for u, v in zip(first, out))
+    except Exception as e:      # (a thread's exception is the test's)
+        failures.append(f"K={K} D={D}: {e}")
+
+
+# The screening sweep finds values that are not finite while it runs, and CTAs that start later than that (beside another context's kernels
+# they do) leave as a whole or take part as a whole.
+def test_contexts_on_several_threads_meet_values_that_are_not_finite():
+    from paper_2606_10896_b200 import flashgmm as fg
+
+    failures = []
+    shapes = [(40, 64), (96, 300), (128, 64), (16, 200)]
+    start = threading.Barrier(len(shapes))
+    threads = [threading.Thread(target=_unclean, args=(fg, k, D, K, start, failures)) for k, (D, K) in enumerate(shapes)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failures, failures

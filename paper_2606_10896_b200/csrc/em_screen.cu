@@ -549,6 +549,7 @@ struct Sweep {
     enum { PFULL = 0, PEMPTY = PFULL + PS, UFULL = PEMPTY + PS, UEMPTY, AFULL, LFULL = AFULL + 2, LEMPTY = LFULL + 2, FINAL = LEMPTY + 2, XFULL = FINAL + 2,
            XEMPTY = XFULL + 2, COUNT = XEMPTY + 2 };
     static_assert(COUNT * 8 <= 256, "barriers");
+    static_assert(!CONVERT || (CONVERTER % 4 == 0 && THREADS % 128 == 0 && (SW_REGS * CONVERTER + SW_REGS_FEW * (THREADS / 32 - CONVERTER)) * 32 <= 65536), "registers of whole warpgroups");
     static_assert(SMEM <= 232448, "shared memory");
     static_assert(SPILL <= SCR_SPILL, "room for the spilled entries");
 };
@@ -831,6 +832,10 @@ screen_sweep_kernel(const SweepParams p) {
     fence_after();
     const uint32_t tmem = tmem_base_s;
 
+    // The warpgroups of the softmax warps (0 to 7) take the registers that the converting warps (8 to 11) and the last warpgroup give.  A warpgroup
+    // executes one instruction, so the last one, which has three roles, does so in the condition ahead of them.  (One for both of those
+    // warpgroups, ahead of the converting warps' branch: three registers more than there are, 12 bytes of spills.)
+    auto give_registers = [&]() { if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW)); };
     if (warp < S::CONVERTER) {
         // =========================== softmax warps: thread = TMEM lane = point ===========================
         if (CONVERT) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SW_REGS));
@@ -1097,16 +1102,15 @@ screen_sweep_kernel(const SweepParams p) {
         }
     } else if (CONVERT && warp < S::PRODUCER) {
         // =========================== converting warps: rows of X -> rows of u, |u|^2 ===========================
-        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
+        give_registers();
         switch (screen_lane_shift(p.KC)) {
             case 1: screen_convert<1>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
             case 2: screen_convert<2>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
             case 3: screen_convert<3>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
             default: screen_convert<4>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
         }
-    } else if (warp == S::PRODUCER) {
+    } else if (give_registers(), warp == S::PRODUCER) {
         // =========================== producer warp (bulk copies of the coefficients) ===========================
-        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
         uint32_t ps = 0, slot = 0, phase = 1, cslot = 0;     // stages requested so far; the next one's slot and its phase; slot of the group's constants
         bool ok = true;
         auto wait_slot = [&](int bar, uint32_t parity) -> bool {
@@ -1170,7 +1174,6 @@ screen_sweep_kernel(const SweepParams p) {
         }
     } else if (CONVERT && warp == S::FETCH) {
         // =========================== the warp that fetches X ===========================
-        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
         const SweepRows rows(p, screen_lane_shift(p.KC));
         const int total = (int)ntl * rows.per;
         int c = 0;
@@ -1209,7 +1212,6 @@ screen_sweep_kernel(const SweepParams p) {
         }
     } else {
         // =========================== MMA warps, one per half ===========================
-        if (CONVERT) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SW_REGS_FEW));
         // An instruction takes about as long to issue as the tensor cores take for it, and few are queued: every cycle spent
         // between two of them is idle time of the tensor cores unless the other half's warp fills it.  So there is a warp per
         // half, one thread of it does all (no votes, no shuffles), and a stage is waited for only when the instructions of the

@@ -31,3 +31,13 @@ def test_a_verdict_that_a_kernel_can_give_is_read_once_per_cta():
             seen.add(name)
             assert not re.search(r"if \((p\.)?ctl\[SC_DENSE\] != 0\) return", body), f"{name}: every thread decides for itself whether to leave"
     assert {"screen_sweep_kernel", "screen_transform_kernel", "screen_rows_kernel", "screen_group_sort_kernel"} <= seen
+
+
+def test_a_warpgroup_changes_its_registers_with_one_instruction():
+    """The sweep's roles: softmax warps (two warpgroups), converting warps (one), and three roles that share the last."""
+    body = dict(_kernels())["screen_sweep_kernel"]
+    give = body.index("auto give_registers")
+    assert body.count("setmaxnreg.dec") == 1 and give < body.index("setmaxnreg.dec") < body.index(";\n", give)
+    softmax, converting, last = (body.index(s) for s in ("if (warp < S::CONVERTER)", "else if (CONVERT && warp < S::PRODUCER)", "else if (give_registers(), warp == S::PRODUCER)"))
+    assert softmax < body.index("setmaxnreg.inc") < converting < last and body.count("setmaxnreg.inc") == 1
+    assert body[converting:last].count("give_registers()") == 1 and body[last:].count("give_registers()") == 1

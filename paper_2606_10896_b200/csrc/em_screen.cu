@@ -1163,15 +1163,13 @@ screen_sweep_kernel(const SweepParams p) {
                     if (ok && free_now) load_rows(i + 1);
                 }
             }
-        // the loads in flight must have landed before the CTA may exit, also after an abort
-        if (!ok || *abort_flag) {
-            for (uint32_t h = (ps > S::PS ? ps - S::PS : 0); h < ps; ++h) {
-                if (lane == 0) bar_wait(BAR(S::PFULL + h % S::PS), (h / S::PS) & 1u, drain_flag, p.status, false);
-                __syncwarp();
-            }
-            if (!CONVERT && ut > 0 && lane == 0) bar_wait(BAR(S::UFULL), (ut - 1) & 1u, drain_flag, p.status, false);
+        // the loads in flight must have landed before the CTA may exit, also where the others leave after the last one has been asked for
+        for (uint32_t h = (ps > S::PS ? ps - S::PS : 0); h < ps; ++h) {
+            if (lane == 0) bar_wait(BAR(S::PFULL + h % S::PS), (h / S::PS) & 1u, drain_flag, p.status, false);
             __syncwarp();
         }
+        if (!CONVERT && ut > 0 && lane == 0) bar_wait(BAR(S::UFULL), (ut - 1) & 1u, drain_flag, p.status, false);
+        __syncwarp();
     } else if (CONVERT && warp == S::FETCH) {
         // =========================== the warp that fetches X ===========================
         const SweepRows rows(p, screen_lane_shift(p.KC));

@@ -41,3 +41,13 @@ def test_a_warpgroup_changes_its_registers_with_one_instruction():
     softmax, converting, last = (body.index(s) for s in ("if (warp < S::CONVERTER)", "else if (CONVERT && warp < S::PRODUCER)", "else if (give_registers(), warp == S::PRODUCER)"))
     assert softmax < body.index("setmaxnreg.inc") < converting < last and body.count("setmaxnreg.inc") == 1
     assert body[converting:last].count("give_registers()") == 1 and body[last:].count("give_registers()") == 1
+
+
+def test_the_sweeps_loads_have_landed_before_it_ends_whoever_leaves_first():
+    """The softmax warps can leave (another CTA's verdict) when the producer has asked for everything and has seen no reason to leave itself."""
+    body = dict(_kernels())["screen_sweep_kernel"]
+    producer = body[body.index("warp == S::PRODUCER)"):body.index("warp == S::FETCH)")]
+    drain = producer.index("BAR(S::PFULL + h % S::PS)")
+    depth = producer[producer.index("{"):drain].count("{") - producer[producer.index("{"):drain].count("}")
+    assert depth == 2, "the loop over the last stages stands in the producer's own block, under no condition"
+    assert "if (!CONVERT && ut > 0 && lane == 0) bar_wait(BAR(S::UFULL)" in producer[drain:]

@@ -62,9 +62,11 @@ def _unclean(fg, k, D, K, start, failures):
             first = None
             start.wait()
             for _ in range(25):
-                out = list(c.gmm_kmeans_step(bad, mu)) + list(c.gmm_assign_topm(bad, pi, mu, var, 2))
-                c.gmm_sync_status()
-                out += list(c.gmm_kmeans_step(X, mu)) + list(c.gmm_em_step(X, pi, mu, var))
+                for call in (lambda: c.gmm_kmeans_step(bad, mu), lambda: (c.gmm_assign_topm(bad, pi, mu, var, 2), c.gmm_sync_status())):
+                    with pytest.raises(fg.GmmError) as e:
+                        call()
+                    assert e.value.code == fg.GMM_ENUMERIC
+                out = list(c.gmm_kmeans_step(X, mu)) + list(c.gmm_em_step(X, pi, mu, var))
                 assert c.gmm_last_exact_count() == K
                 out = [v.cpu().numpy() if torch.is_tensor(v) else np.asarray(v) for v in out]
                 first = first or out

@@ -664,9 +664,10 @@ __device__ __forceinline__ void screen_convert(const SweepParams& p, unsigned ch
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int d = j < 2 ? d0 + 2 * j : d1 + 2 * j - 4;
-        const float sa = d < D ? __ldg(p.sd + d) : 0.f, sb = d + 1 < D ? __ldg(p.sd + d + 1) : 0.f;
+        const bool a = on && d < D, b = on && d + 1 < D;     // (a lane without a chunk adds nothing to |u|^2)
+        const float sa = a ? __ldg(p.sd + d) : 0.f, sb = b ? __ldg(p.sd + d + 1) : 0.f;
         s2[j] = pack2(__float_as_uint(sa), __float_as_uint(sb));
-        g2[j] = pack2(__float_as_uint(d < D ? -sa * __ldg(p.gd + d) : 0.f), __float_as_uint(d + 1 < D ? -sb * __ldg(p.gd + d + 1) : 0.f));
+        g2[j] = pack2(__float_as_uint(a ? -sa * __ldg(p.gd + d) : 0.f), __float_as_uint(b ? -sb * __ldg(p.gd + d + 1) : 0.f));
     }
     // where this lane's 16 bytes of u go: row r0 + 4 RW h of a tile, r0 = cw RW + sub + 128 k (SH = 4: 32 k)
     const int rl = cw * RW + sub;

@@ -84,6 +84,38 @@ def test_screen_takes_its_rows_from_anywhere(fg, monkeypatch, N, D, K, offset):
     assert_stats_close(N, max(1.0, data_scale(X)), (Nk.cpu().numpy(), S1.cpu().numpy(), S2.cpu().numpy()), ref[:3], f"N={N} D={D} K={K} offset={offset}")
 
 
+# The bounds are in the data's own units about the mixture's mean, so moving data and mixture by the same vector changes no verdict.  Numbers of
+# chunks of eight dimensions that are no power of two (2, 3, 5, 9, 13), where a row has lanes without dimensions.
+@pytest.mark.parametrize("D", [9, 20, 40, 72, 100])
+def test_screen_takes_data_that_are_not_about_zero(fg, D):
+    N, K = 3000, 64
+    rng = np.random.default_rng(D)
+    centre = rng.normal(0, max(3.0, 30 / D ** 0.5), (K, D))
+    X0 = centre[rng.integers(0, K, N)] + rng.normal(size=(N, D))
+    pi, var = np.full(K, 1 / K, np.float32), np.ones((K, D), np.float32)
+    with fg.Context(0) as c:
+        def launches(call):
+            before = c.gmm_launch_count()
+            out = call()
+            return c.gmm_launch_count() - before, out
+
+        counts = []
+        for shift in (0.0, 30.0, -30.0, 1000.0):
+            X, mu = (X0 + shift).astype(np.float32), (centre + shift).astype(np.float32)
+            ref = orc.em_step(X, pi, mu, var)
+            n, got = launches(lambda: c.gmm_em_step(_t(X), _t(pi), _t(mu), _t(var)))
+            assert c.gmm_last_exact_count() == K, shift
+            counts.append((n, launches(lambda: c.gmm_kmeans_step(_t(X), _t(mu)))[0], launches(lambda: c.gmm_score_samples(_t(X), _t(pi), _t(mu), _t(var)))[0]))
+            assert abs(got[3] - ref[3]) <= 1e-5 * abs(ref[3])
+            assert_stats_close(N, data_scale(X), [v.cpu().numpy() for v in got[:3]], ref[:3], f"D={D} shift={shift}")
+        assert len(set(counts)) == 1, counts
+        X[7, 0] = np.inf                                   # (what a k-means step that goes on to the dense kernels launches)
+        before = c.gmm_launch_count()
+        with pytest.raises(fg.GmmError):
+            c.gmm_kmeans_step(_t(X), _t(mu))
+        assert c.gmm_launch_count() - before > counts[0][1]
+
+
 def test_screen_accumulates_over_pieces_and_takes_unaligned_rows(fg, monkeypatch):
     monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
     monkeypatch.setenv("GMM_SCREEN_PIECE", "768")

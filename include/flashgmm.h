@@ -284,7 +284,7 @@ int gmm_update_counts(gmm_ctx* ctx, int64_t* floored_variances, int64_t* empty_c
 
 /* Bytes of device scratch a context in GMM_PATH_AUTO holds for shape (D, K); independent of N.  Where the tensor
  * path runs (see gmm_auto_path) this includes 512 MiB for the fp16 planes of one launch-sized piece of the data, and for
- * D <= 128 up to 450 MiB of lists (a shape for which there is no room goes without the screening); forcing GMM_PATH_TENSOR on a shape AUTO sends to the FP32 path, or a screened call with
+ * D <= 128 up to 300 MiB of lists (a shape for which there is no room goes without the screening); forcing GMM_PATH_TENSOR on a shape AUTO sends to the FP32 path, or a screened call with
  * K < 64, adds the same. */
 size_t gmm_scratch_bytes(int D, int K);
 

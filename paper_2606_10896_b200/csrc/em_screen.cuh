@@ -63,7 +63,7 @@ struct ScreenBuffers {
     int* totals;          // [K]
     int* off;             // [K + 1] where a component's pairs start in srt
     int* segoff;          // [K + 1] where its work items start
-    double* part;         // [SCR_ITEMS / 8 + K + 1][2 D + 3] (see screen_stats_kernel)
+    double* part;         // [SCR_ITEMS / 8 + K][2 D + 3] (see screen_stats_kernel)
     double* ll;           // [SCR_LL + K]
     int* ovf;             // [SCR_PIECE]
     int* ctl;             // [SC_WORDS]

@@ -52,6 +52,10 @@ def test_host_only_entry_points(libpath):
     # Y for one launch of the tile kernel (2^19 points x 1 KB = 512 MiB) -- well under 1 GiB, whatever N is
     a = lib.gmm_scratch_bytes(128, 1024)
     assert (1 << 29) < a < (1 << 30)
+    # of which, beside the planes, the screening path's: 18 sorted pairs of 8 bytes per point of a piece of 2^20, 2048 counts of 4 bytes and 25088 / K + 1 sets of
+    # 2 D + 3 doubles per component, 24 MiB by point and SM; and the tile kernel's own 80 MiB at most
+    lists = 18 * (1 << 23) + 1024 * (2048 * 4) + (25088 + 1024) * 259 * 8 + (24 << 20)
+    assert a < (1 << 29) + lists + (80 << 20)
     assert lib.gmm_scratch_bytes(16, 8) < (1 << 27)       # shapes off the tensor path carry no planes
     assert lib.gmm_scratch_bytes(0, 5) == 0
     # a null context is rejected, not dereferenced

@@ -435,9 +435,9 @@ def test_host_streaming_takes_the_data_once_whatever_the_verdict(fg, D, K, broad
     assert_stats_close(N, data_scale(X), out[0][:3], ref[:3], f"K={K} broad={broad}")
 
 
-@pytest.mark.parametrize("D,K,N,left", [(128, 1024, 3000, 800), (96, 48, 200_000, 800)])
+@pytest.mark.parametrize("D,K,N,left", [(128, 1024, 3000, 770), (96, 48, 200_000, 770)])
 def test_screen_does_without_where_memory_is_short(fg, D, K, N, left):
-    """Room (in MiB) for what the dense kernels need, not for the lists on top: the call runs, as it does without a screening path, and the next
+    """Room (in MiB) for what the dense kernels need (at most 590), not for the planes and lists on top (816 in all at 128 x 1024, 783 at 96 x 48): the call runs, as it does without a screening path, and the next
     shape is screened again when there is room."""
     X, pi, mu, var = _mixture(N, D, K, 71)
     ref = orc.em_step(X, pi, mu, var)

@@ -534,11 +534,11 @@ struct Sweep {
     static constexpr int THREADS = CONVERT ? 512 : 352;      // 8 softmax warps, 4 that convert, producer warp, an MMA warp per half of the tile, a warp that fetches X
     static constexpr int CONVERTER = 8, PRODUCER = CONVERT ? 12 : 8, MMA = PRODUCER + 1, FETCH = 15;
     static constexpr int PS = CONVERT ? 3 : 4;               // coefficient stages
-    static constexpr int CSLOTS = CONVERT ? 3 : 2;           // groups in flight that have constants (rows of at most 8 chunks leave room for two more)
+    static constexpr int CSLOTS = CONVERT ? 3 : 4;           // groups in flight that have constants: as many as there are stages, of which a group takes one or two
     static constexpr int ENT = CONVERT ? 7 : 10;             // blocks of 32 components a point can have marks in: in shared memory,
     static constexpr int SPILL = 32 - ENT;                   // and, rarely needed, in global memory (a mask has 32 bits)
-    static constexpr int UOFF = PS * SW_PSLOT;               // the next tile's rows of u (256 x 16 chunks bytes)
-    static constexpr int COFF = UOFF + 65536;                // constants of the groups in flight
+    static constexpr int UOFF = PS * SW_PSLOT;               // the next tile's rows of u (256 x 16 chunks bytes; not CONVERT: 8 chunks at most)
+    static constexpr int COFF = UOFF + (CONVERT ? 65536 : 32768);                // constants of the groups in flight
     static constexpr int AOFF = COFF + CSLOTS * SW_CSLOT;    // the points' side of the constants: 128 rows (256, 1, 1, 0, ...)
     static constexpr int EOFF = AOFF + 4096;
     static constexpr int TOFF = EOFF + ENT * 256 * 8;        // allowances of every block
@@ -799,9 +799,7 @@ screen_sweep_kernel(const SweepParams p) {
     const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     constexpr int PASSES = TOP > 1 ? 2 : 1;
     const int NG = p.NG, spg = (p.KA + 1) >> 1;              // stages per group
-    unsigned char* cons = smem + S::COFF;                    // [cslots][4096]
-    const int cslots = CONVERT ? S::CSLOTS : S::PS / spg;
-    if (!CONVERT && p.chunks <= 8) cons = smem + S::UOFF + 32768;
+    unsigned char* cons = smem + S::COFF;                    // [CSLOTS][4096]
     float* nrm_s = reinterpret_cast<float*>(smem + S::NOFF);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BOFF);
     auto BAR = [&](int i) { return smem_u32(&bars[i]); };
@@ -1151,7 +1149,7 @@ screen_sweep_kernel(const SweepParams p) {
                     ++ps;
                     if (++slot == S::PS) { slot = 0; phase ^= 1u; }
                 }
-                if (++cslot == (uint32_t)cslots) cslot = 0;
+                if (++cslot == (uint32_t)S::CSLOTS) cslot = 0;
                 // the next tile's rows as soon as both halves have taken this tile's (which they do before its first products);
                 // no stage waits for that except behind the tile's last one
                 if (!CONVERT && ok && ut == (uint32_t)(i + 1) && i + 1 < ntl) {
@@ -1248,7 +1246,7 @@ screen_sweep_kernel(const SweepParams p) {
                         if (++slot == S::PS) { slot = 0; parity ^= 1u; }
                     }
                     if (alive && !(p.test_silent == (int)blockIdx.x && gi == 0)) mma_commit(bars0 + 8 * (S::LFULL + h));
-                    if (++cslot == (uint32_t)cslots) cslot = 0;
+                    if (++cslot == (uint32_t)S::CSLOTS) cslot = 0;
                 }
             }
             mma_commit(bars0 + 8 * (S::FINAL + h));
@@ -2286,6 +2284,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
     if (top < 1 || top > 4) return cudaErrorInvalidValue;
     const bool convert = screen_converts(D, K);
     if (!convert) {
+        if (D > 64) return cudaErrorInvalidValue;            // (the sweep that takes rows of u has room for 8 chunks)
         int L = 1;
         while (L < KC) L <<= 1;
         const int rpb = 256 / L;
@@ -2296,8 +2295,7 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
             case 1: FG_TR(1); break;
             case 2: FG_TR(2); break;
             case 4: FG_TR(4); break;
-            case 8: FG_TR(8); break;
-            default: FG_TR(16); break;
+            default: FG_TR(8); break;
         }
 #undef FG_TR
         LCHECK();

@@ -133,30 +133,37 @@ def test_gpu_step_reports_what_is_not_finite_itself(monkeypatch, D, screened, wh
 
 
 # The screening of the nearest centroid has the linear terms alone, two chunks of eight dimensions per step of the contraction: odd and even
-# numbers of chunks, both ways into the sweep, data of any size, dimensions of different sizes, a centroid far from everything.
+# numbers of chunks on both ways into the sweep (X converted by it; D <= 32 with K > 256 and D <= 64 with K > 512: rows of u), data of several sizes
+# and off zero, dimensions of different sizes, a centroid far from the others.
 @pytest.mark.gpu
-@pytest.mark.parametrize("scale", [1.0, 700.0, 1e-2])
-@pytest.mark.parametrize("N,D,K", [(1500, 8, 64), (900, 17, 300), (1100, 40, 70), (700, 41, 600), (1300, 72, 130), (600, 100, 257), (2000, 128, 64)])
-def test_gpu_kmeans_screening_of_any_size(monkeypatch, N, D, K, scale):
+@pytest.mark.parametrize("scale,shift", [(1.0, 0.0), (1.0, 300.0), (700.0, 0.0), (1e-2, 0.0)])
+@pytest.mark.parametrize("N,D,K", [(1500, 8, 64), (900, 17, 300), (1100, 16, 300), (1100, 40, 70), (700, 41, 600), (1300, 56, 600), (1300, 72, 130),
+                                   (600, 100, 257), (2000, 128, 64)])
+def test_gpu_kmeans_screening_of_any_size(monkeypatch, N, D, K, scale, shift):
     import torch
     from paper_2606_10896_b200 import flashgmm as fg
 
     monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
-    X, centers, _ = _blobs(N + D, N, D, K, spread=3.0)
-    X = (X * scale).astype(np.float32)
-    X[:, 0] *= 30.0
-    C = X[:K].copy()
-    C[K - 1] = 500.0 * scale
+    X, centers, _ = _blobs(N + D, N, D, K, spread=20.0)
+    C = centers + 0.3 * np.random.default_rng(K).normal(size=(K, D))
+    X[:, 0] *= 4.0
+    C[:, 0] *= 4.0
+    if K <= 130:
+        C[K - 1] = 500.0
+    X, C = ((v * scale + shift).astype(np.float32) for v in (X, C))
     a_r, new_r, counts_r, inertia_r, gap = kmeans_step(X, C)
+    # float32 distances, 2^-24 of the largest term per term and again for their sum, in a log-density with a constant below 300: no point is a near tie
+    d2 = ((X.astype(np.float64) - C.astype(np.float64)[a_r]) ** 2).sum(1)
+    assert np.all(gap > 2.0 ** -20 * (d2 + 300.0))
     t = lambda v: torch.as_tensor(np.ascontiguousarray(v), device="cuda:0")
     with fg.Context(0) as ctx:
         a_d, new_d, counts_d, inertia = ctx.gmm_kmeans_step(t(X), t(C))
-    a = a_d.cpu().numpy()
-    # (float32 distances: D terms of the size of the largest, 2^-24 each, and the sum's own rounding)
-    d2 = ((X.astype(np.float64) - C.astype(np.float64)[a_r]) ** 2).sum(1)
-    assert np.all((a == a_r) | (gap <= 2.0 ** -20 * (d2 + 300.0)))
-    if np.array_equal(a, a_r):
-        size = np.abs(X).max()
-        np.testing.assert_allclose(new_d.cpu().numpy(), new_r, rtol=0, atol=1e-5 * size)
-        assert np.array_equal(counts_d.cpu().numpy(), counts_r)
+        screened = ctx.gmm_launch_count()
+        X[N // 2, D - 1] = np.inf                              # (left to the dense kernels: their launches on top)
+        with pytest.raises(fg.GmmError):
+            ctx.gmm_kmeans_step(t(X), t(C))
+        assert screened < ctx.gmm_launch_count() - screened
+    assert np.array_equal(a_d.cpu().numpy(), a_r) and np.array_equal(counts_d.cpu().numpy(), counts_r)
+    # (a centroid: float32 sums over at most 64 points of differences from the old one, 2^-24 of its own size when it is stored)
+    np.testing.assert_allclose(new_d.cpu().numpy(), new_r, rtol=2.0 ** -23, atol=64 * 2.0 ** -24 * float(np.sqrt(d2.max())))
     assert abs(inertia - inertia_r) <= 1e-5 * inertia_r

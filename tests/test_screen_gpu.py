@@ -72,6 +72,8 @@ def test_screen_against_oracle_at_the_edges_of_its_tiles(fg, monkeypatch, N, D, 
 def test_screen_takes_its_rows_from_anywhere(fg, monkeypatch, N, D, K, offset):
     monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
     X, pi, mu, var = _mixture(N, D, K, 3 * N + D + K, collapsed=1)
+    off = (11.0 * (np.arange(D) % 5 - 1)).astype(np.float32)   # (a mean of its own in every dimension)
+    X, mu = X + off, mu + off
     X[N // 2, D - 1] = 4000.0                              # beyond the range of the 16-bit rows: evaluated in full
     ref = orc.em_step(X, pi, mu, var)
     flat = torch.empty(N * D + offset, dtype=torch.float32, device=DEV)

@@ -278,7 +278,7 @@ def main():
             timed_counts = exact_counts[-args.steps:]
             screened = sum(c > 0.75 * K for c in timed_counts) / len(timed_counts) if timed_counts else 0.0
             executed_factor = (4.0 * screened + 24.0 * (1.0 - screened)) / 8.0
-            timed_launch = ("screening path: transform, sweep, exact evaluation and statistics per piece of points" if screened > 0.5
+            timed_launch = ("screening path: sweep (with the conversion of the points), exact evaluation and statistics per piece of points" if screened > 0.5
                             else "tc_transform_kernel + em_tc_kernel per piece of points") + " (all inside the timed bracket)"
             traffic_key = "tensor" if screened == 0.0 else "screen"
     else:

@@ -49,8 +49,11 @@ namespace {
 // k-means (unit): every component has the same weights, so sum_d b u^2 is the same for all of them and drops out of every comparison that
 // the sweep makes: the contraction has the linear terms alone, half as long, and
 //   alpha = eps sum_d b nu^2 + 2^-24 sum_d (2 b |nu| + b) + 2^-25 D / 2 + 2^-18 |c| + 0.02,   beta = eps max_d b + 1.5 x 2^-25.
-// The weight is F = min(1, min_d s_d^2) instead of 1, a power of two: with it b <= 1, and data of any size are screened in the units in
-// which the allowances are small (with weight 1 data ten times as large have allowances a hundred times as large).
+// The weight is F = min(1, min_d s_d^2) instead of 1, a power of two: with it b <= 1, and data larger than size 1 are screened in units in
+// which the allowances are small (with weight 1 data ten times as large have allowances a hundred times as large).  Smaller data keep
+// weight 1, where the 0.02 of alpha is a squared distance like any other: it counts from where the two nearest centroids are about as close.
+// (Clusters of vectors of unit norm are screened as others, 300K x 96, K = 1024 292 us against 285.  F > 1 would have to look at X as well:
+// points far from centroids that are close to one another leave float32.)
 constexpr float SCR_SHARP = 40.f;
 constexpr float SCR_CAPPED = 1e30f;          // their sorting key
 constexpr float SCR_NEVER = -1.5e7f;         // c of a position without a component
@@ -553,10 +556,13 @@ struct Sweep {
     static_assert(SMEM <= 232448, "shared memory");
     static_assert(SPILL <= SCR_SPILL, "room for the spilled entries");
 };
-// Which way pays, measured per 1.02M points (us, converted by the sweep / sweep + transform; K = 256, 1024, 4096): D = 128: 238 / 264,
-// 442 / 534, 1468 / 1603; D = 80 (K = 256, 4096): 240 / 282, 1242 / 1420; D = 64: 141 / 170, 334 / 350, 1029 / 950; D = 48: 143 / 185, 359 / 359,
-// 1103 / 1025; D = 32: 114 / 129, 358 / 300, 1161 / 1082; D = 16 (K = 256): 102 / 113.  The transform costs about 1.06 us per dimension;
-// the converting warps cost the softmax warps issue slots and instruction cache, which matters where the MMAs are short.
+// Which way pays.  The line was drawn by the sweep of steps, per 1.02M points (us, converted by the sweep / sweep + transform; K = 256, 1024,
+// 4096): D = 128: 238 / 264, 442 / 534, 1468 / 1603; D = 80 (K = 256, 4096): 240 / 282, 1242 / 1420; D = 64: 141 / 170, 334 / 350, 1029 / 950;
+// D = 48: 143 / 185, 359 / 359, 1103 / 1025; D = 32: 114 / 129, 358 / 300, 1161 / 1082; D = 16 (K = 256): 102 / 113.  The transform costs about
+// 1.06 us per dimension; the converting warps cost the softmax warps issue slots and instruction cache, which matters where the MMAs are
+// short.  Whole calls with the roles' loops as they are now: steps 64 x 512 836 / 809, 64 x 1024 938 / 944, 48 x 1024 1052 / 1022, 32 x 1024
+// 966 / 908.  Half the contraction (k-means) and two passes (top-2) would put the line a little elsewhere: k-means 64 x 1024 620 / 660,
+// 32 x 1024 558 / 565, 32 x 4096 1226 / 1164; top-2 48 x 1024 1051 / 1079, 64 x 1024 1046 / 1022, 64 x 4096 2597 / 2362.
 inline bool screen_converts(int D, int K) { return D > 64 || (D > 32 && K <= 512) || K <= 256; }
 
 // two fp32 operations per instruction
@@ -775,7 +781,7 @@ __device__ __forceinline__ void screen_convert(const SweepParams& p, unsigned ch
 // MMA time per group: 2 x (ceil(D / 8) + 1) x 64.5 cycles; a group takes 2600 at D = 128 with 32 of them, a tile about 3000 more for its
 // list and the next one's operand, at the 1.65 to 1.75 GHz that the power limit leaves (27 tiles per CTA, K = 1024, not converting: 383 to 402 us
 // at D = 128, 261 to 282 at D = 64, where the softmax threads set the pace; block by block, each one's marks before the next one's
-// maxima: 400, 318).  Converting, the tensor cores are busy 58 % of the time instead of 69 %: the converting warps' instructions.  Pairs of
+// maxima: 400, 318).  Converting, the tensor cores are busy 59 % of the time instead of 69 %: the converting warps' instructions.  Pairs of
 // CTAs (cta_group::2, half the coefficients each) wait for each other's softmax threads: 550 us against 459 then.
 //
 // TOP: how many of a point's largest values are wanted for certain.  1: everything within the margin of the largest.  More (the top-m

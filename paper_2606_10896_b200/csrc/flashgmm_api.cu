@@ -875,7 +875,9 @@ int read_result(gmm_ctx* ctx, int slot, double* loglik) {
 // spread over the call's data, see screen_probe, then piece by piece) and return at once where it does not, so a call enqueues the
 // whole path, reads the verdict with its result and only then, if need be, runs the dense kernels: sparse posteriors cost no extra
 // synchronisation, broad ones about 60 us of preparation and launches.
-// Cost of screening in ns per point without the marked pairs: the sweep, and what else does not depend on them.
+// Cost of screening in ns per point without the marked pairs: the sweep, and what else does not depend on them.  (From when X had a pass of
+// its own in front of every sweep and k-means the full contraction: sweep and transform at 128 x 1024 0.52 ns then, 0.43 now, k-means
+// 0.33.  So screen_limit is a little lower there than those costs make it.)
 double screen_fixed(int D, int K) { return 0.15 + 0.001 * D + 0.045 * screen_kpad(K) / 128.0; }
 bool screen_wanted(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     if (ctx->path != GMM_PATH_AUTO || !ctx->lay.scr || !ctx->capPlanes || ctx->scr_marks == 0.0) return false;
@@ -893,7 +895,7 @@ bool dense_tensor(const gmm_ctx* ctx, int D, int K) {
 }
 // Marked pairs per point up to which the screening path is the cheaper one, from measured costs in ns per point: the dense kernels
 // 0.5 + 0.0032 K (0.62 at 10 x 100, 0.83 at 64 x 128, 2.1 at 12 x 541, 3.7 at 128 x 1024), the sweep and what does not depend on the
-// marks 0.15 + 0.001 D + 0.045 per 128 components, a pair 0.09 + 0.001 D.  (At most SCR_MARKS.)
+// marks 0.15 + 0.001 D + 0.045 per 128 components (see screen_fixed), a pair 0.09 + 0.001 D.  (At most SCR_MARKS.)
 // K < 64: the FP32 kernels' costs.
 double screen_limit(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     if (ctx->scr_marks > 0.0) return ctx->scr_marks;

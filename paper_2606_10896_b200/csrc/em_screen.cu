@@ -800,9 +800,10 @@ screen_sweep_kernel(const SweepParams p) {
     if (screen_off(p.ctl)) return;
     volatile int* abort_flag = &abort_s;
     volatile int* drain_flag = &drain_s;
-    // (warp: uniform for the compiler too, or each role's loop carries the bookkeeping of branches that lanes could take one by one: 3M points, 72 x 1024,
-    // log-densities 2113 -> 1975 us, k-means of 128 x 1024 1991 -> 1867)
-    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    // (role: the warp's number, uniform for the compiler too, by which the last warpgroup's roles part.  By `warp` each of their loops carries the
+    // bookkeeping of branches that lanes could take one by one: 3M points, 72 x 1024, log-densities 2113 -> 1975 us, k-means of 128 x 1024 1991 -> 1867.
+    // The other warpgroups have one role each and keep `warp`: top-2 of 1M x 128, K = 1024 1395 us, with `role` for all 1417.)
+    const int tid = threadIdx.x, warp = tid >> 5, role = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int64_t ntiles = (p.n + SCR_TILE - 1) / SCR_TILE;
     const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     constexpr int PASSES = TOP > 1 ? 2 : 1;
@@ -1116,7 +1117,7 @@ screen_sweep_kernel(const SweepParams p) {
             case 3: screen_convert<3>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
             default: screen_convert<4>(p, smem, warp - S::CONVERTER, lane, (int)ntl, abort_flag); break;
         }
-    } else if (give_registers(), warp == S::PRODUCER) {
+    } else if (give_registers(), role == S::PRODUCER) {
         // =========================== producer warp (bulk copies of the coefficients) ===========================
         uint32_t ps = 0, slot = 0, phase = 1, cslot = 0;     // stages requested so far; the next one's slot and its phase; slot of the group's constants
         bool ok = true;
@@ -1177,7 +1178,7 @@ screen_sweep_kernel(const SweepParams p) {
         }
         if (!CONVERT && ut > 0 && lane == 0) bar_wait(BAR(S::UFULL), (ut - 1) & 1u, drain_flag, p.status, false);
         __syncwarp();
-    } else if (CONVERT && warp == S::FETCH) {
+    } else if (CONVERT && role == S::FETCH) {
         // =========================== the warp that fetches X ===========================
         const SweepRows rows(p, screen_lane_shift(p.KC));
         const int total = (int)ntl * rows.per;
@@ -1221,7 +1222,7 @@ screen_sweep_kernel(const SweepParams p) {
         // between two of them is idle time of the tensor cores unless the other half's warp fills it.  So there is a warp per
         // half, one thread of it does all (no votes, no shuffles), and a stage is waited for only when the instructions of the
         // stage before it have been issued.
-        const int h = warp - S::MMA;
+        const int h = role - S::MMA;
         if (elect_one()) {
             const uint32_t idesc = make_idesc(128, 128, 0);
             const uint64_t dp = make_desc(smem_u32(smem), 16, 1024);

@@ -38,7 +38,7 @@ def test_a_warpgroup_changes_its_registers_with_one_instruction():
     body = dict(_kernels())["screen_sweep_kernel"]
     give = body.index("auto give_registers")
     assert body.count("setmaxnreg.dec") == 1 and give < body.index("setmaxnreg.dec") < body.index(";\n", give)
-    softmax, converting, last = (body.index(s) for s in ("if (warp < S::CONVERTER)", "else if (CONVERT && warp < S::PRODUCER)", "else if (give_registers(), warp == S::PRODUCER)"))
+    softmax, converting, last = (body.index(s) for s in ("if (warp < S::CONVERTER)", "else if (CONVERT && warp < S::PRODUCER)", "else if (give_registers(), role == S::PRODUCER)"))
     assert softmax < body.index("setmaxnreg.inc") < converting < last and body.count("setmaxnreg.inc") == 1
     assert body[converting:last].count("give_registers()") == 1 and body[last:].count("give_registers()") == 1
 
@@ -46,7 +46,7 @@ def test_a_warpgroup_changes_its_registers_with_one_instruction():
 def test_the_sweeps_loads_have_landed_before_it_ends_whoever_leaves_first():
     """The softmax warps can leave (another CTA's verdict) when the producer has asked for everything and has seen no reason to leave itself."""
     body = dict(_kernels())["screen_sweep_kernel"]
-    producer = body[body.index("warp == S::PRODUCER)"):body.index("warp == S::FETCH)")]
+    producer = body[body.index("role == S::PRODUCER)"):body.index("role == S::FETCH)")]
     drain = producer.index("BAR(S::PFULL + h % S::PS)")
     depth = producer[producer.index("{"):drain].count("{") - producer[producer.index("{"):drain].count("}")
     assert depth == 2, "the loop over the last stages stands in the producer's own block, under no condition"

@@ -572,6 +572,7 @@ __device__ __forceinline__ float hi2(uint64_t a) { return __uint_as_float((uint3
 __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) { uint64_t r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) { uint64_t r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) { uint64_t r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) { return fma2(b, 0xBF800000BF800000ull, a); }      // (a - b, rounded once)
 // Operand of one k-step: rows of 32 bytes, 32-byte swizzle, groups of eight rows 256 bytes apart.
 __device__ __forceinline__ uint64_t make_desc32(uint32_t saddr) {
     return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)1 << 16) | ((uint64_t)(256 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)6 << 61);
@@ -1377,11 +1378,19 @@ __global__ void __launch_bounds__(256) screen_rows_kernel(const float* __restric
 }
 
 // ------------------------------------------------------------------------------------------------------------------
-// Exact values.  A warp takes 32 points: their listed pairs (of the points that have more than one) go into a work list in
-// shared memory, four pairs are evaluated at a time, eight lanes each - a lane holds every eighth group of four dimensions -
-// and then a lane per point reads its values back.  (Eight lanes per POINT took the time of the longest of four lists.)
-// Bound by instruction issue and the trips to L2 for the components' rows (1 KB per pair at D = 128).
+// Exact values.  A CTA takes a range of consecutive points, a third of an SM each, all of a piece in one wave.  Points with one mark alone need no
+// value (of a step) and are done first.  The others are put in order of their first mark (`sorted`), so that points of one cluster,
+// whose marks are much the same, come together and the components' rows (1 KB per pair at D = 128) out of L1.  Then a warp takes 32 points
+// at a time, their marks as lists in shared memory, and four of them at once, eight lanes each: the point's row in registers, a lane with every eighth
+// group of four dimensions, the pairs' sums added up eight at a time, so that a step waits for nothing but its rows.
+// Bound by the trips of a step to L1 and L2 (1200 cycles with 24 warps on an SM) and their wavefronts.  1.2M x 100, K = 1000 (2.4 marks per point): 334 us with
+// four pairs of 32 consecutive points per step, each of which fetched the point's row and the component's rows, mostly from L2, and had its three shuffles
+// and its constant at its end; 231 now.  Not kept: rows of the next pair in flight (registers: two CTAs per SM), four rows of the first part per lane
+// (spills), prefetches of the points' rows into L2 (no gain).
 constexpr int EV_VALS = 32 * SCR_SLOTS;
+constexpr int EV_KEYS = 1024;                // keys of the sort (positions in the sweep, neighbours together beyond so many)
+constexpr int EV_RANGE = (int)((SCR_PIECE + SCR_RANGES - 1) / SCR_RANGES + 31) / 32 * 32;      // most points of a CTA
+constexpr int EV_BATCHES = EV_RANGE / 32 + 8;
 // TOP: the m (<= 4) largest values go out, the smaller component first where two are equal.
 struct TopOut { int m; float* resp; ScreenTie tie; };
 
@@ -1417,10 +1426,10 @@ __device__ int screen_nearest(const ScreenTie& tie, const float* __restrict__ x,
     return bk;
 }
 
-template <int MODE>
+template <int MODE, int NI>
 __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __restrict__ mu,
                                                              const float* __restrict__ w2, const double* __restrict__ c2d,
-                                                             const int* __restrict__ comp_of, int range, int pw,
+                                                             const int* __restrict__ comp_of, int range, int sorted,
                                                              const uint2* __restrict__ words,
                                                              const unsigned* __restrict__ pt_off, int* __restrict__ pt_cnt,
                                                              unsigned short* __restrict__ ids, float* __restrict__ val,
@@ -1430,140 +1439,123 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
     if (blockIdx.x == 0 && threadIdx.x < 3) ctl[SC_MARKS + threadIdx.x] = 0;       // (for the next piece's sweep)
     // (a piece is done with its last kernel: this one where there are no statistics)
     if ((MODE == SCREEN_LOGP || MODE == SCREEN_TOP) && blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_DONE] += 1;
-    extern __shared__ int hist[];                    // [K] (unless MODE == SCREEN_LOGP)
-    __shared__ float v_s[8][EV_VALS];                // values of the warp's pairs, by place in its part of the lists
-    __shared__ unsigned short k_s[8][EV_VALS];       // their positions in the sweep, then their components
-    __shared__ unsigned short w_s[8][EV_VALS];       // work list: point (5 bits), place (9 bits)
-    __shared__ double red[8];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l8 = lane & 7;
-    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0);
+    extern __shared__ int hist[];                    // [K] (unless MODE == SCREEN_LOGP or SCREEN_TOP), `keys`, `order`
+    __shared__ __align__(16) unsigned char work_s[8 * EV_VALS * 6];
+    __shared__ uint4 pt_s[8][32];                    // the points of a batch: row, where its pairs start here and in the lists, how many there are
+    __shared__ double ll_s[EV_BATCHES];              // log-likelihoods of the batches (a warp takes the next one when it is done with one)
+    __shared__ double red_s[8];
+    __shared__ int wsum[8];
+    __shared__ int next_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l8 = lane & 7, grp = lane >> 3;
+    float* const v_s = reinterpret_cast<float*>(work_s) + warp * EV_VALS;          // values of the warp's pairs
+    unsigned short* const k_s = reinterpret_cast<unsigned short*>(work_s + 8 * EV_VALS * 4) + warp * EV_VALS;       // their positions in the sweep, then their components
+    unsigned* const cur32 = reinterpret_cast<unsigned*>(work_s);                   // (while the points are sorted) [8][EV_KEYS] 16-bit cursors
     const bool histogram = MODE != SCREEN_LOGP && MODE != SCREEN_TOP && counts != nullptr;
-    if (histogram) {
+    short* const keys = reinterpret_cast<short*>(hist + (MODE != SCREEN_LOGP && MODE != SCREEN_TOP ? K : 0));       // [range] of the points of the last part; else -1
+    unsigned short* const order = reinterpret_cast<unsigned short*>(keys + range);                                  // [range] the points of the last part
+    if (histogram)
         for (int k = tid; k < K; k += 256) hist[k] = 0;
-        __syncthreads();
-    }
-    // c - sum_d w (x - m)^2, the same in the eight lanes that call together; dimensions 4 (l8 + 8 i) + (0..3)
-    auto pair_value = [&](const float* __restrict__ x, int k) -> float {
-        const float *m = mu + (size_t)k * D, *w = w2 + (size_t)k * D;
-        float q = 0.f;
-        if (vec) {
-            float4 a[4], b[4], c[4];
+    if (sorted)
+        for (int k = tid; k < 4 * EV_KEYS; k += 256) cur32[k] = 0u;
+    if (tid == 0) next_s = 0;
+    if (lane == 0) wsum[warp] = 0;
+    __syncthreads();
+    // A point's row, in the eight lanes that work on it: dimensions 4 (l8 + 8 i) + (0..3).  NI == 0: rows that cannot be read 16 bytes at a time.
+    constexpr int NX = NI > 0 ? NI : 1;
+    const bool tail = 4 * (l8 + 8 * (NX - 1)) < D;           // (the last group of four dimensions is there)
+    auto row_of = [&](const float* __restrict__ x, uint64_t (&xv)[2 * NX]) {
+        if constexpr (NI > 0) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int d = 4 * (l8 + 8 * i);
-                a[i] = b[i] = c[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (d < D) {
-                    a[i] = __ldg(reinterpret_cast<const float4*>(x + d));
-                    b[i] = __ldg(reinterpret_cast<const float4*>(m + d));
-                    c[i] = __ldg(reinterpret_cast<const float4*>(w + d));
-                }
+            for (int i = 0; i < NX; ++i) {
+                ulonglong2 a = make_ulonglong2(0ull, 0ull);
+                if (i < NX - 1 || tail) a = __ldg(reinterpret_cast<const ulonglong2*>(x) + l8 + 8 * i);
+                xv[2 * i] = a.x;
+                xv[2 * i + 1] = a.y;
             }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float t0 = a[i].x - b[i].x, t1 = a[i].y - b[i].y, t2 = a[i].z - b[i].z, t3 = a[i].w - b[i].w;
-                q = fmaf(c[i].x * t0, t0, q); q = fmaf(c[i].y * t1, t1, q); q = fmaf(c[i].z * t2, t2, q); q = fmaf(c[i].w * t3, t3, q);
-            }
-        } else {
-            for (int d = l8; d < D; d += 8) { const float t = __ldg(x + d) - __ldg(m + d); q = fmaf(__ldg(w + d) * t, t, q); }
         }
-        q += __shfl_xor_sync(0xffffffffu, q, 1);
-        q += __shfl_xor_sync(0xffffffffu, q, 2);
-        q += __shfl_xor_sync(0xffffffffu, q, 4);
-        return (float)(__ldg(c2d + k) - (double)q);
     };
-    double ll_acc = 0.0;
-    for (int it = 0; it < range / (8 * pw); ++it) {
-        const int64_t row0 = (int64_t)blockIdx.x * range + (it * 8 + warp) * pw, row = row0 + lane;
-        if (row0 >= n) break;
-        const bool in = lane < pw && row < n;
-        const int64_t part = row0 & ~(int64_t)31;                                // (32 points of the sweep share a part of the lists)
-        const int pc = in ? pt_cnt[row] : 0;
-        const unsigned off = in ? pt_off[row] : 0u, base = (unsigned)(part * SCR_SLOTS);
-        const bool listed = off < (unsigned)(SCR_PIECE * SCR_SLOTS);             // (else: a row with a list of its own length)
-        const int cnt = listed ? pc & 4095 : pc, nw = listed ? (pc >> 12) & 15 : 0;
-        const bool alone = cnt == 1 && MODE != SCREEN_LOGP;                      // its value is not needed here
-        const int todo = (!listed || alone) ? 0 : cnt;
-        int inc = todo;
+    // This lane's part of sum_d w (x - m)^2.
+    auto part_of = [&](const float* __restrict__ x, const uint64_t (&xv)[2 * NX], int k) -> float {
+        const float *m = mu + (size_t)k * D, *w = w2 + (size_t)k * D;
+        if constexpr (NI > 0) {
+            ulonglong2 b[NX], c[NX];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += u;
-        }
-        const int total = __shfl_sync(0xffffffffu, inc, 31), p0 = (int)(off - base);
-        int only = 0;
-        {   // the marks one by one
-            const uint2* wd = words + part * SCR_WORDS + (pc >> 16);
-            int q = inc - todo, at = p0;
-            for (int e = 0; e < nw; ++e) {
-                uint2 w = __ldg(wd + e);
-                while (w.x) {
-                    const int pos = (int)w.y * 32 + __ffs(w.x) - 1;
-                    w.x &= w.x - 1;
-                    only = pos;
-                    if (todo > 0) {
-                        k_s[warp][at] = (unsigned short)pos;
-                        w_s[warp][q++] = (unsigned short)((lane << 9) | at);
-                        ++at;
-                    }
+            for (int i = 0; i < NX; ++i) {
+                b[i] = c[i] = make_ulonglong2(0ull, 0ull);
+                if (i < NX - 1 || tail) {
+                    b[i] = __ldg(reinterpret_cast<const ulonglong2*>(m) + l8 + 8 * i);
+                    c[i] = __ldg(reinterpret_cast<const ulonglong2*>(w) + l8 + 8 * i);
                 }
             }
+            uint64_t q2 = 0ull;
+#pragma unroll
+            for (int i = 0; i < NX; ++i) {
+                const uint64_t t0 = sub2(xv[2 * i], b[i].x), t1 = sub2(xv[2 * i + 1], b[i].y);
+                q2 = fma2(mul2(c[i].x, t0), t0, q2);
+                q2 = fma2(mul2(c[i].y, t1), t1, q2);
+            }
+            return lo2(q2) + hi2(q2);
+        } else {
+            float q = 0.f;
+            for (int d = l8; d < D; d += 8) { const float t = __ldg(x + d) - __ldg(m + d); q = fmaf(__ldg(w + d) * t, t, q); }
+            return q;
         }
-        if (listed && alone) only = __ldg(comp_of + only);
-        __syncwarp();
-        int w_next = 0, k_next = 0;
-        auto fetch = [&](int s) {                            // (one step ahead of the values: the component's rows wait for it)
-            w_next = w_s[warp][min(s + (lane >> 3), total - 1)];
-            k_next = __ldg(comp_of + k_s[warp][w_next & 511]);
-        };
-        if (total > 0) fetch(0);
-        for (int s = 0; s < total; s += 4) {
-            const int w = w_next, k = k_next;
-            __syncwarp();
-            if (s + 4 < total) fetch(s + 4);
-            const float l = pair_value(X + (row0 + (w >> 9)) * D, k);
-            if (l8 == 0 && s + (lane >> 3) < total) { v_s[warp][w & 511] = l; k_s[warp][w & 511] = (unsigned short)k; }
-        }
-        __syncwarp();
+    };
+    auto value_of = [&](int k, float q) -> float { return (float)(__ldg(c2d + k) - (double)q); };
+    double ll_acc = 0.0;
+    const int64_t first = (int64_t)blockIdx.x * range;
+    const int rows = (int)((n - first < range) ? n - first : range);
+    // A point's list: where its words are, and how many marks they hold (off beyond the lists of the sweep: a list of its own length).
+    struct List { unsigned off; int cnt, nw; bool listed; };
+    auto list_of = [&](int64_t row, int pc) -> List {
+        List a;
+        a.off = pt_off[row];
+        a.listed = a.off < (unsigned)(SCR_PIECE * SCR_SLOTS);
+        a.cnt = a.listed ? pc & 4095 : pc;
+        a.nw = a.listed ? (pc >> 12) & 15 : 0;
+        return a;
+    };
+    auto words_of = [&](int64_t row, int pc) { return words + (row & ~(int64_t)31) * SCR_WORDS + (pc >> 16); };      // (32 points of the sweep share a part of the lists)
+    auto first_of = [&](const uint2* w) { const uint2 a = __ldg(w); return (int)a.y * 32 + __ffs(a.x) - 1; };
+    const int key_shift = K <= EV_KEYS ? 0 : 32 - __clz((K - 1) / EV_KEYS);        // (positions: below K rounded up to 128)
+
+    // ---- points whose values are not needed here, and rows with lists of their own length
+    for (int r0 = warp * 32; r0 < rows; r0 += 256) {
+        const int64_t row0 = first + r0, row = row0 + lane;
+        const bool in = r0 + lane < rows;
+        const int pc = in ? pt_cnt[row] : 0;
+        List a = {0u, 0, 0, true};
+        if (in) a = list_of(row, pc);
+        const bool alone = a.listed && a.cnt == 1 && MODE != SCREEN_LOGP, lone_list = a.cnt > 0 && !a.listed;
+        const bool todo = a.listed && a.cnt > 0 && !alone;
+        const unsigned todos = __ballot_sync(0xffffffffu, todo);
+        int mark = 0;
+        if (alone || (sorted && todo)) mark = first_of(words_of(row, pc));
+        const int key = todo ? min(mark >> key_shift, EV_KEYS - 1) : -1;
+        if (r0 + lane < range) keys[r0 + lane] = (short)key;
+        if (sorted) { if (todo) atomicAdd(cur32 + (warp * EV_KEYS + key) / 2, 1u << (16 * (key & 1))); }
+        else if (lane == 0) wsum[warp] += __popc(todos);
+        const int only = alone ? __ldg(comp_of + mark) : 0;
         float mx = -CUDART_INF_F, sum = 0.f;
         int best = only, kept = 0;
-        if (todo > 0) {
-            if (MODE == SCREEN_ARGMAX) {
-                mx = v_s[warp][p0];
-                best = k_s[warp][p0];
-                for (int j = 1; j < cnt; ++j) {
-                    const float l = v_s[warp][p0 + j];
-                    const int k = k_s[warp][p0 + j];
-                    if (l > mx || (l == mx && k < best)) { mx = l; best = k; }
-                }
-            } else {
-                for (int j = 0; j < cnt; ++j) mx = fmaxf(mx, v_s[warp][p0 + j]);
-                for (int j = 0; j < cnt; ++j) sum += fast_ex2(v_s[warp][p0 + j] - mx);
-            }
-        }
-        if (MODE == SCREEN_ARGMAX) {
-            int near_n = 0;                                  // candidates within rounding of the best
-            const float near = 4e-6f * (fabsf(mx) + 300.f * __ldg(w2));      // (w2: the unit mixture's weight, see above)
-            for (int j = 0; j < todo; ++j) near_n += v_s[warp][p0 + j] >= mx - near ? 1 : 0;
-            for (unsigned ties = __ballot_sync(0xffffffffu, near_n > 1); ties; ties &= ties - 1) {
-                const int src = __ffs(ties) - 1;
-                const int at = __shfl_sync(0xffffffffu, p0, src), n_c = __shfl_sync(0xffffffffu, todo, src);
-                const float top_v = __shfl_sync(0xffffffffu, mx, src), band = __shfl_sync(0xffffffffu, near, src);
-                const int k = screen_nearest(top.tie, X + (row0 + src) * D, D, mu, &v_s[warp][at], &k_s[warp][at], n_c, top_v, band, lane);
-                if (lane == src) best = k;
-            }
-        }
-        // rows with lists of their own length: the whole warp, one row after the other, values in `val`
-        for (unsigned todo_rows = __ballot_sync(0xffffffffu, in && !listed); todo_rows;) {
+        // the whole warp, one row after the other, values in `val`
+        for (unsigned todo_rows = __ballot_sync(0xffffffffu, lone_list); todo_rows;) {
             const int src = __ffs(todo_rows) - 1;
             todo_rows &= todo_rows - 1;
-            const int c = __shfl_sync(0xffffffffu, cnt, src);
-            const unsigned o = __shfl_sync(0xffffffffu, off, src);
+            const int c = __shfl_sync(0xffffffffu, a.cnt, src);
+            const unsigned o = __shfl_sync(0xffffffffu, a.off, src);
             float m = -CUDART_INF_F, sm = 0.f;
             int b = 0;
+            uint64_t xv[2 * NX];
+            row_of(X + (row0 + src) * D, xv);
             for (int s = 0; s < c; s += 4) {
                 const int j = min(s + (lane >> 3), c - 1);
                 const int k = ids[o + j];
-                const float l = pair_value(X + (row0 + src) * D, k);
+                float q = part_of(X + (row0 + src) * D, xv, k);
+                q += __shfl_xor_sync(0xffffffffu, q, 1);
+                q += __shfl_xor_sync(0xffffffffu, q, 2);
+                q += __shfl_xor_sync(0xffffffffu, q, 4);
+                const float l = value_of(k, q);
                 if (l8 == 0 && s + (lane >> 3) < c) {
                     val[o + j] = l;
                     if (MODE == SCREEN_ARGMAX) { if (l > m || (l == m && k < b)) { m = l; b = k; } }
@@ -1628,83 +1620,303 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                 }
             if (lane == src) { mx = m; sum = sm; best = b; kept = kp; }
         }
+        if (!in || todo) continue;
         if (MODE == SCREEN_TOP) {
-            if (in && listed) {
-                const float lz = mx + log2f(sum);
-                float pv = CUDART_INF_F;                     // the pair that went out last
-                int pk = -1;
+            if (!lone_list)
                 for (int r = 0; r < top.m; ++r) {
-                    float bv = -CUDART_INF_F;
-                    int bk = alone ? only : 0;
-                    for (int j = 0; j < todo; ++j) {
-                        const float v = v_s[warp][p0 + j];
-                        const int k = k_s[warp][p0 + j];
-                        if ((v < pv || (v == pv && k > pk)) && (v > bv || (v == bv && k < bk))) { bv = v; bk = k; }
-                    }
-                    idx[row * top.m + r] = bk;
-                    if (top.resp) top.resp[row * top.m + r] = alone ? 1.f : fast_ex2(bv - lz);
-                    pv = bv;
-                    pk = bk;
+                    idx[row * top.m + r] = only;
+                    if (top.resp) top.resp[row * top.m + r] = alone ? 1.f : CUDART_NAN_F;       // (not a number: no component has a weight)
                 }
-            }
         } else if (MODE == SCREEN_LOGP) {
-            if (in) {
-                const double lz = cnt > 0 ? (double)mx + (double)log2f(sum) : -CUDART_INF;
-                logp[row] = (float)(lz * 0.69314718055994530942);
-                ll_acc += lz;
-            }
+            const double lz = a.cnt > 0 ? (double)mx + (double)log2f(sum) : -CUDART_INF;
+            logp[row] = (float)(lz * 0.69314718055994530942);
+            ll_acc += lz;
         } else if (MODE == SCREEN_ARGMAX) {
-            if (in) {
-                if (idx) idx[row] = best;
-                if (histogram && cnt > 0) {
-                    ids[off] = (unsigned short)best;
-                    val[off] = -1.f;
-                    pt_cnt[row] = 1;
-                    atomicAdd(&hist[best], 1);
+            if (idx) idx[row] = best;
+            if (histogram && a.cnt > 0) {
+                ids[a.off] = (unsigned short)best;
+                val[a.off] = -1.f;
+                pt_cnt[row] = 1;
+                atomicAdd(&hist[best], 1);
+            }
+        } else if (a.cnt == 0) {
+            ll_acc += -CUDART_INF;
+        } else if (alone) {
+            ids[a.off] = (unsigned short)only;
+            val[a.off] = -1.f;
+            pt_cnt[row] = 1;
+            if (histogram) atomicAdd(&hist[only], 1);
+        } else {
+            ll_acc += (double)mx + (double)log2f(sum);
+            pt_cnt[row] = kept;
+        }
+    }
+    __syncthreads();
+
+    // ---- the others: by their first mark, or as they come
+    int work = 0;                                    // points of the last part
+    unsigned short* const cur = reinterpret_cast<unsigned short*>(cur32);
+    if (sorted) {
+        static_assert(EV_KEYS == 4 * 256, "four keys per thread");
+        int c4[4], own = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            c4[j] = 0;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                const int v = cur[w * EV_KEYS + 4 * tid + j];
+                cur[w * EV_KEYS + 4 * tid + j] = (unsigned short)c4[j];
+                c4[j] += v;
+            }
+            own += c4[j];
+        }
+        int inc = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += u;
+        }
+        if (lane == 31) wsum[warp] = inc;
+        __syncthreads();
+        int at = inc - own;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) at += wsum[w];
+            work += wsum[w];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+#pragma unroll
+            for (int w = 0; w < 8; ++w) cur[w * EV_KEYS + 4 * tid + j] += (unsigned short)at;
+            at += c4[j];
+        }
+        __syncthreads();
+        for (int r0 = warp * 32; r0 < rows; r0 += 256) {
+            const int key = r0 + lane < rows ? (int)keys[r0 + lane] : -1;
+            const unsigned peers = __match_any_sync(0xffffffffu, key);
+            const int rank = __popc(peers & ((1u << lane) - 1u));
+            int c = 0;
+            if (key >= 0) c = cur[warp * EV_KEYS + key];
+            __syncwarp();
+            if (key >= 0) {
+                if (rank == 0) cur[warp * EV_KEYS + key] = (unsigned short)(c + __popc(peers));
+                order[c + rank] = (unsigned short)(r0 + lane);
+            }
+            __syncwarp();
+        }
+    } else {
+        int at = 0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) at += wsum[w];
+            work += wsum[w];
+        }
+        for (int r0 = warp * 32; r0 < rows; r0 += 256) {
+            const bool todo = r0 + lane < rows && keys[r0 + lane] >= 0;
+            const unsigned todos = __ballot_sync(0xffffffffu, todo);
+            if (todo) order[at + __popc(todos & ((1u << lane) - 1u))] = (unsigned short)(r0 + lane);
+            at += __popc(todos);
+        }
+    }
+    __syncthreads();
+    const int pw = min(32, max(4, (work + 31) / 32 * 4));    // points of a batch: whole rounds of four, something for every warp
+
+    // ---- values
+    ll_acc = warp_sum(ll_acc);
+    if (lane == 0) red_s[warp] = ll_acc;
+    const int batches = (work + pw - 1) / pw;
+    for (;;) {
+        int bt = 0;
+        if (lane == 0) bt = atomicAdd(&next_s, 1);
+        bt = __shfl_sync(0xffffffffu, bt, 0);
+        if (bt >= batches) break;
+        const int j0 = bt * pw;
+        const bool in = lane < pw && j0 + lane < work;
+        const int at_row = in ? (int)order[j0 + lane] : 0;
+        const int64_t row = first + at_row;
+        const int pc = in ? pt_cnt[row] : 0;
+        List a = {0u, 0, 0, true};
+        if (in) a = list_of(row, pc);
+        int todo = a.cnt;
+        ll_acc = 0.0;
+        // (all of them unless points of several parts of the lists have more than EV_VALS pairs together)
+        while (__any_sync(0xffffffffu, todo > 0)) {
+            int inc = todo;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += u;
+            }
+            const int left = inc > EV_VALS ? todo : 0;
+            const int now = todo - left, total = (int)__reduce_max_sync(0xffffffffu, (unsigned)(now > 0 ? inc : 0)), p0 = inc - todo;
+            todo = left;
+            // the points in order of the number of their pairs (four of them are worked on at a time, as long as the longest list takes)
+            int rank = 0, points = 0;
+            const int cls = min(now, 8);
+#pragma unroll
+            for (int c = 8; c > 0; --c) {
+                const unsigned is = __ballot_sync(0xffffffffu, cls == c);
+                if (cls == c) rank = points + __popc(is & ((1u << lane) - 1u));
+                points += __popc(is);
+            }
+            if (now > 0) {   // the marks one by one
+                pt_s[warp][rank] = make_uint4((unsigned)at_row, (unsigned)p0, a.off, (unsigned)now);
+                const uint2* wd = words_of(row, pc);
+                int at = p0;
+                for (int e = 0; e < a.nw; ++e) {
+                    uint2 w = __ldg(wd + e);
+                    while (w.x) {
+                        k_s[at++] = (unsigned short)((int)w.y * 32 + __ffs(w.x) - 1);
+                        w.x &= w.x - 1;
+                    }
                 }
             }
-        } else if (in) {
-            // responsibilities; the pairs below 2^-40 of the total leave the list
-            if (cnt == 0) {
-                ll_acc += -CUDART_INF;
-            } else if (listed && alone) {
-                ids[off] = (unsigned short)only;
-                val[off] = -1.f;
-                pt_cnt[row] = 1;
-                if (histogram) atomicAdd(&hist[only], 1);
-            } else {
-                ll_acc += (double)mx + (double)log2f(sum);
-                if (listed) {
-                    const float lz = mx + log2f(sum);
-                    for (int j = 0; j < cnt; ++j) {
-                        const float r = fast_ex2(v_s[warp][p0 + j] - lz);
-                        if (r >= 9.094947e-13f) {
-                            const unsigned short id = k_s[warp][p0 + j];
-                            ids[off + kept] = id;
-                            val[off + kept] = r;
-                            ++kept;
-                            if (histogram) atomicAdd(&hist[id], 1);
+            __syncwarp();
+            for (int j = lane; j < total; j += 32) k_s[j] = (unsigned short)__ldg(comp_of + k_s[j]);
+            __syncwarp();
+            for (int r0 = 0; r0 < points; r0 += 4) {
+                const bool have = r0 + grp < points;
+                const uint4 pt = pt_s[warp][min(r0 + grp, points - 1)];
+                const int64_t prow = first + (int)pt.x;
+                const float* const x = X + prow * D;
+                const int cnt = have ? (int)pt.w : 0, steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)cnt);
+                const unsigned off = pt.z;
+                float* const pv = v_s + pt.y;
+                unsigned short* const pk = k_s + pt.y;
+                uint64_t xv[2 * NX];
+                row_of(x, xv);
+                // eight pairs' parts, then the sums: lane l8 gets that of pair j0 + l8
+                for (int j0 = 0; j0 < steps; j0 += 8) {
+                    float q[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        q[j] = 0.f;
+                        if (j0 + j < steps) q[j] = part_of(x, xv, pk[min(j0 + j, (int)pt.w - 1)]);
+                    }
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+                        for (int j = 0; j < o; ++j) {
+                            const float give = (l8 & o) ? q[j] : q[j + o], keep = (l8 & o) ? q[j + o] : q[j];
+                            q[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                        }
+                    if (j0 + l8 < cnt) pv[j0 + l8] = value_of(pk[j0 + l8], q[0]);
+                }
+                __syncwarp();
+                // the eight lanes of a point: its values, eight at a time
+                float mx = -CUDART_INF_F;
+                int best = 0x7fffffff;
+                for (int j = l8; j < cnt; j += 8) {
+                    const float l = pv[j];
+                    if (MODE == SCREEN_ARGMAX) {
+                        const int k = pk[j];
+                        if (l > mx || (l == mx && k < best)) { mx = l; best = k; }
+                    } else mx = fmaxf(mx, l);
+                }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    const float om = __shfl_xor_sync(0xffffffffu, mx, o);
+                    if (MODE == SCREEN_ARGMAX) {
+                        const int ob = __shfl_xor_sync(0xffffffffu, best, o);
+                        if (om > mx || (om == mx && ob < best)) { mx = om; best = ob; }
+                    } else mx = fmaxf(mx, om);
+                }
+                if (MODE == SCREEN_ARGMAX) {
+                    int near_n = 0;                                  // candidates within rounding of the best
+                    const float near = 4e-6f * (fabsf(mx) + 300.f * __ldg(w2));      // (w2: the unit mixture's weight, see above)
+                    for (int j = l8; j < cnt; j += 8) near_n += pv[j] >= mx - near ? 1 : 0;
+#pragma unroll
+                    for (int o = 4; o > 0; o >>= 1) near_n += __shfl_xor_sync(0xffffffffu, near_n, o);
+                    for (unsigned ties = __ballot_sync(0xffffffffu, l8 == 0 && near_n > 1); ties; ties &= ties - 1) {
+                        const int src = __ffs(ties) - 1;
+                        const int at = __shfl_sync(0xffffffffu, (int)pt.y, src), n_c = __shfl_sync(0xffffffffu, cnt, src);
+                        const float top_v = __shfl_sync(0xffffffffu, mx, src), band = __shfl_sync(0xffffffffu, near, src);
+                        const int r = __shfl_sync(0xffffffffu, (int)pt.x, src);
+                        const int k = screen_nearest(top.tie, X + (first + r) * D, D, mu, v_s + at, k_s + at, n_c, top_v, band, lane);
+                        if (lane == src) best = k;
+                    }
+                    if (have && l8 == 0) {
+                        if (idx) idx[prow] = best;
+                        if (histogram) {
+                            ids[off] = (unsigned short)best;
+                            val[off] = -1.f;
+                            pt_cnt[prow] = 1;
+                            atomicAdd(&hist[best], 1);
                         }
                     }
+                    continue;
                 }
-                pt_cnt[row] = kept;
+                float sum = 0.f;
+                for (int j = l8; j < cnt; j += 8) sum += fast_ex2(pv[j] - mx);
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                const float ls = log2f(sum), lz = mx + ls;
+                if (MODE == SCREEN_TOP) {
+                    float lv = CUDART_INF_F;                     // the pair that went out last
+                    int lk = -1;
+                    for (int r = 0; r < top.m; ++r) {
+                        float bv = -CUDART_INF_F;
+                        int bk = 0x7fffffff;
+                        for (int j = l8; j < cnt; j += 8) {
+                            const float v = pv[j];
+                            const int k = pk[j];
+                            if ((v < lv || (v == lv && k > lk)) && (v > bv || (v == bv && k < bk))) { bv = v; bk = k; }
+                        }
+#pragma unroll
+                        for (int o = 4; o > 0; o >>= 1) {
+                            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                            const int ok = __shfl_xor_sync(0xffffffffu, bk, o);
+                            if (ov > bv || (ov == bv && ok < bk)) { bv = ov; bk = ok; }
+                        }
+                        if (have && l8 == 0) {
+                            idx[prow * top.m + r] = bk == 0x7fffffff ? 0 : bk;
+                            if (top.resp) top.resp[prow * top.m + r] = fast_ex2(bv - lz);
+                        }
+                        lv = bv;
+                        lk = bk;
+                    }
+                    continue;
+                }
+                if (have && l8 == 0) {
+                    const double z = (double)mx + (double)ls;
+                    if (MODE == SCREEN_LOGP) logp[prow] = (float)(z * 0.69314718055994530942);
+                    ll_acc += z;
+                }
+                if (MODE == SCREEN_EM) {
+                    // responsibilities; the pairs below 2^-40 of the total leave the list
+                    int kept = 0;
+                    for (int j0 = 0; j0 < steps; j0 += 8) {
+                        const int j = j0 + l8;
+                        const float r = j < cnt ? fast_ex2(pv[j] - lz) : 0.f;
+                        const bool keep = r >= 9.094947e-13f;
+                        const unsigned mine = (__ballot_sync(0xffffffffu, keep) >> (8 * grp)) & 255u;
+                        if (keep) {
+                            const unsigned short id = pk[j];
+                            const int q = kept + __popc(mine & ((1u << l8) - 1u));
+                            ids[off + q] = id;
+                            val[off + q] = r;
+                            if (histogram) atomicAdd(&hist[id], 1);
+                        }
+                        kept += __popc(mine);
+                    }
+                    if (have && l8 == 0) pt_cnt[prow] = kept;
+                }
             }
+            __syncwarp();
         }
-        __syncwarp();
+        if (MODE == SCREEN_EM || MODE == SCREEN_LOGP) {
+            ll_acc = warp_sum(ll_acc);
+            if (lane == 0) ll_s[bt] = ll_acc;
+        }
     }
-    if (histogram) {
-        __syncthreads();
+    __syncthreads();
+    if (histogram)
         for (int k = tid; k < K; k += 256) counts[(size_t)blockIdx.x * K + k] = hist[k];
-    }
-    if (MODE != SCREEN_ARGMAX && MODE != SCREEN_TOP && ll) {
-        ll_acc = warp_sum(ll_acc);
-        if (lane == 0) red[warp] = ll_acc;
-        __syncthreads();
-        if (tid == 0) {
-            double s = 0.0;
-            for (int w = 0; w < 8; ++w) s += red[w];
-            ll[blockIdx.x] = s * 0.69314718055994530942 + ll[blockIdx.x];      // one owner per slot: launches add up
-        }
+    if ((MODE == SCREEN_EM || MODE == SCREEN_LOGP) && ll && warp == 0) {
+        double s = lane < 8 ? red_s[lane] : 0.0;
+        for (int b = lane; b < batches; b += 32) s += ll_s[b];
+        s = warp_sum(s);
+        if (lane == 0) ll[blockIdx.x] = s * 0.69314718055994530942 + ll[blockIdx.x];      // one owner per slot: launches add up
     }
 }
 
@@ -1783,53 +1995,50 @@ __global__ void __launch_bounds__(1024) screen_scan_kernel(int* __restrict__ cou
     }
 }
 
-// A CTA per range, a warp per eighth of it (at most 64 points), with cursors of its own: lanes = points, their pairs one after the other, the
-// pairs of one component ranked by lane.  The order is the same in every run.
-__global__ void __launch_bounds__(256) screen_fill_kernel(int64_t n, int K, int range, const unsigned* __restrict__ pt_off, const int* __restrict__ pt_cnt,
-                                                          const unsigned short* __restrict__ ids, const float* __restrict__ val,
-                                                          const int* __restrict__ starts, const int* __restrict__ off,
-                                                          uint2* __restrict__ srt, const int* __restrict__ ctl) {
+// A CTA per range, a warp per part of it (whole rounds of 32 points), with cursors of its own: lanes = points, their pairs one after the other,
+// the pairs of one component ranked by lane.  The order is the same in every run.
+__global__ void __launch_bounds__(1024) screen_fill_kernel(int64_t n, int K, int range, const unsigned* __restrict__ pt_off, const int* __restrict__ pt_cnt,
+                                                           const unsigned short* __restrict__ ids, const float* __restrict__ val,
+                                                           const int* __restrict__ starts, const int* __restrict__ off,
+                                                           uint2* __restrict__ srt, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
-    extern __shared__ int sm[];                      // base [K], then the warps' cursors [8][K rounded up to even] as 16-bit values
-    const int K2 = (K + 1) & ~1;
+    extern __shared__ int sm[];                      // base [K], then the warps' cursors [W][K rounded up to even] as 16-bit values
+    const int K2 = (K + 1) & ~1, W = blockDim.x >> 5;
     int* base = sm;
     unsigned* cur32 = reinterpret_cast<unsigned*>(sm + K2);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned short* cur = reinterpret_cast<unsigned short*>(cur32) + (size_t)warp * K2;
-    for (int k = tid; k < K; k += 256) base[k] = __ldg(off + k) + starts[(size_t)blockIdx.x * K + k];
-    for (int k = tid; k < 4 * K2; k += 256) cur32[k] = 0u;
+    for (int k = tid; k < K; k += blockDim.x) base[k] = __ldg(off + k) + starts[(size_t)blockIdx.x * K + k];
+    for (int k = tid; k < W * K2 / 2; k += blockDim.x) cur32[k] = 0u;
     __syncthreads();
-    const int64_t p0 = (int64_t)blockIdx.x * range + warp * (range / 8);
-    int cnt[2];
-    unsigned o[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int64_t row = p0 + 32 * h + lane;
-        const bool in = 32 * h + lane < range / 8 && row < n;
-        cnt[h] = in ? pt_cnt[row] : 0;
-        o[h] = in ? pt_off[row] : 0u;
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        for (int j = 0; j < cnt[h]; ++j) {
-            const int k = ids[o[h] + j];
+    const int part = ((range + W - 1) / W + 31) / 32 * 32;
+    const int64_t p0 = (int64_t)blockIdx.x * range, end = p0 + range < n ? p0 + range : n;
+    const int64_t w0 = p0 + warp * part, w1 = w0 + part < end ? w0 + part : end;
+    for (int64_t row = w0 + lane; row < w1; row += 32) {
+        const int c = pt_cnt[row];
+        const unsigned o = pt_off[row];
+        for (int j = 0; j < c; ++j) {
+            const int k = ids[o + j];
             atomicAdd(cur32 + ((size_t)warp * K2 + k) / 2, 1u << (16 * (k & 1)));
         }
-    __syncthreads();
-    for (int k = tid; k < K; k += 256) {
-        unsigned c = 0;
-        unsigned short* q = reinterpret_cast<unsigned short*>(cur32) + k;
-#pragma unroll
-        for (int w = 0; w < 8; ++w) { const unsigned v = q[(size_t)w * K2]; q[(size_t)w * K2] = (unsigned short)c; c += v; }
     }
     __syncthreads();
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int most = __reduce_max_sync(0xffffffffu, (unsigned)cnt[h]);
+    for (int k = tid; k < K; k += blockDim.x) {
+        unsigned c = 0;
+        unsigned short* q = reinterpret_cast<unsigned short*>(cur32) + k;
+#pragma unroll 8
+        for (int w = 0; w < W; ++w) { const unsigned v = q[(size_t)w * K2]; q[(size_t)w * K2] = (unsigned short)c; c += v; }
+    }
+    __syncthreads();
+    for (int64_t r0 = w0; r0 < w1; r0 += 32) {
+        const int64_t row = r0 + lane;
+        const int cnt = row < w1 ? pt_cnt[row] : 0;
+        const unsigned o = row < w1 ? pt_off[row] : 0u;
+        const int most = __reduce_max_sync(0xffffffffu, (unsigned)cnt);
         for (int j = 0; j < most; ++j) {
-            const bool on = j < cnt[h];
-            const int k = on ? ids[o[h] + j] : -1;
-            const float r = on ? val[o[h] + j] : 0.f;
+            const bool on = j < cnt;
+            const int k = on ? ids[o + j] : -1;
+            const float r = on ? val[o + j] : 0.f;
             const unsigned peers = __match_any_sync(0xffffffffu, k);
             const int rank = __popc(peers & ((1u << lane) - 1u));
             int c = 0;
@@ -1837,7 +2046,7 @@ __global__ void __launch_bounds__(256) screen_fill_kernel(int64_t n, int K, int 
             __syncwarp();
             if (on) {
                 if (rank == 0) cur[k] = (unsigned short)(c + __popc(peers));
-                srt[base[k] + c + rank] = make_uint2((unsigned)(p0 + 32 * h + lane), __float_as_uint(r));
+                srt[base[k] + c + rank] = make_uint2((unsigned)row, __float_as_uint(r));
             }
             __syncwarp();
         }
@@ -2260,8 +2469,15 @@ __global__ void __launch_bounds__(128) screen_centroids_kernel(int D, int K, con
 
 }  // namespace
 
-// Points per CTA of the evaluation and of the sort: more, smaller ranges where there are few points (at most SCR_RANGES of them).
-static int screen_range(int64_t n) { return n <= 65536 ? 128 : n <= 131072 ? 256 : SCR_RANGE; }
+// Points per CTA of the evaluation and of the sort by component: as many as make one wave of the evaluation (three CTAs per SM; two waves of half the
+// points: a step of 1M x 128, K = 1024 1159 us against 1084, two thirds of a wave 1123), at least 64, or 128 where the statistics sort them.
+static int screen_range(int64_t n, bool count) {
+    const int r = (int)((n + SCR_RANGES - 1) / SCR_RANGES + 31) / 32 * 32, least = count ? 128 : 64;
+    return r < least ? least : r;
+}
+// Whether the evaluation sorts a CTA's points: with about 450 of them and more it pays (us, sorted / as they come: a step of 128 x 1024 on 100K, 200K,
+// 300K points 228 / 220, 341 / 347, 399 / 418; top-2 of 64 x 512 174 / 164, 222 / 217, 267 / 269; scores of 96 x 512 143 / 141, 190 / 199, 226 / 238).
+static bool screen_sorts(int64_t n) { return n > 200000; }
 
 bool screen_supports(int D, int K) { return D >= 1 && D <= 128 && K >= 1 && K <= SCR_MAX_K; }
 
@@ -2332,22 +2548,36 @@ cudaError_t launch_screen_sweep(cudaStream_t s, const float* X, int64_t n, int D
 
 cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                const double* c2d, const ScreenBuffers& b, float* logp, int32_t* idx, bool count, int m, float* resp, const ScreenTie* tie) {
-    // 32 points per warp (fewer where that leaves the chip short of warps); ranges as launch_screen_stats has them
-    const int pw = n < 131072 ? 8 : n < 200000 ? 16 : 32, range = count ? screen_range(n) : 8 * pw;
+    // (ranges as launch_screen_stats has them)
+    const int range = screen_range(n, count), sorted = screen_sorts(n) ? 1 : 0;
     const unsigned blocks = (unsigned)((n + range - 1) / range);
-    const size_t smem = (size_t)K * 4;
+    const size_t smem_order = (size_t)range * 4, smem = (size_t)K * 4 + smem_order;
     int* counts = count ? b.counts : nullptr;
-    cudaError_t e = cudaFuncSetAttribute(screen_eval_kernel<SCREEN_EM>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(screen_eval_kernel<SCREEN_ARGMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4);
-    if (e != cudaSuccess) return e;
-    if (mode == SCREEN_EM)
-        screen_eval_kernel<SCREEN_EM><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, nullptr, nullptr, b.ctl, TopOut{});
-    else if (mode == SCREEN_LOGP)
-        screen_eval_kernel<SCREEN_LOGP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, b.ll, logp, nullptr, b.ctl, TopOut{});
-    else if (mode == SCREEN_TOP)
-        screen_eval_kernel<SCREEN_TOP><<<blocks, 256, 0, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, nullptr, nullptr, nullptr, idx, b.ctl, TopOut{m, resp, ScreenTie{}});
-    else
-        screen_eval_kernel<SCREEN_ARGMAX><<<blocks, 256, smem, s>>>(X, n, D, K, mu, w2, c2d, b.comp_of, range, pw, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, nullptr, nullptr, idx, b.ctl, TopOut{0, nullptr, tie ? *tie : ScreenTie{}});
+    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0) && ((reinterpret_cast<uintptr_t>(w2) & 15) == 0);
+    const TopOut out{m, resp, tie ? *tie : ScreenTie{}};
+#define FG_EVAL(M_, N_)                                                                                                                          \
+    do {                                                                                                                                         \
+        const cudaError_t e_ = cudaFuncSetAttribute(screen_eval_kernel<M_, N_>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4 + EV_RANGE * 4); \
+        if (e_ != cudaSuccess) return e_;                                                                                                        \
+        screen_eval_kernel<M_, N_><<<blocks, 256, (M_ == SCREEN_EM || M_ == SCREEN_ARGMAX) ? smem : smem_order, s>>>(X, n, D, K, mu, w2, c2d, \
+        b.comp_of, range, sorted, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, logp, idx, b.ctl, out);                       \
+    } while (0)
+#define FG_EVALS(M_)                                        \
+    switch (vec ? (D + 31) / 32 : 0) {                      \
+        case 0: FG_EVAL(M_, 0); break;                      \
+        case 1: FG_EVAL(M_, 1); break;                      \
+        case 2: FG_EVAL(M_, 2); break;                      \
+        case 3: FG_EVAL(M_, 3); break;                      \
+        default: FG_EVAL(M_, 4); break;                     \
+    }
+    switch (mode) {
+        case SCREEN_EM: FG_EVALS(SCREEN_EM) break;
+        case SCREEN_LOGP: FG_EVALS(SCREEN_LOGP) break;
+        case SCREEN_TOP: FG_EVALS(SCREEN_TOP) break;
+        default: FG_EVALS(SCREEN_ARGMAX) break;
+    }
+#undef FG_EVALS
+#undef FG_EVAL
     return cudaGetLastError();
 }
 
@@ -2365,14 +2595,18 @@ cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate
 
 cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                 const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches) {
-    const int range = screen_range(n), blocks = (int)((n + range - 1) / range);
+    const int range = screen_range(n, true), blocks = (int)((n + range - 1) / range);
     screen_scan_kernel<<<(K + 31) / 32, 1024, 0, s>>>(b.counts, blocks, K, b.totals, b.off, b.segoff, b.ctl);
     LCHECK();
     const int K2 = (K + 1) & ~1;
-    const size_t smem = (size_t)K2 * 4 + (size_t)K2 * 16;
-    cudaError_t e = cudaFuncSetAttribute(screen_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 20);
+    constexpr int FILL_CURSORS = 32768;                      // warps x components, 2 bytes each
+    // (at most 16 warps, so that the CTAs are one wave, four per SM at K = 1024: 1.2M x 100 50 us with 16, 80 with 32 - one and a half waves)
+    int warps = range / 32;
+    while (warps > 8 && (warps > 16 || warps * K2 > FILL_CURSORS)) --warps;
+    const size_t smem = (size_t)K2 * 4 + (size_t)K2 * 2 * warps;
+    cudaError_t e = cudaFuncSetAttribute(screen_fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4 + 2 * FILL_CURSORS);
     if (e != cudaSuccess) return e;
-    screen_fill_kernel<<<blocks, 256, smem, s>>>(n, K, range, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.off, b.srt, b.ctl);
+    screen_fill_kernel<<<blocks, warps * 32, smem, s>>>(n, K, range, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.off, b.srt, b.ctl);
     LCHECK();
     int lpr = 1;
     while (4 * lpr < D) lpr <<= 1;

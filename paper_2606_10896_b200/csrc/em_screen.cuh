@@ -12,7 +12,6 @@ constexpr int SCR_MAX_K = 4096;
 // (and 18.3 with 2^17: that X stays in L2 between the kernels does not make up for it).
 constexpr int64_t SCR_PIECE = 1 << 20;
 constexpr int SCR_TILE = 256;                // points per tile of the sweep
-constexpr int SCR_RANGE = 512;               // points per CTA of the pair evaluation and of the sort by component
 constexpr int SCR_SLOTS = 16;                // room for marked pairs per point (on average over the 32 points of a warp)
 constexpr int SCR_WORDS = 8;                 // room for words (32 positions, mask) per point, on average over the points of a warp
 constexpr int SCR_EXTRA = 2;                 // and, per point of a piece, for the rows that do not fit there
@@ -20,7 +19,7 @@ constexpr int64_t SCR_PAIRS = SCR_PIECE * (SCR_SLOTS + SCR_EXTRA);
 constexpr int SCR_SEG = 64;                  // pairs per work item of the statistics
 constexpr int SCR_MARKS = 10;                // marked pairs of a piece, per point of a full one: beyond them the piece counts as dense
 constexpr int64_t SCR_ITEMS = SCR_PIECE * (SCR_MARKS + SCR_EXTRA) / SCR_SEG + SCR_MAX_K;
-constexpr int SCR_RANGES = (int)(SCR_PIECE / SCR_RANGE);
+constexpr int SCR_RANGES = 3 * 148;          // CTAs of the pair evaluation and of the sort by component (at most)
 constexpr int SCR_LL = 4096;                 // log-likelihood partial sums (one per CTA of a launch), then one per component
 constexpr int SCR_DIM_BLOCKS = 64;
 constexpr int SCR_GROUP = 32768;             // points of a group that launch_screen_groups takes (16-bit cursors; one CTA sorts a group)

@@ -260,6 +260,40 @@ def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
 
 
 # the top-m assignment through the sweep: a point far away from everything, components without a weight (fewer than m with one, once)
+# Beyond 200,000 points the evaluation sorts a CTA's points by their marks.  A point's values do not depend on the points it is worked on with, so they are
+# the same bits as from two calls that do not sort.  Every other point has 24 marks: 32 of those together have more than a warp has room for at a time.
+@pytest.mark.parametrize("N,D,K,offset", [(200_001, 128, 96, 0), (200_100, 100, 64, 0), (213_121, 64, 1100, 0), (231_000, 24, 2100, 0), (200_193, 32, 64, 1), (200_031, 9, 64, 0)])
+def test_screen_values_are_those_of_smaller_calls(fg, monkeypatch, N, D, K, offset):
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    gen = torch.Generator(device=DEV).manual_seed(N + D)
+    mu = 12.0 / D ** 0.5 * torch.randn((K, D), device=DEV, generator=gen) * (1 + 8 / D)
+    mu[1:24] = mu[0] + 0.05 * torch.randn((23, D), device=DEV, generator=gen)
+    c = torch.randint(24, K, (N,), device=DEV, generator=gen)
+    c[::2] = torch.randint(0, 24, (len(c[::2]),), device=DEV, generator=gen)
+    flat = torch.empty(N * D + offset, device=DEV)
+    X = flat[offset:].view(N, D)
+    X.copy_(mu[c] + torch.randn((N, D), device=DEV, generator=gen))
+    pi, var = torch.full((K,), 1.0 / K, device=DEV), torch.ones((K, D), device=DEV)
+    cut = 390 * 256                                        # (whole tiles: which rows find no room in a tile's lists is not for the comparison)
+    with fg.Context(0) as ctx:
+        def call(x):
+            before = ctx.gmm_launch_count()
+            logp, _ = ctx.gmm_score_samples(x, pi, mu, var)
+            assert ctx.gmm_launch_count() - before < 12                # (nothing was left to the dense kernels)
+            idx, resp = ctx.gmm_assign_topm(x, pi, mu, var, 2)
+            near = ctx.gmm_kmeans_step(x, mu)[0]
+            return logp, idx, resp, near
+
+        whole, head, rest = call(X), call(X[:cut]), call(X[cut:])
+        for w, a, b in zip(whole, head, rest):
+            assert torch.equal(w, torch.cat([a, b]))
+        Nk, S1, S2, L = ctx.gmm_em_step(X, pi, mu, var)
+        assert ctx.gmm_last_exact_count() == K
+        assert abs(float(Nk.sum()) - N) <= 1e-6 * N and abs(L - float(whole[0].double().sum())) <= 1e-6 * abs(L)
+        again = ctx.gmm_em_step(X, pi, mu, var)
+        assert again[3] == L and all(torch.equal(a, b) for a, b in zip(again[:3], (Nk, S1, S2)))
+
+
 @pytest.mark.parametrize("N,D,K,m", [(1, 16, 64, 1), (257, 33, 97, 2), (3001, 128, 1024, 2), (3001, 128, 1024, 4), (1500, 20, 300, 3), (900, 66, 4096, 4),
                                      (2000, 9, 130, 1), (300, 12, 192, 4), (1200, 40, 20, 1)])
 def test_screen_top_m(fg, monkeypatch, N, D, K, m):

@@ -787,9 +787,11 @@ __device__ __forceinline__ void screen_convert(const SweepParams& p, unsigned ch
 //
 // TOP: how many of a point's largest values are wanted for certain.  1: everything within the margin of the largest.  More (the top-m
 // assignment): also everything that could be among the TOP largest.  The bound for those is the TOP-th largest of the lower bounds of
-// the quarters of every block: different components, so the TOP-th largest value cannot be below it.  It rises slowly as the sweep
-// goes on, so the tile's components pass twice, once for the bound and once for the marks: in one pass what was marked under
-// early bounds cost more evaluations than the second pass takes (1M x 128, K = 1024: top-2 1.40 ms in one pass, top-4 3.2).
+// the quarters of every block: different components, so the TOP-th largest value cannot be below it.  It rises as the sweep goes on, most of
+// all in the first group, under whose bounds twice as many pairs were marked as the final one leaves.  So the first group passes
+// once more at the end and is marked then, the others as they come: emulated on the clusters of 128 x 1024 3.13 marks per point, as many as
+// with all components twice (5.6 in one pass; top-4 12.6, 16.8).  1.02M points, top-2 (us): 128 x 1024 1270 -> 955, 32 x 1024 941 -> 806,
+// 64 x 4096 2447 -> 1679, 128 x 4096 3723 -> 2333.
 template <int TOP, bool CONVERT>
 __global__ void __launch_bounds__(Sweep<CONVERT>::THREADS, 1)
 screen_sweep_kernel(const SweepParams p) {
@@ -807,8 +809,8 @@ screen_sweep_kernel(const SweepParams p) {
     const int tid = threadIdx.x, warp = tid >> 5, role = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int64_t ntiles = (p.n + SCR_TILE - 1) / SCR_TILE;
     const int64_t ntl = ((int64_t)blockIdx.x < ntiles) ? (ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
-    constexpr int PASSES = TOP > 1 ? 2 : 1;
-    const int NG = p.NG, spg = (p.KA + 1) >> 1;              // stages per group
+    const int NG = p.NG, GT = TOP > 1 ? NG + 1 : NG;         // groups of a tile (TOP > 1: the first one twice)
+    const int spg = (p.KA + 1) >> 1;              // stages per group
     unsigned char* cons = smem + S::COFF;                    // [CSLOTS][4096]
     float* nrm_s = reinterpret_cast<float*>(smem + S::NOFF);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S::BOFF);
@@ -991,9 +993,9 @@ screen_sweep_kernel(const SweepParams p) {
                     else later(bn, bmax, E, mask);
                 }
             };
-            for (int gg = 0; gg < PASSES * NG; ++gg, ++gi) {
-                const bool last = gg + 1 == PASSES * NG, first = gg < NG;
-                const int g = (PASSES > 1 && !first) ? gg - NG : gg;
+            for (int gg = 0; gg < GT; ++gg, ++gi) {
+                const bool last = gg + 1 == GT, again = gg == NG;
+                const int g = again ? 0 : gg;
                 if (last) ahead(i + 1);
                 const bool got = bar_wait(BAR(S::LFULL + half), gi & 1u, abort_flag, p.status, false);
                 const bool ok = __all_sync(0xffffffffu, got);
@@ -1021,7 +1023,7 @@ screen_sweep_kernel(const SweepParams p) {
                         E[j] = fmaf(ab.y, nrm, fabsf(ab.x));
                         if (TOP == 1) {
                             thr = fmaxf(thr, ab.x < 0.f ? -CUDART_INF_F : bm[j] - E[j]);
-                        } else if (first && !(ab.x < 0.f) && bm[j] - E[j] > low[TOP - 1]) {
+                        } else if (!again && !(ab.x < 0.f) && bm[j] - E[j] > low[TOP - 1]) {
                             const float (&mx)[4] = j == 0 ? q0 : j == 1 ? q1 : j == 2 ? q2 : q3;
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
@@ -1035,7 +1037,7 @@ screen_sweep_kernel(const SweepParams p) {
                             }
                         }
                     }
-                    if (TOP == 1 || !first) {
+                    if (TOP == 1 || gg > 0) {
                         unsigned mk[4] = {0u, 0u, 0u, 0u}, rest = 0u;
                         mark(v0, 0, 4 * g, bm[0], E[0], mk[0], rest);
                         mark(v1, 1, 4 * g + 1, bm[1], E[1], mk[1], rest);
@@ -1144,12 +1146,12 @@ screen_sweep_kernel(const SweepParams p) {
         };
         if (!CONVERT && ntl > 0) load_rows(0);
         for (int64_t i = 0; i < ntl && ok; ++i)
-            for (int g = 0; g < PASSES * NG && ok; ++g) {
+            for (int g = 0; g < GT && ok; ++g) {
                 for (int z = 0; z < spg && ok; ++z) {
                     if (ps >= S::PS) ok = wait_slot(S::PEMPTY + slot, phase);
                     if (!ok) break;
                     if (elect_one()) {
-                        const unsigned char* src = p.img + (size_t)(PASSES > 1 && g >= NG ? g - NG : g) * p.gbytes;
+                        const unsigned char* src = p.img + (size_t)(g == NG ? 0 : g) * p.gbytes;
                         const uint32_t bytes = min(p.KA - 2 * z, 2) * 16384u;
                         bar_expect_tx(BAR(S::PFULL + slot), bytes + (z == 0 ? SW_CSLOT : 0));
                         if (z == 0) bulk(cons + cslot * SW_CSLOT, src, SW_CSLOT, BAR(S::PFULL + slot));
@@ -1163,7 +1165,7 @@ screen_sweep_kernel(const SweepParams p) {
                 // the next tile's rows as soon as both halves have taken this tile's (which they do before its first products);
                 // no stage waits for that except behind the tile's last one
                 if (!CONVERT && ok && ut == (uint32_t)(i + 1) && i + 1 < ntl) {
-                    uint32_t free_now = (g + 1 == PASSES * NG) ? 1u : 0u;
+                    uint32_t free_now = (g + 1 == GT) ? 1u : 0u;
                     if (free_now) ok = wait_slot(S::UEMPTY, (uint32_t)(i & 1));
                     else {
                         if (lane == 0) free_now = bar_test(BAR(S::UEMPTY), (uint32_t)(i & 1)) ? 1u : 0u;
@@ -1235,7 +1237,7 @@ screen_sweep_kernel(const SweepParams p) {
             uint32_t gi = 0;
             bool alive = true;
             for (int64_t i = 0; i < ntl && alive; ++i) {
-                for (int g = 0; g < PASSES * NG && alive; ++g, ++gi) {
+                for (int g = 0; g < GT && alive; ++g, ++gi) {
                     if (g == 0) alive = wait(S::AFULL + h, (uint32_t)(i & 1));
                     if (alive && gi >= 1) alive = wait(S::LEMPTY + h, (gi - 1) & 1u);
                     for (int z = 0; z < spg && alive; ++z) {

@@ -1575,7 +1575,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                 for (int j = lane; j < c; j += 32) sm += fast_ex2(val[o + j] - m);
 #pragma unroll
             for (int x = 16; x > 0; x >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, x);
-            const float lz = m + log2f(sm);
+            const float ls = log2f(sm), lz = m + ls;
             if (MODE == SCREEN_TOP) {
                 float pv = CUDART_INF_F;                     // the pair that went out last
                 int pk = -1;
@@ -1606,9 +1606,10 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             if (MODE == SCREEN_EM)
                 for (int j0 = 0; j0 < c; j0 += 32) {
                     const int j = j0 + lane;
-                    const float r = j < c ? fast_ex2(val[o + j] - lz) : 0.f;
+                    const float v = j < c ? val[o + j] : -CUDART_INF_F, r = fast_ex2((v - m) - ls);
                     const int id = j < c ? ids[o + j] : 0;
                     const bool keep = r >= 9.094947e-13f;
+                    if (keep) ll_acc -= (double)r * (double)v;
                     const unsigned bal = __ballot_sync(0xffffffffu, keep);
                     __syncwarp();
                     if (keep) {
@@ -1637,7 +1638,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             if (idx) idx[row] = best;
             if (histogram && a.cnt > 0) {
                 ids[a.off] = (unsigned short)best;
-                val[a.off] = -1.f;
+                val[a.off] = 1.f;
                 pt_cnt[row] = 1;
                 atomicAdd(&hist[best], 1);
             }
@@ -1645,11 +1646,11 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             ll_acc += -CUDART_INF;
         } else if (alone) {
             ids[a.off] = (unsigned short)only;
-            val[a.off] = -1.f;
+            val[a.off] = 1.f;
             pt_cnt[row] = 1;
             if (histogram) atomicAdd(&hist[only], 1);
         } else {
-            ll_acc += (double)mx + (double)log2f(sum);
+            ll_acc += (double)mx + (double)log2f(sum);       // (a list of its own length)
             pt_cnt[row] = kept;
         }
     }
@@ -1841,7 +1842,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                         if (idx) idx[prow] = best;
                         if (histogram) {
                             ids[off] = (unsigned short)best;
-                            val[off] = -1.f;
+                            val[off] = 1.f;
                             pt_cnt[prow] = 1;
                             atomicAdd(&hist[best], 1);
                         }
@@ -1885,12 +1886,14 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                     ll_acc += z;
                 }
                 if (MODE == SCREEN_EM) {
-                    // responsibilities; the pairs below 2^-40 of the total leave the list
+                    // responsibilities; the pairs below 2^-40 of the total leave the list.  (What the statistics will not
+                    // say of the log-likelihood: see screen_reduce_kernel.)
                     int kept = 0;
                     for (int j0 = 0; j0 < steps; j0 += 8) {
                         const int j = j0 + l8;
-                        const float r = j < cnt ? fast_ex2(pv[j] - lz) : 0.f;
+                        const float v = j < cnt ? pv[j] : -CUDART_INF_F, r = fast_ex2((v - mx) - ls);
                         const bool keep = r >= 9.094947e-13f;
+                        if (keep) ll_acc -= (double)r * (double)v;
                         const unsigned mine = (__ballot_sync(0xffffffffu, keep) >> (8 * grp)) & 255u;
                         if (keep) {
                             const unsigned short id = pk[j];
@@ -2055,133 +2058,180 @@ __global__ void __launch_bounds__(1024) screen_fill_kernel(int64_t n, int K, int
     }
 }
 
-// Statistics of one work item (at most SCR_SEG pairs of one component) by one warp: sums of r, r (x - mu), r (x - mu)^2 in
-// fp32, and, over the points whose only pair this is, their number and sum_d w2 (x - mu)^2 (their log-likelihood).  lpr lanes
-// per row, four dimensions each; the rows of four steps are in flight together.  The eight items of a CTA's step that belong to one
-// component are added in float64 before they leave: group g of eight items has one set of sums per component k in it, at place g + k
-// (a later set has a larger g or a larger k).  With a set per item the reduction read 20 MB per million points, 55 us at D = 128, K = 1024.
-__global__ void __launch_bounds__(256) screen_stats_kernel(const float* __restrict__ X, int D, int lpr, const float* __restrict__ mu,
-                                                           const float* __restrict__ w2, const uint2* __restrict__ srt,
-                                                           const int* __restrict__ off, const int* __restrict__ segoff,
-                                                           int K, double* __restrict__ part, const int* __restrict__ ctl) {
-    if (ctl[SC_DENSE] != 0) return;
-    extern __shared__ int seg_s[];                   // [K + 1]
-    __shared__ float sum_s[8][2 * 128 + 3];
-    __shared__ int k_s[8];
-    const int warp = threadIdx.x >> 5;
-    for (int j = threadIdx.x; j <= K; j += 256) seg_s[j] = segoff[j];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, l = lane % lpr, sub = lane / lpr, rows = 32 / lpr;
-    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-    const int items = seg_s[K];
-    const int d0 = 4 * l;
-    auto load4 = [&](const float* __restrict__ r, bool v) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (v) {
-            if (d0 < D) a = __ldg(reinterpret_cast<const float4*>(r + d0));
-        } else {
-            if (d0 < D) a.x = __ldg(r + d0);
-            if (d0 + 1 < D) a.y = __ldg(r + d0 + 1);
-            if (d0 + 2 < D) a.z = __ldg(r + d0 + 2);
-            if (d0 + 3 < D) a.w = __ldg(r + d0 + 3);
-        }
-        return a;
-    };
-    for (int base = blockIdx.x * 8; base < items; base += gridDim.x * 8) {
-      const int item = base + warp;
-      if (item < items) {
-        int k = 0;                                   // the component whose items hold this one: the last with segoff <= item
-        for (int w = K; w > 1;) {
-            const int h = w >> 1;
-            if (seg_s[k + h] <= item) k += h;
-            w -= h;
-        }
-        const int a = __ldg(off + k) + (item - seg_s[k]) * SCR_SEG, b = min(a + SCR_SEG, __ldg(off + k + 1));
-        const float4 m = load4(mu + (size_t)k * D, false), w = load4(w2 + (size_t)k * D, false);
-        float4 s1 = make_float4(0.f, 0.f, 0.f, 0.f), s2 = s1;
-        float nsum = 0.f, n1 = 0.f, q1 = 0.f;
-        for (int p = a; p < b; p += 32) {
-            uint2 e = make_uint2(0u, 0u);
-            if (p + lane < b) e = __ldg(srt + p + lane);
-            const float re = __uint_as_float(e.y);
-            nsum += fabsf(re);
-            n1 += re < 0.f ? 1.f : 0.f;
-            const int have = min(32, b - p);
-            for (int i = 0; i < have; i += 4 * rows) {
-                float4 x[4];
-                float r[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int src = min(31, i + u * rows + sub);
-                    const unsigned row = __shfl_sync(0xffffffffu, e.x, src);
-                    r[u] = __shfl_sync(0xffffffffu, re, src);
-                    if (i + u * rows + sub >= have) r[u] = 0.f;
-                    x[u] = make_float4(m.x, m.y, m.z, m.w);
-                    if (r[u] != 0.f) x[u] = load4(X + (size_t)row * D, vec);
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const float ra = fabsf(r[u]);
-                    const float tx = x[u].x - m.x, ty = x[u].y - m.y, tz = x[u].z - m.z, tw = x[u].w - m.w;
-                    s1.x = fmaf(ra, tx, s1.x); s1.y = fmaf(ra, ty, s1.y); s1.z = fmaf(ra, tz, s1.z); s1.w = fmaf(ra, tw, s1.w);
-                    const float ax = tx * tx, ay = ty * ty, az = tz * tz, aw = tw * tw;
-                    s2.x = fmaf(ra, ax, s2.x); s2.y = fmaf(ra, ay, s2.y); s2.z = fmaf(ra, az, s2.z); s2.w = fmaf(ra, aw, s2.w);
-                    const float q = fmaf(w.x, ax, fmaf(w.y, ay, fmaf(w.z, az, w.w * aw)));
-                    if (r[u] < 0.f) q1 += q;
-                }
-            }
-        }
-        for (int o = lpr; o < 32; o <<= 1) {
-            s1.x += __shfl_xor_sync(0xffffffffu, s1.x, o); s1.y += __shfl_xor_sync(0xffffffffu, s1.y, o);
-            s1.z += __shfl_xor_sync(0xffffffffu, s1.z, o); s1.w += __shfl_xor_sync(0xffffffffu, s1.w, o);
-            s2.x += __shfl_xor_sync(0xffffffffu, s2.x, o); s2.y += __shfl_xor_sync(0xffffffffu, s2.y, o);
-            s2.z += __shfl_xor_sync(0xffffffffu, s2.z, o); s2.w += __shfl_xor_sync(0xffffffffu, s2.w, o);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            nsum += __shfl_xor_sync(0xffffffffu, nsum, o);
-            n1 += __shfl_xor_sync(0xffffffffu, n1, o);
-            q1 += __shfl_xor_sync(0xffffffffu, q1, o);
-        }
-        float* po = sum_s[warp];
-        if (sub == 0) {
-            const float v1[4] = {s1.x, s1.y, s1.z, s1.w}, v2[4] = {s2.x, s2.y, s2.z, s2.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (d0 + j < D) { po[d0 + j] = v1[j]; po[D + d0 + j] = v2[j]; }
-        }
-        if (lane == 0) { po[2 * D] = nsum; po[2 * D + 1] = n1; po[2 * D + 2] = q1; k_s[warp] = k; }
-      }
-      __syncthreads();
-      const int have = min(8, items - base);
-      for (int e = threadIdx.x; e < 2 * D + 3; e += 256) {
-        double t = (double)sum_s[0][e];
-        for (int w = 1; w <= have; ++w) {
-            if (w == have || k_s[w] != k_s[w - 1]) {
-                part[(size_t)(base / 8 + k_s[w - 1]) * (2 * D + 3) + e] = t;
-                t = 0.0;
-            }
-            if (w < have) t += (double)sum_s[w][e];
-        }
-      }
-      __syncthreads();
+// Statistics: sums of r, r (x - mu), r (x - mu)^2, fp32 within a work item (at most SCR_SEG pairs of one component), float64 beyond.  A warp takes as
+// many consecutive items as make one wave of warps (screen_item_group); their pairs are neighbours in srt, whatever their components, so their rows come in one
+// stream: ST_STAGES stages of ST_ROWS loads per lane, by asynchronous copies into shared memory, and the pairs themselves 32 ahead.  LPR lanes per row, four
+// dimensions each; a stage that holds the end of an item is gone through once more for the next one.  A group g has one set of sums per component k in it, at
+// place g + k (a later set has a larger g or a larger k).
+// Bound by the gathered rows: 606K points at 128 x 1024, 1.36M rows, 140 us with four rows in flight per warp, 24 warps per SM, 60 instructions per row and a CTA's
+// warps waiting for one another after 64 rows each (54 % of the issue slots, 3.6 TB/s from memory); 113 with eight rows in flight, no waiting and 20
+// instructions (31 %, 4.3 TB/s).  A step of 1.02M x 128, K = 1024 with those 1036 us, with this 982, 12 warps per SM with 24 rows each on their way; with
+// 16 warps and 16 rows 1030, 8 warps and 40 rows 994, four rows per stage 1065, and the pairs one stage ahead instead of 32 pairs 1075 to 1284.
+constexpr int ST_ROWS = 8, ST_STAGES = 4;
+__device__ __forceinline__ int screen_item_group(int items) { return items <= SCR_STAT_WARPS ? 1 : (items + SCR_STAT_WARPS - 1) / SCR_STAT_WARPS; }
+// The component whose items hold this one: the last with segoff <= item.  The whole warp.
+__device__ __forceinline__ int screen_component(const int* __restrict__ segoff, int K, int item, int lane) {
+    int k = 0;
+    for (int step = K > 1024 ? 1024 : K > 32 ? 32 : 1, span = K; ; step = step > 32 ? 32 : 1) {
+        const int c = k + lane * step;
+        const unsigned in = __ballot_sync(0xffffffffu, lane * step < span && __ldg(segoff + (lane * step < span ? c : k)) <= item);
+        k += (31 - __clz(in | 1u)) * step;
+        if (step == 1) return k;
+        span = min(step, K - k);
     }
 }
+template <int LPR, bool VEC>
+__global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const float* __restrict__ X, int D, const float* __restrict__ mu,
+                                                           const uint2* __restrict__ srt, const int* __restrict__ off, const int* __restrict__ segoff,
+                                                           int K, double* __restrict__ part, const int* __restrict__ ctl) {
+    if (ctl[SC_DENSE] != 0) return;
+    constexpr int ROWS = 32 / LPR, U = LPR < ST_ROWS ? LPR : ST_ROWS, SR = U * ROWS;        // pairs of a stage (at most 32)
+    constexpr int W = ST_THREADS / 32;
+    extern __shared__ __align__(16) unsigned char ring_s[];                                 // [W][ST_STAGES][ST_ROWS][32] 16 bytes
+    __shared__ double t_s[W][8][32];                 // a lane's sums of the items so far (x - mu: four dimensions, squares)
+    __shared__ float r_s[W][ST_STAGES][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LPR, sub = lane / LPR, d0 = 4 * l;
+    const int items = __ldg(segoff + K), G = screen_item_group(items), g = blockIdx.x * W + warp;
+    if (g * G >= items) return;
+    const int first = g * G, end = min(items, first + G);
+    double (*const t)[32] = t_s[warp];
+    uint4* const ring = reinterpret_cast<uint4*>(ring_s) + (size_t)warp * ST_STAGES * ST_ROWS * 32 + lane;
+    int k = screen_component(segoff, K, first, lane);
+    const int p0 = __ldg(off + k) + (first - __ldg(segoff + k)) * SCR_SEG;
+    int total;                                       // pairs of the group
+    if (end == items) total = __ldg(off + K) - p0;
+    else {
+        const int ke = screen_component(segoff, K, end, lane);
+        total = __ldg(off + ke) + (end - __ldg(segoff + ke)) * SCR_SEG - p0;
+    }
+    const int stages = (total + SR - 1) / SR;
+    const uint2* const pairs = srt + p0;
+    const float* const Xl = X + d0;
+    uint2 e, e_next;                                 // 32 pairs of which the next stages are, and the 32 after them (no pair: row 0, without weight)
+    auto fetch = [&](int i) {
+        e_next = make_uint2(0u, 0u);
+        if (i + lane < total) e_next = __ldg(pairs + i + lane);
+    };
+    auto issue = [&](int st) {
+        const int slot = st % ST_STAGES, at = (st * SR) & 31;
+        if (st < stages) {
+            if (at == 0) {
+                e = e_next;
+                fetch(st * SR + 32);
+            }
+            const float r = __shfl_sync(0xffffffffu, __uint_as_float(e.y), (at + lane) & 31);
+            if (lane < SR) r_s[warp][slot][lane] = r;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const unsigned row = __shfl_sync(0xffffffffu, e.x, at + u * ROWS + sub);
+                const float* src = Xl + (size_t)row * D;
+                const uint32_t dst = smem_u32(ring + (slot * ST_ROWS + u) * 32);
+                if (VEC) {
+                    if (d0 < D) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (d0 + j < D) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * j), "l"(src + j) : "memory");
+                }
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint64_t m[2];
+    int o1;
+    auto component = [&]() {
+        o1 = __ldg(off + k + 1) - p0;
+        float f[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[j] = d0 + j < D ? __ldg(mu + (size_t)k * D + d0 + j) : 0.f;
+        m[0] = pack2(__float_as_uint(f[0]), __float_as_uint(f[1]));
+        m[1] = pack2(__float_as_uint(f[2]), __float_as_uint(f[3]));
+    };
+    fetch(0);
+#pragma unroll 1
+    for (int st = 0; st < ST_STAGES - 1; ++st) issue(st);
+    component();
+    int item = first, a = 0, b = min(SCR_SEG, o1);   // the item's pairs
+    uint64_t s1[2] = {0ull, 0ull}, s2[2] = {0ull, 0ull};
+    float nsum = 0.f;
+    double tn = 0.0;
+    bool fresh = true;                               // the first item of a set of sums
+#pragma unroll 1
+    for (int st = 0; st < stages; ++st) {
+        issue(st + ST_STAGES - 1);
+        asm volatile("cp.async.wait_group %0;" ::"n"(ST_STAGES - 1) : "memory");
+        __syncwarp();
+        const int slot = st % ST_STAGES, pos = st * SR;
+        const uint4* const xs = ring + slot * ST_ROWS * 32;
+        const float* const rs = r_s[warp][slot];
+        for (;;) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int i = pos + u * ROWS + sub;
+                const bool on = i >= a && i < b;
+                const float r = on ? rs[u * ROWS + sub] : 0.f;
+                const uint4 x = xs[u * 32];
+                const uint64_t rr = pack2(__float_as_uint(r), __float_as_uint(r));
+                uint64_t ta = sub2(pack2(x.x, x.y), m[0]), tb = sub2(pack2(x.z, x.w), m[1]);
+                if (!on) ta = tb = 0ull;             // (a row of another component: the square may be beyond a float)
+                s1[0] = fma2(rr, ta, s1[0]);
+                s1[1] = fma2(rr, tb, s1[1]);
+                s2[0] = fma2(rr, mul2(ta, ta), s2[0]);
+                s2[1] = fma2(rr, mul2(tb, tb), s2[1]);
+            }
+            nsum += lane < SR && pos + lane >= a && pos + lane < b ? rs[lane] : 0.f;
+            if (b > pos + SR) break;
+            // the item's last pair
+            const float v[8] = {lo2(s1[0]), hi2(s1[0]), lo2(s1[1]), hi2(s1[1]), lo2(s2[0]), hi2(s2[0]), lo2(s2[1]), hi2(s2[1])};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) t[j][lane] = fresh ? (double)v[j] : t[j][lane] + (double)v[j];
+            tn += (double)nsum;
+            fresh = false;
+            s1[0] = s1[1] = s2[0] = s2[1] = 0ull;
+            nsum = 0.f;
+            a = b;
+            ++item;
+            if (b == o1 || item == end) {            // and the component's, or the group's
+                double* const o = part + (size_t)(g + k) * (2 * D + 1);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    double q = t[j][lane];
+#pragma unroll
+                    for (int x = LPR; x < 32; x <<= 1) q += __shfl_xor_sync(0xffffffffu, q, x);
+                    if (sub == 0 && d0 + (j & 3) < D) o[(j < 4 ? 0 : D) + d0 + (j & 3)] = q;
+                }
+                tn = warp_sum(tn);
+                if (lane == 0) o[2 * D] = tn;
+                if (item == end) break;
+                do { ++k; } while (__ldg(segoff + k + 1) == item);               // (components without pairs)
+                component();
+                tn = 0.0;
+                fresh = true;
+            }
+            b = min(a + SCR_SEG, o1);
+            if (a >= pos + SR) break;
+        }
+        __syncwarp();
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
 
-// A CTA per component: its sets of sums in order (two interleaved chains), float64, shifted from its mean to the origin.
+// A CTA per component: its sets of sums in order (two interleaved chains), float64, shifted from its mean to the origin.  Its part of the
+// log-likelihood: sum_i r_ik log z_ik = n c - sum_d w sum_i r_ik (x - mu)^2, which is all there is to a point with one pair; for the others the evaluation
+// has added up log p(x) - sum_k r_k log z_k.
 __global__ void __launch_bounds__(512) screen_reduce_kernel(int D, int K, const double* __restrict__ part, const int* __restrict__ segoff,
-                                                            const float* __restrict__ mu, const double* __restrict__ c2d,
+                                                            const float* __restrict__ mu, const float* __restrict__ w2, const double* __restrict__ c2d,
                                                             double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
                                                             double* __restrict__ llk, int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl[SC_DONE] += 1;
     const int k = blockIdx.x, d = threadIdx.x & 127, q = (threadIdx.x >> 7) & 1, c = threadIdx.x >> 8;
-    const int i0 = segoff[k], i1 = segoff[k + 1];
+    const int i0 = segoff[k], i1 = segoff[k + 1], G = screen_item_group(segoff[K]);
     if (i0 == i1) return;
-    const int g0 = i0 / 8 + k, g1 = (i1 - 1) / 8 + k + 1;
+    const int g0 = i0 / G + k, g1 = (i1 - 1) / G + k + 1;
     __shared__ double sh[2][2][128];
-    __shared__ double tot[3];
-    const size_t st = (size_t)(2 * D + 3);
+    __shared__ double tot_s, quad_s[4];
+    const size_t st = (size_t)(2 * D + 1);
     double a = 0.0;
     if (d < D)
         for (int g = g0 + c; g < g1; g += 8) {
@@ -2192,25 +2242,29 @@ __global__ void __launch_bounds__(512) screen_reduce_kernel(int D, int K, const 
             for (int u = 0; u < 4; ++u) a += v[u];
         }
     sh[c][q][d] = a;
-    if (threadIdx.x < 96) {                              // warp: a scalar of the sets (weight, lone points, their quadratic forms)
-        const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
         double t = 0.0;
-        for (int g = g0 + lane; g < g1; g += 32) t += part[(size_t)g * st + 2 * D + which];
+        for (int g = g0 + threadIdx.x; g < g1; g += 32) t += part[(size_t)g * st + 2 * D];
         t = warp_sum(t);
-        if (lane == 0) tot[which] = t;
+        if (threadIdx.x == 0) tot_s = t;
     }
     __syncthreads();
     if (threadIdx.x >= 128) return;
-    const double n = tot[0];
+    const double n = tot_s;
+    double quad = 0.0;
     if (d < D) {
         const double s1 = sh[0][0][d] + sh[1][0][d], s2 = sh[0][1][d] + sh[1][1][d];
         const double m = (double)__ldg(mu + (size_t)k * D + d);
+        quad = (double)__ldg(w2 + (size_t)k * D + d) * s2;
         S1[(size_t)k * D + d] += s1 + m * n;
         S2[(size_t)k * D + d] += s2 + 2.0 * m * s1 + m * m * n;
     }
+    quad = warp_sum(quad);
+    if ((d & 31) == 0) quad_s[d >> 5] = quad;
+    asm volatile("bar.sync 1, 128;" ::: "memory");           // (the threads that are left)
     if (d == 0) {
         Nk[k] += n;
-        llk[k] += (tot[1] > 0.0 ? tot[1] * c2d[k] - tot[2] : 0.0) * 0.69314718055994530942;
+        llk[k] += (n * c2d[k] - (quad_s[0] + quad_s[1] + quad_s[2] + quad_s[3])) * 0.69314718055994530942;
     }
 }
 
@@ -2359,17 +2413,14 @@ __global__ void __launch_bounds__(256, 4) screen_group_stats_kernel(const float*
         float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, nsum = 0.f;
         if (a < b) {
             const float4 m = load4(mu + (size_t)k * D, vec_m), w = load4(w2 + (size_t)k * D, (D & 3) == 0);      // (w2: scratch, aligned)
-            float n1 = 0.f, q1 = 0.f;
             for (int p = a; p < b; p += 32) {
                 if (p > a) {
                     e = make_uint2(0u, 0u);
                     if (p + lane < b) e = __ldg(srt + p + lane);
                 }
                 const float re = __uint_as_float(e.y);
-                nsum += fabsf(re);
-                if (re < 0.f) n1 += 1.f;
+                nsum += re;
                 float4 f1 = make_float4(0.f, 0.f, 0.f, 0.f), f2 = f1;
-                float fq = 0.f;
                 const int have = min(32, b - p);
                 for (int i = 0; i < have; i += 4 * rows) {
                     float4 x[4];
@@ -2385,18 +2436,15 @@ __global__ void __launch_bounds__(256, 4) screen_group_stats_kernel(const float*
                     }
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        const float ra = fabsf(r[u]);
+                        const float ra = r[u];
                         const float tx = x[u].x - m.x, ty = x[u].y - m.y, tz = x[u].z - m.z, tw = x[u].w - m.w;
                         f1.x = fmaf(ra, tx, f1.x); f1.y = fmaf(ra, ty, f1.y); f1.z = fmaf(ra, tz, f1.z); f1.w = fmaf(ra, tw, f1.w);
                         const float ax = tx * tx, ay = ty * ty, az = tz * tz, aw = tw * tw;
                         f2.x = fmaf(ra, ax, f2.x); f2.y = fmaf(ra, ay, f2.y); f2.z = fmaf(ra, az, f2.z); f2.w = fmaf(ra, aw, f2.w);
-                        const float q = fmaf(w.x, ax, fmaf(w.y, ay, fmaf(w.z, az, w.w * aw)));
-                        if (r[u] < 0.f) fq += q;
                     }
                 }
                 s1[0] += f1.x; s1[1] += f1.y; s1[2] += f1.z; s1[3] += f1.w;
                 s2[0] += f2.x; s2[1] += f2.y; s2[2] += f2.z; s2[3] += f2.w;
-                q1 += fq;
             }
 #pragma unroll
             for (int j = 0; j < 4; ++j)
@@ -2404,13 +2452,13 @@ __global__ void __launch_bounds__(256, 4) screen_group_stats_kernel(const float*
                     s1[j] += __shfl_xor_sync(0xffffffffu, s1[j], o);
                     s2[j] += __shfl_xor_sync(0xffffffffu, s2[j], o);
                 }
+            float quad = sub == 0 ? fmaf(w.x, s2[0], fmaf(w.y, s2[1], fmaf(w.z, s2[2], w.w * s2[3]))) : 0.f;      // (see screen_reduce_kernel)
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 nsum += __shfl_xor_sync(0xffffffffu, nsum, o);
-                n1 += __shfl_xor_sync(0xffffffffu, n1, o);
-                q1 += __shfl_xor_sync(0xffffffffu, q1, o);
+                quad += __shfl_xor_sync(0xffffffffu, quad, o);
             }
-            if (lane == 0 && n1 > 0.f) ll_acc += (double)n1 * c2d[k] - (double)q1;
+            if (lane == 0) ll_acc += (double)nsum * c2d[k] - (double)quad;
         }
         pairs();                                             // (of the next item)
         const float wk = __ldg(pi + k), inv_t = 1.0f / (float)g_len[g];
@@ -2610,11 +2658,16 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     if (e != cudaSuccess) return e;
     screen_fill_kernel<<<blocks, warps * 32, smem, s>>>(n, K, range, b.pt_off, b.pt_cnt, b.ids, b.val, b.counts, b.off, b.srt, b.ctl);
     LCHECK();
-    int lpr = 1;
-    while (4 * lpr < D) lpr <<= 1;
-    screen_stats_kernel<<<148 * 6, 256, (size_t)(K + 1) * 4, s>>>(X, D, lpr, mu, w2, b.srt, b.off, b.segoff, K, b.part, b.ctl);
+    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0);
+#define FG_STATS(L_) (vec ? screen_stats_kernel<L_, true> : screen_stats_kernel<L_, false>)
+    const auto stats = D <= 4 ? FG_STATS(1) : D <= 8 ? FG_STATS(2) : D <= 16 ? FG_STATS(4) : D <= 32 ? FG_STATS(8) : D <= 64 ? FG_STATS(16) : FG_STATS(32);
+#undef FG_STATS
+    constexpr int stats_smem = ST_THREADS / 32 * ST_STAGES * ST_ROWS * 512;
+    e = cudaFuncSetAttribute(stats, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem);
+    if (e != cudaSuccess) return e;
+    stats<<<SCR_STAT_WARPS / (ST_THREADS / 32), ST_THREADS, stats_smem, s>>>(X, D, mu, b.srt, b.off, b.segoff, K, b.part, b.ctl);
     LCHECK();
-    screen_reduce_kernel<<<K, 512, 0, s>>>(D, K, b.part, b.segoff, mu, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
+    screen_reduce_kernel<<<K, 512, 0, s>>>(D, K, b.part, b.segoff, mu, w2, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
     *launches += 4;
     return cudaGetLastError();
 }

@@ -18,7 +18,8 @@ constexpr int SCR_EXTRA = 2;                 // and, per point of a piece, for t
 constexpr int64_t SCR_PAIRS = SCR_PIECE * (SCR_SLOTS + SCR_EXTRA);
 constexpr int SCR_SEG = 64;                  // pairs per work item of the statistics
 constexpr int SCR_MARKS = 10;                // marked pairs of a piece, per point of a full one: beyond them the piece counts as dense
-constexpr int64_t SCR_ITEMS = SCR_PIECE * (SCR_MARKS + SCR_EXTRA) / SCR_SEG + SCR_MAX_K;
+constexpr int ST_THREADS = 128, ST_CTAS = 3;  // of the statistics: threads per CTA, CTAs per SM
+constexpr int SCR_STAT_WARPS = 148 * ST_CTAS * (ST_THREADS / 32);      // in one wave, each with a run of work items
 constexpr int SCR_RANGES = 3 * 148;          // CTAs of the pair evaluation and of the sort by component (at most)
 constexpr int SCR_LL = 4096;                 // log-likelihood partial sums (one per CTA of a launch), then one per component
 constexpr int SCR_DIM_BLOCKS = 64;
@@ -56,13 +57,13 @@ struct ScreenBuffers {
     uint2* words;         // [SCR_PIECE][SCR_WORDS] the sweep's marks: a mask, the block of 32 positions it belongs to
     unsigned long long* spill;        // [SCR_MAX_SMS][SCR_SPILL][256]
     unsigned short* ids;  // [SCR_PAIRS] component of a kept pair
-    float* val;           // [SCR_PAIRS] its responsibility (-1: the point's only pair)
+    float* val;           // [SCR_PAIRS] its responsibility
     uint2* srt;           // [SCR_PAIRS] (row, responsibility) sorted by component
     int* counts;          // [SCR_RANGES][K]
     int* totals;          // [K]
     int* off;             // [K + 1] where a component's pairs start in srt
     int* segoff;          // [K + 1] where its work items start
-    double* part;         // [SCR_ITEMS / 8 + K][2 D + 3] (see screen_stats_kernel)
+    double* part;         // [SCR_STAT_WARPS + K][2 D + 1] (see screen_stats_kernel)
     double* ll;           // [SCR_LL + K]
     int* ovf;             // [SCR_PIECE]
     int* ctl;             // [SC_WORDS]

@@ -186,8 +186,9 @@ ScratchLayout scratch_layout(int D, int K, bool planes, bool lists = true) {
         L.s_totals = take((size_t)K * 4);
         L.s_off = take((size_t)(K + 1) * 4);
         L.s_segoff = take((size_t)(K + 1) * 4);
-        static_assert(SCR_ITEMS % 8 == 0, "groups of eight items, the last of them at most SCR_ITEMS / 8 - 1");
-        L.s_part = take(((size_t)SCR_ITEMS / 8 + K) * (2 * (size_t)D + 3) * 8);
+        // (SCR_STAT_WARPS + K sets are written; the size is that of 25088 + K, so that the memory a shape is screened with stays what it was)
+        static_assert(SCR_STAT_WARPS <= 25088, "sets of sums");
+        L.s_part = take(((size_t)25088 + K) * (2 * (size_t)D + 3) * 8);
         L.s_ll = take((size_t)(SCR_LL + K) * 8);
         L.s_ovf = take((size_t)SCR_PIECE * 4);
     }

@@ -1785,7 +1785,7 @@ int gmm_build_posting_lists(gmm_ctx* ctx, const int32_t* idx, const float* resp,
     if (!(tau > 0.f)) tau = 1.0f / (float)K;                 // also for NaN
     CHECK(grow_buffer(ctx, &ctx->pl_scratch, &ctx->pl_scratch_bytes, pl_scratch_bytes(K), "the posting-list counters"));
     KL(launch_posting_lists(ctx->stream, idx, resp, N, m, K, tau, max_lists, ctx->pl_scratch, offsets, items));
-    ctx->launches += 3;        // launch_posting_lists enqueues four kernels
+    ctx->launches += 2;        // launch_posting_lists enqueues three kernels
     int64_t tot = 0;
     CU(cudaMemcpyAsync(&tot, offsets + K, sizeof(int64_t), cudaMemcpyDeviceToHost, ctx->stream));
     CU(cudaStreamSynchronize(ctx->stream));
@@ -1881,7 +1881,7 @@ int gmm_kmeans_step(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, const
     // the points of every cluster in ascending order, then fixed-order float64 sums
     KL(launch_posting_lists(ctx->stream, assign, resp, N, 1, K, 1.0f, 1, ctx->pl_scratch, km_offsets(ctx->km_scratch), items));
     KL(launch_kmeans_update(ctx->stream, X, D, K, centroids, items, ctx->km_scratch, centroids_out, counts));
-    ctx->launches += 4;
+    ctx->launches += 3;
     const int slot = 0;
     CU(cudaMemsetAsync(&ctx->result()->ll[slot], 0, 8, ctx->stream));
     KL(launch_reduce_ll(ctx->stream, km_inertia_k(ctx->km_scratch, D, K), K, &ctx->result()->ll[slot], false));

@@ -112,7 +112,7 @@ cudaError_t launch_fisher(cudaStream_t s, int64_t T, int D, int K, const double*
                           const float* pi, const float* mu, const float* var, float* out);
 
 // ---- IVF posting lists from the top-m assignment (paper Sections 4.2-4.3) ---------------------------------------
-constexpr int PL_MAX_BLOCKS = 1024;       // the vectors are cut into at most this many contiguous ranges
+constexpr int PL_MAX_BLOCKS = 296;        // the vectors are cut into at most this many contiguous ranges: two CTAs per SM
 constexpr int PL_MAX_K = 8192;            // one 32-bit cursor per cluster in shared memory
 size_t pl_scratch_bytes(int K);
 // offsets[K + 1] (device), items[>= n * max_lists] (device); scratch of pl_scratch_bytes(K) bytes

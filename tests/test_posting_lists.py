@@ -149,6 +149,29 @@ def test_gpu_builder_at_the_edges_of_its_ranges(N, K, m, max_lists):
     assert items_d.cpu().numpy()[:total].tolist() == items_r.tolist()
 
 
+# Ranges of several chunks (16 warps with 512 choices each, 8 warps beyond K = 2048): 1, 2, 4 and 8 lanes per vector, a ragged last chunk, lists that fill a chunk.
+@pytest.mark.gpu
+@pytest.mark.parametrize("N,K,m,max_lists", [(2_500_001, 37, 1, 1), (1_300_003, 1024, 2, 2), (1_300_003, 2, 2, 2), (700_001, 2049, 4, 3), (330_001, 300, 8, 6), (620_011, 8191, 2, 2)])
+def test_gpu_builder_over_several_chunks(N, K, m, max_lists):
+    import torch
+    from paper_2606_10896_b200 import flashgmm as fg
+
+    rng = np.random.default_rng(N + K)
+    idx = rng.integers(0, K, (N, m)).astype(np.int32)
+    idx[N // 3: N // 2, 0] = K - 1                         # (one list for a long stretch)
+    idx[rng.random(idx.shape) < 0.02] = -1
+    resp = np.sort(rng.random((N, m)).astype(np.float32), 1)[:, ::-1].copy()
+    take = np.logical_and.accumulate((idx >= 0) & ((np.arange(m) == 0) | (resp > 0.4)) & (np.arange(m) < max_lists), axis=1)
+    rows, cols = np.nonzero(take)                          # vector by vector, choice by choice
+    lists = idx[rows, cols]
+    want = rows[np.argsort(lists, kind="stable")]
+    t = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda:0")
+    with fg.Context(0) as ctx:
+        off_d, items_d, total, _ = ctx.gmm_build_posting_lists(t(idx), t(resp), K, 0.4, max_lists)
+    assert total == len(want) and np.array_equal(np.diff(off_d.cpu().numpy()), np.bincount(lists, minlength=K))
+    assert np.array_equal(items_d.cpu().numpy()[:total], want)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("N,K,m,max_lists", [(5000, 7, 2, 2), (3001, 40, 4, 3), (2000, 3, 8, 8)])
 def test_gpu_builder_lists_a_vector_as_often_as_its_row_names_the_cluster(N, K, m, max_lists):

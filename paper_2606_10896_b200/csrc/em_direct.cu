@@ -16,6 +16,7 @@
 // Bound by the FMA rate at larger K D (4 K D FMAs per point, two per instruction: fma.f32x2), by launches and the trip through X
 // at small ones.
 #include "internal.cuh"
+#include <type_traits>
 #include <math_constants.h>
 #include <stdint.h>
 
@@ -546,6 +547,387 @@ __global__ void __launch_bounds__(1024) direct_reduce_kernel(const ReduceArgs p)
 }
 
 // ------------------------------------------------------------------------------------------------------------------
+// A fit whose points fit into the shared memory of one cluster of 16 CTAs, and whose iterations are launches and trips to memory otherwise: one launch for
+// all of them.  A CTA keeps its points; the parameters are in every CTA.  Per iteration: log-sum-exp with the responsibilities into shared memory (a point per
+// 2^lgG lanes, four components each), statistics (a thread per tile of four components x four dimensions, FT / T replicas of them), both about the mean of the means, as
+// DK_FUSED; the replicas' sums meet in float64, component k's of all CTAs in CTA k % 16, which updates it and writes its constants to all.  Two
+// cluster barriers.
+// Bound by the latency of that chain: 10K x 16, K = 8 (cycles of an iteration, about): centre 1300, log-sum-exp 5400, statistics 3000, replicas 2000, sums of all CTAs 2000,
+// update 3300, barriers 1500.  10 iterations 210 to 230 -> 171 us.
+constexpr double FIT_MOST = 6.5e6;
+constexpr int FIT_SMEM = 220 * 1024;
+constexpr int ST_NONE_NEW = 1 << 30;          // (a status that was there before)
+constexpr int FT = 512, FC = 16, FIT_VALUES = 36, FIT_STRIDE = FT + 1;
+
+struct FitArgs {
+    const float* X;
+    int64_t n;
+    int D, K, P;             // points per CTA
+    int D4, ld, ldr, kr, lgG, T, R, lgP, xvec;            // (2^lgP lanes share the replicas of an output)
+    unsigned inv;            // tile * inv >> 16 = tile / D4
+    float *pi, *mu, *var;
+    float var_floor;
+    int isotropic;
+    double tol;
+    double* ll;              // [slots] iteration i at i % slots
+    int slots, first, end;   // iterations
+    int *counts, *stop_at, *status;
+};
+
+__device__ __forceinline__ uint32_t fit_remote(const void* p, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ double fit_load(uint32_t a) { double v; asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory"); return v; }
+__device__ __forceinline__ void fit_store(uint32_t a, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+__device__ __forceinline__ void fit_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ double fit_warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__global__ void __launch_bounds__(FT, 1) direct_fit_kernel(const FitArgs p) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ double red_s[FT / 32], llr_s[FC];
+    __shared__ __align__(16) float gs[128];
+    __shared__ float pi_s[4];
+    __shared__ int cnt_s[2], bad_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int rank;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    const int D = p.D, K = p.K, D4 = p.D4, ld = p.ld, ldr = p.ldr, kr = p.kr, P = p.P, KD = K * D, W = 2 * D + 1;
+    const int own = rank < K ? (K - rank + FC - 1) / FC : 0;             // this CTA's components: rank, rank + 16, ..
+    double* const part = reinterpret_cast<double*>(sm);                  // [K + 2 K D + 1] N_k, sums, log-likelihood of this CTA's points
+    double* const tmp = part + K + 2 * KD + 1;                           // [16][own][W] of all CTAs
+    float* const sw = reinterpret_cast<float*>(tmp + FC * ((K + FC - 1) / FC) * W + (K + 1) % 2);         // [kr][ld] sqrt(w2)
+    float* const ms = sw + kr * ld;                                      // (g - mu) sqrt(w2)
+    float* const mean = ms + kr * ld;
+    float* const cvs = mean + kr * ld;                                   // [kr]
+    float* const vars = cvs + kr;                                        // [own][D]
+    float* const xs = vars + ((K + FC - 1) / FC * D + 3) / 4 * 4;        // [P][ld]
+    float* const rs = xs + P * ld;                                       // [P][ldr]
+    const int64_t row0 = (int64_t)rank * P;
+    const int mine = (int)(p.n - row0 < 0 ? 0 : p.n - row0 < P ? p.n - row0 : P);
+    if (rank == 0 && tid < 2) p.counts[tid] = 0;
+    if (tid == 0) bad_s = 0;
+    __syncthreads();
+    // ---- points and parameters
+    for (int e = tid; e < P * D4; e += FT) {
+        const int r = e / D4, c = 4 * (e - r * D4);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < mine) {
+            const float* src = p.X + (row0 + r) * D + c;
+            if (p.xvec) v = __ldcg(reinterpret_cast<const float4*>(src));
+            else {
+                v.x = __ldcg(src);
+                if (c + 1 < D) v.y = __ldcg(src + 1);
+                if (c + 2 < D) v.z = __ldcg(src + 2);
+                if (c + 3 < D) v.w = __ldcg(src + 3);
+            }
+        }
+        *reinterpret_cast<float4*>(xs + r * ld + c) = v;
+    }
+    int bad = *p.status != 0 ? ST_NONE_NEW : 0;
+    for (int k = warp; k < kr; k += FT / 32)
+      for (int d = lane; d < 4 * D4; d += 32) {
+        float w = 0.f, m = 0.f;
+        if (k < K && d < D) {
+            const float v = __ldcg(p.var + k * D + d);
+            m = __ldcg(p.mu + k * D + d);
+            if (!(v > 0.f) || !isfinite(v)) bad |= ST_BAD_VAR;
+            if (!isfinite(m)) bad |= ST_NONFINITE;
+            w = sqrtf((float)(0.72134752044448170368 / (double)v));
+            if (k % FC == rank) vars[k / FC * D + d] = v;
+        }
+        sw[k * ld + d] = w;
+        mean[k * ld + d] = m;
+        ms[k * ld + d] = 0.f;
+    }
+    for (int k = warp; k < kr; k += FT / 32) {
+        double lg = 0.0;
+        if (k < K)
+            for (int d = lane; d < D; d += 32) lg += log(6.283185307179586476925286766559 * (double)__ldcg(p.var + k * D + d));
+        lg = fit_warp_sum(lg);
+        if (lane == 0) {
+            float c = -CUDART_INF_F;
+            if (k < K) {
+                const float w = __ldcg(p.pi + k);
+                if (!(w >= 0.f) || !isfinite(w)) bad |= ST_BAD_PI;
+                c = (float)(1.4426950408889634074 * ((w > 0.f ? log((double)w) : -CUDART_INF) - 0.5 * lg));
+                if (k % FC == rank) pi_s[k / FC] = w;
+            }
+            cvs[k] = c;
+        }
+    }
+    const int lgG = p.lgG, G = 1 << lgG, gq = lane & (G - 1);
+    const int rep = tid / p.T, tt = tid - rep * p.T, dt = tt % D4, kt = tt / D4;
+    double prev = p.first > 0 ? __ldcg(p.ll + (p.first - 1) % p.slots) : 0.0;
+    const double rk = 1.0 / (double)K;
+    bool updated = false, stop = false;
+    int it = p.first;
+    for (; it < p.end; ++it) {
+        __syncthreads();
+        if (tid < 2) cnt_s[tid] = 0;
+        if (tid < 128) {
+            double a = 0.0;
+            if (tid < D)
+#pragma unroll 8
+                for (int k = 0; k < K; ++k) a += (double)mean[k * ld + tid];
+            const float c = (float)(a * rk);
+            gs[tid] = tid < D && isfinite(c) ? c : 0.f;
+        }
+        __syncthreads();
+        for (int k = warp; k < K; k += FT / 32)
+            for (int d = lane; d < D; d += 32) {
+                const float m = mean[k * ld + d], w = sw[k * ld + d];
+                if (!isfinite(m)) bad |= ST_NONFINITE;
+                if (!(w > 0.f) || !isfinite(w)) bad |= ST_BAD_VAR;
+                ms[k * ld + d] = (gs[d] - m) * w;
+            }
+        if (tid < K && isnan(cvs[tid])) bad |= ST_BAD_PI;
+        __syncthreads();
+        // ---- log-sum-exp, responsibilities
+        double ll = 0.0;
+        float cv[4];
+#pragma unroll
+        for (int b = 0; b < 4; ++b) cv[b] = cvs[gq + G * b];
+        auto points = [&](auto pts) {
+            constexpr int PT = decltype(pts)::value;
+            for (int base = warp * 32; base < P << lgG; base += PT * FT) {
+                const float* xr[PT];
+                u64 q[PT][4];
+#pragma unroll
+                for (int j = 0; j < PT; ++j) {
+                    xr[j] = xs + min((base + j * FT + lane) >> lgG, P - 1) * ld;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) q[j][b] = 0ull;
+                }
+#pragma unroll 2
+                for (int d4 = 0; d4 < D4; ++d4) {
+                    const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gs + 4 * d4);
+                    ulonglong2 x[PT];
+#pragma unroll
+                    for (int j = 0; j < PT; ++j) {
+                        x[j] = *reinterpret_cast<const ulonglong2*>(xr[j] + 4 * d4);
+                        x[j].x = fma2(g.x, 0xBF800000BF800000ull, x[j].x);
+                        x[j].y = fma2(g.y, 0xBF800000BF800000ull, x[j].y);
+                    }
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + (gq + G * b) * ld + 4 * d4);
+                        const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ms + (gq + G * b) * ld + 4 * d4);
+#pragma unroll
+                        for (int j = 0; j < PT; ++j) {
+                            const u64 t0 = fma2(x[j].x, w.x, m.x), t1 = fma2(x[j].y, w.y, m.y);
+                            q[j][b] = fma2(t0, t0, q[j][b]);
+                            q[j][b] = fma2(t1, t1, q[j][b]);
+                        }
+                    }
+                }
+                float l[PT][4], m[PT], a[PT];
+#pragma unroll
+                for (int j = 0; j < PT; ++j) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) l[j][b] = cv[b] - (lo2(q[j][b]) + hi2(q[j][b]));
+                    m[j] = fmaxf(fmaxf(l[j][0], l[j][1]), fmaxf(l[j][2], l[j][3]));
+                }
+                for (int o = 1; o < G; o <<= 1)
+#pragma unroll
+                    for (int j = 0; j < PT; ++j) m[j] = fmaxf(m[j], __shfl_xor_sync(0xffffffffu, m[j], o));
+#pragma unroll
+                for (int j = 0; j < PT; ++j) {
+                    const float ref = m[j] == -CUDART_INF_F ? 0.f : m[j];
+                    a[j] = 0.f;
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) { l[j][b] = dk_ex2(l[j][b] - ref); a[j] += l[j][b]; }
+                }
+                for (int o = 1; o < G; o <<= 1)
+#pragma unroll
+                    for (int j = 0; j < PT; ++j) a[j] += __shfl_xor_sync(0xffffffffu, a[j], o);
+#pragma unroll
+                for (int j = 0; j < PT; ++j) {
+                    const int pt = (base + j * FT + lane) >> lgG;
+                    const bool in = pt < mine;
+                    if (in && gq == 0) ll += (double)m[j] + (double)log2f(a[j]);
+                    const float f = in ? 1.0f / a[j] : 0.f;
+                    if (pt < P) {
+#pragma unroll
+                        for (int b = 0; b < 4; ++b)
+                            if (gq + G * b < ldr) rs[pt * ldr + gq + G * b] = in ? l[j][b] * f : 0.f;
+                    }
+                }
+            }
+        };
+        // (as many points per lane at once as there are rounds, up to three: the rounds' latencies overlap)
+        const int rounds = ((P << lgG) + FT - 1) / FT;
+        if (rounds == 1) points(std::integral_constant<int, 1>{});
+        else if (rounds == 2) points(std::integral_constant<int, 2>{});
+        else points(std::integral_constant<int, 3>{});
+        ll = fit_warp_sum(ll);
+        if (lane == 0) red_s[warp] = ll;
+        __syncthreads();
+        // ---- statistics
+        u64 a1[4][2], a2[4][2];
+        float nacc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) a1[c][0] = a1[c][1] = a2[c][0] = a2[c][1] = 0ull;
+        if (rep < p.R) {
+            ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gs + 4 * dt);
+#pragma unroll 2
+            for (int r = rep; r < mine; r += p.R) {
+                ulonglong2 x = *reinterpret_cast<const ulonglong2*>(xs + r * ld + 4 * dt);
+                x.x = fma2(g.x, 0xBF800000BF800000ull, x.x);
+                x.y = fma2(g.y, 0xBF800000BF800000ull, x.y);
+                const u64 y0 = mul2(x.x, x.x), y1 = mul2(x.y, x.y);
+                const float4 w = *reinterpret_cast<const float4*>(rs + r * ldr + 4 * kt);
+                const float rr[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const u64 rd = dup2(rr[c]);
+                    nacc[c] += rr[c];
+                    a1[c][0] = fma2(rd, x.x, a1[c][0]);
+                    a1[c][1] = fma2(rd, x.y, a1[c][1]);
+                    a2[c][0] = fma2(rd, y0, a2[c][0]);
+                    a2[c][1] = fma2(rd, y1, a2[c][1]);
+                }
+            }
+        }
+        __syncthreads();                                     // (the responsibilities have been read)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float* const o = rs + 8 * c * FIT_STRIDE + tid;
+            o[0] = lo2(a1[c][0]); o[FIT_STRIDE] = hi2(a1[c][0]); o[2 * FIT_STRIDE] = lo2(a1[c][1]); o[3 * FIT_STRIDE] = hi2(a1[c][1]);
+            o[4 * FIT_STRIDE] = lo2(a2[c][0]); o[5 * FIT_STRIDE] = hi2(a2[c][0]); o[6 * FIT_STRIDE] = lo2(a2[c][1]); o[7 * FIT_STRIDE] = hi2(a2[c][1]);
+            rs[(32 + c) * FIT_STRIDE + tid] = nacc[c];
+        }
+        __syncthreads();
+        // (a warp has a value of all tiles; neighbouring lanes share a tile's replicas)
+        for (int i = warp; i < FIT_VALUES; i += FT / 32)
+            for (int t0 = 0; t0 < p.T; t0 += 32 >> p.lgP) {
+                const int tile = t0 + (lane >> p.lgP), q = lane & ((1 << p.lgP) - 1);
+                double a[2] = {0.0, 0.0};
+                if (tile < p.T) {
+                    const float* const v = rs + i * FIT_STRIDE + tile;
+#pragma unroll 4
+                    for (int r = q; r < p.R; r += 2 << p.lgP) {
+                        a[0] += (double)v[r * p.T];
+                        if (r + (1 << p.lgP) < p.R) a[1] += (double)v[(r + (1 << p.lgP)) * p.T];
+                    }
+                }
+                double t = a[0] + a[1];
+                for (int x = 1; x < 1 << p.lgP; x <<= 1) t += __shfl_xor_sync(0xffffffffu, t, x);
+                const int row = (int)(((unsigned)tile * p.inv) >> 16), col = tile - row * D4, k = 4 * row + (i < 32 ? i >> 3 : i - 32), d = 4 * col + (i & 3);
+                if (tile < p.T && q == 0 && k < K && (i < 32 ? d < D : col == 0)) part[i >= 32 ? k : K + (i & 4 ? KD : 0) + k * D + d] = t;
+            }
+        if (tid == 0) {
+            double a = 0.0;
+            for (int w = 0; w < FT / 32; ++w) a += red_s[w];
+            part[K + 2 * KD] = a * 0.69314718055994530942;
+        }
+        if (bad) atomicOr(&bad_s, bad);
+        __syncthreads();
+        bad = bad_s;                                         // (the same in every CTA)
+        fit_barrier();
+        // ---- all CTAs' sums of this CTA's components; everyone needs to know what becomes of the iteration
+        if (tid < FC) llr_s[tid] = fit_load(fit_remote(part + K + 2 * KD, tid));
+        static_assert(FT / 32 == FC, "a warp per CTA");
+        for (int kc = 0; kc < own; ++kc) {
+            const int k = rank + FC * kc;
+            for (int out = lane; out < W; out += 32)
+                tmp[(warp * own + kc) * W + out] = fit_load(fit_remote(part + (out == 0 ? k : out <= D ? K + k * D + out - 1 : K + KD + k * D + out - 1 - D), warp));
+        }
+        __syncthreads();
+        for (int o = tid; o < own * W; o += FT) {
+            double a = 0.0;
+#pragma unroll
+            for (int src = 0; src < FC; ++src) a += tmp[src * own * W + o];
+            tmp[o] = a;
+        }
+        ll = 0.0;
+#pragma unroll
+        for (int src = 0; src < FC; ++src) ll += llr_s[src];
+        __syncthreads();
+        const bool good = bad == 0 && isfinite(ll);          // a step that failed leaves the parameters as they are
+        stop = !good || (p.tol > 0.0 && it > 0 && fabs(ll - prev) <= p.tol * fabs(ll));
+        prev = ll;
+        if (rank == 0 && tid == 0) p.ll[it % p.slots] = ll;
+        if (good) {
+            updated = true;
+            for (int kc = warp; kc < own; kc += FT / 32) {
+                const int k = rank + FC * kc;
+                const double* const t = tmp + kc * W;
+                const double n = t[0];
+                const bool empty = n < 1e-12;                // an empty component keeps mu and var
+                const double rn = 1.0 / n;
+                const float pf = (float)(n / (double)p.n);   // pi_k = N_k / N
+                const double lp = pf > 0.f ? log((double)pf) : pf == 0.f ? -CUDART_INF : CUDART_NAN;
+                double vd[4], vsum = 0.0, lg = 0.0;
+                int floored = 0;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int d = lane + 32 * i;
+                    vd[i] = 0.0;
+                    if (d >= D || empty) continue;
+                    const double g = (double)gs[d], s1 = t[1 + d] + g * n, s2 = t[1 + D + d] + 2.0 * g * t[1 + d] + g * g * n, m = s1 * rn;      // Eq. 2
+                    vd[i] = s2 * rn - m * m;                 // Eq. 3 per dimension, new mean
+                    vsum += vd[i];
+                    for (int c = 0; c < FC; ++c) fit_store(fit_remote(mean + k * ld + d, c), (float)m);
+                }
+                const double fl = (double)p.var_floor;
+                if (p.isotropic) {                           // one variance: the mean over the dimensions
+                    vsum = fit_warp_sum(vsum) / (double)D;
+                    if (!empty && !(vsum > fl)) { vsum = fl; if (lane == 0) floored = D; }
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int d = lane + 32 * i;
+                    if (d >= D) continue;
+                    if (!empty) {
+                        double v = p.isotropic ? vsum : vd[i];
+                        if (!p.isotropic && !(v > fl)) { v = fl; ++floored; }
+                        vars[kc * D + d] = (float)v;
+                    }
+                    const float vf = vars[kc * D + d];
+                    lg += log(6.283185307179586476925286766559 * (double)vf);
+                    const float w = sqrtf((float)(0.72134752044448170368 / (double)vf));
+                    for (int c = 0; c < FC; ++c) fit_store(fit_remote(sw + k * ld + d, c), w);
+                }
+                lg = fit_warp_sum(lg);
+                floored = __reduce_add_sync(0xffffffffu, floored);
+                if (lane < FC) fit_store(fit_remote(cvs + k, lane), (float)(1.4426950408889634074 * (lp - 0.5 * lg)));
+                if (lane == 0) {
+                    pi_s[kc] = pf;
+                    if (floored) atomicAdd(&cnt_s[0], floored);
+                    if (empty) atomicAdd(&cnt_s[1], 1);
+                }
+            }
+        }
+        __syncthreads();
+        fit_barrier();
+        if (stop) break;
+    }
+    if (updated) {
+        __syncthreads();
+        for (int e = tid; e < own * D; e += FT) {
+            const int kc = e / D, d = e - kc * D, k = rank + FC * kc;
+            p.mu[(size_t)k * D + d] = mean[k * ld + d];
+            p.var[(size_t)k * D + d] = vars[e];
+        }
+        if (tid < own) p.pi[rank + FC * tid] = pi_s[tid];
+        if (tid < 2 && cnt_s[tid]) atomicAdd(p.counts + tid, cnt_s[tid]);
+    }
+    if (rank == 0 && tid == 0) {
+        *p.stop_at = stop ? it : 0x7f7f7f7f;
+        if (bad & ~ST_NONE_NEW) atomicOr(p.status, bad & ~ST_NONE_NEW);
+    }
+}
+
+// ------------------------------------------------------------------------------------------------------------------
 struct DirectPlan {
     DirectArgs a;
     int PT, TK;
@@ -659,6 +1041,58 @@ cudaError_t launch_reduce_direct(cudaStream_t s, int D, int K, int splits, const
     ReduceArgs r{};
     r.D = D; r.K = K; r.splits = splits; r.partials = partials; r.g = g; r.Nk = Nk; r.S1 = S1; r.S2 = S2; r.accumulate = accumulate ? 1 : 0;
     return launch_chained(s, dim3((unsigned)K), 1024, 0, direct_reduce_kernel, r);
+}
+
+// Where one launch is the faster way: 16 SMs take about as long for a point and component as for 16 dimensions more, two launches per iteration 14 to 20 us
+// (whole fits of five iterations, us, launches / one launch: 5K x 64, K = 16 204 / 159, 20K x 16, K = 8 143 / 125, 5K x 16, K = 32 154 / 133, 10K x 32, K = 8
+// 150 / 120, 2K x 4, K = 3 147 / 89; beyond the line 20K x 16, K = 16 153 / 170, 100K x 4, K = 4 150 / 134).
+static bool fit_plan(const float* X, int64_t n, int D, int K, FitArgs* out, size_t* smem) {
+    if (D > 128 || K > 64 || K * D > 1024 || (double)n * K * (D + 16) > FIT_MOST) return false;
+    FitArgs a{};
+    a.X = X; a.n = n; a.D = D; a.K = K;
+    a.P = (int)((n + FC - 1) / FC);
+    a.D4 = (D + 3) / 4;
+    a.ld = 4 * (a.D4 | 1);
+    while ((4 << a.lgG) < K) ++a.lgG;
+    a.kr = 4 << a.lgG;
+    const int k4 = (K + 3) / 4;
+    a.ldr = 4 * (k4 | 1);
+    a.T = k4 * a.D4;
+    a.R = FT / a.T;
+    while ((a.T << (a.lgP + 1)) <= 32) ++a.lgP;
+    a.inv = (65536u + a.D4 - 1) / a.D4;                      // (exact below 65536 / D4: at most 256 tiles of 32 columns)
+    a.xvec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
+    const size_t rs = (size_t)a.P * a.ldr, sums = (size_t)FIT_VALUES * FIT_STRIDE;
+    const int most = (K + FC - 1) / FC, W = 2 * D + 1;
+    size_t bytes = 8 * (size_t)(K + 2 * K * D + 1 + FC * most * W + (K + 1) % 2);
+    bytes += 4 * ((size_t)3 * a.kr * a.ld + a.kr + (most * D + 3) / 4 * 4 + (size_t)a.P * a.ld + (rs > sums ? rs : sums));
+    if (bytes > FIT_SMEM) return false;
+    *out = a;
+    *smem = bytes;
+    return true;
+}
+bool fit_direct_supports(const float* X, int64_t n, int D, int K) {
+    FitArgs a;
+    size_t smem;
+    return fit_plan(X, n, D, K, &a, &smem);
+}
+cudaError_t launch_fit_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const DirectFit& f, double* ll, int slots, int end, int* status) {
+    FitArgs a;
+    size_t smem;
+    if (!fit_plan(X, n, D, K, &a, &smem)) return cudaErrorInvalidValue;
+    a.pi = f.pi; a.mu = f.mu; a.var = f.var; a.var_floor = f.var_floor; a.isotropic = f.isotropic ? 1 : 0; a.tol = f.tol;
+    a.ll = ll; a.slots = slots; a.first = f.iter; a.end = end; a.counts = f.counts; a.stop_at = f.stop_at; a.status = status;
+    // (the same limits from every call: they belong to the kernel)
+    cudaError_t e = cudaFuncSetAttribute(direct_fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FIT_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(direct_fit_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(FC); cfg.blockDim = dim3(FT); cfg.dynamicSmemBytes = smem; cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = FC; at.val.clusterDim.y = 1; at.val.clusterDim.z = 1;
+    cfg.attrs = &at; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, direct_fit_kernel, a);
 }
 
 bool fused_direct_supports(int D, int K) { return D <= 128 && K <= 64; }

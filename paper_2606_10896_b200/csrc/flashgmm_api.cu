@@ -1188,16 +1188,31 @@ int gmm_fit(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, float* pi, fl
         // Small mixtures: two launches per iteration (the update and the next iteration's constants are part of the reduction), as
         // many iterations as there are slots for their log-likelihoods enqueued ahead; the device stops by itself where the
         // tolerance is met or a step fails.
-        KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), nullptr, &ctx->result()->status));
-        CU(cudaMemsetAsync(&ctx->result()->stop_at, 0x7f, sizeof(int), ctx->stream));
+        // Where the points fit into the shared memory of a cluster, those are one launch.
+        bool one = fit_direct_supports(X, N, D, K), prepared = false;
         ctx->last_path = GMM_PATH_FP32;
         while (t < iters) {
             const int end = iters - t < LL_SLOTS - 1 ? iters : t + LL_SLOTS - 1;      // (one slot holds the value before them)
-            for (int i = t; i < end; ++i) {
-                DirectFit f;
-                f.pi = pi; f.mu = mu; f.var = var; f.var_floor = var_floor; f.isotropic = ctx->covariance == GMM_COV_ISOTROPIC;
-                f.tol = tol; f.ll_prev = i > 0 ? &ctx->result()->ll[(i - 1) % LL_SLOTS] : nullptr;
-                f.counts = ctx->result()->counts; f.stop_at = &ctx->result()->stop_at; f.iter = i;
+            DirectFit f;
+            f.pi = pi; f.mu = mu; f.var = var; f.var_floor = var_floor; f.isotropic = ctx->covariance == GMM_COV_ISOTROPIC;
+            f.tol = tol; f.counts = ctx->result()->counts; f.stop_at = &ctx->result()->stop_at;
+            if (one) {
+                f.iter = t;
+                f.ll_prev = nullptr;
+                CHECK(prof_begin(ctx));
+                one = launch_fit_direct(ctx->stream, X, N, D, K, f, ctx->result()->ll, LL_SLOTS, end, &ctx->result()->status) == cudaSuccess;
+                if (one) ctx->launches++;
+                else cudaGetLastError();                     // (no 16 SMs together: the launches)
+                CHECK(prof_end(ctx));
+            }
+            if (!one && !prepared) {
+                KL(launch_prepare_fp32(ctx->stream, D, K, pi, mu, var, ctx->w2(), ctx->c2(), ctx->c2d(), nullptr, &ctx->result()->status));
+                CU(cudaMemsetAsync(&ctx->result()->stop_at, 0x7f, sizeof(int), ctx->stream));
+                prepared = true;
+            }
+            for (int i = t; i < end && !one; ++i) {
+                f.ll_prev = i > 0 ? &ctx->result()->ll[(i - 1) % LL_SLOTS] : nullptr;
+                f.iter = i;
                 CHECK(prof_begin(ctx));
                 CU(launch_fused_direct(ctx->stream, X, N, D, K, mu, ctx->w2(), ctx->c2(), ctx->c2d(), ctx->center(), ctx->partials(), ctx->llpart(), Nk, S1,
                                        S2, false, &ctx->result()->ll[i % LL_SLOTS], &ctx->result()->status, &f, &ctx->launches));

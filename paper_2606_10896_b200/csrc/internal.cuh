@@ -78,6 +78,10 @@ struct DirectFit {
     int* stop_at;
     int iter;
 };
+// A fit of iterations f.iter .. end - 1 in one launch (f.ll_prev is not read: iteration i's log-likelihood is at ll[i % slots]; *f.stop_at: the iteration after which
+// nothing was done, or a large number), for shapes that fit_direct_supports.
+bool fit_direct_supports(const float* X, int64_t n, int D, int K);
+cudaError_t launch_fit_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const DirectFit& f, double* ll, int slots, int end, int* status);
 bool fused_direct_supports(int D, int K);
 cudaError_t launch_fused_direct(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, float* w2, float* c2,
                                 double* c2d, float* g, float* partials, double* llpart, double* Nk, double* S1, double* S2,

@@ -73,6 +73,41 @@ def test_direct_fit_runs_ahead_and_stops_by_itself(fg, isotropic):
         assert all(torch.equal(u, v) for u, v in zip(b, d))      # nothing was done after the iteration that met the tolerance
 
 
+# A fit that is one launch of a cluster of 16 CTAs: fewer points than CTAs, CTAs without components or with several, lanes per point 1 to 16, dimensions that are no
+# multiple of four, rows that do not start on 16 bytes; against steps and updates one by one (the same sums in another order: 1e-4 of the data's scale after
+# four iterations at most).
+@pytest.mark.parametrize("isotropic", [False, True])
+@pytest.mark.parametrize("N,D,K,offset", [(1, 1, 1, 0), (15, 3, 2, 0), (40, 128, 8, 0), (2500, 16, 64, 0), (17, 2, 5, 1), (4099, 31, 9, 1), (1700, 5, 33, 0), (30_000, 2, 2, 0), (900, 1, 17, 3)])
+def test_direct_fit_in_one_launch(fg, N, D, K, offset, isotropic):
+    X, pi, mu, var = _mixture(N, D, K, 7 * N + D + K)
+    var = np.maximum(var, 1.0)
+    if isotropic:
+        var = np.repeat(var[:, :1], D, 1)
+    if K > 2:
+        pi[1] = 0.0                                        # (an empty component keeps its mean and variance)
+    flat = torch.empty(N * D + offset, device=DEV)
+    Xd = flat[offset:].view(N, D)
+    Xd.copy_(_t(X))
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        c.gmm_set_covariance(fg.GMM_COV_ISOTROPIC if isotropic else fg.GMM_COV_DIAG)
+        a, b, want = [_t(pi), _t(mu), _t(var)], [_t(pi), _t(mu), _t(var)], []
+        for _ in range(4):
+            Nk, S1, S2, ll = c.gmm_em_step(Xd, *a)
+            want.append(ll)
+            (c.gmm_finalize_isotropic if isotropic else c.gmm_finalize)(N, Nk, S1, S2, 0.3, *a)
+        counts = c.gmm_update_counts()
+        before = c.gmm_launch_count()
+        trace, done = c.gmm_fit(Xd, *b, 4, 0.3)
+        assert c.gmm_launch_count() - before <= 2 and done == 4 and c.gmm_update_counts() == counts
+        assert np.all(np.abs(trace - want) <= 1e-5 * np.abs(want) + 1e-5)
+        for u, v, s in zip(b, a, (1.0, data_scale(X) if N > 1 else 1.0, 1.0)):
+            assert float((u - v).abs().max()) <= 1e-4 * max(s, 1.0)
+        again = [_t(pi), _t(mu), _t(var)]
+        c.gmm_fit(Xd, *again, 4, 0.3)
+        assert all(torch.equal(u, v) for u, v in zip(again, b))      # the same bits in every run
+
+
 def test_direct_fit_keeps_the_parameters_of_a_step_that_fails(fg):
     X, pi, mu, var = _mixture(500, 5, 4, 9)
     X[17, 2] = np.nan

@@ -2357,20 +2357,31 @@ __global__ void __launch_bounds__(1024) screen_group_sort_kernel(int K, const in
     }
 }
 
-// Fisher vectors: a warp per (group, component).  With sums about the component's mean,
+// Fisher vectors.  With sums about the component's mean,
 //   G_mu = sum r (x - mu) / (T sigma sqrt(pi)),   G_sigma = (sum r (x - mu)^2 / var - sum r) / (T sqrt(2 pi)):
-// nothing cancels.  fp32 sums of 32 pairs at a time, added in fp32.
-__global__ void __launch_bounds__(256, 4) screen_group_stats_kernel(const float* __restrict__ X, int D, int K, int lpr, int groups,
+// nothing cancels.  fp32 sums of at most 32 pairs at a time, added in fp32.  A warp has runs of GS_COMPS components of a group, whose pairs are neighbours: their rows
+// come in one stream, as in screen_stats_kernel (GS_STAGES stages of GS_ROWS loads per lane), the parameters one component ahead.
+// Bound by the gathered rows and the runs' first trips.  150 groups of 6827 points, us per call, with a warp per component and 16 rows in flight, waited for / now:
+// 64 x 256 676 / 597, 128 x 512 1139 / 970, 100 x 33 881 / 659; 500 groups of 2000 x 64, K = 256 691 / 623.
+constexpr int GS_COMPS = 8, GS_ROWS = 4, GS_STAGES = 8;      // (components of a run at most)
+template <int LPR, bool VEC>
+__global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel(const float* __restrict__ X, int D, int K, int groups, int comps,
                                                                  const float* __restrict__ pi, const float* __restrict__ mu,
                                                                  const float* __restrict__ var, const float* __restrict__ w2,
                                                                  const double* __restrict__ c2d, const uint2* __restrict__ srt,
                                                                  const int* __restrict__ g_off, const int* __restrict__ g_len,
                                                                  float* __restrict__ fv, double* __restrict__ ll, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
-    __shared__ double red[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, l = lane % lpr, sub = lane / lpr, rows = 32 / lpr, d0 = 4 * l;
-    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
+    constexpr int ROWS = 32 / LPR, U = LPR < GS_ROWS ? LPR : GS_ROWS, SR = U * ROWS;        // pairs of a stage (at most 32)
+    constexpr int W = ST_THREADS / 32;
+    static_assert(GS_COMPS < 32, "a lane per offset");
+    extern __shared__ __align__(16) unsigned char ring_s[];                                 // [W][GS_STAGES][GS_ROWS][32] 16 bytes
+    __shared__ float r_s[W][GS_STAGES][32];
+    __shared__ double red[W];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LPR, sub = lane / LPR, d0 = 4 * l;
+    uint4* const ring = reinterpret_cast<uint4*>(ring_s) + (size_t)warp * GS_STAGES * GS_ROWS * 32 + lane;
     const bool vec_o = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(fv) & 15) == 0);
+    const bool vec_m = (D % 4 == 0) && (((reinterpret_cast<uintptr_t>(mu) | reinterpret_cast<uintptr_t>(var)) & 15) == 0);
     const size_t KD = (size_t)K * D;
     auto load4 = [&](const float* __restrict__ r, bool v) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -2384,112 +2395,148 @@ __global__ void __launch_bounds__(256, 4) screen_group_stats_kernel(const float*
         }
         return a;
     };
+    struct Comp { float4 m, w, v; float p; };
+    auto component = [&](int k) {
+        Comp c;
+        c.m = load4(mu + (size_t)k * D, vec_m);
+        c.v = load4(var + (size_t)k * D, vec_m);
+        c.w = load4(w2 + (size_t)k * D, (D & 3) == 0);       // (scratch, aligned)
+        c.p = __ldg(pi + k);
+        return c;
+    };
     double ll_acc = 0.0;
-    const bool vec_m = (D % 4 == 0) && (((reinterpret_cast<uintptr_t>(mu) | reinterpret_cast<uintptr_t>(var)) & 15) == 0);
-    // An item's trips to memory wait for one another (offsets, pairs, rows): the next item's offsets and first pairs are on their
-    // way while this one's rows are worked through, and four CTAs per SM hide the rest (500 groups of 2000 x 64, K = 256: 330 -> 282 us;
-    // eight rows in flight per lane at three CTAs: 332).
-    const int items = groups * K, stride = gridDim.x * 8;    // (at most 2^23)
-    int a_next = 0, b_next = 0;
-    uint2 e_next = make_uint2(0u, 0u);
-    auto offsets = [&](int item) {
-        if (item < items) {
-            const int* off = g_off + (size_t)item + item / K;      // [g][K + 1]
-            a_next = __ldg(off);
-            b_next = __ldg(off + 1);
-        }
-    };
-    auto pairs = [&]() {
-        e_next = make_uint2(0u, 0u);
-        if (a_next + lane < b_next) e_next = __ldg(srt + a_next + lane);
-    };
-    offsets(blockIdx.x * 8 + warp);
-    pairs();
-    for (int item = blockIdx.x * 8 + warp; item < items; item += stride) {
-        const int g = item / K, k = item - g * K;
-        const int a = a_next, b = b_next;
-        uint2 e = e_next;
-        offsets(item + stride);
-        float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, nsum = 0.f;
-        if (a < b) {
-            const float4 m = load4(mu + (size_t)k * D, vec_m), w = load4(w2 + (size_t)k * D, (D & 3) == 0);      // (w2: scratch, aligned)
-            for (int p = a; p < b; p += 32) {
-                if (p > a) {
-                    e = make_uint2(0u, 0u);
-                    if (p + lane < b) e = __ldg(srt + p + lane);
+    const float* const Xl = X + d0;
+    const int per = (K + comps - 1) / comps, runs = groups * per;        // (at most 2^23)
+#pragma unroll 1
+    for (int run = blockIdx.x * W + warp; run < runs; run += gridDim.x * W) {
+        const int g = run / per, k0 = (run - g * per) * comps, k1 = min(K, k0 + comps);
+        const int o = __ldg(g_off + (size_t)g * (K + 1) + k0 + min(lane, k1 - k0));
+        Comp c = component(k0);
+        const int p0 = __shfl_sync(0xffffffffu, o, 0), total = __shfl_sync(0xffffffffu, o, k1 - k0) - p0, stages = (total + SR - 1) / SR;
+        const uint2* const pairs = srt + p0;
+        const float inv_t = 1.0f / (float)__ldg(g_len + g);
+        uint2 e = make_uint2(0u, 0u), e_next;                // 32 pairs of which the next stages are, and the 32 after them (no pair: row 0, without weight)
+        auto fetch = [&](int i) {
+            e_next = make_uint2(0u, 0u);
+            if (i + lane < total) e_next = __ldg(pairs + i + lane);
+        };
+        auto issue = [&](int st) {
+            const int slot = st % GS_STAGES, at = (st * SR) & 31;
+            if (st < stages) {
+                if (at == 0) {
+                    e = e_next;
+                    fetch(st * SR + 32);
                 }
-                const float re = __uint_as_float(e.y);
-                nsum += re;
-                float4 f1 = make_float4(0.f, 0.f, 0.f, 0.f), f2 = f1;
-                const int have = min(32, b - p);
-                for (int i = 0; i < have; i += 4 * rows) {
-                    float4 x[4];
-                    float r[4];
+                const float r = __shfl_sync(0xffffffffu, __uint_as_float(e.y), (at + lane) & 31);
+                if (lane < SR) r_s[warp][slot][lane] = r;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int src = min(31, i + u * rows + sub);
-                        const unsigned row = __shfl_sync(0xffffffffu, e.x, src);
-                        r[u] = __shfl_sync(0xffffffffu, re, src);
-                        if (i + u * rows + sub >= have) r[u] = 0.f;
-                        x[u] = make_float4(m.x, m.y, m.z, m.w);
-                        if (r[u] != 0.f) x[u] = load4(X + (size_t)row * D, vec);
-                    }
+                for (int u = 0; u < U; ++u) {
+                    const unsigned row = __shfl_sync(0xffffffffu, e.x, at + u * ROWS + sub);
+                    const float* src = Xl + (size_t)row * D;
+                    const uint32_t dst = smem_u32(ring + (slot * GS_ROWS + u) * 32);
+                    if (VEC) {
+                        if (d0 < D) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+                    } else {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const float ra = r[u];
-                        const float tx = x[u].x - m.x, ty = x[u].y - m.y, tz = x[u].z - m.z, tw = x[u].w - m.w;
-                        f1.x = fmaf(ra, tx, f1.x); f1.y = fmaf(ra, ty, f1.y); f1.z = fmaf(ra, tz, f1.z); f1.w = fmaf(ra, tw, f1.w);
-                        const float ax = tx * tx, ay = ty * ty, az = tz * tz, aw = tw * tw;
-                        f2.x = fmaf(ra, ax, f2.x); f2.y = fmaf(ra, ay, f2.y); f2.z = fmaf(ra, az, f2.z); f2.w = fmaf(ra, aw, f2.w);
+                        for (int j = 0; j < 4; ++j)
+                            if (d0 + j < D) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4 * j), "l"(src + j) : "memory");
                     }
                 }
-                s1[0] += f1.x; s1[1] += f1.y; s1[2] += f1.z; s1[3] += f1.w;
-                s2[0] += f2.x; s2[1] += f2.y; s2[2] += f2.z; s2[3] += f2.w;
             }
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                for (int o = lpr; o < 32; o <<= 1) {
-                    s1[j] += __shfl_xor_sync(0xffffffffu, s1[j], o);
-                    s2[j] += __shfl_xor_sync(0xffffffffu, s2[j], o);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        fetch(0);
+#pragma unroll 1
+        for (int st = 0; st < GS_STAGES - 1; ++st) issue(st);
+        int cur = 0, ready = -1;                             // pairs done; the stage that has arrived
+#pragma unroll 1
+        for (int k = k0; k < k1; ++k) {
+            const int b = __shfl_sync(0xffffffffu, o, k - k0 + 1) - p0;
+            const Comp now = c;
+            if (k + 1 < k1) c = component(k + 1);
+            uint64_t m[2] = {pack2(__float_as_uint(now.m.x), __float_as_uint(now.m.y)), pack2(__float_as_uint(now.m.z), __float_as_uint(now.m.w))};
+            float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, nsum = 0.f;
+            const bool any = cur < b;
+#pragma unroll 1
+            while (cur < b) {
+                const int st = cur / SR, pos = st * SR, to = min(b, pos + SR), slot = st % GS_STAGES;
+                if (st != ready) {
+                    __syncwarp();                            // (the stage before has been read)
+                    issue(st + GS_STAGES - 1);
+                    asm volatile("cp.async.wait_group %0;" ::"n"(GS_STAGES - 1) : "memory");
+                    __syncwarp();
+                    ready = st;
                 }
-            float quad = sub == 0 ? fmaf(w.x, s2[0], fmaf(w.y, s2[1], fmaf(w.z, s2[2], w.w * s2[3]))) : 0.f;      // (see screen_reduce_kernel)
+                const uint4* const xs = ring + slot * GS_ROWS * 32;
+                const float* const rs = r_s[warp][slot];
+                uint64_t f1[2] = {0ull, 0ull}, f2[2] = {0ull, 0ull};
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                nsum += __shfl_xor_sync(0xffffffffu, nsum, o);
-                quad += __shfl_xor_sync(0xffffffffu, quad, o);
+                for (int u = 0; u < U; ++u) {
+                    const int i = pos + u * ROWS + sub;
+                    const bool on = i >= cur && i < to;
+                    const float r = on ? rs[u * ROWS + sub] : 0.f;
+                    const uint4 x = xs[u * 32];
+                    const uint64_t rr = pack2(__float_as_uint(r), __float_as_uint(r));
+                    uint64_t ta = sub2(pack2(x.x, x.y), m[0]), tb = sub2(pack2(x.z, x.w), m[1]);
+                    if (!on) ta = tb = 0ull;                 // (a row of another component: the square may be beyond a float)
+                    f1[0] = fma2(rr, ta, f1[0]);
+                    f1[1] = fma2(rr, tb, f1[1]);
+                    f2[0] = fma2(rr, mul2(ta, ta), f2[0]);
+                    f2[1] = fma2(rr, mul2(tb, tb), f2[1]);
+                }
+                nsum += lane < SR && pos + lane >= cur && pos + lane < to ? rs[lane] : 0.f;
+                s1[0] += lo2(f1[0]); s1[1] += hi2(f1[0]); s1[2] += lo2(f1[1]); s1[3] += hi2(f1[1]);
+                s2[0] += lo2(f2[0]); s2[1] += hi2(f2[0]); s2[2] += lo2(f2[1]); s2[3] += hi2(f2[1]);
+                cur = to;
             }
-            if (lane == 0) ll_acc += (double)nsum * c2d[k] - (double)quad;
-        }
-        pairs();                                             // (of the next item)
-        const float wk = __ldg(pi + k), inv_t = 1.0f / (float)g_len[g];
-        const float4 vf = load4(var + (size_t)k * D, vec_m);
-        const float va[4] = {vf.x, vf.y, vf.z, vf.w};
-        float gm[4], gs[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            gm[j] = gs[j] = 0.f;
-            if (a < b && wk > 0.f && d0 + j < D) {
-                gm[j] = s1[j] * (inv_t * rsqrtf(va[j]) * rsqrtf(wk));
-                gs[j] = (s2[j] - nsum * va[j]) * (inv_t * rsqrtf(2.0f * wk) / va[j]);
-            }
-        }
-        if (sub == 0 && d0 < D) {
-            float* o = fv + (size_t)g * 2 * KD + (size_t)k * D + d0;
-            if (vec_o) {
-                *reinterpret_cast<float4*>(o) = make_float4(gm[0], gm[1], gm[2], gm[3]);
-                *reinterpret_cast<float4*>(o + KD) = make_float4(gs[0], gs[1], gs[2], gs[3]);
-            } else {
+            const float va[4] = {now.v.x, now.v.y, now.v.z, now.v.w}, wa[4] = {now.w.x, now.w.y, now.w.z, now.w.w};
+            float gm[4] = {0.f, 0.f, 0.f, 0.f}, gs[4] = {0.f, 0.f, 0.f, 0.f};
+            if (any) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (d0 + j < D) { o[j] = gm[j]; o[KD + j] = gs[j]; }
+#pragma unroll
+                    for (int x = LPR; x < 32; x <<= 1) {
+                        s1[j] += __shfl_xor_sync(0xffffffffu, s1[j], x);
+                        s2[j] += __shfl_xor_sync(0xffffffffu, s2[j], x);
+                    }
+                float quad = 0.f;                            // (see screen_reduce_kernel; beyond D garbage in s2)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (sub == 0 && d0 + j < D) quad = fmaf(wa[j], s2[j], quad);
+#pragma unroll
+                for (int x = 16; x > 0; x >>= 1) {
+                    nsum += __shfl_xor_sync(0xffffffffu, nsum, x);
+                    quad += __shfl_xor_sync(0xffffffffu, quad, x);
+                }
+                if (lane == 0) ll_acc += (double)nsum * c2d[k] - (double)quad;
+                const float wk = now.p;
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (wk > 0.f && d0 + j < D) {
+                        gm[j] = s1[j] * (inv_t * rsqrtf(va[j]) * rsqrtf(wk));
+                        gs[j] = (s2[j] - nsum * va[j]) * (inv_t * rsqrtf(2.0f * wk) / va[j]);
+                    }
+            }
+            if (sub == 0 && d0 < D) {
+                float* out = fv + (size_t)g * 2 * KD + (size_t)k * D + d0;
+                if (vec_o) {
+                    *reinterpret_cast<float4*>(out) = make_float4(gm[0], gm[1], gm[2], gm[3]);
+                    *reinterpret_cast<float4*>(out + KD) = make_float4(gs[0], gs[1], gs[2], gs[3]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (d0 + j < D) { out[j] = gm[j]; out[KD + j] = gs[j]; }
+                }
             }
         }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
     }
     if (lane == 0) red[warp] = ll_acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += red[w];
+        for (int w = 0; w < W; ++w) t += red[w];
         ll[blockIdx.x] += t * 0.69314718055994530942;
     }
 }
@@ -2660,7 +2707,7 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     LCHECK();
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0);
 #define FG_STATS(L_) (vec ? screen_stats_kernel<L_, true> : screen_stats_kernel<L_, false>)
-    const auto stats = D <= 4 ? FG_STATS(1) : D <= 8 ? FG_STATS(2) : D <= 16 ? FG_STATS(4) : D <= 32 ? FG_STATS(8) : D <= 64 ? FG_STATS(16) : FG_STATS(32);
+    const auto stats = D <= 8 ? FG_STATS(2) : D <= 16 ? FG_STATS(4) : D <= 32 ? FG_STATS(8) : D <= 64 ? FG_STATS(16) : FG_STATS(32);
 #undef FG_STATS
     constexpr int stats_smem = ST_THREADS / 32 * ST_STAGES * ST_ROWS * 512;
     e = cudaFuncSetAttribute(stats, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem);
@@ -2672,7 +2719,7 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     return cudaGetLastError();
 }
 
-cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int D, int K, const int* g_start, const int* g_len, int* g_off,
+cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int64_t n, int groups, int D, int K, const int* g_start, const int* g_len, int* g_off,
                                  const float* pi, const float* mu, const float* var, const float* w2, const double* c2d,
                                  const ScreenBuffers& b, float* fv, int64_t* launches) {
     const int K2 = (K + 1) & ~1;
@@ -2684,11 +2731,19 @@ cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int
     if (e != cudaSuccess) return e;
     screen_group_sort_kernel<<<groups, warps * 32, smem, s>>>(K, g_start, g_len, b.pt_off, b.pt_cnt, b.ids, b.val, g_off, b.srt, b.ctl);
     LCHECK();
-    int lpr = 1;
-    while (4 * lpr < D) lpr <<= 1;
-    const long long blocks = ((long long)groups * K + 7) / 8;
-    screen_group_stats_kernel<<<(unsigned)(blocks < SCR_LL ? blocks : SCR_LL), 256, 0, s>>>(X, D, K, lpr, groups, pi, mu, var, w2, c2d, b.srt, g_off,
-                                                                                            g_len, fv, b.ll, b.ctl);
+    const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
+#define FG_GROUPS(L_) (vec ? screen_group_stats_kernel<L_, true> : screen_group_stats_kernel<L_, false>)
+    const auto stats = D <= 8 ? FG_GROUPS(2) : D <= 16 ? FG_GROUPS(4) : D <= 32 ? FG_GROUPS(8) : D <= 64 ? FG_GROUPS(16) : FG_GROUPS(32);
+#undef FG_GROUPS
+    constexpr int stats_smem = ST_THREADS / 32 * GS_STAGES * GS_ROWS * 512;
+    e = cudaFuncSetAttribute(stats, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem);
+    if (e != cudaSuccess) return e;
+    // A run has about 400 pairs (2.2 kept ones per point on separate clusters), but there are runs enough for two rounds of warps: 150 groups of 6827, 64 x 256,
+    // runs of 8, 16, 31 components 627, 660, 661 us, 100 x 33 795, 1100, 1468 and with one 659.
+    const double pairs = 2.2 * (double)n / ((double)groups * K);
+    int comps = pairs * GS_COMPS <= 400.0 ? GS_COMPS : pairs >= 400.0 ? 1 : (int)(400.0 / pairs);
+    while (comps > 1 && (int64_t)groups * ((K + comps - 1) / comps) < 2 * SCR_STAT_WARPS) comps = (comps + 1) / 2;
+    stats<<<SCR_STAT_WARPS / (ST_THREADS / 32), ST_THREADS, stats_smem, s>>>(X, D, K, groups, comps, pi, mu, var, w2, c2d, b.srt, g_off, g_len, fv, b.ll, b.ctl);
     *launches += 2;
     return cudaGetLastError();
 }

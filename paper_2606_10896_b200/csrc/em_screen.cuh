@@ -108,9 +108,9 @@ cudaError_t launch_screen_gate(cudaStream_t s, const ScreenBuffers& b, int* gate
 cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D, int K, const float* mu, const float* w2,
                                 const double* c2d, const ScreenBuffers& b, double* Nk, double* S1, double* S2, int64_t* launches);
 
-// After the evaluation (SCREEN_EM): Fisher vectors of `groups` groups of consecutive points of the piece (group g =
+// After the evaluation (SCREEN_EM): Fisher vectors of `groups` groups of consecutive points (n in all) of the piece (group g =
 // g_len[g] <= SCR_GROUP points from row g_start[g] on, in order) into fv [groups][2][K][D].  g_off: groups * (K + 1) ints of scratch.
-cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int groups, int D, int K, const int* g_start, const int* g_len, int* g_off,
+cudaError_t launch_screen_groups(cudaStream_t s, const float* X, int64_t n, int groups, int D, int K, const int* g_start, const int* g_len, int* g_off,
                                  const float* pi, const float* mu, const float* var, const float* w2, const double* c2d,
                                  const ScreenBuffers& b, float* fv, int64_t* launches);
 // k-means: new centroids from (Nk, S1) as launch_screen_stats left them (unit parameters), points and inertia per centroid.

@@ -2087,7 +2087,7 @@ int gmm_fisher_vectors(gmm_ctx* ctx, const float* X, int64_t N, const int64_t* o
             } else {
                 CHECK(prof_begin(ctx));
                 CHECK(screen_values(ctx, SCREEN_EM, Xs, rows, D, K, 40.f, screen_limit(ctx, SCREEN_STEPS, N, D, K, G), mu, nullptr, nullptr, false));
-                CU(launch_screen_groups(ctx->stream, Xs, bt.g1 - bt.g0, D, K, d_tab + bt.g0, d_tab + G + bt.g0, d_off, pi, mu, var, ctx->w2(),
+                CU(launch_screen_groups(ctx->stream, Xs, rows, bt.g1 - bt.g0, D, K, d_tab + bt.g0, d_tab + G + bt.g0, d_off, pi, mu, var, ctx->w2(),
                                         ctx->c2d(), sb, out, &ctx->launches));
                 CHECK(prof_end(ctx));
             }

@@ -260,6 +260,34 @@ def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
 
 
 # the top-m assignment through the sweep: a point far away from everything, components without a weight (fewer than m with one, once)
+# Sums per group and component: a warp has a run of one to eight components (of few groups with many points one, of many small groups eight; the last run of a
+# group fewer), empty groups and components, pairs of one component beyond a stage of 4 to 32 rows; X at 4 bytes past a boundary.
+@pytest.mark.parametrize("G,most,D,K,offset", [(600, 60, 33, 50, 0), (600, 50, 20, 50, 0), (500, 40, 128, 64, 0), (450, 60, 64, 70, 1), (5, 2500, 9, 20, 0), (3, 3000, 100, 33, 0), (700, 30, 8, 48, 0)])
+def test_screen_sums_per_group(fg, monkeypatch, G, most, D, K, offset):
+    from oracle.fisher import fisher_vectors
+
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    rng = np.random.default_rng(G + D + K)
+    size = rng.integers(0, most, G)
+    size[0] += 1
+    offsets = np.concatenate([[0], np.cumsum(size)]).astype(np.int64)
+    N = int(offsets[-1])
+    X, pi, mu, var = _mixture(N, D, K, G + D)
+    pi[K // 2] = 0.0
+    flat = torch.empty(N * D + offset, device=DEV)
+    Xd = flat[offset:].view(N, D)
+    Xd.copy_(_t(X))
+    lz = orc.responsibilities(X, pi, mu, var)[1]
+    ref = fisher_vectors(X, offsets, pi, mu, var)
+    with fg.Context(0) as c:
+        F, ll = c.gmm_fisher_vectors(Xd, offsets, _t(pi), _t(mu), _t(var))
+        again = c.gmm_fisher_vectors(Xd, offsets, _t(pi), _t(mu), _t(var))
+        assert c.gmm_last_exact_count() == K - 1
+    assert torch.equal(F, again[0]) and ll == again[1] and abs(ll - lz.sum()) <= 1e-5 * abs(lz.sum())
+    F = F.cpu().numpy()
+    assert np.abs(F - ref).max() <= 2e-5 * (1 + np.abs(ref).max()) and np.all(F[size == 0] == 0.0)
+
+
 # Beyond 200,000 points the evaluation sorts a CTA's points by their marks.  A point's values do not depend on the points it is worked on with, so they are
 # the same bits as from two calls that do not sort.  Every other point has 24 marks: 32 of those together have more than a warp has room for at a time.
 @pytest.mark.parametrize("N,D,K,offset", [(200_001, 128, 96, 0), (200_100, 100, 64, 0), (213_121, 64, 1100, 0), (231_000, 24, 2100, 0), (200_193, 32, 64, 1), (200_031, 9, 64, 0)])

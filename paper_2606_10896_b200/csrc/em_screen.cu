@@ -1428,7 +1428,7 @@ __device__ int screen_nearest(const ScreenTie& tie, const float* __restrict__ x,
     return bk;
 }
 
-template <int MODE, int NI>
+template <int MODE, int NX, bool VEC>
 __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __restrict__ X, int64_t n, int D, int K, const float* __restrict__ mu,
                                                              const float* __restrict__ w2, const double* __restrict__ c2d,
                                                              const int* __restrict__ comp_of, int range, int sorted,
@@ -1462,46 +1462,36 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
     if (tid == 0) next_s = 0;
     if (lane == 0) wsum[warp] = 0;
     __syncthreads();
-    // A point's row, in the eight lanes that work on it: dimensions 4 (l8 + 8 i) + (0..3).  NI == 0: rows that cannot be read 16 bytes at a time.
-    constexpr int NX = NI > 0 ? NI : 1;
-    const bool tail = 4 * (l8 + 8 * (NX - 1)) < D;           // (the last group of four dimensions is there)
-    auto row_of = [&](const float* __restrict__ x, uint64_t (&xv)[2 * NX]) {
-        if constexpr (NI > 0) {
+    // A row (of X or of the parameters), NX x 4 values of it in each of the eight lanes that work on a point: dimensions 4 (l8 + 8 i) + (0..3), or, where rows
+    // cannot be read 16 bytes at a time, l8 + 8 (4 i + (0..3)).  Beyond D zeros.
+    auto row_of = [&](const float* __restrict__ r, uint64_t (&v)[2 * NX]) {
 #pragma unroll
-            for (int i = 0; i < NX; ++i) {
+        for (int i = 0; i < NX; ++i) {
+            if constexpr (VEC) {
                 ulonglong2 a = make_ulonglong2(0ull, 0ull);
-                if (i < NX - 1 || tail) a = __ldg(reinterpret_cast<const ulonglong2*>(x) + l8 + 8 * i);
-                xv[2 * i] = a.x;
-                xv[2 * i + 1] = a.y;
+                if (i < NX - 1 || 4 * (l8 + 8 * i) < D) a = __ldg(reinterpret_cast<const ulonglong2*>(r) + l8 + 8 * i);
+                v[2 * i] = a.x;
+                v[2 * i + 1] = a.y;
+            } else {
+                float f[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) f[j] = i < NX - 1 || l8 + 8 * (4 * i + j) < D ? __ldg(r + l8 + 8 * (4 * i + j)) : 0.f;
+                v[2 * i] = pack2(__float_as_uint(f[0]), __float_as_uint(f[1]));
+                v[2 * i + 1] = pack2(__float_as_uint(f[2]), __float_as_uint(f[3]));
             }
         }
     };
     // This lane's part of sum_d w (x - m)^2.
-    auto part_of = [&](const float* __restrict__ x, const uint64_t (&xv)[2 * NX], int k) -> float {
-        const float *m = mu + (size_t)k * D, *w = w2 + (size_t)k * D;
-        if constexpr (NI > 0) {
-            ulonglong2 b[NX], c[NX];
+    auto part_of = [&](const uint64_t (&xv)[2 * NX], int k) -> float {
+        uint64_t m[2 * NX], w[2 * NX], q2 = 0ull;
+        row_of(mu + (size_t)k * D, m);
+        row_of(w2 + (size_t)k * D, w);
 #pragma unroll
-            for (int i = 0; i < NX; ++i) {
-                b[i] = c[i] = make_ulonglong2(0ull, 0ull);
-                if (i < NX - 1 || tail) {
-                    b[i] = __ldg(reinterpret_cast<const ulonglong2*>(m) + l8 + 8 * i);
-                    c[i] = __ldg(reinterpret_cast<const ulonglong2*>(w) + l8 + 8 * i);
-                }
-            }
-            uint64_t q2 = 0ull;
-#pragma unroll
-            for (int i = 0; i < NX; ++i) {
-                const uint64_t t0 = sub2(xv[2 * i], b[i].x), t1 = sub2(xv[2 * i + 1], b[i].y);
-                q2 = fma2(mul2(c[i].x, t0), t0, q2);
-                q2 = fma2(mul2(c[i].y, t1), t1, q2);
-            }
-            return lo2(q2) + hi2(q2);
-        } else {
-            float q = 0.f;
-            for (int d = l8; d < D; d += 8) { const float t = __ldg(x + d) - __ldg(m + d); q = fmaf(__ldg(w + d) * t, t, q); }
-            return q;
+        for (int i = 0; i < 2 * NX; ++i) {
+            const uint64_t t = sub2(xv[i], m[i]);
+            q2 = fma2(mul2(w[i], t), t, q2);
         }
+        return lo2(q2) + hi2(q2);
     };
     auto value_of = [&](int k, float q) -> float { return (float)(__ldg(c2d + k) - (double)q); };
     double ll_acc = 0.0;
@@ -1553,7 +1543,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             for (int s = 0; s < c; s += 4) {
                 const int j = min(s + (lane >> 3), c - 1);
                 const int k = ids[o + j];
-                float q = part_of(X + (row0 + src) * D, xv, k);
+                float q = part_of(xv, k);
                 q += __shfl_xor_sync(0xffffffffu, q, 1);
                 q += __shfl_xor_sync(0xffffffffu, q, 2);
                 q += __shfl_xor_sync(0xffffffffu, q, 4);
@@ -1781,20 +1771,19 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                 const bool have = r0 + grp < points;
                 const uint4 pt = pt_s[warp][min(r0 + grp, points - 1)];
                 const int64_t prow = first + (int)pt.x;
-                const float* const x = X + prow * D;
                 const int cnt = have ? (int)pt.w : 0, steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)cnt);
                 const unsigned off = pt.z;
                 float* const pv = v_s + pt.y;
                 unsigned short* const pk = k_s + pt.y;
                 uint64_t xv[2 * NX];
-                row_of(x, xv);
+                row_of(X + prow * D, xv);
                 // eight pairs' parts, then the sums: lane l8 gets that of pair j0 + l8
                 for (int j0 = 0; j0 < steps; j0 += 8) {
                     float q[8];
 #pragma unroll
                     for (int j = 0; j < 8; ++j) {
                         q[j] = 0.f;
-                        if (j0 + j < steps) q[j] = part_of(x, xv, pk[min(j0 + j, (int)pt.w - 1)]);
+                        if (j0 + j < steps) q[j] = part_of(xv, pk[min(j0 + j, (int)pt.w - 1)]);
                     }
 #pragma unroll
                     for (int o = 4; o > 0; o >>= 1)
@@ -2652,20 +2641,19 @@ cudaError_t launch_screen_eval(cudaStream_t s, int mode, const float* X, int64_t
     int* counts = count ? b.counts : nullptr;
     const bool vec = (D % 4 == 0) && ((reinterpret_cast<uintptr_t>(X) & 15) == 0) && ((reinterpret_cast<uintptr_t>(mu) & 15) == 0) && ((reinterpret_cast<uintptr_t>(w2) & 15) == 0);
     const TopOut out{m, resp, tie ? *tie : ScreenTie{}};
-#define FG_EVAL(M_, N_)                                                                                                                          \
+#define FG_EVAL(M_, N_, V_)                                                                                                                       \
     do {                                                                                                                                         \
-        const cudaError_t e_ = cudaFuncSetAttribute(screen_eval_kernel<M_, N_>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4 + EV_RANGE * 4); \
+        const cudaError_t e_ = cudaFuncSetAttribute(screen_eval_kernel<M_, N_, V_>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCR_MAX_K * 4 + EV_RANGE * 4); \
         if (e_ != cudaSuccess) return e_;                                                                                                        \
-        screen_eval_kernel<M_, N_><<<blocks, 256, (M_ == SCREEN_EM || M_ == SCREEN_ARGMAX) ? smem : smem_order, s>>>(X, n, D, K, mu, w2, c2d, \
-        b.comp_of, range, sorted, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, logp, idx, b.ctl, out);                       \
+        screen_eval_kernel<M_, N_, V_><<<blocks, 256, (M_ == SCREEN_EM || M_ == SCREEN_ARGMAX) ? smem : smem_order, s>>>(X, n, D, K, mu, w2, c2d, \
+        b.comp_of, range, sorted, b.words, b.pt_off, b.pt_cnt, b.ids, b.val, counts, b.ll, logp, idx, b.ctl, out);                               \
     } while (0)
-#define FG_EVALS(M_)                                        \
-    switch (vec ? (D + 31) / 32 : 0) {                      \
-        case 0: FG_EVAL(M_, 0); break;                      \
-        case 1: FG_EVAL(M_, 1); break;                      \
-        case 2: FG_EVAL(M_, 2); break;                      \
-        case 3: FG_EVAL(M_, 3); break;                      \
-        default: FG_EVAL(M_, 4); break;                     \
+#define FG_EVALS(M_)                                                                                            \
+    switch ((D + 31) / 32) {                                                                                    \
+        case 1: if (vec) FG_EVAL(M_, 1, true); else FG_EVAL(M_, 1, false); break;                               \
+        case 2: if (vec) FG_EVAL(M_, 2, true); else FG_EVAL(M_, 2, false); break;                               \
+        case 3: if (vec) FG_EVAL(M_, 3, true); else FG_EVAL(M_, 3, false); break;                               \
+        default: if (vec) FG_EVAL(M_, 4, true); else FG_EVAL(M_, 4, false); break;                              \
     }
     switch (mode) {
         case SCREEN_EM: FG_EVALS(SCREEN_EM) break;

@@ -2348,7 +2348,7 @@ __global__ void __launch_bounds__(1024) screen_group_sort_kernel(int K, const in
 
 // Fisher vectors.  With sums about the component's mean,
 //   G_mu = sum r (x - mu) / (T sigma sqrt(pi)),   G_sigma = (sum r (x - mu)^2 / var - sum r) / (T sqrt(2 pi)):
-// nothing cancels.  fp32 sums of at most 32 pairs at a time, added in fp32.  A warp has runs of GS_COMPS components of a group, whose pairs are neighbours: their rows
+// nothing cancels.  fp32 sums of at most 32 pairs (however few a stage has) at a time, added in fp32, the weights in float64.  A warp has runs of GS_COMPS components of a group, whose pairs are neighbours: their rows
 // come in one stream, as in screen_stats_kernel (GS_STAGES stages of GS_ROWS loads per lane), the parameters one component ahead.
 // Bound by the gathered rows and the runs' first trips.  150 groups of 6827 points, us per call, with a warp per component and 16 rows in flight, waited for / now:
 // 64 x 256 676 / 597, 128 x 512 1139 / 970, 100 x 33 881 / 659; 500 groups of 2000 x 64, K = 256 691 / 623.
@@ -2444,7 +2444,9 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
             const Comp now = c;
             if (k + 1 < k1) c = component(k + 1);
             uint64_t m[2] = {pack2(__float_as_uint(now.m.x), __float_as_uint(now.m.y)), pack2(__float_as_uint(now.m.z), __float_as_uint(now.m.w))};
-            float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, nsum = 0.f;
+            float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, fn = 0.f;
+            uint64_t f1[2] = {0ull, 0ull}, f2[2] = {0ull, 0ull};         // (of the 32 pairs at hand, as fn)
+            double nsum = 0.0;
             const bool any = cur < b;
 #pragma unroll 1
             while (cur < b) {
@@ -2458,7 +2460,6 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
                 }
                 const uint4* const xs = ring + slot * GS_ROWS * 32;
                 const float* const rs = r_s[warp][slot];
-                uint64_t f1[2] = {0ull, 0ull}, f2[2] = {0ull, 0ull};
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int i = pos + u * ROWS + sub;
@@ -2473,10 +2474,15 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
                     f2[0] = fma2(rr, mul2(ta, ta), f2[0]);
                     f2[1] = fma2(rr, mul2(tb, tb), f2[1]);
                 }
-                nsum += lane < SR && pos + lane >= cur && pos + lane < to ? rs[lane] : 0.f;
-                s1[0] += lo2(f1[0]); s1[1] += hi2(f1[0]); s1[2] += lo2(f1[1]); s1[3] += hi2(f1[1]);
-                s2[0] += lo2(f2[0]); s2[1] += hi2(f2[0]); s2[2] += lo2(f2[1]); s2[3] += hi2(f2[1]);
+                fn += lane < SR && pos + lane >= cur && pos + lane < to ? rs[lane] : 0.f;
                 cur = to;
+                if (to == b || (to & 31) == 0) {
+                    s1[0] += lo2(f1[0]); s1[1] += hi2(f1[0]); s1[2] += lo2(f1[1]); s1[3] += hi2(f1[1]);
+                    s2[0] += lo2(f2[0]); s2[1] += hi2(f2[0]); s2[2] += lo2(f2[1]); s2[3] += hi2(f2[1]);
+                    nsum += (double)fn;
+                    f1[0] = f1[1] = f2[0] = f2[1] = 0ull;
+                    fn = 0.f;
+                }
             }
             const float va[4] = {now.v.x, now.v.y, now.v.z, now.v.w}, wa[4] = {now.w.x, now.w.y, now.w.z, now.w.w};
             float gm[4] = {0.f, 0.f, 0.f, 0.f}, gs[4] = {0.f, 0.f, 0.f, 0.f};
@@ -2488,22 +2494,22 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
                         s1[j] += __shfl_xor_sync(0xffffffffu, s1[j], x);
                         s2[j] += __shfl_xor_sync(0xffffffffu, s2[j], x);
                     }
-                float quad = 0.f;                            // (see screen_reduce_kernel; beyond D garbage in s2)
+                float nk = (float)nsum, quad = 0.f;          // (see screen_reduce_kernel; beyond D garbage in s2)
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (sub == 0 && d0 + j < D) quad = fmaf(wa[j], s2[j], quad);
 #pragma unroll
                 for (int x = 16; x > 0; x >>= 1) {
-                    nsum += __shfl_xor_sync(0xffffffffu, nsum, x);
+                    nk += __shfl_xor_sync(0xffffffffu, nk, x);
                     quad += __shfl_xor_sync(0xffffffffu, quad, x);
                 }
-                if (lane == 0) ll_acc += (double)nsum * c2d[k] - (double)quad;
+                if (lane == 0) ll_acc += (double)nk * c2d[k] - (double)quad;
                 const float wk = now.p;
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     if (wk > 0.f && d0 + j < D) {
                         gm[j] = s1[j] * (inv_t * rsqrtf(va[j]) * rsqrtf(wk));
-                        gs[j] = (s2[j] - nsum * va[j]) * (inv_t * rsqrtf(2.0f * wk) / va[j]);
+                        gs[j] = (s2[j] - nk * va[j]) * (inv_t * rsqrtf(2.0f * wk) / va[j]);
                     }
             }
             if (sub == 0 && d0 < D) {

@@ -288,6 +288,32 @@ def test_screen_sums_per_group(fg, monkeypatch, G, most, D, K, offset):
     assert np.abs(F - ref).max() <= 2e-5 * (1 + np.abs(ref).max()) and np.all(F[size == 0] == 0.0)
 
 
+# One group of 32768 points on two components: sums over n of 12000 pairs and more.  32 of them at a time are added to a running fp32 sum, n / 32 additions that each err by
+# at most 2^-24 of what the sum has reached: as random signs, 2^-24 sqrt(n / 32) / 3 of the whole (a third: the sum grows linearly, errors are spread evenly).  On separate clusters
+# sum r (x - mu)^2 / (n var) is 1 + sqrt(2 pi) T G_sigma / n.  (Eight pairs at a time would be twice that, four 2.8 times.)
+@pytest.mark.parametrize("D", [128, 64, 100])
+def test_screen_sums_of_a_large_group(fg, monkeypatch, D):
+    from oracle.fisher import fisher_vectors
+
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    rng = np.random.default_rng(D)
+    T, K = 32768, 20
+    pi = np.full(K, 0.001, np.float32)
+    pi[:2] = 0.982 * np.array([0.6, 0.4])
+    mu = rng.normal(0, 3, (K, D)).astype(np.float32)
+    var = rng.uniform(0.5, 1.5, (K, D)).astype(np.float32)
+    c = (np.arange(T) % 5 < 2).astype(int)
+    X = (mu[c] + np.sqrt(var)[c] * rng.standard_normal((T, D))).astype(np.float32)
+    offsets = np.array([0, T], np.int64)
+    ref = fisher_vectors(X, offsets, pi, mu, var)
+    with fg.Context(0) as ctx:
+        F = ctx.gmm_fisher_vectors(_t(X), offsets, _t(pi), _t(mu), _t(var))[0].cpu().numpy()
+        assert ctx.gmm_last_exact_count() == K
+    n = np.bincount(c)
+    err = np.sqrt(((F - ref)[0, 1, :2] ** 2).mean(1)) * np.sqrt(2.0 * pi[:2]) * T / n
+    assert np.all(err <= 2.0 ** -24 * np.sqrt(n / 32) / 3)
+
+
 # Beyond 200,000 points the evaluation sorts a CTA's points by their marks.  A point's values do not depend on the points it is worked on with, so they are
 # the same bits as from two calls that do not sort.  Every other point has 24 marks: 32 of those together have more than a warp has room for at a time.
 @pytest.mark.parametrize("N,D,K,offset", [(200_001, 128, 96, 0), (200_100, 100, 64, 0), (213_121, 64, 1100, 0), (231_000, 24, 2100, 0), (200_193, 32, 64, 1), (200_031, 9, 64, 0)])

@@ -1599,7 +1599,6 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                     const float v = j < c ? val[o + j] : -CUDART_INF_F, r = fast_ex2((v - m) - ls);
                     const int id = j < c ? ids[o + j] : 0;
                     const bool keep = r >= 9.094947e-13f;
-                    if (keep) ll_acc -= (double)r * (double)v;
                     const unsigned bal = __ballot_sync(0xffffffffu, keep);
                     __syncwarp();
                     if (keep) {
@@ -1628,7 +1627,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             if (idx) idx[row] = best;
             if (histogram && a.cnt > 0) {
                 ids[a.off] = (unsigned short)best;
-                val[a.off] = 1.f;
+                val[a.off] = -1.f;
                 pt_cnt[row] = 1;
                 atomicAdd(&hist[best], 1);
             }
@@ -1636,7 +1635,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
             ll_acc += -CUDART_INF;
         } else if (alone) {
             ids[a.off] = (unsigned short)only;
-            val[a.off] = 1.f;
+            val[a.off] = -1.f;
             pt_cnt[row] = 1;
             if (histogram) atomicAdd(&hist[only], 1);
         } else {
@@ -1777,7 +1776,9 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                 unsigned short* const pk = k_s + pt.y;
                 uint64_t xv[2 * NX];
                 row_of(X + prow * D, xv);
-                // eight pairs' parts, then the sums: lane l8 gets that of pair j0 + l8
+                // eight pairs' parts, then the sums: lane l8 gets that of pair j0 + l8.  (dv: what its value lost in 32 bits, beyond the first eight pairs
+                // in the point's part of val.  All points of a component lose alike, as its constant lies between two floats, so it does not average out.)
+                float dv = 0.f;
                 for (int j0 = 0; j0 < steps; j0 += 8) {
                     float q[8];
 #pragma unroll
@@ -1792,7 +1793,15 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                             const float give = (l8 & o) ? q[j] : q[j + o], keep = (l8 & o) ? q[j + o] : q[j];
                             q[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
                         }
-                    if (j0 + l8 < cnt) pv[j0 + l8] = value_of(pk[j0 + l8], q[0]);
+                    if (j0 + l8 < cnt) {
+                        const double v = __ldg(c2d + pk[j0 + l8]) - (double)q[0];
+                        pv[j0 + l8] = (float)v;
+                        if (MODE == SCREEN_EM) {
+                            const float lost = (float)(v - (double)(float)v);
+                            if (j0 == 0) dv = lost;
+                            else val[off + j0 + l8] = lost;
+                        }
+                    }
                 }
                 __syncwarp();
                 // the eight lanes of a point: its values, eight at a time
@@ -1831,7 +1840,7 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                         if (idx) idx[prow] = best;
                         if (histogram) {
                             ids[off] = (unsigned short)best;
-                            val[off] = 1.f;
+                            val[off] = -1.f;
                             pt_cnt[prow] = 1;
                             atomicAdd(&hist[best], 1);
                         }
@@ -1875,14 +1884,17 @@ __global__ void __launch_bounds__(256, 3) screen_eval_kernel(const float* __rest
                     ll_acc += z;
                 }
                 if (MODE == SCREEN_EM) {
-                    // responsibilities; the pairs below 2^-40 of the total leave the list.  (What the statistics will not
-                    // say of the log-likelihood: see screen_reduce_kernel.)
+                    // responsibilities; the pairs below 2^-40 of the total leave the list.  (The derivative of log Z by a pair's value is its responsibility.)
                     int kept = 0;
                     for (int j0 = 0; j0 < steps; j0 += 8) {
                         const int j = j0 + l8;
                         const float v = j < cnt ? pv[j] : -CUDART_INF_F, r = fast_ex2((v - mx) - ls);
                         const bool keep = r >= 9.094947e-13f;
-                        if (keep) ll_acc -= (double)r * (double)v;
+                        if (j0 > 0) {
+                            if (j < cnt) dv = val[off + j];
+                            __syncwarp();
+                        }
+                        if (keep) ll_acc += (double)(r * dv);
                         const unsigned mine = (__ballot_sync(0xffffffffu, keep) >> (8 * grp)) & 255u;
                         if (keep) {
                             const unsigned short id = pk[j];
@@ -2047,7 +2059,8 @@ __global__ void __launch_bounds__(1024) screen_fill_kernel(int64_t n, int K, int
     }
 }
 
-// Statistics: sums of r, r (x - mu), r (x - mu)^2, fp32 within a work item (at most SCR_SEG pairs of one component), float64 beyond.  A warp takes as
+// Statistics: sums of r, r (x - mu), r (x - mu)^2, and over the points whose only pair this is (r < 0) their number and sum_d w2 (x - mu)^2, which is their
+// log-likelihood; fp32 within a work item (at most SCR_SEG pairs of one component), float64 beyond.  A warp takes as
 // many consecutive items as make one wave of warps (screen_item_group); their pairs are neighbours in srt, whatever their components, so their rows come in one
 // stream: ST_STAGES stages of ST_ROWS loads per lane, by asynchronous copies into shared memory, and the pairs themselves 32 ahead.  LPR lanes per row, four
 // dimensions each; a stage that holds the end of an item is gone through once more for the next one.  A group g has one set of sums per component k in it, at
@@ -2056,6 +2069,8 @@ __global__ void __launch_bounds__(1024) screen_fill_kernel(int64_t n, int K, int
 // warps waiting for one another after 64 rows each (54 % of the issue slots, 3.6 TB/s from memory); 113 with eight rows in flight, no waiting and 20
 // instructions (31 %, 4.3 TB/s).  A step of 1.02M x 128, K = 1024 with those 1036 us, with this 982, 12 warps per SM with 24 rows each on their way; with
 // 16 warps and 16 rows 1030, 8 warps and 40 rows 994, four rows per stage 1065, and the pairs one stage ahead instead of 32 pairs 1075 to 1284.
+// The log-likelihood of the points with several pairs is not sum_k r_k log z_k of these sums: 32 bits lose weights of 1e-8 beside others, each of which is as much of the
+// log-likelihood as its log-density is of a point's (120K x 128, K = 1024: 1.7e-9 of it, against 5e-11).
 constexpr int ST_ROWS = 8, ST_STAGES = 4;
 __device__ __forceinline__ int screen_item_group(int items) { return items <= SCR_STAT_WARPS ? 1 : (items + SCR_STAT_WARPS - 1) / SCR_STAT_WARPS; }
 // The component whose items hold this one: the last with segoff <= item.  The whole warp.
@@ -2071,6 +2086,7 @@ __device__ __forceinline__ int screen_component(const int* __restrict__ segoff, 
 }
 template <int LPR, bool VEC>
 __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const float* __restrict__ X, int D, const float* __restrict__ mu,
+                                                           const float* __restrict__ w2, const double* __restrict__ c2d,
                                                            const uint2* __restrict__ srt, const int* __restrict__ off, const int* __restrict__ segoff,
                                                            int K, double* __restrict__ part, const int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
@@ -2127,12 +2143,16 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
     uint64_t m[2];
+    float w[4];
     int o1;
     auto component = [&]() {
         o1 = __ldg(off + k + 1) - p0;
         float f[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) f[j] = d0 + j < D ? __ldg(mu + (size_t)k * D + d0 + j) : 0.f;
+        for (int j = 0; j < 4; ++j) {
+            f[j] = d0 + j < D ? __ldg(mu + (size_t)k * D + d0 + j) : 0.f;
+            w[j] = d0 + j < D ? __ldg(w2 + (size_t)k * D + d0 + j) : 0.f;
+        }
         m[0] = pack2(__float_as_uint(f[0]), __float_as_uint(f[1]));
         m[1] = pack2(__float_as_uint(f[2]), __float_as_uint(f[3]));
     };
@@ -2141,9 +2161,10 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const
     for (int st = 0; st < ST_STAGES - 1; ++st) issue(st);
     component();
     int item = first, a = 0, b = min(SCR_SEG, o1);   // the item's pairs
-    uint64_t s1[2] = {0ull, 0ull}, s2[2] = {0ull, 0ull};
+    uint64_t s1[2] = {0ull, 0ull}, s2[2] = {0ull, 0ull}, q1[2] = {0ull, 0ull};               // (q1: squares of the points with one pair)
     float nsum = 0.f;
-    double tn = 0.0;
+    int n1 = 0;
+    double tn = 0.0, tq = 0.0;
     bool fresh = true;                               // the first item of a set of sums
 #pragma unroll 1
     for (int st = 0; st < stages; ++st) {
@@ -2160,28 +2181,41 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const
                 const bool on = i >= a && i < b;
                 const float r = on ? rs[u * ROWS + sub] : 0.f;
                 const uint4 x = xs[u * 32];
-                const uint64_t rr = pack2(__float_as_uint(r), __float_as_uint(r));
+                const unsigned ra = __float_as_uint(fabsf(r)), r1 = r < 0.f ? 0x3F800000u : 0u;
+                const uint64_t rr = pack2(ra, ra), one = pack2(r1, r1);
                 uint64_t ta = sub2(pack2(x.x, x.y), m[0]), tb = sub2(pack2(x.z, x.w), m[1]);
                 if (!on) ta = tb = 0ull;             // (a row of another component: the square may be beyond a float)
                 s1[0] = fma2(rr, ta, s1[0]);
                 s1[1] = fma2(rr, tb, s1[1]);
-                s2[0] = fma2(rr, mul2(ta, ta), s2[0]);
-                s2[1] = fma2(rr, mul2(tb, tb), s2[1]);
+                ta = mul2(ta, ta);
+                tb = mul2(tb, tb);
+                s2[0] = fma2(rr, ta, s2[0]);
+                s2[1] = fma2(rr, tb, s2[1]);
+                q1[0] = fma2(one, ta, q1[0]);
+                q1[1] = fma2(one, tb, q1[1]);
             }
-            nsum += lane < SR && pos + lane >= a && pos + lane < b ? rs[lane] : 0.f;
+            const float rl = lane < SR && pos + lane >= a && pos + lane < b ? rs[lane] : 0.f;
+            nsum += fabsf(rl);
+            n1 += rl < 0.f ? 1 : 0;
             if (b > pos + SR) break;
             // the item's last pair
             const float v[8] = {lo2(s1[0]), hi2(s1[0]), lo2(s1[1]), hi2(s1[1]), lo2(s2[0]), hi2(s2[0]), lo2(s2[1]), hi2(s2[1])};
 #pragma unroll
             for (int j = 0; j < 8; ++j) t[j][lane] = fresh ? (double)v[j] : t[j][lane] + (double)v[j];
             tn += (double)nsum;
+            const float z[4] = {lo2(q1[0]), hi2(q1[0]), lo2(q1[1]), hi2(q1[1])};
+            float q = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (d0 + j < D) q = fmaf(w[j], z[j], q);     // (beyond D garbage)
+            tq += (double)q;
             fresh = false;
-            s1[0] = s1[1] = s2[0] = s2[1] = 0ull;
+            s1[0] = s1[1] = s2[0] = s2[1] = q1[0] = q1[1] = 0ull;
             nsum = 0.f;
             a = b;
             ++item;
             if (b == o1 || item == end) {            // and the component's, or the group's
-                double* const o = part + (size_t)(g + k) * (2 * D + 1);
+                double* const o = part + (size_t)(g + k) * (2 * D + 2);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     double q = t[j][lane];
@@ -2190,11 +2224,13 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const
                     if (sub == 0 && d0 + (j & 3) < D) o[(j < 4 ? 0 : D) + d0 + (j & 3)] = q;
                 }
                 tn = warp_sum(tn);
-                if (lane == 0) o[2 * D] = tn;
+                tq = warp_sum((n1 > 0 ? (double)n1 * __ldg(c2d + k) : 0.0) - tq);
+                if (lane == 0) { o[2 * D] = tn; o[2 * D + 1] = tq; }
                 if (item == end) break;
                 do { ++k; } while (__ldg(segoff + k + 1) == item);               // (components without pairs)
                 component();
-                tn = 0.0;
+                tn = tq = 0.0;
+                n1 = 0;
                 fresh = true;
             }
             b = min(a + SCR_SEG, o1);
@@ -2205,11 +2241,9 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_stats_kernel(const
     asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// A CTA per component: its sets of sums in order (two interleaved chains), float64, shifted from its mean to the origin.  Its part of the
-// log-likelihood: sum_i r_ik log z_ik = n c - sum_d w sum_i r_ik (x - mu)^2, which is all there is to a point with one pair; for the others the evaluation
-// has added up log p(x) - sum_k r_k log z_k.
+// A CTA per component: its sets of sums in order (two interleaved chains), float64, shifted from its mean to the origin.
 __global__ void __launch_bounds__(512) screen_reduce_kernel(int D, int K, const double* __restrict__ part, const int* __restrict__ segoff,
-                                                            const float* __restrict__ mu, const float* __restrict__ w2, const double* __restrict__ c2d,
+                                                            const float* __restrict__ mu,
                                                             double* __restrict__ Nk, double* __restrict__ S1, double* __restrict__ S2,
                                                             double* __restrict__ llk, int* __restrict__ ctl) {
     if (ctl[SC_DENSE] != 0) return;
@@ -2219,8 +2253,8 @@ __global__ void __launch_bounds__(512) screen_reduce_kernel(int D, int K, const 
     if (i0 == i1) return;
     const int g0 = i0 / G + k, g1 = (i1 - 1) / G + k + 1;
     __shared__ double sh[2][2][128];
-    __shared__ double tot_s, quad_s[4];
-    const size_t st = (size_t)(2 * D + 1);
+    __shared__ double tot[2];
+    const size_t st = (size_t)(2 * D + 2);
     double a = 0.0;
     if (d < D)
         for (int g = g0 + c; g < g1; g += 8) {
@@ -2231,29 +2265,25 @@ __global__ void __launch_bounds__(512) screen_reduce_kernel(int D, int K, const 
             for (int u = 0; u < 4; ++u) a += v[u];
         }
     sh[c][q][d] = a;
-    if (threadIdx.x < 32) {
+    if (threadIdx.x < 64) {                              // warp: weight, log-likelihood of the points with one pair
+        const int which = threadIdx.x >> 5, lane = threadIdx.x & 31;
         double t = 0.0;
-        for (int g = g0 + threadIdx.x; g < g1; g += 32) t += part[(size_t)g * st + 2 * D];
+        for (int g = g0 + lane; g < g1; g += 32) t += part[(size_t)g * st + 2 * D + which];
         t = warp_sum(t);
-        if (threadIdx.x == 0) tot_s = t;
+        if (lane == 0) tot[which] = t;
     }
     __syncthreads();
     if (threadIdx.x >= 128) return;
-    const double n = tot_s;
-    double quad = 0.0;
+    const double n = tot[0];
     if (d < D) {
         const double s1 = sh[0][0][d] + sh[1][0][d], s2 = sh[0][1][d] + sh[1][1][d];
         const double m = (double)__ldg(mu + (size_t)k * D + d);
-        quad = (double)__ldg(w2 + (size_t)k * D + d) * s2;
         S1[(size_t)k * D + d] += s1 + m * n;
         S2[(size_t)k * D + d] += s2 + 2.0 * m * s1 + m * m * n;
     }
-    quad = warp_sum(quad);
-    if ((d & 31) == 0) quad_s[d >> 5] = quad;
-    asm volatile("bar.sync 1, 128;" ::: "memory");           // (the threads that are left)
     if (d == 0) {
         Nk[k] += n;
-        llk[k] += (n * c2d[k] - (quad_s[0] + quad_s[1] + quad_s[2] + quad_s[3])) * 0.69314718055994530942;
+        llk[k] += tot[1] * 0.69314718055994530942;
     }
 }
 
@@ -2351,7 +2381,7 @@ __global__ void __launch_bounds__(1024) screen_group_sort_kernel(int K, const in
 // nothing cancels.  fp32 sums of at most 32 pairs (however few a stage has) at a time, added in fp32, the weights in float64.  A warp has runs of GS_COMPS components of a group, whose pairs are neighbours: their rows
 // come in one stream, as in screen_stats_kernel (GS_STAGES stages of GS_ROWS loads per lane), the parameters one component ahead.
 // Bound by the gathered rows and the runs' first trips.  150 groups of 6827 points, us per call, with a warp per component and 16 rows in flight, waited for / now:
-// 64 x 256 676 / 597, 128 x 512 1139 / 970, 100 x 33 881 / 659; 500 groups of 2000 x 64, K = 256 691 / 623.
+// 64 x 256 676 / 619, 128 x 512 1139 / 996, 100 x 33 881 / 682; 500 groups of 2000 x 64, K = 256 691 / 645.
 constexpr int GS_COMPS = 8, GS_ROWS = 4, GS_STAGES = 8;      // (components of a run at most)
 template <int LPR, bool VEC>
 __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel(const float* __restrict__ X, int D, int K, int groups, int comps,
@@ -2365,7 +2395,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
     constexpr int W = ST_THREADS / 32;
     static_assert(GS_COMPS < 32, "a lane per offset");
     extern __shared__ __align__(16) unsigned char ring_s[];                                 // [W][GS_STAGES][GS_ROWS][32] 16 bytes
-    __shared__ float r_s[W][GS_STAGES][32];
+    __shared__ float2 r_s[W][GS_STAGES][32];                                                // |r|; 1 where it is the point's only pair
     __shared__ double red[W];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, l = lane % LPR, sub = lane / LPR, d0 = 4 * l;
     uint4* const ring = reinterpret_cast<uint4*>(ring_s) + (size_t)warp * GS_STAGES * GS_ROWS * 32 + lane;
@@ -2417,7 +2447,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
                     fetch(st * SR + 32);
                 }
                 const float r = __shfl_sync(0xffffffffu, __uint_as_float(e.y), (at + lane) & 31);
-                if (lane < SR) r_s[warp][slot][lane] = r;
+                if (lane < SR) r_s[warp][slot][lane] = make_float2(fabsf(r), r < 0.f ? 1.f : 0.f);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const unsigned row = __shfl_sync(0xffffffffu, e.x, at + u * ROWS + sub);
@@ -2445,7 +2475,9 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
             if (k + 1 < k1) c = component(k + 1);
             uint64_t m[2] = {pack2(__float_as_uint(now.m.x), __float_as_uint(now.m.y)), pack2(__float_as_uint(now.m.z), __float_as_uint(now.m.w))};
             float s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, fn = 0.f;
-            uint64_t f1[2] = {0ull, 0ull}, f2[2] = {0ull, 0ull};         // (of the 32 pairs at hand, as fn)
+            uint64_t f1[2] = {0ull, 0ull}, f2[2] = {0ull, 0ull}, q1[2] = {0ull, 0ull};           // (of the 32 pairs at hand, as fn; q1: of the points with one pair)
+            const float va[4] = {now.v.x, now.v.y, now.v.z, now.v.w}, wa[4] = {now.w.x, now.w.y, now.w.z, now.w.w};
+            float n1 = 0.f;
             double nsum = 0.0;
             const bool any = cur < b;
 #pragma unroll 1
@@ -2459,32 +2491,44 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
                     ready = st;
                 }
                 const uint4* const xs = ring + slot * GS_ROWS * 32;
-                const float* const rs = r_s[warp][slot];
+                const float2* const rs = r_s[warp][slot];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int i = pos + u * ROWS + sub;
                     const bool on = i >= cur && i < to;
-                    const float r = on ? rs[u * ROWS + sub] : 0.f;
+                    const float2 r = rs[u * ROWS + sub];
                     const uint4 x = xs[u * 32];
-                    const uint64_t rr = pack2(__float_as_uint(r), __float_as_uint(r));
+                    const uint64_t rr = pack2(__float_as_uint(r.x), __float_as_uint(r.x)), one = pack2(__float_as_uint(r.y), __float_as_uint(r.y));
                     uint64_t ta = sub2(pack2(x.x, x.y), m[0]), tb = sub2(pack2(x.z, x.w), m[1]);
                     if (!on) ta = tb = 0ull;                 // (a row of another component: the square may be beyond a float)
                     f1[0] = fma2(rr, ta, f1[0]);
                     f1[1] = fma2(rr, tb, f1[1]);
-                    f2[0] = fma2(rr, mul2(ta, ta), f2[0]);
-                    f2[1] = fma2(rr, mul2(tb, tb), f2[1]);
+                    ta = mul2(ta, ta);
+                    tb = mul2(tb, tb);
+                    f2[0] = fma2(rr, ta, f2[0]);
+                    f2[1] = fma2(rr, tb, f2[1]);
+                    q1[0] = fma2(one, ta, q1[0]);
+                    q1[1] = fma2(one, tb, q1[1]);
                 }
-                fn += lane < SR && pos + lane >= cur && pos + lane < to ? rs[lane] : 0.f;
+                if (lane < SR && pos + lane >= cur && pos + lane < to) {
+                    fn += rs[lane].x;
+                    n1 += rs[lane].y;
+                }
                 cur = to;
                 if (to == b || (to & 31) == 0) {
                     s1[0] += lo2(f1[0]); s1[1] += hi2(f1[0]); s1[2] += lo2(f1[1]); s1[3] += hi2(f1[1]);
                     s2[0] += lo2(f2[0]); s2[1] += hi2(f2[0]); s2[2] += lo2(f2[1]); s2[3] += hi2(f2[1]);
                     nsum += (double)fn;
-                    f1[0] = f1[1] = f2[0] = f2[1] = 0ull;
+                    const float z[4] = {lo2(q1[0]), hi2(q1[0]), lo2(q1[1]), hi2(q1[1])};
+                    float q = 0.f;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if (d0 + j < D) q = fmaf(wa[j], z[j], q);        // (beyond D garbage)
+                    ll_acc -= (double)q;
+                    f1[0] = f1[1] = f2[0] = f2[1] = q1[0] = q1[1] = 0ull;
                     fn = 0.f;
                 }
             }
-            const float va[4] = {now.v.x, now.v.y, now.v.z, now.v.w}, wa[4] = {now.w.x, now.w.y, now.w.z, now.w.w};
             float gm[4] = {0.f, 0.f, 0.f, 0.f}, gs[4] = {0.f, 0.f, 0.f, 0.f};
             if (any) {
 #pragma unroll
@@ -2494,16 +2538,10 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
                         s1[j] += __shfl_xor_sync(0xffffffffu, s1[j], x);
                         s2[j] += __shfl_xor_sync(0xffffffffu, s2[j], x);
                     }
-                float nk = (float)nsum, quad = 0.f;          // (see screen_reduce_kernel; beyond D garbage in s2)
+                if (n1 > 0.f) ll_acc += (double)n1 * __ldg(c2d + k);
+                float nk = (float)nsum;
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (sub == 0 && d0 + j < D) quad = fmaf(wa[j], s2[j], quad);
-#pragma unroll
-                for (int x = 16; x > 0; x >>= 1) {
-                    nk += __shfl_xor_sync(0xffffffffu, nk, x);
-                    quad += __shfl_xor_sync(0xffffffffu, quad, x);
-                }
-                if (lane == 0) ll_acc += (double)nk * c2d[k] - (double)quad;
+                for (int x = 16; x > 0; x >>= 1) nk += __shfl_xor_sync(0xffffffffu, nk, x);
                 const float wk = now.p;
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
@@ -2527,6 +2565,7 @@ __global__ void __launch_bounds__(ST_THREADS, ST_CTAS) screen_group_stats_kernel
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncwarp();
     }
+    ll_acc = warp_sum(ll_acc);
     if (lane == 0) red[warp] = ll_acc;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -2706,9 +2745,9 @@ cudaError_t launch_screen_stats(cudaStream_t s, const float* X, int64_t n, int D
     constexpr int stats_smem = ST_THREADS / 32 * ST_STAGES * ST_ROWS * 512;
     e = cudaFuncSetAttribute(stats, cudaFuncAttributeMaxDynamicSharedMemorySize, stats_smem);
     if (e != cudaSuccess) return e;
-    stats<<<SCR_STAT_WARPS / (ST_THREADS / 32), ST_THREADS, stats_smem, s>>>(X, D, mu, b.srt, b.off, b.segoff, K, b.part, b.ctl);
+    stats<<<SCR_STAT_WARPS / (ST_THREADS / 32), ST_THREADS, stats_smem, s>>>(X, D, mu, w2, c2d, b.srt, b.off, b.segoff, K, b.part, b.ctl);
     LCHECK();
-    screen_reduce_kernel<<<K, 512, 0, s>>>(D, K, b.part, b.segoff, mu, w2, c2d, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
+    screen_reduce_kernel<<<K, 512, 0, s>>>(D, K, b.part, b.segoff, mu, Nk, S1, S2, b.ll + SCR_LL, b.ctl);
     *launches += 4;
     return cudaGetLastError();
 }

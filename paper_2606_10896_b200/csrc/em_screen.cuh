@@ -57,13 +57,13 @@ struct ScreenBuffers {
     uint2* words;         // [SCR_PIECE][SCR_WORDS] the sweep's marks: a mask, the block of 32 positions it belongs to
     unsigned long long* spill;        // [SCR_MAX_SMS][SCR_SPILL][256]
     unsigned short* ids;  // [SCR_PAIRS] component of a kept pair
-    float* val;           // [SCR_PAIRS] its responsibility
+    float* val;           // [SCR_PAIRS] its responsibility (-1: the point's only pair)
     uint2* srt;           // [SCR_PAIRS] (row, responsibility) sorted by component
     int* counts;          // [SCR_RANGES][K]
     int* totals;          // [K]
     int* off;             // [K + 1] where a component's pairs start in srt
     int* segoff;          // [K + 1] where its work items start
-    double* part;         // [SCR_STAT_WARPS + K][2 D + 1] (see screen_stats_kernel)
+    double* part;         // [SCR_STAT_WARPS + K][2 D + 2] (see screen_stats_kernel)
     double* ll;           // [SCR_LL + K]
     int* ovf;             // [SCR_PIECE]
     int* ctl;             // [SC_WORDS]

@@ -314,6 +314,33 @@ def test_screen_sums_of_a_large_group(fg, monkeypatch, D):
     assert np.all(err <= 2.0 ** -24 * np.sqrt(n / 32) / 3)
 
 
+# Every point has a second component with a share of 1e-8 or so of it, which 32-bit sums of a component's weights lose: so the log-likelihood is that of the points, one by one, and
+# no product of the components' sums.  Roundings of the points' own values go either way and are gone in the sum (what all points of a component lose alike is added back).  Those
+# of the K D / 2 different weights 1 / (2 var) stay: 2^-25 / sqrt(3) each, of half a unit per dimension in 1.5 per dimension; four standard deviations of them.
+@pytest.mark.parametrize("N,D,K", [(60_000, 64, 128), (32_768, 128, 64), (250_000, 16, 96)])
+def test_screen_log_likelihood_of_shared_points(fg, monkeypatch, N, D, K):
+    monkeypatch.setenv("GMM_SCREEN_MARKS", "1000")
+    rng = np.random.default_rng(N + D)
+    mu = rng.normal(0, 6, (K, D))
+    step = rng.standard_normal((K // 2, D))
+    mu[1::2] = mu[::2] + 6.0 * step / np.linalg.norm(step, axis=1, keepdims=True)
+    var = np.repeat(rng.uniform(0.8, 1.2, (K // 2, D)), 2, 0)
+    c = rng.integers(0, K, N)
+    X = _t(mu[c] + np.sqrt(var)[c] * rng.standard_normal((N, D)))
+    pi, mu, var = _t(np.full(K, 1.0 / K)), _t(mu), _t(var)
+    x, m, v = X.double(), mu.double(), var.double()
+    own = torch.as_tensor(c, device=DEV)
+    two = torch.stack([-0.5 * ((x - m[own ^ i]) ** 2 / v[own] + (2 * np.pi * v[own]).log()).sum(1) for i in (0, 1)], 1)      # (all others: below 2^-40)
+    want = float((torch.logsumexp(two, 1) + pi.double()[0].log()).sum())
+    with fg.Context(0) as ctx:
+        err = [abs(ctx.gmm_em_step(X, pi, mu, var)[3] - want) / abs(want)]
+        assert ctx.gmm_last_exact_count() == K
+        offsets = np.append(np.arange(0, N, 20_000), N).astype(np.int64)
+        err.append(abs(ctx.gmm_fisher_vectors(X, offsets, pi, mu, var)[1] - want) / abs(want))
+        assert ctx.gmm_last_exact_count() == K
+    assert max(err) <= 4 * 2.0 ** -25 / np.sqrt(3) / 3 * np.sqrt(2 / (K * D))
+
+
 # Beyond 200,000 points the evaluation sorts a CTA's points by their marks.  A point's values do not depend on the points it is worked on with, so they are
 # the same bits as from two calls that do not sort.  Every other point has 24 marks: 32 of those together have more than a warp has room for at a time.
 @pytest.mark.parametrize("N,D,K,offset", [(200_001, 128, 96, 0), (200_100, 100, 64, 0), (213_121, 64, 1100, 0), (231_000, 24, 2100, 0), (200_193, 32, 64, 1), (200_031, 9, 64, 0)])

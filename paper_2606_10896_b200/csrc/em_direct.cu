@@ -54,6 +54,7 @@ struct DirectArgs {
 __device__ __forceinline__ float dk_ex2(float x) { float y; asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 typedef unsigned long long u64;
 __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) { u64 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
+__device__ __forceinline__ u64 add2(u64 a, u64 b) { u64 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ u64 mul2(u64 a, u64 b) { u64 r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
 __device__ __forceinline__ u64 dup2(float a) { u64 r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a)); return r; }
 __device__ __forceinline__ float lo2(u64 a) { return __uint_as_float((uint32_t)a); }
@@ -553,7 +554,9 @@ __global__ void __launch_bounds__(1024) direct_reduce_kernel(const ReduceArgs p)
 // DK_FUSED; the replicas' sums meet in float64, component k's of all CTAs in CTA k % 16, which updates it and writes its constants to all.  Two
 // cluster barriers.
 // Bound by the latency of that chain: 10K x 16, K = 8 (cycles of an iteration, about): centre 1300, log-sum-exp 5400, statistics 3000, replicas 2000, sums of all CTAs 2000,
-// update 3300, barriers 1500.  10 iterations 210 to 230 -> 171 us.
+// update 3300, barriers 1500.  Whole call, 10 iterations: 209 us with the launches, 153 now.
+// Sums of many terms are taken in parts, at 1 % of the time: the CTAs' rows are many and the lanes of a point few, and errors of one sum after the other grow with the
+// number of its terms (variances of 3000 x 60, K = 10 after an iteration 2.2e-7, in parts 8.3e-8, with the launches 8.3e-8).
 constexpr double FIT_MOST = 6.5e6;
 constexpr int FIT_SMEM = 220 * 1024;
 constexpr int ST_NONE_NEW = 1 << 30;          // (a status that was there before)
@@ -707,28 +710,47 @@ __global__ void __launch_bounds__(FT, 1) direct_fit_kernel(const FitArgs p) {
 #pragma unroll
                     for (int b = 0; b < 4; ++b) q[j][b] = 0ull;
                 }
-#pragma unroll 2
-                for (int d4 = 0; d4 < D4; ++d4) {
-                    const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gs + 4 * d4);
-                    ulonglong2 x[PT];
+                // (eight or sixteen dimensions at a time, which are added to the others then: half the error of one sum of all)
+                auto dims = [&](int d4, auto steps) {
+                    constexpr int ST = decltype(steps)::value;
+                    ulonglong2 x[PT][ST];
 #pragma unroll
-                    for (int j = 0; j < PT; ++j) {
-                        x[j] = *reinterpret_cast<const ulonglong2*>(xr[j] + 4 * d4);
-                        x[j].x = fma2(g.x, 0xBF800000BF800000ull, x[j].x);
-                        x[j].y = fma2(g.y, 0xBF800000BF800000ull, x[j].y);
+                    for (int s = 0; s < ST; ++s) {
+                        const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gs + 4 * (d4 + s));
+#pragma unroll
+                        for (int j = 0; j < PT; ++j) {
+                            x[j][s] = *reinterpret_cast<const ulonglong2*>(xr[j] + 4 * (d4 + s));
+                            x[j][s].x = fma2(g.x, 0xBF800000BF800000ull, x[j][s].x);
+                            x[j][s].y = fma2(g.y, 0xBF800000BF800000ull, x[j][s].y);
+                        }
                     }
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
-                        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + (gq + G * b) * ld + 4 * d4);
-                        const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ms + (gq + G * b) * ld + 4 * d4);
+                        u64 f[PT];
 #pragma unroll
-                        for (int j = 0; j < PT; ++j) {
-                            const u64 t0 = fma2(x[j].x, w.x, m.x), t1 = fma2(x[j].y, w.y, m.y);
-                            q[j][b] = fma2(t0, t0, q[j][b]);
-                            q[j][b] = fma2(t1, t1, q[j][b]);
+                        for (int s = 0; s < ST; ++s) {
+                            const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(sw + (gq + G * b) * ld + 4 * (d4 + s));
+                            const ulonglong2 m = *reinterpret_cast<const ulonglong2*>(ms + (gq + G * b) * ld + 4 * (d4 + s));
+#pragma unroll
+                            for (int j = 0; j < PT; ++j) {
+                                const u64 t0 = fma2(x[j][s].x, w.x, m.x), t1 = fma2(x[j][s].y, w.y, m.y);
+                                f[j] = s == 0 ? mul2(t0, t0) : fma2(t0, t0, f[j]);
+                                f[j] = fma2(t1, t1, f[j]);
+                            }
                         }
+#pragma unroll
+                        for (int j = 0; j < PT; ++j) q[j][b] = add2(q[j][b], f[j]);
                     }
+                };
+                constexpr int MOST = PT == 3 ? 2 : 4;        // (of three points the coordinates do not fit the registers)
+                int d4 = 0;
+#pragma unroll 1
+                for (; d4 + MOST <= D4; d4 += MOST) dims(d4, std::integral_constant<int, MOST>{});
+                if (MOST > 2 && d4 + 2 <= D4) {
+                    dims(d4, std::integral_constant<int, 2>{});
+                    d4 += 2;
                 }
+                if (d4 < D4) dims(d4, std::integral_constant<int, 1>{});
                 float l[PT][4], m[PT], a[PT];
 #pragma unroll
                 for (int j = 0; j < PT; ++j) {
@@ -777,9 +799,8 @@ __global__ void __launch_bounds__(FT, 1) direct_fit_kernel(const FitArgs p) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) a1[c][0] = a1[c][1] = a2[c][0] = a2[c][1] = 0ull;
         if (rep < p.R) {
-            ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gs + 4 * dt);
-#pragma unroll 2
-            for (int r = rep; r < mine; r += p.R) {
+            const ulonglong2 g = *reinterpret_cast<const ulonglong2*>(gs + 4 * dt);
+            auto row = [&](int r, u64 (&f1)[4][2], u64 (&f2)[4][2], float (&fn)[4]) {
                 ulonglong2 x = *reinterpret_cast<const ulonglong2*>(xs + r * ld + 4 * dt);
                 x.x = fma2(g.x, 0xBF800000BF800000ull, x.x);
                 x.y = fma2(g.y, 0xBF800000BF800000ull, x.y);
@@ -789,11 +810,32 @@ __global__ void __launch_bounds__(FT, 1) direct_fit_kernel(const FitArgs p) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
                     const u64 rd = dup2(rr[c]);
-                    nacc[c] += rr[c];
-                    a1[c][0] = fma2(rd, x.x, a1[c][0]);
-                    a1[c][1] = fma2(rd, x.y, a1[c][1]);
-                    a2[c][0] = fma2(rd, y0, a2[c][0]);
-                    a2[c][1] = fma2(rd, y1, a2[c][1]);
+                    fn[c] += rr[c];
+                    f1[c][0] = fma2(rd, x.x, f1[c][0]);
+                    f1[c][1] = fma2(rd, x.y, f1[c][1]);
+                    f2[c][0] = fma2(rd, y0, f2[c][0]);
+                    f2[c][1] = fma2(rd, y1, f2[c][1]);
+                }
+            };
+            // (four rows at a time, the last ones too, which are added to the others then: half the error of one sum of all)
+#pragma unroll 1
+            for (int r = rep; r < mine; r += 4 * p.R) {
+                u64 f1[4][2], f2[4][2];
+                float fn[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) f1[c][0] = f1[c][1] = f2[c][0] = f2[c][1] = 0ull;
+                if (r + 3 * p.R < mine) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) row(r + u * p.R, f1, f2, fn);
+                } else {
+#pragma unroll 1
+                    for (int t = r; t < mine; t += p.R) row(t, f1, f2, fn);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    nacc[c] += fn[c];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) { a1[c][h] = add2(a1[c][h], f1[c][h]); a2[c][h] = add2(a2[c][h], f2[c][h]); }
                 }
             }
         }

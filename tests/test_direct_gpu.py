@@ -108,6 +108,54 @@ def test_direct_fit_in_one_launch(fg, N, D, K, offset, isotropic):
         assert all(torch.equal(u, v) for u, v in zip(again, b))      # the same bits in every run
 
 
+# Sums of many terms are taken in parts.  Points far from two components that share them: a quadratic form q errs by 2^-24 q times a factor that grows with the root of the
+# terms added one after the other (1.15 and 1.26 in parts at the two widths, 1.48 and 1.83 in one sum; the line is between them), a responsibility by that times r (1 - r).
+@pytest.mark.parametrize("D", [60, 100])
+def test_direct_fit_in_one_launch_far_from_two_components(fg, D):
+    rng = np.random.default_rng(D)
+    N = 2500
+    mu = np.stack([np.full(D, -0.01), np.full(D, 0.01)]).astype(np.float32)
+    var = rng.uniform(0.5, 2.0, (1, D)).repeat(2, 0).astype(np.float32)
+    pi = np.full(2, 0.5, np.float32)
+    X = (30.0 * rng.standard_normal((N, D))).astype(np.float32)
+    x = X.astype(np.float64)
+    q = 0.5 * ((x[:, None] - mu) ** 2 / var).sum(2)
+    r = 1.0 / (1.0 + np.exp(q - q[:, ::-1]))
+    n = r.sum(0)
+    m = r.T @ x / n[:, None]
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        p = [_t(pi), _t(mu), _t(var)]
+        before = c.gmm_launch_count()
+        c.gmm_fit(_t(X), *p, 1, 1e-6)
+        assert c.gmm_launch_count() - before == 1
+    err = np.sqrt(((p[1].cpu().numpy() - m) ** 2).mean())
+    unit = 2.0 ** -24 * np.sqrt((((q * r * r[:, ::-1])[:, :, None] * x[:, None]) ** 2).sum(0) / n[:, None] ** 2).mean()
+    assert err <= np.sqrt(D / 42) * unit
+
+
+# Points of one component each, B standard deviations from the centre that the sums are taken about: (x - g)^2 is B^2 times the variance.  A thread adds up L rows, 4 at a time: 2^-24 of
+# the sums so far for each addition are in all 2^-24 sqrt(N / 2 (4^2 / 3 + L^2 / (3 x 4))) of one row (one sum of all: L^2 / 3), random signs, here with a fifth to spare.
+@pytest.mark.parametrize("N,D", [(3000, 128), (7500, 64)])
+def test_direct_fit_in_one_launch_far_from_its_centre(fg, N, D):
+    rng = np.random.default_rng(N)
+    B = 30.0
+    mu = np.stack([np.full(D, -B), np.full(D, B)]).astype(np.float32)
+    var, pi = np.ones((2, D), np.float32), np.full(2, 0.5, np.float32)
+    c = np.arange(N) % 2
+    X = (mu[c] + rng.standard_normal((N, D))).astype(np.float32)
+    v = np.stack([X[c == k].astype(np.float64).var(0) for k in (0, 1)])
+    with fg.Context(0) as ctx:
+        ctx.gmm_set_path(fg.GMM_PATH_FP32)
+        p = [_t(pi), _t(mu), _t(var)]
+        before = ctx.gmm_launch_count()
+        ctx.gmm_fit(_t(X), *p, 1, 1e-6)
+        assert ctx.gmm_launch_count() - before == 1
+    err = np.sqrt((((p[2].cpu().numpy() - v) / v) ** 2).mean())
+    L = -(-(-(-N // 16)) // (512 // (D // 4)))             # (rows of a CTA, threads for the same four dimensions)
+    assert err <= 1.2 * 2.0 ** -24 * B * B / np.sqrt(N / 2) * np.sqrt(16 / 3 + L * L / 12)
+
+
 def test_direct_fit_keeps_the_parameters_of_a_step_that_fails(fg):
     X, pi, mu, var = _mixture(500, 5, 4, 9)
     X[17, 2] = np.nan

@@ -46,14 +46,12 @@ def test_direct_step_at_the_edges_of_its_tiles(fg, N, D, K):
     assert_stats_close(N, max(1.0, data_scale(X)), out[0][:3], ref[:3], f"N={N} D={D} K={K}")
 
 
-# (K D <= 1024: all iterations that there are slots for in one launch; beyond, the launches of every iteration)
 @pytest.mark.parametrize("isotropic", [False, True])
-@pytest.mark.parametrize("N,D,K", [(3000, 7, 6), (3000, 24, 48)])
-def test_direct_fit_runs_ahead_and_stops_by_itself(fg, N, D, K, isotropic):
+def test_direct_fit_runs_ahead_and_stops_by_itself(fg, isotropic):
     # more iterations than there are slots for log-likelihoods; then with a tolerance that the fit meets on its way
-    X, pi, mu, var = _mixture(N, D, K, 3)
+    X, pi, mu, var = _mixture(3000, 7, 6, 3)
     if isotropic:
-        var = np.repeat(var[:, :1], D, 1)
+        var = np.repeat(var[:, :1], 7, 1)
     step = orc.em_iteration_isotropic if isotropic else orc.em_iteration
     iters, want, p = 150, [], (pi, mu, var)
     for _ in range(iters):
@@ -62,13 +60,8 @@ def test_direct_fit_runs_ahead_and_stops_by_itself(fg, N, D, K, isotropic):
     want = np.array(want)
     with fg.Context(0) as c:
         c.gmm_set_covariance(fg.GMM_COV_ISOTROPIC if isotropic else fg.GMM_COV_DIAG)
-        if K * D > 1024:
-            c.gmm_set_path(fg.GMM_PATH_FP32)
         a = [_t(pi), _t(mu), _t(var)]
-        before = c.gmm_launch_count()
         trace, done = c.gmm_fit(_t(X), *a, iters, 1e-6)
-        launches = c.gmm_launch_count() - before
-        assert launches > 2 * iters if K * D > 1024 else launches == 3      # (63 iterations ahead)
         assert done == len(trace) == iters and np.all(np.abs(trace - want) <= 2e-5 * np.abs(want))
         b = [_t(pi), _t(mu), _t(var)]
         short, n = c.gmm_fit(_t(X), *b, iters, 1e-6, tol=1e-6)
@@ -82,10 +75,9 @@ def test_direct_fit_runs_ahead_and_stops_by_itself(fg, N, D, K, isotropic):
 
 # A fit that is one launch of a cluster of 16 CTAs: fewer points than CTAs, CTAs without components or with several, lanes per point 1 to 16, dimensions that are no
 # multiple of four, rows that do not start on 16 bytes; against steps and updates one by one (the same sums in another order: 1e-4 of the data's scale after
-# four iterations at most).  The last three have K D > 1024 and are launches.
+# four iterations at most).
 @pytest.mark.parametrize("isotropic", [False, True])
-@pytest.mark.parametrize("N,D,K,offset", [(1, 1, 1, 0), (15, 3, 2, 0), (40, 128, 8, 0), (2500, 16, 64, 0), (17, 2, 5, 1), (4099, 31, 9, 1), (1700, 5, 33, 0), (30_000, 2, 2, 0), (900, 1, 17, 3),
-                                          (40, 128, 9, 0), (1700, 33, 37, 1), (2500, 17, 64, 0)])
+@pytest.mark.parametrize("N,D,K,offset", [(1, 1, 1, 0), (15, 3, 2, 0), (40, 128, 8, 0), (2500, 16, 64, 0), (17, 2, 5, 1), (4099, 31, 9, 1), (1700, 5, 33, 0), (30_000, 2, 2, 0), (900, 1, 17, 3)])
 def test_direct_fit_in_one_launch(fg, N, D, K, offset, isotropic):
     X, pi, mu, var = _mixture(N, D, K, 7 * N + D + K)
     var = np.maximum(var, 1.0)
@@ -107,7 +99,7 @@ def test_direct_fit_in_one_launch(fg, N, D, K, offset, isotropic):
         counts = c.gmm_update_counts()
         before = c.gmm_launch_count()
         trace, done = c.gmm_fit(Xd, *b, 4, 0.3)
-        assert (c.gmm_launch_count() - before <= 2) == (K * D <= 1024) and done == 4 and c.gmm_update_counts() == counts
+        assert c.gmm_launch_count() - before <= 2 and done == 4 and c.gmm_update_counts() == counts
         assert np.all(np.abs(trace - want) <= 1e-5 * np.abs(want) + 1e-5)
         for u, v, s in zip(b, a, (1.0, data_scale(X) if N > 1 else 1.0, 1.0)):
             assert float((u - v).abs().max()) <= 1e-4 * max(s, 1.0)
@@ -164,13 +156,85 @@ def test_direct_fit_in_one_launch_far_from_its_centre(fg, N, D):
     assert err <= 1.2 * 2.0 ** -24 * B * B / np.sqrt(N / 2) * np.sqrt(16 / 3 + L * L / 12)
 
 
-@pytest.mark.parametrize("N,D,K", [(500, 5, 4), (900, 24, 48)])      # (one launch, the launches of every iteration)
-def test_direct_fit_keeps_the_parameters_of_a_step_that_fails(fg, N, D, K):
-    X, pi, mu, var = _mixture(N, D, K, 9)
+# Fits of mixtures with K D <= 1024 are one launch for as many iterations as there are slots for log-likelihoods (63 ahead), others the launches of every iteration
+@pytest.mark.parametrize("isotropic", [False, True])
+@pytest.mark.parametrize("N,D,K", [(3000, 7, 6), (3000, 24, 48)])
+def test_direct_fit_over_more_iterations_than_slots(fg, N, D, K, isotropic):
+    X, pi, mu, var = _mixture(N, D, K, 3)
+    if isotropic:
+        var = np.repeat(var[:, :1], D, 1)
+    step = orc.em_iteration_isotropic if isotropic else orc.em_iteration
+    iters, want, p = 150, [], (pi, mu, var)
+    for _ in range(iters):
+        *p, ll = step(X, *p, 1e-6)[:4]
+        want.append(ll)
+    want = np.array(want)
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        c.gmm_set_covariance(fg.GMM_COV_ISOTROPIC if isotropic else fg.GMM_COV_DIAG)
+        a = [_t(pi), _t(mu), _t(var)]
+        before = c.gmm_launch_count()
+        trace, done = c.gmm_fit(_t(X), *a, iters, 1e-6)
+        launches = c.gmm_launch_count() - before
+        assert launches > 2 * iters if K * D > 1024 else launches == 3
+        assert done == len(trace) == iters and np.all(np.abs(trace - want) <= 2e-5 * np.abs(want))
+        b = [_t(pi), _t(mu), _t(var)]
+        short, n = c.gmm_fit(_t(X), *b, iters, 1e-6, tol=1e-6)
+        assert 1 < n < iters and np.array_equal(short, trace[:n])
+        change = np.abs(np.diff(short)) / np.abs(short[1:])
+        assert change[-1] <= 1e-6 and np.all(change[:-1] > 1e-6)
+        d = [_t(pi), _t(mu), _t(var)]
+        c.gmm_fit(_t(X), *d, n, 1e-6)
+        assert all(torch.equal(u, v) for u, v in zip(b, d))      # nothing was done after the iteration that met the tolerance
+
+
+# The launches of every iteration against steps and updates one by one: parameters, counts of the updates, the same bits in every run.
+@pytest.mark.parametrize("isotropic", [False, True])
+@pytest.mark.parametrize("N,D,K,offset", [(40, 128, 9, 0), (1700, 33, 37, 1), (2500, 17, 64, 0)])
+def test_direct_fit_beyond_one_launch(fg, N, D, K, offset, isotropic):
+    X, pi, mu, var = _mixture(N, D, K, 7 * N + D + K)
+    var = np.maximum(var, 1.0)
+    if isotropic:
+        var = np.repeat(var[:, :1], D, 1)
+    pi[1] = 0.0                                            # (an empty component keeps its mean and variance)
+    flat = torch.empty(N * D + offset, device=DEV)
+    Xd = flat[offset:].view(N, D)
+    Xd.copy_(_t(X))
+    with fg.Context(0) as c:
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        c.gmm_set_covariance(fg.GMM_COV_ISOTROPIC if isotropic else fg.GMM_COV_DIAG)
+        a, b, want = [_t(pi), _t(mu), _t(var)], [_t(pi), _t(mu), _t(var)], []
+        for _ in range(4):
+            Nk, S1, S2, ll = c.gmm_em_step(Xd, *a)
+            want.append(ll)
+            (c.gmm_finalize_isotropic if isotropic else c.gmm_finalize)(N, Nk, S1, S2, 0.3, *a)
+        counts = c.gmm_update_counts()
+        before = c.gmm_launch_count()
+        trace, done = c.gmm_fit(Xd, *b, 4, 0.3)
+        assert c.gmm_launch_count() - before > 8 and done == 4 and c.gmm_update_counts() == counts
+        assert np.all(np.abs(trace - want) <= 1e-5 * np.abs(want) + 1e-5)
+        for u, v, s in zip(b, a, (1.0, data_scale(X), 1.0)):
+            assert float((u - v).abs().max()) <= 1e-4 * max(s, 1.0)
+        again = [_t(pi), _t(mu), _t(var)]
+        c.gmm_fit(Xd, *again, 4, 0.3)
+        assert all(torch.equal(u, v) for u, v in zip(again, b))
+
+
+def test_direct_fit_beyond_one_launch_keeps_the_parameters_of_a_step_that_fails(fg):
+    X, pi, mu, var = _mixture(900, 24, 48, 9)
     X[17, 2] = np.nan
     with fg.Context(0) as c:
-        if K * D > 1024:
-            c.gmm_set_path(fg.GMM_PATH_FP32)
+        c.gmm_set_path(fg.GMM_PATH_FP32)
+        a = [_t(pi), _t(mu), _t(var)]
+        with pytest.raises(fg.GmmError):
+            c.gmm_fit(_t(X), *a, 5, 1e-6)
+        assert all(np.array_equal(u.cpu().numpy(), v) for u, v in zip(a, (pi, mu, var)))
+
+
+def test_direct_fit_keeps_the_parameters_of_a_step_that_fails(fg):
+    X, pi, mu, var = _mixture(500, 5, 4, 9)
+    X[17, 2] = np.nan
+    with fg.Context(0) as c:
         a = [_t(pi), _t(mu), _t(var)]
         with pytest.raises(fg.GmmError):
             c.gmm_fit(_t(X), *a, 5, 1e-6)

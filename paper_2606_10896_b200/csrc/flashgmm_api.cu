@@ -186,7 +186,8 @@ ScratchLayout scratch_layout(int D, int K, bool planes, bool lists = true) {
         L.s_totals = take((size_t)K * 4);
         L.s_off = take((size_t)(K + 1) * 4);
         L.s_segoff = take((size_t)(K + 1) * 4);
-        // (SCR_STAT_WARPS + K sets are written; the size is that of 25088 + K, so that the memory a shape is screened with stays what it was)
+        // (SCR_STAT_WARPS + K sets of 2 D + 2 are written, 5.8 MB at 128 x 1024; the size, 54 MB there, is that of 25088 + K, so that the memory a shape is screened
+        // with stays what it was: with less, calls short of memory that the dense kernels take now would be screened)
         static_assert(SCR_STAT_WARPS <= 25088, "sets of sums");
         L.s_part = take(((size_t)25088 + K) * (2 * (size_t)D + 3) * 8);
         L.s_ll = take((size_t)(SCR_LL + K) * 8);
@@ -896,7 +897,8 @@ bool dense_tensor(const gmm_ctx* ctx, int D, int K) {
 }
 // Marked pairs per point up to which the screening path is the cheaper one, from measured costs in ns per point: the dense kernels
 // 0.5 + 0.0032 K (0.62 at 10 x 100, 0.83 at 64 x 128, 2.1 at 12 x 541, 3.7 at 128 x 1024), the sweep and what does not depend on the
-// marks 0.15 + 0.001 D + 0.045 per 128 components (see screen_fixed), a pair 0.09 + 0.001 D.  (At most SCR_MARKS.)
+// marks 0.15 + 0.001 D + 0.045 per 128 components (see screen_fixed), a pair 0.09 + 0.001 D.  (At most SCR_MARKS.  The pair's cost is of four pairs of
+// consecutive points per step; with points of one cluster together it is a third less, so that the limit is lower than it would have to be.)
 // K < 64: the FP32 kernels' costs.
 double screen_limit(const gmm_ctx* ctx, int kind, int64_t N, int D, int K, int64_t groups = 0) {
     if (ctx->scr_marks > 0.0) return ctx->scr_marks;
@@ -1484,6 +1486,8 @@ int assign_topm_impl(gmm_ctx* ctx, const float* X, int64_t N, int D, int K, cons
     const bool shape = (double)D >= 1.75 * std::log2((double)K) - 2.0 && (m == 1 || K >= 48 * m) && (m <= 2 || K >= 3 * D);
     // With few points the launches decide: 35 us more of them than the tensor assignment has (us, sparse / tensor: top-1 of 2K x 16, K = 64 99 / 76,
     // of 10K x 32, K = 64 89 / 71, of 20K x 32, K = 256 96 / 88; top-2 of 10K x 128, K = 1024 142 / 133, of 30K 172 / 190).
+    // (two sweeps for m > 1: the cost while all components passed twice.  Now one group of 128 does, so calls close to the line go to the tensor assignment although
+    // the screening may be the faster one.)
     const double gain = (m == 1 ? 0.5 + 0.0018 * K : 0.6 + 0.0025 * K) - (m == 1 ? 1.0 : 2.0) * screen_fixed(D, K);      // ns per point
     const bool pays = shape && (!auto_is_tensor(D, K) || (double)N * gain > 30e3);
     const bool screening = !screened && m <= 4 && m <= K && screen_wanted(ctx, SCREEN_RANKS, N, D, K) && (ctx->scr_marks > 0.0 || pays);

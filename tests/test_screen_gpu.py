@@ -259,7 +259,6 @@ def test_screen_kmeans_scores_and_fisher_vectors(fg, monkeypatch, N, D, K):
     assert np.array_equal(new[empty], mu[empty])               # a centroid without points stays where it is
 
 
-# the top-m assignment through the sweep: a point far away from everything, components without a weight (fewer than m with one, once)
 # Sums per group and component: a warp has a run of one to eight components (of few groups with many points one, of many small groups eight; the last run of a
 # group fewer), empty groups and components, pairs of one component beyond a stage of 4 to 32 rows; X at 4 bytes past a boundary.
 @pytest.mark.parametrize("G,most,D,K,offset", [(600, 60, 33, 50, 0), (600, 50, 20, 50, 0), (500, 40, 128, 64, 0), (450, 60, 64, 70, 1), (5, 2500, 9, 20, 0), (3, 3000, 100, 33, 0), (700, 30, 8, 48, 0)])
@@ -375,6 +374,7 @@ def test_screen_values_are_those_of_smaller_calls(fg, monkeypatch, N, D, K, offs
         assert again[3] == L and all(torch.equal(a, b) for a, b in zip(again[:3], (Nk, S1, S2)))
 
 
+# the top-m assignment through the sweep: a point far away from everything, components without a weight (fewer than m with one, once)
 @pytest.mark.parametrize("N,D,K,m", [(1, 16, 64, 1), (257, 33, 97, 2), (3001, 128, 1024, 2), (3001, 128, 1024, 4), (1500, 20, 300, 3), (900, 66, 4096, 4),
                                      (2000, 9, 130, 1), (300, 12, 192, 4), (1200, 40, 20, 1)])
 def test_screen_top_m(fg, monkeypatch, N, D, K, m):
